@@ -11,6 +11,11 @@ import ctypes
 import os
 from typing import Optional
 
+try:
+    from . import _fastcall                  # csrc/fastcall.c: marshalling of the hot entry points
+except ImportError as _e:                    # not built: an error when one of them is called
+    _fastcall, _fastcall_error = None, str(_e)
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 # DBSPMSPV_LIBRARY: another build of the same library (the range-checked one, for the tests)
 LIB_PATH = os.environ.get("DBSPMSPV_LIBRARY") or os.path.join(HERE, "libdbspmspv.so")
@@ -152,6 +157,43 @@ def _stream() -> int:
     return torch.cuda.current_stream().cuda_stream
 
 
+def _raise(status: int, where: str) -> None:
+    raise DbSpmspvError(status, where)
+
+
+def _load_fast() -> None:
+    """First call of a hot entry point: hands its address in the loaded library to the extension,
+    with torch's raw getters of the current device and stream."""
+    import torch
+    torch.cuda.init()
+    L = lib()
+    _fastcall.setup(tuple(ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _FAST), _raise,
+                    torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+
+
+# The hot entry points.  Arguments as in the header, tensors (or numpy arrays) for the pointers,
+# None for NULL; `stream` (last, optional) is a raw stream, by default torch's current one.
+#   dbspmspv_run(h, x_idx, x_val, nnz_x, semiring, y_idx, y_val, y_capacity, y_nnz, stream=None)
+#   dbspmspv_run_masked(h, x_idx, x_val, nnz_x, semiring, row_mask, complement, y_idx, y_val,
+#                       y_capacity, y_nnz, stream=None)
+#   dbspmspv_decode(h, x, y, stream=None)
+#   dbspmspv_decode_batch(h, x, ldx, y, ldy, batch, stream=None)
+#   db_bfs(h, src, levels, stream=None)
+#   db_sssp(h, src, dist, stream=None) -> number of (min, +) products the search made
+_FAST = ("dbspmspv_run", "dbspmspv_run_masked", "dbspmspv_decode", "dbspmspv_decode_batch", "db_bfs", "db_sssp")
+
+
+def _not_built(*_args, **_kwargs):
+    raise RuntimeError(f"the _fastcall extension is missing ({_fastcall_error}): build it with "
+                       "`python -m paper_2608_16308_b200.build` (there is no fallback)")
+
+
+if _fastcall is not None:
+    _fastcall.set_loader(_load_fast)
+dbspmspv_run, dbspmspv_run_masked, dbspmspv_decode, dbspmspv_decode_batch, db_bfs, db_sssp = (
+    getattr(_fastcall, name, _not_built) for name in _FAST)
+
+
 def default_create_opts() -> CreateOpts:
     o = CreateOpts()
     lib().dbspmspv_default_create_opts(ctypes.byref(o))
@@ -183,29 +225,6 @@ def dbspmspv_create_coo(m, n, nnz, row, col, val, dtype, block_size=16,
                                    _stream() if stream is None else stream)
     _check(st, "dbspmspv_create_coo")
     return h.value
-
-
-def dbspmspv_run(h, x_idx, x_val, nnz_x, semiring, y_idx, y_val, y_capacity, y_nnz,
-                 stream: Optional[int] = None) -> None:
-    _check(lib().dbspmspv_run(h, _ptr(x_idx), _ptr(x_val), nnz_x, semiring, _ptr(y_idx), _ptr(y_val),
-                              y_capacity, _ptr(y_nnz), _stream() if stream is None else stream),
-           "dbspmspv_run")
-
-
-def db_bfs(h, src, levels, stream: Optional[int] = None) -> None:
-    _check(lib().db_bfs(h, src, _ptr(levels), _stream() if stream is None else stream), "db_bfs")
-
-
-def db_sssp(h, src, dist, stream: Optional[int] = None) -> int:
-    """Returns the number of (min, +) products the search made."""
-    steps = ctypes.c_int32(0)
-    _check(lib().db_sssp(h, src, _ptr(dist), ctypes.byref(steps), _stream() if stream is None else stream), "db_sssp")
-    return int(steps.value)
-
-
-def dbspmspv_decode(h, x, y, stream: Optional[int] = None) -> None:
-    _check(lib().dbspmspv_decode(h, _ptr(x), _ptr(y), _stream() if stream is None else stream),
-           "dbspmspv_decode")
 
 
 def dbspmspv_get_stats(h, raise_on_device_status: bool = True) -> Stats:
@@ -243,18 +262,6 @@ def dbspmspv_compact_noalloc(acc, hit_bitmap, m, y_idx, y_val, y_capacity, y_nnz
 def dbspmspv_test_bounded_wait(h, max_tries: int, stream: Optional[int] = None) -> None:
     _check(lib().dbspmspv_test_bounded_wait(h, max_tries, _stream() if stream is None else stream),
            "dbspmspv_test_bounded_wait")
-
-
-def dbspmspv_run_masked(h, x_idx, x_val, nnz_x: int, semiring: int, row_mask, complement: int, y_idx, y_val,
-                        y_capacity: int, y_nnz, stream: Optional[int] = None) -> None:
-    _check(lib().dbspmspv_run_masked(h, _ptr(x_idx), _ptr(x_val), nnz_x, semiring, _ptr(row_mask), complement, _ptr(y_idx),
-                                     _ptr(y_val), y_capacity, _ptr(y_nnz), _stream() if stream is None else stream),
-           "dbspmspv_run_masked")
-
-
-def dbspmspv_decode_batch(h, x, ldx: int, y, ldy: int, batch: int, stream: Optional[int] = None) -> None:
-    _check(lib().dbspmspv_decode_batch(h, _ptr(x), ldx, _ptr(y), ldy, batch, _stream() if stream is None else stream),
-           "dbspmspv_decode_batch")
 
 
 def dbspmspv_test_corrupt_entry(h, position: int, block_index: int) -> None:

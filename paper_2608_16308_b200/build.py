@@ -4,6 +4,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -11,6 +12,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdbspmspv.so")
 LIB_CHECKED = os.path.join(HERE, "libdbspmspv_check.so")   # the range-checked build (-DDBS_BOUNDS_CHECK)
+EXT = os.path.join(HERE, "_fastcall.so")       # the binding's CPython extension (csrc/fastcall.c)
 SOURCES = ("create.cu", "run.cu", "bfs.cu", "api.cu", "noalloc.cu", "measure.cu")
 HEADERS = ("internal.cuh", "microkernels.cuh", "worklist.cuh", "staging.cuh", "lean_pull.cuh", "decode_batch.cuh", "mma_block.cuh", "minplus.cuh", "small_call.cuh")
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -29,9 +31,21 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_extension(force: bool = False) -> str:
+    """Compiles the binding's extension module (plain C against the Python headers)."""
+    src = os.path.join(CSRC, "fastcall.c")
+    if force or _stale(EXT, [src]):
+        r = subprocess.run(["gcc", "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], src, "-o", EXT],
+                           capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError("gcc failed on fastcall.c\n" + r.stderr)
+    return EXT
+
+
 def build_library(force: bool = False, verbose: bool = False, checked: bool = False) -> str:
     """Compiles the sources that changed and links the library; checked=True builds the
     range-checked variant beside it (own object files, own .so)."""
+    build_extension(force)
     lib = LIB_CHECKED if checked else LIB
     extra = ["-DDBS_BOUNDS_CHECK"] if checked else []
     deps_common = [os.path.join(CSRC, h) for h in HEADERS] + [os.path.join(ROOT, "include", "dbspmspv.h"),
