@@ -2,6 +2,7 @@
 // coordinates (used to check that create() loses nothing).
 #include <cub/cub.cuh>
 
+#include "call_graph.cuh"
 #include "internal.cuh"
 
 namespace dbs {
@@ -212,6 +213,7 @@ int dbspmspv_destroy(dbspmspv_handle_t h) {
     if (h->sssp_host) cudaFreeHost(h->sssp_host);
     if (h->ev[0]) cudaEventDestroy(h->ev[0]);
     if (h->ev[1]) cudaEventDestroy(h->ev[1]);
+    delete h->graphs;
     delete h;
     return DBSPMSPV_OK;
 }

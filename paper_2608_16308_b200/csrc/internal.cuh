@@ -253,6 +253,8 @@ struct Device {           // everything the kernels need, passed by value
     Workspace ws;
 };
 
+struct CallGraphs;        // call_graph.cuh: the kept launch graphs of a handle
+
 }  // namespace dbs
 
 struct dbspmspv_handle_s {
@@ -289,6 +291,7 @@ struct dbspmspv_handle_s {
     void *ws_arena;             // the one allocation that holds the whole workspace
     void *sssp_arena;           // db_sssp: frontier lists, y and counters (allocated by the first search)
     int32_t *sssp_host;         // db_sssp: page-locked word the size of the next frontier is copied to
+    dbs::CallGraphs *graphs;    // launch graphs of the calls made on this handle
     cudaStream_t last_stream;   // stream of the last run / decode / bfs call (get_stats waits on it)
 };
 

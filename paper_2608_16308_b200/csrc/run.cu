@@ -4,6 +4,7 @@
 // decode entry (Section 4.3).  Nothing here allocates or synchronises, except db_sssp (a host
 // loop over (min, +) products, at the end of the file).
 #include "internal.cuh"
+#include "call_graph.cuh"
 #include "microkernels.cuh"
 #include "staging.cuh"
 #include "worklist.cuh"
@@ -1883,23 +1884,6 @@ template <typename T> static int dev_alloc_zero(T **p, size_t count, int64_t *to
     return DBSPMSPV_OK;
 }
 
-// Launch with the programmatic-stream-serialisation attribute (see pdl_wait): the kernel may be
-// scheduled while its predecessor in the stream is still draining.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
-}
-
 // Persistent grid of the traversal kernel: as many thread blocks as fit (0 on error).
 template <int DT, typename Out, int MODE> static int compute_grid(int sm_count) {
     const size_t smem = compute_dyn_smem<MODE>();
@@ -1910,25 +1894,20 @@ template <int DT, typename Out, int MODE> static int compute_grid(int sm_count) 
 }
 
 template <int DT, typename Out, int MODE>
-static int launch_compute(dbspmspv_handle_s *h, Out out, float th3, bool pdl, cudaStream_t st, int pull_done = 0) {
+static int launch_compute(dbspmspv_handle_s *h, CallList &calls, Out out, float th3, int pull_done = 0) {
     // (one handle launches one instantiation per output kind; the decode entry of a handle and its
     // run entry differ in Out, hence the two slots)
     int &grid = Out::MASKS ? h->grid_compute : h->grid_compute_dense;
     if (!grid) grid = compute_grid<DT, Out, MODE>(h->sm_count);
     if (!grid) return DBSPMSPV_ERR_CUDA;
     const size_t smem = compute_dyn_smem<MODE>();
-    if (pdl) {
-        DBS_CUDA(launch_pdl(k_compute<DT, Out, MODE>, grid, CTA, smem, st, h->d, out, th3, h->ropts.force_path, h->ropts.popc_threshold, pull_done));
-    } else {
-        k_compute<DT, Out, MODE><<<grid, CTA, smem, st>>>(h->d, out, th3, h->ropts.force_path, h->ropts.popc_threshold, pull_done);
-    }
-    ++h->kernel_launches;
+    calls.add(k_compute<DT, Out, MODE>, grid, CTA, smem, true, h->d, out, th3, h->ropts.force_path, h->ropts.popc_threshold, pull_done);
     return DBSPMSPV_OK;
 }
 
 // The streaming pull of hypersparse handles (lean_pull.cuh), launched behind k_compute.
 template <int DT, typename Out>
-static int launch_lean(dbspmspv_handle_s *h, Out out, float th3, cudaStream_t st) {
+static int launch_lean(dbspmspv_handle_s *h, CallList &calls, Out out, float th3) {
     bool &configured = Out::MINPLUS ? h->lean_configured_min : Out::MASKS ? h->lean_configured : h->lean_configured_dense;
     // filter size: the power of two that holds one bit per column, capped
     const int n_words = (h->d.nb + 1) / 2;
@@ -1940,9 +1919,7 @@ static int launch_lean(dbspmspv_handle_s *h, Out out, float th3, cudaStream_t st
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DBSPMSPV_ERR_CUDA;
         configured = true;
     }
-    DBS_CUDA(launch_pdl(k_pull_lean<DT, Out>, h->sm_count, LEAN_CTA, smem, st, h->d, out, th3, h->ropts.force_path,
-                        h->ropts.popc_threshold, filter_words));
-    ++h->kernel_launches;
+    calls.add(k_pull_lean<DT, Out>, h->sm_count, LEAN_CTA, smem, true, h->d, out, th3, h->ropts.force_path, h->ropts.popc_threshold, filter_words);
     return DBSPMSPV_OK;
 }
 
@@ -2028,6 +2005,7 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
                      int semiring, int32_t *y_idx, float *y_val, int64_t y_capacity, int32_t *y_nnz,
                      cudaStream_t st, const uint32_t *row_mask = nullptr, int complement = 0) {
     const Device &d = h->d;
+    CallList calls;
     // a short x on a hypersparse handle: the whole call as one kernel of one thread-block cluster (small_call.cuh)
     {
         const size_t ywords = (size_t)(d.mb + 1) / 2, cbwords = (size_t)(d.nb + 31) / 32;
@@ -2036,10 +2014,8 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
             !h->ropts.no_small_call && h->ropts.force_path != DBSPMSPV_PATH_PULL && !pull_possible(h, nnz_x, h->ropts.th3) &&
             smem <= SMALL_MAX_SMEM && (int64_t)ywords * 32 * (int64_t)sizeof(int32_t) <= d.ws.task_capacity * (int64_t)sizeof(*d.ws.tasks)) {
             const int mode = semiring == DBSPMSPV_OR_AND ? 1 : semiring == DBSPMSPV_MIN_PLUS ? 2 : 0;
-            k_run_small<DT><<<SMALL_CLUSTER, SMALL_CTA, smem, st>>>(d, x_idx, x_val, nnz_x, mode, y_idx, y_val, y_capacity, y_nnz, row_mask, complement);
-            ++h->kernel_launches;
-            DBS_CUDA(cudaGetLastError());
-            return DBSPMSPV_OK;
+            calls.add(k_run_small<DT>, SMALL_CLUSTER, SMALL_CTA, smem, false, d, x_idx, x_val, nnz_x, mode, y_idx, y_val, y_capacity, y_nnz, row_mask, complement);
+            return submit_calls(h, calls, st);
         }
     }
     // x lists a quarter of the columns or more: a pull is likely (on hypersparse matrices), so
@@ -2052,18 +2028,16 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
     if (nnz_x > 0) {
         const int g = (nnz_x + XB_TPB - 1) / XB_TPB;
         if (late_emit) {
-            k_xblock_sparse<DT, false><<<g, XB_TPB, 0, st>>>(d, x_idx, xv, nnz_x, h->ropts.validate);
+            calls.add(k_xblock_sparse<DT, false>, g, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
             int ge = ((d.nb + 1) / 2 + 7) / 8;
             if (ge > 8 * h->sm_count) ge = 8 * h->sm_count;
-            DBS_CUDA(launch_pdl(k_emit_from_masks, ge, 256, 0, st, d, h->ropts.th3, h->ropts.force_path));
-            ++h->kernel_launches;
+            calls.add(k_emit_from_masks, ge, 256, 0, true, d, h->ropts.th3, h->ropts.force_path);
         } else {
-            k_xblock_sparse<DT, true><<<g, XB_TPB, 0, st>>>(d, x_idx, xv, nnz_x, h->ropts.validate);
+            calls.add(k_xblock_sparse<DT, true>, g, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
         }
-        ++h->kernel_launches;
     }
     OutSparse out{d.ws.y_acc, d.ws.y_hit8};
-    if (h->ropts.timing) DBS_CUDA(cudaEventRecord(h->ev[0], st));
+    if (h->ropts.timing) calls.ev_before = calls.n;
     // private accumulators for the hub row blocks: when x is long enough for their atomics to
     // queue up, and not so long that the call will most likely pull
     const int hub_min = h->ropts.hub_min_nnz_x ? h->ropts.hub_min_nnz_x : HUB_MIN_NNZ_X;
@@ -2072,42 +2046,38 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
     if (minplus && nnz_x > 0 && d.n_entries > 0) {
         const int fp = minplus_pull ? h->ropts.force_path : DBSPMSPV_PATH_PUSH;
         if (fp != DBSPMSPV_PATH_PULL) {
-            DBS_CUDA(launch_pdl(k_minplus_push<DT>, 4 * h->sm_count, MINPLUS_CTA, 0, st, d, h->ropts.th3, fp));
-            ++h->kernel_launches;
+            calls.add(k_minplus_push<DT>, 4 * h->sm_count, MINPLUS_CTA, 0, true, d, h->ropts.th3, fp);
         }
         if (minplus_pull && pull_possible(h, nnz_x, h->ropts.th3)) {
-            const int s = launch_lean<DT, OutSparseMin>(h, OutSparseMin{d.ws.y_acc, d.ws.y_hit8}, h->ropts.th3, st);
+            const int s = launch_lean<DT, OutSparseMin>(h, calls, OutSparseMin{d.ws.y_acc, d.ws.y_hit8}, h->ropts.th3);
             if (s != DBSPMSPV_OK) return s;
         }
     } else if (nnz_x > 0 && d.n_entries > 0) {
         int s = DBSPMSPV_OK;
         if (h->heavy_stage) {
-            s = launch_compute<DT, OutSparse, 1>(h, out, h->ropts.th3, true, st);
+            s = launch_compute<DT, OutSparse, 1>(h, calls, out, h->ropts.th3);
         } else {
             // push by k_compute, pull by the streaming kernel: each returns at once when the
             // selector (evaluated on the device) chose the other; a kernel whose path cannot be
             // chosen is not launched at all
-            if (h->ropts.force_path != DBSPMSPV_PATH_PULL) s = launch_compute<DT, OutSparse, 0>(h, out, h->ropts.th3, true, st);
-            if (s == DBSPMSPV_OK && pull_possible(h, nnz_x, h->ropts.th3)) s = launch_lean<DT, OutSparse>(h, out, h->ropts.th3, st);
+            if (h->ropts.force_path != DBSPMSPV_PATH_PULL) s = launch_compute<DT, OutSparse, 0>(h, calls, out, h->ropts.th3);
+            if (s == DBSPMSPV_OK && pull_possible(h, nnz_x, h->ropts.th3)) s = launch_lean<DT, OutSparse>(h, calls, out, h->ropts.th3);
         }
         if (s != DBSPMSPV_OK) return s;
         if (d.hub_on) {
-            DBS_CUDA(launch_pdl(k_fold_hubs, (d.n_hub_blocks + 3) / 4, 128, 0, st, d));
-            ++h->kernel_launches;
+            calls.add(k_fold_hubs, (d.n_hub_blocks + 3) / 4, 128, 0, true, d);
         }
     }
-    if (h->ropts.timing) { DBS_CUDA(cudaEventRecord(h->ev[1], st)); h->timed = true; }
-    h->kernel_launches += 2;
+    if (h->ropts.timing) { calls.ev_after = calls.n; h->timed = true; }
     const int nt = d.ws.n_tiles;
     const int parity = (int)(++h->compact_calls & 1u);
-    DBS_CUDA(launch_pdl(k_compact_count, nt, TILE_WORDS, 0, st, d, parity, row_mask, complement));
+    calls.add(k_compact_count, nt, TILE_WORDS, 0, true, d, parity, row_mask, complement);
     int extra = (nnz_x + CMP_TPB * 8 - 1) / (CMP_TPB * 8);
     if (extra > 4 * h->sm_count) extra = 4 * h->sm_count;
     const int clear_all = (int64_t)nnz_x * 8 > d.n;     // scattered clears cost more than a full sweep
-    DBS_CUDA(launch_pdl(k_compact_write, nt + extra, CMP_TPB, 0, st, d, y_idx, y_val, y_capacity, y_nnz,
-                        minplus ? 2 : (int)(semiring == DBSPMSPV_OR_AND || DT == DBSPMSPV_PATTERN), x_idx, nnz_x, clear_all, parity, row_mask, complement));
-    DBS_CUDA(cudaGetLastError());
-    return DBSPMSPV_OK;
+    calls.add(k_compact_write, nt + extra, CMP_TPB, 0, true, d, y_idx, y_val, y_capacity, y_nnz,
+              minplus ? 2 : (int)(semiring == DBSPMSPV_OR_AND || DT == DBSPMSPV_PATTERN), x_idx, nnz_x, clear_all, parity, row_mask, complement);
+    return submit_calls(h, calls, st);
 }
 
 // payload bytes of one stage of a warp's ring in the streaming decode: what shared memory leaves
@@ -2127,6 +2097,7 @@ int decode_stage_bytes(const Device &d) {
 template <int DT>
 static int decode_typed(dbspmspv_handle_s *h, const void *x, float *y, cudaStream_t st) {
     const Device &d = h->d;
+    CallList calls;
     h->d.decode_tau = h->ropts.decode_threshold;
     h->d.decode_relu = h->ropts.decode_relu != 0;
     h->d.decode_x_f32 = h->ropts.decode_x_f32 != 0;
@@ -2145,14 +2116,10 @@ static int decode_typed(dbspmspv_handle_s *h, const void *x, float *y, cudaStrea
             if (per_sm < 1) return DBSPMSPV_ERR_CUDA;
             h->stream_grid = per_sm * h->sm_count;
         }
-        if (h->ropts.timing) DBS_CUDA(cudaEventRecord(h->ev[0], st));
-        k_fill_u32<<<(int)((d.m + 1023) / 1024), 256, 0, st>>>(reinterpret_cast<uint32_t *>(y), d.m, 0u);
-        DBS_CUDA(launch_pdl(k_decode_stream<DT>, h->stream_grid, STREAM_CTA, (size_t)lay.total, st, d, x, y, h->ropts.th3_decode, h->ropts.force_path));
-        ++h->kernel_launches;
-        if (h->ropts.timing) { DBS_CUDA(cudaEventRecord(h->ev[1], st)); h->timed = true; }
-        ++h->kernel_launches;
-        DBS_CUDA(cudaGetLastError());
-        return DBSPMSPV_OK;
+        if (h->ropts.timing) { calls.ev_before = 0; calls.ev_after = 2; h->timed = true; }
+        calls.add(k_fill_u32, (int)((d.m + 1023) / 1024), 256, 0, false, reinterpret_cast<uint32_t *>(y), d.m, 0u);
+        calls.add(k_decode_stream<DT>, h->stream_grid, STREAM_CTA, (size_t)lay.total, true, d, x, y, h->ropts.th3_decode, h->ropts.force_path);
+        return submit_calls(h, calls, st);
     }
     if (h->heavy_stage && h->ropts.no_fused_decode != 1) {
         // one kernel for the whole call, when x fits in shared memory
@@ -2168,21 +2135,18 @@ static int decode_typed(dbspmspv_handle_s *h, const void *x, float *y, cudaStrea
                 DBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSED_MAX_SMEM));
                 done = true;
             }
-            if (h->ropts.timing) DBS_CUDA(cudaEventRecord(h->ev[0], st));
-            kernel<<<d.mb, nw * 32, lay.total, st>>>(d, x, y, h->ropts.th3_decode, h->ropts.force_path);
-            if (h->ropts.timing) { DBS_CUDA(cudaEventRecord(h->ev[1], st)); h->timed = true; }
-            ++h->kernel_launches;
-            DBS_CUDA(cudaGetLastError());
-            return DBSPMSPV_OK;
+            if (h->ropts.timing) { calls.ev_before = 0; calls.ev_after = 1; h->timed = true; }
+            calls.add(kernel, d.mb, nw * 32, (size_t)lay.total, false, d, x, y, h->ropts.th3_decode, h->ropts.force_path);
+            return submit_calls(h, calls, st);
         }
     }
     const int64_t padded = (int64_t)((d.nb + 1) / 2) * 32;
     int64_t work = padded > d.m ? padded : d.m;
     int g = (int)((work + 255) / 256);
     if (g > 8 * h->sm_count) g = 8 * h->sm_count;
-    k_xblock_dense<DT><<<g, 256, 0, st>>>(d, x, y);
+    calls.add(k_xblock_dense<DT>, g, 256, 0, false, d, x, y);
     OutDense out{y, nullptr};
-    if (h->ropts.timing) DBS_CUDA(cudaEventRecord(h->ev[0], st));
+    if (h->ropts.timing) calls.ev_before = calls.n;
     if (d.n_entries > 0) {
         int s;
         if (h->heavy_stage) {
@@ -2193,23 +2157,20 @@ static int decode_typed(dbspmspv_handle_s *h, const void *x, float *y, cudaStrea
                 if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_decode_pull<DT>, CTA, 0) != cudaSuccess || per_sm < 1) return DBSPMSPV_ERR_CUDA;
                 grid = per_sm * h->sm_count;
             }
-            DBS_CUDA(launch_pdl(k_decode_pull<DT>, grid, CTA, 0, st, d, (const int32_t *)h->block_row, y, h->ropts.th3_decode, h->ropts.force_path));
-            ++h->kernel_launches;
-            s = launch_compute<DT, OutDense, 1>(h, out, h->ropts.th3_decode, true, st, 1);
+            calls.add(k_decode_pull<DT>, grid, CTA, 0, true, d, (const int32_t *)h->block_row, y, h->ropts.th3_decode, h->ropts.force_path);
+            s = launch_compute<DT, OutDense, 1>(h, calls, out, h->ropts.th3_decode, 1);
         } else {
             s = DBSPMSPV_OK;
-            if (h->ropts.force_path != DBSPMSPV_PATH_PULL) s = launch_compute<DT, OutDense, 0>(h, out, h->ropts.th3_decode, true, st);
-            if (s == DBSPMSPV_OK && pull_possible(h, d.n, h->ropts.th3_decode)) s = launch_lean<DT, OutDense>(h, out, h->ropts.th3_decode, st);
+            if (h->ropts.force_path != DBSPMSPV_PATH_PULL) s = launch_compute<DT, OutDense, 0>(h, calls, out, h->ropts.th3_decode);
+            if (s == DBSPMSPV_OK && pull_possible(h, d.n, h->ropts.th3_decode)) s = launch_lean<DT, OutDense>(h, calls, out, h->ropts.th3_decode);
         }
         if (s != DBSPMSPV_OK) return s;
     }
-    if (h->ropts.timing) { DBS_CUDA(cudaEventRecord(h->ev[1], st)); h->timed = true; }
-    h->kernel_launches += 2;
+    if (h->ropts.timing) { calls.ev_after = calls.n; h->timed = true; }
     int gc = ((d.nb + 1) / 2 + 255) / 256;
     if (gc > h->sm_count) gc = h->sm_count;
-    DBS_CUDA(launch_pdl(k_decode_cleanup, gc, 256, 0, st, d));
-    DBS_CUDA(cudaGetLastError());
-    return DBSPMSPV_OK;
+    calls.add(k_decode_cleanup, gc, 256, 0, true, d);
+    return submit_calls(h, calls, st);
 }
 
 // dbspmspv_decode_batch: where the handle has the streaming form, groups of vectors share one
@@ -2235,7 +2196,7 @@ static int decode_batch_typed(dbspmspv_handle_s *h, const void *x, int64_t ldx, 
     h->d.decode_relu = h->ropts.decode_relu != 0;
     h->d.decode_x_f32 = h->ropts.decode_x_f32 != 0;
     // the per-column kernel on vectors [b0, b0 + g), g <= 4
-    auto scalar_group = [&](const void *xg, float *yg, int g, int only_as_fallback) -> int {
+    auto scalar_group = [&](CallList &calls, const void *xg, float *yg, int g, int only_as_fallback) -> int {
         const int nb = g <= 2 ? 2 : 4;
         const BatchLayout lay(d.nb, nb, d.stage_bytes);
         auto kernel = nb == 2 ? k_decode_stream_batch<DT, 2> : k_decode_stream_batch<DT, 4>;
@@ -2244,8 +2205,7 @@ static int decode_batch_typed(dbspmspv_handle_s *h, const void *x, int64_t ldx, 
             DBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, STREAM_MAX_SMEM));
             done = true;
         }
-        DBS_CUDA(launch_pdl(kernel, h->sm_count, BATCH_CTA, (size_t)lay.total, st, d, xg, ldx, yg, ldy, g, only_as_fallback));
-        ++h->kernel_launches;
+        calls.add(kernel, h->sm_count, BATCH_CTA, (size_t)lay.total, true, d, xg, ldx, yg, ldy, g, only_as_fallback);
         return DBSPMSPV_OK;
     };
     for (int32_t b0 = 0; b0 < batch;) {
@@ -2260,9 +2220,9 @@ static int decode_batch_typed(dbspmspv_handle_s *h, const void *x, int64_t ldx, 
             b0 += 1;
             continue;
         }
-        if (h->ropts.timing) DBS_CUDA(cudaEventRecord(h->ev[0], st));
-        k_zero_rows<<<(int)((d.m + 1023) / 1024), 256, 0, st>>>(yg, ldy, d.m, g);
-        ++h->kernel_launches;
+        CallList calls;
+        if (h->ropts.timing) calls.ev_before = 0;
+        calls.add(k_zero_rows, (int)((d.m + 1023) / 1024), 256, 0, false, yg, ldy, d.m, g);
         if (DT == DBSPMSPV_BF16 && max_mma > 1) {
             const int nb = g <= 2 ? 2 : g <= 4 ? 4 : 8;
             const BatchMmaLayout lay(d.nb, nb, d.stage_bytes);
@@ -2272,20 +2232,20 @@ static int decode_batch_typed(dbspmspv_handle_s *h, const void *x, int64_t ldx, 
                 DBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, STREAM_MAX_SMEM));
                 done = true;
             }
-            DBS_CUDA(launch_pdl(kernel, h->sm_count, BATCH_MMA_CTA, (size_t)lay.total, st, d, xg, ldx, yg, ldy, g));
-            ++h->kernel_launches;
+            calls.add(kernel, h->sm_count, BATCH_MMA_CTA, (size_t)lay.total, true, d, xg, ldx, yg, ldy, g);
             // the fallback for non-finite activations: returns at once unless the kernel above asked for it
             for (int q = 0; q < g; q += 4) {
                 const int gq = g - q < 4 ? g - q : 4;
-                const int s = scalar_group(static_cast<const uint8_t *>(xg) + (size_t)q * (size_t)ldx * esize, yg + (size_t)q * (size_t)ldy, gq, 1);
+                const int s = scalar_group(calls, static_cast<const uint8_t *>(xg) + (size_t)q * (size_t)ldx * esize, yg + (size_t)q * (size_t)ldy, gq, 1);
                 if (s != DBSPMSPV_OK) return s;
             }
         } else {
-            const int s = scalar_group(xg, yg, g, 0);
+            const int s = scalar_group(calls, xg, yg, g, 0);
             if (s != DBSPMSPV_OK) return s;
         }
-        if (h->ropts.timing) { DBS_CUDA(cudaEventRecord(h->ev[1], st)); h->timed = true; }
-        DBS_CUDA(cudaGetLastError());
+        if (h->ropts.timing) { calls.ev_after = calls.n; h->timed = true; }
+        const int s = submit_calls(h, calls, st);
+        if (s != DBSPMSPV_OK) return s;
         b0 += g;
     }
     return DBSPMSPV_OK;

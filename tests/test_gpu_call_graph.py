@@ -1,0 +1,57 @@
+"""From its second call on, a sequence of kernels is launched as a graph that the handle keeps, with
+the arguments and grids of the new call; a call on a capturing stream becomes part of the
+caller's graph instead.  Either way a call gives the oracle's result for its own x."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2608_16308_b200 import binding as B
+from paper_2608_16308_b200 import workloads as wl
+from gpu_util import Handle, DEV, check_against_oracle, ref_matrix
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("counts", [(1, 40, 256), (300, 2000, 301), (5, 3000, 9000)], ids=["short", "general", "mixed"])
+def test_repeated_calls_take_new_arguments(counts):
+    csr = wl.rmat(14, 16, seed=6)
+    A = ref_matrix(csr)
+    h = Handle(csr, B.F32)
+    streams = [torch.cuda.current_stream(), torch.cuda.Stream()]
+    for rep in range(3):
+        for i, k in enumerate(counts):
+            x = wl.sparse_x(50 + 10 * rep + i, 0, csr.n, k)
+            torch.cuda.synchronize()
+            with torch.cuda.stream(streams[(rep + i) % 2]):
+                check_against_oracle(h.run(x), oracle.ref_pull(A, x.idx, x.val))
+    h.close()
+
+
+@pytest.mark.parametrize("count", [64, 1500])
+def test_calls_inside_a_captured_graph(count):
+    csr = wl.rmat(13, 16, seed=8)
+    A = ref_matrix(csr)
+    h = Handle(csr, B.F32)
+    x = wl.sparse_x(3, 0, csr.n, count)
+    xi, xv = torch.from_numpy(x.idx).to(DEV), torch.from_numpy(x.val).to(DEV)
+
+    def call():
+        B.dbspmspv_run(h.h, xi, xv, count, B.PLUS_TIMES, h.y_idx, h.y_val, csr.m, h.y_nnz)
+
+    call(); call()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        call()
+    want = oracle.ref_pull(A, x.idx, x.val)
+    for scale in (1.0, -2.0):
+        xv.copy_(torch.from_numpy((x.val * scale).astype(np.float32)))
+        h.y_nnz.fill_(-7)
+        g.replay()
+        torch.cuda.synchronize()
+        k = int(h.y_nnz.item())
+        check_against_oracle((h.y_idx[:k].cpu().numpy(), h.y_val[:k].cpu().numpy(), k),
+                             (want[0], want[1] * scale, want[2] * abs(scale)))
+    check_against_oracle(h.run(x), want)                     # and ordinary calls afterwards
+    h.close()
