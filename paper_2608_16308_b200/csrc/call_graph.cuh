@@ -1,17 +1,22 @@
-// The kernels of one library call, collected first and then submitted together -- from the second
-// call of the same kind on as ONE launch of a CUDA graph that the handle keeps.
+// The kernels of one library call, collected first and then submitted together.
 //
-// What bounds a short call is the host: on the B200 machine a kernel launch costs 2.3 - 2.9 us of the
-// calling thread, so a product of four kernels cost 10 - 14 us to enqueue before any of them had
-// work, as much as the kernels themselves took.  A graph of the same four kernels launches in 1.2 us,
-// plus 0.25 us for every node whose arguments or grid changed since its last launch
-// (cudaGraphExecKernelNodeSetParams on the kept graph; launches already enqueued are not affected).
-// Inside the graph the kernels keep their programmatic dependency edges (see pdl_wait).
+// What bounds a short call is its launches.  On the B200 machine a kernel launch costs 2.3 - 2.9 us of the
+// calling thread; a kernel that waits for the one before it to end starts on a 2 us grid (one 8 us
+// kernel after the other: 10.24 us a call), while one launched with the programmatic
+// attribute starts as its predecessor drains (8.44 us).  And a graph of the same kernels launches
+// in 1.2 us, plus 0.25 us for every node whose arguments or grid changed, with the programmatic
+// edges inside it but not in front of it.  So:
+//   * the stream still has work (cudaStreamQuery, 0.2 us): the calling thread is ahead of the GPU. The kernels are
+//     launched one by one, every one of them -- the first too -- with the programmatic attribute
+//     (each begins with pdl_wait, so it touches nothing before its predecessor is done);
+//   * the stream is idle: the call's latency counts, and the host's share of it is the largest. From
+//     the second call of the same sequence of kernels on, one launch of a graph that the handle keeps
+//     (cudaGraphExecKernelNodeSetParams takes over the new arguments).
 //
 // A handle keeps at most CALL_GRAPHS graphs, one per sequence of kernels (the paths that a handle's
-// calls take), and replaces the least recently used one.  The first call of a sequence launches
-// its kernels one by one, so a handle that is used once never builds a graph; so do calls on a
-// stream that is being captured (the kernels then become nodes of the caller's graph) and calls
+// calls take), and replaces the least recently used one.  A sequence's first call on an idle stream
+// launches its kernels one by one, so a handle that is used once never builds a graph; so do calls
+// on a stream that is being captured (the kernels then become nodes of the caller's graph) and calls
 // with kernel timing switched on (events between the kernels).
 #pragma once
 
@@ -111,7 +116,7 @@ struct CallGraphs {
     ~CallGraphs() { for (CallGraph &c : g) clear(c); }
 };
 
-inline cudaError_t launch_node(CallNode &k, cudaStream_t st) {
+inline cudaError_t launch_node(CallNode &k, cudaStream_t st, bool chained) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = k.grid;
     cfg.blockDim = k.block;
@@ -121,18 +126,18 @@ inline cudaError_t launch_node(CallNode &k, cudaStream_t st) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = k.pdl ? 1 : 0;
+    cfg.numAttrs = k.pdl || chained ? 1 : 0;
     void *p[CALL_MAX_ARGS];
     k.pointers(p);
     return cudaLaunchKernelExC(&cfg, k.func, p);
 }
 
-// The kernels one by one.
-inline int launch_plain(dbspmspv_handle_s *h, CallList &l, cudaStream_t st) {
+// The kernels one by one; `chained`: the first one too may start while its predecessor drains.
+inline int launch_plain(dbspmspv_handle_s *h, CallList &l, cudaStream_t st, bool chained = false) {
     for (int i = 0; i < l.n; ++i) {
         if (i == l.ev_before) DBS_CUDA(cudaEventRecord(h->ev[0], st));
         if (i == l.ev_after) DBS_CUDA(cudaEventRecord(h->ev[1], st));
-        DBS_CUDA(launch_node(l.node[i], st));
+        DBS_CUDA(launch_node(l.node[i], st, chained));
     }
     if (l.n == l.ev_before) DBS_CUDA(cudaEventRecord(h->ev[0], st));
     if (l.n == l.ev_after) DBS_CUDA(cudaEventRecord(h->ev[1], st));
@@ -165,6 +170,7 @@ inline int submit_calls(dbspmspv_handle_s *h, CallList &l, cudaStream_t st) {
         (void)cudaGetLastError();
         return launch_plain(h, l, st);
     }
+    if (cudaStreamQuery(st) == cudaErrorNotReady) return launch_plain(h, l, st, true);
     CallGraphs &s = *h->graphs;
     CallGraph *c = nullptr, *oldest = &s.g[0];
     for (CallGraph &q : s.g) {

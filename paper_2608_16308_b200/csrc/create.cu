@@ -481,6 +481,20 @@ __global__ void k_csc_colptr(int32_t nb, const uint64_t *keys_sorted, int32_t n,
     colptr[t] = lo;
 }
 
+// Chunks of the direct push's list when every column is listed (see PD_LONG).
+__global__ void k_long_chunks(int32_t nb, const int32_t *ptr, const int32_t *colptr, int32_t *total) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    int c = 0;
+    if (t < (int64_t)nb * 16) {
+        const int32_t *cp = colptr + 17 * (t >> 4);
+        const int deg = cp[(t & 15) + 1] - cp[t & 15], pdeg = cp[0] - ptr[t >> 4];
+        if (deg > PD_LONG) c += (deg + PD_CHUNK - 1) / PD_CHUNK;
+        c += (pdeg + 31) / 32;
+    }
+    c = __reduce_add_sync(0xFFFFFFFFu, c);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(total, c);
+}
+
 __global__ void k_csc_gather(int32_t n_blocks, const uint64_t *keys_sorted,
                              const int32_t *csc2csr, const uint32_t *csr_idx,
                              const uint32_t *csr_w, const uint8_t *csr_aux, uint32_t *csc_idx,
@@ -924,6 +938,16 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         }
         k_lower_bounds<<<grid_for(d.nb + 1), TPB, 0, st>>>(d.nb, bcol_sorted, n_entries, d.csc.ptr);
         k_csc_colptr<<<grid_for((int64_t)d.nb * 17), TPB, 0, st>>>(d.nb, k2, n_entries, d.csc.colptr);
+        d.long_cap = 0;
+        if (!h->heavy_stage) {
+            int32_t *total;
+            DBS_GET(total, 1);
+            DBS_CUDA(cudaMemsetAsync(total, 0, 4, st));
+            k_long_chunks<<<grid_for((int64_t)d.nb * 16), TPB, 0, st>>>(d.nb, d.csc.ptr, d.csc.colptr, total);
+            DBS_CUDA(cudaMemcpyAsync(&d.long_cap, total, 4, cudaMemcpyDeviceToHost, st));
+            DBS_CUDA(cudaStreamSynchronize(st));
+            tp.release(total);
+        }
         DBS_CUDA(cudaStreamSynchronize(st));
         tp.release(k2); tp.release(k2_alt); tp.release(ids); tp.release(ids_alt); tp.release(bcol_sorted);
     }

@@ -75,8 +75,20 @@ constexpr int HUB_COPIES = DBS_HUB_COPIES;              // private accumulator c
 constexpr int HUB_BLOCKS_MAX = DBS_HUB_BLOCKS_MAX;      // hub row blocks per handle, at most
 constexpr int HUB_BLOCK_MIN_ENTRIES = DBS_HUB_MIN_ENTRIES; // view entries that make a row block a hub
 constexpr uint16_t HUB_NONE = 0xFFFFu;
-constexpr int HUB_MIN_NNZ_X = 32768;        // shorter x: too few products for a queue, and the fold kernel is one more step in the chain
-constexpr uint32_t HUB_CLEAR = 0x80000000u; // an untouched private accumulator: -0.0f (see push_private)
+constexpr int HUB_ALL_NNZ_X = 65536;        // shorter x: four copies are enough, and the fold is a quarter
+constexpr int HUB_MIN_NNZ_X = 4096;          // shorter x: too few products for a queue
+constexpr uint32_t HUB_CLEAR = 0x80000000u; // an untouched private accumulator (= ACC_CLEAR)
+// The dense accumulator of a product (Workspace::y_acc).  A row that nothing was added to holds
+// ACC_CLEAR = -0.0f, and any sum of products that are each at least ACC_FLAG_MIN in magnitude
+// differs from it in its bits: such products are multiples of 2^-123, so are all their partial
+// sums (rounding only coarsens the grid), hence a sum is +0 (x + -x in round-to-nearest) or too large to be
+// flushed as a subnormal.  So a product is one atomic whose reply nobody reads, and the structural
+// hit is read off the accumulator; only a smaller product -- a stored zero, a listed zero, 1e-31 --
+// or a NaN sets the row's bit in Workspace::y_mask32 as well.  (A flag byte per row, stored when the atomic
+// returned a cleared sum, cost every product the wait for the reply.)  For (min, +) the same word is
+// the smallest int, which every key exceeds (minplus.cuh).
+constexpr uint32_t ACC_CLEAR = 0x80000000u;
+constexpr float ACC_FLAG_MIN = 7.8886090522101181e-31f;     // 2^-100
 constexpr uint32_t PAD_IDX = 7u << TYPE_SHIFT;   // class code of the slack behind the last view entry: no kernel acts on it
 // The streaming pull of hypersparse handles takes the block-CSR view in chunks of LEAN_CHUNK
 // entries, one chunk (eight entries per lane) per warp pass.
@@ -89,6 +101,14 @@ constexpr int LEAN_CHUNK = DBS_LEAN_CHUNK;
 #endif
 constexpr int PUSH_CHUNK = DBS_PUSH_CHUNK;   // CSC-view entries per push task (32 per warp step)
 static_assert(PUSH_CHUNK == 32, "a push task is one warp step; its record stores the exact entry count in 5 bits");
+// Direct push (push_direct.cuh): a column run longer than PD_LONG entries goes, in chunks of PD_CHUNK entries, to a
+// list that a second kernel walks, a warp per chunk; so does, in chunks of 32, the run of a listed column's payload entries.
+constexpr int PD_CTA = 256;
+#ifndef DBS_PD_LONG
+#define DBS_PD_LONG 128
+#endif
+constexpr int PD_LONG = DBS_PD_LONG;
+constexpr int PD_CHUNK = 128;
 // A run of the push worklist with at least HUB_MIN_ENTRIES entries (a hub column) is not cut
 // into tasks: it is listed once and every warp of the traversal strides over its 32-entry steps.
 constexpr int HUB_MIN_ENTRIES = 8192;
@@ -161,6 +181,8 @@ struct Counters {    // device-resident scalars of one call
     int32_t bfs_levels, bfs_reached;
     int32_t pad;
     int32_t batch_fallback;   // decode_batch: the tensor-core kernel left its vectors to the per-column kernel behind it
+    int32_t finish_ticket;  // k_finish: thread blocks started in this call, plus FINISH_PARITY in every other call
+    int32_t n_long;         // direct push: chunks listed in this call
     int32_t n_hubs;         // hub runs of this call's push worklist (may exceed HUB_CAP: the rest became tasks)
     int32_t bfs_hubs[3];    // BFS: the same per level (the per-level counters rotate three ways: the
                             // level's own, the ones it accumulates for the next level, and a spare
@@ -178,11 +200,12 @@ struct Workspace {
     uint32_t *x_mask32;   // vector-block masks, two 16-bit masks per word
     uint2 *tasks;         // push worklist: (column block | (entries - 1) << 27, first CSC-view position)
     int4 *hubs;           // 3 x HUB_CAP hub runs (column block, first position, entries, -): see worklist.cuh
-    float *y_acc;         // m (padded): dense accumulator, all zero between calls
-    uint32_t *y_mask32;   // run: hit masks packed by the compaction pass; BFS: next-frontier masks
-    uint8_t *y_hit8;      // run: one structural-hit flag byte per row, all zero between calls
-    int32_t *tile_count;  // compaction: result entries per tile of row blocks
-    int32_t *tile_group;  // compaction: [2][n_tile_groups] totals of groups of 32 tiles, by call parity
+    float *y_acc;         // m (padded): dense accumulator, all ACC_CLEAR between calls
+    uint32_t *y_mask32;   // run: structural-hit bits, all zero between calls (flags of tiny products, then the
+                          // whole mask, written by the counting pass); BFS: next-frontier masks
+    int4 *long_runs;      // direct push: {first position, entries, x value, 0 or 256 + local column of payload entries} of the listed chunks
+    int32_t *tile_status; // end of a call: result entries of every tile of rows, times two, plus the call's parity
+    unsigned long long *tile_group;   // ... and per group of 32 tiles, by parity: tiles counted << 32 | their entries
     int32_t n_tile_groups;
     uint32_t *visited32;  // BFS: visited masks
     uint32_t *z_mask32;   // BFS: third mask buffer (frontier / next / being cleared rotate)
@@ -243,12 +266,13 @@ struct Device {           // everything the kernels need, passed by value
     // Hub row blocks (null / 0 when the matrix has none): hub_slot[rb] = slot of row block rb or
     // HUB_NONE; hub_acc[(copy * n_hub_blocks + slot) * 16 + row] = private accumulators, all
     // HUB_CLEAR between calls.
-    // hub_rb[slot] = the row block; hub_on: this call's push uses them (set per call by the host).
+    // hub_rb[slot] = the row block; hub_on: how many copies this call's push uses (set per call by the host).
     const uint16_t *hub_slot;
     const int32_t *hub_rb;
     float *hub_acc;
     int32_t n_hub_blocks;
-    int32_t hub_on;
+    int32_t hub_on;           // copies in use (0: none)
+    int32_t long_cap;         // direct push: chunks of all long runs and payload runs together (0: the matrix has none)
     const uint32_t *row_present32;  // per row block: rows that hold a stored element (two 16-bit masks per word)
     Workspace ws;
 };
@@ -277,7 +301,6 @@ struct dbspmspv_handle_s {
     bool fused_configured[3];
     bool batch_configured[2];
     bool batch_mma_configured[3];
-    uint32_t compact_calls;     // compaction launches so far (their parity picks the group-total buffer)
     int stream_grid;            // thread blocks of the streaming decode (0: not configured yet)
     int32_t *x_nnz_seen_host;   // host view of Device::x_nnz_seen (page-locked, mapped)
     bool heavy_stage;           // most stored elements sit in mask-based blocks: MODE 1 kernels
@@ -362,6 +385,9 @@ __device__ __forceinline__ void chk_entry(const Device &d, bool csr_view, uint32
 __device__ __forceinline__ uint32_t mask_of(const uint32_t *mask32, int blk) {
     return reinterpret_cast<const uint16_t *>(mask32)[blk];
 }
+
+// Adds one sum to a row of the accumulator (see ACC_CLEAR).
+__device__ __forceinline__ bool acc_needs_flag(float v) { return !(fabsf(v) >= ACC_FLAG_MIN); }
 
 // value loads from the payload, widened to fp32
 template <int DT> struct Val;

@@ -87,12 +87,10 @@ __device__ __forceinline__ LeanRegs lean_fetch(const Device &d, int c, int lane)
 template <int DT, typename Out>
 __device__ __forceinline__ void lean_add(Out out, int row, float v) {
     if (Out::MINPLUS) {          // keep the smaller sum (an atomic whose reply nobody waits for)
-        atomicMax(reinterpret_cast<uint32_t *>(out.acc) + row, minplus_key(v));
-        out.hit8[row] = 1;
+        atomicMax(reinterpret_cast<int *>(out.acc) + row, minplus_word(v));
         return;
     }
-    if (DT != DBSPMSPV_PATTERN) atomicAdd(out.acc + row, v);
-    if (Out::MASKS) out.hit8[row] = 1;
+    out_add(out, row, DT != DBSPMSPV_PATTERN ? v : 1.0f);
 }
 // The semiring of the segmented reduction: (+, *) or, for Out::MINPLUS, (min, +).
 template <typename Out> __device__ __forceinline__ float lean_identity() { return Out::MINPLUS ? __int_as_float(0x7F800000) : 0.f; }
@@ -291,8 +289,7 @@ k_pull_lean(Device d, Out out, float th3, int force_path, int popc_threshold, in
         const int rb = d.entry_row[pos];
         if (Out::MINPLUS) {
             block_rows_min_warp<DT>(type, d.csr.w[pos], d.csr.aux[pos], xm, d.ws.x_dense + (size_t)cb * 16, d.payload, lane, [&](int r, uint32_t key) {
-                atomicMax(reinterpret_cast<uint32_t *>(out.acc) + (size_t)rb * 16 + r, key);
-                out.hit8[(size_t)rb * 16 + r] = 1;
+                atomicMax(reinterpret_cast<int *>(out.acc) + (size_t)rb * 16 + r, minplus_word_of_key(key));
             });
             continue;
         }
@@ -306,10 +303,7 @@ k_pull_lean(Device d, Out out, float th3, int force_path, int popc_threshold, in
             __syncwarp();
             sum = warp_block<DT>(type, blk, nnz, xm, ls->sx, ls->stmp, lane, popc_threshold, hits);
         }
-        if (lane < 16 && ((hits >> lane) & 1u)) {
-            if (DT != DBSPMSPV_PATTERN) atomicAdd(out.acc + (size_t)rb * 16 + lane, sum);
-            if (Out::MASKS) out.hit8[(size_t)rb * 16 + lane] = 1;
-        }
+        if (lane < 16 && ((hits >> lane) & 1u)) out_add(out, (size_t)rb * 16 + lane, DT != DBSPMSPV_PATTERN ? sum : 1.0f);
     }
 }
 

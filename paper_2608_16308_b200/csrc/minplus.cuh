@@ -7,13 +7,15 @@
 // 32-bit KEY of the smallest sum so far instead of a running sum:
 //     ordered(v) = bits(v) ^ (v < 0 ? 0xFFFFFFFF : 0x80000000)     (monotone in v)
 //     key(v)     = ~ordered(v)                                      (smaller v -> larger key)
-// so "take the minimum" is one atomicMax on an unsigned word, its identity is the all-zero
-// word -- exactly the cleared state the compaction leaves the accumulator in -- and the first
-// sum to reach a row is the one whose atomicMax returns 0 (it sets the row's flag).  The only
+//     word(v)    = key(v) ^ 0x80000000                              (the same order on signed words)
+// so "take the minimum" is one atomicMax on a signed word, and its identity is the smallest
+// int -- exactly the cleared state of the accumulator (ACC_CLEAR), which every word exceeds, so a
+// row was reached iff its word is no longer that.  The only
 // value whose key would be 0 is the NaN 0x7FFFFFFF; NaN has no place in a (min, +) product and
-// its key is stored as 1.  The compaction turns the keys back into values.
+// its key is stored as 1.  The compaction turns the words back into values.
 //
-// Traversal.  Push (this file): a warp takes one task of the push worklist, 32 entries of the
+// Traversal.  Push: hypersparse handles through the direct push (push_direct.cuh); handles whose elements sit
+// mostly in mask-based blocks (this file): a warp takes one task of the push worklist, 32 entries of the
 // block-CSC view, lane = entry; a lane walks all stored elements of its block that sit in
 // listed columns, whatever the block's class.  Pull: on hypersparse valued handles the streaming
 // pull kernel runs with the semiring swapped (lean_pull.cuh); the selector is the same
@@ -35,6 +37,11 @@ __device__ __forceinline__ float minplus_value(uint32_t key) {
     const uint32_t o = ~key;
     return __uint_as_float((o >> 31) ? o ^ 0x80000000u : ~o);
 }
+
+// the word the accumulator keeps
+__device__ __forceinline__ int minplus_word_of_key(uint32_t key) { return (int)(key ^ 0x80000000u); }
+__device__ __forceinline__ int minplus_word(float v) { return minplus_word_of_key(minplus_key(v)); }
+__device__ __forceinline__ float minplus_of_word(uint32_t word) { return minplus_value(word ^ 0x80000000u); }
 
 // Every stored element (r, c, a) of one block whose column c is set in xm, by one lane.
 template <int DT, typename F>
@@ -167,7 +174,7 @@ __global__ void __launch_bounds__(MINPLUS_CTA, 4) k_minplus_push(Device d, float
     const int n_recs = ctr->n_tasks, n_hubs = min(ctr->n_hubs, HUB_CAP);
     const HubTable hubs = load_hub_table(d.ws.hubs, n_hubs, lane);
     const int n_tasks = n_recs + hubs.total;
-    uint32_t *keys = reinterpret_cast<uint32_t *>(d.ws.y_acc);
+    int *words = reinterpret_cast<int *>(d.ws.y_acc);
     for (int t = gwarp; t < n_tasks; t += nwarps) {
         const uint2 task = worklist_item(d.ws.tasks, n_recs, hubs, t);
         const int jb = (int)(task.x & IDX_MASK), cnt = (int)(task.x >> 27) + 1, start = (int)task.y;
@@ -179,8 +186,7 @@ __global__ void __launch_bounds__(MINPLUS_CTA, 4) k_minplus_push(Device d, float
         const float *xb = d.ws.x_dense + (size_t)jb * 16;
         const size_t row0 = (size_t)(idx & IDX_MASK) * 16;
         block_elements<DT>((int)(idx >> TYPE_SHIFT), w, aux, xm, d.payload, [&](int r, int c, float a) {
-            const uint32_t old = atomicMax(keys + row0 + r, minplus_key(a + xb[c]));
-            if (old == 0u) d.ws.y_hit8[row0 + r] = 1;
+            atomicMax(words + row0 + r, minplus_word(a + xb[c]));
         });
     }
 }

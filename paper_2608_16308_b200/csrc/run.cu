@@ -12,8 +12,37 @@
 
 namespace dbs {
 __device__ __forceinline__ int select_path(const Device &d, float th3, int force_path);
+
+// ------------------------------------------------------------------------------------------
+// Output of a traversal.  The sparse path accumulates into the handle's dense accumulator (see
+// ACC_CLEAR); the decode path adds straight into the caller's y.
+// ------------------------------------------------------------------------------------------
+struct OutSparse {
+    float *acc;
+    uint32_t *flag32;  // bits of the rows that a tiny sum reached
+    static constexpr bool MASKS = true;
+    static constexpr bool MINPLUS = false;
+};
+struct OutDense {
+    float *acc;
+    uint32_t *flag32;
+    static constexpr bool MASKS = false;
+    static constexpr bool MINPLUS = false;
+};
+// (min, +) semiring: the accumulator holds words of the smallest sum so far (minplus.cuh)
+struct OutSparseMin {
+    float *acc;
+    uint32_t *flag32;
+    static constexpr bool MASKS = true;
+    static constexpr bool MINPLUS = true;
+};
+template <typename Out> __device__ __forceinline__ void out_add(Out out, size_t row, float v) {
+    atomicAdd(out.acc + row, v);
+    if (Out::MASKS && acc_needs_flag(v)) atomicOr(out.flag32 + (row >> 5), 1u << (row & 31));
+}
 }
 #include "lean_pull.cuh"
+#include "push_direct.cuh"
 
 namespace dbs {
 
@@ -21,28 +50,29 @@ constexpr int CTA = 128;            // four warps per thread block (Section 3.3.
 constexpr int WARPS = CTA / 32;
 constexpr int XB_TPB = 512;         // vector blocking of a sparse x: threads per block
 constexpr int CMP_TPB = 256;        // compaction: threads per tile
-constexpr int TILE_WORDS = CMP_TPB / 4;  // a tile: 64 mask words = 2048 rows; placement uses 8 rows per thread
+constexpr int TILE_WORDS = CMP_TPB / 4;  // a tile: 64 mask words = 2048 rows, 8 rows per thread
 
 // ------------------------------------------------------------------------------------------
-// Vector blocking (Section 3.2.2) fused with the push worklist (Section 3.3.2).
-// Sparse input: one thread per listed nonzero scatters the value into the dense copy and sets
-// its mask bit; the thread that turns a vector block from empty to nonempty emits the block's
-// push tasks (runs of <= 32 entries of its block-CSC column).  Space in the worklist is
+// Vector blocking (Section 3.2.2) of a sparse x: one thread per listed nonzero scatters the value
+// into the dense copy and sets its mask bit.
+// EMIT (handles whose elements sit mostly in blocks with a payload: banded matrices, pruned
+// layers): fused with the push worklist (Section 3.3.2) -- the thread that turns a vector block from
+// empty to nonempty emits the push tasks of its whole block-CSC column (runs of <= 32 entries; the
+// INLINE elements among them are filtered by the mask in the traversal).  Space in the worklist is
 // claimed with a warp scan, a sum over the thread block's warps and one atomic per thread
 // block; the count of nonempty vector blocks is aggregated the same way (Section 4.1).
+// Without EMIT: the dense copy, the masks and the count only -- hypersparse handles whose path is
+// decided on the device; the direct push then takes its columns from the masks.
 // ------------------------------------------------------------------------------------------
-// EMIT = false: only the dense copy, the masks and the count -- the worklist is then built by
-// k_emit_from_masks, and only if the selector chooses the push (used when x is so dense that a
-// pull is likely: the tasks of half a million columns would be written for nothing).
 template <int DT, bool EMIT>
 __global__ void k_xblock_sparse(Device d, const int32_t *__restrict__ x_idx, const void *__restrict__ x_val,
                                 int32_t nnz_x, int validate) {
+    pdl_wait();
     pdl_launch_dependents();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
-    bool newly = false, fresh = false;
-    int jb = 0, jcol = 0;
-    int first = 0, deg = 0, pfirst = 0, pdeg = 0;
+    bool newly = false;
+    int jb = 0, first = 0, end = 0;
     if (t < nnz_x) {
         const int j = x_idx[t];
         // an index outside [0, n) is never written through: the entry is skipped and the call
@@ -58,72 +88,20 @@ __global__ void k_xblock_sparse(Device d, const int32_t *__restrict__ x_idx, con
             // a listed NaN that happens to carry the marker's bit pattern is stored as the
             // canonical quiet NaN, so the marker itself never appears as data
             d.ws.x_dense[j] = __float_as_uint(v) == X_ABSENT ? __uint_as_float(0x7FC00000u) : v;
-            // the runs this thread may have to turn into tasks are fetched before the atomic
-            // whose result decides it (the loads are independent of it; the chain is shorter)
-            if (EMIT) { column_run(d, j, first, deg); payload_run(d, j >> 4, pfirst, pdeg); }
-            const int sh = ((j >> 4) & 1) * 16;
+            jb = j >> 4;
+            // (fetched before the atomic whose result decides whether it is needed)
+            if (EMIT) { first = d.csc.ptr[jb]; end = d.csc.ptr[jb + 1]; }
+            const int sh = (jb & 1) * 16;
             const uint32_t old = atomicOr(&d.ws.x_mask32[j >> 5], 1u << ((j & 15) + sh));
             newly = ((old >> sh) & 0xFFFFu) == 0;
-            fresh = ((old >> ((j & 15) + sh)) & 1u) == 0;     // (an index listed twice emits once)
-            if (validate && !fresh) d.ws.ctr->status = DBSPMSPV_ERR_INVALID_ARG;   // optional check: duplicate index
-            jb = j >> 4;
-            jcol = j;
+            if (validate && ((old >> ((j & 15) + sh)) & 1u)) d.ws.ctr->status = DBSPMSPV_ERR_INVALID_ARG;   // optional check: duplicate index
         }
     }
-    if (!EMIT) {                                              // count the nonempty vector blocks, nothing else
-        emit_tasks<true>(d, newly, jb, 0, 0, lane, &d.ws.ctr->n_tasks, &d.ws.ctr->n_nzblk);
-        return;
-    }
-    // push tasks: the INLINE elements of this column; and, by the thread that turned the vector
-    // block nonempty, the column block's entries with a payload
-    if (d.payload_chunk == PUSH_CHUNK) {
-        // Matrices whose elements sit mostly in blocks with a payload (banded matrices, pruned
-        // layers): the thread that turned the vector block nonempty emits the whole column block
-        // in one run -- payload entries and INLINE elements, the latter filtered by the mask in
-        // the traversal.  Per-column runs would split a column block over several half-empty
-        // tasks here (measured on the stencil: 30 % slower).
-        first = pfirst;
-        deg = newly ? d.csc.ptr[jb + 1] - pfirst : 0;
-        emit_tasks<true>(d, newly, jb, first, deg, lane, &d.ws.ctr->n_tasks, &d.ws.ctr->n_nzblk, PUSH_CHUNK, &d.ws.ctr->n_hubs, d.ws.hubs);
-        return;
-    }
-    if (!fresh) deg = 0;
-    merge_column_runs(fresh, jcol, first, deg, lane);
-    emit_tasks<true>(d, newly, jb, first, deg, lane, &d.ws.ctr->n_tasks, &d.ws.ctr->n_nzblk, PUSH_CHUNK, &d.ws.ctr->n_hubs, d.ws.hubs);
-    if (!newly) pdeg = 0;
-    if (__syncthreads_or(pdeg > 0))
-        emit_tasks<true>(d, false, jb, pfirst, pdeg, lane, &d.ws.ctr->n_tasks, &d.ws.ctr->n_nzblk, d.payload_chunk);
+    emit_tasks<true>(d, newly, jb, first, EMIT && newly ? end - first : 0, lane, &d.ws.ctr->n_tasks, &d.ws.ctr->n_nzblk, PUSH_CHUNK,
+                     EMIT ? &d.ws.ctr->n_hubs : nullptr, d.ws.hubs);
 }
 
 __device__ __forceinline__ int select_path(const Device &d, float th3, int force_path);
-
-// The push worklist from the finished vector-block masks (hypersparse matrices): runs only if
-// the selector chooses the push.  A warp takes one mask word (two vector blocks) at a time,
-// lane = column: listed columns emit their INLINE runs (adjacent ones merged), lanes 0 and 16
-// the payload runs of the two blocks.
-__global__ void k_emit_from_masks(Device d, float th3, int force_path) {
-    pdl_wait();
-    pdl_launch_dependents();
-    if (select_path(d, th3, force_path) != DBSPMSPV_PATH_PUSH) return;
-    const int lane = threadIdx.x & 31;
-    const int gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int n_words = (d.nb + 1) / 2;
-    Counters *ctr = d.ws.ctr;
-    for (int wd = gwarp; wd < n_words; wd += nwarps) {
-        const uint32_t word = d.ws.x_mask32[wd];
-        if (!word) continue;                                   // warp-uniform
-        const int jb = 2 * wd + (lane >> 4), j = jb * 16 + (lane & 15);
-        const bool listed = (word >> lane) & 1u;
-        int first = 0, deg = 0;
-        if (listed) column_run(d, j, first, deg);
-        merge_column_runs(listed, j, first, deg, lane);
-        emit_tasks(d, false, jb, first, deg, lane, &ctr->n_tasks, &ctr->pad, PUSH_CHUNK, &ctr->n_hubs, d.ws.hubs);
-        first = 0; deg = 0;
-        if ((lane & 15) == 0 && ((word >> lane) & 0xFFFFu)) payload_run(d, jb, first, deg);
-        if (__any_sync(FULL, deg > 0)) emit_tasks(d, false, jb, first, deg, lane, &ctr->n_tasks, &ctr->pad, d.payload_chunk);
-    }
-}
 
 // Dense input (Sections 4.1, 4.3): every warp reads 32 elements, one ballot gives the two
 // 16-bit masks of its two vector blocks.  Also clears the dense output.
@@ -135,6 +113,7 @@ __device__ __forceinline__ bool decode_takes_part(const Device &d, float v) {
 
 template <int DT>
 __global__ void k_xblock_dense(Device d, const void *__restrict__ x, float *__restrict__ y) {
+    pdl_wait();
     pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
     const int64_t padded = (int64_t)((d.nb + 1) / 2) * 32;
@@ -172,29 +151,8 @@ __global__ void k_xblock_dense(Device d, const void *__restrict__ x, float *__re
 }
 
 // ------------------------------------------------------------------------------------------
-// Traversal.  Output goes through `Out`: the sparse path accumulates into the handle's dense
-// accumulator and structural-hit masks; the decode path adds straight into the caller's y.
+// Traversal.
 // ------------------------------------------------------------------------------------------
-struct OutSparse {
-    float *acc;
-    uint8_t *hit8;     // one byte per row: 1 = structurally hit (plain idempotent stores, no atomics)
-    static constexpr bool MASKS = true;
-    static constexpr bool MINPLUS = false;
-};
-struct OutDense {
-    float *acc;
-    uint8_t *hit8;
-    static constexpr bool MASKS = false;
-    static constexpr bool MINPLUS = false;
-};
-// (min, +) semiring: the accumulator holds keys of the smallest sum so far (minplus.cuh)
-struct OutSparseMin {
-    float *acc;
-    uint8_t *hit8;
-    static constexpr bool MASKS = true;
-    static constexpr bool MINPLUS = true;
-};
-
 // One lane owns one hypersparse block (INLINE or COO).  `emit(r, v)` receives the products,
 // already summed per row where the entries of a row are adjacent (COO is stored row-major);
 // `xin` is the x entry of an INLINE block's single column (fetched by the caller in parallel
@@ -279,44 +237,17 @@ __device__ __forceinline__ void warp_flat_coo(int cnt, uint32_t w, uint32_t xm, 
     }
 }
 
-// Structural-hit marking: one byte per output row, set with a plain store.  Stores of the same
-// value to the same byte need no atomic and no read, so hub rows that are hit by thousands of
-// products per call cost nothing extra; the compaction pass packs the bytes into masks.
-__device__ __forceinline__ void mark_rows(uint8_t *hit8, int rb, uint32_t rows16) {
-    uint8_t *base = hit8 + (size_t)rb * 16;
-    while (rows16) {
-        base[__ffs(rows16) - 1] = 1;
-        rows16 &= rows16 - 1;
-    }
+// Structural hits of a pattern block: a count per row instead of a sum.
+template <typename Out>
+__device__ __forceinline__ void mark_rows(Out out, int rb, uint32_t rows16) {
+    for (; rows16; rows16 &= rows16 - 1) out_add(out, (size_t)rb * 16 + __ffs(rows16) - 1, 1.0f);
 }
 
 // Writeback of one block handled outside the shared-memory accumulator: lanes 0..15 own the 16
-// rows; one global atomic and one flag store per touched row.
-template <typename Out>
+// rows; one global atomic per touched row.
+template <int DT, typename Out>
 __device__ __forceinline__ void flush_rows(Out out, int rb, uint32_t hits, float v, int lane) {
-    if (lane < 16 && ((hits >> lane) & 1u)) {
-        atomicAdd(out.acc + (size_t)rb * 16 + lane, v);
-        if (Out::MASKS) out.hit8[(size_t)rb * 16 + lane] = 1;
-    }
-}
-
-// One product of an INLINE element whose row block is a hub (HUB_FLAG): added to one of the
-// HUB_COPIES private accumulators of that row block, picked by the CTA, with an atomic whose
-// reply nobody reads.  The L2 serves atomics on one line one after the other: on an R-MAT
-// matrix one line of the accumulator receives 1-2 % of ALL products, and that queue, not the
-// traversal, set the duration of the push (58 -> 35 us at 10 % x density when the same atomics
-// go to distinct lines).  A private accumulator that nothing touched holds -0.0f: any sum of
-// finite products that are neither zero nor subnormal differs from it in its bits (x + -x is
-// +0 in round-to-nearest), so the fold of the compaction needs no flags.  Products that are
-// zero or subnormal (an atomic may flush them to a signed zero) return false and take the
-// ordinary path.
-template <typename Out>
-__device__ __forceinline__ bool push_private(const Device &d, uint32_t idx, uint32_t aux, float prod) {
-    if (!Out::MASKS || !d.hub_on || !(idx & HUB_FLAG) || !(fabsf(prod) >= 1.17549435e-38f)) return false;
-    const int slot = d.hub_slot[idx & IDX_MASK];
-    if (!DBS_CHK_INDEX(d, slot, d.n_hub_blocks)) return false;
-    atomicAdd(d.hub_acc + (((size_t)(blockIdx.x & (HUB_COPIES - 1)) * d.n_hub_blocks + slot) * 16 + (aux >> 4)), prod);
-    return true;
+    if (lane < 16 && ((hits >> lane) & 1u)) out_add(out, (size_t)rb * 16 + lane, DT != DBSPMSPV_PATTERN ? v : 1.0f);
 }
 
 // Per-warp staging area in shared memory: two stages of view entries for the pull; the push
@@ -438,22 +369,9 @@ __device__ void push_body(const Device &d, Out out, int popc_threshold, float *s
             }
             if (have) {
                 if (type == DBSPMSPV_BLK_INLINE) {
-                    float *row0 = out.acc + (size_t)brow * 16;
-                    // The structural-hit flag is stored only when the atomic returns zero: the first
-                    // product that reaches a row always sees the cleared accumulator, so the flag is
-                    // set once per row instead of once per product (a later zero -- an explicitly
-                    // stored zero, a cancellation -- only repeats the store).  The repeated byte
-                    // stores to the hub rows of a power-law matrix, not the atomics, were what the
-                    // push waited for: 77 -> 57 us at 10 % x density, 326 -> 170 us at 50 %.  (The
-                    // per-block writebacks of mask-based blocks keep the plain atomic and the
-                    // unconditional store: on the stencil the returning atomic cost 7-15 %.)
-                    bool first = false;
                     const uint32_t hit = lane_block<DT>(type, w[u], aux[u], xm, s_x[aux[u] & 15], s_x, pl,
-                                                        [&](int r, float v) { if (!push_private<Out>(d, idx[u], aux[u], v)) first |= atomicAdd(row0 + r, v) == 0.0f; });
-                    // (pattern matrices have no product: they count the hits in the accumulator,
-                    // which the compaction clears like any other, to get the same first-touch test)
-                    if (DT == DBSPMSPV_PATTERN && hit && !push_private<Out>(d, idx[u], aux[u], 1.0f)) first = atomicAdd(row0 + (aux[u] >> 4), 1.0f) == 0.0f;
-                    if (Out::MASKS && hit && first) mark_rows(out.hit8, brow, hit);
+                                                        [&](int r, float v) { out_add(out, (size_t)brow * 16 + r, v); });
+                    if (DT == DBSPMSPV_PATTERN) mark_rows(out, brow, hit);
                 } else if (type == DBSPMSPV_BLK_COO && aux[u] < COO_SERIAL_MAX) {
                     coo_cnt = (int)aux[u] + 1;
                 } else {
@@ -461,16 +379,10 @@ __device__ void push_body(const Device &d, Out out, int popc_threshold, float *s
                 }
             }
             if (__any_sync(FULL, coo_cnt)) {
-                uint32_t *s_hit = reinterpret_cast<uint32_t *>(s_tmp);   // per-owner-lane hit masks
-                s_hit[lane] = 0u;
-                __syncwarp();
                 warp_flat_coo<DT>(coo_cnt, w[u], xm, (uint32_t)brow, 0u, pl, lane,
-                                  [&](uint32_t tag, uint32_t, int r, int c, float a, int owner) {
-                                      if (DT != DBSPMSPV_PATTERN) atomicAdd(out.acc + (size_t)tag * 16 + r, a * s_x[c]);
-                                      if (Out::MASKS) atomicOr(&s_hit[owner], 1u << r);
+                                  [&](uint32_t tag, uint32_t, int r, int c, float a, int) {
+                                      out_add(out, (size_t)tag * 16 + r, DT != DBSPMSPV_PATTERN ? a * s_x[c] : 1.0f);
                                   });
-                __syncwarp();
-                if (Out::MASKS && coo_cnt && s_hit[lane]) mark_rows(out.hit8, brow, s_hit[lane]);
                 __syncwarp();
             }
             // dense vector block and several mask-based blocks in the step: half-warp streaming
@@ -481,8 +393,7 @@ __device__ void push_body(const Device &d, Out out, int popc_threshold, float *s
                 const uint32_t cs = __ballot_sync(FULL, mk);
                 if (__popc(cs) >= HEAVY_LANE_MIN) {
                     auto emit = [&](int erb, int erow, float esum) {
-                        atomicAdd(out.acc + (size_t)erb * 16 + erow, esum);
-                        if (Out::MASKS) out.hit8[(size_t)erb * 16 + erow] = 1;
+                        out_add(out, (size_t)erb * 16 + erow, esum);
                     };
                     const uint32_t rows = __ballot_sync(FULL, mk && is_row_major(type));
                     const uint32_t tagged = (idx[u] & ~IDX_MASK) | (uint32_t)jb;     // class bits + the task's column block
@@ -512,8 +423,7 @@ __device__ void push_body(const Device &d, Out out, int popc_threshold, float *s
                     }
                     for (uint32_t hh = hits; hh; hh &= hh - 1) {
                         const int r = __ffs(hh) - 1;
-                        if (DT != DBSPMSPV_PATTERN) atomicAdd(out.acc + (size_t)brow * 16 + r, acc[r * LANE_ACC_STRIDE]);
-                        if (Out::MASKS) out.hit8[(size_t)brow * 16 + r] = 1;
+                        out_add(out, (size_t)brow * 16 + r, DT != DBSPMSPV_PATTERN ? acc[r * LANE_ACC_STRIDE] : 1.0f);
                     }
                 }
                 __syncwarp();
@@ -532,7 +442,7 @@ __device__ void push_body(const Device &d, Out out, int popc_threshold, float *s
                 float sum = 0.f;
                 if (DT == DBSPMSPV_PATTERN) hits = warp_block_bool<DT>(btype, blk, nnz, xm, lane);
                 else sum = warp_block<DT>(btype, blk, nnz, xm, s_x, s_tmp, lane, popc_threshold, hits);
-                flush_rows(out, bbrow, hits, sum, lane);
+                flush_rows<DT>(out, bbrow, hits, sum, lane);
             }
         }
         __syncwarp();
@@ -656,13 +566,12 @@ __device__ void pull_body(const Device &d, Out out, int popc_threshold, float *s
                     __syncwarp();
                     if (lane < 16) {
                         if ((hit >> lane) & 1u) {
+                            float t = DT != DBSPMSPV_PATTERN ? 0.f : 1.0f;
                             if (DT != DBSPMSPV_PATTERN) {
-                                float t = 0.f;
 #pragma unroll
                                 for (int k = 0; k < SY_COPIES; ++k) { t += s_y[k * 16 + lane]; s_y[k * 16 + lane] = 0.f; }
-                                atomicAdd(out.acc + (size_t)cur_rb * 16 + lane, t);
                             }
-                            if (Out::MASKS) out.hit8[(size_t)cur_rb * 16 + lane] = 1;
+                            out_add(out, (size_t)cur_rb * 16 + lane, t);
                         }
                     }
                     hit = 0;
@@ -678,8 +587,7 @@ __device__ void pull_body(const Device &d, Out out, int popc_threshold, float *s
                         if (DT != DBSPMSPV_PATTERN) atomicAdd(&my_y[r], v);
                         hit |= 1u << r;
                     } else {
-                        if (DT != DBSPMSPV_PATTERN) atomicAdd(out.acc + (size_t)rb * 16 + r, v);
-                        if (Out::MASKS) out.hit8[(size_t)rb * 16 + r] = 1;
+                        out_add(out, (size_t)rb * 16 + r, DT != DBSPMSPV_PATTERN ? v : 1.0f);
                     }
                 }
                 const bool other = have && !inl;
@@ -697,17 +605,10 @@ __device__ void pull_body(const Device &d, Out out, int popc_threshold, float *s
                     }
                 }
                 if (__any_sync(FULL, coo_cnt)) {
-                    uint32_t *s_hit = reinterpret_cast<uint32_t *>(s_tmp);   // per-owner-lane hit masks
-                    s_hit[lane] = 0u;
-                    __syncwarp();
                     warp_flat_coo<DT>(coo_cnt, w[u], xm, (uint32_t)rb, (uint32_t)bcol_l, d.payload, lane,
-                                      [&](uint32_t trb, uint32_t tcol, int r, int c, float a, int owner) {
-                                          if (DT != DBSPMSPV_PATTERN)
-                                              atomicAdd(out.acc + (size_t)trb * 16 + r, a * d.ws.x_dense[(size_t)tcol * 16 + c]);
-                                          if (Out::MASKS) atomicOr(&s_hit[owner], 1u << r);
+                                      [&](uint32_t trb, uint32_t tcol, int r, int c, float a, int) {
+                                          out_add(out, (size_t)trb * 16 + r, DT != DBSPMSPV_PATTERN ? a * d.ws.x_dense[(size_t)tcol * 16 + c] : 1.0f);
                                       });
-                    __syncwarp();
-                    if (Out::MASKS && coo_cnt && s_hit[lane]) mark_rows(out.hit8, rb, s_hit[lane]);
                     __syncwarp();
                 }
                 // runs of mask-based blocks (pruned layers, banded matrices): half-warp streaming form
@@ -720,8 +621,7 @@ __device__ void pull_body(const Device &d, Out out, int popc_threshold, float *s
                                 atomicAdd(&my_y[erow], esum);
                                 hit |= 1u << erow;
                             } else {
-                                atomicAdd(out.acc + (size_t)erb * 16 + erow, esum);
-                                if (Out::MASKS) out.hit8[(size_t)erb * 16 + erow] = 1;
+                                out_add(out, (size_t)erb * 16 + erow, esum);
                             }
                         };
                         const uint32_t rows = __ballot_sync(FULL, mk && is_row_major(type));
@@ -765,8 +665,7 @@ __device__ void pull_body(const Device &d, Out out, int popc_threshold, float *s
                     if (lane_form && !in_cur) {
                         for (uint32_t hh = hits; hh; hh &= hh - 1) {
                             const int r = __ffs(hh) - 1;
-                            if (DT != DBSPMSPV_PATTERN) atomicAdd(out.acc + (size_t)rb * 16 + r, acc[r * LANE_ACC_STRIDE]);
-                            if (Out::MASKS) out.hit8[(size_t)rb * 16 + r] = 1;
+                            out_add(out, (size_t)rb * 16 + r, DT != DBSPMSPV_PATTERN ? acc[r * LANE_ACC_STRIDE] : 1.0f);
                         }
                     }
                     __syncwarp();
@@ -793,7 +692,7 @@ __device__ void pull_body(const Device &d, Out out, int popc_threshold, float *s
                         __syncwarp();
                         sum = warp_block<DT>(btype, blk, nnz, bxm, s_x, s_tmp, lane, popc_threshold, hits);
                     }
-                    flush_rows(out, brb, hits, sum, lane);
+                    flush_rows<DT>(out, brb, hits, sum, lane);
                 }
             }
         }
@@ -802,13 +701,12 @@ __device__ void pull_body(const Device &d, Out out, int popc_threshold, float *s
         __syncwarp();
         if (lane < 16) {
             if ((hit >> lane) & 1u) {
+                float t = DT != DBSPMSPV_PATTERN ? 0.f : 1.0f;
                 if (DT != DBSPMSPV_PATTERN) {
-                    float t = 0.f;
 #pragma unroll
                     for (int k = 0; k < SY_COPIES; ++k) { t += s_y[k * 16 + lane]; s_y[k * 16 + lane] = 0.f; }
-                    atomicAdd(out.acc + (size_t)cur_rb * 16 + lane, t);
                 }
-                if (Out::MASKS) out.hit8[(size_t)cur_rb * 16 + lane] = 1;
+                out_add(out, (size_t)cur_rb * 16 + lane, t);
             }
         }
         __syncwarp();
@@ -1268,6 +1166,8 @@ k_decode_fused(Device d, const void *__restrict__ x, float *__restrict__ y, floa
     uint16_t *s_xm = reinterpret_cast<uint16_t *>(s_dyn + lay.xm_off);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint4 *slot = reinterpret_cast<uint4 *>(s_dyn + lay.slot_off + tid * wc_slot_bytes(wc_ilp(NW)));
+    pdl_wait();
+    pdl_launch_dependents();
     if (tid == 0) { s_cnt[0] = 0; s_cnt[1] = 0; }
     if (tid < 16) s_y[tid] = 0.f;
     __syncthreads();
@@ -1640,163 +1540,180 @@ namespace dbs {
 // sorted.  Pass 1 counts per tile, pass 2 places the entries, clears the accumulator and the
 // masks it read, clears the vector-block state of this call's x, and rolls the counters over.
 // ------------------------------------------------------------------------------------------
-// Fold of the private accumulators of one hub row block (see push_private), by a whole warp:
-// every lane takes four rows of two copies, a shuffle tree adds the copies up in a fixed
-// order, the totals go into the accumulator proper (no atomics: every push has ended) and the
-// rows that any copy touched get their structural-hit flag; touched copies are put back to
-// HUB_CLEAR.  A kernel of its own, one warp per hub row block, between the traversal and the
-// compaction: hub row blocks are neighbours (the low vertex numbers of an R-MAT graph), so a
-// fold inside the compaction, by the warp that owns the rows, took 40 folds one after the other.
-static_assert(HUB_COPIES % 8 == 0, "a warp folds eight copies per step");
-__device__ __forceinline__ void fold_hub_block(const Device &d, int rb, int slot, int lane) {
-    const int q = lane & 3;
-    float4 tot = make_float4(0.f, 0.f, 0.f, 0.f);
-    uint32_t touched = 0u;
-#pragma unroll
-    for (int k = 0; k < HUB_COPIES / 8; ++k) {
-        const int c = (lane >> 2) + 8 * k;
-        float4 *p = reinterpret_cast<float4 *>(d.hub_acc + ((size_t)c * d.n_hub_blocks + slot) * 16) + q;
-        const float4 v = __ldcg(p);
-        const uint32_t t = (__float_as_uint(v.x) != HUB_CLEAR ? 1u : 0u) | (__float_as_uint(v.y) != HUB_CLEAR ? 2u : 0u) |
-                           (__float_as_uint(v.z) != HUB_CLEAR ? 4u : 0u) | (__float_as_uint(v.w) != HUB_CLEAR ? 8u : 0u);
-        // (an untouched -0.0f adds nothing)
-        tot.x += v.x; tot.y += v.y; tot.z += v.z; tot.w += v.w;
-        if (t) { const float z = __uint_as_float(HUB_CLEAR); *p = make_float4(z, z, z, z); }
-        touched |= t;
-    }
-#pragma unroll
-    for (int o = 4; o < 32; o <<= 1) {
-        tot.x += __shfl_xor_sync(FULL, tot.x, o); tot.y += __shfl_xor_sync(FULL, tot.y, o);
-        tot.z += __shfl_xor_sync(FULL, tot.z, o); tot.w += __shfl_xor_sync(FULL, tot.w, o);
-        touched |= __shfl_xor_sync(FULL, touched, o);
-    }
-    if (lane < 4 && touched) {
-        float *a = d.ws.y_acc + (size_t)rb * 16 + 4 * q;
-        uint8_t *f = d.ws.y_hit8 + (size_t)rb * 16 + 4 * q;
-        if (touched & 1u) { a[0] += tot.x; f[0] = 1; }
-        if (touched & 2u) { a[1] += tot.y; f[1] = 1; }
-        if (touched & 4u) { a[2] += tot.z; f[2] = 1; }
-        if (touched & 8u) { a[3] += tot.w; f[3] = 1; }
-    }
-}
 
-__global__ void __launch_bounds__(128) k_fold_hubs(Device d) {
-    pdl_wait();
-    pdl_launch_dependents();
-    const int slot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (slot < d.n_hub_blocks && DBS_CHK_INDEX(d, d.hub_rb[slot], d.mb)) fold_hub_block(d, d.hub_rb[slot], slot, threadIdx.x & 31);
-}
-
-__global__ void __launch_bounds__(TILE_WORDS) k_compact_count(Device d, int parity, const uint32_t *__restrict__ row_mask, int complement) {
-    __shared__ int s_red[TILE_WORDS / 32];
-    pdl_wait();
-    pdl_launch_dependents();
-    const int n_words = (d.mb + 1) / 2;
-    const int wi = blockIdx.x * TILE_WORDS + threadIdx.x;
-    int c = 0;
-    if (wi < n_words) {
-        // 32 row flags (bytes, 0 or 1) -> one mask word; the flags are cleared for the next call
-        uint4 *f4 = reinterpret_cast<uint4 *>(d.ws.y_hit8 + (size_t)wi * 32);
-        const uint4 a = f4[0], b = f4[1];
-        const uint32_t v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        uint32_t word = 0;
+// Fold of the private accumulators of eight rows of a hub row block into the accumulator proper, by the
+// thread that owns the rows: the copies are fetched four at a time (all at once took the kernel to 128
+// registers, two thread blocks per SM) and added up in a fixed order; (min, +)
+// words are folded by their maximum.  Touched copies are put back to HUB_CLEAR.
+__device__ __forceinline__ void fold_hub_rows(const Device &d, int slot, int half, int minplus, uint32_t (&acc)[8]) {
+#pragma unroll 1
+    for (int c0 = 0; c0 < d.hub_on; c0 += 4) {
+        uint4 *p = reinterpret_cast<uint4 *>(d.hub_acc + ((size_t)c0 * d.n_hub_blocks + slot) * 16 + 8 * half);
+        const size_t next = (size_t)d.n_hub_blocks * 4;          // 16-byte words from copy to copy
+        uint4 v[4][2];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) word |= (((v[q] & 0x01010101u) * 0x01020408u) >> 24 & 0xFu) << (4 * q);
-        if (word) {
-            f4[0] = make_uint4(0u, 0u, 0u, 0u);
-            f4[1] = make_uint4(0u, 0u, 0u, 0u);
+        for (int k = 0; k < 4; ++k) { v[k][0] = __ldcg(p + k * next); v[k][1] = __ldcg(p + k * next + 1); }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t w[8] = {v[k][0].x, v[k][0].y, v[k][0].z, v[k][0].w, v[k][1].x, v[k][1].y, v[k][1].z, v[k][1].w};
+            uint32_t touched = 0u;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                touched |= w[r] ^ HUB_CLEAR;
+                // (an untouched -0.0f adds nothing)
+                if (minplus) acc[r] = (uint32_t)max((int)acc[r], (int)w[r]);
+                else acc[r] = __float_as_uint(__uint_as_float(acc[r]) + __uint_as_float(w[r]));
+            }
+            if (touched) {
+                p[k * next] = make_uint4(HUB_CLEAR, HUB_CLEAR, HUB_CLEAR, HUB_CLEAR);
+                p[k * next + 1] = make_uint4(HUB_CLEAR, HUB_CLEAR, HUB_CLEAR, HUB_CLEAR);
+            }
         }
-        d.ws.y_mask32[wi] = word;
-        // (an output mask drops rows from y; their accumulator entries are still cleared by pass 2)
-        c = __popc(row_mask ? word & (complement ? ~row_mask[wi] : row_mask[wi]) : word);
-    }
-    c = __reduce_add_sync(FULL, c);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int t = 0;
-        for (int k = 0; k < TILE_WORDS / 32; ++k) t += s_red[k];
-        d.ws.tile_count[blockIdx.x] = t;
-        // totals of groups of 32 tiles, so that pass 2 adds up a few dozen numbers per tile
-        // instead of one per earlier tile (all thread blocks reading the same few lines of
-        // counts was most of pass 2 on a large m: 2,100 tiles -> 2.2 M loads on 64 lines)
-        if (t) atomicAdd(d.ws.tile_group + parity * d.ws.n_tile_groups + (blockIdx.x >> 5), t);
     }
 }
 
-__global__ void __launch_bounds__(CMP_TPB) k_compact_write(Device d, int32_t *__restrict__ y_idx, float *__restrict__ y_val,
-                                                           int64_t y_capacity, int32_t *__restrict__ y_nnz, int boolean,
-                                                           const int32_t *__restrict__ x_idx, int32_t nnz_x, int clear_all, int parity,
-                                                           const uint32_t *__restrict__ row_mask, int complement) {
-    __shared__ int s_before[CMP_TPB / 32], s_cnt[CMP_TPB / 32];
-    __shared__ int32_t s_oidx[TILE_WORDS * 32];
-    __shared__ float s_oval[TILE_WORDS * 32];
-    const int n_tiles = d.ws.n_tiles;
+// What the last kernel of a call clears of the vector-block state of its x.
+enum { CLEAR_MASKS = 1, CLEAR_DENSE = 2, CLEAR_SWEEP = 4 };   // SWEEP: whole arrays instead of entry by entry
+
+constexpr int TILE_WAIT_LIMIT = 1 << 20;
+constexpr int FINISH_PARITY = 1 << 30;
+constexpr int FINISH_GROUP = 32;          // tiles per group
+__device__ __forceinline__ unsigned long long load_relaxed64(const unsigned long long *p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int load_relaxed32(const int32_t *p) {
+    int v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// Result entries in all tiles before `tile`, by one warp (see k_finish): the sums of the complete groups before its
+// own, the status words of the tiles before it in its group.  -1 when a wait ran out.
+__device__ __forceinline__ int entries_before(const Device &d, int tile, int parity, int lane) {
+    const int g = tile / FINISH_GROUP, r = tile % FINISH_GROUP;
+    const unsigned long long *groups = d.ws.tile_group + parity * d.ws.n_tile_groups;
+    int sum = 0;
+    bool ok = true;
+    if (lane < r) {
+        int v = 0, i = 0;
+        do v = load_relaxed32(d.ws.tile_status + g * FINISH_GROUP + lane); while ((v & 1) != parity && ++i < TILE_WAIT_LIMIT);
+        ok = i < TILE_WAIT_LIMIT;
+        sum = v >> 1;
+    }
+    for (int k = lane; k < g; k += 32) {
+        unsigned long long v = 0;
+        int i = 0;
+        do v = load_relaxed64(groups + k); while ((int)(v >> 32) != FINISH_GROUP && ++i < TILE_WAIT_LIMIT);
+        ok = ok && i < TILE_WAIT_LIMIT;
+        sum += (int)(uint32_t)v;
+    }
+    sum = __reduce_add_sync(FULL, sum);
+    return __all_sync(FULL, ok) ? sum : -1;
+}
+
+// The end of a call in one kernel: which rows were hit (see ACC_CLEAR), their order, y, and everything
+// put back.  A thread block takes a tile of 2048 rows, a thread eight of them in two 16-byte loads that
+// stay in registers; the tile publishes its count -- in a status word and, added up, in the word of its group of
+// 32 tiles -- and one warp adds up the words of the groups and tiles before it (no chain from tile to
+// tile), so y comes out sorted.  (With every thread polling a word of every earlier tile the polls
+// queued up on the lines that the counts had to get into: 16 us.)
+// A tile only waits for tiles with a lower ticket, and a ticket is taken when the thread block starts:
+// the blocks it waits for are running.  The status of a tile carries the parity of the call
+// (every call rewrites every tile), so nothing has to be reset.
+// It replaces a counting pass and a placing pass: as two kernels they were two waits for the
+// predecessor's last store and the accumulator was fetched twice (9.3 us exposed behind the traversal on a
+// million rows; 5 here).
+__global__ void __launch_bounds__(CMP_TPB, 5) k_finish(Device d, int32_t *__restrict__ y_idx, float *__restrict__ y_val,
+                                                    int64_t y_capacity, int32_t *__restrict__ y_nnz, int boolean,
+                                                    const int32_t *__restrict__ x_idx, int32_t nnz_x, int clear, int fold,
+                                                    const uint32_t *__restrict__ row_mask, int complement) {
+    __shared__ int s_cnt[CMP_TPB / 32], s_ticket, s_parity, s_base;
+    __shared__ int32_t s_oidx[CMP_TPB * 8];
+    __shared__ float s_oval[CMP_TPB * 8];
+    Counters *ctr = d.ws.ctr;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    pdl_wait();
-    // The kernel is a chain of dependent loads, not bandwidth: everything that can be fetched
-    // up front is fetched before the first barrier.
+    // Ticket and parity of the call come from one word.  They are taken before the wait for the predecessor: the kernels in front of this
+    // one in the call were let go only after the call before had ended.  (An empty x has no such kernel.)
+    if (nnz_x == 0) pdl_wait();
+    if (threadIdx.x == 0) { const int w = atomicAdd(&ctr->finish_ticket, 1); s_ticket = w & (FINISH_PARITY - 1); s_parity = w & FINISH_PARITY ? 1 : 0; }
+    __syncthreads();
+    const int tile = s_ticket, parity = s_parity, n_tiles = d.ws.n_tiles;
     const int stride = gridDim.x * CMP_TPB;
-    const int k0 = blockIdx.x * CMP_TPB + threadIdx.x;
-    const int j0 = (!clear_all && k0 < nnz_x) ? x_idx[k0] : -1;
-    if ((int)blockIdx.x < n_tiles) {
-        const int n_words = (d.mb + 1) / 2;
-        // every thread owns 8 consecutive rows (a quarter of a mask word)
-        const int wi = blockIdx.x * TILE_WORDS + (threadIdx.x >> 2);
-        const int sub = threadIdx.x & 3;
-        const uint32_t word = wi < n_words ? d.ws.y_mask32[wi] : 0u;
-        int before = 0;               // entries in all earlier tiles: whole groups of 32, then the tiles of this group
-        {
-            const int g = (int)blockIdx.x >> 5, r = (int)blockIdx.x & 31;
-            const int32_t *grp = d.ws.tile_group + parity * d.ws.n_tile_groups;
-            for (int k = threadIdx.x; k < g + r; k += CMP_TPB) before += k < g ? grp[k] : d.ws.tile_count[g * 32 + (k - g)];
-            // the group totals of the other parity served the call before: cleared for the next one
-            if (blockIdx.x == 0)
-                for (int k = threadIdx.x; k < d.ws.n_tile_groups; k += CMP_TPB) d.ws.tile_group[(parity ^ 1) * d.ws.n_tile_groups + k] = 0;
+    const int bi = tile * CMP_TPB + threadIdx.x;      // byte of the hit mask: rows 8 bi .. 8 bi + 7
+    const int j0 = (!(clear & CLEAR_SWEEP) && bi < nnz_x) ? x_idx[bi] : -1;      // (x is the caller's: nothing of this call writes it)
+    pdl_wait();
+    pdl_launch_dependents();
+    if (tile < n_tiles) {
+        const int n_bytes = (d.mb + 1) / 2 * 4;
+        uint8_t *mask8 = reinterpret_cast<uint8_t *>(d.ws.y_mask32);
+        uint32_t hits = 0, keep = 0xFFu;                // rows to clear; rows that may go to y
+        uint32_t v[8];
+        if (bi < n_bytes) {
+            uint4 *acc4 = reinterpret_cast<uint4 *>(d.ws.y_acc + (size_t)bi * 8);
+            const uint4 a = __ldcg(acc4), b = __ldcg(acc4 + 1);
+            const uint32_t flags = mask8[bi];
+            if (row_mask) keep = reinterpret_cast<const uint8_t *>(row_mask)[bi] ^ (complement ? 0xFFu : 0u);
+            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+            hits = flags;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) hits |= (v[r] != ACC_CLEAR ? 1u : 0u) << r;
+            if (hits) {
+                acc4[0] = make_uint4(ACC_CLEAR, ACC_CLEAR, ACC_CLEAR, ACC_CLEAR);
+                acc4[1] = make_uint4(ACC_CLEAR, ACC_CLEAR, ACC_CLEAR, ACC_CLEAR);
+            }
+            if (flags) mask8[bi] = 0;
+            if (fold) {
+                const int slot = d.hub_slot[bi >> 1];
+                if (slot != HUB_NONE && DBS_CHK_INDEX(d, slot, d.n_hub_blocks)) {
+                    fold_hub_rows(d, slot, bi & 1, fold == 2, v);
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) hits |= (v[r] != ACC_CLEAR ? 1u : 0u) << r;
+                }
+            }
         }
-        const uint32_t keep = row_mask && wi < n_words ? (complement ? ~row_mask[wi] : row_mask[wi]) : 0xFFFFFFFFu;
-        const uint32_t hits = (word >> (8 * sub)) & 0xFFu;    // rows to clear
-        const uint32_t bits = hits & (keep >> (8 * sub));     // rows that go to y
+        const uint32_t bits = hits & keep;
         const int c = __popc(bits);
-        const int row0 = wi * 32 + sub * 8;
-        float4 v4[2];
-        if (hits) {                   // two independent 16-byte loads fetch the 8 accumulator entries
-            float4 *acc4 = reinterpret_cast<float4 *>(d.ws.y_acc + row0);
-            v4[0] = acc4[0]; v4[1] = acc4[1];
-            acc4[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-            acc4[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
         int incl = c;
+#pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(FULL, incl, o);
+            const int t = __shfl_up_sync(FULL, incl, o);
             if (lane >= o) incl += t;
         }
-        before = __reduce_add_sync(FULL, before);
         if (lane == 31) s_cnt[warp] = incl;
-        if (lane == 0) s_before[warp] = before;
         __syncthreads();
-        int base = 0, local = 0, tile_total = 0;
+        int local = 0, tile_total = 0;
 #pragma unroll
         for (int k = 0; k < CMP_TPB / 32; ++k) {
-            base += s_before[k];
             if (k < warp) local += s_cnt[k];
             tile_total += s_cnt[k];
         }
-        // the tile's entries are gathered in shared memory, then written out in whole lines
+        if (threadIdx.x == 0) {
+            asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(d.ws.tile_status + tile), "r"(tile_total * 2 + parity) : "memory");
+            atomicAdd(d.ws.tile_group + parity * d.ws.n_tile_groups + tile / FINISH_GROUP, (1ull << 32) + (unsigned)tile_total);
+        }
+        // (the group words of the other parity served the call before: cleared for the next one)
+        if (tile == 0)
+            for (int k = threadIdx.x; k < d.ws.n_tile_groups; k += CMP_TPB) d.ws.tile_group[(parity ^ 1) * d.ws.n_tile_groups + k] = 0ull;
+        // the tile's entries are gathered in shared memory (while the other tiles' counts arrive), then written out in whole lines
         if (bits) {
-            const float *v = reinterpret_cast<const float *>(v4);
             int pos = local + incl - c;
 #pragma unroll
             for (int bit = 0; bit < 8; ++bit) {
                 if ((bits >> bit) & 1u) {
-                    s_oidx[pos] = row0 + bit;
-                    // boolean 1: a Boolean result; 2: the accumulator holds (min, +) keys
-                    s_oval[pos] = boolean == 1 ? 1.0f : boolean == 2 ? minplus_value(__float_as_uint(v[bit])) : v[bit];
+                    s_oidx[pos] = bi * 8 + bit;
+                    // boolean 1: a Boolean result; 2: the accumulator holds (min, +) words; else a sum (a row of -0 products is 0)
+                    s_oval[pos] = boolean == 1 ? 1.0f : boolean == 2 ? minplus_of_word(v[bit]) : __uint_as_float(v[bit]) + 0.0f;
                     ++pos;
                 }
             }
         }
+        if (warp == 0) {
+            const int before = entries_before(d, tile, parity, lane);
+            if (lane == 0) { s_base = before; if (before < 0) ctr->status = DBSPMSPV_ERR_TIMEOUT; }
+        }
         __syncthreads();
+        const int base = max(s_base, 0);
         for (int k = threadIdx.x; k < tile_total; k += CMP_TPB) {
             const int64_t pos = (int64_t)base + k;
             if (pos < y_capacity) {
@@ -1804,40 +1721,46 @@ __global__ void __launch_bounds__(CMP_TPB) k_compact_write(Device d, int32_t *__
                 if (y_val) y_val[pos] = s_oval[k];
             }
         }
-        if ((int)blockIdx.x == n_tiles - 1 && threadIdx.x == 0) {
-            Counters *c2 = d.ws.ctr;
+        if (tile == n_tiles - 1 && threadIdx.x == 0) {
             const int total = base + tile_total;
             *y_nnz = total;
-            if (total > y_capacity) c2->status = DBSPMSPV_ERR_CAPACITY;
-            c2->last_y_nnz = total;
-            c2->last_n_nzblk = c2->n_nzblk;
-            c2->last_n_tasks = c2->n_tasks;
-            c2->last_path = c2->path;
-            c2->n_nzblk = 0;
-            c2->n_tasks = 0;
-            c2->n_hubs = 0;
+            if (total > y_capacity) ctr->status = DBSPMSPV_ERR_CAPACITY;
+            ctr->last_y_nnz = total;
+            ctr->last_n_nzblk = ctr->n_nzblk;
+            ctr->last_n_tasks = ctr->n_tasks;
+            ctr->last_path = ctr->path;
+            ctr->n_nzblk = 0;
+            ctr->n_tasks = 0;
+            ctr->n_hubs = 0;
+            ctr->n_long = 0;
         }
     }
+    // the block with the last ticket: all tickets are taken
+    if (tile == (int)gridDim.x - 1 && threadIdx.x == 0) ctr->finish_ticket = parity ? 0 : FINISH_PARITY;
     // vector-block state of this call's x: clear the masks and put the "not listed" marker back
     // -- entry by entry, or, for an x that lists a good part of all columns, by streaming over
-    // the whole dense copy (full-line stores instead of scattered 4-byte ones)
-    if (clear_all) {
+    // the whole arrays (full-line stores instead of scattered 4-byte ones)
+    if (clear & CLEAR_SWEEP) {
         const int n_words = (d.nb + 1) / 2;
-        const uint32_t mk = X_ABSENT;
-        uint4 *xd4 = reinterpret_cast<uint4 *>(d.ws.x_dense);
-        for (int k = k0; k < n_words * 8; k += stride) xd4[k] = make_uint4(mk, mk, mk, mk);
-        for (int k = k0; k < n_words; k += stride) d.ws.x_mask32[k] = 0u;
+        if (clear & CLEAR_DENSE) {
+            uint4 *xd4 = reinterpret_cast<uint4 *>(d.ws.x_dense);
+            for (int k = bi; k < n_words * 8; k += stride) xd4[k] = make_uint4(X_ABSENT, X_ABSENT, X_ABSENT, X_ABSENT);
+        }
+        for (int k = bi; k < n_words; k += stride) d.ws.x_mask32[k] = 0u;
         return;
     }
-    if (j0 >= 0 && j0 < d.n) { d.ws.x_mask32[j0 >> 5] = 0u; d.ws.x_dense[j0] = __uint_as_float(X_ABSENT); }
-    for (int k = k0 + stride; k < nnz_x; k += stride) {
-        const int j = x_idx[k];
-        if (j >= 0 && j < d.n) { d.ws.x_mask32[j >> 5] = 0u; d.ws.x_dense[j] = __uint_as_float(X_ABSENT); }
-    }
+    auto drop = [&](int j) {
+        if (j < 0 || j >= d.n) return;
+        d.ws.x_mask32[j >> 5] = 0u;
+        if (clear & CLEAR_DENSE) d.ws.x_dense[j] = __uint_as_float(X_ABSENT);
+    };
+    drop(j0);
+    for (int k = bi + stride; k < nnz_x; k += stride) drop(x_idx[k]);
 }
 
 __global__ void k_decode_cleanup(Device d) {
     pdl_wait();
+    pdl_launch_dependents();
     const int n_words = (d.nb + 1) / 2;
     const int stride = gridDim.x * blockDim.x;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n_words; k += stride) d.ws.x_mask32[k] = 0u;
@@ -1868,6 +1791,8 @@ __global__ void k_wait_probe(Device d, int max_tries) {
 }
 
 __global__ void k_fill_u32(uint32_t *p, int64_t n, uint32_t v) {
+    pdl_wait();
+    pdl_launch_dependents();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = v;
 }
 
@@ -1961,11 +1886,11 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     };
     const size_t zwords = xwords > ywords ? xwords : ywords;
     const size_t o_xd = carve(xwords * 32 * sizeof(float)), o_yacc = carve(ywords * 32 * sizeof(float)),
-                 o_hit = carve(ywords * 32), o_tasks = carve((size_t)ws.task_capacity * sizeof(*ws.tasks)),
+                 o_long = carve((size_t)d.long_cap * sizeof(*ws.long_runs)), o_tasks = carve((size_t)ws.task_capacity * sizeof(*ws.tasks)),
                  o_xm = carve(xwords * 4), o_ym = carve(ywords * 4), o_zm = carve(zwords * 4),
                  o_words = carve(4 * zwords * sizeof(*ws.bfs_words)), o_vis = carve((d.m == d.n ? ywords : 1) * 4),
-                 o_hubs = carve((size_t)3 * HUB_CAP * sizeof(*ws.hubs)), o_tile = carve((size_t)ws.n_tiles * sizeof(*ws.tile_count)),
-                 o_group = carve((size_t)2 * ((ws.n_tiles + 31) / 32) * sizeof(*ws.tile_group)),
+                 o_hubs = carve((size_t)3 * HUB_CAP * sizeof(*ws.hubs)), o_tile = carve((size_t)ws.n_tiles * sizeof(*ws.tile_status)),
+                 o_group = carve((size_t)2 * ((ws.n_tiles + FINISH_GROUP - 1) / FINISH_GROUP) * sizeof(*ws.tile_group)),
                  o_ctr = carve(sizeof(*ws.ctr));
     void *arena = nullptr;
     if (cudaMalloc(&arena, off) != cudaSuccess) return DBSPMSPV_ERR_ALLOC;
@@ -1974,7 +1899,7 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     uint8_t *base = static_cast<uint8_t *>(arena);
     ws.x_dense = reinterpret_cast<decltype(ws.x_dense)>(base + o_xd);
     ws.y_acc = reinterpret_cast<decltype(ws.y_acc)>(base + o_yacc);
-    ws.y_hit8 = reinterpret_cast<decltype(ws.y_hit8)>(base + o_hit);
+    ws.long_runs = reinterpret_cast<decltype(ws.long_runs)>(base + o_long);
     ws.tasks = reinterpret_cast<decltype(ws.tasks)>(base + o_tasks);
     ws.x_mask32 = reinterpret_cast<decltype(ws.x_mask32)>(base + o_xm);
     ws.y_mask32 = reinterpret_cast<decltype(ws.y_mask32)>(base + o_ym);
@@ -1983,16 +1908,19 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     ws.bfs_words_stride = (int32_t)zwords;
     ws.visited32 = reinterpret_cast<decltype(ws.visited32)>(base + o_vis);
     ws.hubs = reinterpret_cast<decltype(ws.hubs)>(base + o_hubs);
-    ws.tile_count = reinterpret_cast<decltype(ws.tile_count)>(base + o_tile);
+    ws.tile_status = reinterpret_cast<decltype(ws.tile_status)>(base + o_tile);
     ws.tile_group = reinterpret_cast<decltype(ws.tile_group)>(base + o_group);
-    ws.n_tile_groups = (ws.n_tiles + 31) / 32;
+    ws.n_tile_groups = (ws.n_tiles + FINISH_GROUP - 1) / FINISH_GROUP;
     ws.ctr = reinterpret_cast<decltype(ws.ctr)>(base + o_ctr);
     total = (int64_t)off;
     h->stats.workspace_bytes = total;
+    // (status words of parity 1: the first call waits for words of parity 0)
+    if (cudaMemset(ws.tile_status, 0xFF, (size_t)ws.n_tiles * sizeof(*ws.tile_status)) != cudaSuccess) return DBSPMSPV_ERR_CUDA;
     if (cudaMemset(ws.x_dense, 0xFF, xwords * 32 * sizeof(float)) != cudaSuccess) return DBSPMSPV_ERR_CUDA;
     {   // 0xFFFFFFFF -> the marker pattern 0x7FFFFFFF needs a kernel; a tiny fill does it
         uint32_t *p = reinterpret_cast<uint32_t *>(ws.x_dense);
         k_fill_u32<<<256, 256>>>(p, (int64_t)xwords * 32, X_ABSENT);
+        k_fill_u32<<<256, 256>>>(reinterpret_cast<uint32_t *>(ws.y_acc), (int64_t)ywords * 32, ACC_CLEAR);
         if (cudaDeviceSynchronize() != cudaSuccess) return DBSPMSPV_ERR_CUDA;
     }
     // events for the optional kernel timing are made here so that run-time calls create nothing
@@ -2018,65 +1946,72 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
             return submit_calls(h, calls, st);
         }
     }
-    // x lists a quarter of the columns or more: a pull is likely (on hypersparse matrices), so
-    // the worklist is built afterwards from the masks, and only if the selector does choose the push
-    const bool minplus = semiring == DBSPMSPV_MIN_PLUS;
-    // (min, +) pulls only with the streaming kernel of hypersparse valued handles
-    const bool minplus_pull = minplus && !h->heavy_stage && DT != DBSPMSPV_PATTERN;
-    const bool late_emit = (!minplus || minplus_pull) && !h->heavy_stage && h->ropts.force_path != DBSPMSPV_PATH_PUSH && (int64_t)nnz_x * 4 >= d.n;
+    const bool minplus = semiring == DBSPMSPV_MIN_PLUS, boolean = semiring == DBSPMSPV_OR_AND || (DT == DBSPMSPV_PATTERN && !minplus);
     const void *xv = semiring == DBSPMSPV_OR_AND ? nullptr : x_val;
-    if (nnz_x > 0) {
-        const int g = (nnz_x + XB_TPB - 1) / XB_TPB;
-        if (late_emit) {
-            calls.add(k_xblock_sparse<DT, false>, g, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
-            int ge = ((d.nb + 1) / 2 + 7) / 8;
-            if (ge > 8 * h->sm_count) ge = 8 * h->sm_count;
-            calls.add(k_emit_from_masks, ge, 256, 0, true, d, h->ropts.th3, h->ropts.force_path);
-        } else {
-            calls.add(k_xblock_sparse<DT, true>, g, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
+    const bool any = nnz_x > 0 && d.n_entries > 0;
+    const int fp = h->ropts.force_path;
+    int clear = CLEAR_MASKS | CLEAR_DENSE;
+    h->d.hub_on = 0;
+    if (!h->heavy_stage) {
+        // Hypersparse handles: direct push, pull by the streaming kernel.  (min, +) pulls only on valued handles.
+        const bool may_pull = (!minplus || DT != DBSPMSPV_PATTERN) && pull_possible(h, nnz_x, h->ropts.th3);
+        const bool may_push = !may_pull || fp != DBSPMSPV_PATH_PULL;
+        const int mode = boolean ? 1 : minplus ? 2 : 0;
+        // private accumulators for the hub row blocks, when x is long enough for their atomics to queue up
+        const int hub_min = h->ropts.hub_min_nnz_x ? h->ropts.hub_min_nnz_x : HUB_MIN_NNZ_X;
+        h->d.hub_on = may_push && d.n_hub_blocks > 0 && hub_min > 0 && nnz_x >= hub_min ? (nnz_x < HUB_ALL_NNZ_X ? 4 : HUB_COPIES) : 0;
+        if (may_pull && nnz_x > 0) calls.add(k_xblock_sparse<DT, false>, (nnz_x + XB_TPB - 1) / XB_TPB, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
+        if (h->ropts.timing) calls.ev_before = calls.n;
+        if (nnz_x > 0 && may_push) {
+            auto push = [&](auto list_kernel, auto mask_kernel, auto long_kernel) {
+                if (may_pull) {
+                    // (decided on the device) 32 mask words per thread block and round
+                    const int n_words = (d.nb + 1) / 2;
+                    int g = (n_words + PD_MASK_WORDS - 1) / PD_MASK_WORDS;
+                    if (g > 65536) g = 65536;
+                    calls.add(mask_kernel, g, PD_CTA, 0, true, d, x_idx, xv, nnz_x, 0, h->ropts.th3, fp, 0, (n_words + PD_MASK_WORDS * g - 1) / (PD_MASK_WORDS * g));
+                } else {
+                    // columns per thread block: few enough to fill the GPU, at least eight
+                    const int most = pd_per_sm(false) * h->sm_count;
+                    int cols = (nnz_x + most - 1) / most;
+                    cols = cols <= 8 ? 8 : cols >= PD_CTA ? PD_CTA : (cols + 7) & ~7;
+                    int g = (nnz_x + cols - 1) / cols;
+                    if (g > most) g = most;
+                    calls.add(list_kernel, g, PD_CTA, 0, false, d, x_idx, xv, nnz_x, (int)h->ropts.validate, h->ropts.th3, fp, cols, (nnz_x + cols * g - 1) / (cols * g));
+                }
+                if (d.long_cap) calls.add(long_kernel, 6 * h->sm_count, PD_CTA, 0, true, d);
+            };
+            if (mode == 1) push(k_push_direct<DT, 1, false>, k_push_direct<DT, 1, true>, k_push_long<DT, 1>);
+            else if (mode == 2) push(k_push_direct<DT, 2, false>, k_push_direct<DT, 2, true>, k_push_long<DT, 2>);
+            else if (DT != DBSPMSPV_PATTERN) {
+                constexpr int VT = DT == DBSPMSPV_PATTERN ? DBSPMSPV_F32 : DT;       // (pattern handles have no (+, *))
+                push(k_push_direct<VT, 0, false>, k_push_direct<VT, 0, true>, k_push_long<VT, 0>);
+            };
         }
-    }
-    OutSparse out{d.ws.y_acc, d.ws.y_hit8};
-    if (h->ropts.timing) calls.ev_before = calls.n;
-    // private accumulators for the hub row blocks: when x is long enough for their atomics to
-    // queue up, and not so long that the call will most likely pull
-    const int hub_min = h->ropts.hub_min_nnz_x ? h->ropts.hub_min_nnz_x : HUB_MIN_NNZ_X;
-    h->d.hub_on = !minplus && d.n_hub_blocks > 0 && hub_min > 0 && nnz_x >= hub_min && h->ropts.force_path != DBSPMSPV_PATH_PULL &&
-                  (!late_emit || h->heavy_stage);
-    if (minplus && nnz_x > 0 && d.n_entries > 0) {
-        const int fp = minplus_pull ? h->ropts.force_path : DBSPMSPV_PATH_PUSH;
-        if (fp != DBSPMSPV_PATH_PULL) {
-            calls.add(k_minplus_push<DT>, 4 * h->sm_count, MINPLUS_CTA, 0, true, d, h->ropts.th3, fp);
-        }
-        if (minplus_pull && pull_possible(h, nnz_x, h->ropts.th3)) {
-            const int s = launch_lean<DT, OutSparseMin>(h, calls, OutSparseMin{d.ws.y_acc, d.ws.y_hit8}, h->ropts.th3);
+        if (any && may_pull) {
+            const int s = minplus ? launch_lean<DT, OutSparseMin>(h, calls, OutSparseMin{d.ws.y_acc, d.ws.y_mask32}, h->ropts.th3)
+                                  : launch_lean<DT, OutSparse>(h, calls, OutSparse{d.ws.y_acc, d.ws.y_mask32}, h->ropts.th3);
             if (s != DBSPMSPV_OK) return s;
         }
-    } else if (nnz_x > 0 && d.n_entries > 0) {
-        int s = DBSPMSPV_OK;
-        if (h->heavy_stage) {
-            s = launch_compute<DT, OutSparse, 1>(h, calls, out, h->ropts.th3);
-        } else {
-            // push by k_compute, pull by the streaming kernel: each returns at once when the
-            // selector (evaluated on the device) chose the other; a kernel whose path cannot be
-            // chosen is not launched at all
-            if (h->ropts.force_path != DBSPMSPV_PATH_PULL) s = launch_compute<DT, OutSparse, 0>(h, calls, out, h->ropts.th3);
-            if (s == DBSPMSPV_OK && pull_possible(h, nnz_x, h->ropts.th3)) s = launch_lean<DT, OutSparse>(h, calls, out, h->ropts.th3);
-        }
-        if (s != DBSPMSPV_OK) return s;
-        if (d.hub_on) {
-            calls.add(k_fold_hubs, (d.n_hub_blocks + 3) / 4, 128, 0, true, d);
+        if (!may_pull) clear = CLEAR_MASKS;
+    } else {
+        if (nnz_x > 0) calls.add(k_xblock_sparse<DT, true>, (nnz_x + XB_TPB - 1) / XB_TPB, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
+        if (h->ropts.timing) calls.ev_before = calls.n;
+        if (any && minplus) {
+            calls.add(k_minplus_push<DT>, 4 * h->sm_count, MINPLUS_CTA, 0, true, d, h->ropts.th3, (int)DBSPMSPV_PATH_PUSH);
+        } else if (any) {
+            const int s = launch_compute<DT, OutSparse, 1>(h, calls, OutSparse{d.ws.y_acc, d.ws.y_mask32}, h->ropts.th3);
+            if (s != DBSPMSPV_OK) return s;
         }
     }
     if (h->ropts.timing) { calls.ev_after = calls.n; h->timed = true; }
     const int nt = d.ws.n_tiles;
-    const int parity = (int)(++h->compact_calls & 1u);
-    calls.add(k_compact_count, nt, TILE_WORDS, 0, true, d, parity, row_mask, complement);
     int extra = (nnz_x + CMP_TPB * 8 - 1) / (CMP_TPB * 8);
     if (extra > 4 * h->sm_count) extra = 4 * h->sm_count;
-    const int clear_all = (int64_t)nnz_x * 8 > d.n;     // scattered clears cost more than a full sweep
-    calls.add(k_compact_write, nt + extra, CMP_TPB, 0, true, d, y_idx, y_val, y_capacity, y_nnz,
-              minplus ? 2 : (int)(semiring == DBSPMSPV_OR_AND || DT == DBSPMSPV_PATTERN), x_idx, nnz_x, clear_all, parity, row_mask, complement);
+    // scattered clears cost more than a full sweep once x lists a good part of the columns (a sweep of the masks alone is 32 times shorter)
+    if ((int64_t)nnz_x * (clear & CLEAR_DENSE ? 8 : 128) > d.n) clear |= CLEAR_SWEEP;
+    calls.add(k_finish, nt + extra, CMP_TPB, 0, calls.n > 0, d, y_idx, y_val, y_capacity, y_nnz, minplus ? 2 : (int)boolean, x_idx, nnz_x, clear,
+              d.hub_on ? (minplus ? 2 : 1) : 0, row_mask, complement);
     return submit_calls(h, calls, st);
 }
 

@@ -63,6 +63,8 @@ k_run_small(Device d, const int32_t *__restrict__ x_idx, const void *__restrict_
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) uint32_t s_small[];
     __shared__ SmallShared sh;
+    pdl_wait();
+    pdl_launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = (int)cluster.block_rank();
 #ifdef DBS_SMALL_STAMPS
@@ -80,9 +82,9 @@ k_run_small(Device d, const int32_t *__restrict__ x_idx, const void *__restrict_
     cluster.sync();
     STAMP();
     SmallShared *sh0 = cluster.map_shared_rank(&sh, 0);
-    uint32_t *keys = reinterpret_cast<uint32_t *>(d.ws.y_acc);
+    int *words = reinterpret_cast<int *>(d.ws.y_acc);
     auto add = [&](int row, float a, float xv) {
-        if (mode == 2) atomicMax(keys + row, minplus_key(a + xv));
+        if (mode == 2) atomicMax(words + row, minplus_word(a + xv));
         else if (mode == 0 && DT != DBSPMSPV_PATTERN) atomicAdd(d.ws.y_acc + row, a * xv);
         const int wi = row >> 5, owner = wi / yper;
         atomicOr(cluster.map_shared_rank(s_small, owner) + (wi - owner * yper), 1u << (row & 31));
@@ -215,7 +217,7 @@ k_run_small(Device d, const int32_t *__restrict__ x_idx, const void *__restrict_
         for (uint32_t bb = word; bb; bb &= bb - 1) {
             const int bit = __ffs(bb) - 1, row = (wbase + wi) * 32 + bit;
             if (((keep >> bit) & 1u) && pos < room) rows[pos++] = row;
-            else { if ((keep >> bit) & 1u) ++pos; d.ws.y_acc[row] = 0.f; }
+            else { if ((keep >> bit) & 1u) ++pos; d.ws.y_acc[row] = __uint_as_float(ACC_CLEAR); }
         }
     }
     cluster.sync();          // (release / acquire at cluster scope: the row list is visible to every block)
@@ -235,9 +237,9 @@ k_run_small(Device d, const int32_t *__restrict__ x_idx, const void *__restrict_
         for (int u = 0; u < SMALL_ILP; ++u) {
             if (r[u] < 0) continue;
             const int64_t q = p0 + (int64_t)u * SMALL_CLUSTER * SMALL_CTA;
-            d.ws.y_acc[r[u]] = 0.f;
+            d.ws.y_acc[r[u]] = __uint_as_float(ACC_CLEAR);
             y_idx[q] = r[u];
-            if (y_val) y_val[q] = mode == 1 || (mode == 0 && DT == DBSPMSPV_PATTERN) ? 1.0f : mode == 2 ? minplus_value(__float_as_uint(v[u])) : v[u];
+            if (y_val) y_val[q] = mode == 1 || (mode == 0 && DT == DBSPMSPV_PATTERN) ? 1.0f : mode == 2 ? minplus_of_word(__float_as_uint(v[u])) : v[u] + 0.0f;      // (+ 0: a row of -0 products is 0)
         }
     }
     if (rank == 0 && tid == 0) {
