@@ -333,18 +333,19 @@ __host__ __device__ inline T ceil_div(T a, T b) { return (a + b - 1) / b; }
 // on this handle (0: none).
 int decode_stage_bytes(const Device &d);
 
-// Programmatic dependent launch: a kernel launched with the stream-serialisation attribute may
-// start while its predecessor drains; `pdl_wait` blocks until the predecessor has completed and
-// its writes are visible (a no-op for a normally launched kernel), `pdl_launch_dependents`
-// lets the successor's launch proceed early.  This hides the launch latency between the short
-// kernels of one call.
+// Programmatic dependent launch: a kernel launched with the stream-serialisation attribute is set up
+// while its predecessor drains; `pdl_wait` blocks until the predecessor has completed and its
+// writes are visible (a no-op for a normally launched kernel).  Every kernel of a call begins with
+// it (or reads nothing that an earlier kernel of the stream may write before it).
+// No kernel lets its successor go early (griddepcontrol.launch_dependents): the successor's thread
+// blocks then sit on the SMs, waiting, in the place of its own later blocks and of the persistent
+// kernel behind them (stencil 160^3, x = 5 %: traversal 43 instead of 32 us, call 73 instead of 53; every other path 0 - 4 % slower).
 __device__ __forceinline__ unsigned long long global_timer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Range-checked build (-DDBS_BOUNDS_CHECK; it stands in for a memory checker on the small parity
 // cases): every index that a kernel READS from the handle's arrays -- the other-dimension block

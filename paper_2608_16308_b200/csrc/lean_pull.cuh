@@ -243,7 +243,6 @@ k_pull_lean(Device d, Out out, float th3, int force_path, int popc_threshold, in
     uint32_t *filter = reinterpret_cast<uint32_t *>(s_lean);
     LeanScratch *ls = reinterpret_cast<LeanScratch *>(s_lean + (size_t)filter_words * 4) + warp;
     pdl_wait();
-    pdl_launch_dependents();
     if (select_path(d, th3, force_path) != DBSPMSPV_PATH_PULL) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) d.ws.ctr->path = DBSPMSPV_PATH_PULL;
     const int gwarp = blockIdx.x * LEAN_WARPS + warp;

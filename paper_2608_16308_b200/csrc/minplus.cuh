@@ -164,7 +164,6 @@ __device__ __forceinline__ int select_path(const Device &d, float th3, int force
 template <int DT>
 __global__ void __launch_bounds__(MINPLUS_CTA, 4) k_minplus_push(Device d, float th3, int force_path) {
     pdl_wait();
-    pdl_launch_dependents();
     if (select_path(d, th3, force_path) != DBSPMSPV_PATH_PUSH) return;
     const int lane = threadIdx.x & 31;
     const int gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;

@@ -88,7 +88,6 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
     __shared__ int s_cnt[PD_WARPS], s_sum[PD_WARPS], s_rec[PD_WARPS], s_base;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     pdl_wait();
-    pdl_launch_dependents();
     if (MASKS && select_path(d, th3, force_path) != DBSPMSPV_PATH_PUSH) return;
     Counters *ctr = d.ws.ctr;
     if (blockIdx.x == 0 && tid == 0) ctr->path = DBSPMSPV_PATH_PUSH;
@@ -240,7 +239,6 @@ __global__ void __launch_bounds__(PD_CTA, 6) k_push_long(Device d) {
     const int lane = threadIdx.x & 31;
     const int gwarp = (int)(blockIdx.x * PD_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * PD_CTA) >> 5;
     pdl_wait();
-    pdl_launch_dependents();
     const int n = min(d.ws.ctr->n_long, d.long_cap);
     int4 next = gwarp < n ? d.ws.long_runs[gwarp] : make_int4(0, 0, 0, 0);
     for (int i = gwarp; i < n; i += nwarps) {

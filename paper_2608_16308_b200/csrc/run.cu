@@ -68,7 +68,6 @@ template <int DT, bool EMIT>
 __global__ void k_xblock_sparse(Device d, const int32_t *__restrict__ x_idx, const void *__restrict__ x_val,
                                 int32_t nnz_x, int validate) {
     pdl_wait();
-    pdl_launch_dependents();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     bool newly = false;
@@ -114,7 +113,6 @@ __device__ __forceinline__ bool decode_takes_part(const Device &d, float v) {
 template <int DT>
 __global__ void k_xblock_dense(Device d, const void *__restrict__ x, float *__restrict__ y) {
     pdl_wait();
-    pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
     const int64_t padded = (int64_t)((d.nb + 1) / 2) * 32;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -753,7 +751,6 @@ __global__ void __launch_bounds__(CTA, MODE >= 1 ? DBS_MIN_CTAS_HEAVY : DBS_MIN_
     float *s_lacc = reinterpret_cast<float *>(s_dyn + WARPS * sizeof(PullWarp));
     const int warp = threadIdx.x >> 5;
     pdl_wait();
-    pdl_launch_dependents();
     const int path = select_path(d, th3, force_path);
     if (blockIdx.x == 0 && threadIdx.x == 0) d.ws.ctr->path = path;
     float *lacc = HV ? s_lacc + warp * 16 * LANE_ACC_STRIDE : nullptr;
@@ -896,7 +893,6 @@ __global__ void __launch_bounds__(CTA) k_decode_pull(Device d, const int32_t *__
                                                      float *__restrict__ y, float th3, int force_path) {
     __shared__ __align__(16) uint8_t s_slots[CTA * LBC_SLOT_BYTES];
     pdl_wait();
-    pdl_launch_dependents();
     if (select_path(d, th3, force_path) != DBSPMSPV_PATH_PULL) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) d.ws.ctr->path = DBSPMSPV_PATH_PULL;
     const int lane = threadIdx.x & 31;
@@ -1167,7 +1163,6 @@ k_decode_fused(Device d, const void *__restrict__ x, float *__restrict__ y, floa
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint4 *slot = reinterpret_cast<uint4 *>(s_dyn + lay.slot_off + tid * wc_slot_bytes(wc_ilp(NW)));
     pdl_wait();
-    pdl_launch_dependents();
     if (tid == 0) { s_cnt[0] = 0; s_cnt[1] = 0; }
     if (tid < 16) s_y[tid] = 0.f;
     __syncthreads();
@@ -1624,7 +1619,10 @@ __device__ __forceinline__ int entries_before(const Device &d, int tile, int par
 // It replaces a counting pass and a placing pass: as two kernels they were two waits for the
 // predecessor's last store and the accumulator was fetched twice (9.3 us exposed behind the traversal on a
 // million rows; 5 here).
-__global__ void __launch_bounds__(CMP_TPB, 5) k_finish(Device d, int32_t *__restrict__ y_idx, float *__restrict__ y_val,
+// FOLD: the call's push used private accumulators (more registers: a kernel of its own, so that the other keeps eight
+// thread blocks per SM -- on four million rows the tiles come in waves).
+template <bool FOLD>
+__global__ void __launch_bounds__(CMP_TPB, FOLD ? 5 : 8) k_finish(Device d, int32_t *__restrict__ y_idx, float *__restrict__ y_val,
                                                     int64_t y_capacity, int32_t *__restrict__ y_nnz, int boolean,
                                                     const int32_t *__restrict__ x_idx, int32_t nnz_x, int clear, int fold,
                                                     const uint32_t *__restrict__ row_mask, int complement) {
@@ -1643,7 +1641,6 @@ __global__ void __launch_bounds__(CMP_TPB, 5) k_finish(Device d, int32_t *__rest
     const int bi = tile * CMP_TPB + threadIdx.x;      // byte of the hit mask: rows 8 bi .. 8 bi + 7
     const int j0 = (!(clear & CLEAR_SWEEP) && bi < nnz_x) ? x_idx[bi] : -1;      // (x is the caller's: nothing of this call writes it)
     pdl_wait();
-    pdl_launch_dependents();
     if (tile < n_tiles) {
         const int n_bytes = (d.mb + 1) / 2 * 4;
         uint8_t *mask8 = reinterpret_cast<uint8_t *>(d.ws.y_mask32);
@@ -1663,7 +1660,7 @@ __global__ void __launch_bounds__(CMP_TPB, 5) k_finish(Device d, int32_t *__rest
                 acc4[1] = make_uint4(ACC_CLEAR, ACC_CLEAR, ACC_CLEAR, ACC_CLEAR);
             }
             if (flags) mask8[bi] = 0;
-            if (fold) {
+            if (FOLD) {
                 const int slot = d.hub_slot[bi >> 1];
                 if (slot != HUB_NONE && DBS_CHK_INDEX(d, slot, d.n_hub_blocks)) {
                     fold_hub_rows(d, slot, bi & 1, fold == 2, v);
@@ -1760,7 +1757,6 @@ __global__ void __launch_bounds__(CMP_TPB, 5) k_finish(Device d, int32_t *__rest
 
 __global__ void k_decode_cleanup(Device d) {
     pdl_wait();
-    pdl_launch_dependents();
     const int n_words = (d.nb + 1) / 2;
     const int stride = gridDim.x * blockDim.x;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n_words; k += stride) d.ws.x_mask32[k] = 0u;
@@ -1792,7 +1788,6 @@ __global__ void k_wait_probe(Device d, int max_tries) {
 
 __global__ void k_fill_u32(uint32_t *p, int64_t n, uint32_t v) {
     pdl_wait();
-    pdl_launch_dependents();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = v;
 }
 
@@ -2010,7 +2005,7 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
     if (extra > 4 * h->sm_count) extra = 4 * h->sm_count;
     // scattered clears cost more than a full sweep once x lists a good part of the columns (a sweep of the masks alone is 32 times shorter)
     if ((int64_t)nnz_x * (clear & CLEAR_DENSE ? 8 : 128) > d.n) clear |= CLEAR_SWEEP;
-    calls.add(k_finish, nt + extra, CMP_TPB, 0, calls.n > 0, d, y_idx, y_val, y_capacity, y_nnz, minplus ? 2 : (int)boolean, x_idx, nnz_x, clear,
+    calls.add(d.hub_on ? k_finish<true> : k_finish<false>, nt + extra, CMP_TPB, 0, calls.n > 0, d, y_idx, y_val, y_capacity, y_nnz, minplus ? 2 : (int)boolean, x_idx, nnz_x, clear,
               d.hub_on ? (minplus ? 2 : 1) : 0, row_mask, complement);
     return submit_calls(h, calls, st);
 }

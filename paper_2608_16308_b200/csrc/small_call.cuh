@@ -64,7 +64,6 @@ k_run_small(Device d, const int32_t *__restrict__ x_idx, const void *__restrict_
     extern __shared__ __align__(16) uint32_t s_small[];
     __shared__ SmallShared sh;
     pdl_wait();
-    pdl_launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = (int)cluster.block_rank();
 #ifdef DBS_SMALL_STAMPS
