@@ -10,6 +10,7 @@
 
 #include "call_graph.cuh"
 #include "internal.cuh"
+#include "minplus.cuh"
 
 namespace dbs {
 namespace {
@@ -479,6 +480,21 @@ __global__ void k_csc_colptr(int32_t nb, const uint64_t *keys_sorted, int32_t n,
         if ((keys_sorted[mid] >> CSC_KEY_GROUP_SHIFT) < target) lo = mid + 1; else hi = mid;
     }
     colptr[t] = lo;
+}
+
+// The weights of one view entry into the column copy (decode_columns.cuh), a thread per entry.
+__global__ void k_columns_copy(Device d, const int32_t *block_row, uint16_t *out, int32_t *bad) {
+    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (p >= d.n_entries) return;
+    const uint32_t idx = d.csr.idx[p];
+    const int64_t row0 = (int64_t)block_row[p] * 16, col0 = (int64_t)(idx & IDX_MASK) * 16;
+    block_elements<DBSPMSPV_BF16>((int)(idx >> TYPE_SHIFT), d.csr.w[p], d.csr.aux[p], 0xFFFFu, d.payload, [&](int r, int c, float a) {
+        uint32_t u = __float_as_uint(a) >> 16;
+        if ((u & 0x7F80u) == 0x7F80u) *bad = 1;
+        if (u == DC_ABSENT) u = 0u;
+        const int64_t row = row0 + r;
+        out[((row / DC_ROWS) * d.n + col0 + c) * DC_ROWS + row % DC_ROWS] = (uint16_t)u;
+    });
 }
 
 // Chunks of the direct push's list when every column is listed (see PD_LONG).
@@ -1009,6 +1025,30 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         tp.release(cnt); tp.release(first);
         d.stage_chunks = chunks;
         h->stage_index_bytes = (int64_t)d.n_stage_chunks * 16;
+    }
+
+    // Decode over columns of bf16 layers (decode_columns.cuh): the weights once more, column by column in strips of
+    // rows.  Not built when it does not fit, nor for weights that are not finite (a batched call multiplies absent x entries as zeros).
+    d.cols = nullptr;
+    if (h->heavy_stage && d.dtype == DBSPMSPV_BF16 && m >= DC_MIN_ROWS && n <= DC_MAX_COLUMNS) {
+        const int64_t bytes = (m + DC_ROWS - 1) / DC_ROWS * DC_ROWS * n * 2;
+        void *p = nullptr;
+        if (bytes <= DC_MAX_RATIO * h->payload_bytes) {
+            if (cudaMalloc(&p, (size_t)bytes) != cudaSuccess) { (void)cudaGetLastError(); p = nullptr; }
+        }
+        if (p) {
+            int32_t *bad, bad_h = 0;
+            DBS_GET(bad, 1);
+            DBS_CUDA(cudaMemsetAsync(bad, 0, 4, st));
+            k_fill_words<<<grid_for(bytes / 4), TPB, 0, st>>>(static_cast<uint32_t *>(p), bytes / 4, DC_ABSENT * 0x10001u);
+            k_columns_copy<<<grid_for(n_entries), TPB, 0, st>>>(d, h->block_row, static_cast<uint16_t *>(p), bad);
+            cudaError_t e = cudaMemcpyAsync(&bad_h, bad, 4, cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            tp.release(bad);
+            if (e != cudaSuccess || bad_h) cudaFree(p);
+            if (e != cudaSuccess) return DBSPMSPV_ERR_CUDA;
+            if (!bad_h) { d.cols = static_cast<const uint4 *>(p); h->stage_index_bytes += bytes; }
+        }
     }
 
     // Streaming pull of hypersparse handles: the list of rows that hold INLINE elements (the

@@ -119,6 +119,12 @@ constexpr int HUB_CAP = 32;
 #define DBS_STAGE_BYTES (6 * 1024)
 #endif
 constexpr int STAGE_BYTES = DBS_STAGE_BYTES;
+// Decode over columns (decode_columns.cuh): rows of a strip; the bf16 pattern of an absent element; where the copy is built.
+constexpr int DC_ROWS = 32;
+constexpr uint32_t DC_ABSENT = 0x8000u;
+constexpr int DC_MIN_ROWS = 1024;           // (fewer rows make too few strips: the block kernels deal the payload out over all SMs)
+constexpr int DC_MAX_COLUMNS = 25600;       // the list of active columns has to fit in shared memory
+constexpr int DC_MAX_RATIO = 4;             // copy / payload, at most
 constexpr int HDR_BYTES = 48;               // masks + starts of a valued mid-class block
 
 // Payload size in 4-byte words; every block is padded to 16 bytes so that it can be moved with
@@ -257,6 +263,7 @@ struct Device {           // everything the kernels need, passed by value
     const int4 *stage_chunks;
     int32_t n_stage_chunks;
     int32_t stage_bytes;        // payload bytes of one stage (a multiple of 512)
+    const uint4 *cols;          // bf16 weights once more, [strip of DC_ROWS rows][column][row] (null: not built)
     int32_t has_inline;         // the handle holds INLINE elements at all
     float decode_tau;           // per call: activation magnitude cut of dbspmspv_decode (run option)
     int32_t decode_relu;        // per call: ReLU fused into the cut (x_j > tau instead of |x_j| > tau)
@@ -301,6 +308,8 @@ struct dbspmspv_handle_s {
     bool fused_configured[3];
     bool batch_configured[2];
     bool batch_mma_configured[3];
+    bool cols_configured;
+    int cols_grid[2];           // resident clusters of the batched decode over columns (4 / 8 vectors; 0: does not fit)
     int stream_grid;            // thread blocks of the streaming decode (0: not configured yet)
     int32_t *x_nnz_seen_host;   // host view of Device::x_nnz_seen (page-locked, mapped)
     bool heavy_stage;           // most stored elements sit in mask-based blocks: MODE 1 kernels

@@ -1528,6 +1528,7 @@ k_decode_stream(Device d, const void *__restrict__ x, float *__restrict__ y, flo
 }  // namespace dbs
 #include "decode_batch.cuh"
 #include "small_call.cuh"
+#include "decode_columns.cuh"
 namespace dbs {
 
 // ------------------------------------------------------------------------------------------
@@ -2024,6 +2025,54 @@ int decode_stage_bytes(const Device &d) {
     return 0;
 }
 
+// Decode over columns: `nvec` vectors (1, or as many as decode_columns_group says) in one kernel.
+template <int C>
+static int decode_columns_c(dbspmspv_handle_s *h, CallList &calls, const void *x, int64_t ldx, float *y, int64_t ldy, int nvec) {
+    const Device &d = h->d;
+    const int strips = (int)((d.m + DC_ROWS - 1) / DC_ROWS);
+    if (!h->cols_configured) {
+        DBS_CUDA(cudaFuncSetAttribute(k_decode_cols<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSED_MAX_SMEM));
+        // (the attribute belongs to the kernel, not to the handle: all that its static shared memory leaves)
+        DBS_CUDA(cudaFuncSetAttribute(k_decode_cols_batch<4, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, STREAM_MAX_SMEM - dcb_static(4, C)));
+        DBS_CUDA(cudaFuncSetAttribute(k_decode_cols_batch<8, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, STREAM_MAX_SMEM - dcb_static(8, C)));
+        int per_sm = 0;
+        DBS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_decode_cols_batch<4, C>, DCB_CTA, DcBatchLayout(d.nb, 4, C).total));
+        h->cols_grid[0] = per_sm * h->sm_count / C;
+        DBS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_decode_cols_batch<8, C>, DCB_CTA, DcBatchLayout(d.nb, 8, C).total));
+        h->cols_grid[1] = per_sm * h->sm_count / C;
+        h->cols_configured = true;
+    }
+    if (nvec == 1) {
+        calls.add(k_decode_cols<C>, strips * C, DC_CTA, (size_t)((d.nb + C - 1) / C) * 16 * sizeof(float2), false, d, x, y, h->ropts.th3_decode, h->ropts.force_path);
+        return DBSPMSPV_OK;
+    }
+    const int slots = h->cols_grid[nvec <= 4 ? 0 : 1], g = (strips < slots ? strips : slots) * C;
+    if (g < 1) return DBSPMSPV_ERR_CUDA;
+    calls.add(nvec <= 4 ? k_decode_cols_batch<4, C> : k_decode_cols_batch<8, C>, g, DCB_CTA, (size_t)DcBatchLayout(d.nb, nvec <= 4 ? 4 : 8, C).total, false,
+              d, x, ldx, y, ldy, nvec, h->ropts.th3_decode, h->ropts.force_path);
+    return DBSPMSPV_OK;
+}
+static int decode_columns(dbspmspv_handle_s *h, const void *x, int64_t ldx, float *y, int64_t ldy, int nvec, cudaStream_t st) {
+    CallList calls;
+    int s = DBSPMSPV_OK;
+    switch (dc_cluster(h->d.m, h->sm_count)) {
+        case 1: s = decode_columns_c<1>(h, calls, x, ldx, y, ldy, nvec); break;
+        case 2: s = decode_columns_c<2>(h, calls, x, ldx, y, ldy, nvec); break;
+        case 4: s = decode_columns_c<4>(h, calls, x, ldx, y, ldy, nvec); break;
+        default: s = decode_columns_c<8>(h, calls, x, ldx, y, ldy, nvec); break;
+    }
+    if (s != DBSPMSPV_OK) return s;
+    if (h->ropts.timing) { calls.ev_before = 0; calls.ev_after = calls.n; h->timed = true; }
+    return submit_calls(h, calls, st);
+}
+// vectors of one batched call over columns, at most (1: the lists of several do not fit in shared memory)
+static int decode_columns_group(const dbspmspv_handle_s *h) {
+    const int c = dc_cluster(h->d.m, h->sm_count);
+    for (int nv : {8, 4})
+        if (DcBatchLayout(h->d.nb, nv, c).total + dcb_static(nv, c) <= STREAM_MAX_SMEM) return nv;
+    return 1;
+}
+
 template <int DT>
 static int decode_typed(dbspmspv_handle_s *h, const void *x, float *y, cudaStream_t st) {
     const Device &d = h->d;
@@ -2031,6 +2080,7 @@ static int decode_typed(dbspmspv_handle_s *h, const void *x, float *y, cudaStrea
     h->d.decode_tau = h->ropts.decode_threshold;
     h->d.decode_relu = h->ropts.decode_relu != 0;
     h->d.decode_x_f32 = h->ropts.decode_x_f32 != 0;
+    if (DT == DBSPMSPV_BF16 && d.cols && h->ropts.no_fused_decode == 0) return decode_columns(h, x, 0, y, 0, 1, st);
     // (-1: no decode call has reported yet)
     const int seen = h->x_nnz_seen_host ? *const_cast<volatile int32_t *>(h->x_nnz_seen_host) : -1;
     const bool sparse_x = seen >= 0 && (float)seen < STREAM_MIN_X_DENSITY * (float)d.n;
@@ -2125,6 +2175,7 @@ static int decode_batch_typed(dbspmspv_handle_s *h, const void *x, int64_t ldx, 
     h->d.decode_tau = h->ropts.decode_threshold;
     h->d.decode_relu = h->ropts.decode_relu != 0;
     h->d.decode_x_f32 = h->ropts.decode_x_f32 != 0;
+    const int cols_group = DT == DBSPMSPV_BF16 && d.cols && h->ropts.no_fused_decode == 0 ? decode_columns_group(h) : 0;
     // the per-column kernel on vectors [b0, b0 + g), g <= 4
     auto scalar_group = [&](CallList &calls, const void *xg, float *yg, int g, int only_as_fallback) -> int {
         const int nb = g <= 2 ? 2 : 4;
@@ -2142,12 +2193,18 @@ static int decode_batch_typed(dbspmspv_handle_s *h, const void *x, int64_t ldx, 
         const int left = batch - b0;
         const void *xg = static_cast<const uint8_t *>(x) + (size_t)b0 * (size_t)ldx * esize;
         float *yg = y + (size_t)b0 * (size_t)ldy;
-        const int cap = DT == DBSPMSPV_BF16 && max_mma > 1 ? max_mma : max_nb;
+        const int cap = cols_group > 1 ? cols_group : DT == DBSPMSPV_BF16 && max_mma > 1 ? max_mma : max_nb;
         const int g = left < cap ? left : cap;
         if (g == 1) {
             const int s = decode_typed<DT>(h, xg, yg, st);
             if (s != DBSPMSPV_OK) return s;
             b0 += 1;
+            continue;
+        }
+        if (cols_group > 1) {
+            const int s = decode_columns(h, xg, ldx, yg, ldy, g, st);
+            if (s != DBSPMSPV_OK) return s;
+            b0 += g;
             continue;
         }
         CallList calls;

@@ -1,0 +1,72 @@
+"""The decode over columns of bf16 layers (automatic mode, 1024 rows or more): strips of 32 rows, one or
+several thread blocks per strip, one to nine vectors, sizes off every tile edge, activation options,
+non-finite activations, a weight that is stored as -0."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2608_16308_b200 import binding as B
+from paper_2608_16308_b200 import workloads as wl
+from gpu_util import Handle, ref_matrix, DEV, TOL
+
+pytestmark = pytest.mark.gpu
+
+
+def bits(a):
+    return torch.from_numpy(wl.f32_to_bf16_bits(a).view(np.int16)).to(DEV)
+
+
+def check(y, want, scale):
+    fin = np.isfinite(want)
+    assert (np.isnan(y) == np.isnan(want)).all() and (y[np.isinf(want)] == want[np.isinf(want)]).all()
+    assert (np.abs(y[fin].astype(np.float64) - want[fin]) <= TOL * scale[fin]).all()
+    assert (y[fin & (scale == 0)] == 0.0).all()
+
+
+# 33 strips (8 then 4 blocks each), 128 / 149 strips (1), rows and columns off the tiles, and a wide one
+@pytest.mark.parametrize("shape,prune", [((1025, 333), 0.5), ((1100, 1000), 0.7), ((2400, 17), 0.6), ((4768, 260), 0.5), ((1024, 12289), 0.5)])
+@pytest.mark.parametrize("x_f32", [0, 1])
+def test_decode_over_columns(shape, prune, x_f32):
+    m, n = shape
+    w = wl.pruned_weight(m, n, prune, seed=5, stream=m + n)
+    w.val[3] = np.float32(-0.0)
+    h = Handle(w, B.BF16)
+    A = ref_matrix(w, bf16=True)
+    nv, ldx, ldy = 9, n + (8 if n % 8 == 0 else 3), m + 5
+    xs = np.zeros((nv, ldx), np.float32)
+    for b, zf in enumerate((0.7, 0.9, 0.05, 1.0, 0.99, 0.3, 0.8, 0.6, 0.95)):
+        if zf < 1.0:
+            xs[b, :n] = wl.relu_activation(n, zf, seed=5, stream=90 + b)
+    xs[2, :n] *= np.where(np.arange(n) % 3 == 0, -1.0, 1.0)
+    for special in (False, True):
+        if special:
+            xs[1, w.col_idx[5]], xs[1, w.col_idx[-1]] = np.inf, np.nan
+        xr = wl.bf16_bits_to_f32(wl.f32_to_bf16_bits(xs))
+        xd = torch.from_numpy(xs * np.float32(1 + 2.0 ** -11)).to(DEV) if x_f32 else bits(xs)      # (rounds back to the bf16 values)
+        for relu, tau in ((0, 0.0), (1, 0.3)):
+            h.set_opts(decode_relu=relu, decode_threshold=tau, decode_x_f32=x_f32)
+            refs = []
+            for b in range(nv):
+                xt = xr[b, :n]
+                with np.errstate(invalid="ignore"):
+                    keep = ~(xt <= np.float32(tau)) if relu else ~(np.abs(xt) <= np.float32(tau))
+                refs.append(oracle.ref_decode(A, np.where(keep, xt, 0.0).astype(np.float32)) + (keep,))
+            for batch in (1, 2, 4, 5, 9):
+                y = torch.full((batch, ldy), 55.0, device=DEV)
+                before = h.get_stats().kernel_launches
+                if batch == 1:
+                    B.dbspmspv_decode(h.h, xd, y)
+                    torch.cuda.synchronize()
+                    assert h.get_stats().kernel_launches - before == 1
+                    pad = np.zeros((n + 15) // 16 * 16, bool)
+                    pad[:n] = refs[0][2]
+                    assert h.get_stats().last_n_nzblk == int(pad.reshape(-1, 16).any(axis=1).sum())
+                else:
+                    B.dbspmspv_decode_batch(h.h, xd, ldx, y, ldy, batch)
+                torch.cuda.synchronize()
+                yh = y.cpu().numpy()
+                for b in range(batch):
+                    check(yh[b, :m], *refs[b][:2])
+                assert (yh[:, m:] == 55.0).all()
+    h.close()
