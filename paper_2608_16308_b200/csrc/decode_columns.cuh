@@ -4,7 +4,7 @@
 // What such a call cannot do without is the surviving weights of the active columns; the block
 // payload holds them in pieces of 15 - 32 bytes behind 48-byte headers, so that a call either read
 // everything (12288 x 4096 pruned by half: 84 MB whatever x holds, 27 us) or fetched the pieces in chains of dependent loads.  Here the
-// weights lie once more, column by column: strips of DC_ROWS = 32 rows, [strip][column][row], 64 contiguous
+// weights lie once more, column by column: strips of DC_ROWS = 64 rows, [strip][column][row], 128 contiguous
 // bytes per column and strip, absent elements as DC_ABSENT (a -0.0 that no stored weight uses: a
 // stored -0 is kept as +0, which gives the same products up to the sign of a zero).  A call then reads the
 // active columns only, every lane 16 bytes at a time, all loads independent of each other, and the arithmetic is one shift
@@ -18,7 +18,7 @@
 //   * x is blocked by every thread block for itself (a few KB, from L2): the entries that take part become a list of
 //     (column, value) in shared memory.
 //   * Several vectors (k_decode_cols_batch) share one pass over the union of their columns on the tensor cores: D[vector][row] += X[vector][k] W[k][row],
-//     16 columns per mma.sync m16n8k16, the W fragments straight from global memory -- a lane loads four rows of the four columns its fragment
+//     16 columns per mma.sync m16n8k16, the W fragments straight from global memory -- a lane loads eight rows of the four columns its fragment
 //     holds and pairs the columns with byte permutes, no shared memory and no expansion in between.
 //   * A non-finite x entry may only meet stored elements: such calls (checked while x is blocked) take a plain loop that tests every element.
 #pragma once
@@ -34,41 +34,49 @@ __device__ __forceinline__ float dc_x(const Device &d, const void *x, int64_t ld
     if (d.decode_x_f32) return __bfloat162float(__float2bfloat16_rn(static_cast<const float *>(x)[b * ldx + j]));
     return __bfloat162float(static_cast<const __nv_bfloat16 *>(x)[b * ldx + j]);
 }
-// eight consecutive entries j0 .. j0 + 7 (j0 a multiple of 8; entries past n are 0 and never take part)
-__device__ __forceinline__ void dc_load8(const Device &d, const void *x, int64_t ldx, int b, int64_t j0, bool aligned, float (&v)[8]) {
+// eight consecutive entries j0 .. j0 + 7 (j0 a multiple of 8) as bf16; entries past n are 0
+__device__ __forceinline__ uint4 dc_load8(const Device &d, const void *x, int64_t ldx, int b, int64_t j0, bool aligned) {
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+    if (aligned && !d.decode_x_f32 && j0 + 8 <= d.n) return *reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(x) + b * ldx + j0);
     if (aligned && j0 + 8 <= d.n) {
-        if (d.decode_x_f32) {
-            const float4 *p = reinterpret_cast<const float4 *>(static_cast<const float *>(x) + b * ldx + j0);
-            const float4 f = p[0], g = p[1];
-            const float w[8] = {f.x, f.y, f.z, f.w, g.x, g.y, g.z, g.w};
+        const float4 *p = reinterpret_cast<const float4 *>(static_cast<const float *>(x) + b * ldx + j0);
+        const float4 f = p[0], g = p[1];
+        const float v[8] = {f.x, f.y, f.z, f.w, g.x, g.y, g.z, g.w};
 #pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = __bfloat162float(__float2bfloat16_rn(w[k]));
-        } else {
-            const uint4 u = *reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(x) + b * ldx + j0);
-            const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+        for (int k = 0; k < 8; ++k) w[k >> 1] |= (__float_as_uint(__bfloat162float(__float2bfloat16_rn(v[k]))) >> 16) << (16 * (k & 1));
+    } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) { v[2 * k] = __uint_as_float(w[k] << 16); v[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u); }
-        }
-        return;
+        for (int k = 0; k < 8; ++k)
+            if (j0 + k < d.n) w[k >> 1] |= (__float_as_uint(dc_x(d, x, ldx, b, j0 + k)) >> 16) << (16 * (k & 1));
     }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = j0 + k < d.n ? dc_x(d, x, ldx, b, j0 + k) : 0.f;
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ float dc_entry(const uint4 &u, int k) {       // entry k of eight
+    const uint32_t w = k < 2 ? u.x : k < 4 ? u.y : k < 6 ? u.z : u.w;
+    return __uint_as_float(k & 1 ? w & 0xFFFF0000u : w << 16);
 }
 __device__ __forceinline__ bool dc_finite(float v) { return (__float_as_uint(v) & 0x7F800000u) != 0x7F800000u; }
 
-// The calls with a non-finite x entry: lane = row, a column at a time, every element tested.
+// The calls with a non-finite x entry: a lane takes the rows lane, lane + 32 of the strip, a column at a time, every element tested.
+constexpr int DC_PER_LANE = DC_ROWS / 32;
 template <int NV>
-__device__ __forceinline__ void dc_slow(const Device &d, const void *x, int64_t ldx, int nvec, int strip, int warp, int step, int lane, float (&acc)[NV]) {
+__device__ __forceinline__ void dc_slow(const Device &d, const void *x, int64_t ldx, int nvec, int strip, int warp, int step, int lane, float (&acc)[NV][DC_PER_LANE]) {
     const uint16_t *w = reinterpret_cast<const uint16_t *>(d.cols) + (size_t)strip * d.n * DC_ROWS + lane;
 #pragma unroll
-    for (int b = 0; b < NV; ++b) acc[b] = 0.f;
+    for (int b = 0; b < NV; ++b)
+#pragma unroll
+        for (int h = 0; h < DC_PER_LANE; ++h) acc[b][h] = 0.f;
     for (int64_t j = warp; j < d.n; j += step) {
-        const uint32_t u = w[j * DC_ROWS];
 #pragma unroll
         for (int b = 0; b < NV; ++b) {
             if (b >= nvec) break;
             const float v = dc_x(d, x, ldx, b, j);
-            if (u != DC_ABSENT && decode_takes_part(d, v)) acc[b] += __uint_as_float(u << 16) * v;
+            if (!decode_takes_part(d, v)) continue;
+#pragma unroll
+            for (int h = 0; h < DC_PER_LANE; ++h) {
+                const uint32_t u = w[j * DC_ROWS + 32 * h];
+                if (u != DC_ABSENT) acc[b][h] += __uint_as_float(u << 16) * v;
+            }
         }
     }
 }
@@ -83,18 +91,23 @@ __device__ __forceinline__ void dc_record(const Device &d, int n_nzblk, float th
     c->last_y_nnz = (int32_t)d.m;
 }
 
-constexpr int DC_WARPS = 8;
+constexpr int DC_WARPS = 16;
 constexpr int DC_CTA = DC_WARPS * 32;
 constexpr int DC_ILP = 8;            // 16-byte loads in flight per lane: 4 KB per warp
+constexpr int DC_LANES = DC_ROWS / 8;    // lanes that share a column (eight rows each)
+constexpr int DC_SLOTS = 32 / DC_LANES;  // columns of a warp's load
+constexpr int DC_XILP = 4;           // groups of eight x entries a thread fetches at once
+static_assert(DC_ROWS == 64, "two halving exchanges over the column slots");
 
-// One vector.  Lane (q, p) = (lane / 4, lane % 4): rows 8 p .. 8 p + 7 of the strip, every eighth column of the list.
+// One vector.  Lane (q, p) = (lane / 8, lane % 8): rows 8 p .. 8 p + 7 of the strip, every fourth column of the list.
 template <int C>
-__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(DC_CTA)
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(DC_CTA, 2)
 k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float th3, int force_path) {
     namespace cg = cooperative_groups;
     extern __shared__ __align__(16) uint8_t s_dyn[];
     float2 *s_list = reinterpret_cast<float2 *>(s_dyn);              // (column bits, value)
-    __shared__ float s_part[DC_WARPS][DC_ROWS], s_sum[C][DC_ROWS];
+    __shared__ __align__(8) float s_part[DC_WARPS][DC_ROWS];
+    __shared__ float s_sum[C][DC_ROWS];
     __shared__ int s_n, s_nz, s_seen[C];                             // entries; nonzero vector blocks; those of every rank, plus DC_SLOW_FLAG if it met a non-finite entry
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = C > 1 ? (int)cg::this_cluster().block_rank() : 0, strip = blockIdx.x / C;
@@ -107,15 +120,23 @@ k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float
         const bool aligned = (reinterpret_cast<uintptr_t>(x) & 15u) == 0;
         const int units = (d.nb - rank + C - 1) / C * 2;             // halves of this rank's vector blocks
         int nz = 0;
-        for (int u0 = warp * 32; u0 < units; u0 += DC_CTA) {
-            const int u = u0 + lane;
-            const int64_t j0 = ((int64_t)(u >> 1) * C + rank) * 16 + (u & 1) * 8;
-            float v[8];
-            uint32_t bits = 0;
-            if (u < units) {
-                dc_load8(d, x, 0, 0, j0, aligned, v);
+        for (int u0 = warp * 32; u0 < units; u0 += DC_CTA * DC_XILP) {
+            uint4 v[DC_XILP];
+            int j0[DC_XILP];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) { bits |= (j0 + k < d.n && decode_takes_part(d, v[k]) ? 1u : 0u) << k; }
+            for (int q = 0; q < DC_XILP; ++q) {
+                const int u = u0 + q * DC_CTA + lane;
+                j0[q] = ((u >> 1) * C + rank) * 16 + (u & 1) * 8;
+                v[q] = make_uint4(0u, 0u, 0u, 0u);
+                if (u < units) v[q] = dc_load8(d, x, 0, 0, j0[q], aligned);
+            }
+            uint32_t bits = 0;                                        // eight per group
+#pragma unroll
+            for (int q = 0; q < DC_XILP; ++q) {
+                if (u0 + q * DC_CTA >= units) break;                  // warp-uniform
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    bits |= (j0[q] + k < (int)d.n && decode_takes_part(d, dc_entry(v[q], k)) ? 1u : 0u) << (8 * q + k);
             }
             const int cnt = __popc(bits);
             int incl = cnt;
@@ -124,10 +145,19 @@ k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float
             int base = 0;
             if (lane == 31 && incl) base = atomicAdd(&s_n, incl);
             int at = __shfl_sync(FULL, base, 31) + incl - cnt;
+            const uint32_t both = bits | __shfl_xor_sync(FULL, bits, 1);
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if ((bits >> k) & 1u) { s_list[at++] = make_float2(__int_as_float((int)j0 + k), v[k]); odd |= !dc_finite(v[k]); }
-            nz += __popc(__ballot_sync(FULL, bits | __shfl_xor_sync(FULL, bits, 1)) & 0x55555555u);
+            for (int q = 0; q < DC_XILP; ++q) {
+                if (u0 + q * DC_CTA >= units) break;
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if ((bits >> (8 * q + k)) & 1u) {
+                        const float e = dc_entry(v[q], k);
+                        s_list[at++] = make_float2(__int_as_float(j0[q] + k), e);
+                        odd |= !dc_finite(e);
+                    }
+                nz += __popc(__ballot_sync(FULL, (both >> (8 * q)) & 0xFFu) & 0x55555555u);
+            }
         }
         if (lane == 0 && nz) atomicAdd(&s_nz, nz);
         odd = __syncthreads_or(odd);
@@ -148,24 +178,28 @@ k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float
             dc_record(d, total, th3, force_path);
         }
         if (odd) {
-            float a[1];
+            float a[1][DC_PER_LANE];
             dc_slow<1>(d, x, 0, 1, strip, warp * C + rank, DC_WARPS * C, lane, a);
-            s_part[warp][lane] = a[0];
-        } else s_part[warp][lane] = 0.f;
+#pragma unroll
+            for (int h = 0; h < DC_PER_LANE; ++h) s_part[warp][lane + 32 * h] = a[0][h];
+        } else {
+#pragma unroll
+            for (int h = 0; h < DC_PER_LANE; ++h) s_part[warp][lane + 32 * h] = 0.f;
+        }
     }
     __syncthreads();
     const int n = odd ? 0 : s_n;
     if (n > 0) {                                                      // block-uniform
-        const uint4 *w = d.cols + (size_t)strip * d.n * (DC_ROWS / 8) + (lane & 3);
+        const uint4 *w = d.cols + (size_t)strip * d.n * (DC_ROWS / 8) + (lane & (DC_LANES - 1));
         float acc[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) acc[r] = 0.f;
-        for (int k0 = warp * 8 + (lane >> 2); k0 - (lane >> 2) < n; k0 += DC_WARPS * 8 * DC_ILP) {
+        for (int k0 = warp * DC_SLOTS + lane / DC_LANES; k0 - lane / DC_LANES < n; k0 += DC_WARPS * DC_SLOTS * DC_ILP) {
             uint4 v[DC_ILP];
             float xv[DC_ILP];
 #pragma unroll
             for (int u = 0; u < DC_ILP; ++u) {
-                const int k = k0 + u * DC_WARPS * 8;
+                const int k = k0 + u * DC_WARPS * DC_SLOTS;
                 v[u] = make_uint4(0u, 0u, 0u, 0u);
                 xv[u] = 0.f;
                 if (k < n) { const float2 e = s_list[k]; xv[u] = e.y; v[u] = __ldcs(w + (size_t)__float_as_int(e.x) * (DC_ROWS / 8)); }
@@ -180,15 +214,14 @@ k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float
                 }
             }
         }
-        // sums over the eight column slots of the warp: three halving exchanges leave one row per lane
-        const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+        // sums over the four column slots of the warp: two halving exchanges leave two rows per lane
+        const bool h16 = lane & 16, h8 = lane & 8;
         float a4[4], a2[2];
 #pragma unroll
         for (int i = 0; i < 4; ++i) a4[i] = (h16 ? acc[i + 4] : acc[i]) + __shfl_xor_sync(FULL, h16 ? acc[i] : acc[i + 4], 16);
 #pragma unroll
         for (int i = 0; i < 2; ++i) a2[i] = (h8 ? a4[i + 2] : a4[i]) + __shfl_xor_sync(FULL, h8 ? a4[i] : a4[i + 2], 8);
-        const float a1 = (h4 ? a2[1] : a2[0]) + __shfl_xor_sync(FULL, h4 ? a2[0] : a2[1], 4);
-        s_part[warp][(lane & 3) * 8 + (h16 ? 4 : 0) + (h8 ? 2 : 0) + (h4 ? 1 : 0)] = a1;
+        *reinterpret_cast<float2 *>(&s_part[warp][(lane & 7) * 8 + (h16 ? 4 : 0) + (h8 ? 2 : 0)]) = make_float2(a2[0], a2[1]);
     }
     __syncthreads();
     float sum = 0.f;
@@ -212,186 +245,193 @@ k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float
 
 constexpr int DCB_WARPS = 16;
 constexpr int DCB_CTA = DCB_WARPS * 32;
-constexpr int DCB_ILP = 2;           // steps of 16 columns in flight per warp: 2 KB
-static_assert(DCB_WARPS * 32 >= 8 * DC_ROWS, "a thread per vector and row");
+constexpr int DCB_ILP = 2;           // steps of 16 columns in flight per warp: 4 KB
+constexpr int DCB_SLOTS = 4;         // partial sums kept in shared memory: four warps at a time add theirs
+constexpr int DCB_ROUNDS = 8;        // groups of eight x entries a thread may own (a byte of its mask each)
+static_assert(DCB_CTA >= 8 * DC_ROWS, "a thread per vector and row");
+static_assert(DC_MAX_COLUMNS < 65536 && DC_MAX_COLUMNS <= DCB_CTA * DCB_ROUNDS * 8, "16-bit columns; every entry has an owner");
 
-// Shared memory of a batched call: values by pairs of list entries, [pair][vector][2] bf16; columns; partial sums.
+// Shared memory of a batched call: values by pairs of list entries, [pair][vector] 2 x bf16; columns; partial sums.
 struct DcBatchLayout {
-    int cap, col_off, red_off, total;
-    __host__ __device__ DcBatchLayout(int nb, int nv, int c) {
-        cap = (nb + c - 1) / c * 16 + 16;                             // entries of a rank, padded to whole steps
+    int col_off, red_off, total;
+    __host__ __device__ DcBatchLayout(int nb, int nv) {
+        const int cap = nb * 16 + 16;
         col_off = cap * nv * 2;
         red_off = (col_off + cap * 2 + 15) & ~15;
-        total = red_off + DCB_WARPS / 2 * nv * DC_ROWS * 4;
+        total = red_off + DCB_SLOTS * nv * DC_ROWS * 4;
     }
 };
 
-static_assert(DC_MAX_COLUMNS < 65536, "16-bit columns");
-// its static shared memory (the sums of the ranks, a few words), rounded up
-__host__ __device__ constexpr int dcb_static(int nv, int c) { return (c > 1 ? c : 1) * nv * DC_ROWS * 4 + 256; }
-
-// Up to NV vectors.  Fragment lane (g, t) = (lane / 4, lane % 4) of a step: rows 4 g .. 4 g + 3 of columns 2 t, 2 t + 1, 2 t + 8, 2 t + 9.  N tile i
-// holds the rows 4 g' + i, g' = 0 .. 7, so that a lane's four rows of a column are its elements of the four tiles.
-template <int NV, int C>
-__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(DCB_CTA, 2)
+// Up to NV vectors, one thread block per SM; y is zeroed in front.  The work -- strips times steps of 16 columns of the
+// list -- is cut into equal pieces, one per thread block, whatever strip they begin in; a piece ends in one atomic per row and vector for every strip it
+// touches.  (A thread block per strip left 172 strips to 148 SMs: 42 us for 11008 x 4096 and eight vectors.)
+// Every thread block builds the same list (counts and scans, no atomics), and stages the x values of the steps it visits.
+// Fragment lane (g, t) = (lane / 4, lane % 4) of a step: rows 8 g .. 8 g + 7 of columns 2 t, 2 t + 1, 2 t + 8, 2 t + 9.  N tile i
+// holds the rows 8 g' + i, g' = 0 .. 7, so that a lane's eight rows of a column are its elements of the eight tiles.
+template <int NV>
+__global__ void __launch_bounds__(DCB_CTA, 1)
 k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__restrict__ y, int64_t ldy, int nvec, float th3, int force_path) {
-    namespace cg = cooperative_groups;
     extern __shared__ __align__(16) uint8_t s_dyn[];
-    const DcBatchLayout lay(d.nb, NV, C);
-    uint16_t *s_x = reinterpret_cast<uint16_t *>(s_dyn);
+    const DcBatchLayout lay(d.nb, NV);
+    uint32_t *s_x = reinterpret_cast<uint32_t *>(s_dyn);
     uint16_t *s_col = reinterpret_cast<uint16_t *>(s_dyn + lay.col_off);
     float *s_red = reinterpret_cast<float *>(s_dyn + lay.red_off);
-    __shared__ float s_sum[C > 1 ? C : 1][NV * DC_ROWS];
-    __shared__ int s_n, s_nz, s_seen[C];
+    __shared__ int s_cnt[DCB_WARPS], s_nz[DCB_WARPS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int rank = C > 1 ? (int)cg::this_cluster().block_rank() : 0;
-    if (tid == 0) { s_n = 0; s_nz = 0; }
     pdl_wait();
-    if (C > 1) cg::this_cluster().sync(); else __syncthreads();
+    // ---- the list: columns that some vector reaches.  A warp owns consecutive groups of eight entries.
     bool odd = false;
+    uint64_t bits = 0;
+    const int groups = d.nb * 2, rounds = (groups + DCB_CTA - 1) / DCB_CTA, u0 = warp * rounds * 32 + lane;
     {
         const bool aligned = (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && (ldx & 7) == 0;
-        const int units = (d.nb - rank + C - 1) / C * 2;
         int nz = 0;
-        for (int u0 = warp * 32; u0 < units; u0 += DCB_CTA) {
-            const int u = u0 + lane;
-            const int64_t j0 = ((int64_t)(u >> 1) * C + rank) * 16 + (u & 1) * 8;
-            uint32_t h[NV][4];                                        // the entries as bf16 pairs, 0 where one does not take part
-            uint32_t bits = 0;
+        for (int r = 0; r < rounds; ++r) {
+            const int u = u0 + 32 * r, j0 = u * 8;
+            uint4 h[NV];
+            uint32_t in = 0;
 #pragma unroll
             for (int b = 0; b < NV; ++b) {
-                h[b][0] = h[b][1] = h[b][2] = h[b][3] = 0u;
-                if (u < units && b < nvec) {
-                    float v[8];
-                    dc_load8(d, x, ldx, b, j0, aligned, v);
+                h[b] = make_uint4(0u, 0u, 0u, 0u);
+                if (u < groups && b < nvec) h[b] = dc_load8(d, x, ldx, b, j0, aligned);
+            }
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const bool in = j0 + k < d.n && decode_takes_part(d, v[k]);
-                        odd |= in && !dc_finite(v[k]);
-                        bits |= (in ? 1u : 0u) << k;
-                        if (in) h[b][k >> 1] |= (__float_as_uint(v[k]) >> 16) << (16 * (k & 1));
+            for (int b = 0; b < NV; ++b) {
+                if (b >= nvec) break;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const float e = dc_entry(h[b], k);
+                    if (j0 + k < (int)d.n && decode_takes_part(d, e)) { in |= 1u << k; odd |= !dc_finite(e); }
+                }
+            }
+            bits |= (uint64_t)in << (8 * r);
+            nz += __popc(__ballot_sync(FULL, in | __shfl_xor_sync(FULL, in, 1)) & 0x55555555u);
+        }
+        const int cnt = __popcll(bits);
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
+        if (lane == 31) { s_cnt[warp] = incl; s_nz[warp] = nz; }
+        odd = __syncthreads_or(odd);
+        int at = incl - cnt;
+        for (int k = 0; k < warp; ++k) at += s_cnt[k];
+        for (int r = 0; r < rounds; ++r)
+            for (uint32_t m = (uint32_t)(bits >> (8 * r)) & 0xFFu; m; m &= m - 1) s_col[at++] = (uint16_t)((u0 + 32 * r) * 8 + __ffs(m) - 1);
+    }
+    int n = 0;
+#pragma unroll
+    for (int k = 0; k < DCB_WARPS; ++k) n += s_cnt[k];
+    if (blockIdx.x == 0 && tid == 0) {
+        int nz = 0;
+        for (int k = 0; k < DCB_WARPS; ++k) nz += s_nz[k];
+        dc_record(d, nz, th3, force_path);
+    }
+    const int n_steps = (n + 15) >> 4, strips = (int)((d.m + DC_ROWS - 1) / DC_ROWS);
+    if (n + tid < n_steps * 16) s_col[n + tid] = 0;                   // (at most 15: the last step is filled up with column 0 times 0)
+    __syncthreads();
+    // this block's piece; a non-finite entry: whole strips instead, element by element
+    const int64_t work = (int64_t)strips * (odd ? 1 : n_steps);
+    const int64_t lo = work * blockIdx.x / gridDim.x, hi = work * (blockIdx.x + 1) / gridDim.x;
+    if (lo >= hi) return;                                             // block-uniform
+    if (!odd) {
+        // the values, a thread per pair of list entries.  The vector's place is rotated by the pair so that neither the writes
+        // here (32 pairs, one vector) nor the fragment reads (four pairs, NV vectors) meet in a bank.
+        const int first = (int)(lo % n_steps), last = (int)((hi - 1) % n_steps);
+        const bool whole = hi - lo >= n_steps;
+        for (int p = tid; p < n_steps * 8; p += DCB_CTA) {
+            const int s = p >> 3;
+            if (!whole && (first <= last ? s < first || s > last : s < first && s > last)) continue;
+            const uint32_t c2 = reinterpret_cast<const uint32_t *>(s_col)[p];
+            float v[NV][2];
+#pragma unroll
+            for (int b = 0; b < NV; ++b) {
+                v[b][0] = v[b][1] = 0.f;
+                if (b < nvec) { v[b][0] = dc_x(d, x, ldx, b, c2 & 0xFFFFu); v[b][1] = dc_x(d, x, ldx, b, c2 >> 16); }
+            }
+            const int rot = (p / (32 / NV)) & (NV - 1);
+#pragma unroll
+            for (int b = 0; b < NV; ++b) {
+                uint32_t w = 0;
+                if (b < nvec && 2 * p < n && decode_takes_part(d, v[b][0])) w = __float_as_uint(v[b][0]) >> 16;
+                if (b < nvec && 2 * p + 1 < n && decode_takes_part(d, v[b][1])) w |= __float_as_uint(v[b][1]) & 0xFFFF0000u;
+                s_x[p * NV + (b ^ rot)] = w;
+            }
+        }
+        __syncthreads();
+    }
+    const int g = lane >> 2, t = lane & 3;
+    for (int64_t pos = lo; pos < hi;) {
+        const int per = odd ? 1 : n_steps, strip = (int)(pos / per), sa = (int)(pos % per);
+        const int sb = (int)(hi - pos < per - sa ? sa + (hi - pos) : per);
+        float *red = s_red + (warp % DCB_SLOTS) * NV * DC_ROWS;
+        if (odd) {
+            float a[NV][DC_PER_LANE];
+            dc_slow<NV>(d, x, ldx, nvec, strip, warp, DCB_WARPS, lane, a);
+            for (int q = DCB_WARPS / DCB_SLOTS - 1; q >= 0; --q) {
+                if (warp / DCB_SLOTS == q)
+#pragma unroll
+                    for (int k = 0; k < NV * DC_PER_LANE; ++k) red[k * 32 + lane] = a[k / DC_PER_LANE][k % DC_PER_LANE] + (q == DCB_WARPS / DCB_SLOTS - 1 ? 0.f : red[k * 32 + lane]);
+                __syncthreads();
+            }
+        } else {
+            float acc[8][4];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+            const uint4 *w = d.cols + (size_t)strip * d.n * (DC_ROWS / 8) + g;
+            for (int s0 = sa + warp; s0 < sb; s0 += DCB_WARPS * DCB_ILP) {
+                uint4 v[DCB_ILP][4];
+#pragma unroll
+                for (int u = 0; u < DCB_ILP; ++u) {
+                    const int s = s0 + u * DCB_WARPS;
+                    if (s < sb) {                                     // warp-uniform
+                        const uint32_t c01 = *reinterpret_cast<const uint32_t *>(s_col + s * 16 + 2 * t), c89 = *reinterpret_cast<const uint32_t *>(s_col + s * 16 + 8 + 2 * t);
+                        v[u][0] = __ldcs(w + (size_t)(c01 & 0xFFFFu) * (DC_ROWS / 8));
+                        v[u][1] = __ldcs(w + (size_t)(c01 >> 16) * (DC_ROWS / 8));
+                        v[u][2] = __ldcs(w + (size_t)(c89 & 0xFFFFu) * (DC_ROWS / 8));
+                        v[u][3] = __ldcs(w + (size_t)(c89 >> 16) * (DC_ROWS / 8));
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < DCB_ILP; ++u) {
+                    const int s = s0 + u * DCB_WARPS;
+                    if (s >= sb) break;
+                    uint32_t a0 = 0u, a2 = 0u;
+                    if (g < NV) {
+                        const int p = s * 8 + t;
+                        a0 = s_x[p * NV + (g ^ ((p / (32 / NV)) & (NV - 1)))];
+                        a2 = s_x[(p + 4) * NV + (g ^ (((p + 4) / (32 / NV)) & (NV - 1)))];
+                    }
+                    const uint32_t q[4][4] = {{v[u][0].x, v[u][0].y, v[u][0].z, v[u][0].w}, {v[u][1].x, v[u][1].y, v[u][1].z, v[u][1].w},
+                                              {v[u][2].x, v[u][2].y, v[u][2].z, v[u][2].w}, {v[u][3].x, v[u][3].y, v[u][3].z, v[u][3].w}};
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const uint32_t sel = i & 1 ? 0x7632u : 0x5410u;
+                        mma_bf16_m16n8k16(acc[i], a0, 0u, a2, 0u, __byte_perm(q[0][i >> 1], q[1][i >> 1], sel), __byte_perm(q[2][i >> 1], q[3][i >> 1], sel));
                     }
                 }
             }
-            const int cnt = __popc(bits);
-            int incl = cnt;
+            // sums over the warps, four at a time.  acc[i][0], acc[i][1]: vector g, rows 16 t + i and 16 t + 8 + i
+            for (int q = DCB_WARPS / DCB_SLOTS - 1; q >= 0; --q) {
+                if (warp / DCB_SLOTS == q && g < NV)
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
-            int base = 0;
-            if (lane == 31 && incl) base = atomicAdd(&s_n, incl);
-            int at = __shfl_sync(FULL, base, 31) + incl - cnt;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                if (!((bits >> k) & 1u)) continue;
-                s_col[at] = (uint16_t)(j0 + k);
-#pragma unroll
-                for (int b = 0; b < NV; ++b) s_x[((at >> 1) * NV + b) * 2 + (at & 1)] = (uint16_t)(h[b][k >> 1] >> (16 * (k & 1)));
-                ++at;
-            }
-            nz += __popc(__ballot_sync(FULL, bits | __shfl_xor_sync(FULL, bits, 1)) & 0x55555555u);
-        }
-        if (lane == 0 && nz) atomicAdd(&s_nz, nz);
-        odd = __syncthreads_or(odd);
-        if (C > 1) {
-            cg::cluster_group cluster = cg::this_cluster();
-            if (tid < C) cluster.map_shared_rank(s_seen, tid)[rank] = s_nz | (odd ? DC_SLOW_FLAG : 0);
-            cluster.sync();
-#pragma unroll
-            for (int r = 0; r < C; ++r) odd |= (s_seen[r] & DC_SLOW_FLAG) != 0;
-        } else if (tid == 0) {
-            s_seen[0] = s_nz;
-        }
-        if (blockIdx.x == 0 && tid == 0) {
-            int total = 0;
-#pragma unroll
-            for (int r = 0; r < C; ++r) total += s_seen[r] & (DC_SLOW_FLAG - 1);
-            dc_record(d, total, th3, force_path);
-        }
-    }
-    const int n = s_n, n_steps = (n + 15) >> 4;
-    if (tid < 16 && n + tid < n_steps * 16) {                         // the last step is filled up with column 0 times 0
-        const int at = n + tid;
-        s_col[at] = 0;
-        for (int b = 0; b < NV; ++b) s_x[((at >> 1) * NV + b) * 2 + (at & 1)] = 0;
-    }
-    __syncthreads();
-    const int g = lane >> 2, t = lane & 3;
-    const uint32_t *xw = reinterpret_cast<const uint32_t *>(s_x);
-    for (int strip = blockIdx.x / C; strip * DC_ROWS < d.m; strip += gridDim.x / C) {
-        float acc[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
-        const uint2 *w = reinterpret_cast<const uint2 *>(d.cols) + (size_t)strip * d.n * (DC_ROWS / 4) + g;
-        for (int s0 = odd ? n_steps : warp; s0 < n_steps; s0 += DCB_WARPS * DCB_ILP) {
-            uint2 v[DCB_ILP][4];
-#pragma unroll
-            for (int u = 0; u < DCB_ILP; ++u) {
-                const int s = s0 + u * DCB_WARPS;
-                if (s < n_steps) {                                    // warp-uniform
-                    const uint32_t lo = *reinterpret_cast<const uint32_t *>(s_col + s * 16 + 2 * t), hi = *reinterpret_cast<const uint32_t *>(s_col + s * 16 + 8 + 2 * t);
-                    v[u][0] = __ldcs(w + (size_t)(lo & 0xFFFFu) * (DC_ROWS / 4));
-                    v[u][1] = __ldcs(w + (size_t)(lo >> 16) * (DC_ROWS / 4));
-                    v[u][2] = __ldcs(w + (size_t)(hi & 0xFFFFu) * (DC_ROWS / 4));
-                    v[u][3] = __ldcs(w + (size_t)(hi >> 16) * (DC_ROWS / 4));
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < DCB_ILP; ++u) {
-                const int s = s0 + u * DCB_WARPS;
-                if (s >= n_steps) break;
-                const uint32_t a0 = g < NV ? xw[(s * 8 + t) * NV + g] : 0u, a2 = g < NV ? xw[(s * 8 + t + 4) * NV + g] : 0u;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint32_t sel = i & 1 ? 0x7632u : 0x5410u;
-                    const uint32_t b0 = __byte_perm(i < 2 ? v[u][0].x : v[u][0].y, i < 2 ? v[u][1].x : v[u][1].y, sel);
-                    const uint32_t b1 = __byte_perm(i < 2 ? v[u][2].x : v[u][2].y, i < 2 ? v[u][3].x : v[u][3].y, sel);
-                    mma_bf16_m16n8k16(acc[i], a0, 0u, a2, 0u, b0, b1);
-                }
+                    for (int i = 0; i < 8; ++i) {
+                        float *o = red + g * DC_ROWS + 16 * t + i;
+                        const bool add = q != DCB_WARPS / DCB_SLOTS - 1;
+                        o[0] = acc[i][0] + (add ? o[0] : 0.f);
+                        o[8] = acc[i][1] + (add ? o[8] : 0.f);
+                    }
+                __syncthreads();
             }
         }
-        // sums over the warps: the upper half hands its sums to the lower half, then a thread per (vector, row) adds up.
-        // acc[i][0], acc[i][1]: vector g, rows 8 t + i and 8 t + 4 + i
-        float *red = s_red + (warp % (DCB_WARPS / 2)) * NV * DC_ROWS;
-        if (odd) {
-            float a[NV];
-            dc_slow<NV>(d, x, ldx, nvec, strip, warp * C + rank, DCB_WARPS * C, lane, a);
-            if (warp >= DCB_WARPS / 2)
+        if (tid < nvec * DC_ROWS) {
+            float sum = 0.f;
 #pragma unroll
-                for (int b = 0; b < NV; ++b) red[b * DC_ROWS + lane] = a[b];
-            __syncthreads();
-            if (warp < DCB_WARPS / 2)
-#pragma unroll
-                for (int b = 0; b < NV; ++b) red[b * DC_ROWS + lane] += a[b];
-        } else {
-            if (warp >= DCB_WARPS / 2 && g < NV)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) { red[g * DC_ROWS + 8 * t + i] = acc[i][0]; red[g * DC_ROWS + 8 * t + 4 + i] = acc[i][1]; }
-            __syncthreads();
-            if (warp < DCB_WARPS / 2 && g < NV)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) { red[g * DC_ROWS + 8 * t + i] += acc[i][0]; red[g * DC_ROWS + 8 * t + 4 + i] += acc[i][1]; }
+            for (int k = 0; k < DCB_SLOTS; ++k) sum += s_red[k * NV * DC_ROWS + tid];
+            const int64_t row = (int64_t)strip * DC_ROWS + tid % DC_ROWS;
+            if (row < d.m) atomicAdd(y + (tid / DC_ROWS) * ldy + row, sum);
         }
         __syncthreads();
-        float sum = 0.f;
-        if (tid < NV * DC_ROWS) {
-#pragma unroll
-            for (int k = 0; k < DCB_WARPS / 2; ++k) sum += s_red[k * NV * DC_ROWS + tid];
-        }
-        if (C > 1) {
-            cg::cluster_group cluster = cg::this_cluster();
-            if (tid < NV * DC_ROWS) cluster.map_shared_rank(&s_sum[0][0], 0)[rank * NV * DC_ROWS + tid] = sum;
-            cluster.sync();
-            if (rank == 0 && tid < NV * DC_ROWS) {
-                sum = 0.f;
-#pragma unroll
-                for (int r = 0; r < C; ++r) sum += s_sum[C > 1 ? r : 0][tid];
-            }
-            cluster.sync();                                           // (the next strip overwrites the sums)
-        }
-        const int b = tid / DC_ROWS;
-        const int64_t row = (int64_t)strip * DC_ROWS + tid % DC_ROWS;
-        if (rank == 0 && b < nvec && b < NV && row < d.m) y[b * ldy + row] = sum;
-        __syncthreads();
+        pos += sb - sa;
     }
 }
 

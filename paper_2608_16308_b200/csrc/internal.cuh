@@ -120,7 +120,7 @@ constexpr int HUB_CAP = 32;
 #endif
 constexpr int STAGE_BYTES = DBS_STAGE_BYTES;
 // Decode over columns (decode_columns.cuh): rows of a strip; the bf16 pattern of an absent element; where the copy is built.
-constexpr int DC_ROWS = 32;
+constexpr int DC_ROWS = 64;
 constexpr uint32_t DC_ABSENT = 0x8000u;
 constexpr int DC_MIN_ROWS = 1024;           // (fewer rows make too few strips: the block kernels deal the payload out over all SMs)
 constexpr int DC_MAX_COLUMNS = 25600;       // the list of active columns has to fit in shared memory
@@ -308,8 +308,7 @@ struct dbspmspv_handle_s {
     bool fused_configured[3];
     bool batch_configured[2];
     bool batch_mma_configured[3];
-    bool cols_configured;
-    int cols_grid[2];           // resident clusters of the batched decode over columns (4 / 8 vectors; 0: does not fit)
+    bool cols_configured, cols_batch_configured[2];
     int stream_grid;            // thread blocks of the streaming decode (0: not configured yet)
     int32_t *x_nnz_seen_host;   // host view of Device::x_nnz_seen (page-locked, mapped)
     bool heavy_stage;           // most stored elements sit in mask-based blocks: MODE 1 kernels

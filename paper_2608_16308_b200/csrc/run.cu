@@ -1308,6 +1308,7 @@ constexpr int STREAM_CTA = STREAM_WARPS * 32;
 #endif
 constexpr int STREAM_DEPTH = DBS_STREAM_DEPTH;
 constexpr int STREAM_MAX_SMEM = 227 * 1024;   // all a thread block may have
+constexpr int DCB_MAX_SMEM = STREAM_MAX_SMEM - 256;   // (static shared memory of k_decode_cols_batch)
 __host__ __device__ constexpr int stream_stride(int stage_bytes) { return (stage_bytes + 127) & ~127; }
 struct StreamLayout {
     int xm_off, cnt_off, active_off, bar_off, ring_off, total;
@@ -2025,51 +2026,48 @@ int decode_stage_bytes(const Device &d) {
     return 0;
 }
 
-// Decode over columns: `nvec` vectors (1, or as many as decode_columns_group says) in one kernel.
+// Decode over columns: `nvec` vectors (1, or at most as many as decode_columns_group says).
 template <int C>
-static int decode_columns_c(dbspmspv_handle_s *h, CallList &calls, const void *x, int64_t ldx, float *y, int64_t ldy, int nvec) {
+static int decode_columns_c(dbspmspv_handle_s *h, CallList &calls, const void *x, float *y) {
     const Device &d = h->d;
     const int strips = (int)((d.m + DC_ROWS - 1) / DC_ROWS);
     if (!h->cols_configured) {
         DBS_CUDA(cudaFuncSetAttribute(k_decode_cols<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSED_MAX_SMEM));
-        // (the attribute belongs to the kernel, not to the handle: all that its static shared memory leaves)
-        DBS_CUDA(cudaFuncSetAttribute(k_decode_cols_batch<4, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, STREAM_MAX_SMEM - dcb_static(4, C)));
-        DBS_CUDA(cudaFuncSetAttribute(k_decode_cols_batch<8, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, STREAM_MAX_SMEM - dcb_static(8, C)));
-        int per_sm = 0;
-        DBS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_decode_cols_batch<4, C>, DCB_CTA, DcBatchLayout(d.nb, 4, C).total));
-        h->cols_grid[0] = per_sm * h->sm_count / C;
-        DBS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_decode_cols_batch<8, C>, DCB_CTA, DcBatchLayout(d.nb, 8, C).total));
-        h->cols_grid[1] = per_sm * h->sm_count / C;
         h->cols_configured = true;
     }
-    if (nvec == 1) {
-        calls.add(k_decode_cols<C>, strips * C, DC_CTA, (size_t)((d.nb + C - 1) / C) * 16 * sizeof(float2), false, d, x, y, h->ropts.th3_decode, h->ropts.force_path);
-        return DBSPMSPV_OK;
-    }
-    const int slots = h->cols_grid[nvec <= 4 ? 0 : 1], g = (strips < slots ? strips : slots) * C;
-    if (g < 1) return DBSPMSPV_ERR_CUDA;
-    calls.add(nvec <= 4 ? k_decode_cols_batch<4, C> : k_decode_cols_batch<8, C>, g, DCB_CTA, (size_t)DcBatchLayout(d.nb, nvec <= 4 ? 4 : 8, C).total, false,
-              d, x, ldx, y, ldy, nvec, h->ropts.th3_decode, h->ropts.force_path);
+    calls.add(k_decode_cols<C>, strips * C, DC_CTA, (size_t)((d.nb + C - 1) / C) * 16 * sizeof(float2), false, d, x, y, h->ropts.th3_decode, h->ropts.force_path);
     return DBSPMSPV_OK;
 }
 static int decode_columns(dbspmspv_handle_s *h, const void *x, int64_t ldx, float *y, int64_t ldy, int nvec, cudaStream_t st) {
     CallList calls;
+    const Device &d = h->d;
     int s = DBSPMSPV_OK;
-    switch (dc_cluster(h->d.m, h->sm_count)) {
-        case 1: s = decode_columns_c<1>(h, calls, x, ldx, y, ldy, nvec); break;
-        case 2: s = decode_columns_c<2>(h, calls, x, ldx, y, ldy, nvec); break;
-        case 4: s = decode_columns_c<4>(h, calls, x, ldx, y, ldy, nvec); break;
-        default: s = decode_columns_c<8>(h, calls, x, ldx, y, ldy, nvec); break;
+    if (nvec == 1) {
+        switch (dc_cluster(d.m, h->sm_count)) {
+            case 1: s = decode_columns_c<1>(h, calls, x, y); break;
+            case 2: s = decode_columns_c<2>(h, calls, x, y); break;
+            case 4: s = decode_columns_c<4>(h, calls, x, y); break;
+            default: s = decode_columns_c<8>(h, calls, x, y); break;
+        }
+        if (s != DBSPMSPV_OK) return s;
+    } else {
+        const int nv = nvec <= 4 ? 4 : 8;
+        auto kernel = nv == 4 ? k_decode_cols_batch<4> : k_decode_cols_batch<8>;
+        if (!h->cols_batch_configured[nv / 8]) {
+            // (the attribute belongs to the kernel, not to the handle: the largest size)
+            DBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DCB_MAX_SMEM));
+            h->cols_batch_configured[nv / 8] = true;
+        }
+        calls.add(k_zero_rows, (int)((d.m + 1023) / 1024), 256, 0, false, y, ldy, d.m, nvec);
+        calls.add(kernel, h->sm_count, DCB_CTA, (size_t)DcBatchLayout(d.nb, nv).total, true, d, x, ldx, y, ldy, nvec, h->ropts.th3_decode, h->ropts.force_path);
     }
-    if (s != DBSPMSPV_OK) return s;
     if (h->ropts.timing) { calls.ev_before = 0; calls.ev_after = calls.n; h->timed = true; }
     return submit_calls(h, calls, st);
 }
 // vectors of one batched call over columns, at most (1: the lists of several do not fit in shared memory)
 static int decode_columns_group(const dbspmspv_handle_s *h) {
-    const int c = dc_cluster(h->d.m, h->sm_count);
     for (int nv : {8, 4})
-        if (DcBatchLayout(h->d.nb, nv, c).total + dcb_static(nv, c) <= STREAM_MAX_SMEM) return nv;
+        if (DcBatchLayout(h->d.nb, nv).total <= DCB_MAX_SMEM) return nv;
     return 1;
 }
 

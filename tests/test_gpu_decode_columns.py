@@ -1,4 +1,4 @@
-"""The decode over columns of bf16 layers (automatic mode, 1024 rows or more): strips of 32 rows, one or
+"""The decode over columns of bf16 layers (automatic mode, 1024 rows or more): strips of 64 rows, one or
 several thread blocks per strip, one to nine vectors, sizes off every tile edge, activation options,
 non-finite activations, a weight that is stored as -0."""
 import numpy as np
@@ -24,7 +24,7 @@ def check(y, want, scale):
     assert (y[fin & (scale == 0)] == 0.0).all()
 
 
-# 33 strips (8 then 4 blocks each), 128 / 149 strips (1), rows and columns off the tiles, and a wide one
+# 17 / 18 strips (8 blocks each), 38 (2), 75 (1), 16 (8); rows and columns off the tiles, and a wide one
 @pytest.mark.parametrize("shape,prune", [((1025, 333), 0.5), ((1100, 1000), 0.7), ((2400, 17), 0.6), ((4768, 260), 0.5), ((1024, 12289), 0.5)])
 @pytest.mark.parametrize("x_f32", [0, 1])
 def test_decode_over_columns(shape, prune, x_f32):
