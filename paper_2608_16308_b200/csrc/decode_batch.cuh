@@ -515,6 +515,8 @@ k_decode_batch_mma(Device d, const void *__restrict__ x, int64_t ldx, float *__r
 
 __global__ void k_zero_rows(float *y, int64_t ldy, int64_t m, int nvec) {
     pdl_wait();
+    // the one early start: the kernel behind blocks x meanwhile, which takes a thread block per SM and none of this kernel's room
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int v = 0; v < nvec; ++v)
         for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += stride) y[(size_t)v * ldy + i] = 0.f;

@@ -55,7 +55,24 @@ __device__ __forceinline__ float dc_entry(const uint4 &u, int k) {       // entr
     const uint32_t w = k < 2 ? u.x : k < 4 ? u.y : k < 6 ? u.z : u.w;
     return __uint_as_float(k & 1 ? w & 0xFFFF0000u : w << 16);
 }
-__device__ __forceinline__ bool dc_finite(float v) { return (__float_as_uint(v) & 0x7F800000u) != 0x7F800000u; }
+
+// Which entries of a pair of bf16 take part (see decode_takes_part), two at a time: magnitude bits compared by a carry
+// into the halfword's top bit.  |v| > tau is a comparison of magnitude bits (tau's own low half can be dropped); with the
+// ReLU a negative entry takes part only if it is a NaN.
+struct DcTest {
+    uint32_t k, s;
+    __device__ __forceinline__ explicit DcTest(const Device &d) {
+        k = (0x7FFFu - (__float_as_uint(d.decode_tau) >> 16)) * 0x10001u;
+        s = d.decode_relu ? 0u : 0xFFFFFFFFu;
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t w) const {       // bits 15 and 31
+        const uint32_t a = w & 0x7FFF7FFFu;
+        return (a + k) & (~w | s | (a + 0x007F007Fu)) & 0x80008000u;
+    }
+};
+__device__ __forceinline__ uint32_t dc_odd(uint32_t w) { return ((w & 0x7FFF7FFFu) + 0x00800080u) & 0x80008000u; }     // infinite or NaN
+__device__ __forceinline__ uint32_t dc_pair_bits(uint32_t m) { return ((m >> 15) & 1u) | ((m >> 30) & 2u); }
+__device__ __forceinline__ uint32_t dc_pair_mask(uint32_t m) { return ((m >> 15) & 0x00010001u) * 0xFFFFu; }
 
 // The calls with a non-finite x entry: a lane takes the rows lane, lane + 32 of the strip, a column at a time, every element tested.
 constexpr int DC_PER_LANE = DC_ROWS / 32;
@@ -118,6 +135,7 @@ k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float
     // ---- the list of the entries that take part: eight consecutive ones per thread and round, this rank's vector blocks only
     {
         const bool aligned = (reinterpret_cast<uintptr_t>(x) & 15u) == 0;
+        const DcTest test(d);
         const int units = (d.nb - rank + C - 1) / C * 2;             // halves of this rank's vector blocks
         int nz = 0;
         for (int u0 = warp * 32; u0 < units; u0 += DC_CTA * DC_XILP) {
@@ -134,9 +152,13 @@ k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float
 #pragma unroll
             for (int q = 0; q < DC_XILP; ++q) {
                 if (u0 + q * DC_CTA >= units) break;                  // warp-uniform
+                const uint32_t w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};       // (entries past n are 0: they never take part)
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    bits |= (j0[q] + k < (int)d.n && decode_takes_part(d, dc_entry(v[q], k)) ? 1u : 0u) << (8 * q + k);
+                for (int k = 0; k < 4; ++k) {
+                    const uint32_t m = test(w[k]);
+                    bits |= dc_pair_bits(m) << (8 * q + 2 * k);
+                    odd |= (m & dc_odd(w[k])) != 0u;
+                }
             }
             const int cnt = __popc(bits);
             int incl = cnt;
@@ -152,9 +174,7 @@ k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
                     if ((bits >> (8 * q + k)) & 1u) {
-                        const float e = dc_entry(v[q], k);
-                        s_list[at++] = make_float2(__int_as_float(j0[q] + k), e);
-                        odd |= !dc_finite(e);
+                        s_list[at++] = make_float2(__int_as_float(j0[q] + k), dc_entry(v[q], k));
                     }
                 nz += __popc(__ballot_sync(FULL, (both >> (8 * q)) & 0xFFu) & 0x55555555u);
             }
@@ -265,7 +285,7 @@ struct DcBatchLayout {
 // Up to NV vectors, one thread block per SM; y is zeroed in front.  The work -- strips times steps of 16 columns of the
 // list -- is cut into equal pieces, one per thread block, whatever strip they begin in; a piece ends in one atomic per row and vector for every strip it
 // touches.  (A thread block per strip left 172 strips to 148 SMs: 42 us for 11008 x 4096 and eight vectors.)
-// Every thread block builds the same list (counts and scans, no atomics), and stages the x values of the steps it visits.
+// Every thread block builds the same list (counts and scans, no atomics).
 // Fragment lane (g, t) = (lane / 4, lane % 4) of a step: rows 8 g .. 8 g + 7 of columns 2 t, 2 t + 1, 2 t + 8, 2 t + 9.  N tile i
 // holds the rows 8 g' + i, g' = 0 .. 7, so that a lane's eight rows of a column are its elements of the eight tiles.
 template <int NV>
@@ -278,46 +298,54 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
     float *s_red = reinterpret_cast<float *>(s_dyn + lay.red_off);
     __shared__ int s_cnt[DCB_WARPS], s_nz[DCB_WARPS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    pdl_wait();
-    // ---- the list: columns that some vector reaches.  A warp owns consecutive groups of eight entries.
+    // (x may be read before the wait: the kernel in front zeroes y, and let this one start when everything before it had ended)
+    // ---- x into shared memory: the entries that take part, by pairs of columns, and the union of the vectors' columns.
+    // A warp owns consecutive groups of eight columns; word (pair, vector) is rotated inside its row of 32 words so that neither the
+    // writes (32 pairs, one vector) nor the fragment reads (four pairs, NV vectors) meet in a bank.
+    constexpr int PAIRS = 32 / NV;                                     // pairs per row
+    auto place = [&](int p, int b) { return p / PAIRS * 32 + (((p % PAIRS) * NV + b) ^ (p / PAIRS & 31)); };
     bool odd = false;
     uint64_t bits = 0;
     const int groups = d.nb * 2, rounds = (groups + DCB_CTA - 1) / DCB_CTA, u0 = warp * rounds * 32 + lane;
+    const DcTest test(d);
     {
         const bool aligned = (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && (ldx & 7) == 0;
         int nz = 0;
         for (int r = 0; r < rounds; ++r) {
-            const int u = u0 + 32 * r, j0 = u * 8;
+            const int u = u0 + 32 * r;
             uint4 h[NV];
-            uint32_t in = 0;
 #pragma unroll
             for (int b = 0; b < NV; ++b) {
                 h[b] = make_uint4(0u, 0u, 0u, 0u);
-                if (u < groups && b < nvec) h[b] = dc_load8(d, x, ldx, b, j0, aligned);
+                if (u < groups && b < nvec) h[b] = dc_load8(d, x, ldx, b, (int64_t)u * 8, aligned);
             }
+            uint32_t any[4] = {0u, 0u, 0u, 0u}, strange = 0u;
 #pragma unroll
             for (int b = 0; b < NV; ++b) {
-                if (b >= nvec) break;
+                const uint32_t w[4] = {h[b].x, h[b].y, h[b].z, h[b].w};
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const float e = dc_entry(h[b], k);
-                    if (j0 + k < (int)d.n && decode_takes_part(d, e)) { in |= 1u << k; odd |= !dc_finite(e); }
+                for (int k = 0; k < 4; ++k) {
+                    const uint32_t m = test(w[k]);
+                    any[k] |= m;
+                    strange |= m & dc_odd(w[k]);
+                    if (u < groups) s_x[place(u * 4 + k, b)] = w[k] & dc_pair_mask(m);
                 }
             }
+            odd |= strange != 0u;
+            uint32_t in = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) in |= dc_pair_bits(any[k]) << (2 * k);
             bits |= (uint64_t)in << (8 * r);
             nz += __popc(__ballot_sync(FULL, in | __shfl_xor_sync(FULL, in, 1)) & 0x55555555u);
         }
-        const int cnt = __popcll(bits);
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
-        if (lane == 31) { s_cnt[warp] = incl; s_nz[warp] = nz; }
-        odd = __syncthreads_or(odd);
-        int at = incl - cnt;
-        for (int k = 0; k < warp; ++k) at += s_cnt[k];
-        for (int r = 0; r < rounds; ++r)
-            for (uint32_t m = (uint32_t)(bits >> (8 * r)) & 0xFFu; m; m &= m - 1) s_col[at++] = (uint16_t)((u0 + 32 * r) * 8 + __ffs(m) - 1);
+        if (lane == 31) s_nz[warp] = nz;
     }
+    const int cnt = __popcll(bits);
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
+    if (lane == 31) s_cnt[warp] = incl;
+    odd = __syncthreads_or(odd);
     int n = 0;
 #pragma unroll
     for (int k = 0; k < DCB_WARPS; ++k) n += s_cnt[k];
@@ -326,35 +354,37 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
         for (int k = 0; k < DCB_WARPS; ++k) nz += s_nz[k];
         dc_record(d, nz, th3, force_path);
     }
-    const int n_steps = (n + 15) >> 4, strips = (int)((d.m + DC_ROWS - 1) / DC_ROWS);
-    if (n + tid < n_steps * 16) s_col[n + tid] = 0;                   // (at most 15: the last step is filled up with column 0 times 0)
-    __syncthreads();
+    // Most columns reached: all of them are taken, as they lie.  Else the union becomes a list, and the values are staged once more, by list entry.
+    const bool all = (int64_t)n * 4 >= d.n * 3;
+    const int n_steps = all ? d.nb : (n + 15) >> 4, strips = (int)((d.m + DC_ROWS - 1) / DC_ROWS);
     // this block's piece; a non-finite entry: whole strips instead, element by element
     const int64_t work = (int64_t)strips * (odd ? 1 : n_steps);
     const int64_t lo = work * blockIdx.x / gridDim.x, hi = work * (blockIdx.x + 1) / gridDim.x;
     if (lo >= hi) return;                                             // block-uniform
-    if (!odd) {
-        // the values, a thread per pair of list entries.  The vector's place is rotated by the pair so that neither the writes
-        // here (32 pairs, one vector) nor the fragment reads (four pairs, NV vectors) meet in a bank.
+    if (!odd && !all) {
+        int at = incl - cnt;
+        for (int k = 0; k < warp; ++k) at += s_cnt[k];
+        for (int r = 0; r < rounds; ++r)
+            for (uint32_t m = (uint32_t)(bits >> (8 * r)) & 0xFFu; m; m &= m - 1) s_col[at++] = (uint16_t)((u0 + 32 * r) * 8 + __ffs(m) - 1);
+        if (n + tid < n_steps * 16) s_col[n + tid] = 0;               // (at most 15: the last step is filled up with column 0 times 0)
+        __syncthreads();
         const int first = (int)(lo % n_steps), last = (int)((hi - 1) % n_steps);
         const bool whole = hi - lo >= n_steps;
         for (int p = tid; p < n_steps * 8; p += DCB_CTA) {
             const int s = p >> 3;
-            if (!whole && (first <= last ? s < first || s > last : s < first && s > last)) continue;
+            if (!whole && (first <= last ? s < first || s > last : s < first && s > last)) continue;      // (a step this block does not visit)
             const uint32_t c2 = reinterpret_cast<const uint32_t *>(s_col)[p];
             float v[NV][2];
 #pragma unroll
             for (int b = 0; b < NV; ++b) {
                 v[b][0] = v[b][1] = 0.f;
-                if (b < nvec) { v[b][0] = dc_x(d, x, ldx, b, c2 & 0xFFFFu); v[b][1] = dc_x(d, x, ldx, b, c2 >> 16); }
+                if (b < nvec && 2 * p < n) v[b][0] = dc_x(d, x, ldx, b, c2 & 0xFFFFu);
+                if (b < nvec && 2 * p + 1 < n) v[b][1] = dc_x(d, x, ldx, b, c2 >> 16);
             }
-            const int rot = (p / (32 / NV)) & (NV - 1);
 #pragma unroll
             for (int b = 0; b < NV; ++b) {
-                uint32_t w = 0;
-                if (b < nvec && 2 * p < n && decode_takes_part(d, v[b][0])) w = __float_as_uint(v[b][0]) >> 16;
-                if (b < nvec && 2 * p + 1 < n && decode_takes_part(d, v[b][1])) w |= __float_as_uint(v[b][1]) & 0xFFFF0000u;
-                s_x[p * NV + (b ^ rot)] = w;
+                const uint32_t w = (__float_as_uint(v[b][0]) >> 16) | (__float_as_uint(v[b][1]) & 0xFFFF0000u);
+                s_x[place(p, b)] = w & dc_pair_mask(test(w));
             }
         }
         __syncthreads();
@@ -384,11 +414,16 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
                 for (int u = 0; u < DCB_ILP; ++u) {
                     const int s = s0 + u * DCB_WARPS;
                     if (s < sb) {                                     // warp-uniform
-                        const uint32_t c01 = *reinterpret_cast<const uint32_t *>(s_col + s * 16 + 2 * t), c89 = *reinterpret_cast<const uint32_t *>(s_col + s * 16 + 8 + 2 * t);
-                        v[u][0] = __ldcs(w + (size_t)(c01 & 0xFFFFu) * (DC_ROWS / 8));
-                        v[u][1] = __ldcs(w + (size_t)(c01 >> 16) * (DC_ROWS / 8));
-                        v[u][2] = __ldcs(w + (size_t)(c89 & 0xFFFFu) * (DC_ROWS / 8));
-                        v[u][3] = __ldcs(w + (size_t)(c89 >> 16) * (DC_ROWS / 8));
+                        uint32_t c[4];
+                        if (all) {                                    // (a column past n has no values: any address will do)
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) c[k] = min((uint32_t)(s * 16 + 2 * t + (k & 1) + 4 * (k & 2)), (uint32_t)d.n - 1u);
+                        } else {
+                            const uint32_t c01 = *reinterpret_cast<const uint32_t *>(s_col + s * 16 + 2 * t), c89 = *reinterpret_cast<const uint32_t *>(s_col + s * 16 + 8 + 2 * t);
+                            c[0] = c01 & 0xFFFFu; c[1] = c01 >> 16; c[2] = c89 & 0xFFFFu; c[3] = c89 >> 16;
+                        }
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) v[u][k] = __ldcs(w + (size_t)c[k] * (DC_ROWS / 8));
                     }
                 }
 #pragma unroll
@@ -398,8 +433,8 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
                     uint32_t a0 = 0u, a2 = 0u;
                     if (g < NV) {
                         const int p = s * 8 + t;
-                        a0 = s_x[p * NV + (g ^ ((p / (32 / NV)) & (NV - 1)))];
-                        a2 = s_x[(p + 4) * NV + (g ^ (((p + 4) / (32 / NV)) & (NV - 1)))];
+                        a0 = s_x[place(p, g)];
+                        a2 = s_x[place(p + 4, g)];
                     }
                     const uint32_t q[4][4] = {{v[u][0].x, v[u][0].y, v[u][0].z, v[u][0].w}, {v[u][1].x, v[u][1].y, v[u][1].z, v[u][1].w},
                                               {v[u][2].x, v[u][2].y, v[u][2].z, v[u][2].w}, {v[u][3].x, v[u][3].y, v[u][3].z, v[u][3].w}};
@@ -423,6 +458,7 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
                 __syncthreads();
             }
         }
+        pdl_wait();                                                   // (y has been zeroed)
         if (tid < nvec * DC_ROWS) {
             float sum = 0.f;
 #pragma unroll

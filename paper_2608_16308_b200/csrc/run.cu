@@ -2058,7 +2058,7 @@ static int decode_columns(dbspmspv_handle_s *h, const void *x, int64_t ldx, floa
             DBS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DCB_MAX_SMEM));
             h->cols_batch_configured[nv / 8] = true;
         }
-        calls.add(k_zero_rows, (int)((d.m + 1023) / 1024), 256, 0, false, y, ldy, d.m, nvec);
+        calls.add(k_zero_rows, (int)((d.m + 255) / 256), 256, 0, false, y, ldy, d.m, nvec);
         calls.add(kernel, h->sm_count, DCB_CTA, (size_t)DcBatchLayout(d.nb, nv).total, true, d, x, ldx, y, ldy, nvec, h->ropts.th3_decode, h->ropts.force_path);
     }
     if (h->ropts.timing) { calls.ev_before = 0; calls.ev_after = calls.n; h->timed = true; }
@@ -2207,7 +2207,7 @@ static int decode_batch_typed(dbspmspv_handle_s *h, const void *x, int64_t ldx, 
         }
         CallList calls;
         if (h->ropts.timing) calls.ev_before = 0;
-        calls.add(k_zero_rows, (int)((d.m + 1023) / 1024), 256, 0, false, yg, ldy, d.m, g);
+        calls.add(k_zero_rows, (int)((d.m + 255) / 256), 256, 0, false, yg, ldy, d.m, g);
         if (DT == DBSPMSPV_BF16 && max_mma > 1) {
             const int nb = g <= 2 ? 2 : g <= 4 ? 4 : 8;
             const BatchMmaLayout lay(d.nb, nb, d.stage_bytes);
