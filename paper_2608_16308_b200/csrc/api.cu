@@ -211,6 +211,7 @@ int dbspmspv_destroy(dbspmspv_handle_t h) {
     cudaFree(h->csc2csr); cudaFree(h->block_row);
     cudaFree(h->ws_arena);
     cudaFree(h->sssp_arena);
+    cudaFree(h->sssp_state);
     if (h->sssp_host) cudaFreeHost(h->sssp_host);
     if (h->ev[0]) cudaEventDestroy(h->ev[0]);
     if (h->ev[1]) cudaEventDestroy(h->ev[1]);

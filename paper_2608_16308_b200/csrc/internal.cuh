@@ -321,7 +321,8 @@ struct dbspmspv_handle_s {
     int64_t stage_index_bytes;
     void *ws_arena;             // the one allocation that holds the whole workspace
     void *sssp_arena;           // db_sssp: frontier lists, y and counters (allocated by the first search)
-    int32_t *sssp_host;         // db_sssp: page-locked word the size of the next frontier is copied to
+    void *sssp_state;           // db_sssp in one launch: words, frontiers, counters (allocated by the first search)
+    int32_t *sssp_host;         // db_sssp: page-locked words the size of the next frontier is copied to
     dbs::CallGraphs *graphs;    // launch graphs of the calls made on this handle
     cudaStream_t last_stream;   // stream of the last run / decode / bfs call (get_stats waits on it)
 };

@@ -1530,6 +1530,7 @@ k_decode_stream(Device d, const void *__restrict__ x, float *__restrict__ y, flo
 #include "decode_batch.cuh"
 #include "small_call.cuh"
 #include "decode_columns.cuh"
+#include "sssp.cuh"
 namespace dbs {
 
 // ------------------------------------------------------------------------------------------
@@ -2287,15 +2288,49 @@ __global__ void k_sssp_relax(Device d, const int32_t *__restrict__ y_idx, const 
     }
 }
 
+// The whole search as one cooperative launch (sssp.cuh).
+template <int DT>
+static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32_t *n_steps, cudaStream_t st) {
+    const Device &d = h->d;
+    SsspState s;
+    s.n_words = (int32_t)((d.n + 31) / 32);
+    const size_t word_bytes = ((size_t)s.n_words * 32 * sizeof(int) + 255) & ~(size_t)255, bit_bytes = ((size_t)s.n_words * 4 + 255) & ~(size_t)255;
+    if (!h->sssp_host && cudaHostAlloc(reinterpret_cast<void **>(&h->sssp_host), 4 * sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess) { h->sssp_host = nullptr; return DBSPMSPV_ERR_ALLOC; }
+    if (!h->sssp_state) {
+        if (cudaMalloc(&h->sssp_state, word_bytes + 2 * bit_bytes + 64) != cudaSuccess) { h->sssp_state = nullptr; return DBSPMSPV_ERR_ALLOC; }
+        DBS_CUDA(cudaFuncSetAttribute(k_sssp<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsspShared)));
+    }
+    uint8_t *p = static_cast<uint8_t *>(h->sssp_state);
+    s.word = reinterpret_cast<int *>(p);
+    s.bits[0] = reinterpret_cast<uint32_t *>(p + word_bytes);
+    s.bits[1] = reinterpret_cast<uint32_t *>(p + word_bytes + bit_bytes);
+    s.ctr = reinterpret_cast<int32_t *>(p + word_bytes + 2 * bit_bytes);
+    s.report = h->sssp_host;
+    Device dev = d;
+    int start = 1;
+    for (int64_t made = 0;; start = 0) {
+        int max_steps = (int)(d.n + 1 - made < SSSP_MAX_STEPS ? d.n + 1 - made : SSSP_MAX_STEPS);
+        void *args[] = {&dev, &s, &src, &dist, &start, &max_steps};
+        DBS_CUDA(cudaLaunchCooperativeKernel((void *)k_sssp<DT>, dim3(h->sm_count), dim3(SSSP_CTA), args, sizeof(SsspShared), st));
+        ++h->kernel_launches;
+        DBS_CUDA(cudaStreamSynchronize(st));
+        made = h->sssp_host[0];
+        if (h->sssp_host[1] == 0) { if (n_steps) *n_steps = (int32_t)made; return DBSPMSPV_OK; }
+        if (made >= d.n + 1) return DBSPMSPV_ERR_UNSUPPORTED;          // a cycle of negative weight
+    }
+}
+
 template <int DT>
 static int sssp_typed(dbspmspv_handle_s *h, int32_t src, float *dist, int32_t *n_steps, cudaStream_t st) {
     const Device &d = h->d;
     const int64_t n = d.n;
+    if (!h->heavy_stage && h->ropts.force_path == DBSPMSPV_PATH_AUTO) return sssp_one_launch<DT>(h, src, dist, n_steps, st);
+    // handles whose elements sit mostly in blocks with a payload, and forced directions: (min, +) products in a host loop
     if (!h->sssp_arena) {
         // two x lists (the relaxation writes the one the running product does not read), y, two counters
         const size_t bytes = (size_t)n * (4 * sizeof(int32_t) + 2 * sizeof(float)) + 64;
         if (cudaMalloc(&h->sssp_arena, bytes) != cudaSuccess) { h->sssp_arena = nullptr; return DBSPMSPV_ERR_ALLOC; }
-        if (cudaHostAlloc(reinterpret_cast<void **>(&h->sssp_host), 4 * sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess) return DBSPMSPV_ERR_ALLOC;
+        if (!h->sssp_host && cudaHostAlloc(reinterpret_cast<void **>(&h->sssp_host), 4 * sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess) return DBSPMSPV_ERR_ALLOC;
     }
     int32_t *xi[2], *y_idx, *ctr;
     float *xv[2], *y_val;

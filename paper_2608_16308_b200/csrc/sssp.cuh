@@ -1,0 +1,280 @@
+// db_sssp on hypersparse handles: the whole search in one cooperative launch, no accumulator and no sparse vectors in between.
+//
+// The search is the synchronous iteration of (min, +) products: step t relaxes the out-edges of the
+// vertices whose distance improved in step t - 1, with the distances they had at the end of that step.  As a host loop over
+// dbspmspv_run it paid, per step, a blocking of x, an accumulator that was filled and compacted, a relaxation pass and a
+// round trip to the host (R-MAT scale 20: 9 steps, 1.17 ms, of which 0.2 ms an idle GPU).  Here a step is
+//   expand   the columns of the frontier (a bitmap) laid end to end per thread block as in the direct push (push_direct.cuh); a candidate
+//            distance goes straight into the target's word with an atomic minimum, and the thread whose atomic lowered
+//            it marks the target in the next frontier;
+//   long     the listed long runs and payload runs, a warp per chunk (only if there are any);
+//   settle   the marked vertices copy their word into the caller's distances -- the values the next
+//            step starts from, which no one lowers meanwhile -- and are counted;
+// with a grid barrier after each.  A step finds the same improvements, distance for distance, as the product did: `word`
+// holds the minimum over everything seen so far, a vertex is marked iff its word went below the distance it had before the step.
+//
+// What bounds a large step is the gather of one target word per edge.  It goes through L1 first (a stale word is never too small,
+// so a candidate that does not beat it is done); only a candidate that does looks at L2, and only one that beats that too pays an atomic:
+// the words of hub rows, which thousands of edges reach, settle after a few atomics.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include "internal.cuh"
+#include "minplus.cuh"
+#include "push_direct.cuh"
+
+namespace dbs {
+
+constexpr int SSSP_CTA = 1024;
+constexpr int SSSP_WARPS = SSSP_CTA / 32;
+constexpr int SSSP_WORDS = SSSP_CTA / 8;          // frontier words of a thread block's round: eight threads per word, four columns each
+constexpr int SSSP_COLS = SSSP_CTA * 4;
+constexpr int SSSP_ILP = 4;                       // warp steps in flight
+constexpr int SSSP_MAX_STEPS = 1024;              // steps of one launch, at most: a cycle of negative weight ends on the host
+
+struct SsspState {
+    int *word;                // n: ordered words of the smallest distance seen
+    uint32_t *bits[2];        // frontiers of alternating steps, one bit per vertex
+    int32_t *ctr;             // [0..2] vertices of the frontier, [3..5] listed chunks (sets rotate by step), [6] steps made
+    int32_t *report;          // page-locked host words: steps made, vertices of the frontier that was left
+    int32_t n_words;
+};
+
+// ordered(v): monotone in v, and the bits themselves where v >= 0
+__device__ __forceinline__ int sssp_word(float v) { const int b = __float_as_int(v); return b ^ ((b >> 31) & 0x7FFFFFFF); }
+__device__ __forceinline__ float sssp_value(int w) { return __int_as_float(w ^ ((w >> 31) & 0x7FFFFFFF)); }
+
+struct SsspShared {
+    int pre[SSSP_COLS + 1];                       // elements before a column of the round
+    int2 run[SSSP_COLS];                          // position of its first entry minus that; its distance
+    uint16_t own[SSSP_COLS * PD_LONG / 32];       // column that owns the first element of a step of 32
+    int cnt[SSSP_WARPS], sum[SSSP_WARPS], rec[SSSP_WARPS], base;
+};
+
+// The candidates of up to U targets per lane (target < 0: none).
+template <int U>
+__device__ __forceinline__ void sssp_relax(const SsspState &s, uint32_t *next, const int (&target)[U], const float (&cand)[U]) {
+    int seen[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) seen[u] = target[u] >= 0 ? __ldca(s.word + target[u]) : 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        if (target[u] < 0) continue;
+        const int c = sssp_word(cand[u]);
+        if (c >= seen[u] || c >= __ldcg(s.word + target[u])) continue;
+        if (c < atomicMin(s.word + target[u], c)) atomicOr(next + (target[u] >> 5), 1u << (target[u] & 31));
+    }
+}
+
+template <int DT>
+__device__ void sssp_expand(const Device &d, const SsspState &s, const float *dist, const uint32_t *F, uint32_t *next, int32_t *n_long, SsspShared &sh) {
+    constexpr bool VAL = DT != DBSPMSPV_PATTERN;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rounds = (s.n_words + SSSP_WORDS * (int)gridDim.x - 1) / (SSSP_WORDS * (int)gridDim.x);
+    for (int round = 0; round < rounds; ++round) {
+        int first[4], deg[4], pfirst = 0, pdeg = 0, col0 = 0;
+        float xv[4];
+        uint32_t listed = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { first[k] = 0; deg[k] = 0; xv[k] = 0.f; }
+        const int64_t wi = (int64_t)(round * SSSP_WORDS + (tid >> 3)) * gridDim.x + blockIdx.x;
+        if (wi < s.n_words) listed = (__ldcg(F + wi) >> (4 * (tid & 7))) & 15u;
+        if (!__syncthreads_or(listed != 0u)) continue;
+        int n_rec = 0;
+        if (listed) {
+            const int j0 = (int)wi * 32 + 4 * (tid & 7);
+            col0 = j0 & 15;
+            const int32_t *cp = d.csc.colptr + 17 * (j0 >> 4) + col0;
+            int c[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) c[k] = cp[k];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if ((listed >> k) & 1u) { first[k] = c[k]; deg[k] = c[k + 1] - c[k]; xv[k] = __ldcg(dist + j0 + k); if (!DBS_CHK_RANGE(d, first[k], deg[k])) deg[k] = 0; }
+            if (d.n_payload) payload_run(d, j0 >> 4, pfirst, pdeg);
+            // long runs and runs of payload entries: chunks for the second half of the step
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (deg[k] > PD_LONG) { n_rec += (deg[k] + PD_CHUNK - 1) / PD_CHUNK; deg[k] = -deg[k]; }      // (negative: listed)
+            if (pdeg > 0) n_rec += __popc(listed) * ((pdeg + 31) / 32);
+        }
+        int n_cols = 0, n_elems = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { n_cols += deg[k] > 0; n_elems += max(deg[k], 0); }
+        int ic = n_cols, is = n_elems, ir = n_rec;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_up_sync(FULL, ic, o), b = __shfl_up_sync(FULL, is, o), c = __shfl_up_sync(FULL, ir, o);
+            if (lane >= o) { ic += a; is += b; ir += c; }
+        }
+        if (lane == 31) { sh.cnt[warp] = ic; sh.sum[warp] = is; sh.rec[warp] = ir; }
+        __syncthreads();
+        // (a lane per warp: the sums before it and the totals)
+        const int vc = sh.cnt[lane], vs = sh.sum[lane], vr = sh.rec[lane];
+        const int tot_c = __reduce_add_sync(FULL, vc), tot_e = __reduce_add_sync(FULL, vs), tot_r = __reduce_add_sync(FULL, vr);
+        int c = ic - n_cols + __reduce_add_sync(FULL, lane < warp ? vc : 0), e = is - n_elems + __reduce_add_sync(FULL, lane < warp ? vs : 0);
+        int at = ir - n_rec + __reduce_add_sync(FULL, lane < warp ? vr : 0);
+        if (tid == 0) {
+            sh.base = tot_r ? atomicAdd(n_long, tot_r) : 0;
+            sh.pre[tot_c] = tot_e;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (deg[k] <= 0) continue;
+            sh.pre[c] = e;
+            sh.run[c] = make_int2(first[k] - e, __float_as_int(xv[k]));
+            for (int q = (e + 31) >> 5; q * 32 < e + deg[k]; ++q) sh.own[q] = (uint16_t)c;
+            ++c;
+            e += deg[k];
+        }
+        __syncthreads();
+        if (tot_r) {                                   // block-uniform; a thread's runs are written by its whole warp
+            at += sh.base;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                for (uint32_t todo = __ballot_sync(FULL, deg[k] < 0); todo; todo &= todo - 1) {
+                    const int src = __ffs(todo) - 1;
+                    const int f = __shfl_sync(FULL, first[k], src), n = -__shfl_sync(FULL, deg[k], src), o = __shfl_sync(FULL, at, src);
+                    const int xb = __shfl_sync(FULL, __float_as_int(xv[k]), src);
+                    const int n_chunks = (n + PD_CHUNK - 1) / PD_CHUNK;
+                    for (int q = lane; q < n_chunks; q += 32) d.ws.long_runs[o + q] = make_int4(f + q * PD_CHUNK, min(PD_CHUNK, n - q * PD_CHUNK), xb, 0);
+                    if (lane == src) at += n_chunks;
+                }
+            if (pdeg > 0)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if ((listed >> k) & 1u)
+                        for (int q = 0; q < pdeg; q += 32) d.ws.long_runs[at++] = make_int4(pfirst + q, min(32, pdeg - q), __float_as_int(xv[k]), 0x100 | (col0 + k));
+        }
+        for (int s0 = warp * 32; s0 < tot_e; s0 += SSSP_CTA * SSSP_ILP) {
+            uint32_t idx[SSSP_ILP], w[SSSP_ILP], aux[SSSP_ILP];
+            float cand[SSSP_ILP];
+            int target[SSSP_ILP];
+#pragma unroll
+            for (int u = 0; u < SSSP_ILP; ++u) {
+                const int e0 = s0 + u * SSSP_CTA;
+                idx[u] = PAD_IDX; w[u] = 0u; aux[u] = 0u; cand[u] = 0.f;
+                if (e0 < tot_e) {                      // warp-uniform; the step's first owner, then every lane's own (see k_push_direct)
+                    const int lo = sh.own[e0 >> 5];
+                    const uint32_t b = (uint32_t)(sh.pre[min(lo + 1 + lane, tot_c)] - e0);
+                    const uint32_t m = __reduce_or_sync(FULL, b < 32u ? 1u << b : 0u);
+                    if (e0 + lane < tot_e) {
+                        const int2 run = sh.run[lo + __popc(m & ((2u << lane) - 1u))];
+                        cand[u] = __int_as_float(run.y);
+                        push_entry<VAL>(d, run.x + e0 + lane, idx[u], w[u], aux[u]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < SSSP_ILP; ++u) {
+                target[u] = idx[u] < (1u << TYPE_SHIFT) ? (int)((idx[u] & IDX_MASK) * 16u + (aux[u] >> 4)) : -1;
+                cand[u] += Val<DT>::inline_value(w[u]);
+            }
+            sssp_relax<SSSP_ILP>(s, next, target, cand);
+        }
+        __syncthreads();                               // (the next round overwrites the layout)
+    }
+}
+
+template <int DT>
+__device__ void sssp_long(const Device &d, const SsspState &s, uint32_t *next, int n) {
+    constexpr bool VAL = DT != DBSPMSPV_PATTERN;
+    constexpr int U = PD_CHUNK / 32;
+    const int lane = threadIdx.x & 31;
+    const int gwarp = (int)(blockIdx.x * SSSP_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
+    int4 ahead = gwarp < n ? __ldcg(d.ws.long_runs + gwarp) : make_int4(0, 0, 0, 0);
+    for (int i = gwarp; i < n; i += nwarps) {
+        const int4 run = ahead;
+        if (i + nwarps < n) ahead = __ldcg(d.ws.long_runs + i + nwarps);
+        if (!DBS_CHK_RANGE(d, run.x, run.y)) continue;
+        const float x = __int_as_float(run.z);
+        if (run.w) {                                   // payload entries: one per lane, up to 16 elements each
+            if (lane < run.y) {
+                uint32_t idx = d.csc.idx[run.x + lane], w = d.csc.w[run.x + lane], aux = d.csc.aux[run.x + lane];
+                DBS_CHK_ENTRY(d, false, idx, w, aux);
+                block_elements<DT>((int)(idx >> TYPE_SHIFT), w, aux, 1u << (run.w & 15), d.payload, [&](int r, int, float a) {
+                    const int target[1] = {(int)((idx & IDX_MASK) * 16u) + r};
+                    const float cand[1] = {x + a};
+                    sssp_relax<1>(s, next, target, cand);
+                });
+            }
+            continue;
+        }
+        uint32_t idx[U], w[U], aux[U];
+        float cand[U];
+        int target[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int k = u * 32 + lane;
+            idx[u] = PAD_IDX; w[u] = 0u; aux[u] = 0u;
+            if (k < run.y) push_entry<VAL>(d, run.x + k, idx[u], w[u], aux[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            target[u] = idx[u] < (1u << TYPE_SHIFT) ? (int)((idx[u] & IDX_MASK) * 16u + (aux[u] >> 4)) : -1;
+            cand[u] = x + Val<DT>::inline_value(w[u]);
+        }
+        sssp_relax<U>(s, next, target, cand);
+    }
+}
+
+template <int DT>
+__global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int32_t src, float *dist, int start, int max_steps) {
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) uint8_t s_dyn[];
+    SsspShared &sh = *reinterpret_cast<SsspShared *>(s_dyn);
+    cg::grid_group grid = cg::this_grid();
+    const int tid = blockIdx.x * SSSP_CTA + threadIdx.x, nthreads = gridDim.x * SSSP_CTA, lane = threadIdx.x & 31;
+    if (start) {                                       // (a later launch of the same search continues where the one before stopped)
+        const int64_t n = d.n;
+        for (int64_t v = tid; v < n; v += nthreads) { s.word[v] = v == src ? 0 : 0x7F800000; dist[v] = v == src ? 0.0f : __int_as_float(0x7F800000); }
+        for (int k = tid; k < s.n_words; k += nthreads) { s.bits[0][k] = k == src >> 5 ? 1u << (src & 31) : 0u; s.bits[1][k] = 0u; }
+        if (tid < 6) s.ctr[tid] = tid == 0 ? 1 : 0;
+        if (tid == 6) s.ctr[6] = 0;
+        grid.sync();
+    }
+    int t = s.ctr[6];
+    for (int made = 0; made < max_steps && __ldcg(s.ctr + t % 3) != 0; ++made, ++t) {
+        uint32_t *F = s.bits[t & 1], *next = s.bits[(t + 1) & 1];
+        int32_t *n_long = s.ctr + 3 + t % 3;
+        if (tid == 0) s.ctr[3 + (t + 1) % 3] = 0;      // (its last reader was step t - 2)
+        sssp_expand<DT>(d, s, dist, F, next, n_long, sh);
+        grid.sync();
+        const int n = __ldcg(n_long);
+        if (n > 0) {                                   // grid-uniform
+            sssp_long<DT>(d, s, next, n);
+            grid.sync();
+        }
+        if (tid == 0) s.ctr[(t + 2) % 3] = 0;
+        int found = 0;
+        const int gwarp = tid >> 5, nwarps = nthreads >> 5;
+        for (int w0 = gwarp; w0 < s.n_words; w0 += 8 * nwarps) {
+            uint32_t b[8];
+            int v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) { const int w = w0 + q * nwarps; b[q] = w < s.n_words ? __ldcg(next + w) : 0u; }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) { v[q] = 0; if ((b[q] >> lane) & 1u) v[q] = __ldcg(s.word + (int64_t)(w0 + q * nwarps) * 32 + lane); }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int w = w0 + q * nwarps;
+                if (w >= s.n_words) break;
+                if ((b[q] >> lane) & 1u) dist[(int64_t)w * 32 + lane] = sssp_value(v[q]);
+                if (lane == 0) F[w] = 0u;
+                found += __popc(b[q]);
+            }
+        }
+        if (lane == 0) sh.cnt[threadIdx.x >> 5] = found;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const int total = __reduce_add_sync(FULL, sh.cnt[lane]);
+            if (lane == 0 && total) atomicAdd(s.ctr + (t + 1) % 3, total);
+        }
+        grid.sync();
+    }
+    // (everyone read ctr[6] before the first barrier, or leaves without a step)
+    if (tid == 0) { s.ctr[6] = t; s.report[0] = t; s.report[1] = __ldcg(s.ctr + t % 3); }
+}
+
+}  // namespace dbs
