@@ -505,7 +505,7 @@ __global__ void k_long_chunks(int32_t nb, const int32_t *ptr, const int32_t *col
         const int32_t *cp = colptr + 17 * (t >> 4);
         const int deg = cp[(t & 15) + 1] - cp[t & 15], pdeg = cp[0] - ptr[t >> 4];
         if (deg > PD_LONG) c += (deg + PD_CHUNK - 1) / PD_CHUNK;
-        c += (pdeg + 31) / 32;
+        c += (pdeg + PD_PAYLOAD - 1) / PD_PAYLOAD;
     }
     c = __reduce_add_sync(0xFFFFFFFFu, c);
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(total, c);

@@ -102,13 +102,14 @@ constexpr int LEAN_CHUNK = DBS_LEAN_CHUNK;
 constexpr int PUSH_CHUNK = DBS_PUSH_CHUNK;   // CSC-view entries per push task (32 per warp step)
 static_assert(PUSH_CHUNK == 32, "a push task is one warp step; its record stores the exact entry count in 5 bits");
 // Direct push (push_direct.cuh): a column run longer than PD_LONG entries goes, in chunks of PD_CHUNK entries, to a
-// list that a second kernel walks, a warp per chunk; so does, in chunks of 32, the run of a listed column's payload entries.
+// list that a second kernel walks, a warp per chunk; so does, in chunks of PD_PAYLOAD, the run of a listed column's payload entries.
 constexpr int PD_CTA = 256;
 #ifndef DBS_PD_LONG
 #define DBS_PD_LONG 128
 #endif
 constexpr int PD_LONG = DBS_PD_LONG;
 constexpr int PD_CHUNK = 128;
+constexpr int PD_PAYLOAD = 8;
 // A run of the push worklist with at least HUB_MIN_ENTRIES entries (a hub column) is not cut
 // into tasks: it is listed once and every warp of the traversal strides over its 32-entry steps.
 constexpr int HUB_MIN_ENTRIES = 8192;

@@ -66,13 +66,54 @@ __device__ __forceinline__ void push_entry(const Device &d, int p, uint32_t &idx
     DBS_CHK_ENTRY(d, false, idx, w, aux);
 }
 
-// One entry with a payload under one listed column: at most 16 elements.
-template <int DT, int MODE>
-__device__ __forceinline__ void push_payload_entry(const Device &d, int p, int col, float xv) {
-    uint32_t idx = d.csc.idx[p], w = d.csc.w[p], aux = d.csc.aux[p];
-    DBS_CHK_ENTRY(d, false, idx, w, aux);
-    block_elements<DT>((int)(idx >> TYPE_SHIFT), w, aux, 1u << col, d.payload,
-                       [&](int r, int, float a) { push_product<DT, MODE>(d, idx & IDX_MASK, r, a, xv); });
+// Elements (row, col) of the blocks with a payload behind the CSC-view entries first .. first + count - 1: value and row block
+// where one is stored.  A half-warp takes an entry, lane = row, U of them side by side: entry, header and
+// value are one trip each, for all rows and all entries at once.
+template <int DT, int U>
+__device__ __forceinline__ void payload_elements(const Device &d, int first, int count, int col, int lane, bool (&in)[U], float (&value)[U], uint32_t (&rb)[U]) {
+    const int row = lane & 15;
+    uint32_t idx[U], w[U], aux[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int k = 2 * u + (lane >> 4), p = first + (k < count ? k : 0);
+        in[u] = k < count;
+        idx[u] = d.csc.idx[p]; w[u] = d.csc.w[p]; aux[u] = d.csc.aux[p];
+        DBS_CHK_ENTRY(d, false, idx[u], w[u], aux[u]);
+        rb[u] = idx[u] & IDX_MASK;
+        value[u] = 1.0f;
+    }
+    uint32_t m[U], start[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int type = (int)(idx[u] >> TYPE_SHIFT);
+        m[u] = 0u; start[u] = 0u;
+        if (type > DBSPMSPV_BLK_COO) {
+            const uint8_t *blk = d.payload + (size_t)w[u] * 4;
+            const int major = is_row_major(type) ? row : col;
+            m[u] = reinterpret_cast<const uint16_t *>(blk)[major];
+            if (DT != DBSPMSPV_PATTERN && type != DBSPMSPV_BLK_DENSE) start[u] = blk[32 + major];
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int type = (int)(idx[u] >> TYPE_SHIFT), minor = is_row_major(type) ? col : row;
+        const uint8_t *blk = d.payload + (size_t)w[u] * 4;
+        if (type > DBSPMSPV_BLK_COO) {
+            in[u] = in[u] && ((m[u] >> minor) & 1u);
+            if (DT != DBSPMSPV_PATTERN && in[u])
+                value[u] = type == DBSPMSPV_BLK_DENSE ? Val<DT>::load(blk + 32, col * 16 + row)
+                                                      : Val<DT>::load(blk + HDR_BYTES, start[u] + __popc(m[u] & ((1u << minor) - 1u)));
+        } else if (type == DBSPMSPV_BLK_COO) {             // (only with forced formats)
+            const int nnz = (int)aux[u] + 1;
+            bool found = false;
+            for (int k = 0; k < nnz && in[u]; ++k)
+                if (blk[k] == (uint32_t)(row << 4 | col)) { value[u] = Val<DT>::load(blk + ((nnz + 3) & ~3), k); found = true; break; }
+            in[u] = in[u] && found;
+        } else {                                           // (only in the range-checked build: a replaced entry)
+            value[u] = Val<DT>::inline_value(w[u]);
+            in[u] = in[u] && (int)(aux[u] & 15) == col && (int)(aux[u] >> 4) == row;
+        }
+    }
 }
 
 template <int DT, int MODE, bool MASKS>
@@ -148,7 +189,7 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
 #pragma unroll
             for (int k = 0; k < PER; ++k)
                 if (deg[k] > PD_LONG) { n_rec += (deg[k] + PD_CHUNK - 1) / PD_CHUNK; deg[k] = -deg[k]; }      // (negative: listed)
-            if (pdeg > 0) n_rec += __popc(listed) * ((pdeg + 31) / 32);
+            if (pdeg > 0) n_rec += __popc(listed) * ((pdeg + PD_PAYLOAD - 1) / PD_PAYLOAD);
         }
         // lay the nonempty short runs end to end
         int n_cols = 0, n_elems = 0;
@@ -202,7 +243,7 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
 #pragma unroll
                 for (int k = 0; k < PER; ++k)
                     if ((listed >> k) & 1u)
-                        for (int q = 0; q < pdeg; q += 32) d.ws.long_runs[at++] = make_int4(pfirst + q, min(32, pdeg - q), __float_as_int(xv[k]), 0x100 | (col0 + k));
+                        for (int q = 0; q < pdeg; q += PD_PAYLOAD) d.ws.long_runs[at++] = make_int4(pfirst + q, min(PD_PAYLOAD, pdeg - q), __float_as_int(xv[k]), 0x100 | (col0 + k));
         }
         for (int s0 = warp * 32; s0 < tot_e; s0 += PD_CTA * PD_ILP) {
             uint32_t idx[PD_ILP], w[PD_ILP], aux[PD_ILP];
@@ -246,8 +287,14 @@ __global__ void __launch_bounds__(PD_CTA, 6) k_push_long(Device d) {
         if (i + nwarps < n) next = d.ws.long_runs[i + nwarps];
         if (!DBS_CHK_RANGE(d, run.x, run.y)) continue;
         const float xs = __int_as_float(run.z);
-        if (run.w) {                                   // payload entries: one per lane, up to 16 products each
-            if (lane < run.y) push_payload_entry<DT, MODE>(d, run.x + lane, run.w & 15, xs);
+        if (run.w) {                                   // payload entries: a half-warp each
+            bool in[PD_PAYLOAD / 2];
+            float a[PD_PAYLOAD / 2];
+            uint32_t rb[PD_PAYLOAD / 2];
+            payload_elements<DT, PD_PAYLOAD / 2>(d, run.x, run.y, run.w & 15, lane, in, a, rb);
+#pragma unroll
+            for (int u = 0; u < PD_PAYLOAD / 2; ++u)
+                if (in[u]) push_product<DT, MODE>(d, rb[u], lane & 15, a[u], xs);
             continue;
         }
         uint32_t idx[U], w[U], aux[U];

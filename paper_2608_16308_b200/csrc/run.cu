@@ -2297,7 +2297,7 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     const size_t word_bytes = ((size_t)s.n_words * 32 * sizeof(int) + 255) & ~(size_t)255, bit_bytes = ((size_t)s.n_words * 4 + 255) & ~(size_t)255;
     if (!h->sssp_host && cudaHostAlloc(reinterpret_cast<void **>(&h->sssp_host), 4 * sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess) { h->sssp_host = nullptr; return DBSPMSPV_ERR_ALLOC; }
     if (!h->sssp_state) {
-        if (cudaMalloc(&h->sssp_state, word_bytes + 2 * bit_bytes + 64) != cudaSuccess) { h->sssp_state = nullptr; return DBSPMSPV_ERR_ALLOC; }
+        if (cudaMalloc(&h->sssp_state, word_bytes + 2 * bit_bytes + 128) != cudaSuccess) { h->sssp_state = nullptr; return DBSPMSPV_ERR_ALLOC; }
         DBS_CUDA(cudaFuncSetAttribute(k_sssp<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsspShared)));
     }
     uint8_t *p = static_cast<uint8_t *>(h->sssp_state);
@@ -2305,12 +2305,15 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     s.bits[0] = reinterpret_cast<uint32_t *>(p + word_bytes);
     s.bits[1] = reinterpret_cast<uint32_t *>(p + word_bytes + bit_bytes);
     s.ctr = reinterpret_cast<int32_t *>(p + word_bytes + 2 * bit_bytes);
+    s.low = s.ctr + 8;
+    s.edges = reinterpret_cast<unsigned long long *>(s.ctr + 12);
     s.report = h->sssp_host;
     Device dev = d;
     int start = 1;
     for (int64_t made = 0;; start = 0) {
         int max_steps = (int)(d.n + 1 - made < SSSP_MAX_STEPS ? d.n + 1 - made : SSSP_MAX_STEPS);
-        void *args[] = {&dev, &s, &src, &dist, &start, &max_steps};
+        unsigned long long pull_edges = (unsigned long long)(DBS_SSSP_PULL_SHARE * (float)d.n_entries);
+        void *args[] = {&dev, &s, &src, &dist, &start, &max_steps, &pull_edges};
         DBS_CUDA(cudaLaunchCooperativeKernel((void *)k_sssp<DT>, dim3(h->sm_count), dim3(SSSP_CTA), args, sizeof(SsspShared), st));
         ++h->kernel_launches;
         DBS_CUDA(cudaStreamSynchronize(st));

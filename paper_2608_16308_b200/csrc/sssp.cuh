@@ -21,6 +21,7 @@
 #include <cooperative_groups.h>
 
 #include "internal.cuh"
+#include "lean_pull.cuh"
 #include "minplus.cuh"
 #include "push_direct.cuh"
 
@@ -31,12 +32,18 @@ constexpr int SSSP_WARPS = SSSP_CTA / 32;
 constexpr int SSSP_WORDS = SSSP_CTA / 8;          // frontier words of a thread block's round: eight threads per word, four columns each
 constexpr int SSSP_COLS = SSSP_CTA * 4;
 constexpr int SSSP_ILP = 4;                       // warp steps in flight
+// A step whose frontier reaches more than this share of the stored elements is pulled.
+#ifndef DBS_SSSP_PULL_SHARE
+#define DBS_SSSP_PULL_SHARE 0.1f
+#endif
 constexpr int SSSP_MAX_STEPS = 1024;              // steps of one launch, at most: a cycle of negative weight ends on the host
 
 struct SsspState {
     int *word;                // n: ordered words of the smallest distance seen
     uint32_t *bits[2];        // frontiers of alternating steps, one bit per vertex
     int32_t *ctr;             // [0..2] vertices of the frontier, [3..5] listed chunks (sets rotate by step), [6] steps made
+    int *low;                 // smallest word of the frontier, rotating with the counters
+    unsigned long long *edges;   // out-edges of the frontier in INLINE runs, likewise
     int32_t *report;          // page-locked host words: steps made, vertices of the frontier that was left
     int32_t n_words;
 };
@@ -45,7 +52,13 @@ struct SsspState {
 __device__ __forceinline__ int sssp_word(float v) { const int b = __float_as_int(v); return b ^ ((b >> 31) & 0x7FFFFFFF); }
 __device__ __forceinline__ float sssp_value(int w) { return __int_as_float(w ^ ((w >> 31) & 0x7FFFFFFF)); }
 
+// Per warp: the rows that the chunk adds to and their words.
+constexpr int SSSP_ROWS = 32;
+struct SsspRows { int row[SSSP_ROWS], word[SSSP_ROWS]; };
+
 struct SsspShared {
+    SsspRows pull[SSSP_WARPS];
+    unsigned long long edges[SSSP_WARPS];
     int pre[SSSP_COLS + 1];                       // elements before a column of the round
     int2 run[SSSP_COLS];                          // position of its first entry minus that; its distance
     uint16_t own[SSSP_COLS * PD_LONG / 32];       // column that owns the first element of a step of 32
@@ -97,7 +110,7 @@ __device__ void sssp_expand(const Device &d, const SsspState &s, const float *di
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if (deg[k] > PD_LONG) { n_rec += (deg[k] + PD_CHUNK - 1) / PD_CHUNK; deg[k] = -deg[k]; }      // (negative: listed)
-            if (pdeg > 0) n_rec += __popc(listed) * ((pdeg + 31) / 32);
+            if (pdeg > 0) n_rec += __popc(listed) * ((pdeg + PD_PAYLOAD - 1) / PD_PAYLOAD);
         }
         int n_cols = 0, n_elems = 0;
 #pragma unroll
@@ -145,32 +158,38 @@ __device__ void sssp_expand(const Device &d, const SsspState &s, const float *di
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
                     if ((listed >> k) & 1u)
-                        for (int q = 0; q < pdeg; q += 32) d.ws.long_runs[at++] = make_int4(pfirst + q, min(32, pdeg - q), __float_as_int(xv[k]), 0x100 | (col0 + k));
+                        for (int q = 0; q < pdeg; q += PD_PAYLOAD) d.ws.long_runs[at++] = make_int4(pfirst + q, min(PD_PAYLOAD, pdeg - q), __float_as_int(xv[k]), 0x100 | (col0 + k));
         }
-        for (int s0 = warp * 32; s0 < tot_e; s0 += SSSP_CTA * SSSP_ILP) {
-            uint32_t idx[SSSP_ILP], w[SSSP_ILP], aux[SSSP_ILP];
-            float cand[SSSP_ILP];
-            int target[SSSP_ILP];
+        // 32 elements per warp step, SSSP_ILP steps at a time; the entries of the next ones are fetched before these are relaxed
+        uint32_t idx[SSSP_ILP], w[SSSP_ILP], aux[SSSP_ILP];
+        float x[SSSP_ILP];
+        auto fetch = [&](int s0) {
 #pragma unroll
             for (int u = 0; u < SSSP_ILP; ++u) {
                 const int e0 = s0 + u * SSSP_CTA;
-                idx[u] = PAD_IDX; w[u] = 0u; aux[u] = 0u; cand[u] = 0.f;
+                idx[u] = PAD_IDX; w[u] = 0u; aux[u] = 0u; x[u] = 0.f;
                 if (e0 < tot_e) {                      // warp-uniform; the step's first owner, then every lane's own (see k_push_direct)
                     const int lo = sh.own[e0 >> 5];
                     const uint32_t b = (uint32_t)(sh.pre[min(lo + 1 + lane, tot_c)] - e0);
                     const uint32_t m = __reduce_or_sync(FULL, b < 32u ? 1u << b : 0u);
                     if (e0 + lane < tot_e) {
                         const int2 run = sh.run[lo + __popc(m & ((2u << lane) - 1u))];
-                        cand[u] = __int_as_float(run.y);
+                        x[u] = __int_as_float(run.y);
                         push_entry<VAL>(d, run.x + e0 + lane, idx[u], w[u], aux[u]);
                     }
                 }
             }
+        };
+        if (warp * 32 < tot_e) fetch(warp * 32);
+        for (int s0 = warp * 32; s0 < tot_e; s0 += SSSP_CTA * SSSP_ILP) {
+            float cand[SSSP_ILP];
+            int target[SSSP_ILP];
 #pragma unroll
             for (int u = 0; u < SSSP_ILP; ++u) {
                 target[u] = idx[u] < (1u << TYPE_SHIFT) ? (int)((idx[u] & IDX_MASK) * 16u + (aux[u] >> 4)) : -1;
-                cand[u] += Val<DT>::inline_value(w[u]);
+                cand[u] = x[u] + Val<DT>::inline_value(w[u]);
             }
+            if (s0 + SSSP_CTA * SSSP_ILP < tot_e) fetch(s0 + SSSP_CTA * SSSP_ILP);
             sssp_relax<SSSP_ILP>(s, next, target, cand);
         }
         __syncthreads();                               // (the next round overwrites the layout)
@@ -183,44 +202,145 @@ __device__ void sssp_long(const Device &d, const SsspState &s, uint32_t *next, i
     constexpr int U = PD_CHUNK / 32;
     const int lane = threadIdx.x & 31;
     const int gwarp = (int)(blockIdx.x * SSSP_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
-    int4 ahead = gwarp < n ? __ldcg(d.ws.long_runs + gwarp) : make_int4(0, 0, 0, 0);
-    for (int i = gwarp; i < n; i += nwarps) {
-        const int4 run = ahead;
-        if (i + nwarps < n) ahead = __ldcg(d.ws.long_runs + i + nwarps);
-        if (!DBS_CHK_RANGE(d, run.x, run.y)) continue;
-        const float x = __int_as_float(run.z);
-        if (run.w) {                                   // payload entries: one per lane, up to 16 elements each
-            if (lane < run.y) {
-                uint32_t idx = d.csc.idx[run.x + lane], w = d.csc.w[run.x + lane], aux = d.csc.aux[run.x + lane];
-                DBS_CHK_ENTRY(d, false, idx, w, aux);
-                block_elements<DT>((int)(idx >> TYPE_SHIFT), w, aux, 1u << (run.w & 15), d.payload, [&](int r, int, float a) {
-                    const int target[1] = {(int)((idx & IDX_MASK) * 16u) + r};
-                    const float cand[1] = {x + a};
-                    sssp_relax<1>(s, next, target, cand);
-                });
-            }
-            continue;
-        }
-        uint32_t idx[U], w[U], aux[U];
-        float cand[U];
-        int target[U];
+    // a chunk's record two rounds ahead, its entries one
+    uint32_t idx[U], w[U], aux[U];
+    auto record = [&](int i) { return i < n ? __ldcg(d.ws.long_runs + i) : make_int4(0, 0, 0, 0); };
+    auto fetch = [&](const int4 &run) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int k = u * 32 + lane;
             idx[u] = PAD_IDX; w[u] = 0u; aux[u] = 0u;
-            if (k < run.y) push_entry<VAL>(d, run.x + k, idx[u], w[u], aux[u]);
+            if (!run.w && k < run.y && DBS_CHK_RANGE(d, run.x, run.y)) push_entry<VAL>(d, run.x + k, idx[u], w[u], aux[u]);
         }
+    };
+    int4 run = record(gwarp), ahead = record(gwarp + nwarps);
+    fetch(run);
+    for (int i = gwarp; i < n; i += nwarps) {
+        const float x = __int_as_float(run.z);
+        float cand[U];
+        int target[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             target[u] = idx[u] < (1u << TYPE_SHIFT) ? (int)((idx[u] & IDX_MASK) * 16u + (aux[u] >> 4)) : -1;
             cand[u] = x + Val<DT>::inline_value(w[u]);
         }
+        if (run.w && DBS_CHK_RANGE(d, run.x, run.y)) { // payload entries: a half-warp each
+            static_assert(PD_PAYLOAD / 2 == U, "one element per lane and step either way");
+            bool in[U];
+            uint32_t rb[U];
+            payload_elements<DT, U>(d, run.x, run.y, run.w & 15, lane, in, cand, rb);
+#pragma unroll
+            for (int u = 0; u < U; ++u) { target[u] = in[u] ? (int)(rb[u] * 16u) + (lane & 15) : -1; cand[u] += x; }
+        }
+        run = ahead;
+        ahead = record(i + 2 * nwarps);
+        fetch(run);
         sssp_relax<U>(s, next, target, cand);
     }
 }
 
+// A large step pulled: every stored element once, in the order of the block-CSR view (see lean_pull.cuh: chunks of LEAN_CHUNK entries, eight
+// consecutive ones per lane, the next chunk's in registers already).  A row's elements are adjacent, so its word is at hand, and an element whose
+// weight alone rules it out -- smallest distance of the frontier + weight is no improvement -- costs a comparison and no gather: four fifths of them in
+// the late large steps of an R-MAT search.  The others gather the column's distance (columns outside the frontier too: they improve nothing, their edges were
+// relaxed when they entered it).  Improvements are few: an atomic each, one per warp where the whole chunk lies in one row.
 template <int DT>
-__global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int32_t src, float *dist, int start, int max_steps) {
+__device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist, uint32_t *next, int low, SsspRows &rows) {
+    constexpr bool VAL = DT != DBSPMSPV_PATTERN;
+    constexpr int K = LEAN_PER_LANE;
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    const int gwarp = (int)(blockIdx.x * SSSP_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
+    const float xmin = sssp_value(low);
+    auto lower = [&](int row, int best) {
+        if (best < atomicMin(s.word + row, best)) atomicOr(next + (row >> 5), 1u << (row & 31));
+    };
+    // rows ord - 1, ord, ... of the row list: the first one runs into the chunk
+    auto rows_of = [&](int c) {
+        if (c >= d.n_lean_chunks) return -1;
+        const int o = d.lean_chunk_ord[c] - 1 + lane;
+        return o >= 0 && o < d.n_lean_rows ? __ldg(d.lean_rows + o) : -1;
+    };
+    auto word_of = [&](int row) { return row >= 0 ? __ldcg(s.word + row) : 0; };
+    LeanRegs nxt = {};
+    int row1 = rows_of(gwarp), row2 = rows_of(gwarp + nwarps), word1 = word_of(row1);
+    if (gwarp < d.n_lean_chunks) nxt = lean_fetch<VAL>(d, gwarp, lane);
+    for (int c = gwarp; c < d.n_lean_chunks; c += nwarps) {
+        const LeanRegs r = nxt;
+        __syncwarp();                                  // (the previous chunk's look-ups are over)
+        rows.row[lane] = row1;
+        rows.word[lane] = word1;
+        __syncwarp();
+        const int ord = d.lean_chunk_ord[c];
+        if (c + nwarps < d.n_lean_chunks) nxt = lean_fetch<VAL>(d, c + nwarps, lane);
+        row1 = row2;
+        word1 = word_of(row1);
+        row2 = rows_of(c + 2 * nwarps);
+        const uint32_t idx[K] = {r.i0.x, r.i0.y, r.i0.z, r.i0.w, r.i1.x, r.i1.y, r.i1.z, r.i1.w};
+        const uint32_t wv[K] = {r.w0.x, r.w0.y, r.w0.z, r.w0.w, r.w1.x, r.w1.y, r.w1.z, r.w1.w};
+        uint32_t hb = 0u;                              // bit k: entry k starts a row
+#pragma unroll
+        for (int k = 0; k < K; ++k) hb |= ((idx[k] >> 27) & 1u) << k;
+        const int cnt = __popc(hb);
+        int excl = cnt;                                // row starts in the lanes below
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, excl, o); if (lane >= o) excl += t; }
+        const int total = __shfl_sync(FULL, excl, 31);
+        excl -= cnt;
+        auto row_at = [&](int q) { return q < SSSP_ROWS ? rows.row[q] : d.lean_rows[ord - 1 + q]; };
+        auto word_at = [&](int q) { return q < SSSP_ROWS ? rows.word[q] : __ldcg(s.word + d.lean_rows[ord - 1 + q]); };
+        // which entries may improve their row
+        float x[K];
+        {
+            int q = excl;
+            float have = sssp_value(word_at(q));
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                if ((hb >> k) & 1u) have = sssp_value(word_at(++q));
+                x[k] = __int_as_float(0x7F800000);
+                const bool go = idx[k] < (1u << TYPE_SHIFT) && xmin + Val<DT>::inline_value(wv[k]) < have && DBS_CHK_INDEX(d, idx[k] & IDX_MASK, d.nb);
+                const uint32_t a = k < 4 ? r.a.x : r.a.y;
+                if (go) x[k] = __ldca(dist + ((idx[k] & IDX_MASK) * 16u + ((a >> (8 * (k & 3))) & 15u)));
+            }
+        }
+        if (total == 0) {                              // the whole chunk lies in one row
+            int best = 0x7F800000;
+#pragma unroll
+            for (int k = 0; k < K; ++k) best = min(best, sssp_word(x[k] + Val<DT>::inline_value(wv[k])));
+            best = __reduce_min_sync(FULL, best);
+            if (lane == 0 && best < rows.word[0]) lower(rows.row[0], best);
+            continue;
+        }
+        int q = excl, best = 0x7F800000;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if ((hb >> k) & 1u) {
+                if (best < 0x7F800000 && best < word_at(q)) lower(row_at(q), best);
+                best = 0x7F800000;
+                ++q;
+            }
+            best = min(best, sssp_word(x[k] + Val<DT>::inline_value(wv[k])));
+        }
+        if (best < 0x7F800000 && best < word_at(q)) lower(row_at(q), best);
+    }
+    // entries with a payload: one block per warp at a time
+    for (int q = gwarp; q < d.n_payload; q += nwarps) {
+        const int pos = d.payload_pos[q];
+        if (!DBS_CHK_INDEX(d, pos, d.n_entries)) continue;            // warp-uniform
+        uint32_t idx = d.csr.idx[pos], w = d.csr.w[pos], aux = d.csr.aux[pos];
+        DBS_CHK_ENTRY(d, true, idx, w, aux);
+        const int type = (int)(idx >> TYPE_SHIFT), cb = (int)(idx & IDX_MASK), rb = d.entry_row[pos];
+        if (type == DBSPMSPV_BLK_INLINE || !DBS_CHK_INDEX(d, rb, d.mb)) continue;      // (only a replaced entry is INLINE here)
+        const uint32_t xm = (int64_t)cb * 16 + 16 <= d.n ? 0xFFFFu : (1u << (d.n - (int64_t)cb * 16)) - 1u;
+        block_rows_min_warp<DT>(type, w, aux, xm, dist + (size_t)cb * 16, d.payload, lane, [&](int r, uint32_t key) {
+            const int c = sssp_word(minplus_value(key)), row = rb * 16 + r;
+            if (c < __ldcg(s.word + row)) lower(row, c);
+        });
+    }
+}
+
+template <int DT>
+__global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int32_t src, float *dist, int start, int max_steps, unsigned long long pull_edges) {
     namespace cg = cooperative_groups;
     extern __shared__ __align__(16) uint8_t s_dyn[];
     SsspShared &sh = *reinterpret_cast<SsspShared *>(s_dyn);
@@ -231,7 +351,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int
         for (int64_t v = tid; v < n; v += nthreads) { s.word[v] = v == src ? 0 : 0x7F800000; dist[v] = v == src ? 0.0f : __int_as_float(0x7F800000); }
         for (int k = tid; k < s.n_words; k += nthreads) { s.bits[0][k] = k == src >> 5 ? 1u << (src & 31) : 0u; s.bits[1][k] = 0u; }
         if (tid < 6) s.ctr[tid] = tid == 0 ? 1 : 0;
-        if (tid == 6) s.ctr[6] = 0;
+        if (tid == 6) { s.ctr[6] = 0; for (int k = 0; k < 3; ++k) { s.low[k] = k == 0 ? 0 : 0x7F800000; s.edges[k] = 0ull; } }
         grid.sync();
     }
     int t = s.ctr[6];
@@ -239,23 +359,37 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int
         uint32_t *F = s.bits[t & 1], *next = s.bits[(t + 1) & 1];
         int32_t *n_long = s.ctr + 3 + t % 3;
         if (tid == 0) s.ctr[3 + (t + 1) % 3] = 0;      // (its last reader was step t - 2)
-        sssp_expand<DT>(d, s, dist, F, next, n_long, sh);
-        grid.sync();
-        const int n = __ldcg(n_long);
-        if (n > 0) {                                   // grid-uniform
-            sssp_long<DT>(d, s, next, n);
+        if (__ldcg(s.edges + t % 3) > pull_edges) {    // grid-uniform
+            sssp_pull<DT>(d, s, dist, next, __ldcg(s.low + t % 3), sh.pull[threadIdx.x >> 5]);
             grid.sync();
+        } else {
+            sssp_expand<DT>(d, s, dist, F, next, n_long, sh);
+            grid.sync();
+            const int n = __ldcg(n_long);
+            if (n > 0) {                               // grid-uniform
+                sssp_long<DT>(d, s, next, n);
+                grid.sync();
+            }
         }
-        if (tid == 0) s.ctr[(t + 2) % 3] = 0;
-        int found = 0;
+        if (tid == 0) { s.ctr[(t + 2) % 3] = 0; s.low[(t + 2) % 3] = 0x7F800000; s.edges[(t + 2) % 3] = 0ull; }
+        int found = 0, low = 0x7F800000;
+        unsigned long long edges = 0;
         const int gwarp = tid >> 5, nwarps = nthreads >> 5;
         for (int w0 = gwarp; w0 < s.n_words; w0 += 8 * nwarps) {
             uint32_t b[8];
-            int v[8];
+            int v[8], deg[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) { const int w = w0 + q * nwarps; b[q] = w < s.n_words ? __ldcg(next + w) : 0u; }
 #pragma unroll
-            for (int q = 0; q < 8; ++q) { v[q] = 0; if ((b[q] >> lane) & 1u) v[q] = __ldcg(s.word + (int64_t)(w0 + q * nwarps) * 32 + lane); }
+            for (int q = 0; q < 8; ++q) {
+                v[q] = 0x7F800000; deg[q] = 0;
+                if ((b[q] >> lane) & 1u) {
+                    const int j = (w0 + q * nwarps) * 32 + lane;
+                    v[q] = __ldcg(s.word + j);
+                    const int32_t *cp = d.csc.colptr + 17 * (j >> 4) + (j & 15);
+                    deg[q] = cp[1] - cp[0];
+                }
+            }
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 const int w = w0 + q * nwarps;
@@ -263,13 +397,22 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int
                 if ((b[q] >> lane) & 1u) dist[(int64_t)w * 32 + lane] = sssp_value(v[q]);
                 if (lane == 0) F[w] = 0u;
                 found += __popc(b[q]);
+                low = min(low, v[q]);
+                edges += (unsigned)deg[q];
             }
         }
-        if (lane == 0) sh.cnt[threadIdx.x >> 5] = found;
+        low = __reduce_min_sync(FULL, low);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) edges += __shfl_xor_sync(FULL, edges, o);
+        if (lane == 0) { sh.cnt[threadIdx.x >> 5] = found; sh.sum[threadIdx.x >> 5] = low; sh.edges[threadIdx.x >> 5] = edges; }
         __syncthreads();
         if (threadIdx.x < 32) {
-            const int total = __reduce_add_sync(FULL, sh.cnt[lane]);
-            if (lane == 0 && total) atomicAdd(s.ctr + (t + 1) % 3, total);
+            found = __reduce_add_sync(FULL, sh.cnt[lane]);
+            low = __reduce_min_sync(FULL, sh.sum[lane]);
+            edges = sh.edges[lane];
+#pragma unroll
+            for (int o = 16; o; o >>= 1) edges += __shfl_xor_sync(FULL, edges, o);
+            if (lane == 0 && found) { atomicAdd(s.ctr + (t + 1) % 3, found); atomicMin(s.low + (t + 1) % 3, low); atomicAdd(s.edges + (t + 1) % 3, edges); }
         }
         grid.sync();
     }
