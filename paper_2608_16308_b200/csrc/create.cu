@@ -540,6 +540,25 @@ __global__ void k_rowrun_keys(int32_t n_entries, int64_t m, const int32_t *entry
     vals[p] = (idx & IDX_MASK) | ((rc & 15u) << 27);
 }
 
+// The INLINE elements by row and weight (see Device::weightrun): key, and the position in the view as value.
+__global__ void k_weightrun_keys(int32_t n_entries, int64_t m, const int32_t *entry_row, const uint32_t *csr_idx, const uint32_t *csr_w,
+                                 const uint8_t *csr_aux, uint64_t *keys, uint32_t *vals) {
+    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (p >= n_entries) return;
+    const bool inl = (csr_idx[p] >> TYPE_SHIFT) == DBSPMSPV_BLK_INLINE;
+    const uint64_t row = inl ? (uint64_t)entry_row[p] * 16 + (csr_aux[p] >> 4) : (uint64_t)m;   // others sort behind every row
+    const uint32_t w = (uint32_t)ordered_word((int)csr_w[p]) ^ 0x80000000u;
+    keys[p] = (row << SSSP_WEIGHT_BITS) | (inl ? w >> (32 - SSSP_WEIGHT_BITS) : 0u);
+    vals[p] = (uint32_t)p;
+}
+__global__ void k_weightrun(int32_t n_inline, const uint32_t *pos, const uint32_t *csr_idx, const uint32_t *csr_w, const uint8_t *csr_aux, uint2 *out) {
+    int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= n_inline + 4) return;
+    if (k >= n_inline) { out[k] = make_uint2(0u, 0x7F800000u); return; }                        // (slack: groups of four are read whole)
+    const uint32_t p = pos[k];
+    out[k] = make_uint2((csr_idx[p] & IDX_MASK) * 16u + (csr_aux[p] & 15u), csr_w[p]);
+}
+
 // ptr[i] = first position whose row is >= i, i = 0..m
 __global__ void k_rowrun_ptr(int64_t m, const uint64_t *keys_sorted, int32_t n, int32_t *ptr) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -969,7 +988,7 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
     }
 
     // row-run index for the pull levels of DB-BFS
-    d.rowrun_ptr = nullptr; d.rowrun_idx = nullptr;
+    d.rowrun_ptr = nullptr; d.rowrun_idx = nullptr; d.weightrun = nullptr;
     if (m == n && !h->copts.no_bfs_index) {
         uint64_t *rk, *rk_alt;
         uint32_t *rv, *rv_alt;
@@ -992,6 +1011,18 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         DBS_CUDA(cudaStreamSynchronize(st));
         tp.release(rk); tp.release(rk_alt); tp.release(rv); tp.release(rv_alt);
         h->bfs_index_bytes = ((int64_t)m + 1) * 4 + (int64_t)n_inline * 4;
+        if (d.dtype == DBSPMSPV_F32 && !h->heavy_stage && n_inline) {
+            DBS_GET(rk, n_entries); DBS_GET(rk_alt, n_entries); DBS_GET(rv, n_entries); DBS_GET(rv_alt, n_entries);
+            k_weightrun_keys<<<grid_for(n_entries), TPB, 0, st>>>(n_entries, m, h->block_row, d.csr.idx, d.csr.w, d.csr.aux, rk, rv);
+            DBS_TRY(sort_pairs(tp, rk, rk_alt, rv, rv_alt, (int64_t)n_entries, SSSP_WEIGHT_BITS + bits_for((uint64_t)m), st));
+            uint2 *wr;
+            DBS_KEEP(wr, (int64_t)n_inline + 4);
+            d.weightrun = wr;
+            k_weightrun<<<grid_for((int64_t)n_inline + 4), TPB, 0, st>>>(n_inline, rv, d.csr.idx, d.csr.w, d.csr.aux, wr);
+            DBS_CUDA(cudaStreamSynchronize(st));
+            tp.release(rk); tp.release(rk_alt); tp.release(rv); tp.release(rv_alt);
+            h->bfs_index_bytes += (int64_t)n_inline * 8;
+        }
     }
 
     // Streaming decode of payload-dominated handles: the chunk table

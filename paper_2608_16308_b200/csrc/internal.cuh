@@ -89,6 +89,7 @@ constexpr uint32_t HUB_CLEAR = 0x80000000u; // an untouched private accumulator 
 // the smallest int, which every key exceeds (minplus.cuh).
 constexpr uint32_t ACC_CLEAR = 0x80000000u;
 constexpr float ACC_FLAG_MIN = 7.8886090522101181e-31f;     // 2^-100
+constexpr int SSSP_WEIGHT_BITS = 16;
 constexpr uint32_t PAD_IDX = 7u << TYPE_SHIFT;   // class code of the slack behind the last view entry: no kernel acts on it
 // The streaming pull of hypersparse handles takes the block-CSR view in chunks of LEAN_CHUNK
 // entries, one chunk (eight entries per lane) per warp pass.
@@ -244,6 +245,9 @@ struct Device {           // everything the kernels need, passed by value
     // neighbour.  Null when not built.
     const int32_t *rowrun_ptr;
     const uint32_t *rowrun_idx;
+    // The same elements of fp32 handles once more, every row's by weight (column, weight bits), for the large steps of
+    // db_sssp: a row stops at the first weight that cannot improve it.  Ordered by the upper SSSP_WEIGHT_BITS bits of the ordered weight.  Null when not built.
+    const uint2 *weightrun;
     // Block-CSR view: csr_inl[rb] = first INLINE element of row block rb; its entries with a
     // payload are [csr.ptr[rb], csr_inl[rb]), its INLINE elements [csr_inl[rb], csr.ptr[rb + 1]).
     const int32_t *csr_inl;
@@ -396,6 +400,9 @@ __device__ __forceinline__ void chk_entry(const Device &d, bool csr_view, uint32
 __device__ __forceinline__ uint32_t mask_of(const uint32_t *mask32, int blk) {
     return reinterpret_cast<const uint16_t *>(mask32)[blk];
 }
+
+// Order-preserving map of fp32 to signed words: monotone, and the bits themselves where v >= 0.
+__host__ __device__ inline int ordered_word(int bits) { return bits ^ ((bits >> 31) & 0x7FFFFFFF); }
 
 // Adds one sum to a row of the accumulator (see ACC_CLEAR).
 __device__ __forceinline__ bool acc_needs_flag(float v) { return !(fabsf(v) >= ACC_FLAG_MIN); }

@@ -21,7 +21,6 @@
 #include <cooperative_groups.h>
 
 #include "internal.cuh"
-#include "lean_pull.cuh"
 #include "minplus.cuh"
 #include "push_direct.cuh"
 
@@ -34,7 +33,7 @@ constexpr int SSSP_COLS = SSSP_CTA * 4;
 constexpr int SSSP_ILP = 4;                       // warp steps in flight
 // A step whose frontier reaches more than this share of the stored elements is pulled.
 #ifndef DBS_SSSP_PULL_SHARE
-#define DBS_SSSP_PULL_SHARE 0.1f
+#define DBS_SSSP_PULL_SHARE 0.05f
 #endif
 constexpr int SSSP_MAX_STEPS = 1024;              // steps of one launch, at most: a cycle of negative weight ends on the host
 
@@ -49,15 +48,10 @@ struct SsspState {
 };
 
 // ordered(v): monotone in v, and the bits themselves where v >= 0
-__device__ __forceinline__ int sssp_word(float v) { const int b = __float_as_int(v); return b ^ ((b >> 31) & 0x7FFFFFFF); }
-__device__ __forceinline__ float sssp_value(int w) { return __int_as_float(w ^ ((w >> 31) & 0x7FFFFFFF)); }
-
-// Per warp: the rows that the chunk adds to and their words.
-constexpr int SSSP_ROWS = 32;
-struct SsspRows { int row[SSSP_ROWS], word[SSSP_ROWS]; };
+__device__ __forceinline__ int sssp_word(float v) { return ordered_word(__float_as_int(v)); }
+__device__ __forceinline__ float sssp_value(int w) { return __int_as_float(ordered_word(w)); }
 
 struct SsspShared {
-    SsspRows pull[SSSP_WARPS];
     unsigned long long edges[SSSP_WARPS];
     int pre[SSSP_COLS + 1];                       // elements before a column of the round
     int2 run[SSSP_COLS];                          // position of its first entry minus that; its distance
@@ -239,89 +233,118 @@ __device__ void sssp_long(const Device &d, const SsspState &s, uint32_t *next, i
     }
 }
 
-// A large step pulled: every stored element once, in the order of the block-CSR view (see lean_pull.cuh: chunks of LEAN_CHUNK entries, eight
-// consecutive ones per lane, the next chunk's in registers already).  A row's elements are adjacent, so its word is at hand, and an element whose
-// weight alone rules it out -- smallest distance of the frontier + weight is no improvement -- costs a comparison and no gather: four fifths of them in
-// the late large steps of an R-MAT search.  The others gather the column's distance (columns outside the frontier too: they improve nothing, their edges were
-// relaxed when they entered it).  Improvements are few: an atomic each, one per warp where the whole chunk lies in one row.
+// A large step pulled.  Every row walks its own elements, which lie by weight (Device::weightrun), and stops at the first that
+// cannot improve it: smallest distance of the frontier + weight >= the row's best.  In the late large steps of an R-MAT search that leaves a
+// seventh of the elements, and a row reached for the first time soon has a best of its own.  Columns outside the
+// frontier improve nothing (their edges were relaxed when they entered it), so they need no test.
+// A lane walks the rows of its own, four elements (one 32-byte sector) a round, row after row, the next row's place fetched meanwhile; a row that has not
+// stopped after SSSP_ROUNDS rounds is finished by the whole warp.  Handles of unit weights walk the row-run index.
+constexpr int SSSP_ROUNDS = 8;
 template <int DT>
-__device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist, uint32_t *next, int low, SsspRows &rows) {
+__device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist, uint32_t *next, int low) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
-    constexpr int K = LEAN_PER_LANE;
+    constexpr int NONE = 0x7F800000;
     const int lane = threadIdx.x & 31;
-    const uint32_t lt = (1u << lane) - 1u;
     const int gwarp = (int)(blockIdx.x * SSSP_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
     const float xmin = sssp_value(low);
     auto lower = [&](int row, int best) {
         if (best < atomicMin(s.word + row, best)) atomicOr(next + (row >> 5), 1u << (row & 31));
     };
-    // rows ord - 1, ord, ... of the row list: the first one runs into the chunk
-    auto rows_of = [&](int c) {
-        if (c >= d.n_lean_chunks) return -1;
-        const int o = d.lean_chunk_ord[c] - 1 + lane;
-        return o >= 0 && o < d.n_lean_rows ? __ldg(d.lean_rows + o) : -1;
+    // element k of the runs: its column and weight
+    auto four = [&](int k0, uint32_t (&col)[4], float (&w)[4]) {       // k0 a multiple of four
+        if (VAL) {
+            const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(d.weightrun + k0)), b = __ldcs(reinterpret_cast<const uint4 *>(d.weightrun + k0 + 2));
+            col[0] = a.x; w[0] = __uint_as_float(a.y); col[1] = a.z; w[1] = __uint_as_float(a.w);
+            col[2] = b.x; w[2] = __uint_as_float(b.y); col[3] = b.z; w[3] = __uint_as_float(b.w);
+        } else {
+            const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(d.rowrun_idx + k0));
+            const uint32_t v[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) { col[j] = (v[j] & IDX_MASK) * 16u + (v[j] >> 27); w[j] = 1.0f; }
+        }
     };
-    auto word_of = [&](int row) { return row >= 0 ? __ldcg(s.word + row) : 0; };
-    LeanRegs nxt = {};
-    int row1 = rows_of(gwarp), row2 = rows_of(gwarp + nwarps), word1 = word_of(row1);
-    if (gwarp < d.n_lean_chunks) nxt = lean_fetch<VAL>(d, gwarp, lane);
-    for (int c = gwarp; c < d.n_lean_chunks; c += nwarps) {
-        const LeanRegs r = nxt;
-        __syncwarp();                                  // (the previous chunk's look-ups are over)
-        rows.row[lane] = row1;
-        rows.word[lane] = word1;
-        __syncwarp();
-        const int ord = d.lean_chunk_ord[c];
-        if (c + nwarps < d.n_lean_chunks) nxt = lean_fetch<VAL>(d, c + nwarps, lane);
-        row1 = row2;
-        word1 = word_of(row1);
-        row2 = rows_of(c + 2 * nwarps);
-        const uint32_t idx[K] = {r.i0.x, r.i0.y, r.i0.z, r.i0.w, r.i1.x, r.i1.y, r.i1.z, r.i1.w};
-        const uint32_t wv[K] = {r.w0.x, r.w0.y, r.w0.z, r.w0.w, r.w1.x, r.w1.y, r.w1.z, r.w1.w};
-        uint32_t hb = 0u;                              // bit k: entry k starts a row
+    // no element behind one of weight w can do better than this (the order goes by the upper bits)
+    auto bound = [&](float w) { return sssp_word(xmin + (VAL ? sssp_value(sssp_word(w) & ~((1 << (32 - SSSP_WEIGHT_BITS)) - 1)) : w)); };
+    // 32 rows per lane where there are that many, fewer on a small graph (see bfs_pull_rows)
+    const int n_groups = (int)((d.n + 31) / 32);
+    int W = 32;
+    while (W > 1 && (int64_t)nwarps * (W / 2) >= n_groups) W >>= 1;
+    for (int g0 = gwarp * W; g0 < n_groups; g0 += nwarps * W) {
+        int k = 0, row = -1, p = 0, e = 0, have = 0, best = NONE, rounds = 0;      // the row being walked: elements [p, e)
+        int row_n = -1, p_n = 0, e_n = 0, have_n = 0;                              // the next one
+        uint32_t longm = 0u;
+        // (row of group g0 + k: lane + k mod 32, so that no lane gets the heavy rows of every group)
+        auto fetch = [&]() {
+            row_n = -1;
+            if (k < W && g0 + k < n_groups) {
+                const int64_t r = (int64_t)(g0 + k) * 32 + ((lane + k) & 31);
+                if (r < d.n) { row_n = (int)r; p_n = d.rowrun_ptr[r]; e_n = d.rowrun_ptr[r + 1]; have_n = __ldcg(s.word + r); }
+                else row_n = -2;                       // no such row, but the walk goes on
+                ++k;
+            }
+        };
+        fetch();
+        while (__any_sync(FULL, row >= 0 || row_n != -1)) {
+            if (row < 0 && row_n != -1) {
+                row = row_n; p = p_n; e = e_n; have = have_n; best = have_n; rounds = 0;
+                if (row < 0 || p >= e) row = -1;
+                fetch();
+            }
+            if (row >= 0) {
+                uint32_t col[4];
+                float w[4], x[4];
+                const int q0 = p & ~3;
+                four(q0, col, w);
 #pragma unroll
-        for (int k = 0; k < K; ++k) hb |= ((idx[k] >> 27) & 1u) << k;
-        const int cnt = __popc(hb);
-        int excl = cnt;                                // row starts in the lanes below
+                for (int j = 0; j < 4; ++j) {
+                    x[j] = __int_as_float(NONE);
+                    if (q0 + j >= p && q0 + j < e && sssp_word(xmin + w[j]) < best && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
+                }
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, excl, o); if (lane >= o) excl += t; }
-        const int total = __shfl_sync(FULL, excl, 31);
-        excl -= cnt;
-        auto row_at = [&](int q) { return q < SSSP_ROWS ? rows.row[q] : d.lean_rows[ord - 1 + q]; };
-        auto word_at = [&](int q) { return q < SSSP_ROWS ? rows.word[q] : __ldcg(s.word + d.lean_rows[ord - 1 + q]); };
-        // which entries may improve their row
-        float x[K];
-        {
-            int q = excl;
-            float have = sssp_value(word_at(q));
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                if ((hb >> k) & 1u) have = sssp_value(word_at(++q));
-                x[k] = __int_as_float(0x7F800000);
-                const bool go = idx[k] < (1u << TYPE_SHIFT) && xmin + Val<DT>::inline_value(wv[k]) < have && DBS_CHK_INDEX(d, idx[k] & IDX_MASK, d.nb);
-                const uint32_t a = k < 4 ? r.a.x : r.a.y;
-                if (go) x[k] = __ldca(dist + ((idx[k] & IDX_MASK) * 16u + ((a >> (8 * (k & 3))) & 15u)));
+                for (int j = 0; j < 4; ++j) best = min(best, sssp_word(x[j] + w[j]));
+                p = q0 + 4;
+                if (p >= e || bound(w[3]) >= best) { if (best < have) lower(row, best); row = -1; }
+                else if (++rounds == SSSP_ROUNDS) {     // a long row: what has been found so far counts, the rest below
+                    if (best < have) lower(row, best);
+                    longm |= 1u << (((row >> 5) - g0) & 31);
+                    row = -1;
+                }
             }
         }
-        if (total == 0) {                              // the whole chunk lies in one row
-            int best = 0x7F800000;
+        uint32_t lanes_long = __ballot_sync(FULL, longm != 0u);
+        while (lanes_long) {
+            const int src = __ffs(lanes_long) - 1;
+            lanes_long &= lanes_long - 1;
+            for (uint32_t lm = __shfl_sync(FULL, longm, src); lm; lm &= lm - 1) {
+                const int kk = __ffs(lm) - 1;
+                const int64_t r = (int64_t)(g0 + kk) * 32 + ((src + kk) & 31);
+                const int end = d.rowrun_ptr[r + 1];
+                int q = (d.rowrun_ptr[r] & ~3) + SSSP_ROUNDS * 4;
+                const int had = __ldcg(s.word + r);
+                int now = had;
+                for (; q < end; q += 128) {            // four elements per lane
+                    uint32_t col[4];
+                    float w[4], x[4];
+                    const int k0 = q + 4 * lane;
+                    w[3] = 0.f;
+                    int mine = now;
+                    if (k0 < end) {
+                        four(k0, col, w);
 #pragma unroll
-            for (int k = 0; k < K; ++k) best = min(best, sssp_word(x[k] + Val<DT>::inline_value(wv[k])));
-            best = __reduce_min_sync(FULL, best);
-            if (lane == 0 && best < rows.word[0]) lower(rows.row[0], best);
-            continue;
-        }
-        int q = excl, best = 0x7F800000;
+                        for (int j = 0; j < 4; ++j) {
+                            x[j] = __int_as_float(NONE);
+                            if (k0 + j < end && sssp_word(xmin + w[j]) < now && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
+                        }
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            if ((hb >> k) & 1u) {
-                if (best < 0x7F800000 && best < word_at(q)) lower(row_at(q), best);
-                best = 0x7F800000;
-                ++q;
+                        for (int j = 0; j < 4; ++j) mine = min(mine, sssp_word(x[j] + w[j]));
+                    }
+                    now = __reduce_min_sync(FULL, mine);
+                    const bool over = k0 + 3 >= end || bound(w[3]) >= now;
+                    if (__shfl_sync(FULL, (int)over, 31)) break;       // (the last lane's weight is the largest of the step)
+                }
+                if (lane == 0 && now < had) lower((int)r, now);
             }
-            best = min(best, sssp_word(x[k] + Val<DT>::inline_value(wv[k])));
         }
-        if (best < 0x7F800000 && best < word_at(q)) lower(row_at(q), best);
     }
     // entries with a payload: one block per warp at a time
     for (int q = gwarp; q < d.n_payload; q += nwarps) {
@@ -360,7 +383,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int
         int32_t *n_long = s.ctr + 3 + t % 3;
         if (tid == 0) s.ctr[3 + (t + 1) % 3] = 0;      // (its last reader was step t - 2)
         if (__ldcg(s.edges + t % 3) > pull_edges) {    // grid-uniform
-            sssp_pull<DT>(d, s, dist, next, __ldcg(s.low + t % 3), sh.pull[threadIdx.x >> 5]);
+            sssp_pull<DT>(d, s, dist, next, __ldcg(s.low + t % 3));
             grid.sync();
         } else {
             sssp_expand<DT>(d, s, dist, F, next, n_long, sh);
