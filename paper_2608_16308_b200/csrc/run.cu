@@ -2296,8 +2296,10 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     s.n_words = (int32_t)((d.n + 31) / 32);
     const size_t word_bytes = ((size_t)s.n_words * 32 * sizeof(int) + 255) & ~(size_t)255, bit_bytes = ((size_t)s.n_words * 4 + 255) & ~(size_t)255;
     if (!h->sssp_host && cudaHostAlloc(reinterpret_cast<void **>(&h->sssp_host), 4 * sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess) { h->sssp_host = nullptr; return DBSPMSPV_ERR_ALLOC; }
+    // chunks of long rows: a row has more than 4 (SSSP_ROUNDS - 1) elements before any of it is listed
+    const size_t chunk_bytes = ((size_t)d.n_entries / (4 * (SSSP_ROUNDS - 1)) + (size_t)d.n_entries / SSSP_CHUNK + 64) * sizeof(int4);
     if (!h->sssp_state) {
-        if (cudaMalloc(&h->sssp_state, word_bytes + 2 * bit_bytes + 128) != cudaSuccess) { h->sssp_state = nullptr; return DBSPMSPV_ERR_ALLOC; }
+        if (cudaMalloc(&h->sssp_state, word_bytes + 2 * bit_bytes + 256 + chunk_bytes) != cudaSuccess) { h->sssp_state = nullptr; return DBSPMSPV_ERR_ALLOC; }
         DBS_CUDA(cudaFuncSetAttribute(k_sssp<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsspShared)));
     }
     uint8_t *p = static_cast<uint8_t *>(h->sssp_state);
@@ -2307,6 +2309,7 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     s.ctr = reinterpret_cast<int32_t *>(p + word_bytes + 2 * bit_bytes);
     s.low = s.ctr + 8;
     s.edges = reinterpret_cast<unsigned long long *>(s.ctr + 12);
+    s.chunks = reinterpret_cast<int4 *>(p + word_bytes + 2 * bit_bytes + 256);
     s.report = h->sssp_host;
     Device dev = d;
     int start = 1;

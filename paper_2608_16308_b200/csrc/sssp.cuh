@@ -35,6 +35,8 @@ constexpr int SSSP_ILP = 4;                       // warp steps in flight
 #ifndef DBS_SSSP_PULL_SHARE
 #define DBS_SSSP_PULL_SHARE 0.05f
 #endif
+constexpr int SSSP_ROUNDS = 8;                    // rounds of four elements that a lane walks of a row
+constexpr int SSSP_CHUNK = 512;                   // elements of a listed chunk of a longer row
 constexpr int SSSP_MAX_STEPS = 1024;              // steps of one launch, at most: a cycle of negative weight ends on the host
 
 struct SsspState {
@@ -43,6 +45,7 @@ struct SsspState {
     int32_t *ctr;             // [0..2] vertices of the frontier, [3..5] listed chunks (sets rotate by step), [6] steps made
     int *low;                 // smallest word of the frontier, rotating with the counters
     unsigned long long *edges;   // out-edges of the frontier in INLINE runs, likewise
+    int4 *chunks;             // {row, first, end, -} of the listed chunks of long rows
     int32_t *report;          // page-locked host words: steps made, vertices of the frontier that was left
     int32_t n_words;
 };
@@ -233,38 +236,46 @@ __device__ void sssp_long(const Device &d, const SsspState &s, uint32_t *next, i
     }
 }
 
+// A row's new best.
+__device__ __forceinline__ void sssp_lower(const SsspState &s, uint32_t *next, int row, int best) {
+    if (best < atomicMin(s.word + row, best)) atomicOr(next + (row >> 5), 1u << (row & 31));
+}
+// Elements k0 .. k0 + 3 (k0 a multiple of four) of the runs: columns and weights.
+template <bool VAL>
+__device__ __forceinline__ void sssp_four(const Device &d, int k0, uint32_t (&col)[4], float (&w)[4]) {
+    if (VAL) {
+        const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(d.weightrun + k0)), b = __ldcs(reinterpret_cast<const uint4 *>(d.weightrun + k0 + 2));
+        col[0] = a.x; w[0] = __uint_as_float(a.y); col[1] = a.z; w[1] = __uint_as_float(a.w);
+        col[2] = b.x; w[2] = __uint_as_float(b.y); col[3] = b.z; w[3] = __uint_as_float(b.w);
+    } else {
+        const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(d.rowrun_idx + k0));
+        const uint32_t v[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { col[j] = (v[j] & IDX_MASK) * 16u + (v[j] >> 27); w[j] = 1.0f; }
+    }
+}
+// No element behind one of weight w can do better than this (the order goes by the upper bits).
+template <bool VAL>
+__device__ __forceinline__ int sssp_bound(float xmin, float w) {
+    return sssp_word(xmin + (VAL ? sssp_value(sssp_word(w) & ~((1 << (32 - SSSP_WEIGHT_BITS)) - 1)) : w));
+}
+
 // A large step pulled.  Every row walks its own elements, which lie by weight (Device::weightrun), and stops at the first that
 // cannot improve it: smallest distance of the frontier + weight >= the row's best.  In the late large steps of an R-MAT search that leaves a
 // seventh of the elements, and a row reached for the first time soon has a best of its own.  Columns outside the
 // frontier improve nothing (their edges were relaxed when they entered it), so they need no test.
-// A lane walks the rows of its own, four elements (one 32-byte sector) a round, row after row, the next row's place fetched meanwhile; a row that has not
-// stopped after SSSP_ROUNDS rounds is finished by the whole warp.  Handles of unit weights walk the row-run index.
-constexpr int SSSP_ROUNDS = 8;
+// A lane walks the rows of its own, four elements (one 32-byte sector) a round, row after row, the next row's place fetched meanwhile; what is left of a row that has not
+// stopped after SSSP_ROUNDS rounds is listed in chunks, which all warps share out behind a grid barrier (walked by the warp that met them, the
+// hub rows of an R-MAT graph, neighbours all, took one warp 300 us).  Handles of unit weights walk the row-run index.
 template <int DT>
-__device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist, uint32_t *next, int low) {
+__device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist, uint32_t *next, int low, int32_t *n_long) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int NONE = 0x7F800000;
     const int lane = threadIdx.x & 31;
     const int gwarp = (int)(blockIdx.x * SSSP_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
     const float xmin = sssp_value(low);
-    auto lower = [&](int row, int best) {
-        if (best < atomicMin(s.word + row, best)) atomicOr(next + (row >> 5), 1u << (row & 31));
-    };
-    // element k of the runs: its column and weight
-    auto four = [&](int k0, uint32_t (&col)[4], float (&w)[4]) {       // k0 a multiple of four
-        if (VAL) {
-            const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(d.weightrun + k0)), b = __ldcs(reinterpret_cast<const uint4 *>(d.weightrun + k0 + 2));
-            col[0] = a.x; w[0] = __uint_as_float(a.y); col[1] = a.z; w[1] = __uint_as_float(a.w);
-            col[2] = b.x; w[2] = __uint_as_float(b.y); col[3] = b.z; w[3] = __uint_as_float(b.w);
-        } else {
-            const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(d.rowrun_idx + k0));
-            const uint32_t v[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) { col[j] = (v[j] & IDX_MASK) * 16u + (v[j] >> 27); w[j] = 1.0f; }
-        }
-    };
-    // no element behind one of weight w can do better than this (the order goes by the upper bits)
-    auto bound = [&](float w) { return sssp_word(xmin + (VAL ? sssp_value(sssp_word(w) & ~((1 << (32 - SSSP_WEIGHT_BITS)) - 1)) : w)); };
+    auto lower = [&](int row, int best) { sssp_lower(s, next, row, best); };
+    auto bound = [&](float w) { return sssp_bound<VAL>(xmin, w); };
     // 32 rows per lane where there are that many, fewer on a small graph (see bfs_pull_rows)
     const int n_groups = (int)((d.n + 31) / 32);
     int W = 32;
@@ -273,6 +284,7 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
         int k = 0, row = -1, p = 0, e = 0, have = 0, best = NONE, rounds = 0;      // the row being walked: elements [p, e)
         int row_n = -1, p_n = 0, e_n = 0, have_n = 0;                              // the next one
         uint32_t longm = 0u;
+        int n_chunks = 0;
         // (row of group g0 + k: lane + k mod 32, so that no lane gets the heavy rows of every group)
         auto fetch = [&]() {
             row_n = -1;
@@ -294,7 +306,7 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
                 uint32_t col[4];
                 float w[4], x[4];
                 const int q0 = p & ~3;
-                four(q0, col, w);
+                sssp_four<VAL>(d, q0, col, w);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     x[j] = __int_as_float(NONE);
@@ -307,42 +319,22 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
                 else if (++rounds == SSSP_ROUNDS) {     // a long row: what has been found so far counts, the rest below
                     if (best < have) lower(row, best);
                     longm |= 1u << (((row >> 5) - g0) & 31);
+                    n_chunks += (e - p + SSSP_CHUNK - 1) / SSSP_CHUNK;
                     row = -1;
                 }
             }
         }
-        uint32_t lanes_long = __ballot_sync(FULL, longm != 0u);
-        while (lanes_long) {
-            const int src = __ffs(lanes_long) - 1;
-            lanes_long &= lanes_long - 1;
-            for (uint32_t lm = __shfl_sync(FULL, longm, src); lm; lm &= lm - 1) {
-                const int kk = __ffs(lm) - 1;
-                const int64_t r = (int64_t)(g0 + kk) * 32 + ((src + kk) & 31);
-                const int end = d.rowrun_ptr[r + 1];
-                int q = (d.rowrun_ptr[r] & ~3) + SSSP_ROUNDS * 4;
-                const int had = __ldcg(s.word + r);
-                int now = had;
-                for (; q < end; q += 128) {            // four elements per lane
-                    uint32_t col[4];
-                    float w[4], x[4];
-                    const int k0 = q + 4 * lane;
-                    w[3] = 0.f;
-                    int mine = now;
-                    if (k0 < end) {
-                        four(k0, col, w);
+        if (__any_sync(FULL, n_chunks > 0)) {
+            int incl = n_chunks;
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            x[j] = __int_as_float(NONE);
-                            if (k0 + j < end && sssp_word(xmin + w[j]) < now && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
-                        }
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) mine = min(mine, sssp_word(x[j] + w[j]));
-                    }
-                    now = __reduce_min_sync(FULL, mine);
-                    const bool over = k0 + 3 >= end || bound(w[3]) >= now;
-                    if (__shfl_sync(FULL, (int)over, 31)) break;       // (the last lane's weight is the largest of the step)
-                }
-                if (lane == 0 && now < had) lower((int)r, now);
+            for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
+            int base = 0;
+            if (lane == 31) base = atomicAdd(n_long, incl);
+            int at = __shfl_sync(FULL, base, 31) + incl - n_chunks;
+            for (; longm; longm &= longm - 1) {
+                const int kk = __ffs(longm) - 1;
+                const int r = (g0 + kk) * 32 + ((lane + kk) & 31), end = d.rowrun_ptr[r + 1];
+                for (int q = (d.rowrun_ptr[r] & ~3) + SSSP_ROUNDS * 4; q < end; q += SSSP_CHUNK) s.chunks[at++] = make_int4(r, q, min(end, q + SSSP_CHUNK), 0);
             }
         }
     }
@@ -359,6 +351,47 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
             const int c = sssp_word(minplus_value(key)), row = rb * 16 + r;
             if (c < __ldcg(s.word + row)) lower(row, c);
         });
+    }
+}
+
+// The listed chunks of long rows, a warp per chunk, four elements per lane and step.
+template <int DT>
+__device__ void sssp_pull_long(const Device &d, const SsspState &s, const float *dist, uint32_t *next, int low, int n) {
+    constexpr bool VAL = DT != DBSPMSPV_PATTERN;
+    const int lane = threadIdx.x & 31;
+    const int gwarp = (int)(blockIdx.x * SSSP_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
+    const float xmin = sssp_value(low);
+    int4 ahead = gwarp < n ? __ldcg(s.chunks + gwarp) : make_int4(0, 0, 0, 0);
+    for (int i = gwarp; i < n; i += nwarps) {
+        const int4 c = ahead;
+        if (i + nwarps < n) ahead = __ldcg(s.chunks + i + nwarps);
+        const int had = __ldcg(s.word + c.x);
+        int now = had;
+        uint32_t col[4], col_n[4];
+        float w[4], w_n[4];
+        const int k0 = c.y + 4 * lane;
+        if (k0 < c.z) sssp_four<VAL>(d, k0, col, w);
+        for (int q = k0; q - 4 * lane < c.z; q += 128) {
+            if (q + 128 < c.z) sssp_four<VAL>(d, q + 128, col_n, w_n);
+            float x[4];
+            int mine = now;
+            bool over = true;
+            if (q < c.z) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    x[j] = __int_as_float(0x7F800000);
+                    if (q + j < c.z && sssp_word(xmin + w[j]) < now && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) mine = min(mine, sssp_word(x[j] + w[j]));
+            }
+            now = __reduce_min_sync(FULL, mine);
+            if (q < c.z) over = sssp_bound<VAL>(xmin, w[3]) >= now;
+            if (__shfl_sync(FULL, (int)over, 31)) break;               // (the last lane's weight is the largest of the step; past the end: done)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) { col[j] = col_n[j]; w[j] = w_n[j]; }
+        }
+        if (lane == 0 && now < had) sssp_lower(s, next, c.x, now);
     }
 }
 
@@ -383,8 +416,14 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int
         int32_t *n_long = s.ctr + 3 + t % 3;
         if (tid == 0) s.ctr[3 + (t + 1) % 3] = 0;      // (its last reader was step t - 2)
         if (__ldcg(s.edges + t % 3) > pull_edges) {    // grid-uniform
-            sssp_pull<DT>(d, s, dist, next, __ldcg(s.low + t % 3));
+            const int low = __ldcg(s.low + t % 3);
+            sssp_pull<DT>(d, s, dist, next, low, n_long);
             grid.sync();
+            const int n = __ldcg(n_long);
+            if (n > 0) {                               // grid-uniform
+                sssp_pull_long<DT>(d, s, dist, next, low, n);
+                grid.sync();
+            }
         } else {
             sssp_expand<DT>(d, s, dist, F, next, n_long, sh);
             grid.sync();
