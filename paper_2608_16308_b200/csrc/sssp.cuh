@@ -276,20 +276,20 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
     const float xmin = sssp_value(low);
     auto lower = [&](int row, int best) { sssp_lower(s, next, row, best); };
     auto bound = [&](float w) { return sssp_bound<VAL>(xmin, w); };
-    // 32 rows per lane where there are that many, fewer on a small graph (see bfs_pull_rows)
+    // Up to 32 groups of 32 rows per warp, spread over the matrix: on an R-MAT graph that was not relabelled neighbouring rows are heavy together
+    // (a warp that took eight neighbouring groups of hubs: 136 us where the step takes 60).
     const int n_groups = (int)((d.n + 31) / 32);
-    int W = 32;
-    while (W > 1 && (int64_t)nwarps * (W / 2) >= n_groups) W >>= 1;
-    for (int g0 = gwarp * W; g0 < n_groups; g0 += nwarps * W) {
-        int k = 0, row = -1, p = 0, e = 0, have = 0, best = NONE, rounds = 0;      // the row being walked: elements [p, e)
-        int row_n = -1, p_n = 0, e_n = 0, have_n = 0;                              // the next one
+    for (int64_t g0 = gwarp; g0 < n_groups; g0 += 32ll * nwarps) {
+        int k = 0, row = -1, p = 0, e = 0, have = 0, best = NONE, q_long = 0;      // the row being walked: elements [p, e), from q_long on it is long
+        int k_row = 0, k_n = 0, row_n = -1, p_n = 0, e_n = 0, have_n = 0;                              // the next one
         uint32_t longm = 0u;
         int n_chunks = 0;
-        // (row of group g0 + k: lane + k mod 32, so that no lane gets the heavy rows of every group)
+        // (row lane + k mod 32 of the k-th group, so that no lane gets the heavy rows of every group)
         auto fetch = [&]() {
             row_n = -1;
-            if (k < W && g0 + k < n_groups) {
-                const int64_t r = (int64_t)(g0 + k) * 32 + ((lane + k) & 31);
+            if (k < 32 && g0 + (int64_t)k * nwarps < n_groups) {
+                const int64_t r = (g0 + (int64_t)k * nwarps) * 32 + ((lane + k) & 31);
+                k_n = k;
                 if (r < d.n) { row_n = (int)r; p_n = d.rowrun_ptr[r]; e_n = d.rowrun_ptr[r + 1]; have_n = __ldcg(s.word + r); }
                 else row_n = -2;                       // no such row, but the walk goes on
                 ++k;
@@ -298,28 +298,33 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
         fetch();
         while (__any_sync(FULL, row >= 0 || row_n != -1)) {
             if (row < 0 && row_n != -1) {
-                row = row_n; p = p_n; e = e_n; have = have_n; best = have_n; rounds = 0;
+                row = row_n; k_row = k_n; p = p_n; e = e_n; have = have_n; best = have_n; q_long = (p & ~3) + SSSP_ROUNDS * 4;
                 if (row < 0 || p >= e) row = -1;
                 fetch();
             }
             if (row >= 0) {
-                uint32_t col[4];
-                float w[4], x[4];
+                // (a row that was never reached needs several rounds: two groups at a time until something is found)
+                uint32_t col[8];
+                float w[8], x[8];
                 const int q0 = p & ~3;
-                sssp_four<VAL>(d, q0, col, w);
+                const bool two = best == NONE && q0 + 4 < e;
+                sssp_four<VAL>(d, q0, reinterpret_cast<uint32_t (&)[4]>(col[0]), reinterpret_cast<float (&)[4]>(w[0]));
+                if (two) sssp_four<VAL>(d, q0 + 4, reinterpret_cast<uint32_t (&)[4]>(col[4]), reinterpret_cast<float (&)[4]>(w[4]));
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < 8; ++j) {
                     x[j] = __int_as_float(NONE);
-                    if (q0 + j >= p && q0 + j < e && sssp_word(xmin + w[j]) < best && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
+                    if ((j < 4 || two) && q0 + j >= p && q0 + j < e && sssp_word(xmin + w[j]) < best && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
                 }
+                float last = w[3];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) best = min(best, sssp_word(x[j] + w[j]));
-                p = q0 + 4;
-                if (p >= e || bound(w[3]) >= best) { if (best < have) lower(row, best); row = -1; }
-                else if (++rounds == SSSP_ROUNDS) {     // a long row: what has been found so far counts, the rest below
+                for (int j = 0; j < 8; ++j)
+                    if (j < 4 || two) { best = min(best, sssp_word(x[j] + w[j])); last = w[j]; }
+                p = q0 + (two ? 8 : 4);
+                if (p >= e || bound(last) >= best) { if (best < have) lower(row, best); row = -1; }
+                else if (p >= q_long) {     // a long row: what has been found so far counts, the rest below
                     if (best < have) lower(row, best);
-                    longm |= 1u << (((row >> 5) - g0) & 31);
-                    n_chunks += (e - p + SSSP_CHUNK - 1) / SSSP_CHUNK;
+                    longm |= 1u << k_row;
+                    n_chunks += (e - q_long + SSSP_CHUNK - 1) / SSSP_CHUNK;
                     row = -1;
                 }
             }
@@ -333,7 +338,7 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
             int at = __shfl_sync(FULL, base, 31) + incl - n_chunks;
             for (; longm; longm &= longm - 1) {
                 const int kk = __ffs(longm) - 1;
-                const int r = (g0 + kk) * 32 + ((lane + kk) & 31), end = d.rowrun_ptr[r + 1];
+                const int r = (int)((g0 + (int64_t)kk * nwarps) * 32 + ((lane + kk) & 31)), end = d.rowrun_ptr[r + 1];
                 for (int q = (d.rowrun_ptr[r] & ~3) + SSSP_ROUNDS * 4; q < end; q += SSSP_CHUNK) s.chunks[at++] = make_int4(r, q, min(end, q + SSSP_CHUNK), 0);
             }
         }
