@@ -97,8 +97,9 @@ typedef struct {
     int32_t w_inline;        /* ... of an INLINE view entry                         (1)      */
     int32_t w_dense_sparse;  /* Dense / CSR-like weights used instead when such blocks are a */
     int32_t w_mid_sparse;    /* minority of the matrix (hypersparse matrices)  (128 / 64)    */
-    int32_t no_bfs_index;    /* 1: do not build the row-run index that square matrices get for
-                                the pull levels of db_bfs (4 bytes per stored element; a pull
+    int32_t no_bfs_index;    /* 1: do not build the row-run indexes that square matrices get for
+                                the pull levels of db_bfs (4 bytes per stored element) and, fp32,
+                                the pulled steps of db_sssp (8 bytes per stored element; a pull
                                 level then walks whole row-block segments)          (0)    */
     int32_t reserved[2];
 } dbspmspv_create_opts;
@@ -277,13 +278,14 @@ int db_bfs(dbspmspv_handle_t h, int32_t src, int32_t *levels, dbspmspv_stream_t 
  *   dist     out: n fp32 on the device; source 0, unreachable +infinity.  Every path sum is
  *            accumulated in fp32 in path order.
  *   n_steps  out (host, may be NULL): products made, the last one with an empty result
- * Direction per step: run_opts.force_path if set; else a step whose x holds more than a tenth
- * of the stored elements as out-edges is pulled (hypersparse F32 handles; the others always
- * push), the rest pushed.
- * Unlike the other calls this one is a host loop: it waits on `stream` once per step to read
- * the size of the next x and its out-edge count (16 bytes), and the first call on a handle allocates 24 n bytes of
- * device memory and one page-locked word (freed by dbspmspv_destroy).  More than n + 1 steps
- * (a negative cycle) end the search with ERR_UNSUPPORTED.
+ * Hypersparse handles (most elements in blocks without a payload) run the whole search as one
+ * cooperative launch; each step relaxes the out-edges of x, or, where x reaches more than a twentieth of
+ * the stored elements, lets every row look for its best in-edge.  The others, and calls with
+ * run_opts.force_path set, iterate products from the host.
+ * Unlike the other calls this one waits on `stream`: once at its end (the host loop: once per step), to read
+ * the number of steps; and the first call on a handle allocates about 5 n bytes and half a byte per stored
+ * element (the host loop: 24 n bytes) of device memory and one page-locked word (freed by
+ * dbspmspv_destroy).  More than n + 1 steps (a negative cycle) end the search with ERR_UNSUPPORTED.
  */
 int db_sssp(dbspmspv_handle_t h, int32_t src, float *dist, int32_t *n_steps, dbspmspv_stream_t stream);
 
