@@ -60,23 +60,81 @@ __device__ __forceinline__ void append_words(int word, int32_t *list, int32_t *c
     if (word >= 0) list[base + __popc(m & ((1u << lane) - 1u))] = word;
 }
 
+// Where a push level puts what it finds: the next level's frontier and worklist.
+struct NextLevel {
+    uint32_t *N;                 // frontier masks
+    int32_t *words, *n_words;    // list of the words that became nonzero
+    int32_t *n_blocks, *n_tasks, *n_hubs;
+    int4 *hubs;
+    uint2 *tasks;
+    bool emit;                   // the worklist is written by this level itself
+};
+// A push level of at most this many warp steps writes the next level's worklist itself, one phase and one grid barrier (with a pass of its
+// own behind a barrier of its own a level that moves next to nothing took 8.5 us, now 6).  In a larger one the warps would
+// queue for space in the list, and the level behind it is a pull more often than not.
+#ifndef DBS_BFS_EMIT_STEPS
+#define DBS_BFS_EMIT_STEPS 256
+#endif
+
 // Boolean push: tasks of the active frontier blocks (a task is at most PUSH_CHUNK = 32 view
 // entries: one warp step); newly reached rows are claimed with one atomicOr per entry on the
 // next-frontier masks (the winner writes the level).  Like the pull, the loop is software-
 // pipelined: while task k is evaluated, the visited masks of k+1, the view entries of k+2 and
-// the task record of k+3 (in this warp's stride) are in flight.  The thread whose atomic turns a
-// word of the next-frontier masks nonzero lists that word, so that the bookkeeping after the
-// level visits the nonzero words only.
+// the task record of k+3 (in this warp's stride) are in flight.
+// The winner also does the level's bookkeeping for the vertex: it is marked visited, the word it turned nonzero
+// is listed, and (NextLevel::emit) the tasks of its column go to the next level's worklist.
 template <int DT>
-__device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, uint32_t *N, int n_recs, const int4 *hubs, int n_hubs,
-                         int32_t *levels, int depth, int32_t *words_out, int32_t *nwords_out) {
+__device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, const uint2 *tasks, int n_recs, const int4 *hubs, int n_hubs,
+                         int32_t *levels, int depth, const NextLevel &nx) {
     static_assert(PUSH_CHUNK == 32, "one warp step per task");
     const int lane = threadIdx.x & 31;
     const int gwarp = sc.gwarp, nwarps = sc.nwarps;
     const HubTable table = load_hub_table(hubs, n_hubs, lane);
     const int n_tasks = n_recs + table.total;                    // task records, then the steps of the hub runs
-    auto item = [&](int i) { return worklist_item(d.ws.tasks, n_recs, table, i); };
+    auto item = [&](int i) { return worklist_item(tasks, n_recs, table, i); };
     const uint2 none = make_uint2(0u, 0u);
+    int found = 0, blocks = 0;
+    // claims the rows `hit` of row block `brow` (called by a full warp; hit = 0: nothing in this lane)
+    auto publish = [&](int brow, uint32_t hit) {
+        uint32_t old = 0, fresh = 0;
+        const int sh = (brow & 1) * 16;
+        if (hit) {
+            old = atomicOr(&nx.N[brow >> 1], hit << sh);
+            fresh = hit & ~(old >> sh);
+        }
+        if (!__any_sync(FULL, fresh != 0u)) return;
+        const bool newly = fresh && ((old >> sh) & 0xFFFFu) == 0;
+        if (fresh) {
+            atomicOr(&d.ws.visited32[brow >> 1], fresh << sh);
+            write_levels(levels, brow, fresh, depth);
+            found += __popc(fresh);
+            blocks += newly;
+        }
+        append_words(fresh && !old ? brow >> 1 : -1, nx.words, nx.n_words, lane);
+        if (!nx.emit) return;
+        // the vertices found, 32 at a time (blocks with a payload reach several rows at once): vertex k belongs to the last lane whose prefix is <= k
+        int incl = __popc(fresh);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
+        const int excl = incl - __popc(fresh), total = __shfl_sync(FULL, incl, 31);
+        for (int k0 = 0; k0 < total; k0 += 32) {
+            const int k = k0 + lane;
+            int o = 0;
+#pragma unroll
+            for (int st = 16; st; st >>= 1) { const int t = __shfl_sync(FULL, excl, o + st); if (t <= k) o += st; }
+            uint32_t m = __shfl_sync(FULL, fresh, o);
+            const int vb = __shfl_sync(FULL, brow, o), skip = k - __shfl_sync(FULL, excl, o);
+            int first = 0, deg = 0;
+            if (k < total) {
+                for (int t = 0; t < skip; ++t) m &= m - 1;
+                column_run(d, vb * 16 + __ffs(m) - 1, first, deg);
+            }
+            emit_tasks(d, false, vb, first, deg, lane, nx.n_tasks, nx.n_blocks, PUSH_CHUNK, nx.n_hubs, nx.hubs, nx.tasks);
+        }
+        int pfirst = 0, pdeg = 0;
+        if (newly) payload_run(d, brow, pfirst, pdeg);
+        if (__any_sync(FULL, pdeg > 0)) emit_tasks(d, false, brow, pfirst, pdeg, lane, nx.n_tasks, nx.n_blocks, d.payload_chunk, nullptr, nullptr, nx.tasks);
+    };
     struct Entries { uint32_t idx, aux, xm; int n, start; };   // n: entries of the task (0 = no task)
     auto entries_of = [&](int t, const uint2 &task) {
         Entries e{0u, 0u, 0u, 0, 0};
@@ -112,9 +170,8 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, ui
             const int type = idx >> TYPE_SHIFT, brow = idx & IDX_MASK;
             bool heavy = false;
             uint32_t w = 0;
-            int fresh_word = -1;           // a mask word this lane turned nonzero
+            uint32_t hit = 0;
             if (need0) {
-                uint32_t hit = 0;
                 if (type == DBSPMSPV_BLK_INLINE) {
                     hit = ((xm >> (aux & 15)) & 1u) << (aux >> 4);
                 } else {
@@ -127,14 +184,8 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, ui
                     }
                 }
                 hit &= need0;
-                if (hit) {
-                    const int sh = (brow & 1) * 16;
-                    const uint32_t old = atomicOr(&N[brow >> 1], hit << sh);
-                    write_levels(levels, brow, hit & ~(old >> sh), depth);
-                    if (!old) fresh_word = brow >> 1;
-                }
             }
-            append_words(fresh_word, words_out, nwords_out, lane);
+            publish(brow, hit);
             uint32_t hv = __ballot_sync(FULL, heavy);
             while (hv) {
                 const int src = __ffs(hv) - 1;
@@ -145,17 +196,15 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, ui
                 const int btype = bidx >> TYPE_SHIFT, bbrow = bidx & IDX_MASK;
                 uint32_t hits = warp_block_bool<DT>(btype, d.payload + (size_t)bw * 4, nnz, xm, lane);
                 hits &= ~mask_of(d.ws.visited32, bbrow);
-                if (lane == 0 && hits) {
-                    const int sh = (bbrow & 1) * 16;
-                    const uint32_t old = atomicOr(&N[bbrow >> 1], hits << sh);
-                    write_levels(levels, bbrow, hits & ~(old >> sh), depth);
-                    if (!old) words_out[atomicAdd(nwords_out, 1)] = bbrow >> 1;
-                }
+                publish(bbrow, lane == 0 ? hits : 0u);
             }
         }
         // rotate the pipeline
         e0 = e1; e1 = e2; need0 = need1; t2 = t3;
     }
+    found = __reduce_add_sync(FULL, found);
+    blocks = __reduce_add_sync(FULL, blocks);
+    if (lane == 0 && found) { atomicAdd(&d.ws.ctr->bfs_reached, found); atomicAdd(nx.n_blocks, blocks); }
 }
 
 // Boolean pull: one warp per row-block segment (a segment has at most MAX_SEG_ENTRIES = 4 x 32
@@ -469,37 +518,28 @@ __device__ __forceinline__ int bfs_path(int n_nzblk, int nb, float th3, int forc
     return ((float)n_nzblk / (float)nb < th3) ? DBSPMSPV_PATH_PUSH : DBSPMSPV_PATH_PULL;
 }
 
-// Worklist of the frontier F from the listed nonzero words of its masks: a warp takes one word
+// Worklist of the frontier F from the listed nonzero words of its masks (behind a pull level): a warp takes one word
 // (two vector blocks) at a time, lane = column; frontier columns emit their INLINE runs (adjacent
 // ones merged), lanes 0 and 16 the payload runs of the two blocks.  (With the words in index
 // order, the few warps that held the hub blocks of an early frontier wrote almost the whole
-// worklist.)  With UPDATE the same pass also does the level's bookkeeping for the word: visited
-// is updated and the vertices found and the nonempty blocks are counted.
-template <bool UPDATE>
+// worklist.)
 __device__ void bfs_worklist(const Device &d, const Scope &sc, const uint32_t *F, const int32_t *words, int n_listed,
-                             int32_t *n_tasks, int32_t *n_hubs, int4 *hubs, int32_t *nz_out) {
+                             int32_t *n_tasks, int32_t *n_hubs, int4 *hubs, uint2 *tasks) {
     const int lane = threadIdx.x & 31;
     Counters *ctr = d.ws.ctr;
-    int found = 0, nz = 0;
     for (int i = sc.gwarp; i < n_listed; i += sc.nwarps) {
         const int wd = words[i];
         const uint32_t word = F[wd];
-        if (UPDATE) {
-            if (lane == 0) d.ws.visited32[wd] |= word;
-            found += __popc(word);
-            nz += ((word & 0xFFFFu) != 0) + ((word >> 16) != 0);
-        }
         const int jb = 2 * wd + (lane >> 4), j = jb * 16 + (lane & 15);
         const bool listed = (word >> lane) & 1u;
         int first = 0, deg = 0;
         if (listed) column_run(d, j, first, deg);
         merge_column_runs(listed, j, first, deg, lane);
-        emit_tasks(d, false, jb, first, deg, lane, n_tasks, &ctr->pad, PUSH_CHUNK, n_hubs, hubs);
+        emit_tasks(d, false, jb, first, deg, lane, n_tasks, &ctr->pad, PUSH_CHUNK, n_hubs, hubs, tasks);
         first = 0; deg = 0;
         if ((lane & 15) == 0 && ((word >> lane) & 0xFFFFu)) payload_run(d, jb, first, deg);
-        if (__any_sync(FULL, deg > 0)) emit_tasks(d, false, jb, first, deg, lane, n_tasks, &ctr->pad, d.payload_chunk);
+        if (__any_sync(FULL, deg > 0)) emit_tasks(d, false, jb, first, deg, lane, n_tasks, &ctr->pad, d.payload_chunk, nullptr, nullptr, tasks);
     }
-    if (UPDATE && lane == 0 && found) { atomicAdd(&ctr->bfs_reached, found); atomicAdd(nz_out, nz); }
 }
 
 // Path of the level whose counters are set `cur` (Section 3.3.1): push iff the ratio of nonempty
@@ -563,34 +603,15 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
                           (float)n_nzblk < BFS_WIDE_PULL * (float)d.nb, s_need + (threadIdx.x >> 5) * 32);
         grid.sync();
     } else if (path == DBSPMSPV_PATH_PUSH) {
-        bfs_push<DT>(d, sc, F, N, n_tasks, d.ws.hubs + cur * HUB_CAP, min(ctr->bfs_hubs[cur], HUB_CAP), levels, depth,
-                     words_out, &ctr->bfs_nwords[q_out]);
-        grid.sync();
         // Z (the frontier before this one) is cleared through its list
         const int nz_words = ctr->bfs_nwords[q_z];
         for (int i = sc.tid; i < nz_words; i += sc.nthreads) Z[words_z[i]] = 0u;
-        const int n_listed = ctr->bfs_nwords[q_out];
-        // With so few nonzero words that the next level is a push whatever their content, the
-        // bookkeeping and the next worklist are one pass (one barrier less); otherwise the
-        // bookkeeping first, then -- the selector's input being known -- the worklist if needed.
-        const bool surely_push = bfs_path(min(2 * n_listed, d.nb), d.nb, th3, force_path) == DBSPMSPV_PATH_PUSH;
-        if (surely_push) {
-            bfs_worklist<true>(d, sc, N, words_out, n_listed, &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], hubs_next, &ctr->bfs_cnt[nxt][0]);
-            grid.sync();
-            return;
-        }
-        int found = 0, nz = 0;
-        for (int i = sc.tid; i < n_listed; i += sc.nthreads) {
-            const int k = words_out[i];
-            const uint32_t nm = N[k];
-            d.ws.visited32[k] |= nm;
-            found += __popc(nm);
-            nz += ((nm & 0xFFFFu) != 0) + ((nm >> 16) != 0);
-        }
-        found = __reduce_add_sync(FULL, found);
-        nz = __reduce_add_sync(FULL, nz);
-        if (lane == 0 && found) { atomicAdd(&ctr->bfs_reached, found); atomicAdd(&ctr->bfs_cnt[nxt][0], nz); }
+        const int n_hubs = min(ctr->bfs_hubs[cur], HUB_CAP);
+        const NextLevel nx{N, words_out, &ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][0], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], hubs_next,
+                           lv & 1 ? d.ws.tasks : d.ws.tasks2, n_hubs == 0 && n_tasks <= DBS_BFS_EMIT_STEPS};
+        bfs_push<DT>(d, sc, F, lv & 1 ? d.ws.tasks2 : d.ws.tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
         grid.sync();
+        if (nx.emit) return;                           // (the next level's worklist is there)
     } else {
         // pull over the row-block segments (no row-run index): the masks produced are scanned as a
         // whole: visited is updated, the nonempty blocks counted, the nonzero words listed
@@ -620,7 +641,7 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
     // selector's input is known now; the level may still turn to a pull when the list is long)
     const int next_n = ctr->bfs_cnt[nxt][0];
     if (next_n && bfs_path(next_n, d.nb, th3, force_path) == DBSPMSPV_PATH_PUSH) {
-        bfs_worklist<false>(d, sc, N, words_out, ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], hubs_next, nullptr);
+        bfs_worklist(d, sc, N, words_out, ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], hubs_next, lv & 1 ? d.ws.tasks : d.ws.tasks2);
         grid.sync();
     }
 }
@@ -645,31 +666,32 @@ __global__ void __launch_bounds__(BFS_CTA) k_bfs(Device d, int32_t src, int32_t 
         if (head > d.n) head = d.n;
         const int64_t n4 = (d.n - head) / 4;
         int4 *mid = reinterpret_cast<int4 *>(levels + head);
-        for (int64_t v = tid; v < n4; v += nthreads) mid[v] = make_int4(-1, -1, -1, -1);
-        for (int64_t v = tid; v < head; v += nthreads) levels[v] = -1;
-        for (int64_t v = head + n4 * 4 + tid; v < d.n; v += nthreads) levels[v] = -1;
+        const int64_t at = (int64_t)src - head;            // the source's place in the middle
+        for (int64_t v = tid; v < n4; v += nthreads) mid[v] = v == (at >> 2) && at >= 0 ? make_int4((at & 3) ? -1 : 0, (at & 3) == 1 ? 0 : -1, (at & 3) == 2 ? 0 : -1, (at & 3) == 3 ? 0 : -1) : make_int4(-1, -1, -1, -1);
+        for (int64_t v = tid; v < head; v += nthreads) levels[v] = v == src ? 0 : -1;
+        for (int64_t v = head + n4 * 4 + tid; v < d.n; v += nthreads) levels[v] = v == src ? 0 : -1;
     }
     // rows without a stored element can never be reached through a pull: they start out as
     // "visited", so that a row block is skipped (and a segment left early) once every row that
     // can be found has been found
-    for (int k = tid; k < n_words; k += nthreads) { d.ws.visited32[k] = ~d.row_present32[k]; d.ws.x_mask32[k] = 0u; d.ws.y_mask32[k] = 0u; d.ws.z_mask32[k] = 0u; }
-    if (tid == 0) {
-        for (int k = 0; k < 3; ++k) { ctr->bfs_cnt[k][0] = 0; ctr->bfs_cnt[k][1] = 0; ctr->bfs_hubs[k] = 0; }
-        for (int k = 0; k < 4; ++k) ctr->bfs_nwords[k] = 0;
-        ctr->bfs_reached = 1;
+    // The source is the first frontier: whoever initialises its word and its level sets them right, so one barrier is enough.
+    const int src_word = src >> 5;
+    const uint32_t src_bit = 1u << (src & 31);
+    for (int k = tid; k < n_words; k += nthreads) {
+        const bool mine = k == src_word;
+        d.ws.visited32[k] = ~d.row_present32[k] | (mine ? src_bit : 0u);
+        d.ws.x_mask32[k] = mine ? src_bit : 0u; d.ws.y_mask32[k] = 0u; d.ws.z_mask32[k] = 0u;
     }
-    grid.sync();
-    // level 0: the source is the first frontier (its mask word is list 3 = "produced by level -1")
     if (blockIdx.x == 0 && threadIdx.x < 32) {
-        const int jb = src >> 4;
         if (lane == 0) {
-            levels[src] = 0;
-            const uint32_t bit = 1u << ((src & 15) + (jb & 1) * 16);
-            d.ws.x_mask32[jb >> 1] = bit;
-            d.ws.visited32[jb >> 1] |= bit;
-            d.ws.bfs_words[(size_t)3 * d.ws.bfs_words_stride] = jb >> 1;
-            ctr->bfs_nwords[3] = 1;
+            for (int k = 0; k < 3; ++k) { ctr->bfs_cnt[k][0] = 0; ctr->bfs_cnt[k][1] = 0; ctr->bfs_hubs[k] = 0; }
+            for (int k = 0; k < 4; ++k) ctr->bfs_nwords[k] = k == 3;         // (the source's mask word is list 3 = "produced by level -1")
+            ctr->bfs_reached = 1;
+            d.ws.bfs_words[(size_t)3 * d.ws.bfs_words_stride] = src_word;
         }
+        __syncwarp();
+        __threadfence();
+        const int jb = src >> 4;
         int first = 0, deg = 0;
         if (lane == 0) column_run(d, src, first, deg);
         else if (lane == 1) payload_run(d, jb, first, deg);

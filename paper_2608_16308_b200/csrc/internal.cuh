@@ -206,6 +206,7 @@ struct Counters {    // device-resident scalars of one call
 struct Workspace {
     float *x_dense;       // n (padded to a multiple of 32): dense copy of x (Section 3.2.2)
     uint32_t *x_mask32;   // vector-block masks, two 16-bit masks per word
+    uint2 *tasks2;        // BFS: a second worklist (a push level writes the next level's while it reads its own)
     uint2 *tasks;         // push worklist: (column block | (entries - 1) << 27, first CSC-view position)
     int4 *hubs;           // 3 x HUB_CAP hub runs (column block, first position, entries, -): see worklist.cuh
     float *y_acc;         // m (padded): dense accumulator, all ACC_CLEAR between calls

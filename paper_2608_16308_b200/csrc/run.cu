@@ -1867,7 +1867,11 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     // microseconds while the others have long finished).
     d.payload_chunk = h->heavy_stage ? PUSH_CHUNK : 4;
     // one partial task at most per column (INLINE run) and per column block (payload run)
-    ws.task_capacity = (int64_t)d.n_entries / d.payload_chunk + 17 * (int64_t)d.nb + 32;
+    // (Handles whose elements sit mostly in blocks with a payload take a column block as one run; elsewhere its entries with a payload
+    // and its columns are runs of their own.)
+    ws.task_capacity = h->heavy_stage ? (int64_t)d.n_entries / PUSH_CHUNK + 17 * (int64_t)d.nb + 32
+                                      : (int64_t)d.n_entries / PUSH_CHUNK + (int64_t)d.n_payload / d.payload_chunk + 17 * (int64_t)d.nb + 32;
+    if (ws.task_capacity < (d.m + 1) / 2 + 32) ws.task_capacity = (d.m + 1) / 2 + 32;      // (the short call parks the result's rows there)
     ws.n_tiles = (int32_t)ceil_div<int64_t>((d.mb + 1) / 2, TILE_WORDS);
     if (ws.n_tiles < 1) ws.n_tiles = 1;
     // One allocation for the whole workspace, carved at 512-byte boundaries (a dozen cudaMalloc
@@ -1885,6 +1889,7 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     const size_t zwords = xwords > ywords ? xwords : ywords;
     const size_t o_xd = carve(xwords * 32 * sizeof(float)), o_yacc = carve(ywords * 32 * sizeof(float)),
                  o_long = carve((size_t)d.long_cap * sizeof(*ws.long_runs)), o_tasks = carve((size_t)ws.task_capacity * sizeof(*ws.tasks)),
+                 o_tasks2 = carve((d.m == d.n ? (size_t)ws.task_capacity : 1) * sizeof(*ws.tasks)),
                  o_xm = carve(xwords * 4), o_ym = carve(ywords * 4), o_zm = carve(zwords * 4),
                  o_words = carve(4 * zwords * sizeof(*ws.bfs_words)), o_vis = carve((d.m == d.n ? ywords : 1) * 4),
                  o_hubs = carve((size_t)3 * HUB_CAP * sizeof(*ws.hubs)), o_tile = carve((size_t)ws.n_tiles * sizeof(*ws.tile_status)),
@@ -1898,6 +1903,7 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     ws.x_dense = reinterpret_cast<decltype(ws.x_dense)>(base + o_xd);
     ws.y_acc = reinterpret_cast<decltype(ws.y_acc)>(base + o_yacc);
     ws.long_runs = reinterpret_cast<decltype(ws.long_runs)>(base + o_long);
+    ws.tasks2 = reinterpret_cast<decltype(ws.tasks2)>(base + o_tasks2);
     ws.tasks = reinterpret_cast<decltype(ws.tasks)>(base + o_tasks);
     ws.x_mask32 = reinterpret_cast<decltype(ws.x_mask32)>(base + o_xm);
     ws.y_mask32 = reinterpret_cast<decltype(ws.y_mask32)>(base + o_ym);

@@ -17,7 +17,8 @@ namespace dbs {
 template <bool CTA_WIDE = false>
 __device__ __forceinline__ void emit_tasks(const Device &d, bool newly, int jb, int first, int deg, int lane,
                                            int32_t *n_tasks, int32_t *n_nzblk, int chunk = PUSH_CHUNK,
-                                           int32_t *n_hubs = nullptr, int4 *hubs = nullptr) {
+                                           int32_t *n_hubs = nullptr, int4 *hubs = nullptr, uint2 *tasks = nullptr) {
+    if (!tasks) tasks = d.ws.tasks;
     // a hub run is listed, not cut up (writing tens of thousands of task records from one warp
     // took longer than the traversal of the level they belonged to)
     if (n_hubs && deg >= HUB_MIN_ENTRIES) {
@@ -64,7 +65,7 @@ __device__ __forceinline__ void emit_tasks(const Device &d, bool newly, int jb, 
     if (nchunks <= SMALL)
         for (int k = 0; k < nchunks; ++k) {
             const int cnt = min(chunk, deg - k * chunk);
-            d.ws.tasks[base + k] = make_uint2((uint32_t)jb | ((uint32_t)(cnt - 1) << 27), (uint32_t)(first + k * chunk));
+            tasks[base + k] = make_uint2((uint32_t)jb | ((uint32_t)(cnt - 1) << 27), (uint32_t)(first + k * chunk));
         }
     uint32_t big = __ballot_sync(0xFFFFFFFFu, nchunks > SMALL);
     while (big) {
@@ -77,7 +78,7 @@ __device__ __forceinline__ void emit_tasks(const Device &d, bool newly, int jb, 
         const int bn = (bdeg + chunk - 1) / chunk;
         for (int k = lane; k < bn; k += 32) {
             const int cnt = min(chunk, bdeg - k * chunk);
-            d.ws.tasks[bbase + k] = make_uint2((uint32_t)bjb | ((uint32_t)(cnt - 1) << 27), (uint32_t)(bfirst + k * chunk));
+            tasks[bbase + k] = make_uint2((uint32_t)bjb | ((uint32_t)(cnt - 1) << 27), (uint32_t)(bfirst + k * chunk));
         }
     }
 }
