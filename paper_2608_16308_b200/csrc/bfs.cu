@@ -70,11 +70,10 @@ struct NextLevel {
     bool emit;                   // the worklist is written by this level itself
 };
 // A push level of at most this many warp steps writes the next level's worklist itself, one phase and one grid barrier (with a pass of its
-// own behind a barrier of its own a level that moves next to nothing took 8.5 us, now 6).  In a larger one the warps would
-// queue for space in the list, and the level behind it is a pull more often than not.
-#ifndef DBS_BFS_EMIT_STEPS
-#define DBS_BFS_EMIT_STEPS 256
-#endif
+// own behind a barrier of its own a level that moves next to nothing took 8.5 us, now 6).  A larger one reaches thousands of vertices: the
+// warps would queue for space in the list (with 256 steps the level took 13 us, and 100 K vertices 72 us in place of 65), and the level
+// behind it is a pull more often than not.
+constexpr int BFS_EMIT_STEPS = 16;
 
 // Boolean push: tasks of the active frontier blocks (a task is at most PUSH_CHUNK = 32 view
 // entries: one warp step); newly reached rows are claimed with one atomicOr per entry on the
@@ -608,7 +607,7 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
         for (int i = sc.tid; i < nz_words; i += sc.nthreads) Z[words_z[i]] = 0u;
         const int n_hubs = min(ctr->bfs_hubs[cur], HUB_CAP);
         const NextLevel nx{N, words_out, &ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][0], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], hubs_next,
-                           lv & 1 ? d.ws.tasks : d.ws.tasks2, n_hubs == 0 && n_tasks <= DBS_BFS_EMIT_STEPS};
+                           lv & 1 ? d.ws.tasks : d.ws.tasks2, n_hubs == 0 && n_tasks <= BFS_EMIT_STEPS};
         bfs_push<DT>(d, sc, F, lv & 1 ? d.ws.tasks2 : d.ws.tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
         grid.sync();
         if (nx.emit) return;                           // (the next level's worklist is there)
