@@ -21,8 +21,10 @@
 //     sum to global memory -- a row cut by a pass or chunk boundary simply contributes one atomic
 //     per piece.  The row a sum belongs to comes from the row list (lean_rows), indexed by the
 //     running count of ROW_FLAGs; structural hits are tracked as bit masks beside the sums.
-//   * The few entries with a payload are skipped by the stream and taken afterwards, one block
+//   * The few entries with a payload are skipped by the stream and taken before it, one block
 //     per warp at a time, from the list of their positions.
+//   * Bounds, 16 M fp32 entries, half of x listed: 58 us (73 before the filter's loads were spread and the payload entries
+//     moved to the front), L1 data path 76 % busy (gathers, filter look-ups and the stream share it), issue slots 52 %.
 //   * The same kernel serves the (min, +) semiring (Out::MINPLUS): products become sums, sums
 //     minima with identity +infinity, and the writeback keeps the smaller value (minplus.cuh).
 #pragma once
@@ -33,46 +35,24 @@
 
 namespace dbs {
 
-#ifndef DBS_LEAN_WARPS
-#define DBS_LEAN_WARPS 32
-#endif
-constexpr int LEAN_WARPS = DBS_LEAN_WARPS;     // warps per thread block; one thread block per SM
+constexpr int LEAN_WARPS = 32;     // warps per thread block; one thread block per SM
 constexpr int LEAN_CTA = LEAN_WARPS * 32;
 // Presence filter of x in shared memory: one bit per column (folded modulo the filter size when
 // x has more columns than bits), tested before every gather.
 constexpr int LEAN_FILTER_MAX_WORDS = 32768;   // 128 KB: exact up to 1,048,576 columns
-#ifndef DBS_LEAN_FILTER
-#define DBS_LEAN_FILTER 1
-#endif
-#ifndef DBS_LEAN_LDCA
-#define DBS_LEAN_LDCA 1
-#endif
-// The x gathers go through L1: on a power-law matrix a few hundred columns draw a third of all
-// gathers, and with L2-only loads those lines saturate single L2 slices.
-__device__ __forceinline__ float lean_gather(const float *p) {
-#if DBS_LEAN_LDCA
-    return __ldg(p);
-#else
-    return __ldcg(p);
-#endif
-}
 
 constexpr int LEAN_ROWS_CACHED = 64;
 constexpr int LEAN_PER_LANE = LEAN_CHUNK / 32;
 static_assert(LEAN_PER_LANE == 8, "a lane takes two 16-byte loads of view indices");
 
-// A lane's eight consecutive entries of one chunk.
-struct LeanRegs {
-    uint4 i0, i1;      // view indices
-    uint2 a;           // packed coordinates
-    uint4 w0, w1;      // values
-};
+// A lane's eight consecutive entries of one chunk: view indices, packed coordinates, values.
+struct LeanEntries { uint4 i0, i1; uint2 a; uint4 w0, w1; };
 template <bool VAL>
-__device__ __forceinline__ LeanRegs lean_fetch(const Device &d, int c, int lane) {
+__device__ __forceinline__ LeanEntries lean_fetch(const Device &d, int c, int lane) {
     // (always a whole chunk: the view arrays have that much slack behind the last entry, filled
     // with PAD_IDX entries; streaming loads: the bytes are never read again)
     const size_t e = (size_t)c * LEAN_CHUNK + (size_t)LEAN_PER_LANE * lane;
-    LeanRegs r;
+    LeanEntries r;
     r.i0 = __ldcs(reinterpret_cast<const uint4 *>(d.csr.idx + e));
     r.i1 = __ldcs(reinterpret_cast<const uint4 *>(d.csr.idx + e + 4));
     r.a = __ldcs(reinterpret_cast<const uint2 *>(d.csr.aux + e));
@@ -83,6 +63,14 @@ __device__ __forceinline__ LeanRegs lean_fetch(const Device &d, int c, int lane)
     }
     return r;
 }
+// A chunk whose dependent loads are in flight: the x entries, the values, the slice of the row list.
+struct LeanWork {
+    float xin[LEAN_PER_LANE];
+    uint4 w0, w1;
+    int rowp0, rowp1;
+    int ord;             // ROW_FLAGs before the chunk (lean_rows[ord - 1] is the row that runs into it)
+    uint32_t meta;       // bits 0-7: entry k starts a row; 8-16: row starts in the lanes below; 17: some lane holds several
+};
 
 template <int DT, typename Out>
 __device__ __forceinline__ void lean_add(Out out, int row, float v) {
@@ -97,19 +85,26 @@ template <typename Out> __device__ __forceinline__ float lean_identity() { retur
 template <typename Out> __device__ __forceinline__ float lean_mul(float a, float x) { return Out::MINPLUS ? a + x : a * x; }
 template <typename Out> __device__ __forceinline__ float lean_sum(float s, float p) { return Out::MINPLUS ? fminf(s, p) : s + p; }
 
-// One chunk = one warp pass, eight consecutive entries per lane, arranged so that the chunk costs
-// one exposed memory latency: first what needs the entries only (the row-start bits and, from a
-// ballot of them, how many rows start in the lanes below), then all dependent global loads at
-// once (the x gathers and the slice of the row list the chunk adds to), then the sums.
-// `ord` = ROW_FLAGs before the chunk (lean_rows[ord - 1] is the row that runs into it).
-template <int DT, typename Out>
-__device__ __forceinline__ void lean_chunk(const Device &d, Out out, const LeanRegs &r, const uint32_t *filter,
-                                           uint32_t filter_mask, int *s_rows, int ord, int lane) {
-    constexpr bool VAL = DT != DBSPMSPV_PATTERN;
+// First half of a chunk: what needs the entries only (the row-start bits and, from a ballot of them, how many rows start
+// in the lanes below), then all dependent global loads at once -- nothing here waits for them.
+__device__ __forceinline__ void lean_issue(const Device &d, LeanWork &q, const LeanEntries &r, int ord, const uint32_t *filter, uint32_t filter_mask, int lane) {
     constexpr int K = LEAN_PER_LANE;
     const uint32_t lt = (1u << lane) - 1u;
     const uint32_t idx[K] = {r.i0.x, r.i0.y, r.i0.z, r.i0.w, r.i1.x, r.i1.y, r.i1.z, r.i1.w};
-    const uint32_t wv[K] = {r.w0.x, r.w0.y, r.w0.z, r.w0.w, r.w1.x, r.w1.y, r.w1.z, r.w1.w};
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        // INLINE is class 0: any other entry (a block with a payload, the slack) is skipped here
+        bool go = idx[k] < (1u << TYPE_SHIFT) && DBS_CHK_INDEX(d, idx[k] & IDX_MASK, d.nb);
+        const uint32_t a = k < 4 ? r.a.x : r.a.y;
+        const uint32_t col = (idx[k] & IDX_MASK) * 16u + ((a >> (8 * (k & 3))) & 15u);
+        // (a set filter bit may belong to another column when the filter is folded: the gather
+        // then returns the "not listed" marker, as it would without the filter)
+        go = go && ((filter[(col >> 5) & filter_mask] >> (col & 31u)) & 1u);
+        // (through L1: on a power-law matrix a few hundred columns draw a third of all gathers, and with L2-only
+        // loads those lines saturate single L2 slices)
+        q.xin[k] = go ? __ldg(d.ws.x_dense + col) : __uint_as_float(X_ABSENT);
+    }
+    q.w0 = r.w0; q.w1 = r.w1;
     uint32_t hb = 0u;            // bit k: entry k starts a row
 #pragma unroll
     for (int k = 0; k < K; ++k) hb |= ((idx[k] >> 27) & 1u) << k;
@@ -130,35 +125,32 @@ __device__ __forceinline__ void lean_chunk(const Device &d, Out out, const LeanR
         excl = __popc(hm & lt);
         total = __popc(hm);
     }
-    // ---- dependent global loads: the rows this chunk adds to (lean_rows[ord - 1 .. ord + total - 1]:
-    // a lane fetches numbers l and 32 + l of them, they go to shared memory where any lane can
-    // look its rows up; a chunk of rows of one to three entries has more than 64 and reads the
-    // rest from the list directly), and the x entries
-    int rowp0 = 0, rowp1 = 0;
-    {
-        const int o = ord - 1 + lane;
-        if (lane <= total && o >= 0 && o < d.n_lean_rows) rowp0 = __ldg(d.lean_rows + o);
-        if (lane + 32 <= total && o + 32 < d.n_lean_rows) rowp1 = __ldg(d.lean_rows + o + 32);
-    }
+    // the rows this chunk adds to (lean_rows[ord - 1 .. ord + total - 1]: a lane fetches numbers l and 32 + l of
+    // them; a chunk of rows of one to three entries has more than 64 and reads the rest from the list directly)
+    const int o = ord - 1 + lane;
+    q.rowp0 = lane <= total && o >= 0 && o < d.n_lean_rows ? __ldg(d.lean_rows + o) : 0;
+    q.rowp1 = lane + 32 <= total && o + 32 < d.n_lean_rows ? __ldg(d.lean_rows + o + 32) : 0;
+    q.ord = ord;
+    q.meta = hb | (uint32_t)excl << 8 | (multi ? 1u << 17 : 0u);
+}
+
+// Second half: the sums.
+template <int DT, typename Out>
+__device__ __forceinline__ void lean_sums(const Device &d, Out out, const LeanWork &q, int *s_rows, int lane) {
+    constexpr bool VAL = DT != DBSPMSPV_PATTERN;
+    constexpr int K = LEAN_PER_LANE;
+    const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t wv[K] = {q.w0.x, q.w0.y, q.w0.z, q.w0.w, q.w1.x, q.w1.y, q.w1.z, q.w1.w};
+    const float (&xin)[K] = q.xin;
+    const uint32_t hb = q.meta & 0xFFu;
+    const int excl = (int)(q.meta >> 8) & 0x1FF, cnt = __popc(hb), ord = q.ord;
+    const bool multi = (q.meta >> 17) & 1u;
+    const uint32_t hm = __ballot_sync(FULL, hb != 0u);
     // row of the chunk's row start number k (k = 0: the row that runs into the chunk)
     auto row_of = [&](int k) { return k < LEAN_ROWS_CACHED ? s_rows[k] : d.lean_rows[ord - 1 + k]; };
-    float xin[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        // INLINE is class 0: any other entry (a block with a payload, the slack) is skipped here
-        bool go = idx[k] < (1u << TYPE_SHIFT) && DBS_CHK_INDEX(d, idx[k] & IDX_MASK, d.nb);
-        const uint32_t a = k < 4 ? r.a.x : r.a.y;
-        const uint32_t col = (idx[k] & IDX_MASK) * 16u + ((a >> (8 * (k & 3))) & 15u);
-#if DBS_LEAN_FILTER
-        // (a set filter bit may belong to another column when the filter is folded: the gather
-        // then returns the "not listed" marker, as it would without the filter)
-        go = go && ((filter[(col >> 5) & filter_mask] >> (col & 31u)) & 1u);
-#endif
-        xin[k] = go ? lean_gather(d.ws.x_dense + col) : __uint_as_float(X_ABSENT);
-    }
     __syncwarp();                // (the previous chunk's look-ups are over)
-    s_rows[lane] = rowp0;
-    s_rows[lane + 32] = rowp1;
+    s_rows[lane] = q.rowp0;
+    s_rows[lane + 32] = q.rowp1;
     __syncwarp();
     // ---- sums.  Thread-serial part: `lead` = sum of the lane's entries before its first row
     // start (they belong to the row that was open when the lane began), `seg` = sum from its last
@@ -245,15 +237,38 @@ k_pull_lean(Device d, Out out, float th3, int force_path, int popc_threshold, in
     pdl_wait();
     if (select_path(d, th3, force_path) != DBSPMSPV_PATH_PULL) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) d.ws.ctr->path = DBSPMSPV_PATH_PULL;
-    const int gwarp = blockIdx.x * LEAN_WARPS + warp;
+    const int gwarp = warp * gridDim.x + blockIdx.x;      // (neighbouring chunks on different SMs: the last, partial round of chunks is spread over all of them)
     const int nwarps = gridDim.x * LEAN_WARPS;
-    LeanRegs nxt = {};
+    LeanEntries nxt = {};
     int ord_next = 0;
     if (gwarp < d.n_lean_chunks) { nxt = lean_fetch<VAL>(d, gwarp, lane); ord_next = d.lean_chunk_ord[gwarp]; }
     // the filter: the vector-block masks are the presence bitmap of x (bit j of the array = column
     // j); folded by OR when x has more columns than the filter has bits
     {
         const int n_words = (d.nb + 1) / 2;
+        if (n_words <= filter_words && filter_words >= 4 * LEAN_CTA) {
+            // Every thread block reads the same words: four 16-byte loads in flight per thread, and the blocks start at different places.
+            // (One dependent word after the other, all blocks on the same L2 slice at a time, took 14 us of a kernel of 73.)
+            const int n16 = filter_words / 4;
+            for (int k0 = 0; k0 < n16; k0 += 4 * LEAN_CTA) {
+                uint4 v[4];
+                int at[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int k = k0 + u * LEAN_CTA + threadIdx.x;
+                    at[u] = k < n16 ? (int)((k + blockIdx.x * 64u) & (n16 - 1)) : -1;
+                    v[u] = make_uint4(0u, 0u, 0u, 0u);
+                    if (at[u] >= 0 && at[u] * 4 + 3 < n_words) v[u] = __ldcg(reinterpret_cast<const uint4 *>(d.ws.x_mask32) + at[u]);
+                    else if (at[u] >= 0 && at[u] * 4 < n_words) {
+                        v[u].x = d.ws.x_mask32[at[u] * 4];
+                        if (at[u] * 4 + 1 < n_words) v[u].y = d.ws.x_mask32[at[u] * 4 + 1];
+                        if (at[u] * 4 + 2 < n_words) v[u].z = d.ws.x_mask32[at[u] * 4 + 2];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) if (at[u] >= 0) reinterpret_cast<uint4 *>(filter)[at[u]] = v[u];
+            }
+        } else
         for (int f = threadIdx.x; f < filter_words; f += LEAN_CTA) {
             uint32_t v = 0u;
             for (int q = f; q < n_words; q += filter_words) v |= d.ws.x_mask32[q];
@@ -262,14 +277,10 @@ k_pull_lean(Device d, Out out, float th3, int force_path, int popc_threshold, in
     }
     __syncthreads();
     const uint32_t filter_mask = (uint32_t)filter_words - 1u;
-    for (int c = gwarp; c < d.n_lean_chunks; c += nwarps) {
-        const LeanRegs cur = nxt;
-        const int ord = ord_next;
-        if (c + nwarps < d.n_lean_chunks) { nxt = lean_fetch<VAL>(d, c + nwarps, lane); ord_next = d.lean_chunk_ord[c + nwarps]; }
-        lean_chunk<DT, Out>(d, out, cur, filter, filter_mask, ls->rows, ord, lane);
-    }
-    // entries with a payload: one block per warp at a time (they are the exception in these handles)
-    for (int q = gwarp; q < d.n_payload; q += nwarps) {
+    // Entries with a payload: one block per warp at a time (they are the exception in these handles).  Before the stream, with its first
+    // chunk in flight: a block is a chain of six dependent loads, which cost 11 us at the end of a kernel of 60 (5.5 K blocks, 16 M
+    // entries), where nothing else was left to run.  From the last warp on: the last ones have a chunk less in the stream.
+    for (int q = nwarps - 1 - gwarp; q < d.n_payload; q += nwarps) {
         const int pos = d.payload_pos[q];
         if (!DBS_CHK_INDEX(d, pos, d.n_entries)) continue;            // warp-uniform
         uint32_t idx = d.csr.idx[pos];
@@ -303,6 +314,31 @@ k_pull_lean(Device d, Out out, float th3, int force_path, int popc_threshold, in
             sum = warp_block<DT>(type, blk, nnz, xm, ls->sx, ls->stmp, lane, popc_threshold, hits);
         }
         if (lane < 16 && ((hits >> lane) & 1u)) out_add(out, (size_t)rb * 16 + lane, DT != DBSPMSPV_PATTERN ? sum : 1.0f);
+    }
+    // Without values the gathers of a chunk are issued before the sums of the chunk before it (79 us to 61 on 29 M entries, 30 % of x
+    // listed).  With values the registers for two chunks are not there (and 53 us in place of 45 on 16 M entries): the next
+    // chunk's entries fly during the sums, its gathers follow.
+    constexpr int AHEAD = VAL ? 0 : 1;
+    LeanWork cur = {};
+    auto fetch = [&](int c) { if (c < d.n_lean_chunks) { nxt = lean_fetch<VAL>(d, c, lane); ord_next = d.lean_chunk_ord[c]; } };
+    if (AHEAD && gwarp < d.n_lean_chunks) {
+        lean_issue(d, cur, nxt, ord_next, filter, filter_mask, lane);
+        fetch(gwarp + nwarps);
+    }
+    for (int c = gwarp; c < d.n_lean_chunks; c += nwarps) {
+        if (AHEAD) {
+            LeanWork ahead = {};
+            if (c + nwarps < d.n_lean_chunks) lean_issue(d, ahead, nxt, ord_next, filter, filter_mask, lane);
+            fetch(c + 2 * nwarps);
+            lean_sums<DT, Out>(d, out, cur, ls->rows, lane);
+            cur = ahead;
+        } else {
+            const LeanEntries now = nxt;
+            const int ord = ord_next;
+            fetch(c + nwarps);
+            lean_issue(d, cur, now, ord, filter, filter_mask, lane);
+            lean_sums<DT, Out>(d, out, cur, ls->rows, lane);
+        }
     }
 }
 

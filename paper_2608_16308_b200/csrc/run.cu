@@ -1653,6 +1653,7 @@ __global__ void __launch_bounds__(CMP_TPB, FOLD ? 5 : 8) k_finish(Device d, int3
             uint4 *acc4 = reinterpret_cast<uint4 *>(d.ws.y_acc + (size_t)bi * 8);
             const uint4 a = __ldcg(acc4), b = __ldcg(acc4 + 1);
             const uint32_t flags = mask8[bi];
+            const int path = FOLD ? ctr->path : 0;      // (a pull leaves the private accumulators alone)
             if (row_mask) keep = reinterpret_cast<const uint8_t *>(row_mask)[bi] ^ (complement ? 0xFFu : 0u);
             v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
             hits = flags;
@@ -1665,7 +1666,7 @@ __global__ void __launch_bounds__(CMP_TPB, FOLD ? 5 : 8) k_finish(Device d, int3
             if (flags) mask8[bi] = 0;
             if (FOLD) {
                 const int slot = d.hub_slot[bi >> 1];
-                if (slot != HUB_NONE && DBS_CHK_INDEX(d, slot, d.n_hub_blocks)) {
+                if (slot != HUB_NONE && path != DBSPMSPV_PATH_PULL && DBS_CHK_INDEX(d, slot, d.n_hub_blocks)) {
                     fold_hub_rows(d, slot, bi & 1, fold == 2, v);
 #pragma unroll
                     for (int r = 0; r < 8; ++r) hits |= (v[r] != ACC_CLEAR ? 1u : 0u) << r;
