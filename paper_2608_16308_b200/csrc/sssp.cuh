@@ -268,7 +268,7 @@ __device__ __forceinline__ int sssp_bound(float xmin, float w) {
 // stopped after SSSP_ROUNDS rounds is listed in chunks, which all warps share out behind a grid barrier (walked by the warp that met them, the
 // hub rows of an R-MAT graph, neighbours all, took one warp 300 us).  Handles of unit weights walk the row-run index.
 template <int DT>
-__device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist, uint32_t *next, int low, int32_t *n_long) {
+__device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist, const uint32_t *F, uint32_t *next, int low, int32_t *n_long) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int NONE = 0x7F800000;
     const int lane = threadIdx.x & 31;
@@ -343,17 +343,30 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
             }
         }
     }
-    // entries with a payload: one block per warp at a time
+    // entries with a payload: one block per warp at a time, columns of the frontier only (the blocks sit where a power-law graph is dense, among
+    // the vertices that settle first: late large steps skip most of them); the next entry is fetched meanwhile
+    struct Entry { uint32_t idx, w, aux; int rb; };
+    auto entry = [&](int pos) {
+        Entry e{0u, 0u, 0u, 0};
+        if (pos >= 0 && DBS_CHK_INDEX(d, pos, d.n_entries)) {
+            e = Entry{d.csr.idx[pos], d.csr.w[pos], d.csr.aux[pos], d.entry_row[pos]};
+            DBS_CHK_ENTRY(d, true, e.idx, e.w, e.aux);
+        }
+        return e;
+    };
+    auto position = [&](int q) { return q < d.n_payload ? d.payload_pos[q] : -1; };
+    Entry ahead = entry(position(gwarp));
+    int pos = position(gwarp + nwarps);
     for (int q = gwarp; q < d.n_payload; q += nwarps) {
-        const int pos = d.payload_pos[q];
-        if (!DBS_CHK_INDEX(d, pos, d.n_entries)) continue;            // warp-uniform
-        uint32_t idx = d.csr.idx[pos], w = d.csr.w[pos], aux = d.csr.aux[pos];
-        DBS_CHK_ENTRY(d, true, idx, w, aux);
-        const int type = (int)(idx >> TYPE_SHIFT), cb = (int)(idx & IDX_MASK), rb = d.entry_row[pos];
-        if (type == DBSPMSPV_BLK_INLINE || !DBS_CHK_INDEX(d, rb, d.mb)) continue;      // (only a replaced entry is INLINE here)
-        const uint32_t xm = (int64_t)cb * 16 + 16 <= d.n ? 0xFFFFu : (1u << (d.n - (int64_t)cb * 16)) - 1u;
-        block_rows_min_warp<DT>(type, w, aux, xm, dist + (size_t)cb * 16, d.payload, lane, [&](int r, uint32_t key) {
-            const int c = sssp_word(minplus_value(key)), row = rb * 16 + r;
+        const Entry e = ahead;
+        ahead = entry(pos);
+        pos = position(q + 2 * nwarps);
+        const int type = (int)(e.idx >> TYPE_SHIFT), cb = (int)(e.idx & IDX_MASK);
+        if (type == DBSPMSPV_BLK_INLINE || !DBS_CHK_INDEX(d, e.rb, d.mb)) continue;      // (only a replaced entry is INLINE here; warp-uniform)
+        const uint32_t xm = mask_of(F, cb);
+        if (!xm) continue;                                                               // warp-uniform
+        block_rows_min_warp<DT>(type, e.w, e.aux, xm, dist + (size_t)cb * 16, d.payload, lane, [&](int r, uint32_t key) {
+            const int c = sssp_word(minplus_value(key)), row = e.rb * 16 + r;
             if (c < __ldcg(s.word + row)) lower(row, c);
         });
     }
@@ -422,7 +435,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int
         if (tid == 0) s.ctr[3 + (t + 1) % 3] = 0;      // (its last reader was step t - 2)
         if (__ldcg(s.edges + t % 3) > pull_edges) {    // grid-uniform
             const int low = __ldcg(s.low + t % 3);
-            sssp_pull<DT>(d, s, dist, next, low, n_long);
+            sssp_pull<DT>(d, s, dist, F, next, low, n_long);
             grid.sync();
             const int n = __ldcg(n_long);
             if (n > 0) {                               // grid-uniform
