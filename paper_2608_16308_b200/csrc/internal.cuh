@@ -105,10 +105,7 @@ static_assert(PUSH_CHUNK == 32, "a push task is one warp step; its record stores
 // Direct push (push_direct.cuh): a column run longer than PD_LONG entries goes, in chunks of PD_CHUNK entries, to a
 // list that a second kernel walks, a warp per chunk; so does, in chunks of PD_PAYLOAD, the run of a listed column's payload entries.
 constexpr int PD_CTA = 256;
-#ifndef DBS_PD_LONG
-#define DBS_PD_LONG 128
-#endif
-constexpr int PD_LONG = DBS_PD_LONG;
+constexpr int PD_LONG = 128;
 constexpr int PD_CHUNK = 128;
 constexpr int PD_PAYLOAD = 8;
 // A run of the push worklist with at least HUB_MIN_ENTRIES entries (a hub column) is not cut

@@ -2323,7 +2323,7 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     for (int64_t made = 0;; start = 0) {
         int max_steps = (int)(d.n + 1 - made < SSSP_MAX_STEPS ? d.n + 1 - made : SSSP_MAX_STEPS);
         const bool can_pull = DT == DBSPMSPV_PATTERN ? d.rowrun_ptr != nullptr : d.weightrun != nullptr;
-        unsigned long long pull_edges = can_pull ? (unsigned long long)(DBS_SSSP_PULL_SHARE * (float)d.n_entries) : ~0ull;
+        unsigned long long pull_edges = can_pull ? (unsigned long long)(SSSP_PULL_SHARE * (float)d.n_entries) : ~0ull;
         void *args[] = {&dev, &s, &src, &dist, &start, &max_steps, &pull_edges};
         DBS_CUDA(cudaLaunchCooperativeKernel((void *)k_sssp<DT>, dim3(h->sm_count), dim3(SSSP_CTA), args, sizeof(SsspShared), st));
         ++h->kernel_launches;

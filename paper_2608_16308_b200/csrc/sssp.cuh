@@ -32,9 +32,7 @@ constexpr int SSSP_WORDS = SSSP_CTA / 8;          // frontier words of a thread 
 constexpr int SSSP_COLS = SSSP_CTA * 4;
 constexpr int SSSP_ILP = 4;                       // warp steps in flight
 // A step whose frontier reaches more than this share of the stored elements is pulled.
-#ifndef DBS_SSSP_PULL_SHARE
-#define DBS_SSSP_PULL_SHARE 0.05f
-#endif
+constexpr float SSSP_PULL_SHARE = 0.05f;
 constexpr int SSSP_ROUNDS = 8;                    // rounds of four elements that a lane walks of a row
 constexpr int SSSP_CHUNK = 512;                   // elements of a listed chunk of a longer row
 constexpr int SSSP_MAX_STEPS = 1024;              // steps of one launch, at most: a cycle of negative weight ends on the host

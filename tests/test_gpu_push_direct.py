@@ -1,0 +1,57 @@
+"""The direct push of hypersparse handles and the finishing kernel behind it: columns at the limit of a listed chunk, blocks with a
+payload, a hub row, tiles of the finishing kernel and groups of them, x taken from its list and from the masks."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2608_16308_b200 import binding as B
+from paper_2608_16308_b200 import workloads as wl
+from gpu_util import Handle, check_against_oracle, ref_matrix
+
+pytestmark = pytest.mark.gpu
+
+
+def matrix(m, n, seed):
+    """Columns of 127 .. 1025 elements, row 33 full, four full blocks, sparse noise; products down to 2^-122, zeros of both signs."""
+    bg = wl.random_sparse(m, n, 3 * m, seed)
+    rng = np.random.default_rng(seed)
+    rows, cols = [bg.rows(), np.full(n, 33)], [bg.col_idx, np.arange(n)]
+    for c, k in ((3, 127), (4, 128), (21, 129), (300, 257), (n - 1, 1025)):
+        rows.append(rng.choice(m, k, replace=False))
+        cols.append(np.full(k, c))
+    for rb, cb in ((0, 0), (m // 16 - 1, 0), (7, 1), (9, n // 16 - 1)):
+        r, c = np.mgrid[16 * rb:16 * rb + 16, 16 * cb:16 * cb + 16]
+        rows.append(r.ravel())
+        cols.append(c.ravel())
+    keys = wl.sorted_unique(np.concatenate(rows).astype(np.int64) * n + np.concatenate(cols))
+    ptr, idx = wl.csr_from_sorted_keys(m, n, keys)
+    val = rng.choice(np.float32([1.5, -0.75, 0.125, 3.0, 0.0, -0.0, 2.0 ** -60, -2.0 ** -62]), keys.size).astype(np.float32)
+    return wl.CSR(m, n, ptr, idx, val)
+
+
+@pytest.mark.parametrize("m", [2047, 2048, 2049, 33 * 2048 + 5])       # a tile of rows; more than a group of 32 tiles
+@pytest.mark.parametrize("dtype", [B.F32, B.BF16, B.PATTERN])
+def test_direct_push(m, dtype):
+    n = 40009
+    csr = matrix(m, n, 5)
+    h = Handle(csr, dtype)
+    assert h.stats.n_hub_row_blocks > 0
+    A = ref_matrix(csr, bf16=dtype == B.BF16)
+    P = oracle.RefMatrix(csr.m, csr.n, csr.row_ptr, csr.col_idx, None)
+    rng = np.random.default_rng(m)
+    always = np.int32([3, 4, 21, 300, n - 1])
+    lists = [always, np.arange(n // 8, dtype=np.int32)]                 # the list form; enough entries for a pull, too few blocks (masks)
+    lists += [np.unique(np.r_[always, rng.choice(n, k)]).astype(np.int32) for k in (40, 3000, 6000)]
+    for idx in lists:
+        x = wl.SparseVec(n, idx, rng.choice(np.float32([1.0, -2.0, 0.5, -0.0, 2.0 ** -60]), idx.size).astype(np.float32))
+        for semiring in (B.OR_AND, B.MIN_PLUS) if dtype == B.PATTERN else (B.PLUS_TIMES, B.OR_AND, B.MIN_PLUS):
+            h.set_opts(no_small_call=1)
+            got = h.run(x, semiring=semiring)
+            if semiring == B.MIN_PLUS:
+                wi, wv = oracle.ref_minplus(P if dtype == B.PATTERN else A, x.idx, x.val)
+                assert np.array_equal(got[0], wi) and np.array_equal(got[1], wv.astype(np.float32))
+            else:
+                check_against_oracle(got, oracle.ref_pull(P if dtype == B.PATTERN else A, x.idx, x.val), boolean=semiring == B.OR_AND)
+            assert h.get_stats().last_path == B.PATH_PUSH
+    h.close()
