@@ -2,7 +2,7 @@
 
 Workload at N=1: R-MAT scale 20, edge factor 16, fp32 values, with the input-sparsity sweep
 x nnz fraction 1e-5 ... 0.5.  One *step* is one pass of the whole hot path (vector blocking ->
-selector -> worklist -> block microkernels -> writeback -> compaction) over that batch: one
+selector -> block microkernels -> writeback -> sorted sparse y) over that batch: one
 dbspmspv_run call per sweep point, six calls.  L2 is flushed before every timed call, so the
 headline numbers are cold; an L2-warm pass is reported beside them.
 
@@ -119,8 +119,11 @@ class ByteModel:
     def moved(self, x_idx: np.ndarray, path: int, y_nnz: int, fmt: dict | None = None, one_kernel: bool = False) -> dict:
         """Bytes the implementation moves on `path`, each distinct byte once: the format part
         (above), x (the list, the dense copy written and gathered, the masks, the clean-up),
-        y (accumulator read-modify-write, hit flags, the sorted output) and the two O(m) scans
-        of the compaction passes (hit flags in, packed masks out and in).  one_kernel: the
+        y (accumulator read-modify-write, hit flags, the sorted output) and two O(m) scans
+        (hit flags in, packed masks out and in).  The x, y and scan terms are those of a push over a staged
+        x with hit flags and a two-pass compaction; they are kept so that figures compare across versions.  The
+        kernels of today move fewer bytes for x (a push takes it from its list) and more for y: the
+        finishing kernel reads the accumulator itself, 4 m bytes in place of 1.25 m.  one_kernel: the
         single-kernel form of a short call -- x is read once as a list, the row bitmap lives in
         shared memory (no scans), y is the accumulator read-modify-write, the row list written
         and read back, the gather-and-clear and the output."""
@@ -861,7 +864,7 @@ def decode_chain(B, torch, dev, flush):
 def decode_batch(B, torch, dev, flush):
     """Multi-vector decode (the paper's stated limitation, Section 6): 2, 4 and 8 activation
     vectors through the 12288x4096 bf16 layer in one dbspmspv_decode_batch call (one pass over
-    the payload, block products on the tensor cores), beside the same vectors as single calls
+    the columns that any of them reaches, products on the tensor cores), beside the same vectors as single calls
     and a dense bf16 GEMM of the same shape."""
     up = lambda arr: torch.from_numpy(np.ascontiguousarray(arr)).to(dev)
     m, n = wl.DECODE_SHAPES[0]
@@ -917,14 +920,17 @@ def decode_layers(B, torch, dev, flush, peak):
             call()
             torch.cuda.synchronize()
             stt = B.dbspmspv_get_stats(h)
-            streamed = stt.kernel_launches - before == 2       # zero kernel + streaming kernel; the selective form is one kernel
+            streamed = stt.kernel_launches - before == 2       # zero kernel + streaming kernel; the other forms are one kernel
+            columns = stt.segment_bytes >= 2 * m * n           # the handle keeps its weights by columns
             db = decode_bytes(wgt, wl.bf16_bits_to_f32(wl.f32_to_bf16_bits(x)))
             # streaming form: the whole payload, the view entries with a payload (9 bytes), the
             # chunk table (16 bytes per chunk, part of segment_bytes), x once per thread block
             # (from L2 after the first: counted once), y zeroed and added to (4 + 8 bytes per row)
-            db["B_moved"] = int(stt.payload_bytes + 9 * db["view_entries"] + stt.segment_bytes + 2 * n + 12 * m) if streamed else db["B_moved_selective"]
+            # columns: the active columns of the copy, absent weights included, x and y
+            db["B_moved"] = int(2 * np.count_nonzero(x) * m + 2 * n + 4 * m) if columns else \
+                int(stt.payload_bytes + 9 * db["view_entries"] + stt.segment_bytes + 2 * n + 12 * m) if streamed else db["B_moved_selective"]
             rec = {"workload": f"decode_{m}x{n}_bf16_prune50_act{int(zf * 100)}zero", "path": "push" if stt.last_path == B.PATH_PUSH else "pull",
-                   "form": "streaming" if streamed else "selective"}
+                   "form": "columns" if columns else "streaming" if streamed else "selective"}
             rec.update(st)
             rec.update({"us_l2_warm": round(warm, 2), "dense_bf16_gemv_us_same_box": round(gemv, 2),
                         "format_bytes": int(stt.payload_bytes + stt.csr_view_bytes), **db,

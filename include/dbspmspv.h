@@ -14,7 +14,8 @@
  *   - Every array argument is a DEVICE pointer owned by the caller unless stated otherwise.
  *   - `stream` is a cudaStream_t (passed as an opaque pointer; NULL = the legacy default
  *     stream).  dbspmspv_run / db_bfs / dbspmspv_decode only enqueue work on it: they allocate
- *     nothing, never synchronise, and return as soon as the kernels are queued.  Calls on the
+ *     no device memory, never synchronise, and return as soon as the kernels are queued (a handle keeps
+ *     the launch graphs of its last few kinds of call, at most eight, in host memory).  Calls on the
  *     same handle must be stream ordered (the handle owns one workspace).  A handle lives on
  *     the device that was current when it was created; run / db_bfs / decode return
  *     DBSPMSPV_ERR_INVALID_ARG when the calling thread's current device is another one.
@@ -124,11 +125,15 @@ typedef struct {
     float th3_decode;        /* dbspmspv_decode: same rule; the output is dense and every row block
                                 takes part, so pull wins much earlier (0.01, the paper's value) */
     int32_t no_fused_decode; /* dbspmspv_decode on handles whose elements sit mostly in blocks with
-                                a payload and whose x fits in shared memory has two one-kernel
-                                forms: a streaming one (the whole payload is moved through
+                                a payload and whose x fits in shared memory has one-kernel
+                                forms: bf16 handles of at least 1024 rows read their weights
+                                from a copy that lies by columns, active columns only; the
+                                others have a streaming one (the whole payload is moved through
                                 shared memory by bulk copies) and a selective one (only the
                                 block columns x reaches are fetched).
-                                0: streaming, or selective when the x of the handle's previous
+                                0: by columns where that copy exists (finite weights, copy
+                                   at most four times the payload, at most 25,600 columns),
+                                   else streaming, or selective when the x of the handle's previous
                                    decode call had fewer than 15 % nonzero elements (default);
                                 1: neither -- the blocking / traversal / cleanup kernels of
                                    dbspmspv_run;   2: selective only;   3: streaming only      */
@@ -141,8 +146,8 @@ typedef struct {
                                 pulled).  0 = block ratio only, the paper's rule.  Default
                                 0.08, measured (0.06 .. 0.1 are within 1 %)                */
     int32_t hub_min_nnz_x;   /* dbspmspv_run: shortest x list for which the push adds into the
-                                private accumulators of hub row blocks (they cost one more
-                                kernel in the chain); 0 = default (32768), < 0 = never     */
+                                private accumulators of hub row blocks (the finishing kernel
+                                folds them); 0 = default (4096), < 0 = never               */
     float decode_threshold;  /* dbspmspv_decode: activation magnitude cut fused into the vector
                                 blocking (Section 5.3: activation sparsity by magnitude
                                 thresholding) -- x_j takes part iff |x_j| > decode_threshold;
@@ -411,11 +416,12 @@ int dbspmspv_run_masked(dbspmspv_handle_t h, const int32_t *x_idx, const void *x
  * at x + b * ldx entries (the handle's value type; fp32 with run option decode_x_f32); y
  * receives `batch` dense fp32 vectors of m entries, vector b at y + b * ldy.  ldx >= n,
  * ldy >= m.  Every y vector equals what dbspmspv_decode gives for its x vector (up to the
- * order of the fp32 additions).  Where the handle has the streaming decode form, groups of up
- * to four vectors share one pass over the payload (the selector is not evaluated for them: the
+ * order of the fp32 additions).  Where the handle decodes by columns, groups of up to eight
+ * vectors share one pass over the columns that any of them reaches; where it has the streaming form, groups of
+ * up to four share one pass over the payload (the selector is not evaluated for them: the
  * payload is streamed whatever the vectors hold); otherwise the vectors are taken one by one.
  * The activation options (decode_threshold, decode_relu, decode_x_f32) apply to every vector.
- * Device pointers; allocates nothing; asynchronous on `stream`.  Pattern handles:
+ * Device pointers; allocates no device memory; asynchronous on `stream`.  Pattern handles:
  * DBSPMSPV_ERR_UNSUPPORTED.                                                                   */
 int dbspmspv_decode_batch(dbspmspv_handle_t h, const void *x, int64_t ldx, float *y, int64_t ldy, int32_t batch,
                           dbspmspv_stream_t stream);

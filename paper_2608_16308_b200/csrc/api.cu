@@ -207,7 +207,7 @@ int dbspmspv_destroy(dbspmspv_handle_t h) {
     cudaFree(const_cast<int4 *>(d.stage_chunks));
     cudaFree(const_cast<uint4 *>(d.cols));
     if (h->x_nnz_seen_host) cudaFreeHost(h->x_nnz_seen_host);
-    cudaFree(const_cast<uint16_t *>(d.hub_slot)); cudaFree(const_cast<int32_t *>(d.hub_rb)); cudaFree(d.hub_acc);
+    cudaFree(const_cast<uint16_t *>(d.hub_slot)); cudaFree(d.hub_acc);
     cudaFree(h->csc2csr); cudaFree(h->block_row);
     cudaFree(h->ws_arena);
     cudaFree(h->sssp_arena);

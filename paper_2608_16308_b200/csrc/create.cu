@@ -927,7 +927,7 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
 
     // Hub row blocks: the (at most HUB_BLOCKS_MAX) row blocks with the most view entries, if
     // they hold HUB_BLOCK_MIN_ENTRIES or more.  Chosen on the host from the row block pointers.
-    d.hub_slot = nullptr; d.hub_rb = nullptr; d.hub_acc = nullptr; d.n_hub_blocks = 0; d.hub_on = 0;
+    d.hub_slot = nullptr; d.hub_acc = nullptr; d.n_hub_blocks = 0; d.hub_on = 0;
     if (d.mb > 0 && n_entries >= HUB_BLOCK_MIN_ENTRIES) {
         std::vector<int32_t> ptr((size_t)d.mb + 1);
         DBS_CUDA(cudaMemcpyAsync(ptr.data(), d.csr.ptr, ((size_t)d.mb + 1) * 4, cudaMemcpyDeviceToHost, st));
@@ -945,16 +945,14 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         if (!big.empty()) {
             std::vector<uint16_t> slot((size_t)d.mb + 2, HUB_NONE);     // padded: read two at a time
             for (size_t k = 0; k < big.size(); ++k) slot[big[k]] = (uint16_t)k;
-            uint16_t *hs; float *ha; int32_t *hr;
-            DBS_KEEP(hr, big.size());
-            DBS_CUDA(cudaMemcpyAsync(hr, big.data(), big.size() * 4, cudaMemcpyHostToDevice, st));
+            uint16_t *hs; float *ha;
             const int64_t n_acc = (int64_t)HUB_COPIES * (int64_t)big.size() * 16;
             DBS_KEEP(hs, (int64_t)d.mb + 2); DBS_KEEP(ha, n_acc);
             DBS_CUDA(cudaMemcpyAsync(hs, slot.data(), ((size_t)d.mb + 2) * 2, cudaMemcpyHostToDevice, st));
             k_fill_words<<<grid_for(n_acc), TPB, 0, st>>>(reinterpret_cast<uint32_t *>(ha), n_acc, HUB_CLEAR);
             DBS_CUDA(cudaStreamSynchronize(st));
-            d.hub_slot = hs; d.hub_rb = hr; d.hub_acc = ha; d.n_hub_blocks = (int32_t)big.size();
-            h->hub_bytes = ((int64_t)d.mb + 2) * 2 + (int64_t)big.size() * 4 + n_acc * 4;
+            d.hub_slot = hs; d.hub_acc = ha; d.n_hub_blocks = (int32_t)big.size();
+            h->hub_bytes = ((int64_t)d.mb + 2) * 2 + n_acc * 4;
         }
     }
 

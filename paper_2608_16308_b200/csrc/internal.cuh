@@ -60,7 +60,7 @@ constexpr int TYPE_SHIFT = 29;
 constexpr uint32_t ROW_FLAG = 1u << 27;     // block-CSR view: first INLINE element of its row
 // Hub row blocks: the few row blocks that hold a large share of a power-law matrix.  Atomics on
 // one line are served one after the other by the L2 slice that owns it, so the push gives
-// every hub row block HUB_COPIES private accumulators (Device::hub_acc); the compaction folds them.
+// every hub row block HUB_COPIES private accumulators (Device::hub_acc); the finishing kernel folds them.
 constexpr uint32_t HUB_FLAG = 1u << 27;     // block-CSC view: INLINE element whose row block is a hub
 #ifndef DBS_HUB_COPIES
 #define DBS_HUB_COPIES 16
@@ -207,8 +207,8 @@ struct Workspace {
     uint2 *tasks;         // push worklist: (column block | (entries - 1) << 27, first CSC-view position)
     int4 *hubs;           // 3 x HUB_CAP hub runs (column block, first position, entries, -): see worklist.cuh
     float *y_acc;         // m (padded): dense accumulator, all ACC_CLEAR between calls
-    uint32_t *y_mask32;   // run: structural-hit bits, all zero between calls (flags of tiny products, then the
-                          // whole mask, written by the counting pass); BFS: next-frontier masks
+    uint32_t *y_mask32;   // run: bits of the rows that a tiny product reached (see acc_needs_flag), all zero between calls;
+                          // BFS: next-frontier masks
     int4 *long_runs;      // direct push: {first position, entries, x value, 0 or 256 + local column of payload entries} of the listed chunks
     int32_t *tile_status; // end of a call: result entries of every tile of rows, times two, plus the call's parity
     unsigned long long *tile_group;   // ... and per group of 32 tiles, by parity: tiles counted << 32 | their entries
@@ -276,12 +276,10 @@ struct Device {           // everything the kernels need, passed by value
     // Hub row blocks (null / 0 when the matrix has none): hub_slot[rb] = slot of row block rb or
     // HUB_NONE; hub_acc[(copy * n_hub_blocks + slot) * 16 + row] = private accumulators, all
     // HUB_CLEAR between calls.
-    // hub_rb[slot] = the row block; hub_on: how many copies this call's push uses (set per call by the host).
     const uint16_t *hub_slot;
-    const int32_t *hub_rb;
     float *hub_acc;
     int32_t n_hub_blocks;
-    int32_t hub_on;           // copies in use (0: none)
+    int32_t hub_on;           // copies this call's push uses (set per call by the host; 0: none)
     int32_t long_cap;         // direct push: chunks of all long runs and payload runs together (0: the matrix has none)
     const uint32_t *row_present32;  // per row block: rows that hold a stored element (two 16-bit masks per word)
     Workspace ws;

@@ -2,7 +2,7 @@
 // whose x_j is listed -- the product that GraphBLAS-style systems (Sections 1 and 6) iterate for
 // single-source shortest paths; db_sssp below is that iteration.
 //
-// It runs over the same format, vector blocking, push worklist and compaction as the (+, *)
+// It runs over the same format, vector blocking, push and finishing kernel as the (+, *)
 // product; only the traversal and the writeback differ.  The accumulator keeps, per row, a
 // 32-bit KEY of the smallest sum so far instead of a running sum:
 //     ordered(v) = bits(v) ^ (v < 0 ? 0xFFFFFFFF : 0x80000000)     (monotone in v)
@@ -12,7 +12,7 @@
 // int -- exactly the cleared state of the accumulator (ACC_CLEAR), which every word exceeds, so a
 // row was reached iff its word is no longer that.  The only
 // value whose key would be 0 is the NaN 0x7FFFFFFF; NaN has no place in a (min, +) product and
-// its key is stored as 1.  The compaction turns the words back into values.
+// its key is stored as 1.  The finishing kernel turns the words back into values.
 //
 // Traversal.  Push: hypersparse handles through the direct push (push_direct.cuh); handles whose elements sit
 // mostly in mask-based blocks (this file): a warp takes one task of the push worklist, 32 entries of the

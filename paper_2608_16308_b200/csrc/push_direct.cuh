@@ -26,7 +26,7 @@
 //
 // The semirings differ in the last line only: (+, *) adds the product, the Boolean one adds 1, (min, +) keeps
 // the larger key (minplus.cuh).  Products into hub row blocks go to one of HUB_COPIES private
-// accumulators, folded by the compaction (see Device::hub_acc).
+// accumulators, folded by the finishing kernel (see Device::hub_acc).
 #pragma once
 
 #include "internal.cuh"

@@ -1,8 +1,9 @@
-// One SpMSpV call (Sections 3.3 and 4.1): vector blocking + push worklist, device-side path
-// selection, push / pull traversal with per-block microkernels, hierarchical writeback, and
-// compaction of the dense accumulator into a sorted sparse y.  Also the dense-in / dense-out
-// decode entry (Section 4.3).  Nothing here allocates or synchronises, except db_sssp (a host
-// loop over (min, +) products, at the end of the file).
+// One SpMSpV call (Sections 3.3 and 4.1): vector blocking, device-side path selection, push / pull
+// traversal with per-block microkernels, hierarchical writeback, and one finishing kernel that turns
+// the dense accumulator into a sorted sparse y.  (Hypersparse handles push straight from the listed columns,
+// push_direct.cuh; the others through a worklist.)  Also the dense-in / dense-out
+// decode entry (Section 4.3).  Nothing here allocates device memory or synchronises, except db_sssp
+// (one launch, sssp.cuh, or a host loop over (min, +) products, at the end of the file).
 #include "internal.cuh"
 #include "call_graph.cuh"
 #include "microkernels.cuh"
@@ -49,7 +50,7 @@ namespace dbs {
 constexpr int CTA = 128;            // four warps per thread block (Section 3.3.2)
 constexpr int WARPS = CTA / 32;
 constexpr int XB_TPB = 512;         // vector blocking of a sparse x: threads per block
-constexpr int CMP_TPB = 256;        // compaction: threads per tile
+constexpr int CMP_TPB = 256;        // finishing kernel: threads per tile
 constexpr int TILE_WORDS = CMP_TPB / 4;  // a tile: 64 mask words = 2048 rows, 8 rows per thread
 
 // ------------------------------------------------------------------------------------------
@@ -190,10 +191,6 @@ __device__ __forceinline__ uint32_t lane_block(int type, uint32_t w, uint32_t au
         if (DT != DBSPMSPV_PATTERN && cur >= 0) emit(cur, s);
     }
     return hit;
-}
-
-__device__ __forceinline__ bool lane_owned(int type, uint32_t aux) {
-    return type == DBSPMSPV_BLK_INLINE || (type == DBSPMSPV_BLK_COO && aux < COO_SERIAL_MAX);
 }
 
 // The COO blocks held by the 32 lanes of a warp, processed as ONE flat list of stored entries:
@@ -1534,9 +1531,8 @@ k_decode_stream(Device d, const void *__restrict__ x, float *__restrict__ y, flo
 namespace dbs {
 
 // ------------------------------------------------------------------------------------------
-// Output compaction: the hit masks of the row blocks are scanned in order, so y comes out
-// sorted.  Pass 1 counts per tile, pass 2 places the entries, clears the accumulator and the
-// masks it read, clears the vector-block state of this call's x, and rolls the counters over.
+// The end of a call: the rows that were hit, in order, become y; the accumulator and the vector-block
+// state of this call's x are cleared, and the counters are rolled over.
 // ------------------------------------------------------------------------------------------
 
 // Fold of the private accumulators of eight rows of a hub row block into the accumulator proper, by the

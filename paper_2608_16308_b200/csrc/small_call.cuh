@@ -1,7 +1,7 @@
 // dbspmspv_run for a short x on a hypersparse handle, as ONE kernel of ONE thread-block cluster
 // (Section 4.1: vector-metadata construction fused with the SpMSpV kernel, no extra launch, no
-// host round trip).  The chain of the general path -- blocking, traversal, two compaction
-// passes -- costs four dependent launches, each with its own cold first loads, whatever x
+// host round trip).  The chain of the general path -- push, listed chunks, finishing
+// kernel -- costs up to three dependent launches, each with its own cold first loads, whatever x
 // holds; for up to a few hundred listed columns that chain IS the call (18 - 26 us for 10 .. 100
 // nonzeros on a matrix with a million rows; 14 - 22 us here).  Here nothing of x is staged at all:
 //   * a warp takes one listed column j (consecutive columns in different thread blocks): its
@@ -15,11 +15,11 @@
 //     shared memories (4 bytes per 32 rows, an eighth of the rows per thread block; remote bits
 //     are set through distributed shared memory) -- the structural-hit record, exact whatever
 //     the sums are;
-//   * after one cluster barrier the bitmap is the compaction's input: every thread block counts
+//   * after one cluster barrier the bitmap is the list of the result's rows: every thread block counts
 //     its slice, the eight totals are exchanged through distributed shared memory, the set bits
 //     become the result's row list (parked in the unused task array), and all threads of the
 //     cluster take result positions in turn: gather the sum, clear it, write y.
-// The dense copy of x, the vector-block masks, the row flags and the worklist are never
+// The dense copy of x, the vector-block masks and the worklist are never
 // written, so there is nothing to clean up.  Used when x is short, the selector is certain to
 // say push, the bitmap fits, and no option asks for the general path; results are identical
 // to the general path's up to the order of the fp32 additions.  The cluster barriers are the
@@ -122,7 +122,7 @@ k_run_small(Device d, const int32_t *__restrict__ x_idx, const void *__restrict_
     // ---- traversal: a warp per listed column (256 warps in the cluster); consecutive columns go
     // to different thread blocks.  (Several columns per warp were measured too: from about a
     // thousand columns on, the tails of the longer runs make the slowest warp take longer than
-    // the general path's whole chain of kernels, whose worklist spreads them over the GPU.)
+    // the general path's whole chain of kernels, which spreads them over the GPU.)
     constexpr int G = 32;
     static_assert(SMALL_MAX_NNZ_X * G <= SMALL_CLUSTER * SMALL_CTA, "every listed column has its own group of lanes");
     {
@@ -171,7 +171,7 @@ k_run_small(Device d, const int32_t *__restrict__ x_idx, const void *__restrict_
         if (n_hubs) cluster.sync();          // (cluster-uniform: every block read the same count)
     }
     STAMP();
-    // ---- compaction from the bitmap.  This block's slice; thread t owns the words [t * per, (t + 1) * per).
+    // ---- result from the bitmap.  This block's slice; thread t owns the words [t * per, (t + 1) * per).
     const int my_words = max(0, min(yper, ywords - rank * yper));
     const int per = (yper + SMALL_CTA - 1) / SMALL_CTA;
     const int w0 = min(tid * per, my_words), w1 = min(w0 + per, my_words);
