@@ -1606,6 +1606,42 @@ __device__ __forceinline__ int entries_before(const Device &d, int tile, int par
     return __all_sync(FULL, ok) ? sum : -1;
 }
 
+// The counters of the call, by the thread that knows the length of y.
+__device__ __forceinline__ void finish_counters(const Device &d, int total, int64_t y_capacity, int32_t *y_nnz) {
+    Counters *ctr = d.ws.ctr;
+    *y_nnz = total;
+    if (total > y_capacity) ctr->status = DBSPMSPV_ERR_CAPACITY;
+    ctr->last_y_nnz = total;
+    ctr->last_n_nzblk = ctr->n_nzblk;
+    ctr->last_n_tasks = ctr->n_tasks;
+    ctr->last_path = ctr->path;
+    ctr->n_nzblk = 0;
+    ctr->n_tasks = 0;
+    ctr->n_hubs = 0;
+    ctr->n_long = 0;
+}
+// Vector-block state of this call's x: clear the masks and put the "not listed" marker back -- entry by entry, or,
+// for an x that lists a good part of all columns, by streaming over the whole arrays (full-line stores instead of scattered
+// 4-byte ones).  `at`: the thread's number in the grid, `j0`: x_idx[at], fetched ahead (-1: none).
+__device__ __forceinline__ void finish_clear_x(const Device &d, const int32_t *__restrict__ x_idx, int32_t nnz_x, int clear, int at, int stride, int j0) {
+    if (clear & CLEAR_SWEEP) {
+        const int n_words = (d.nb + 1) / 2;
+        if (clear & CLEAR_DENSE) {
+            uint4 *xd4 = reinterpret_cast<uint4 *>(d.ws.x_dense);
+            for (int k = at; k < n_words * 8; k += stride) xd4[k] = make_uint4(X_ABSENT, X_ABSENT, X_ABSENT, X_ABSENT);
+        }
+        for (int k = at; k < n_words; k += stride) d.ws.x_mask32[k] = 0u;
+        return;
+    }
+    auto drop = [&](int j) {
+        if (j < 0 || j >= d.n) return;
+        d.ws.x_mask32[j >> 5] = 0u;
+        if (clear & CLEAR_DENSE) d.ws.x_dense[j] = __uint_as_float(X_ABSENT);
+    };
+    drop(j0);
+    for (int k = at + stride; k < nnz_x; k += stride) drop(x_idx[k]);
+}
+
 // The end of a call in one kernel: which rows were hit (see ACC_CLEAR), their order, y, and everything
 // put back.  A thread block takes a tile of 2048 rows, a thread eight of them in two 16-byte loads that
 // stay in registers; the tile publishes its count -- in a status word and, added up, in the word of its group of
@@ -1718,41 +1754,158 @@ __global__ void __launch_bounds__(CMP_TPB, FOLD ? 5 : 8) k_finish(Device d, int3
                 if (y_val) y_val[pos] = s_oval[k];
             }
         }
-        if (tile == n_tiles - 1 && threadIdx.x == 0) {
-            const int total = base + tile_total;
-            *y_nnz = total;
-            if (total > y_capacity) ctr->status = DBSPMSPV_ERR_CAPACITY;
-            ctr->last_y_nnz = total;
-            ctr->last_n_nzblk = ctr->n_nzblk;
-            ctr->last_n_tasks = ctr->n_tasks;
-            ctr->last_path = ctr->path;
-            ctr->n_nzblk = 0;
-            ctr->n_tasks = 0;
-            ctr->n_hubs = 0;
-            ctr->n_long = 0;
-        }
+        if (tile == n_tiles - 1 && threadIdx.x == 0) finish_counters(d, base + tile_total, y_capacity, y_nnz);
     }
     // the block with the last ticket: all tickets are taken
     if (tile == (int)gridDim.x - 1 && threadIdx.x == 0) ctr->finish_ticket = parity ? 0 : FINISH_PARITY;
-    // vector-block state of this call's x: clear the masks and put the "not listed" marker back
-    // -- entry by entry, or, for an x that lists a good part of all columns, by streaming over
-    // the whole arrays (full-line stores instead of scattered 4-byte ones)
-    if (clear & CLEAR_SWEEP) {
-        const int n_words = (d.nb + 1) / 2;
-        if (clear & CLEAR_DENSE) {
-            uint4 *xd4 = reinterpret_cast<uint4 *>(d.ws.x_dense);
-            for (int k = bi; k < n_words * 8; k += stride) xd4[k] = make_uint4(X_ABSENT, X_ABSENT, X_ABSENT, X_ABSENT);
+    finish_clear_x(d, x_idx, nnz_x, clear, bi, stride, j0);
+}
+
+// The same over FINISH_WIDE tiles at most per thread block, for accumulators of more tiles than fit on the GPU at once (in waves, each tile
+// with its ticket, loads, count and wait: 16 us on four million rows even for an empty result; 8 here).  First all tiles are
+// counted, their loads side by side; then the rows that hold results are fetched again, from L2, and written.  (Four million
+// rows, x = 1 %: 13.9 us, 16.6 in waves.  Lining up results per warp, or writing few of them straight to y, took 15.)
+constexpr int FINISH_WIDE = 4;
+template <bool FOLD>
+__global__ void __launch_bounds__(CMP_TPB, FOLD ? 4 : 8) k_finish_wide(Device d, int per_block, int32_t *__restrict__ y_idx, float *__restrict__ y_val,
+                                                    int64_t y_capacity, int32_t *__restrict__ y_nnz, int boolean,
+                                                    const int32_t *__restrict__ x_idx, int32_t nnz_x, int clear, int fold,
+                                                    const uint32_t *__restrict__ row_mask, int complement) {
+    __shared__ int s_cnt[FINISH_WIDE][CMP_TPB / 32], s_ticket, s_parity, s_base;
+    __shared__ int32_t s_oidx[CMP_TPB * 8];
+    __shared__ float s_oval[CMP_TPB * 8];
+    Counters *ctr = d.ws.ctr;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (nnz_x == 0) pdl_wait();
+    if (threadIdx.x == 0) { const int w = atomicAdd(&ctr->finish_ticket, 1); s_ticket = w & (FINISH_PARITY - 1); s_parity = w & FINISH_PARITY ? 1 : 0; }
+    __syncthreads();
+    const int unit = s_ticket, parity = s_parity, n_units = (d.ws.n_tiles + per_block - 1) / per_block;
+    const int stride = gridDim.x * CMP_TPB, at = unit * CMP_TPB + threadIdx.x;
+    const int j0 = (!(clear & CLEAR_SWEEP) && at < nnz_x) ? x_idx[at] : -1;
+    pdl_wait();
+    if (unit < n_units) {
+        const int n_bytes = (d.mb + 1) / 2 * 4;
+        uint8_t *mask8 = reinterpret_cast<uint8_t *>(d.ws.y_mask32);
+        const int first = unit * per_block * CMP_TPB + threadIdx.x;          // byte of the hit mask in the unit's first tile
+        const int path = FOLD ? ctr->path : 0;
+        uint32_t kept = 0u;                       // per tile: rows of this thread that go to y
+        uint32_t before[2] = {0u, 0u};            // per tile, 16 bits: such rows in the lanes up to this one
+        const uint4 untouched = make_uint4(ACC_CLEAR, ACC_CLEAR, ACC_CLEAR, ACC_CLEAR);
+#pragma unroll
+        for (int t0 = 0; t0 < FINISH_WIDE; t0 += 2) {
+            uint4 a[2], b[2];
+            uint32_t flags[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int bi = first + (t0 + u) * CMP_TPB;
+                a[u] = b[u] = untouched;
+                flags[u] = 0u;
+                if (t0 + u < per_block && bi < n_bytes) {
+                    const uint4 *acc4 = reinterpret_cast<const uint4 *>(d.ws.y_acc + (size_t)bi * 8);
+                    a[u] = __ldcg(acc4); b[u] = __ldcg(acc4 + 1);
+                    flags[u] = mask8[bi];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int t = t0 + u, bi = first + t * CMP_TPB;
+                const bool mine = t < per_block && bi < n_bytes;
+                uint4 *acc4 = reinterpret_cast<uint4 *>(d.ws.y_acc + (size_t)bi * 8);
+                uint32_t v[8] = {a[u].x, a[u].y, a[u].z, a[u].w, b[u].x, b[u].y, b[u].z, b[u].w};
+                uint32_t hits = flags[u];
+                bool folded = false;
+                if (FOLD && mine) {
+                    const int slot = d.hub_slot[bi >> 1];
+                    if (slot != HUB_NONE && path != DBSPMSPV_PATH_PULL && DBS_CHK_INDEX(d, slot, d.n_hub_blocks)) {
+                        fold_hub_rows(d, slot, bi & 1, fold == 2, v);
+                        folded = true;
+                    }
+                }
+                uint32_t differ = 0u;
+#pragma unroll
+                for (int r = 0; r < 8; ++r) differ |= v[r] ^ ACC_CLEAR;
+                if (differ) {                                              // (most rows of a wide accumulator are untouched)
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) hits |= (v[r] != ACC_CLEAR ? 1u : 0u) << r;
+                }
+                uint32_t bits = hits;
+                if (hits && row_mask) bits &= reinterpret_cast<const uint8_t *>(row_mask)[bi] ^ (complement ? 0xFFu : 0u);
+                if (flags[u]) mask8[bi] = 0;
+                if (bits && folded) { acc4[0] = make_uint4(v[0], v[1], v[2], v[3]); acc4[1] = make_uint4(v[4], v[5], v[6], v[7]); }      // (fetched again below)
+                else if (hits && !bits) { acc4[0] = untouched; acc4[1] = untouched; }
+                kept |= bits << (8 * t);
+                int incl = __popc(bits);
+                if (__any_sync(FULL, bits != 0u)) {
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int q = __shfl_up_sync(FULL, incl, o);
+                        if (lane >= o) incl += q;
+                    }
+                }
+                before[t >> 1] |= (uint32_t)incl << (16 * (t & 1));
+                if (lane == 31) s_cnt[t][warp] = incl;
+            }
         }
-        for (int k = bi; k < n_words; k += stride) d.ws.x_mask32[k] = 0u;
-        return;
+        __syncthreads();
+        int unit_total = 0;
+        for (int t = 0; t < per_block; ++t)
+            for (int k = 0; k < CMP_TPB / 32; ++k) unit_total += s_cnt[t][k];
+        // (every call rewrites every tile's word, read or not: the next call may take one tile per thread block)
+        if (threadIdx.x > 0 && threadIdx.x < per_block && unit + threadIdx.x * n_units < d.ws.n_tiles) d.ws.tile_status[unit + threadIdx.x * n_units] = parity;
+        if (threadIdx.x == 0) {
+            asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(d.ws.tile_status + unit), "r"(unit_total * 2 + parity) : "memory");
+            atomicAdd(d.ws.tile_group + parity * d.ws.n_tile_groups + unit / FINISH_GROUP, (1ull << 32) + (unsigned)unit_total);
+        }
+        if (unit == 0)
+            for (int k = threadIdx.x; k < d.ws.n_tile_groups; k += CMP_TPB) d.ws.tile_group[(parity ^ 1) * d.ws.n_tile_groups + k] = 0ull;
+        int base = 0;
+        if (unit_total > 0 || unit == n_units - 1) {                      // (an empty unit has nothing to place)
+            for (int t = 0; t < per_block; ++t) {
+                int local = 0, tile_total = 0;
+#pragma unroll
+                for (int k = 0; k < CMP_TPB / 32; ++k) {
+                    if (k < warp) local += s_cnt[t][k];
+                    tile_total += s_cnt[t][k];
+                }
+                if (tile_total == 0 && t > 0) continue;                    // block-uniform
+                const uint32_t bits = (kept >> (8 * t)) & 0xFFu;
+                if (bits) {
+                    const int bi = first + t * CMP_TPB;
+                    uint4 *acc4 = reinterpret_cast<uint4 *>(d.ws.y_acc + (size_t)bi * 8);
+                    const uint4 a = __ldcg(acc4), b = __ldcg(acc4 + 1);
+                    acc4[0] = untouched; acc4[1] = untouched;
+                    const uint32_t v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+                    int pos = local + (int)((before[t >> 1] >> (16 * (t & 1))) & 0xFFFFu) - __popc(bits);
+#pragma unroll
+                    for (int bit = 0; bit < 8; ++bit) {
+                        if ((bits >> bit) & 1u) {
+                            s_oidx[pos] = bi * 8 + bit;
+                            s_oval[pos] = boolean == 1 ? 1.0f : boolean == 2 ? minplus_of_word(v[bit]) : __uint_as_float(v[bit]) + 0.0f;
+                            ++pos;
+                        }
+                    }
+                }
+                if (t == 0 && warp == CMP_TPB / 32 - 1) {                  // (while the other tiles' counts arrive the first tile is gathered)
+                    const int sum = entries_before(d, unit, parity, lane);
+                    if (lane == 0) { s_base = sum; if (sum < 0) ctr->status = DBSPMSPV_ERR_TIMEOUT; }
+                }
+                __syncthreads();
+                if (t == 0) base = max(s_base, 0);
+                for (int k = threadIdx.x; k < tile_total; k += CMP_TPB) {
+                    const int64_t pos = (int64_t)base + k;
+                    if (pos < y_capacity) {
+                        y_idx[pos] = s_oidx[k];
+                        if (y_val) y_val[pos] = s_oval[k];
+                    }
+                }
+                base += tile_total;
+                __syncthreads();
+            }
+            if (unit == n_units - 1 && threadIdx.x == 0) finish_counters(d, base, y_capacity, y_nnz);
+        }
     }
-    auto drop = [&](int j) {
-        if (j < 0 || j >= d.n) return;
-        d.ws.x_mask32[j >> 5] = 0u;
-        if (clear & CLEAR_DENSE) d.ws.x_dense[j] = __uint_as_float(X_ABSENT);
-    };
-    drop(j0);
-    for (int k = bi + stride; k < nnz_x; k += stride) drop(x_idx[k]);
+    if (unit == (int)gridDim.x - 1 && threadIdx.x == 0) ctr->finish_ticket = parity ? 0 : FINISH_PARITY;
+    finish_clear_x(d, x_idx, nnz_x, clear, at, stride, j0);
 }
 
 __global__ void k_decode_cleanup(Device d) {
@@ -2011,8 +2164,18 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
     if (extra > 4 * h->sm_count) extra = 4 * h->sm_count;
     // scattered clears cost more than a full sweep once x lists a good part of the columns (a sweep of the masks alone is 32 times shorter)
     if ((int64_t)nnz_x * (clear & CLEAR_DENSE ? 8 : 128) > d.n) clear |= CLEAR_SWEEP;
-    calls.add(d.hub_on ? k_finish<true> : k_finish<false>, nt + extra, CMP_TPB, 0, calls.n > 0, d, y_idx, y_val, y_capacity, y_nnz, minplus ? 2 : (int)boolean, x_idx, nnz_x, clear,
-              d.hub_on ? (minplus ? 2 : 1) : 0, row_mask, complement);
+    // several tiles per thread block where they would come in waves (eight thread blocks per SM)
+    const int wave = 8 * h->sm_count;
+    int per_block = (nt + wave - 1) / wave;
+    if (per_block > FINISH_WIDE) per_block = FINISH_WIDE;
+    // (results in good part of the rows: fetching them twice costs more than the waves, 24 us against 19 with nearly all rows)
+    if ((int64_t)nnz_x * 64 > d.n) per_block = 1;
+    if (per_block > 1)
+        calls.add(d.hub_on ? k_finish_wide<true> : k_finish_wide<false>, (nt + per_block - 1) / per_block + extra, CMP_TPB, 0, calls.n > 0, d, per_block, y_idx, y_val, y_capacity, y_nnz,
+                  minplus ? 2 : (int)boolean, x_idx, nnz_x, clear, d.hub_on ? (minplus ? 2 : 1) : 0, row_mask, complement);
+    else
+        calls.add(d.hub_on ? k_finish<true> : k_finish<false>, nt + extra, CMP_TPB, 0, calls.n > 0, d, y_idx, y_val, y_capacity, y_nnz, minplus ? 2 : (int)boolean, x_idx, nnz_x, clear,
+                  d.hub_on ? (minplus ? 2 : 1) : 0, row_mask, complement);
     return submit_calls(h, calls, st);
 }
 

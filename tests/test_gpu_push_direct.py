@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 def matrix(m, n, seed):
     """Columns of 127 .. 1025 elements, row 33 full, four full blocks, sparse noise; products down to 2^-122, zeros of both signs."""
-    bg = wl.random_sparse(m, n, 3 * m, seed)
+    bg = wl.random_sparse(m, n, min(3 * m, 200000), seed)
     rng = np.random.default_rng(seed)
     rows, cols = [bg.rows(), np.full(n, 33)], [bg.col_idx, np.arange(n)]
     for c, k in ((3, 127), (4, 128), (21, 129), (300, 257), (n - 1, 1025)):
@@ -30,7 +30,8 @@ def matrix(m, n, seed):
     return wl.CSR(m, n, ptr, idx, val)
 
 
-@pytest.mark.parametrize("m", [2047, 2048, 2049, 33 * 2048 + 5])       # a tile of rows; more than a group of 32 tiles
+@pytest.mark.parametrize("m", [2047, 2048, 2049, 33 * 2048 + 5,            # a tile of rows; more than a group of 32 tiles
+                               2048 * 1185, 2048 * 2400 + 7])               # two and three tiles per thread block
 @pytest.mark.parametrize("dtype", [B.F32, B.BF16, B.PATTERN])
 def test_direct_push(m, dtype):
     n = 40009
