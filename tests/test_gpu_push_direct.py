@@ -56,3 +56,18 @@ def test_direct_push(m, dtype):
                 check_against_oracle(got, oracle.ref_pull(P if dtype == B.PATTERN else A, x.idx, x.val), boolean=semiring == B.OR_AND)
             assert h.get_stats().last_path == B.PATH_PUSH
     h.close()
+
+
+@pytest.mark.parametrize("dtype", [B.F32, B.PATTERN])
+def test_long_x_on_a_handle_rich_in_payload_goes_by_blocks(dtype):
+    csr = wl.stencil27(40, seed=3)
+    h = Handle(csr, dtype)
+    P = oracle.RefMatrix(csr.m, csr.n, csr.row_ptr, csr.col_idx, None)
+    for lo, hi in ((0, csr.n // 8), (17, csr.n // 2), (0, csr.n)):          # the last one pulls
+        idx = np.arange(lo, hi, dtype=np.int32)
+        x = wl.SparseVec(csr.n, idx, np.random.default_rng(hi).choice(np.float32([1.0, -2.0, 0.5, -0.0]), idx.size).astype(np.float32))
+        for semiring in ([B.OR_AND] if dtype == B.PATTERN else [B.PLUS_TIMES, B.OR_AND]):
+            want = oracle.ref_pull(P if dtype == B.PATTERN else ref_matrix(csr), x.idx, x.val)
+            check_against_oracle(h.run(x, semiring=semiring), want, boolean=semiring == B.OR_AND)
+            assert h.get_stats().last_path == (B.PATH_PULL if hi - lo == csr.n else B.PATH_PUSH)
+    h.close()
