@@ -534,7 +534,7 @@ def main() -> None:
     achieved = b_kernel_dom / (kernel_dom_ms * 1e-3) / 1e9
     dom_pull = info[kdom][0] == B.PATH_PULL
     dom_name = "k_pull_lean" if dom_pull else "k_compute"
-    traffic = ncu_traffic("k_pull_lean_rmat20_x50pct.txt" if dom_pull else "k_compute_push_rmat20_x10pct.txt")
+    traffic = ncu_traffic("k_pull_lean_rmat20_x50pct.txt" if dom_pull else "k_push_direct_rmat20_x10pct.txt")
     line = {"metric": METRIC, "value": round(value, 3), "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": round(ms_per_step, 5), "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
