@@ -533,7 +533,7 @@ def main() -> None:
     kernel_dom_ms = float(np.median(kernel_ms[:, kdom]))
     achieved = b_kernel_dom / (kernel_dom_ms * 1e-3) / 1e9
     dom_pull = info[kdom][0] == B.PATH_PULL
-    dom_name = "k_pull_lean" if dom_pull else "k_compute"
+    dom_name = "k_pull_lean" if dom_pull else "k_push_direct + k_push_long"
     traffic = ncu_traffic("k_pull_lean_rmat20_x50pct.txt" if dom_pull else "k_push_direct_rmat20_x10pct.txt")
     line = {"metric": METRIC, "value": round(value, 3), "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": round(ms_per_step, 5), "higher_is_better": True,
