@@ -360,7 +360,7 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
     // this block's piece; a non-finite entry: whole strips instead, element by element
     const int64_t work = (int64_t)strips * (odd ? 1 : n_steps);
     const int64_t lo = work * blockIdx.x / gridDim.x, hi = work * (blockIdx.x + 1) / gridDim.x;
-    if (lo >= hi) return;                                             // block-uniform
+    if (lo >= hi) { pdl_wait(); return; }                             // block-uniform; (no entry in any vector: nobody has a piece, and y is zeroed all the same before this kernel ends)
     if (!odd && !all) {
         int at = incl - cnt;
         for (int k = 0; k < warp; ++k) at += s_cnt[k];

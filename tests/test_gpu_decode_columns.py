@@ -70,3 +70,34 @@ def test_decode_over_columns(shape, prune, x_f32):
                     check(yh[b, :m], *refs[b][:2])
                 assert (yh[:, m:] == 55.0).all()
     h.close()
+
+
+def check_batches_in_a_row(m, n, launches):
+    """Batches without any active entry, with a non-finite one and ordinary ones, one behind the other on one stream into one y
+    that held NaN: every result is complete, whatever way the kernels of the call before it left."""
+    w = wl.pruned_weight(m, n, 0.5, seed=11, stream=m)
+    h = Handle(w, B.BF16)
+    A = ref_matrix(w, bf16=True)
+    nv = 8
+    kinds = {"zero": np.zeros((nv, n), np.float32), "plain": np.stack([wl.relu_activation(n, 0.7, seed=11, stream=b) for b in range(nv)])}
+    kinds["inf"] = kinds["plain"][::-1].copy()
+    kinds["inf"][5, w.col_idx[7]] = np.inf
+    refs = {k: [oracle.ref_decode(A, wl.bf16_bits_to_f32(wl.f32_to_bf16_bits(v[b])))[:2] for b in range(nv)] for k, v in kinds.items()}
+    dev = {k: bits(v) for k, v in kinds.items()}
+    y = torch.full((nv, m), float("nan"), device=DEV)
+    order = ["zero", "plain", "inf", "zero", "inf", "plain", "zero", "zero", "inf", "inf", "plain", "plain"] * 4
+    before, got = h.get_stats().kernel_launches, []
+    for k in order:
+        B.dbspmspv_decode_batch(h.h, dev[k], n, y, m, nv)
+        got.append((k, y.clone()))
+    torch.cuda.synchronize()
+    assert h.get_stats().kernel_launches - before == launches * len(order)
+    for k, t in got:
+        th = t.cpu().numpy()
+        for b in range(nv):
+            check(th[b], *refs[k][b])
+    h.close()
+
+
+def test_batches_in_a_row_over_columns():
+    check_batches_in_a_row(2400, 1040, 2)
