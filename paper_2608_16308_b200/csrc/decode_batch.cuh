@@ -414,6 +414,7 @@ k_decode_batch_mma(Device d, const void *__restrict__ x, int64_t ldx, float *__r
     if (fallback) {
         // (the copies in flight must have landed before the block ends)
         for (int k = 0; k < issued; ++k) mbar_wait_bounded(&s_bar[k], 0u);
+        pdl_wait();          // (the kernel behind adds into y and waits for this one only: y has to be zeroed before this one ends)
         return;
     }
     // y is zeroed by the kernel in front, which this one may overlap up to here
@@ -515,7 +516,8 @@ k_decode_batch_mma(Device d, const void *__restrict__ x, int64_t ldx, float *__r
 
 __global__ void k_zero_rows(float *y, int64_t ldy, int64_t m, int nvec) {
     pdl_wait();
-    // the one early start: the kernel behind blocks x meanwhile, which takes a thread block per SM and none of this kernel's room
+    // the one early start: the kernel behind blocks x meanwhile, which takes a thread block per SM and none of this kernel's room.
+    // (Every thread block of that kernel executes pdl_wait before it returns, whichever way it leaves: what follows it waits for it alone.)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int v = 0; v < nvec; ++v)

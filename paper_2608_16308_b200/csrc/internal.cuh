@@ -347,7 +347,8 @@ int decode_stage_bytes(const Device &d);
 // while its predecessor drains; `pdl_wait` blocks until the predecessor has completed and its
 // writes are visible (a no-op for a normally launched kernel).  Every kernel of a call begins with
 // it (or reads nothing that an earlier kernel of the stream may write before it).
-// No kernel lets its successor go early (griddepcontrol.launch_dependents): the successor's thread
+// One kernel lets its successor go early (griddepcontrol.launch_dependents): k_zero_rows in front of the batched decode kernels, each
+// block of which therefore executes pdl_wait on every way out.  No other one does: the successor's thread
 // blocks then sit on the SMs, waiting, in the place of its own later blocks and of the persistent
 // kernel behind them (stencil 160^3, x = 5 %: traversal 43 instead of 32 us, call 73 instead of 53; every other path 0 - 4 % slower).
 __device__ __forceinline__ unsigned long long global_timer_ns() {

@@ -101,3 +101,7 @@ def check_batches_in_a_row(m, n, launches):
 
 def test_batches_in_a_row_over_columns():
     check_batches_in_a_row(2400, 1040, 2)
+
+
+def test_batches_in_a_row_over_blocks():
+    check_batches_in_a_row(1008, 1040, 4)           # (too few rows for the column copy: tensor-core kernel and its two fallbacks)
