@@ -69,20 +69,26 @@ struct NextLevel {
     uint2 *tasks;
     bool emit;                   // the worklist is written by this level itself
 };
-// A push level of at most this many warp steps writes the next level's worklist itself, one phase and one grid barrier (with a pass of its
-// own behind a barrier of its own a level that moves next to nothing took 8.5 us, now 6).  A larger one reaches thousands of vertices: the
-// warps would queue for space in the list (with 256 steps the level took 13 us, and 100 K vertices 72 us in place of 65), and the level
-// behind it is a pull more often than not.
+// A push level of at most this many warp steps, behind which the next one is a push whatever it finds, writes the next level's worklist
+// itself, one phase and one grid barrier (with a pass of its own behind a barrier of its own a level that moves next to nothing took 8.5 us,
+// now 6).  A larger one reaches thousands of vertices: the warps would queue for space in the list (with 256 steps the level took 13 us, and
+// 100 K vertices 72 us in place of 65); and a list that a pull follows is written for nothing (17,000 vertices: a level that
+// reaches a fifth of the blocks from two of them 12.4 us with the list, 6.1 without).
 constexpr int BFS_EMIT_STEPS = 16;
+// Up to this many warp steps the bookkeeping is the claiming lanes': a second atomic per vertex found, but neither a pass nor a barrier
+// behind the level.  Larger levels leave it to a pass over the words that became nonzero, one update for up to 32 vertices: levels of 2^22
+// vertices that reach most of them through a few thousand hubs took 78 - 150 us with an atomic each, 59 - 116 with the pass.  (Limit 512:
+// levels of a few thousand steps 2 - 5 us longer; 4096 to 65536: no difference on graphs of 17,000 to 2^22 vertices.)
+constexpr int BFS_MARK_STEPS = 16384;
 
 // Boolean push: tasks of the active frontier blocks (a task is at most PUSH_CHUNK = 32 view
 // entries: one warp step); newly reached rows are claimed with one atomicOr per entry on the
 // next-frontier masks (the winner writes the level).  Like the pull, the loop is software-
 // pipelined: while task k is evaluated, the visited masks of k+1, the view entries of k+2 and
 // the task record of k+3 (in this warp's stride) are in flight.
-// The winner also does the level's bookkeeping for the vertex: it is marked visited, the word it turned nonzero
-// is listed, and (NextLevel::emit) the tasks of its column go to the next level's worklist.
-template <int DT>
+// The winner also lists the word it turned nonzero and, with MARK, does the level's bookkeeping for the vertex: it is marked visited
+// and, if asked for (NextLevel::emit), the tasks of its column go to the next level's worklist.
+template <int DT, bool MARK>
 __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, const uint2 *tasks, int n_recs, const int4 *hubs, int n_hubs,
                          int32_t *levels, int depth, const NextLevel &nx) {
     static_assert(PUSH_CHUNK == 32, "one warp step per task");
@@ -104,13 +110,15 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
         if (!__any_sync(FULL, fresh != 0u)) return;
         const bool newly = fresh && ((old >> sh) & 0xFFFFu) == 0;
         if (fresh) {
-            atomicOr(&d.ws.visited32[brow >> 1], fresh << sh);
             write_levels(levels, brow, fresh, depth);
-            found += __popc(fresh);
-            blocks += newly;
+            if (MARK) {
+                atomicOr(&d.ws.visited32[brow >> 1], fresh << sh);
+                found += __popc(fresh);
+                blocks += newly;
+            }
         }
         append_words(fresh && !old ? brow >> 1 : -1, nx.words, nx.n_words, lane);
-        if (!nx.emit) return;
+        if (!MARK || !nx.emit) return;
         // the vertices found, 32 at a time (blocks with a payload reach several rows at once): vertex k belongs to the last lane whose prefix is <= k
         int incl = __popc(fresh);
 #pragma unroll
@@ -203,7 +211,7 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
     }
     found = __reduce_add_sync(FULL, found);
     blocks = __reduce_add_sync(FULL, blocks);
-    if (lane == 0 && found) { atomicAdd(&d.ws.ctr->bfs_reached, found); atomicAdd(nx.n_blocks, blocks); }
+    if (MARK && lane == 0 && found) { atomicAdd(&d.ws.ctr->bfs_reached, found); atomicAdd(nx.n_blocks, blocks); }
 }
 
 // Boolean pull: one warp per row-block segment (a segment has at most MAX_SEG_ENTRIES = 4 x 32
@@ -517,7 +525,7 @@ __device__ __forceinline__ int bfs_path(int n_nzblk, int nb, float th3, int forc
     return ((float)n_nzblk / (float)nb < th3) ? DBSPMSPV_PATH_PUSH : DBSPMSPV_PATH_PULL;
 }
 
-// Worklist of the frontier F from the listed nonzero words of its masks (behind a pull level): a warp takes one word
+// Worklist of the frontier F from the listed nonzero words of its masks: a warp takes one word
 // (two vector blocks) at a time, lane = column; frontier columns emit their INLINE runs (adjacent
 // ones merged), lanes 0 and 16 the payload runs of the two blocks.  (With the words in index
 // order, the few warps that held the hub blocks of an early frontier wrote almost the whole
@@ -541,22 +549,16 @@ __device__ void bfs_worklist(const Device &d, const Scope &sc, const uint32_t *F
     }
 }
 
-// Path of the level whose counters are set `cur` (Section 3.3.1): push iff the ratio of nonempty
+// Path of a level (Section 3.3.1): push iff the ratio of nonempty
 // frontier blocks is below th3 -- and, the worklist of a push level being built by then, iff that
 // worklist is short: a frontier of a few hub vertices fills few vector blocks but owns a good
 // part of all stored elements, and a pull, which stops every row at its first frontier
 // neighbour, reads less than the push of all those elements would (edge_frac = the share of
-// the view's entries above which the push is given up; 0 = block ratio only).
-__device__ __forceinline__ int bfs_level_path(const Device &d, int cur, float th3, float edge_frac, int force_path) {
-    const Counters *ctr = d.ws.ctr;
-    int path = bfs_path(ctr->bfs_cnt[cur][0], d.nb, th3, force_path);
-    if (path == DBSPMSPV_PATH_PUSH && force_path == DBSPMSPV_PATH_AUTO && edge_frac > 0.f && d.rowrun_ptr != nullptr) {
-        // warp steps of the worklist: the task records plus the steps of the listed hub runs
-        const int n_hubs = min(ctr->bfs_hubs[cur], HUB_CAP);
-        int64_t steps = ctr->bfs_cnt[cur][1];
-        for (int k = 0; k < n_hubs; ++k) steps += (d.ws.hubs[cur * HUB_CAP + k].z + PUSH_CHUNK - 1) / PUSH_CHUNK;
-        if ((float)steps * (float)PUSH_CHUNK > edge_frac * (float)d.n_entries) path = DBSPMSPV_PATH_PULL;
-    }
+// the view's entries above which the push is given up; 0 = block ratio only).  `steps`: warp steps of the worklist.
+__device__ __forceinline__ int bfs_level_path(const Device &d, int n_nzblk, int steps, float th3, float edge_frac, int force_path) {
+    int path = bfs_path(n_nzblk, d.nb, th3, force_path);
+    if (path == DBSPMSPV_PATH_PUSH && force_path == DBSPMSPV_PATH_AUTO && edge_frac > 0.f && d.rowrun_ptr != nullptr &&
+        (float)steps * (float)PUSH_CHUNK > edge_frac * (float)d.n_entries) path = DBSPMSPV_PATH_PULL;
     return path;
 }
 
@@ -581,7 +583,10 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
     const int depth = lv + 1;
     const int n_nzblk = ctr->bfs_cnt[cur][0];
     const int n_tasks = ctr->bfs_cnt[cur][1];
-    const int path = bfs_level_path(d, cur, th3, edge_frac, force_path);
+    const int n_hubs = min(ctr->bfs_hubs[cur], HUB_CAP);
+    int steps = n_tasks;                                // of the worklist: the task records plus the steps of the listed hub runs
+    for (int k = 0; k < n_hubs; ++k) steps += (d.ws.hubs[cur * HUB_CAP + k].z + PUSH_CHUNK - 1) / PUSH_CHUNK;
+    const int path = bfs_level_path(d, n_nzblk, steps, th3, edge_frac, force_path);
     // counters that come into use at the next level are reset now: nobody reads or writes them
     // during this one (the previous level was their last reader, behind a barrier)
     if (sc.tid == 0) {
@@ -605,12 +610,30 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
         // Z (the frontier before this one) is cleared through its list
         const int nz_words = ctr->bfs_nwords[q_z];
         for (int i = sc.tid; i < nz_words; i += sc.nthreads) Z[words_z[i]] = 0u;
-        const int n_hubs = min(ctr->bfs_hubs[cur], HUB_CAP);
-        const NextLevel nx{N, words_out, &ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][0], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], hubs_next,
-                           lv & 1 ? d.ws.tasks : d.ws.tasks2, n_hubs == 0 && n_tasks <= BFS_EMIT_STEPS};
-        bfs_push<DT>(d, sc, F, lv & 1 ? d.ws.tasks2 : d.ws.tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
+        uint2 *const tasks = lv & 1 ? d.ws.tasks2 : d.ws.tasks, *const tasks_next = lv & 1 ? d.ws.tasks : d.ws.tasks2;
+        const bool mark = steps <= BFS_MARK_STEPS;
+        const bool emit = mark && n_hubs == 0 && n_tasks <= BFS_EMIT_STEPS && bfs_path(min(PUSH_CHUNK * n_tasks, d.nb), d.nb, th3, force_path) == DBSPMSPV_PATH_PUSH;
+        const NextLevel nx{N, words_out, &ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][0], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], hubs_next, tasks_next, emit};
+        if (mark) bfs_push<DT, true>(d, sc, F, tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
+        else bfs_push<DT, false>(d, sc, F, tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
         grid.sync();
-        if (nx.emit) return;                           // (the next level's worklist is there)
+        if (emit) return;                              // (the next level's worklist is there)
+        if (!mark) {
+            // visited is updated, the nonempty blocks and the vertices found are counted: over the words that became nonzero
+            const int n_listed = ctr->bfs_nwords[q_out];
+            int found = 0, nz = 0;
+            for (int i = sc.tid; i < n_listed; i += sc.nthreads) {
+                const int k = words_out[i];
+                const uint32_t nm = N[k];
+                d.ws.visited32[k] |= nm;
+                found += __popc(nm);
+                nz += ((nm & 0xFFFFu) != 0) + ((nm >> 16) != 0);
+            }
+            found = __reduce_add_sync(FULL, found);
+            nz = __reduce_add_sync(FULL, nz);
+            if (lane == 0 && found) { atomicAdd(&ctr->bfs_reached, found); atomicAdd(&ctr->bfs_cnt[nxt][0], nz); }
+            grid.sync();
+        }
     } else {
         // pull over the row-block segments (no row-run index): the masks produced are scanned as a
         // whole: visited is updated, the nonempty blocks counted, the nonzero words listed

@@ -157,3 +157,38 @@ def test_hub_column_goes_through_the_hub_list():
         for s in (5, 0, n - 1):
             assert np.array_equal(bfs(h, s), oracle.ref_bfs(A, s)), f"source {s}"
         h.close()
+
+
+@pytest.mark.parametrize("n", [700, 17000, 70001])
+@pytest.mark.parametrize("fan", [15 * 32, 16 * 32, 16 * 32 + 1, 17 * 32])
+def test_small_push_levels(n, fan):
+    """A level of 15 to 17 warp steps, with and without a successor that is surely a push: vertex 3 reaches `fan` vertices,
+    each of them one or two of the others."""
+    rng = np.random.default_rng(fan)
+    first = rng.permutation(np.arange(4, n))[:min(fan, n - 10)]
+    u = np.r_[np.full(first.size, 3), np.repeat(first, 2), [0]]
+    v = np.r_[first, rng.integers(4, n, 2 * first.size), [3]]
+    keys = wl.sorted_unique(v.astype(np.int64) * n + u)
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    g = wl.CSR(n, n, ptr, idx, None)
+    h, A = Handle(g, B.PATTERN), ref_matrix(g)
+    for path in PATHS:
+        h.set_opts(force_path=path)
+        for s in (0, 3, int(first[0])):
+            want = oracle.ref_bfs(A, s)
+            assert np.array_equal(bfs(h, s), want)
+            assert h.get_stats().bfs_reached == int((want >= 0).sum())
+    h.close()
+
+
+def test_push_levels_past_the_step_limit():
+    """Forced pushes whose largest level has more than 16384 warp steps (1.9 M entries), and the automatic search beside them."""
+    g = wl.rmat(16, 16, seed=12, values=False, symmetrise=True)
+    h, A = Handle(g, B.PATTERN), ref_matrix(g)
+    for path in (B.PATH_PUSH, B.PATH_AUTO):
+        h.set_opts(force_path=path)
+        for s in [int(np.argmax(np.diff(g.row_ptr)))] + [int(q) for q in wl.bfs_sources(g, 3, seed=2)]:
+            want = oracle.ref_bfs(A, s)
+            assert np.array_equal(bfs(h, s), want)
+            assert h.get_stats().bfs_reached == int((want >= 0).sum())
+    h.close()
