@@ -877,6 +877,7 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         unsigned long long heavy_nnz = 0;
         for (int c = DBSPMSPV_BLK_FCSR; c <= DBSPMSPV_BLK_DENSE; ++c) heavy_nnz += cls_h[DBSPMSPV_BLK_NCLASS + c];
         h->heavy_stage = heavy_nnz * 2 > (unsigned long long)nnzu;
+        h->payload_rich = !h->heavy_stage && (heavy_nnz + cls_h[DBSPMSPV_BLK_NCLASS + DBSPMSPV_BLK_COO]) * 8 > (unsigned long long)nnzu;
     }
     DBS_KEEP(d.csr.ptr, d.mb + 1); DBS_KEEP(d.csr.idx, n_entries + VIEW_PAD); DBS_KEEP(d.csr.w, n_entries + VIEW_PAD); DBS_KEEP(d.csr.aux, n_entries + VIEW_PAD);
     // the slack behind the last entry is read by whole-group staging copies: a class code that no

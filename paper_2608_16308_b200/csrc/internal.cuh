@@ -108,6 +108,12 @@ constexpr int PD_CTA = 256;
 constexpr int PD_LONG = 128;
 constexpr int PD_CHUNK = 128;
 constexpr int PD_PAYLOAD = 8;
+// Handles with more than an eighth (and less than half) of their elements in blocks with a payload list such a block's run once per four columns
+// instead of once per column when x is at least this long: with x in runs that is a quarter of the records (27-point operator on 150^3
+// cells, x = 5 % in runs of 64: 101 -> 57 us a call, 1 %: 33 -> 25), but a record walks two pairs of columns one after the other and x is staged, which
+// costs a scattered x 2 - 8 us and a short call of either kind 1 (90^3 cells: 1,400 entries 13.4 -> 14.7, 7,200 16.1 -> 15.4, 14,500 19.7 -> 16.6).
+// (R-MAT matrices of 8,192 rows and more are below the eighth; there both take the same time.)
+constexpr int PD_GROUPS_MIN_NNZ_X = 8192;
 // A run of the push worklist with at least HUB_MIN_ENTRIES entries (a hub column) is not cut
 // into tasks: it is listed once and every warp of the traversal strides over its 32-entry steps.
 constexpr int HUB_MIN_ENTRIES = 8192;
@@ -280,6 +286,7 @@ struct Device {           // everything the kernels need, passed by value
     float *hub_acc;
     int32_t n_hub_blocks;
     int32_t hub_on;           // copies this call's push uses (set per call by the host; 0: none)
+    int32_t payload_groups;   // direct push, per call: payload entries are listed once per four columns (payload_rows) instead of once per column
     int32_t long_cap;         // direct push: chunks of all long runs and payload runs together (0: the matrix has none)
     const uint32_t *row_present32;  // per row block: rows that hold a stored element (two 16-bit masks per word)
     Workspace ws;
@@ -313,6 +320,7 @@ struct dbspmspv_handle_s {
     int stream_grid;            // thread blocks of the streaming decode (0: not configured yet)
     int32_t *x_nnz_seen_host;   // host view of Device::x_nnz_seen (page-locked, mapped)
     bool heavy_stage;           // most stored elements sit in mask-based blocks: MODE 1 kernels
+    bool payload_rich;          // not most, but more than an eighth sit in blocks with a payload (see PD_GROUPS_MIN_NNZ_X)
     cudaEvent_t ev[2];          // optional timing of the traversal kernel (run_opts.timing)
     bool timed;
     int64_t kernel_launches;    // kernels this handle has launched (run / decode / bfs)

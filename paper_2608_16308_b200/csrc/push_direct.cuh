@@ -18,7 +18,8 @@
 //
 // A run longer than PD_LONG entries (a hub column of an R-MAT matrix has tens of thousands; left to one
 // thread block it was the whole kernel's time) is cut into chunks that go to a list instead, and so is the run of payload entries of a
-// listed column's block (rare on these handles, and a chain of four dependent loads each); a second kernel, launched
+// listed column's block, a chain of three or four dependent loads each: once per listed column, or, for a longer x on a handle with many of
+// them, once per group of four columns (Device::payload_groups), whose listed ones the second kernel takes from the finished masks; a second kernel, launched
 // only on handles that have such runs, deals the chunks out over the warps of the GPU.  Space in the list is claimed with one
 // atomic per thread block: an atomic per run was up to eight round trips in one thread, and atomics on one word take
 // 1.4 ns each.  (Taking chunks dynamically at the end of the first kernel, from a ticket
@@ -116,6 +117,100 @@ __device__ __forceinline__ void payload_elements(const Device &d, int first, int
     }
 }
 
+// The blocks with a payload behind the CSC-view entries first .. first + count - 1 (at most 2 U, all of one column block) against
+// the listed ones of four of its columns, 4 group .. 4 group + 3.  A half-warp takes an entry, lane = row, U of them side by side: entry, header
+// and (two columns at a time) values are one trip each for all rows and all entries; a lane's products end in one atomic.
+template <int DT, int MODE, int U>
+__device__ __forceinline__ void payload_rows(const Device &d, int first, int count, int group, int lane) {
+    constexpr bool VAL = DT != DBSPMSPV_PATTERN && MODE != 1;
+    const int row = lane & 15, c0 = 4 * (group & 3);
+    const uint32_t xm = (mask_of(d.ws.x_mask32, group >> 2) >> c0) & 15u;           // warp-uniform
+    const float4 x4 = MODE == 1 ? make_float4(1.f, 1.f, 1.f, 1.f) : *reinterpret_cast<const float4 *>(d.ws.x_dense + 4 * (size_t)group);
+    const float x[4] = {x4.x, x4.y, x4.z, x4.w};
+    uint32_t idx[U], w[U], off[U];               // off: place of the row's value of the four columns, a byte each (before: the entry's aux byte)
+    float acc[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int k = 2 * u + (lane >> 4), p = first + (k < count ? k : 0);
+        uint32_t aux = d.csc.aux[p];
+        idx[u] = d.csc.idx[p]; w[u] = d.csc.w[p];
+        DBS_CHK_ENTRY(d, false, idx[u], w[u], aux);
+        off[u] = aux;
+        if (k >= count) idx[u] = PAD_IDX;
+    }
+    uint32_t have = 0u;                          // bits 4 u + k: the row has an element in listed column k of entry u
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int type = (int)(idx[u] >> TYPE_SHIFT);
+        acc[u] = MODE == 2 ? __uint_as_float(ACC_CLEAR) : 0.f;
+        if (type <= DBSPMSPV_BLK_COO || type > BLK_CSR_ROWMAJOR) continue;
+        const uint8_t *blk = d.payload + (size_t)w[u] * 4;
+        const uint16_t *masks = reinterpret_cast<const uint16_t *>(blk);
+        uint32_t in = 0u, o = 0u;
+        if (is_row_major(type)) {
+            const uint32_t m = masks[row], s = VAL ? blk[32 + row] : 0u;
+            in = (m >> c0) & 15u;
+            o = s + __popc(m & ((1u << c0) - 1u));
+            o = (o & 0xFFu) | (o + (in & 1u)) << 8 | (o + __popc(in & 3u)) << 16 | (o + __popc(in & 7u)) << 24;
+        } else {
+            const uint2 m2 = *reinterpret_cast<const uint2 *>(masks + c0);
+            const uint32_t m[4] = {m2.x & 0xFFFFu, m2.x >> 16, m2.y & 0xFFFFu, m2.y >> 16};
+            const uint32_t s = VAL && type != DBSPMSPV_BLK_DENSE ? *reinterpret_cast<const uint32_t *>(blk + 32 + c0) : 0u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                in |= ((m[k] >> row) & 1u) << k;
+                const uint32_t at = type == DBSPMSPV_BLK_DENSE ? (uint32_t)((c0 + k) * 16 + row) : ((s >> (8 * k)) & 0xFFu) + __popc(m[k] & ((1u << row) - 1u));
+                o |= (at & 0xFFu) << (8 * k);
+            }
+        }
+        off[u] = o;
+        have |= (in & xm) << (4 * u);
+        w[u] += (type == DBSPMSPV_BLK_DENSE ? 32 : HDR_BYTES) / 4;
+    }
+#pragma unroll
+    for (int k0 = 0; k0 < 4; k0 += 2) {
+        if (!((xm >> k0) & 3u)) continue;        // warp-uniform
+        float a[U][2];
+        if (VAL)
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    a[u][k] = 0.f;
+                    if ((have >> (4 * u + k0 + k)) & 1u) a[u][k] = Val<DT>::load(d.payload + (size_t)w[u] * 4, (off[u] >> (8 * (k0 + k))) & 0xFFu);
+                }
+        if (MODE != 1)
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                    if ((have >> (4 * u + k0 + k)) & 1u) {
+                        if (MODE == 2) acc[u] = __int_as_float(max(__float_as_int(acc[u]), minplus_word((VAL ? a[u][k] : 1.0f) + x[k0 + k])));
+                        else acc[u] += a[u][k] * x[k0 + k];
+                    }
+    }
+    auto put = [&](size_t r, float v) {
+        if (MODE == 2) { atomicMax(reinterpret_cast<int *>(d.ws.y_acc) + r, __float_as_int(v)); return; }
+        atomicAdd(d.ws.y_acc + r, MODE == 1 ? 1.0f : v);
+        if (MODE == 0 && acc_needs_flag(v)) atomicOr(&d.ws.y_mask32[r >> 5], 1u << (r & 31));
+    };
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const size_t r0 = (size_t)(idx[u] & IDX_MASK) * 16;
+        if ((have >> (4 * u)) & 15u) put(r0 + row, acc[u]);
+        if ((int)(idx[u] >> TYPE_SHIFT) != DBSPMSPV_BLK_COO) continue;
+        // packed coordinate lists (only with forced formats): the half-warp's lanes share the elements out
+        const uint8_t *blk = d.payload + (size_t)w[u] * 4;
+        const int nnz = (int)off[u] + 1;
+        for (int k = row; k < nnz; k += 16) {
+            const int c = (blk[k] & 15) - c0;
+            if (c < 0 || c > 3 || !((xm >> c) & 1u)) continue;
+            const float v = VAL ? Val<DT>::load(blk + ((nnz + 3) & ~3), k) : 1.0f, xv = c == 0 ? x[0] : c == 1 ? x[1] : c == 2 ? x[2] : x[3];
+            put(r0 + (blk[k] >> 4), MODE == 2 ? __int_as_float(minplus_word(v + xv)) : v * xv);
+        }
+    }
+}
+
 template <int DT, int MODE, bool MASKS>
 __global__ void __launch_bounds__(PD_CTA, pd_per_sm(MASKS))
 k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restrict__ x_val, int32_t nnz_x, int validate, float th3,
@@ -133,7 +228,7 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
     Counters *ctr = d.ws.ctr;
     if (blockIdx.x == 0 && tid == 0) ctr->path = DBSPMSPV_PATH_PUSH;
     for (int round = 0; round < rounds; ++round) {
-        int first[PER], deg[PER], pfirst = 0, pdeg = 0, col0 = 0;
+        int first[PER], deg[PER], pfirst = 0, pdeg = 0, col0 = 0;     // INLINE runs of the thread's columns (the first one is col0); payload run of their block
         float xv[PER];
         uint32_t listed = 0;                           // bit k: column col0 + k is listed
         bool newly = false;
@@ -145,8 +240,7 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
             if (wi < n_words) listed = (d.ws.x_mask32[wi] >> (4 * (tid & 7))) & 15u;
             if (listed) {
                 const int j0 = (int)wi * 32 + 4 * (tid & 7);
-                col0 = j0 & 15;
-                const int32_t *cp = d.csc.colptr + 17 * (j0 >> 4) + col0;
+                const int32_t *cp = d.csc.colptr + 17 * (j0 >> 4) + (j0 & 15);
                 int c[5];
 #pragma unroll
                 for (int k = 0; k < 5; ++k) c[k] = cp[k];
@@ -155,7 +249,7 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
 #pragma unroll
                 for (int k = 0; k < PER; ++k)
                     if ((listed >> k) & 1u) { first[k] = c[k]; deg[k] = c[k + 1] - c[k]; xv[k] = vv[k]; if (!DBS_CHK_RANGE(d, first[k], deg[k])) deg[k] = 0; }
-                if (d.n_payload) payload_run(d, j0 >> 4, pfirst, pdeg);
+                if (d.n_payload) { payload_run(d, j0 >> 4, pfirst, pdeg); col0 = j0; }
             }
         } else {
             const int g = tid >> 3;
@@ -174,11 +268,14 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
                     const int sh = ((j >> 4) & 1) * 16;
                     const uint32_t old = atomicOr(&d.ws.x_mask32[j >> 5], 1u << (j & 31));
                     newly = ((old >> sh) & 0xFFFFu) == 0;
-                    col0 = j & 15;
+                    col0 = j;
                     listed = 1u;
                     if ((old >> (j & 31)) & 1u) {         // listed before: contributes once
                         deg[0] = 0; pdeg = 0; listed = 0u;
                         if (validate) ctr->status = DBSPMSPV_ERR_INVALID_ARG;
+                    } else if (d.payload_groups) {
+                        if ((old >> (j & 28)) & 15u) pdeg = 0;               // (listed by the thread that came to these four columns first)
+                        if (MODE != 1) d.ws.x_dense[j] = xv[0];              // (k_push_long takes x from there)
                     }
                 }
             }
@@ -189,7 +286,7 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
 #pragma unroll
             for (int k = 0; k < PER; ++k)
                 if (deg[k] > PD_LONG) { n_rec += (deg[k] + PD_CHUNK - 1) / PD_CHUNK; deg[k] = -deg[k]; }      // (negative: listed)
-            if (pdeg > 0) n_rec += __popc(listed) * ((pdeg + PD_PAYLOAD - 1) / PD_PAYLOAD);
+            if (pdeg > 0) n_rec += (d.payload_groups ? 1 : __popc(listed)) * ((pdeg + PD_PAYLOAD - 1) / PD_PAYLOAD);
         }
         // lay the nonempty short runs end to end
         int n_cols = 0, n_elems = 0;
@@ -239,11 +336,13 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
                     for (int q = lane; q < n_chunks; q += 32) d.ws.long_runs[o + q] = make_int4(f + q * PD_CHUNK, min(PD_CHUNK, n - q * PD_CHUNK), xb, 0);
                     if (lane == src) at += n_chunks;
                 }
-            if (pdeg > 0)
+            if (pdeg > 0 && d.payload_groups)
+                for (int q = 0; q < pdeg; q += PD_PAYLOAD) d.ws.long_runs[at++] = make_int4(pfirst + q, min(PD_PAYLOAD, pdeg - q), col0 >> 2, 0x100);
+            else if (pdeg > 0)
 #pragma unroll
                 for (int k = 0; k < PER; ++k)
                     if ((listed >> k) & 1u)
-                        for (int q = 0; q < pdeg; q += PD_PAYLOAD) d.ws.long_runs[at++] = make_int4(pfirst + q, min(PD_PAYLOAD, pdeg - q), __float_as_int(xv[k]), 0x100 | (col0 + k));
+                        for (int q = 0; q < pdeg; q += PD_PAYLOAD) d.ws.long_runs[at++] = make_int4(pfirst + q, min(PD_PAYLOAD, pdeg - q), __float_as_int(xv[k]), 0x100 | ((col0 + k) & 15));
         }
         for (int s0 = warp * 32; s0 < tot_e; s0 += PD_CTA * PD_ILP) {
             uint32_t idx[PD_ILP], w[PD_ILP], aux[PD_ILP];
@@ -273,7 +372,7 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
 
 // The listed chunks, a warp at a time; the next chunk's record is fetched a round ahead.
 // (Nothing is listed when the path decided on the device is the pull.)
-template <int DT, int MODE>
+template <int DT, int MODE, bool GROUPS>
 __global__ void __launch_bounds__(PD_CTA, 6) k_push_long(Device d) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN && MODE != 1;
     constexpr int U = PD_CHUNK / 32;
@@ -287,7 +386,11 @@ __global__ void __launch_bounds__(PD_CTA, 6) k_push_long(Device d) {
         if (i + nwarps < n) next = d.ws.long_runs[i + nwarps];
         if (!DBS_CHK_RANGE(d, run.x, run.y)) continue;
         const float xs = __int_as_float(run.z);
-        if (run.w) {                                   // payload entries: a half-warp each
+        if (GROUPS && run.w) {                         // payload entries, four columns (warp-uniform)
+            if (DBS_CHK_INDEX(d, run.z, 4 * (int64_t)d.nb)) payload_rows<DT, MODE, PD_PAYLOAD / 2>(d, run.x, run.y, run.z, lane);
+            continue;
+        }
+        if (!GROUPS && run.w) {                        // payload entries, one column: a half-warp each
             bool in[PD_PAYLOAD / 2];
             float a[PD_PAYLOAD / 2];
             uint32_t rb[PD_PAYLOAD / 2];

@@ -2111,23 +2111,14 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
         const bool may_pull = (!minplus || DT != DBSPMSPV_PATTERN) && pull_possible(h, nnz_x, h->ropts.th3);
         const bool may_push = !may_pull || fp != DBSPMSPV_PATH_PULL;
         const int mode = boolean ? 1 : minplus ? 2 : 0;
-        // Where a good part of the elements sits in blocks with a payload, a long x (the path is decided on the device) is pushed
-        // block by block through the worklist: its runs list most columns of a vector block, and the direct push visits
-        // a block's payload once per column (27-point operator on 40^3 cells, x = 40 %: 42 us a call, 27 by blocks).
-        int64_t in_payload = 0;
-        for (int c = 0; c < 6; ++c) if (c != DBSPMSPV_BLK_INLINE) in_payload += h->stats.class_nnz[c];
-        const bool by_blocks = may_pull && may_push && !minplus && in_payload * 8 > h->nnz;
+        h->d.payload_groups = h->payload_rich && nnz_x >= PD_GROUPS_MIN_NNZ_X;
         // private accumulators for the hub row blocks, when x is long enough for their atomics to queue up
         const int hub_min = h->ropts.hub_min_nnz_x ? h->ropts.hub_min_nnz_x : HUB_MIN_NNZ_X;
-        h->d.hub_on = may_push && !by_blocks && d.n_hub_blocks > 0 && hub_min > 0 && nnz_x >= hub_min ? (nnz_x < HUB_ALL_NNZ_X ? 4 : HUB_COPIES) : 0;
-        if (by_blocks && nnz_x > 0) calls.add(k_xblock_sparse<DT, true>, (nnz_x + XB_TPB - 1) / XB_TPB, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
-        else if (may_pull && nnz_x > 0) calls.add(k_xblock_sparse<DT, false>, (nnz_x + XB_TPB - 1) / XB_TPB, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
+        h->d.hub_on = may_push && d.n_hub_blocks > 0 && hub_min > 0 && nnz_x >= hub_min ? (nnz_x < HUB_ALL_NNZ_X ? 4 : HUB_COPIES) : 0;
+        if (may_pull && nnz_x > 0) calls.add(k_xblock_sparse<DT, false>, (nnz_x + XB_TPB - 1) / XB_TPB, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
         if (h->ropts.timing) calls.ev_before = calls.n;
-        if (any && by_blocks) {
-            const int s = launch_compute<DT, OutSparse, 1>(h, calls, OutSparse{d.ws.y_acc, d.ws.y_mask32}, h->ropts.th3, 1);
-            if (s != DBSPMSPV_OK) return s;
-        } else if (nnz_x > 0 && may_push) {
-            auto push = [&](auto list_kernel, auto mask_kernel, auto long_kernel) {
+        if (nnz_x > 0 && may_push) {
+            auto push = [&](auto list_kernel, auto mask_kernel, auto long_kernel, auto groups_kernel) {
                 if (may_pull) {
                     // (decided on the device) 32 mask words per thread block and round
                     const int n_words = (d.nb + 1) / 2;
@@ -2146,13 +2137,13 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
                     if (g > most) g = most;
                     calls.add(list_kernel, g, PD_CTA, 0, false, d, x_idx, xv, nnz_x, (int)h->ropts.validate, h->ropts.th3, fp, cols, (nnz_x + cols * g - 1) / (cols * g));
                 }
-                if (d.long_cap) calls.add(long_kernel, 6 * h->sm_count, PD_CTA, 0, true, d);
+                if (d.long_cap) calls.add(d.payload_groups ? groups_kernel : long_kernel, 6 * h->sm_count, PD_CTA, 0, true, d);
             };
-            if (mode == 1) push(k_push_direct<DT, 1, false>, k_push_direct<DT, 1, true>, k_push_long<DT, 1>);
-            else if (mode == 2) push(k_push_direct<DT, 2, false>, k_push_direct<DT, 2, true>, k_push_long<DT, 2>);
+            if (mode == 1) push(k_push_direct<DT, 1, false>, k_push_direct<DT, 1, true>, k_push_long<DT, 1, false>, k_push_long<DT, 1, true>);
+            else if (mode == 2) push(k_push_direct<DT, 2, false>, k_push_direct<DT, 2, true>, k_push_long<DT, 2, false>, k_push_long<DT, 2, true>);
             else if (DT != DBSPMSPV_PATTERN) {
                 constexpr int VT = DT == DBSPMSPV_PATTERN ? DBSPMSPV_F32 : DT;       // (pattern handles have no (+, *))
-                push(k_push_direct<VT, 0, false>, k_push_direct<VT, 0, true>, k_push_long<VT, 0>);
+                push(k_push_direct<VT, 0, false>, k_push_direct<VT, 0, true>, k_push_long<VT, 0, false>, k_push_long<VT, 0, true>);
             };
         }
         if (any && may_pull) {
@@ -2160,7 +2151,7 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
                                   : launch_lean<DT, OutSparse>(h, calls, OutSparse{d.ws.y_acc, d.ws.y_mask32}, h->ropts.th3);
             if (s != DBSPMSPV_OK) return s;
         }
-        if (!may_pull) clear = CLEAR_MASKS;
+        if (!may_pull && (mode == 1 || !d.payload_groups)) clear = CLEAR_MASKS;      // (x was staged for the payload entries only)
     } else {
         if (nnz_x > 0) calls.add(k_xblock_sparse<DT, true>, (nnz_x + XB_TPB - 1) / XB_TPB, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
         if (h->ropts.timing) calls.ev_before = calls.n;

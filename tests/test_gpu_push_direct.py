@@ -71,3 +71,63 @@ def test_long_x_on_a_handle_rich_in_payload_goes_by_blocks(dtype):
             check_against_oracle(h.run(x, semiring=semiring), want, boolean=semiring == B.OR_AND)
             assert h.get_stats().last_path == (B.PATH_PULL if hi - lo == csr.n else B.PATH_PUSH)
     h.close()
+
+
+def blocks_and_noise(n, seed):
+    """A quarter of the elements in blocks with a payload -- dense, a few full rows, a few full columns, scattered -- of 32 to 256
+    elements each, the rest single."""
+    rng = np.random.default_rng(seed)
+    bg = wl.random_sparse(n, n, 4 * n, seed)
+    rows, cols = [bg.rows()], [bg.col_idx]
+    for k in range(2200):
+        rb, cb = rng.integers(0, n // 16, 2)
+        full = np.zeros((16, 16), bool)
+        if k % 4 == 0:
+            full[:] = rng.random((16, 16)) < 0.9
+        elif k % 4 == 1:
+            full[rng.choice(16, 3, replace=False)] = True
+        elif k % 4 == 2:
+            full[:, rng.choice(16, 3, replace=False)] = True
+        else:
+            full[:] = rng.random((16, 16)) < 0.3
+        r, c = np.nonzero(full)
+        rows.append(16 * rb + r)
+        cols.append(16 * cb + c)
+    keys = wl.sorted_unique(np.concatenate(rows).astype(np.int64) * n + np.concatenate(cols))
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    return wl.CSR(n, n, ptr, idx, rng.choice(np.float32([1.5, -0.75, 0.125, 3.0, 0.0, -0.0, 2.0 ** -60, -2.0 ** -62]), keys.size).astype(np.float32))
+
+
+@pytest.mark.parametrize("dtype", [B.F32, B.BF16, B.PATTERN])
+@pytest.mark.parametrize("fmt", [B.FORMAT_AUTO, B.FORMAT_COO])
+def test_payload_runs_once_per_four_columns(dtype, fmt):
+    """x one entry short of, at and past the length from which payload runs are listed per four columns, from its list and from the
+    masks, clustered and scattered, some entries twice; then a short x, to show that the staged x was cleared."""
+    n = 160021
+    csr = blocks_and_noise(n, 8)
+    o = B.default_create_opts()
+    o.force_format = fmt
+    h = Handle(csr, dtype, opts=o)
+    share = 1 - h.stats.class_nnz[B.BLK_INLINE] / h.stats.nnz
+    assert 1 / 8 < share and (share < 1 / 2 or fmt == B.FORMAT_COO)          # (packed lists do not count towards the other half)
+    A = ref_matrix(csr, bf16=dtype == B.BF16)
+    P = oracle.RefMatrix(csr.m, csr.n, csr.row_ptr, csr.col_idx, None)
+    rng = np.random.default_rng(1)
+    runs = (np.arange(0, 24000, 3)[:, None] * 16 // 3 + np.arange(11)).ravel()            # 11 columns of every 16
+    lists = [np.sort(rng.choice(n, k, replace=False)) for k in (8186, 8187)]               # 8191 and 8192 with the five twice
+    lists += [runs[:9000], np.r_[runs[20000:29000], n - 1], runs[:40000], np.array([5, 700, n - 1])]
+    for idx in lists:
+        idx = idx.astype(np.int32)
+        val = rng.choice(np.float32([1.0, -2.0, 0.5, -0.0, 2.0 ** -60]), idx.size).astype(np.float32)
+        twice = rng.integers(0, idx.size, 5)                                             # (the same value: it contributes once)
+        x = wl.SparseVec(n, idx, val)
+        given = wl.SparseVec(n, np.r_[idx, idx[twice]], np.r_[val, val[twice]]) if idx.size > 256 else x
+        for semiring in (B.OR_AND, B.MIN_PLUS) if dtype == B.PATTERN else (B.PLUS_TIMES, B.OR_AND, B.MIN_PLUS):
+            got = h.run(given, semiring=semiring)
+            if semiring == B.MIN_PLUS:
+                wi, wv = oracle.ref_minplus(P if dtype == B.PATTERN else A, x.idx, x.val)
+                assert np.array_equal(got[0], wi) and np.array_equal(got[1], wv.astype(np.float32))
+            else:
+                check_against_oracle(got, oracle.ref_pull(P if dtype == B.PATTERN else A, x.idx, x.val), boolean=semiring == B.OR_AND)
+            assert h.get_stats().last_path == B.PATH_PUSH
+    h.close()
