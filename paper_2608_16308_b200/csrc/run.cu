@@ -1988,8 +1988,11 @@ static int launch_lean(dbspmspv_handle_s *h, CallList &calls, Out out, float th3
     while (filter_words < n_words && filter_words < LEAN_FILTER_MAX_WORDS) filter_words <<= 1;
     const size_t smem = (size_t)filter_words * 4 + LEAN_WARPS * sizeof(LeanScratch);
     if (!configured) {
+        // (the attribute belongs to the kernel, not to the handle: the largest size, or a handle with few columns would lower it
+        // below what one with many, configured before, asks for)
+        constexpr int most = LEAN_FILTER_MAX_WORDS * 4 + LEAN_WARPS * (int)sizeof(LeanScratch);
         auto kernel = k_pull_lean<DT, Out>;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return DBSPMSPV_ERR_CUDA;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess) return DBSPMSPV_ERR_CUDA;
         configured = true;
     }
     calls.add(k_pull_lean<DT, Out>, h->sm_count, LEAN_CTA, smem, true, h->d, out, th3, h->ropts.force_path, h->ropts.popc_threshold, filter_words);
