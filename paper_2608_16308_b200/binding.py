@@ -161,14 +161,24 @@ def _raise(status: int, where: str) -> None:
     raise DbSpmspvError(status, where)
 
 
+def _plain(o):
+    """What stands behind a ctypes instance or an object with `_as_parameter_`."""
+    while hasattr(o, "_as_parameter_"):
+        o = o._as_parameter_
+    return o.value if isinstance(o, ctypes._SimpleCData) else o
+
+
 def _load_fast() -> None:
-    """First call of a hot entry point: hands its address in the loaded library to the extension,
-    with torch's raw getters of the current device and stream."""
+    """First call of a hot entry point: hands its address in the loaded library to the extension."""
+    L = lib()
+    _fastcall.setup(tuple(ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _FAST), _raise, _bind_streams)
+
+
+def _bind_streams() -> None:
+    """First call without a stream: torch's raw getters of the current device and stream."""
     import torch
     torch.cuda.init()
-    L = lib()
-    _fastcall.setup(tuple(ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _FAST), _raise,
-                    torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+    _fastcall.streams(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
 
 
 # The hot entry points.  Arguments as in the header, tensors (or numpy arrays) for the pointers,
@@ -189,7 +199,7 @@ def _not_built(*_args, **_kwargs):
 
 
 if _fastcall is not None:
-    _fastcall.set_loader(_load_fast)
+    _fastcall.set_loader(_load_fast, _plain)
 dbspmspv_run, dbspmspv_run_masked, dbspmspv_decode, dbspmspv_decode_batch, db_bfs, db_sssp = (
     getattr(_fastcall, name, _not_built) for name in _FAST)
 

@@ -7,7 +7,8 @@
  * getters used here), the rest argument conversion.
  *
  * The extension links neither the library nor torch: binding.py hands it the addresses of the
- * entry points (whichever build of the library was loaded) and the stream getters on first use. */
+ * entry points (whichever build of the library was loaded) on first use, and the stream getters when
+ * the first call without a stream argument asks for them: a call that names its stream needs no torch. */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
@@ -16,7 +17,9 @@ enum { F_RUN, F_RUN_MASKED, F_DECODE, F_DECODE_BATCH, F_BFS, F_SSSP, N_FUNCS };
 
 static void *g_addr[N_FUNCS];
 static PyObject *g_load;          /* called once: loads the library and calls setup() */
+static PyObject *g_plain;         /* (object) -> what stands behind a ctypes instance or an object with _as_parameter_ */
 static PyObject *g_raise;         /* (status, name) -> raises DbSpmspvError */
+static PyObject *g_bind_streams;  /* called once, by the first call without a stream argument: calls streams() */
 static PyObject *g_get_device;    /* () -> int */
 static PyObject *g_get_stream;    /* (device) -> int, the raw current stream */
 static PyObject *s_data_ptr, *s_ctypes, *s_data;
@@ -49,33 +52,50 @@ static int as_pointer(PyObject *o, void **out) {
     return !(*out == NULL && PyErr_Occurred());
 }
 
+/* an argument as a Python integer (or None): as a ctypes prototype, it takes a ctypes instance or an object with _as_parameter_ too */
+static PyObject *plain(PyObject *o) {
+    if (PyLong_Check(o) || o == Py_None) { Py_INCREF(o); return o; }
+    return PyObject_CallOneArg(g_plain, o);
+}
+
 /* a handle or a stream: an integer, or None for NULL */
 static int as_opaque(PyObject *o, void **out) {
-    if (o == Py_None) { *out = NULL; return 1; }
-    *out = PyLong_AsVoidPtr(o);
-    return !(*out == NULL && PyErr_Occurred());
-}
-
-static int as_i64(PyObject *o, int64_t *out) {
-    PyObject *v = PyNumber_Index(o);
+    PyObject *v = plain(o);
     if (!v) return 0;
-    *out = PyLong_AsLongLong(v);
-    Py_DECREF(v);
-    return !(*out == -1 && PyErr_Occurred());
-}
-
-/* (an integer that does not fit 32 bits keeps its low bits, as it does through ctypes) */
-static int as_i32(PyObject *o, int32_t *out) {
-    PyObject *v = PyNumber_Index(o);
-    if (!v) return 0;
-    *out = (int32_t)PyLong_AsUnsignedLongLongMask(v);
+    *out = NULL;
+    if (v != Py_None) {
+        if (!PyLong_Check(v)) PyErr_Format(PyExc_TypeError, "an integer or None is wanted, not %.80s", Py_TYPE(v)->tp_name);
+        else *out = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(v);
+    }
     Py_DECREF(v);
     return !PyErr_Occurred();
+}
+
+/* (an integer that does not fit keeps its low bits, as it does through ctypes) */
+static int as_i64(PyObject *o, int64_t *out) {
+    PyObject *p = plain(o), *v = p ? PyNumber_Index(p) : NULL;
+    Py_XDECREF(p);
+    if (!v) return 0;
+    *out = (int64_t)PyLong_AsUnsignedLongLongMask(v);
+    Py_DECREF(v);
+    return !PyErr_Occurred();
+}
+static int as_i32(PyObject *o, int32_t *out) {
+    int64_t v = 0;
+    if (!as_i64(o, &v)) return 0;
+    *out = (int32_t)v;
+    return 1;
 }
 
 /* the stream argument: None (or absent) is torch's current stream on the current device */
 static int as_stream(PyObject *o, void **out) {
     if (o && o != Py_None) return as_opaque(o, out);
+    if (!g_get_stream) {
+        PyObject *r = PyObject_CallNoArgs(g_bind_streams);
+        if (!r) return 0;
+        Py_DECREF(r);
+        if (!g_get_stream) { PyErr_SetString(PyExc_RuntimeError, "the stream getters have not been set"); return 0; }
+    }
     PyObject *dev = PyObject_CallNoArgs(g_get_device);
     if (!dev) return 0;
     PyObject *s = PyObject_CallOneArg(g_get_stream, dev);
@@ -210,24 +230,35 @@ static PyObject *f_sssp(PyObject *self, PyObject *const *args, Py_ssize_t nargs,
     return PyLong_FromLong(steps);
 }
 
-static PyObject *f_set_loader(PyObject *self, PyObject *load) {
-    Py_INCREF(load);
-    Py_XSETREF(g_load, load);
+/* set_loader(load, plain) */
+static PyObject *f_set_loader(PyObject *self, PyObject *args) {
+    PyObject *load, *pl;
+    if (!PyArg_ParseTuple(args, "OO", &load, &pl)) return NULL;
+    Py_INCREF(load); Py_XSETREF(g_load, load);
+    Py_INCREF(pl); Py_XSETREF(g_plain, pl);
     Py_RETURN_NONE;
 }
 
-/* setup(addresses, raise, get_device, get_stream) */
+/* setup(addresses, raise, bind_streams) */
 static PyObject *f_setup(PyObject *self, PyObject *args) {
-    PyObject *addr, *rs, *gd, *gs;
-    if (!PyArg_ParseTuple(args, "O!OOO", &PyTuple_Type, &addr, &rs, &gd, &gs)) return NULL;
+    PyObject *addr, *rs, *bs;
+    if (!PyArg_ParseTuple(args, "O!OO", &PyTuple_Type, &addr, &rs, &bs)) return NULL;
     if (PyTuple_GET_SIZE(addr) != N_FUNCS) { PyErr_SetString(PyExc_ValueError, "wrong number of addresses"); return NULL; }
     void *p[N_FUNCS];
     for (int i = 0; i < N_FUNCS; ++i)
         if (!as_opaque(PyTuple_GET_ITEM(addr, i), &p[i])) return NULL;
     Py_INCREF(rs); Py_XSETREF(g_raise, rs);
+    Py_INCREF(bs); Py_XSETREF(g_bind_streams, bs);
+    for (int i = 0; i < N_FUNCS; ++i) g_addr[i] = p[i];
+    Py_RETURN_NONE;
+}
+
+/* streams(get_device, get_stream) */
+static PyObject *f_streams(PyObject *self, PyObject *args) {
+    PyObject *gd, *gs;
+    if (!PyArg_ParseTuple(args, "OO", &gd, &gs)) return NULL;
     Py_INCREF(gd); Py_XSETREF(g_get_device, gd);
     Py_INCREF(gs); Py_XSETREF(g_get_stream, gs);
-    for (int i = 0; i < N_FUNCS; ++i) g_addr[i] = p[i];
     Py_RETURN_NONE;
 }
 
@@ -235,7 +266,7 @@ static PyObject *f_setup(PyObject *self, PyObject *args) {
 static PyMethodDef methods[] = {
     FAST("dbspmspv_run", f_run), FAST("dbspmspv_run_masked", f_run_masked), FAST("dbspmspv_decode", f_decode),
     FAST("dbspmspv_decode_batch", f_decode_batch), FAST("db_bfs", f_bfs), FAST("db_sssp", f_sssp),
-    {"set_loader", f_set_loader, METH_O, NULL}, {"setup", f_setup, METH_VARARGS, NULL}, {NULL, NULL, 0, NULL}};
+    {"set_loader", f_set_loader, METH_VARARGS, NULL}, {"setup", f_setup, METH_VARARGS, NULL}, {"streams", f_streams, METH_VARARGS, NULL}, {NULL, NULL, 0, NULL}};
 
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_fastcall", NULL, -1, methods, NULL, NULL, NULL, NULL};
 
