@@ -252,10 +252,12 @@ __device__ __forceinline__ void sssp_four(const Device &d, int k0, uint32_t (&co
         for (int j = 0; j < 4; ++j) { col[j] = (v[j] & IDX_MASK) * 16u + (v[j] >> 27); w[j] = 1.0f; }
     }
 }
-// No element behind one of weight w can do better than this (the order goes by the upper bits).
+// No element behind one of weight w can do better than this (the order goes by the upper bits).  The lower bits of an infinite or NaN weight
+// must not be cut off: below -infinity in the order of words there are only NaNs, and the bound of a NaN would end the row.
 template <bool VAL>
 __device__ __forceinline__ int sssp_bound(float xmin, float w) {
-    return sssp_word(xmin + (VAL ? sssp_value(sssp_word(w) & ~((1 << (32 - SSSP_WEIGHT_BITS)) - 1)) : w));
+    constexpr int least = (int)0x807FFFFFu;        // sssp_word(-infinity)
+    return sssp_word(xmin + (VAL ? sssp_value(max(sssp_word(w) & ~((1 << (32 - SSSP_WEIGHT_BITS)) - 1), least)) : w));
 }
 
 // A large step pulled.  Every row walks its own elements, which lie by weight (Device::weightrun), and stops at the first that

@@ -43,3 +43,36 @@ def test_sssp_one_launch(n, dtype, no_index):
             assert np.array_equal(dist.cpu().numpy().astype(np.float64), oracle.ref_sssp(A, src))
         assert steps[0] == steps[1]
     h.close()
+
+
+@pytest.mark.parametrize("low", [-np.inf, -3.4e38, np.inf])
+def test_rows_that_begin_with_extreme_weights(low):
+    """Rows of a pulled step whose first elements, of the lowest (or highest) weights there are, lead to vertices that were never
+    reached: the search goes on to the finite ones behind them."""
+    n = 4000
+    rng = np.random.default_rng(2)
+    mid = np.arange(1, 1501)
+    rows = [mid, rng.integers(1501, 3000, 4 * mid.size), np.repeat(np.arange(1501, 1601), 12), [3500]]
+    cols = [np.zeros(mid.size, np.int64), np.repeat(mid, 4), np.tile(np.arange(3001, 3013), 100), [1550]]
+    kind = np.r_[np.zeros(mid.size), np.zeros(4 * mid.size), np.ones(1200), [0]]
+    key = np.concatenate(rows).astype(np.int64) * n + np.concatenate(cols)
+    keys, at = np.unique(key, return_index=True)
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    val = np.where(kind[at] == 1, low, (1 + rng.integers(0, 63, keys.size)) / 8.0).astype(np.float32)
+    h = Handle(wl.CSR(n, n, ptr, idx, val), B.F32)
+    dist = torch.empty(n, dtype=torch.float32, device="cuda")
+    want = np.full(n, np.inf, np.float32)
+    want[0] = 0.0
+    r = np.repeat(np.arange(n), np.diff(ptr))
+    for _ in range(4):                                       # (no path has more than three edges)
+        new = want.copy()
+        live = np.isfinite(want[idx])
+        np.minimum.at(new, r[live], want[idx[live]] + val[live])
+        want = new
+    for path in (B.PATH_AUTO, B.PATH_PUSH):
+        h.set_opts(force_path=path)
+        B.db_sssp(h.h, 0, dist)
+        torch.cuda.synchronize()
+        assert np.array_equal(dist.cpu().numpy(), want)
+    assert np.isfinite(want[1501:1601]).sum() > 90
+    h.close()
