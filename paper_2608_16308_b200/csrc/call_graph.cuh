@@ -160,6 +160,15 @@ inline bool build_graph(CallGraph &c, CallList &l) {
     return cudaGraphInstantiate(&c.exec, c.graph, 0) == cudaSuccess;
 }
 
+// While any stream of the process is captured in the global mode, or this thread captures one, the runtime refuses calls that a
+// capture could not express -- cudaStreamQuery and cudaGraphInstantiate among them -- and ends that capture with an error.  Here they
+// concern a stream that is not captured, so they are made in the relaxed mode.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Submits the kernels of one call on `st`.
 inline int submit_calls(dbspmspv_handle_s *h, CallList &l, cudaStream_t st) {
     if (l.overflow) return DBSPMSPV_ERR_CUDA;
@@ -170,6 +179,7 @@ inline int submit_calls(dbspmspv_handle_s *h, CallList &l, cudaStream_t st) {
         (void)cudaGetLastError();
         return launch_plain(h, l, st);
     }
+    RelaxedCapture relaxed;
     if (cudaStreamQuery(st) == cudaErrorNotReady) return launch_plain(h, l, st, true);
     CallGraphs &s = *h->graphs;
     CallGraph *c = nullptr, *oldest = &s.g[0];

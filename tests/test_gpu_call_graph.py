@@ -55,3 +55,52 @@ def test_calls_inside_a_captured_graph(count):
                              (want[0], want[1] * scale, want[2] * abs(scale)))
     check_against_oracle(h.run(x), want)                     # and ordinary calls afterwards
     h.close()
+
+
+@pytest.mark.parametrize("where", ["same thread", "another thread"])
+def test_calls_beside_a_capture(where):
+    """While a stream is being captured in the global mode, calls on another stream that is not captured run as ever, and the
+    capture goes on: first call, second (a graph is built), later ones."""
+    import threading
+
+    csr = wl.rmat(13, 16, seed=8)
+    A = ref_matrix(csr)
+    x = wl.sparse_x(3, 0, csr.n, 1500)
+    want = oracle.ref_pull(A, x.idx, x.val)
+    h = Handle(csr, B.F32)
+    xi, xv = torch.from_numpy(x.idx).to(DEV), torch.from_numpy(x.val).to(DEV)
+    side = torch.cuda.Stream()
+    outs = [(torch.zeros(csr.m, dtype=torch.int32, device=DEV), torch.zeros(csr.m, device=DEV), torch.full((1,), -7, dtype=torch.int32, device=DEV)) for _ in range(4)]
+    count = torch.zeros(4, device=DEV)
+    errors = []
+
+    def calls():
+        try:
+            for yi, yv, k in outs:
+                B.dbspmspv_run(h.h, xi, xv, 1500, B.PLUS_TIMES, yi, yv, csr.m, k, side.cuda_stream)
+                t = threading.Event()
+                t.wait(0.05)                                  # (the stream is idle again: no call of the runtime may ask for it here)
+        except Exception as e:                                # noqa: BLE001
+            errors.append(e)
+
+    count.add_(1.0)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        count.add_(1.0)
+        if where == "same thread":
+            calls()
+        else:
+            t = threading.Thread(target=calls)
+            t.start()
+            t.join()
+        count.mul_(2.0)
+    assert not errors, errors
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    assert (count == 4.0).all()
+    for yi, yv, k in outs:
+        kk = int(k.item())
+        check_against_oracle((yi[:kk].cpu().numpy(), yv[:kk].cpu().numpy(), kk), want)
+    h.close()
