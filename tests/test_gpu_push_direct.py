@@ -131,3 +131,55 @@ def test_payload_runs_once_per_four_columns(dtype, fmt):
                 check_against_oracle(got, oracle.ref_pull(P if dtype == B.PATTERN else A, x.idx, x.val), boolean=semiring == B.OR_AND)
             assert h.get_stats().last_path == B.PATH_PUSH
     h.close()
+
+
+@pytest.mark.parametrize("m", [2048 * 1185, 2048 * 2400 + 7])               # two and three tiles per thread block
+@pytest.mark.parametrize("dtype", [B.F32, B.PATTERN])
+def test_wide_finish_with_private_accumulators(m, dtype):
+    """The finishing kernel of several tiles per thread block behind a push that used private accumulators, with and without a row
+    mask; an unrelated call afterwards shows that accumulators and private copies were left clear."""
+    n = 40009
+    csr = matrix(m, n, 5)
+    h = Handle(csr, dtype)
+    assert h.stats.n_hub_row_blocks > 0
+    A = ref_matrix(csr) if dtype == B.F32 else None
+    P = oracle.RefMatrix(csr.m, csr.n, csr.row_ptr, csr.col_idx, None)
+    rng = np.random.default_rng(m)
+    always = np.int32([3, 4, 21, 300, n - 1])
+    hub_rows = np.bincount(np.repeat(np.arange(csr.m), np.diff(csr.row_ptr))[np.isin(csr.col_idx, always)], minlength=csr.m)
+    drop = rng.random(m) < 0.5
+    drop[33] = True                                                            # (the full row: its row block is a hub)
+    drop[np.flatnonzero(hub_rows)[::3]] = True
+    words = np.packbits(np.r_[drop, np.zeros(-m % 32, bool)], bitorder="little").view(np.int32)
+    mask = torch.from_numpy(words.copy()).to("cuda")
+    h.set_opts(no_small_call=1, hub_min_nnz_x=1)
+    for k in (40, 600):                                                        # (at most n / 64 entries)
+        idx = np.unique(np.r_[always, rng.choice(n, k - 5)]).astype(np.int32)
+        x = wl.SparseVec(n, idx, rng.choice(np.float32([1.0, -2.0, 0.5, -0.0, 2.0 ** -60]), idx.size).astype(np.float32))
+        xi, xv = torch.from_numpy(idx).to("cuda"), torch.from_numpy(x.val).to("cuda")
+        for semiring in (B.OR_AND, B.MIN_PLUS) if dtype == B.PATTERN else (B.PLUS_TIMES, B.OR_AND, B.MIN_PLUS):
+            if semiring == B.MIN_PLUS:
+                wi, wv = oracle.ref_minplus(P if dtype == B.PATTERN else A, x.idx, x.val)
+                want = (wi, wv, np.abs(wv))
+            else:
+                want = oracle.ref_pull(P if dtype == B.PATTERN or semiring == B.OR_AND else A, x.idx, x.val)
+            for complement in (None, 1, 0):
+                if complement is None:
+                    got, w = h.run(x, semiring=semiring), want
+                else:
+                    h.y_nnz.fill_(-7)
+                    B.dbspmspv_run_masked(h.h, xi, xv, idx.size, semiring, mask, complement, h.y_idx, h.y_val, m, h.y_nnz)
+                    kk = int(h.y_nnz.item())
+                    got = (h.y_idx[:kk].cpu().numpy(), h.y_val[:kk].cpu().numpy(), kk)
+                    keep = drop[want[0]] != bool(complement)
+                    w = tuple(v[keep] for v in want)
+                if semiring == B.MIN_PLUS:
+                    assert np.array_equal(got[0], w[0]) and np.array_equal(got[1], w[1].astype(np.float32))
+                else:
+                    check_against_oracle(got, w, boolean=semiring == B.OR_AND)
+            # an unrelated call, without private accumulators
+            one = wl.SparseVec(n, np.int32([700]), np.float32([1.0]))
+            h.set_opts(no_small_call=1, hub_min_nnz_x=-1)
+            check_against_oracle(h.run(one, semiring=B.OR_AND), oracle.ref_pull(P, one.idx, one.val), boolean=True)
+            h.set_opts(no_small_call=1, hub_min_nnz_x=1)
+    h.close()
