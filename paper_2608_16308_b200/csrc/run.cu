@@ -2420,18 +2420,11 @@ static int decode_batch_typed(dbspmspv_handle_s *h, const void *x, int64_t ldx, 
 __global__ void k_sssp_init(float *dist, int64_t n, int32_t src, int32_t *x_idx, float *x_val, int32_t *count) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += stride) dist[v] = v == src ? 0.0f : __int_as_float(0x7F800000);
-    if (blockIdx.x == 0 && threadIdx.x == 0) { x_idx[0] = src; x_val[0] = 0.0f; count[0] = 0; count[2] = 0; count[3] = 0; }
+    if (blockIdx.x == 0 && threadIdx.x == 0) { x_idx[0] = src; x_val[0] = 0.0f; count[0] = 0; }
 }
 
-// A step whose x reaches more than this share of the stored elements is pulled (where the handle
-// has a (min, +) pull): such an x is a handful of hubs or half the graph, its push is a queue of
-// atomics on the hub rows, and the streaming pull reads the matrix once whatever x holds.
-#ifndef DBS_SSSP_PULL_EDGE_FRAC
-#define DBS_SSSP_PULL_EDGE_FRAC 0.1f
-#endif
-
-// count[0]: entries of the next x; count[2..3]: the out-edges they hold (64 bits; INLINE runs of the block-CSC view)
-__global__ void k_sssp_relax(Device d, const int32_t *__restrict__ y_idx, const float *__restrict__ y_val, const int32_t *__restrict__ y_nnz,
+// count[0]: entries of the next x
+__global__ void k_sssp_relax(const int32_t *__restrict__ y_idx, const float *__restrict__ y_val, const int32_t *__restrict__ y_nnz,
                              float *__restrict__ dist, int32_t *__restrict__ x_idx, float *__restrict__ x_val, int32_t *count) {
     const int n = *y_nnz;
     const int lane = threadIdx.x & 31;
@@ -2447,17 +2440,12 @@ __global__ void k_sssp_relax(Device d, const int32_t *__restrict__ y_idx, const 
         int base = 0;
         if (lane == 0) base = atomicAdd(count, __popc(m));
         base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        int deg = 0;
         if (better) {
             const int pos = base + __popc(m & ((1u << lane) - 1u));
             dist[i] = v;
             x_idx[pos] = i;
             x_val[pos] = v;
-            int first;
-            column_run(d, i, first, deg);
         }
-        deg = __reduce_add_sync(0xFFFFFFFFu, deg);
-        if (lane == 0 && deg) atomicAdd(reinterpret_cast<unsigned long long *>(count + 2), (unsigned long long)deg);
     }
 }
 
@@ -2522,33 +2510,26 @@ static int sssp_typed(dbspmspv_handle_s *h, int32_t src, float *dist, int32_t *n
         xv[0] = reinterpret_cast<float *>(p); p += n * sizeof(float);
         xv[1] = reinterpret_cast<float *>(p); p += n * sizeof(float);
         y_val = reinterpret_cast<float *>(p); p += n * sizeof(float);
-        ctr = reinterpret_cast<int32_t *>(p);                 // [0] next x count, [1] y_nnz, [2..3] out-edges of the next x
+        ctr = reinterpret_cast<int32_t *>(p);                 // [0] next x count, [1] y_nnz
     }
     k_sssp_init<<<4 * h->sm_count, 256, 0, st>>>(dist, n, src, xi[0], xv[0], ctr);
     ++h->kernel_launches;
     int32_t nnz_x = 1;
-    int64_t edges = 0;
     int steps = 0, cur = 0, status = DBSPMSPV_OK;
-    const int user_path = h->ropts.force_path;
     while (nnz_x > 0) {
         if (++steps > n + 1) { status = DBSPMSPV_ERR_UNSUPPORTED; break; }          // a cycle of negative weight
-        // direction of this step: the caller's, else by the share of the stored elements x reaches
-        if (user_path == DBSPMSPV_PATH_AUTO)
-            h->ropts.force_path = (double)edges > (double)DBS_SSSP_PULL_EDGE_FRAC * (double)d.n_entries ? DBSPMSPV_PATH_PULL : DBSPMSPV_PATH_PUSH;
         status = run_typed<DT>(h, xi[cur], xv[cur], nnz_x, DBSPMSPV_MIN_PLUS, y_idx, y_val, n, ctr + 1, st);
         if (status != DBSPMSPV_OK) break;
-        k_sssp_relax<<<2 * h->sm_count, 256, 0, st>>>(d, y_idx, y_val, ctr + 1, dist, xi[cur ^ 1], xv[cur ^ 1], ctr);
+        k_sssp_relax<<<2 * h->sm_count, 256, 0, st>>>(y_idx, y_val, ctr + 1, dist, xi[cur ^ 1], xv[cur ^ 1], ctr);
         ++h->kernel_launches;
-        if (cudaMemcpyAsync(h->sssp_host, ctr, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaMemsetAsync(ctr, 0, 4 * sizeof(int32_t), st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
+        if (cudaMemcpyAsync(h->sssp_host, ctr, sizeof(int32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaMemsetAsync(ctr, 0, sizeof(int32_t), st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
             status = DBSPMSPV_ERR_CUDA;
             break;
         }
         nnz_x = h->sssp_host[0];
-        edges = (int64_t)(uint32_t)h->sssp_host[2] | ((int64_t)h->sssp_host[3] << 32);
         cur ^= 1;
     }
-    h->ropts.force_path = user_path;
     if (status != DBSPMSPV_OK) return status;
     if (n_steps) *n_steps = steps;
     return DBSPMSPV_OK;
