@@ -147,7 +147,7 @@ typedef struct {
                                 0.08, measured (0.06 .. 0.1 are within 1 %)                */
     int32_t hub_min_nnz_x;   /* dbspmspv_run: shortest x list for which the push adds into the
                                 private accumulators of hub row blocks (the finishing kernel
-                                folds them); 0 = default (4096), < 0 = never               */
+                                folds them); 0 = default (16384), < 0 = never              */
     float decode_threshold;  /* dbspmspv_decode: activation magnitude cut fused into the vector
                                 blocking (Section 5.3: activation sparsity by magnitude
                                 thresholding) -- x_j takes part iff |x_j| > decode_threshold;

@@ -75,8 +75,11 @@ constexpr int HUB_COPIES = DBS_HUB_COPIES;              // private accumulator c
 constexpr int HUB_BLOCKS_MAX = DBS_HUB_BLOCKS_MAX;      // hub row blocks per handle, at most
 constexpr int HUB_BLOCK_MIN_ENTRIES = DBS_HUB_MIN_ENTRIES; // view entries that make a row block a hub
 constexpr uint16_t HUB_NONE = 0xFFFFu;
+// Private accumulators cost their fold, 1 - 2 us with four copies and 1 more with sixteen, and save the queue of atomics on the hub rows.  R-MAT
+// scale 20, forced push, x of 8 K / 16 K / 32 K / 64 K / 256 K entries: 14.1 / 16.1 / 20.0 / 27.6 / 79 us without, 15.8 / 16.8 / 19.3 / 23.5 / 56.8 with four,
+// 17.6 / 18.4 / 21.1 / 24.7 / 56.2 with sixteen; scale 17: 12.1 / 15.0 / 20.0 / 30.4 without, 12.9 / 14.5 / 18.0 / 24.5 with four.
 constexpr int HUB_ALL_NNZ_X = 65536;        // shorter x: four copies are enough, and the fold is a quarter
-constexpr int HUB_MIN_NNZ_X = 4096;          // shorter x: too few products for a queue
+constexpr int HUB_MIN_NNZ_X = 16384;        // shorter x: the fold costs more than the queue
 constexpr uint32_t HUB_CLEAR = 0x80000000u; // an untouched private accumulator (= ACC_CLEAR)
 // The dense accumulator of a product (Workspace::y_acc).  A row that nothing was added to holds
 // ACC_CLEAR = -0.0f, and any sum of products that are each at least ACC_FLAG_MIN in magnitude
