@@ -15,7 +15,7 @@ Bytes.  Three figures per call (ByteModel below, all computed on the host from t
            under a nonempty vector block (what a purely block-granular method must touch);
   B_min    the format-independent floor of a plain CSC gather.
 
-python bench.py [--gpus N --steps K --warmup W] [--impl reference] [--no-bfs] [--no-extras]
+python bench.py [--gpus N --steps K --warmup W] [--impl reference] [--no-bfs] [--no-extras] [--record FILE]
 Under torchrun every rank runs the same sweep on its own GPU (independent replicas: the path
 has no exchange step), times are the max over ranks, `value` is the whole-job aggregate.
 """
@@ -44,6 +44,7 @@ VIEW_ENTRY_BYTES = 9          # idx 4 + w 4 + aux 1 per view entry
 NOMINAL_HBM_GBS = 8000.0      # the nominal HBM3e figure, reported beside the measured copy bandwidth
 LEAN_CHUNK = 256              # entries per chunk of the streaming pull (whole chunks are read)
 PUSH, PULL = 1, 2
+TH3 = 0.95                    # the selector's default: push below this share of nonempty vector blocks
 
 
 # ---------------------------------------------------------------------------------------------
@@ -117,31 +118,41 @@ class ByteModel:
                 "payload_bytes": int(payload), "pointer_bytes": int(pointers), "active_vector_blocks": int(xb.size)}
 
     def moved(self, x_idx: np.ndarray, path: int, y_nnz: int, fmt: dict | None = None, one_kernel: bool = False) -> dict:
-        """Bytes the implementation moves on `path`, each distinct byte once: the format part
-        (above), x (the list, the dense copy written and gathered, the masks, the clean-up),
-        y (accumulator read-modify-write, hit flags, the sorted output) and two O(m) scans
-        (hit flags in, packed masks out and in).  The x, y and scan terms are those of a push over a staged
-        x with hit flags and a two-pass compaction; they are kept so that figures compare across versions.  The
-        kernels of today move fewer bytes for x (a push takes it from its list) and more for y: the
-        finishing kernel reads the accumulator itself, 4 m bytes in place of 1.25 m.  one_kernel: the
-        single-kernel form of a short call -- x is read once as a list, the row bitmap lives in
-        shared memory (no scans), y is the accumulator read-modify-write, the row list written
-        and read back, the gather-and-clear and the output."""
+        """Bytes the implementation moves on `path`, each distinct byte once per kernel that needs it: the format part (above), x, y.
+        x: the list; a push that is certain takes its columns from the list (masks set and cleared, the indices read once more to
+        clear them, or the masks swept); otherwise x is staged (dense copy and masks written, read by the traversal -- the masks
+        whole --, cleared entry by entry or, for a long x, swept).  y: the accumulator's read-modify-write per result row, its
+        4 bytes per row and the flag bit read by the finishing kernel, the rows that were hit put back, the sorted output.  (The
+        private accumulators of hub rows, at most 256 KB, are not counted.)  one_kernel: the single-kernel form of a short call --
+        x is read once as a list, the row bitmap lives in shared memory, y is the accumulator read-modify-write, the row list
+        written and read back, the gather-and-clear and the output."""
         f = fmt if fmt is not None else self.format_bytes(x_idx, path)
-        m, nx = self.csr.m, x_idx.size
-        if one_kernel:
-            fmt_total = f["view_bytes"] + f["payload_bytes"] + f["pointer_bytes"]
-            xbytes, ybytes = 8.0 * nx, 8.0 * y_nnz + 8.0 * y_nnz + 8.0 * y_nnz + 8.0 * y_nnz
-            return {"format": fmt_total, "x": xbytes, "y": ybytes, "scans": 0.0, "total": fmt_total + xbytes + ybytes,
-                    "traversal_kernel": fmt_total + xbytes + ybytes}
-        xbytes = 8.0 * nx + 4.0 * nx + 4.0 * nx + 2.0 * f["active_vector_blocks"] + 4.0 * nx + 6.0 * nx
-        if path == PULL:
-            xbytes += self.csr.n / 8.0                       # the presence filter, read once per SM from L2
-        ybytes = 8.0 * y_nnz + 2.0 * y_nnz + 8.0 * y_nnz + 8.0 * y_nnz
-        scans = m * 1.0 + (m / 8.0) * 2.0
+        m, n, nx, active = self.csr.m, self.csr.n, x_idx.size, f["active_vector_blocks"]
         fmt_total = f["view_bytes"] + f["payload_bytes"] + f["pointer_bytes"]
-        return {"format": fmt_total, "x": xbytes, "y": ybytes, "scans": scans, "total": fmt_total + xbytes + ybytes + scans,
-                "traversal_kernel": fmt_total + 4.0 * nx + 10.0 * y_nnz + (self.csr.n / 8.0 if path == PULL else 2.0 * f["active_vector_blocks"])}
+        if one_kernel:
+            xbytes, ybytes = 8.0 * nx, 32.0 * y_nnz
+            return {"format": fmt_total, "x": xbytes, "y": ybytes, "accumulator_scan": 0.0, "total": fmt_total + xbytes + ybytes,
+                    "traversal_kernel": fmt_total + xbytes + ybytes}
+        if self.from_list(nx, path):
+            read, x_clear = 8.0 * nx + 4.0 * active, n / 8.0 if 128 * nx > n else 4.0 * nx + 2.0 * active
+            xbytes = read + x_clear
+        else:
+            read = 4.0 * nx + (2.0 * active if self.heavy else n / 8.0)
+            x_clear = 4.0 * n + n / 8.0 if 8 * nx > n else 8.0 * nx + 2.0 * active
+            xbytes = 12.0 * nx + 4.0 * active + read + x_clear
+        ybytes = 8.0 * y_nnz + 4.0 * y_nnz + 8.0 * y_nnz
+        scan = 4.0 * m + m / 8.0
+        return {"format": fmt_total, "x": xbytes, "y": ybytes, "accumulator_scan": scan, "total": fmt_total + xbytes + ybytes + scan,
+                "traversal_kernel": fmt_total + read + 8.0 * y_nnz}
+
+    def from_list(self, nx: int, path: int) -> bool:
+        """A push whose direction the host is certain of: x has too few entries to reach the selector's ratio."""
+        return path == PUSH and not self.heavy and np.float32(min(nx, self.nb)) / np.float32(self.nb) < np.float32(TH3)
+
+    def x_bytes_over_the_bus(self, nx: int, path: int, one_kernel: bool) -> int:
+        """Bytes of x a call reads when x lies in host memory: the list, and the indices once more where they are cleared one by one."""
+        swept = (128 if self.from_list(nx, path) else 8) * nx > self.csr.n
+        return 8 * nx + (0 if one_kernel or swept else 4 * nx)
 
     def touch(self, x_idx: np.ndarray, y_nnz: int, y_row_blocks: int) -> float:
         xb = np.unique(x_idx >> 4)
@@ -262,7 +273,7 @@ def reference_arm(args) -> None:
                 best = dt if best is None or dt < best else best
             t_step += best
             # same numerator as the GPU arm: the bytes the library moves on its default path
-            path = PUSH if np.float32(np.unique(x.idx >> 4).size) / np.float32(model.nb) < np.float32(0.9) else PULL
+            path = PUSH if np.float32(np.unique(x.idx >> 4).size) / np.float32(model.nb) < np.float32(TH3) else PULL
             bytes_step += model.moved(x.idx, path, yi.size, None, path == PUSH and x.idx.size <= 256)["total"]    # (short calls: the one-kernel form)
         if it >= args.warmup:
             per_step.append(t_step)
@@ -345,6 +356,8 @@ def main() -> None:
     ap.add_argument("--stencil-d", type=int, default=160, help="edge length of the stencil grid for --stencil-only")
     ap.add_argument("--crossover", action="store_true",
                     help="print the measured push/pull crossover table (forced paths) and exit")
+    ap.add_argument("--record", metavar="FILE", help="write the whole record, every leg with all its figures, to FILE")
+    ap.add_argument("--full-line", action="store_true", help="print the whole record instead of its summary")
     ap.add_argument("--ablation", action="store_true", help="print the block-format ablation and storage records and exit")
     args = ap.parse_args()
     args.warmup = max(args.warmup, 3)
@@ -488,9 +501,7 @@ def main() -> None:
             stream.synchronize()
             kk = int(y_nnz_h.item())
             tot += e0.elapsed_time(e1)
-            # x is read once by the blocking kernel; its indices once more by the clean-up pass
-            # unless the dense copy is cleared wholesale (x lists more than n / 8 columns)
-            h2d += 8 * n_x + (0 if 8 * n_x > a.n else 4 * n_x)
+            h2d += model.x_bytes_over_the_bus(n_x, info[k][0], one_kernel[k])
             d2h += 4 + 8 * kk
         if s >= 2:
             e2e_ms.append(tot)
@@ -587,9 +598,32 @@ def main() -> None:
     if h is not None:
         B.dbspmspv_destroy(h)
     if rank == 0:
-        print(json.dumps(line))
+        if args.record:
+            with open(args.record, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(line if args.full_line else summary(line)))
     if world > 1:
         dist.destroy_process_group()
+
+
+SUMMARY_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+                "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline", "value_on_B_touch",
+                "value_on_B_min")
+
+
+def summary(line: dict) -> dict:
+    """The printed line: the figures of the timed sweep, and one figure per further leg (--full-line or --record FILE: everything)."""
+    out = {k: line[k] for k in SUMMARY_KEYS if k in line}
+    out["sweep"] = [{k: r[k] for k in ("x_fraction", "path", "us", "us_l2_warm", "traversal_kernel_us", "y_nnz")} for r in line["sweep"]]
+    if "cusparse_spmv_reference" in line:
+        out["cusparse_spmv_us"] = line["cusparse_spmv_reference"].get("us")
+    others = line.get("other_configs")
+    if isinstance(others, list):
+        out["other_us"] = {f"{r['workload']}, {r['x']}" if "x" in r else str(r["workload"]): r.get("us") for r in others if r.get("us") is not None}
+    bfs = line.get("bfs", {})
+    if bfs:
+        out["bfs"] = {k: bfs[k] for k in ("workload", "gteps_harmonic_mean", "ms_median", "sources_matching_oracle", "error") if k in bfs}
+    return out
 
 
 def crossover_table() -> None:
@@ -1113,7 +1147,7 @@ def bfs_level_bytes(g: wl.CSR, lv: np.ndarray, paths):
 
 
 def bench_bfs(args, B, torch, dev, flush, peak):
-    """DB-BFS GTEPS on the symmetrised R-MAT graph, 16 seeded sources (configs[3]); every timed
+    """DB-BFS GTEPS on the symmetrised R-MAT graph, 16 seeded sources; every timed
     source is compared with the oracle; per-level time, direction and algorithmic bytes for the
     first source."""
     g = wl.rmat(args.bfs_scale, 16, seed=3, values=False, symmetrise=True)
