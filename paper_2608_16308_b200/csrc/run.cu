@@ -2171,8 +2171,11 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
     if (extra > 4 * h->sm_count) extra = 4 * h->sm_count;
     // scattered clears cost more than a full sweep once x lists a good part of the columns (a sweep of the masks alone is 32 times shorter)
     if ((int64_t)nnz_x * (clear & CLEAR_DENSE ? 8 : 128) > d.n) clear |= CLEAR_SWEEP;
-    // several tiles per thread block where they would come in waves (eight thread blocks per SM)
-    const int wave = 8 * h->sm_count;
+    // several tiles per thread block where they would come in waves (eight thread blocks per SM); behind a short push of whole blocks, which
+    // leaves most tiles untouched, from two thread blocks per SM on (27-point operator on 97^3, 110^3, 128^3, 130^3 cells, x = 0.03 %: 17.3, 18.0, 18.0, 19.9 us
+    // a call with a tile each, 14.6, 15.7, 14.6, 16.6 so; at 0.5 % the same, at 1 % up to 1.5 slower.  Behind a direct push, whose results lie everywhere,
+    // it is the slower form in one wave: R-MAT scale 20, 0.2 %, 13.2 against 15.0)
+    const int wave = (h->heavy_stage && (int64_t)nnz_x * 128 <= d.n ? 2 : 8) * h->sm_count;
     int per_block = (nt + wave - 1) / wave;
     if (per_block > FINISH_WIDE) per_block = FINISH_WIDE;
     // (results in good part of the rows: fetching them twice costs more than the waves, 24 us against 19 with nearly all rows)
@@ -2361,6 +2364,8 @@ static int decode_batch_typed(dbspmspv_handle_s *h, const void *x, int64_t ldx, 
         calls.add(kernel, h->sm_count, BATCH_CTA, (size_t)lay.total, true, d, xg, ldx, yg, ldy, g, only_as_fallback);
         return DBSPMSPV_OK;
     };
+    // (Over columns, 50 % pruned, 30 % active, two vectors in one pass against two single calls: 2048 x 2048 9.1 against 13.0 us, 4096 x 4096 12.3 / 13.3,
+    // 8192 x 4096 16.6 / 13.4, 12288 x 4096 21.4 / 16.3, 8192 x 12288 34.6 / 38.7; three vectors 19 - 40 against 20 - 58.)
     for (int32_t b0 = 0; b0 < batch;) {
         const int left = batch - b0;
         const void *xg = static_cast<const uint8_t *>(x) + (size_t)b0 * (size_t)ldx * esize;

@@ -183,3 +183,43 @@ def test_wide_finish_with_private_accumulators(m, dtype):
             check_against_oracle(h.run(one, semiring=B.OR_AND), oracle.ref_pull(P, one.idx, one.val), boolean=True)
             h.set_opts(no_small_call=1, hub_min_nnz_x=1)
     h.close()
+
+
+@pytest.mark.parametrize("tiles", [296, 297, 593, 1200])                     # one, two, three and four tiles per thread block (148 SMs)
+def test_wide_finish_behind_a_push_of_whole_blocks(tiles):
+    """A short x on a tall matrix whose elements sit in full blocks, rows at both ends of tiles among them, masked and not."""
+    m, n = 2048 * tiles - 3, 40009
+    rng = np.random.default_rng(tiles)
+    rbs = np.unique(np.r_[0, 127, 128, m // 16 - 1, rng.integers(0, m // 16, 1500)])
+    r = (16 * rbs[:, None] + np.arange(16)).reshape(-1, 16, 1)
+    c = (16 * rng.integers(0, n // 16, rbs.size)[:, None] + np.arange(16)).reshape(-1, 1, 16)
+    keys = wl.sorted_unique((r * np.int64(n) + c).ravel()[rng.random(rbs.size * 256) < 0.8])
+    ptr, idx = wl.csr_from_sorted_keys(m, n, keys)
+    csr = wl.CSR(m, n, ptr, idx, rng.choice(np.float32([1.5, -0.75, 0.0, -0.0, 2.0 ** -60]), keys.size).astype(np.float32))
+    h, A = Handle(csr, B.F32), ref_matrix(csr)
+    assert h.stats.class_nnz[B.BLK_INLINE] * 2 < h.stats.nnz
+    drop = rng.random(m) < 0.5
+    mask = torch.from_numpy(np.packbits(np.r_[drop, np.zeros(-m % 32, bool)], bitorder="little").view(np.int32).copy()).to("cuda")
+    for k in (3, 312):                                                         # (at most n / 128 entries)
+        at = np.unique(np.r_[csr.col_idx[:3], csr.col_idx[-3:], rng.choice(csr.col_idx, k)])[:312].astype(np.int32)
+        x = wl.SparseVec(n, at, rng.choice(np.float32([1.0, -2.0, 2.0 ** -60]), at.size).astype(np.float32))
+        xi, xv = torch.from_numpy(at).to("cuda"), torch.from_numpy(x.val).to("cuda")
+        for semiring in (B.PLUS_TIMES, B.OR_AND, B.MIN_PLUS):
+            if semiring == B.MIN_PLUS:
+                wi, wv = oracle.ref_minplus(A, x.idx, x.val)
+                want = (wi, wv, np.abs(wv))
+            else:
+                want = oracle.ref_pull(A, x.idx, x.val)
+            for complement in (None, 1):
+                if complement is None:
+                    got, w = h.run(x, semiring=semiring), want
+                else:
+                    B.dbspmspv_run_masked(h.h, xi, xv, at.size, semiring, mask, 1, h.y_idx, h.y_val, m, h.y_nnz)
+                    kk = int(h.y_nnz.item())
+                    got = (h.y_idx[:kk].cpu().numpy(), h.y_val[:kk].cpu().numpy(), kk)
+                    w = tuple(v[~drop[want[0]]] for v in want)
+                if semiring == B.MIN_PLUS:
+                    assert np.array_equal(got[0], w[0]) and np.array_equal(got[1], w[1].astype(np.float32))
+                else:
+                    check_against_oracle(got, w, boolean=semiring == B.OR_AND)
+    h.close()
