@@ -108,14 +108,19 @@ typedef struct {
 /* Run-time options; may be changed between calls with dbspmspv_set_run_opts.               */
 typedef struct {
     float th3;               /* dbspmspv_run: push iff the nonempty-vector-block ratio is
-                                below th3.  0.01 in the paper; default 0.95, the crossover
-                                measured on B200 (the table `bench.py --crossover` prints)    */
+                                below th3.  0.01 in the paper; default 0.95.  On B200 the push stays
+                                ahead up to a ratio of 0.97 (uniform rows) and 0.997 (R-MAT scale 20, x
+                                of 30 %: 75 against 77 us); past that the ratio cannot tell 30 % of all
+                                columns from all of them, where the pull is ahead (179 / 110 us)
+                                (the table `bench.py --crossover` prints)                     */
     int32_t force_path;      /* DBSPMSPV_PATH_*                                              */
     int32_t popc_threshold;  /* CSR-class blocks: popc(mask) >= this -> row-driven (pull-style)
                                 microkernel, below -> column-driven (push-style)             */
     int32_t validate;        /* x indices outside [0, n) are always skipped and reported as
                                 ERR_BOUNDS; 1: an index listed twice is reported as well
-                                (deferred ERR_INVALID_ARG; it contributes once either way)   */
+                                (deferred ERR_INVALID_ARG; it contributes once either way -- except in the
+                                one-kernel form of a short call, which validate switches off and
+                                which adds it as often as it is listed)                      */
     int32_t timing;          /* 1: bracket the traversal kernel of run/decode with two CUDA
                                 events (made at create); read back as last_compute_ms      */
     float th3_bfs;           /* db_bfs: same rule per level.  Default 0.05, measured on the
@@ -187,7 +192,8 @@ typedef struct {
     /* last dbspmspv_run / dbspmspv_decode */
     int32_t last_path;             /* DBSPMSPV_PATH_PUSH or _PULL                             */
     int32_t last_n_nzblk;          /* nonempty vector blocks                                  */
-    int32_t last_n_tasks;          /* push worklist length                                    */
+    int32_t last_n_tasks;          /* push worklist length (direct push: warp steps and listed
+                                      chunks; 0 for the one-kernel forms)                     */
     int32_t last_y_nnz;
     /* last db_bfs */
     int32_t bfs_levels;            /* number of expansion steps executed                      */
@@ -257,7 +263,8 @@ int dbspmspv_create_coo(dbspmspv_handle_t *out, int64_t m, int64_t n, int64_t nn
  * x_idx, x_val, y_idx, y_val and y_nnz are device pointers -- or page-locked host memory that
  * the device addresses directly (cudaHostAlloc / cudaHostRegister under unified addressing):
  * the call's kernels then read x and write y across the bus themselves, with no staging copy
- * (x_idx is read a second time by the clean-up pass unless x lists more than n / 8 columns).
+ * (x_idx is read a second time by the clean-up unless x is long -- more than n / 128 columns where the
+ * push is certain, n / 8 elsewhere -- or the call takes its one-kernel form).
  * nnz_x = 0 gives y_nnz = 0.  Errors: INVALID_ARG, UNSUPPORTED synchronously.
  */
 int dbspmspv_run(dbspmspv_handle_t h, const int32_t *x_idx, const void *x_val, int32_t nnz_x,

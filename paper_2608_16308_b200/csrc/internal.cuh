@@ -130,7 +130,9 @@ constexpr int STAGE_BYTES = DBS_STAGE_BYTES;
 // Decode over columns (decode_columns.cuh): rows of a strip; the bf16 pattern of an absent element; where the copy is built.
 constexpr int DC_ROWS = 64;
 constexpr uint32_t DC_ABSENT = 0x8000u;
-constexpr int DC_MIN_ROWS = 1024;           // (fewer rows make too few strips: the block kernels deal the payload out over all SMs)
+// Where the copy by columns is built.  Layers of fewer rows keep the block kernels and half the memory; the copy would be the faster form for
+// them too (128 - 960 rows, 4,096 or 8,192 columns, 30 % active: one vector 4.7 - 6.0 us over columns, 6.5 - 10 by blocks; eight 8.3 - 15 against 18 - 43).
+constexpr int DC_MIN_ROWS = 1024;
 constexpr int DC_MAX_COLUMNS = 25600;       // the list of active columns has to fit in shared memory
 constexpr int DC_MAX_RATIO = 4;             // copy / payload, at most
 constexpr int HDR_BYTES = 48;               // masks + starts of a valued mid-class block
@@ -412,7 +414,7 @@ __device__ __forceinline__ uint32_t mask_of(const uint32_t *mask32, int blk) {
 // Order-preserving map of fp32 to signed words: monotone, and the bits themselves where v >= 0.
 __host__ __device__ inline int ordered_word(int bits) { return bits ^ ((bits >> 31) & 0x7FFFFFFF); }
 
-// Adds one sum to a row of the accumulator (see ACC_CLEAR).
+// Whether a sum that is added to a row of the accumulator has to set the row's flag bit as well (see ACC_CLEAR).
 __device__ __forceinline__ bool acc_needs_flag(float v) { return !(fabsf(v) >= ACC_FLAG_MIN); }
 
 // value loads from the payload, widened to fp32

@@ -59,7 +59,7 @@ def test_direct_push(m, dtype):
 
 
 @pytest.mark.parametrize("dtype", [B.F32, B.PATTERN])
-def test_long_x_on_a_handle_rich_in_payload_goes_by_blocks(dtype):
+def test_long_x_on_a_handle_rich_in_payload(dtype):
     csr = wl.stencil27(40, seed=3)
     h = Handle(csr, dtype)
     P = oracle.RefMatrix(csr.m, csr.n, csr.row_ptr, csr.col_idx, None)
