@@ -291,7 +291,6 @@ struct Device {           // everything the kernels need, passed by value
     float *hub_acc;
     int32_t n_hub_blocks;
     int32_t hub_on;           // copies this call's push uses (set per call by the host; 0: none)
-    int32_t payload_groups;   // direct push, per call: payload entries are listed once per four columns (payload_rows) instead of once per column
     int32_t long_cap;         // direct push: chunks of all long runs and payload runs together (0: the matrix has none)
     const uint32_t *row_present32;  // per row block: rows that hold a stored element (two 16-bit masks per word)
     Workspace ws;

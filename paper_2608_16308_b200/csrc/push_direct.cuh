@@ -19,7 +19,7 @@
 // A run longer than PD_LONG entries (a hub column of an R-MAT matrix has tens of thousands; left to one
 // thread block it was the whole kernel's time) is cut into chunks that go to a list instead, and so is the run of payload entries of a
 // listed column's block, a chain of three or four dependent loads each: once per listed column, or, for a longer x on a handle with many of
-// them, once per group of four columns (Device::payload_groups), whose listed ones the second kernel takes from the finished masks; a second kernel, launched
+// them, once per group of four columns (GROUPS; a form of its own: as a branch it cost calls of two short kernels 0.2 us), whose listed ones the second kernel takes from the finished masks; a second kernel, launched
 // only on handles that have such runs, deals the chunks out over the warps of the GPU.  Space in the list is claimed with one
 // atomic per thread block: an atomic per run was up to eight round trips in one thread, and atomics on one word take
 // 1.4 ns each.  (Taking chunks dynamically at the end of the first kernel, from a ticket
@@ -211,7 +211,7 @@ __device__ __forceinline__ void payload_rows(const Device &d, int first, int cou
     }
 }
 
-template <int DT, int MODE, bool MASKS>
+template <int DT, int MODE, bool MASKS, bool GROUPS>
 __global__ void __launch_bounds__(PD_CTA, pd_per_sm(MASKS))
 k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restrict__ x_val, int32_t nnz_x, int validate, float th3,
               int force_path, int cols, int rounds) {
@@ -273,7 +273,7 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
                     if ((old >> (j & 31)) & 1u) {         // listed before: contributes once
                         deg[0] = 0; pdeg = 0; listed = 0u;
                         if (validate) ctr->status = DBSPMSPV_ERR_INVALID_ARG;
-                    } else if (d.payload_groups) {
+                    } else if (GROUPS) {
                         if ((old >> (j & 28)) & 15u) pdeg = 0;               // (listed by the thread that came to these four columns first)
                         if (MODE != 1) d.ws.x_dense[j] = xv[0];              // (k_push_long takes x from there)
                     }
@@ -286,7 +286,7 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
 #pragma unroll
             for (int k = 0; k < PER; ++k)
                 if (deg[k] > PD_LONG) { n_rec += (deg[k] + PD_CHUNK - 1) / PD_CHUNK; deg[k] = -deg[k]; }      // (negative: listed)
-            if (pdeg > 0) n_rec += (d.payload_groups ? 1 : __popc(listed)) * ((pdeg + PD_PAYLOAD - 1) / PD_PAYLOAD);
+            if (pdeg > 0) n_rec += (GROUPS ? 1 : __popc(listed)) * ((pdeg + PD_PAYLOAD - 1) / PD_PAYLOAD);
         }
         // lay the nonempty short runs end to end
         int n_cols = 0, n_elems = 0;
@@ -336,7 +336,7 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
                     for (int q = lane; q < n_chunks; q += 32) d.ws.long_runs[o + q] = make_int4(f + q * PD_CHUNK, min(PD_CHUNK, n - q * PD_CHUNK), xb, 0);
                     if (lane == src) at += n_chunks;
                 }
-            if (pdeg > 0 && d.payload_groups)
+            if (pdeg > 0 && GROUPS)
                 for (int q = 0; q < pdeg; q += PD_PAYLOAD) d.ws.long_runs[at++] = make_int4(pfirst + q, min(PD_PAYLOAD, pdeg - q), col0 >> 2, 0x100);
             else if (pdeg > 0)
 #pragma unroll

@@ -2114,14 +2114,14 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
         const bool may_pull = (!minplus || DT != DBSPMSPV_PATTERN) && pull_possible(h, nnz_x, h->ropts.th3);
         const bool may_push = !may_pull || fp != DBSPMSPV_PATH_PULL;
         const int mode = boolean ? 1 : minplus ? 2 : 0;
-        h->d.payload_groups = h->payload_rich && nnz_x >= PD_GROUPS_MIN_NNZ_X;
+        const bool groups = h->payload_rich && nnz_x >= PD_GROUPS_MIN_NNZ_X;
         // private accumulators for the hub row blocks, when x is long enough for their atomics to queue up
         const int hub_min = h->ropts.hub_min_nnz_x ? h->ropts.hub_min_nnz_x : HUB_MIN_NNZ_X;
         h->d.hub_on = may_push && d.n_hub_blocks > 0 && hub_min > 0 && nnz_x >= hub_min ? (nnz_x < HUB_ALL_NNZ_X ? 4 : HUB_COPIES) : 0;
         if (may_pull && nnz_x > 0) calls.add(k_xblock_sparse<DT, false>, (nnz_x + XB_TPB - 1) / XB_TPB, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
         if (h->ropts.timing) calls.ev_before = calls.n;
         if (nnz_x > 0 && may_push) {
-            auto push = [&](auto list_kernel, auto mask_kernel, auto long_kernel, auto groups_kernel) {
+            auto push = [&](auto list_kernel, auto mask_kernel, auto long_kernel) {
                 if (may_pull) {
                     // (decided on the device) 32 mask words per thread block and round
                     const int n_words = (d.nb + 1) / 2;
@@ -2140,21 +2140,22 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
                     if (g > most) g = most;
                     calls.add(list_kernel, g, PD_CTA, 0, false, d, x_idx, xv, nnz_x, (int)h->ropts.validate, h->ropts.th3, fp, cols, (nnz_x + cols * g - 1) / (cols * g));
                 }
-                if (d.long_cap) calls.add(d.payload_groups ? groups_kernel : long_kernel, 6 * h->sm_count, PD_CTA, 0, true, d);
+                if (d.long_cap) calls.add(long_kernel, 6 * h->sm_count, PD_CTA, 0, true, d);
             };
-            if (mode == 1) push(k_push_direct<DT, 1, false>, k_push_direct<DT, 1, true>, k_push_long<DT, 1, false>, k_push_long<DT, 1, true>);
-            else if (mode == 2) push(k_push_direct<DT, 2, false>, k_push_direct<DT, 2, true>, k_push_long<DT, 2, false>, k_push_long<DT, 2, true>);
-            else if (DT != DBSPMSPV_PATTERN) {
-                constexpr int VT = DT == DBSPMSPV_PATTERN ? DBSPMSPV_F32 : DT;       // (pattern handles have no (+, *))
-                push(k_push_direct<VT, 0, false>, k_push_direct<VT, 0, true>, k_push_long<VT, 0, false>, k_push_long<VT, 0, true>);
-            };
+            constexpr int VT = DT == DBSPMSPV_PATTERN ? DBSPMSPV_F32 : DT;       // (pattern handles have no (+, *))
+            if (mode == 1 && groups) push(k_push_direct<DT, 1, false, true>, k_push_direct<DT, 1, true, true>, k_push_long<DT, 1, true>);
+            else if (mode == 1) push(k_push_direct<DT, 1, false, false>, k_push_direct<DT, 1, true, false>, k_push_long<DT, 1, false>);
+            else if (mode == 2 && groups) push(k_push_direct<DT, 2, false, true>, k_push_direct<DT, 2, true, true>, k_push_long<DT, 2, true>);
+            else if (mode == 2) push(k_push_direct<DT, 2, false, false>, k_push_direct<DT, 2, true, false>, k_push_long<DT, 2, false>);
+            else if (DT != DBSPMSPV_PATTERN && groups) push(k_push_direct<VT, 0, false, true>, k_push_direct<VT, 0, true, true>, k_push_long<VT, 0, true>);
+            else if (DT != DBSPMSPV_PATTERN) push(k_push_direct<VT, 0, false, false>, k_push_direct<VT, 0, true, false>, k_push_long<VT, 0, false>);
         }
         if (any && may_pull) {
             const int s = minplus ? launch_lean<DT, OutSparseMin>(h, calls, OutSparseMin{d.ws.y_acc, d.ws.y_mask32}, h->ropts.th3)
                                   : launch_lean<DT, OutSparse>(h, calls, OutSparse{d.ws.y_acc, d.ws.y_mask32}, h->ropts.th3);
             if (s != DBSPMSPV_OK) return s;
         }
-        if (!may_pull && (mode == 1 || !d.payload_groups)) clear = CLEAR_MASKS;      // (x was staged for the payload entries only)
+        if (!may_pull && (mode == 1 || !groups)) clear = CLEAR_MASKS;      // (x was staged for the payload entries only)
     } else {
         if (nnz_x > 0) calls.add(k_xblock_sparse<DT, true>, (nnz_x + XB_TPB - 1) / XB_TPB, XB_TPB, 0, false, d, x_idx, xv, nnz_x, h->ropts.validate);
         if (h->ropts.timing) calls.ev_before = calls.n;
