@@ -527,6 +527,13 @@ __global__ void k_csc_gather(int32_t n_blocks, const uint64_t *keys_sorted,
     bcol_sorted[p] = (int32_t)(k >> CSC_KEY_COL_SHIFT);
 }
 
+// Out-degree of a column (its INLINE elements) in eight bits, see degree_code.
+__global__ void k_col_degree(int32_t nb, const int32_t *colptr, uint8_t *code) {
+    int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j >= (int64_t)nb * 16) return;
+    const int32_t *cp = colptr + 17 * (j >> 4) + (j & 15);
+    code[j] = (uint8_t)degree_code((uint32_t)(cp[1] - cp[0]));
+}
 // ---- row-run index of the INLINE elements (DB-BFS pull levels)
 __global__ void k_rowrun_keys(int32_t n_entries, int64_t m, const int32_t *entry_row, const uint32_t *csr_idx,
                               const uint8_t *csr_aux, uint64_t *keys, uint32_t *vals) {
@@ -540,33 +547,40 @@ __global__ void k_rowrun_keys(int32_t n_entries, int64_t m, const int32_t *entry
     vals[p] = (idx & IDX_MASK) | ((rc & 15u) << 27);
 }
 
-// The INLINE elements by row and weight (see Device::weightrun): key, and the position in the view as value.
-__global__ void k_weightrun_keys(int32_t n_entries, int64_t m, const int32_t *entry_row, const uint32_t *csr_idx, const uint32_t *csr_w,
-                                 const uint8_t *csr_aux, uint64_t *keys, uint32_t *vals) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= n_entries) return;
-    const bool inl = (csr_idx[p] >> TYPE_SHIFT) == DBSPMSPV_BLK_INLINE;
-    const uint64_t row = inl ? (uint64_t)entry_row[p] * 16 + (csr_aux[p] >> 4) : (uint64_t)m;   // others sort behind every row
-    const uint32_t w = (uint32_t)ordered_word((int)csr_w[p]) ^ 0x80000000u;
-    keys[p] = (row << SSSP_WEIGHT_BITS) | (inl ? w >> (32 - SSSP_WEIGHT_BITS) : 0u);
-    vals[p] = (uint32_t)p;
+// The stored elements by row and weight (see Device::weightrun): key, and the element's number as value.
+__global__ void k_weightrun_keys(int64_t n, const uint64_t *ukey, const float *uval, uint64_t *keys, uint32_t *vals) {
+    int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (u >= n) return;
+    const uint64_t row = (ukey[u] >> 35) * 16 + ((ukey[u] >> 4) & 15u);
+    const uint32_t w = (uint32_t)ordered_word(__float_as_int(uval[u])) ^ 0x80000000u;
+    keys[u] = (row << SSSP_WEIGHT_BITS) | (w >> (32 - SSSP_WEIGHT_BITS));
+    vals[u] = (uint32_t)u;
 }
-__global__ void k_weightrun(int32_t n_inline, const uint32_t *pos, const uint32_t *csr_idx, const uint32_t *csr_w, const uint8_t *csr_aux, uint2 *out) {
+__global__ void k_weightrun(int64_t n, const uint32_t *from, const uint64_t *ukey, const float *uval, uint2 *out) {
     int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= n_inline + 4) return;
-    if (k >= n_inline) { out[k] = make_uint2(0u, 0x7F800000u); return; }                        // (slack: groups of four are read whole)
-    const uint32_t p = pos[k];
-    out[k] = make_uint2((csr_idx[p] & IDX_MASK) * 16u + (csr_aux[p] & 15u), csr_w[p]);
+    if (k >= n + 4) return;
+    if (k >= n) { out[k] = make_uint2(0u, 0x7F800000u); return; }                               // (slack: groups of four are read whole)
+    const uint64_t e = ukey[from[k]];
+    out[k] = make_uint2((uint32_t)((e >> 8) & IDX_MASK) * 16u + (uint32_t)(e & 15u), __float_as_uint(uval[from[k]]));
+}
+
+// What no element of a row lies below (see sssp_bound: the runs are in order by the upper bits; a weight of -infinity stays one).
+__global__ void k_row_lightest(int64_t m, const int32_t *ptr, const uint2 *weightrun, float *lightest) {
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    int w = 0x7F800000;
+    if (ptr[i] < ptr[i + 1]) w = max(ordered_word((int)weightrun[ptr[i]].y) & ~((1 << (32 - SSSP_WEIGHT_BITS)) - 1), (int)0x807FFFFFu);
+    lightest[i] = __int_as_float(ordered_word(w));
 }
 
 // ptr[i] = first position whose row is >= i, i = 0..m
-__global__ void k_rowrun_ptr(int64_t m, const uint64_t *keys_sorted, int32_t n, int32_t *ptr) {
+__global__ void k_rowrun_ptr(int64_t m, const uint64_t *keys_sorted, int row_shift, int32_t n, int32_t *ptr) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i > m) return;
     int32_t lo = 0, hi = n;
     while (lo < hi) {
         int32_t mid = lo + ((hi - lo) >> 1);
-        if ((keys_sorted[mid] >> 31) < (uint64_t)i) lo = mid + 1; else hi = mid;
+        if ((keys_sorted[mid] >> row_shift) < (uint64_t)i) lo = mid + 1; else hi = mid;
     }
     ptr[i] = lo;
 }
@@ -910,6 +924,28 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
             else DBS_ENCODE(DBSPMSPV_PATTERN);
 #undef DBS_ENCODE
         }
+        // every row's elements by weight, for the pulled steps of db_sssp
+        d.weightrun = nullptr; d.weight_ptr = nullptr; d.row_lightest = nullptr;
+        h->bfs_index_bytes = 0;
+        if (m == n && !h->copts.no_bfs_index && dt == DBSPMSPV_F32 && !h->heavy_stage && nnzu > 0 && nnzu <= 0x7FFFFFF0) {
+            uint64_t *wk, *wk_alt;
+            uint32_t *wv, *wv_alt;
+            int32_t *wp;
+            uint2 *wr;
+            float *lightest;
+            const float *weights = static_cast<const float *>(uval);
+            DBS_GET(wk, nnzu); DBS_GET(wk_alt, nnzu); DBS_GET(wv, nnzu); DBS_GET(wv_alt, nnzu);
+            DBS_KEEP(wp, m + 1); DBS_KEEP(wr, nnzu + 4); DBS_KEEP(lightest, m);
+            d.weight_ptr = wp; d.weightrun = wr; d.row_lightest = lightest;
+            k_weightrun_keys<<<grid_for(nnzu), TPB, 0, st>>>(nnzu, ukey, weights, wk, wv);
+            DBS_TRY(sort_pairs(tp, wk, wk_alt, wv, wv_alt, nnzu, SSSP_WEIGHT_BITS + bits_for((uint64_t)m), st));
+            k_rowrun_ptr<<<grid_for(m + 1), TPB, 0, st>>>(m, wk, SSSP_WEIGHT_BITS, (int32_t)nnzu, wp);
+            k_weightrun<<<grid_for(nnzu + 4), TPB, 0, st>>>(nnzu, wv, ukey, weights, wr);
+            k_row_lightest<<<grid_for(m), TPB, 0, st>>>(m, wp, wr, lightest);
+            DBS_CUDA(cudaStreamSynchronize(st));
+            tp.release(wk); tp.release(wk_alt); tp.release(wv); tp.release(wv_alt);
+            h->bfs_index_bytes += nnzu * 8 + ((int64_t)m * 2 + 1) * 4;
+        }
         DBS_CUDA(cudaStreamSynchronize(st));
         tp.release(ukey); tp.release(uval); tp.release(blk_start); tp.release(block_of); tp.release(poff); tp.release(psize);
         tp.release(brow); tp.release(bcol); tp.release(ecount); tp.release(eoff); tp.release(type);
@@ -987,8 +1023,12 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
     }
 
     // row-run index for the pull levels of DB-BFS
-    d.rowrun_ptr = nullptr; d.rowrun_idx = nullptr; d.weightrun = nullptr;
+    d.rowrun_ptr = nullptr; d.rowrun_idx = nullptr; d.col_degree = nullptr;
     if (m == n && !h->copts.no_bfs_index) {
+        uint8_t *cd;
+        DBS_KEEP(cd, (int64_t)d.nb * 16 + 16);
+        d.col_degree = cd;
+        if (d.nb) k_col_degree<<<grid_for((int64_t)d.nb * 16), TPB, 0, st>>>(d.nb, d.csc.colptr, cd);
         uint64_t *rk, *rk_alt;
         uint32_t *rv, *rv_alt;
         DBS_GET(rk, n_entries); DBS_GET(rk_alt, n_entries); DBS_GET(rv, n_entries); DBS_GET(rv_alt, n_entries);
@@ -999,7 +1039,7 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         int32_t *rp;
         DBS_KEEP(rp, m + 1);
         d.rowrun_ptr = rp;
-        k_rowrun_ptr<<<grid_for(m + 1), TPB, 0, st>>>(m, rk, n_entries, rp);
+        k_rowrun_ptr<<<grid_for(m + 1), TPB, 0, st>>>(m, rk, 31, n_entries, rp);
         int32_t n_inline = 0;      // the entries with a payload sort behind every row
         DBS_CUDA(cudaMemcpyAsync(&n_inline, rp + m, 4, cudaMemcpyDeviceToHost, st));
         DBS_CUDA(cudaStreamSynchronize(st));
@@ -1009,19 +1049,7 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         if (n_inline) DBS_CUDA(cudaMemcpyAsync(ri, rv, (size_t)n_inline * 4, cudaMemcpyDeviceToDevice, st));
         DBS_CUDA(cudaStreamSynchronize(st));
         tp.release(rk); tp.release(rk_alt); tp.release(rv); tp.release(rv_alt);
-        h->bfs_index_bytes = ((int64_t)m + 1) * 4 + (int64_t)n_inline * 4;
-        if (d.dtype == DBSPMSPV_F32 && !h->heavy_stage && n_inline) {
-            DBS_GET(rk, n_entries); DBS_GET(rk_alt, n_entries); DBS_GET(rv, n_entries); DBS_GET(rv_alt, n_entries);
-            k_weightrun_keys<<<grid_for(n_entries), TPB, 0, st>>>(n_entries, m, h->block_row, d.csr.idx, d.csr.w, d.csr.aux, rk, rv);
-            DBS_TRY(sort_pairs(tp, rk, rk_alt, rv, rv_alt, (int64_t)n_entries, SSSP_WEIGHT_BITS + bits_for((uint64_t)m), st));
-            uint2 *wr;
-            DBS_KEEP(wr, (int64_t)n_inline + 4);
-            d.weightrun = wr;
-            k_weightrun<<<grid_for((int64_t)n_inline + 4), TPB, 0, st>>>(n_inline, rv, d.csr.idx, d.csr.w, d.csr.aux, wr);
-            DBS_CUDA(cudaStreamSynchronize(st));
-            tp.release(rk); tp.release(rk_alt); tp.release(rv); tp.release(rv_alt);
-            h->bfs_index_bytes += (int64_t)n_inline * 8;
-        }
+        h->bfs_index_bytes += ((int64_t)m + 1) * 4 + (int64_t)n_inline * 4 + (int64_t)d.nb * 16;
     }
 
     // Streaming decode of payload-dominated handles: the chunk table

@@ -254,9 +254,14 @@ struct Device {           // everything the kernels need, passed by value
     // neighbour.  Null when not built.
     const int32_t *rowrun_ptr;
     const uint32_t *rowrun_idx;
-    // The same elements of fp32 handles once more, every row's by weight (column, weight bits), for the large steps of
-    // db_sssp: a row stops at the first weight that cannot improve it.  Ordered by the upper SSSP_WEIGHT_BITS bits of the ordered weight.  Null when not built.
+    const uint8_t *col_degree;     // degree_code of every column's INLINE elements (null when the index is not built)
+    // All elements of fp32 handles once more, every row's by weight (column, weight bits), for the large steps of
+    // db_sssp: a row stops at the first weight that cannot improve it.  Row i is [weight_ptr[i], weight_ptr[i + 1]), ordered by the upper
+    // SSSP_WEIGHT_BITS bits of the ordered weight; row_lightest[i] = its first weight with the lower bits cut off, a bound from below (+infinity: no elements).
+    // (The blocks with a payload too: beside the rows, a warp at a time, 20,000 of them took half of a search on R-MAT scale 20.)  Null when not built.
     const uint2 *weightrun;
+    const int32_t *weight_ptr;
+    const float *row_lightest;
     // Block-CSR view: csr_inl[rb] = first INLINE element of row block rb; its entries with a
     // payload are [csr.ptr[rb], csr_inl[rb]), its INLINE elements [csr_inl[rb], csr.ptr[rb + 1]).
     const int32_t *csr_inl;
@@ -409,6 +414,15 @@ __device__ __forceinline__ void chk_entry(const Device &d, bool csr_view, uint32
 __device__ __forceinline__ uint32_t mask_of(const uint32_t *mask32, int blk) {
     return reinterpret_cast<const uint16_t *>(mask32)[blk];
 }
+
+// A count in eight bits, monotone: exact below 8, then three bits behind the leading one (the eighth below, at most, is cut off).
+__host__ __device__ inline uint32_t degree_code(uint32_t n) {
+    if (n < 8) return n;
+    int e = 3;
+    while (e < 31 && (n >> (e + 1))) ++e;
+    return (uint32_t)(e - 2) * 8 + ((n >> (e - 3)) & 7u);
+}
+__host__ __device__ inline uint32_t degree_of_code(uint32_t c) { return c < 8 ? c : (8u + (c & 7u)) << (c / 8 - 1); }
 
 // Order-preserving map of fp32 to signed words: monotone, and the bits themselves where v >= 0.
 __host__ __device__ inline int ordered_word(int bits) { return bits ^ ((bits >> 31) & 0x7FFFFFFF); }

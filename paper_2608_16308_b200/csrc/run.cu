@@ -2464,10 +2464,10 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     const size_t word_bytes = ((size_t)s.n_words * 32 * sizeof(int) + 255) & ~(size_t)255, bit_bytes = ((size_t)s.n_words * 4 + 255) & ~(size_t)255;
     if (!h->sssp_host && cudaHostAlloc(reinterpret_cast<void **>(&h->sssp_host), 4 * sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess) { h->sssp_host = nullptr; return DBSPMSPV_ERR_ALLOC; }
     // chunks of long rows: a row has more than 4 (SSSP_ROUNDS - 1) elements before any of it is listed
-    const size_t chunk_bytes = ((size_t)d.n_entries / (4 * (SSSP_ROUNDS - 1)) + (size_t)d.n_entries / SSSP_CHUNK + 64) * sizeof(int4);
+    const size_t chunk_bytes = ((size_t)h->nnz / (4 * (SSSP_ROUNDS - 1)) + (size_t)h->nnz / SSSP_CHUNK + 64) * sizeof(int4);
     if (!h->sssp_state) {
-        if (cudaMalloc(&h->sssp_state, word_bytes + 2 * bit_bytes + 256 + chunk_bytes) != cudaSuccess) { h->sssp_state = nullptr; return DBSPMSPV_ERR_ALLOC; }
-        DBS_CUDA(cudaFuncSetAttribute(k_sssp<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SsspShared)));
+        if (cudaMalloc(&h->sssp_state, word_bytes + 2 * bit_bytes + 256 + 2 * SSSP_LIST * sizeof(int32_t) + chunk_bytes) != cudaSuccess) { h->sssp_state = nullptr; return DBSPMSPV_ERR_ALLOC; }
+        DBS_CUDA(cudaFuncSetAttribute(k_sssp<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SSSP_SMEM));
     }
     uint8_t *p = static_cast<uint8_t *>(h->sssp_state);
     s.word = reinterpret_cast<int *>(p);
@@ -2476,7 +2476,8 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     s.ctr = reinterpret_cast<int32_t *>(p + word_bytes + 2 * bit_bytes);
     s.low = s.ctr + 8;
     s.edges = reinterpret_cast<unsigned long long *>(s.ctr + 12);
-    s.chunks = reinterpret_cast<int4 *>(p + word_bytes + 2 * bit_bytes + 256);
+    for (int k = 0; k < 2; ++k) s.list[k] = reinterpret_cast<int32_t *>(p + word_bytes + 2 * bit_bytes + 256) + k * SSSP_LIST;
+    s.chunks = reinterpret_cast<int4 *>(p + word_bytes + 2 * bit_bytes + 256 + 2 * SSSP_LIST * sizeof(int32_t));
     s.report = h->sssp_host;
     Device dev = d;
     int start = 1;
@@ -2485,7 +2486,7 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
         const bool can_pull = DT == DBSPMSPV_PATTERN ? d.rowrun_ptr != nullptr : d.weightrun != nullptr;
         unsigned long long pull_edges = can_pull ? (unsigned long long)(SSSP_PULL_SHARE * (float)d.n_entries) : ~0ull;
         void *args[] = {&dev, &s, &src, &dist, &start, &max_steps, &pull_edges};
-        DBS_CUDA(cudaLaunchCooperativeKernel((void *)k_sssp<DT>, dim3(h->sm_count), dim3(SSSP_CTA), args, sizeof(SsspShared), st));
+        DBS_CUDA(cudaLaunchCooperativeKernel((void *)k_sssp<DT>, dim3(h->sm_count), dim3(SSSP_CTA), args, SSSP_SMEM, st));
         ++h->kernel_launches;
         DBS_CUDA(cudaStreamSynchronize(st));
         made = h->sssp_host[0];

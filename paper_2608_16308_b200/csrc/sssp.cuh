@@ -10,7 +10,8 @@
 //   long     the listed long runs and payload runs, a warp per chunk (only if there are any);
 //   settle   the marked vertices copy their word into the caller's distances -- the values the next
 //            step starts from, which no one lowers meanwhile -- and are counted;
-// with a grid barrier after each.  A step finds the same improvements, distance for distance, as the product did: `word`
+// with a grid barrier after each.  A step that reaches few edges also lists what it marks; a frontier that is listed and short is expanded
+// from its list in one phase, long runs and payload entries included, and settled by one thread block (sssp_expand_list).  A step finds the same improvements, distance for distance, as the product did: `word`
 // holds the minimum over everything seen so far, a vertex is marked iff its word went below the distance it had before the step.
 //
 // What bounds a large step is the gather of one target word per edge.  It goes through L1 first (a stale word is never too small,
@@ -35,17 +36,24 @@ constexpr int SSSP_ILP = 4;                       // warp steps in flight
 // three sources, 559 - 661 / 561 - 670 / 571 - 664 / 575 - 665 us a search, with its vertices in scattered order 354 - 415 / 355 - 415 / 316 - 372 / 353 - 372;
 // scale 17 within 7 % of each other.
 constexpr float SSSP_PULL_SHARE = 0.05f;
-constexpr int SSSP_ROUNDS = 8;                    // rounds of four elements that a lane walks of a row
+// Rounds of four elements that a lane walks of a row.  2 / 4 / 6 / 8: R-MAT scale 20, two sources, 514 / 466 / 451 / 459 and 418 / 384 / 372 / 381 us a search, with
+// its vertices in scattered order 487 / 436 / - / 423.
+constexpr int SSSP_ROUNDS = 8;
 constexpr int SSSP_CHUNK = 512;                   // elements of a listed chunk of a longer row
+// A step whose frontier reaches at most so many edges lists the vertices it marks; a list of at most SSSP_LIST vertices serves the next step.
+// (The bitmap of 2^20 vertices is two rounds of every thread block, whatever it holds: a step of a few vertices took 14 us, 26 with a long run.)
+constexpr int SSSP_LIST = SSSP_CTA;
+constexpr unsigned SSSP_LIST_EDGES = 1u << 17;
 constexpr int SSSP_MAX_STEPS = 1024;              // steps of one launch, at most: a cycle of negative weight ends on the host
 
 struct SsspState {
     int *word;                // n: ordered words of the smallest distance seen
     uint32_t *bits[2];        // frontiers of alternating steps, one bit per vertex
-    int32_t *ctr;             // [0..2] vertices of the frontier, [3..5] listed chunks (sets rotate by step), [6] steps made
+    int32_t *ctr;             // [0..2] vertices of the frontier, [3..5] listed chunks (sets rotate by step), [6] steps made, [18..20] vertices listed by the step
     int *low;                 // smallest word of the frontier, rotating with the counters
-    unsigned long long *edges;   // out-edges of the frontier in INLINE runs, likewise
+    unsigned long long *edges;   // out-edges of the frontier in INLINE runs (to an eighth), likewise
     int4 *chunks;             // {row, first, end, -} of the listed chunks of long rows
+    int32_t *list[2];         // the vertices marked by alternating steps, SSSP_LIST at most
     int32_t *report;          // page-locked host words: steps made, vertices of the frontier that was left
     int32_t n_words;
 };
@@ -62,23 +70,57 @@ struct SsspShared {
     int cnt[SSSP_WARPS], sum[SSSP_WARPS], rec[SSSP_WARPS], base;
 };
 
-// The candidates of up to U targets per lane (target < 0: none).
+// What a pushed step marks: bits, and (list not null) the list of the vertices whose bit it set.
+struct SsspNext {
+    uint32_t *bits;
+    int32_t *list, *n_list;
+    const float *dist;
+};
+
+// The candidates of up to U targets per lane (target < 0: none); called by a whole warp.
 template <int U>
-__device__ __forceinline__ void sssp_relax(const SsspState &s, uint32_t *next, const int (&target)[U], const float (&cand)[U]) {
+__device__ __forceinline__ void sssp_relax(const SsspState &s, const SsspNext &next, const int (&target)[U], const float (&cand)[U]) {
     int seen[U];
+    if (!next.list) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) seen[u] = target[u] >= 0 ? __ldca(s.word + target[u]) : 0;
+        for (int u = 0; u < U; ++u) seen[u] = target[u] >= 0 ? __ldca(s.word + target[u]) : 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (target[u] < 0) continue;
+            const int c = sssp_word(cand[u]);
+            if (c >= seen[u] || c >= __ldcg(s.word + target[u])) continue;
+            if (c < atomicMin(s.word + target[u], c)) atomicOr(next.bits + (target[u] >> 5), 1u << (target[u] & 31));
+        }
+        return;
+    }
+    // few edges: what counts is the chain.  The atomics go out with no look at the words in front, and the one that found the distance
+    // of the step's beginning was the vertex's first.
+    uint32_t fresh = 0u;
+    float was[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (target[u] >= 0) { was[u] = __ldcg(next.dist + target[u]); seen[u] = atomicMin(s.word + target[u], sssp_word(cand[u])); }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        if (target[u] < 0) continue;
-        const int c = sssp_word(cand[u]);
-        if (c >= seen[u] || c >= __ldcg(s.word + target[u])) continue;
-        if (c < atomicMin(s.word + target[u], c)) atomicOr(next + (target[u] >> 5), 1u << (target[u] & 31));
+        if (target[u] < 0 || sssp_word(cand[u]) >= seen[u] || seen[u] != sssp_word(was[u])) continue;
+        atomicOr(next.bits + (target[u] >> 5), 1u << (target[u] & 31));
+        fresh |= 1u << u;
     }
+    if (!__any_sync(FULL, fresh != 0u)) return;
+    const int lane = threadIdx.x & 31, mine = __popc(fresh);
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
+    int base = 0;
+    if (lane == 31) base = atomicAdd(next.n_list, incl);
+    int at = __shfl_sync(FULL, base, 31) + incl - mine;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if ((fresh >> u) & 1u) { if (at < SSSP_LIST) next.list[at] = target[u]; ++at; }
 }
 
 template <int DT>
-__device__ void sssp_expand(const Device &d, const SsspState &s, const float *dist, const uint32_t *F, uint32_t *next, int32_t *n_long, SsspShared &sh) {
+__device__ void sssp_expand(const Device &d, const SsspState &s, const float *dist, const uint32_t *F, const SsspNext &next, int32_t *n_long, SsspShared &sh) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rounds = (s.n_words + SSSP_WORDS * (int)gridDim.x - 1) / (SSSP_WORDS * (int)gridDim.x);
@@ -194,7 +236,7 @@ __device__ void sssp_expand(const Device &d, const SsspState &s, const float *di
 }
 
 template <int DT>
-__device__ void sssp_long(const Device &d, const SsspState &s, uint32_t *next, int n) {
+__device__ void sssp_long(const Device &d, const SsspState &s, const SsspNext &next, int n) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int U = PD_CHUNK / 32;
     const int lane = threadIdx.x & 31;
@@ -236,17 +278,84 @@ __device__ void sssp_long(const Device &d, const SsspState &s, uint32_t *next, i
     }
 }
 
+// A short listed frontier: every thread block lays the vertices' chunks (of their INLINE runs and of the payload entries of their column
+// blocks) end to end, the warps of the grid share them out.
+struct SsspListShared {
+    int pre[SSSP_LIST + 1];                       // chunks before a vertex
+    int vertex[SSSP_LIST], first[SSSP_LIST], deg[SSSP_LIST], pfirst[SSSP_LIST], pdeg[SSSP_LIST];
+    float x[SSSP_LIST];
+    int sum[SSSP_WARPS];
+};
+template <int DT>
+__device__ void sssp_expand_list(const Device &d, const SsspState &s, const float *dist, const int32_t *list, int cnt, const SsspNext &next, SsspListShared &sh) {
+    constexpr bool VAL = DT != DBSPMSPV_PATTERN;
+    constexpr int U = PD_CHUNK / 32;
+    static_assert(PD_PAYLOAD / 2 == U, "one element per lane and step either way");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int j = 0, first = 0, deg = 0, pfirst = 0, pdeg = 0;
+    if (tid < cnt) {
+        j = __ldcg(list + tid);
+        sh.x[tid] = __ldcg(dist + j);
+        column_run(d, j, first, deg);
+        if (d.n_payload) payload_run(d, j >> 4, pfirst, pdeg);
+        if (!DBS_CHK_RANGE(d, first, deg)) deg = 0;
+        if (!DBS_CHK_RANGE(d, pfirst, pdeg)) pdeg = 0;
+    }
+    sh.vertex[tid] = j; sh.first[tid] = first; sh.deg[tid] = deg; sh.pfirst[tid] = pfirst; sh.pdeg[tid] = pdeg;
+    const int mine = (deg + PD_CHUNK - 1) / PD_CHUNK + (pdeg + PD_PAYLOAD - 1) / PD_PAYLOAD;
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
+    if (lane == 31) sh.sum[warp] = incl;
+    __syncthreads();
+    const int v = sh.sum[lane], total = __reduce_add_sync(FULL, v);
+    sh.pre[tid] = incl - mine + __reduce_add_sync(FULL, lane < warp ? v : 0);
+    if (tid == 0) sh.pre[SSSP_LIST] = total;
+    __syncthreads();
+    // (neighbouring chunks on different SMs)
+    for (int c = warp * (int)gridDim.x + (int)blockIdx.x; c < total; c += (int)gridDim.x * SSSP_WARPS) {
+        int o = 0;                                     // the last vertex with at most c chunks before it
+#pragma unroll
+        for (int st = SSSP_LIST / 2; st; st >>= 1) if (sh.pre[o + st] <= c) o += st;
+        const int k = c - sh.pre[o], n_inline = (sh.deg[o] + PD_CHUNK - 1) / PD_CHUNK;
+        const float x = sh.x[o];
+        float cand[U];
+        int target[U];
+        if (k < n_inline) {                            // warp-uniform
+            const int at = k * PD_CHUNK + lane;
+            uint32_t idx[U], w[U], aux[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                idx[u] = PAD_IDX; w[u] = 0u; aux[u] = 0u;
+                if (at + u * 32 < sh.deg[o]) push_entry<VAL>(d, sh.first[o] + at + u * 32, idx[u], w[u], aux[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                target[u] = idx[u] < (1u << TYPE_SHIFT) ? (int)((idx[u] & IDX_MASK) * 16u + (aux[u] >> 4)) : -1;
+                cand[u] = x + Val<DT>::inline_value(w[u]);
+            }
+        } else {
+            const int at = (k - n_inline) * PD_PAYLOAD;
+            bool in[U];
+            uint32_t rb[U];
+            payload_elements<DT, U>(d, sh.pfirst[o] + at, min(PD_PAYLOAD, sh.pdeg[o] - at), sh.vertex[o] & 15, lane, in, cand, rb);
+#pragma unroll
+            for (int u = 0; u < U; ++u) { target[u] = in[u] ? (int)(rb[u] * 16u) + (lane & 15) : -1; cand[u] += x; }
+        }
+        sssp_relax<U>(s, next, target, cand);
+    }
+}
+
 // A row's new best.
 __device__ __forceinline__ void sssp_lower(const SsspState &s, uint32_t *next, int row, int best) {
     if (best < atomicMin(s.word + row, best)) atomicOr(next + (row >> 5), 1u << (row & 31));
 }
-// Elements k0 .. k0 + 3 (k0 a multiple of four) of the runs: columns and weights.
+// Elements k0 .. k0 + 3 (k0 a multiple of four) of the runs: columns and weights, one 32-byte sector in one load.
 template <bool VAL>
 __device__ __forceinline__ void sssp_four(const Device &d, int k0, uint32_t (&col)[4], float (&w)[4]) {
     if (VAL) {
-        const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(d.weightrun + k0)), b = __ldcs(reinterpret_cast<const uint4 *>(d.weightrun + k0 + 2));
-        col[0] = a.x; w[0] = __uint_as_float(a.y); col[1] = a.z; w[1] = __uint_as_float(a.w);
-        col[2] = b.x; w[2] = __uint_as_float(b.y); col[3] = b.z; w[3] = __uint_as_float(b.w);
+        asm volatile("ld.global.cs.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(col[0]), "=f"(w[0]), "=r"(col[1]), "=f"(w[1]), "=r"(col[2]), "=f"(w[2]), "=r"(col[3]), "=f"(w[3]) : "l"(d.weightrun + k0));
     } else {
         const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(d.rowrun_idx + k0));
         const uint32_t v[4] = {a.x, a.y, a.z, a.w};
@@ -266,86 +375,140 @@ __device__ __forceinline__ int sssp_bound(float xmin, float w) {
 // cannot improve it: smallest distance of the frontier + weight >= the row's best.  In the late large steps of an R-MAT search that leaves a
 // seventh of the elements, and a row reached for the first time soon has a best of its own.  Columns outside the
 // frontier improve nothing (their edges were relaxed when they entered it), so they need no test.
-// A lane walks the rows of its own, four elements (one 32-byte sector) a round, row after row, the next row's place fetched meanwhile; what is left of a row that has not
+// Rows that their lightest element (Device::row_lightest) cannot improve are sorted out 64 at a time; the others go to a queue of the warp, from which
+// a lane takes the next one as soon as it has finished a row, four elements (one 32-byte sector) a round.  What is left of a row that has not
 // stopped after SSSP_ROUNDS rounds is listed in chunks, which all warps share out behind a grid barrier (walked by the warp that met them, the
-// hub rows of an R-MAT graph, neighbours all, took one warp 300 us).  Handles of unit weights walk the row-run index.
+// hub rows of an R-MAT graph, neighbours all, took one warp 300 us); of a row of several chunks only those whose first weight can still improve it.
+// Handles of unit weights walk the row-run index.
+// What bounds it: the L1 tag stage, a distance gathered per element (12 M in the first pulled step of R-MAT scale 20, about one a clock and SM), and the rows that come
+// last.  That step took 156 us when a lane walked seven rows of its own and the blocks with a payload followed, a warp at a time, 80 now; the whole search 669, 561 and
+// 532 us from three sources, 443, 364 and 346 now; in scattered order 355 - 466, 303 - 407 now.  A frontier bitmap in shared memory in front of the gathers: 80 -> 103 (L1 is what it
+// takes away); less shared memory by half the columns a round in sssp_expand: within 2 %.
+struct SsspPullShared {
+    int4 queue[SSSP_WARPS][64];       // {row, first, end, best so far} of the rows that wait for a lane
+    int4 longs[SSSP_WARPS][32];                   // {row, first, end, best} of what is left of long rows
+    int cursor;                                   // groups of rows taken by the thread block's warps
+};
+
+// Chunks of the n <= 32 long rows that a warp has met.
+template <bool VAL>
+__device__ __forceinline__ void sssp_list_long(const Device &d, const SsspState &s, const int4 *longs, int n, float xmin, int32_t *n_long, int lane) {
+    const int4 r = lane < n ? longs[lane] : make_int4(0, 0, 0, 0);
+    int chunks = (r.z - r.y + SSSP_CHUNK - 1) / SSSP_CHUNK;
+    if (VAL)
+        for (uint32_t todo = __ballot_sync(FULL, chunks > 1); todo; todo &= todo - 1) {      // the warp looks at 32 chunks of a row at a time
+            const int src = __ffs(todo) - 1, first = __shfl_sync(FULL, r.y, src), all = __shfl_sync(FULL, chunks, src), best = __shfl_sync(FULL, r.w, src);
+            int kept = 0;
+            while (kept < all) {
+                const int c = kept + lane;
+                const bool in = c < all && (c == 0 || sssp_bound<VAL>(xmin, __uint_as_float(d.weightrun[first + c * SSSP_CHUNK].y)) < best);
+                const uint32_t m = __ballot_sync(FULL, in);
+                if (m != FULL) { kept += __ffs(~m) - 1; break; }
+                kept += 32;
+            }
+            if (lane == src) chunks = kept;
+        }
+    int incl = chunks;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
+    int base = 0;
+    if (lane == 31) base = atomicAdd(n_long, incl);
+    int at = __shfl_sync(FULL, base, 31) + incl - chunks;
+    for (int c = 0; c < chunks; ++c) s.chunks[at++] = make_int4(r.x, r.y + c * SSSP_CHUNK, min(r.z, r.y + (c + 1) * SSSP_CHUNK), 0);
+}
+
 template <int DT>
-__device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist, const uint32_t *F, uint32_t *next, int low, int32_t *n_long) {
+__device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist, const uint32_t *F, uint32_t *next, int low, int32_t *n_long, SsspPullShared &sh) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int NONE = 0x7F800000;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gwarp = (int)(blockIdx.x * SSSP_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
     const float xmin = sssp_value(low);
-    auto lower = [&](int row, int best) { sssp_lower(s, next, row, best); };
+    const int32_t *ptr = VAL ? d.weight_ptr : d.rowrun_ptr;
     auto bound = [&](float w) { return sssp_bound<VAL>(xmin, w); };
-    // Up to 32 groups of 32 rows per warp, spread over the matrix: on an R-MAT graph that was not relabelled neighbouring rows are heavy together
-    // (a warp that took eight neighbouring groups of hubs: 136 us where the step takes 60).
-    const int n_groups = (int)((d.n + 31) / 32);
-    for (int64_t g0 = gwarp; g0 < n_groups; g0 += 32ll * nwarps) {
-        int k = 0, row = -1, p = 0, e = 0, have = 0, best = NONE, q_long = 0;      // the row being walked: elements [p, e), from q_long on it is long
-        int k_row = 0, k_n = 0, row_n = -1, p_n = 0, e_n = 0, have_n = 0;                              // the next one
-        uint32_t longm = 0u;
-        int n_chunks = 0;
-        // (row lane + k mod 32 of the k-th group, so that no lane gets the heavy rows of every group)
-        auto fetch = [&]() {
-            row_n = -1;
-            if (k < 32 && g0 + (int64_t)k * nwarps < n_groups) {
-                const int64_t r = (g0 + (int64_t)k * nwarps) * 32 + ((lane + k) & 31);
-                k_n = k;
-                if (r < d.n) { row_n = (int)r; p_n = d.rowrun_ptr[r]; e_n = d.rowrun_ptr[r + 1]; have_n = __ldcg(s.word + r); }
-                else row_n = -2;                       // no such row, but the walk goes on
-                ++k;
-            }
-        };
-        fetch();
-        while (__any_sync(FULL, row >= 0 || row_n != -1)) {
-            if (row < 0 && row_n != -1) {
-                row = row_n; k_row = k_n; p = p_n; e = e_n; have = have_n; best = have_n; q_long = (p & ~3) + SSSP_ROUNDS * 4;
-                if (row < 0 || p >= e) row = -1;
-                fetch();
-            }
-            if (row >= 0) {
-                // (a row that was never reached needs several rounds: two groups at a time until something is found)
-                uint32_t col[8];
-                float w[8], x[8];
-                const int q0 = p & ~3;
-                const bool two = best == NONE && q0 + 4 < e;
-                sssp_four<VAL>(d, q0, reinterpret_cast<uint32_t (&)[4]>(col[0]), reinterpret_cast<float (&)[4]>(w[0]));
-                if (two) sssp_four<VAL>(d, q0 + 4, reinterpret_cast<uint32_t (&)[4]>(col[4]), reinterpret_cast<float (&)[4]>(w[4]));
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    x[j] = __int_as_float(NONE);
-                    if ((j < 4 || two) && q0 + j >= p && q0 + j < e && sssp_word(xmin + w[j]) < best && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
-                }
-                float last = w[3];
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (j < 4 || two) { best = min(best, sssp_word(x[j] + w[j])); last = w[j]; }
-                p = q0 + (two ? 8 : 4);
-                if (p >= e || bound(last) >= best) { if (best < have) lower(row, best); row = -1; }
-                else if (p >= q_long) {     // a long row: what has been found so far counts, the rest below
-                    if (best < have) lower(row, best);
-                    longm |= 1u << k_row;
-                    n_chunks += (e - q_long + SSSP_CHUNK - 1) / SSSP_CHUNK;
-                    row = -1;
-                }
-            }
+    // The thread block's groups of rows, spread over the matrix, are taken by its warps in turn.  (On an R-MAT graph that was not relabelled neighbouring rows are
+    // heavy together, and so are rows with the same low bits: group i of block b is number b + i of the i-th stretch.  Groups dealt out by the elements they hold,
+    // the heaviest first, from a table: no gain there, 5 % longer on graphs in scattered order.)
+    const int n_groups = (int)((d.n + 31) / 32), per_block = (n_groups + (int)gridDim.x - 1) / (int)gridDim.x;
+    if (threadIdx.x == 0) sh.cursor = 0;
+    __syncthreads();
+    int4 *queue = sh.queue[warp], *longs = sh.longs[warp];
+    int row_g = 0, p_g = 0, e_g = 0, have_g = 0;       // a row of the next group
+    float w_g = 1.0f;
+    bool more = true;
+    auto fetch = [&]() {
+        int i = 0;
+        if (lane == 0) i = atomicAdd(&sh.cursor, 1);
+        i = __shfl_sync(FULL, i, 0);
+        more = i < per_block;
+        if (!more) return;
+        const int64_t r = ((int64_t)i * gridDim.x + (blockIdx.x + i) % gridDim.x) * 32 + lane;
+        row_g = (int)r; p_g = 0; e_g = 0; have_g = 0;
+        if (r < d.n) { p_g = ptr[r]; e_g = ptr[r + 1]; have_g = __ldcg(s.word + r); if (VAL) w_g = d.row_lightest[r]; }
+    };
+    fetch();
+    int head = 0, cnt = 0, n_listed = 0;
+    int row = -1, p = 0, e = 0, have = 0, best = NONE, q_long = 0;      // the row being walked: elements [p, e), from q_long on it is long
+    for (;;) {
+        while (more && cnt < 32) {                     // (no more than that: what a warp has claimed no other one can take)
+            const bool pass = p_g < e_g && sssp_word(xmin + w_g) < have_g;
+            const uint32_t m = __ballot_sync(FULL, pass);
+            if (pass) queue[(head + cnt + __popc(m & lt)) & 63] = make_int4(row_g, p_g, e_g, have_g);
+            cnt += __popc(m);
+            fetch();
         }
-        if (__any_sync(FULL, n_chunks > 0)) {
-            int incl = n_chunks;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
-            int base = 0;
-            if (lane == 31) base = atomicAdd(n_long, incl);
-            int at = __shfl_sync(FULL, base, 31) + incl - n_chunks;
-            for (; longm; longm &= longm - 1) {
-                const int kk = __ffs(longm) - 1;
-                const int r = (int)((g0 + (int64_t)kk * nwarps) * 32 + ((lane + kk) & 31)), end = d.rowrun_ptr[r + 1];
-                for (int q = (d.rowrun_ptr[r] & ~3) + SSSP_ROUNDS * 4; q < end; q += SSSP_CHUNK) s.chunks[at++] = make_int4(r, q, min(end, q + SSSP_CHUNK), 0);
+        __syncwarp();
+        const uint32_t idle = __ballot_sync(FULL, row < 0);
+        if (idle == FULL && cnt == 0) break;
+        if (idle && cnt) {
+            const int k = __popc(idle & lt);
+            if (row < 0 && k < cnt) {
+                const int4 q = queue[(head + k) & 63];
+                row = q.x; p = q.y; e = q.z; have = best = q.w; q_long = (p & ~3) + SSSP_ROUNDS * 4;
             }
+            const int took = min(__popc(idle), cnt);
+            head += took; cnt -= took;
+        }
+        bool left = false;                             // a long row: what has been found so far counts, the rest is listed
+        if (row >= 0) {
+            // (a row that was never reached needs several rounds: two groups at a time until something is found)
+            uint32_t col[8];
+            float w[8], x[8];
+            const int q0 = p & ~3;
+            const bool two = best == NONE && q0 + 4 < e;
+            sssp_four<VAL>(d, q0, reinterpret_cast<uint32_t (&)[4]>(col[0]), reinterpret_cast<float (&)[4]>(w[0]));
+            if (two) sssp_four<VAL>(d, q0 + 4, reinterpret_cast<uint32_t (&)[4]>(col[4]), reinterpret_cast<float (&)[4]>(w[4]));
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                x[j] = __int_as_float(NONE);
+                if ((j < 4 || two) && q0 + j >= p && q0 + j < e && sssp_word(xmin + w[j]) < best && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
+            }
+            float last = w[3];
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (j < 4 || two) { best = min(best, sssp_word(x[j] + w[j])); last = w[j]; }
+            p = q0 + (two ? 8 : 4);
+            const bool over = p >= e || bound(last) >= best;
+            left = !over && p >= q_long;
+            if ((over || left) && best < have) {
+                // (below the best that the step found in place: the row is marked whoever else lowers it, and nobody waits for the replies)
+                atomicMin(s.word + row, best);
+                atomicOr(next + (row >> 5), 1u << (row & 31));
+            }
+            if (over) row = -1;
+        }
+        const uint32_t lm = __ballot_sync(FULL, left);
+        if (lm) {
+            if (n_listed + __popc(lm) > 32) { __syncwarp(); sssp_list_long<VAL>(d, s, longs, n_listed, xmin, n_long, lane); n_listed = 0; __syncwarp(); }
+            if (left) { longs[n_listed + __popc(lm & lt)] = make_int4(row, p, e, best); row = -1; }
+            n_listed += __popc(lm);
         }
     }
-    // entries with a payload: one block per warp at a time, columns of the frontier only (the blocks sit where a power-law graph is dense, among
+    __syncwarp();
+    if (n_listed) sssp_list_long<VAL>(d, s, longs, n_listed, xmin, n_long, lane);
+    if (VAL) return;
+    // entries with a payload (unit weights): one block per warp at a time, columns of the frontier only (the blocks sit where a power-law graph is dense, among
     // the vertices that settle first: late large steps skip most of them); the next entry is fetched meanwhile
     struct Entry { uint32_t idx, w, aux; int rb; };
     auto entry = [&](int pos) {
@@ -369,52 +532,65 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
         if (!xm) continue;                                                               // warp-uniform
         block_rows_min_warp<DT>(type, e.w, e.aux, xm, dist + (size_t)cb * 16, d.payload, lane, [&](int r, uint32_t key) {
             const int c = sssp_word(minplus_value(key)), row = e.rb * 16 + r;
-            if (c < __ldcg(s.word + row)) lower(row, c);
+            if (c < __ldcg(s.word + row)) sssp_lower(s, next, row, c);
         });
     }
 }
 
-// The listed chunks of long rows, a warp per chunk, four elements per lane and step.
+// The listed chunks of long rows, a warp per chunk, four elements per lane and step.  The next chunk's record, best and first elements are
+// fetched while this one's distances arrive.
 template <int DT>
 __device__ void sssp_pull_long(const Device &d, const SsspState &s, const float *dist, uint32_t *next, int low, int n) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     const int lane = threadIdx.x & 31;
     const int gwarp = (int)(blockIdx.x * SSSP_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
     const float xmin = sssp_value(low);
-    int4 ahead = gwarp < n ? __ldcg(s.chunks + gwarp) : make_int4(0, 0, 0, 0);
+    auto record = [&](int i) { return i < n ? __ldcg(s.chunks + i) : make_int4(0, 0, 0, 0); };
+    int4 c = record(gwarp), ahead = record(gwarp + nwarps);
+    uint32_t col[4] = {0u, 0u, 0u, 0u};
+    float w[4] = {0.f, 0.f, 0.f, 0.f};
+    int had = 0;
+    auto first = [&](const int4 &r) {
+        const int k0 = (r.y & ~3) + 4 * lane;
+        if (k0 < r.z) { had = __ldcg(s.word + r.x); sssp_four<VAL>(d, k0, col, w); }
+    };
+    first(c);
     for (int i = gwarp; i < n; i += nwarps) {
-        const int4 c = ahead;
-        if (i + nwarps < n) ahead = __ldcg(s.chunks + i + nwarps);
-        const int had = __ldcg(s.word + c.x);
+        had = __shfl_sync(FULL, had, 0);               // (lane 0 of a chunk always has elements)
+        const int start = had, row = c.x, p = c.y, e = c.z;
         int now = had;
-        uint32_t col[4], col_n[4];
-        float w[4], w_n[4];
-        const int k0 = c.y + 4 * lane;
-        if (k0 < c.z) sssp_four<VAL>(d, k0, col, w);
-        for (int q = k0; q - 4 * lane < c.z; q += 128) {
-            if (q + 128 < c.z) sssp_four<VAL>(d, q + 128, col_n, w_n);
-            float x[4];
-            int mine = now;
-            bool over = true;
-            if (q < c.z) {
+        for (int q = (p & ~3) + 4 * lane;; q += 128) {
+            float x[4], wq[4];
+            const bool in = q < e, more = q - 4 * lane + 128 < e;             // (warp-uniform: the chunk goes on)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    x[j] = __int_as_float(0x7F800000);
-                    if (q + j < c.z && sssp_word(xmin + w[j]) < now && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) mine = min(mine, sssp_word(x[j] + w[j]));
+            for (int j = 0; j < 4; ++j) {
+                x[j] = __int_as_float(0x7F800000);
+                wq[j] = w[j];
+                if (in && q + j >= p && q + j < e && sssp_word(xmin + w[j]) < now && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
             }
-            now = __reduce_min_sync(FULL, mine);
-            if (q < c.z) over = sssp_bound<VAL>(xmin, w[3]) >= now;
-            if (__shfl_sync(FULL, (int)over, 31)) break;               // (the last lane's weight is the largest of the step; past the end: done)
+            if (more) { if (q + 128 < e) sssp_four<VAL>(d, q + 128, col, w); }
+            else { c = ahead; ahead = record(i + 2 * nwarps); first(c); }
+            int mine = now;
+            if (in)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) { col[j] = col_n[j]; w[j] = w_n[j]; }
+                for (int j = 0; j < 4; ++j) mine = min(mine, sssp_word(x[j] + wq[j]));
+            now = __reduce_min_sync(FULL, mine);
+            if (!more) break;
+            const bool over = sssp_bound<VAL>(xmin, wq[3]) >= now;
+            if (__shfl_sync(FULL, (int)over, 31)) {    // (the last lane's weight is the largest of the step)
+                c = ahead; ahead = record(i + 2 * nwarps); first(c);
+                break;
+            }
         }
-        if (lane == 0 && now < had) sssp_lower(s, next, c.x, now);
+        if (lane == 0 && now < start) {
+            atomicMin(s.word + row, now);
+            atomicOr(next + (row >> 5), 1u << (row & 31));
+        }
     }
 }
 
+constexpr int SSSP_SMEM = (int)(sizeof(SsspShared) > sizeof(SsspPullShared) ? sizeof(SsspShared) : sizeof(SsspPullShared));
+static_assert(sizeof(SsspListShared) <= sizeof(SsspShared), "the phases share one allocation");
 template <int DT>
 __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int32_t src, float *dist, int start, int max_steps, unsigned long long pull_edges) {
     namespace cg = cooperative_groups;
@@ -427,23 +603,38 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int
         for (int64_t v = tid; v < n; v += nthreads) { s.word[v] = v == src ? 0 : 0x7F800000; dist[v] = v == src ? 0.0f : __int_as_float(0x7F800000); }
         for (int k = tid; k < s.n_words; k += nthreads) { s.bits[0][k] = k == src >> 5 ? 1u << (src & 31) : 0u; s.bits[1][k] = 0u; }
         if (tid < 6) s.ctr[tid] = tid == 0 ? 1 : 0;
-        if (tid == 6) { s.ctr[6] = 0; for (int k = 0; k < 3; ++k) { s.low[k] = k == 0 ? 0 : 0x7F800000; s.edges[k] = 0ull; } }
+        if (tid == 6) {
+            int first, deg;
+            column_run(d, src, first, deg);
+            s.ctr[6] = 0;
+            for (int k = 0; k < 3; ++k) { s.low[k] = k == 0 ? 0 : 0x7F800000; s.edges[k] = k == 0 ? (unsigned long long)deg : 0ull; s.ctr[18 + k] = 0; }
+            s.list[1][0] = src;
+        }
         grid.sync();
     }
     int t = s.ctr[6];
-    for (int made = 0; made < max_steps && __ldcg(s.ctr + t % 3) != 0; ++made, ++t) {
-        uint32_t *F = s.bits[t & 1], *next = s.bits[(t + 1) & 1];
-        int32_t *n_long = s.ctr + 3 + t % 3;
-        if (tid == 0) s.ctr[3 + (t + 1) % 3] = 0;      // (its last reader was step t - 2)
-        if (__ldcg(s.edges + t % 3) > pull_edges) {    // grid-uniform
+    bool listed = start != 0;                          // the frontier is in list[(t + 1) & 1]
+    for (int made = 0; made < max_steps; ++made, ++t) {
+        const int cnt = __ldcg(s.ctr + t % 3);         // grid-uniform, as all that is decided from it
+        if (cnt == 0) break;
+        uint32_t *F = s.bits[t & 1];
+        const unsigned long long edges_now = __ldcg(s.edges + t % 3);
+        int32_t *n_long = s.ctr + 3 + t % 3, *n_list = s.ctr + 18 + t % 3;
+        const bool pulled = edges_now > pull_edges, lists = !pulled && edges_now <= SSSP_LIST_EDGES;
+        const SsspNext next{s.bits[(t + 1) & 1], lists ? s.list[t & 1] : nullptr, n_list, dist};
+        if (tid == 0) { s.ctr[3 + (t + 1) % 3] = 0; s.ctr[18 + (t + 1) % 3] = 0; }      // (their last reader was step t - 2)
+        if (pulled) {
             const int low = __ldcg(s.low + t % 3);
-            sssp_pull<DT>(d, s, dist, F, next, low, n_long);
+            sssp_pull<DT>(d, s, dist, F, next.bits, low, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn));
             grid.sync();
             const int n = __ldcg(n_long);
             if (n > 0) {                               // grid-uniform
-                sssp_pull_long<DT>(d, s, dist, next, low, n);
+                sssp_pull_long<DT>(d, s, dist, next.bits, low, n);
                 grid.sync();
             }
+        } else if (listed) {
+            sssp_expand_list<DT>(d, s, dist, s.list[(t + 1) & 1], cnt, next, *reinterpret_cast<SsspListShared *>(s_dyn));
+            grid.sync();
         } else {
             sssp_expand<DT>(d, s, dist, F, next, n_long, sh);
             grid.sync();
@@ -454,33 +645,51 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int
             }
         }
         if (tid == 0) { s.ctr[(t + 2) % 3] = 0; s.low[(t + 2) % 3] = 0x7F800000; s.edges[(t + 2) % 3] = 0ull; }
+        const bool was_listed = listed;
+        const int n_marked = lists ? __ldcg(n_list) : 0;
+        listed = lists && n_marked <= SSSP_LIST;
         int found = 0, low = 0x7F800000;
         unsigned long long edges = 0;
-        const int gwarp = tid >> 5, nwarps = nthreads >> 5;
-        for (int w0 = gwarp; w0 < s.n_words; w0 += 8 * nwarps) {
-            uint32_t b[8];
-            int v[8], deg[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) { const int w = w0 + q * nwarps; b[q] = w < s.n_words ? __ldcg(next + w) : 0u; }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                v[q] = 0x7F800000; deg[q] = 0;
-                if ((b[q] >> lane) & 1u) {
-                    const int j = (w0 + q * nwarps) * 32 + lane;
-                    v[q] = __ldcg(s.word + j);
-                    const int32_t *cp = d.csc.colptr + 17 * (j >> 4) + (j & 15);
-                    deg[q] = cp[1] - cp[0];
+        if (listed) {                                  // one thread block settles, the others clear the old frontier if it is not listed
+            if (!was_listed) for (int k = tid; k < s.n_words; k += nthreads) F[k] = 0u;
+            if (blockIdx.x == 0) {
+                if (was_listed && (int)threadIdx.x < cnt) F[__ldcg(s.list[(t + 1) & 1] + threadIdx.x) >> 5] = 0u;
+                if ((int)threadIdx.x < n_marked) {
+                    const int j = __ldcg(s.list[t & 1] + threadIdx.x);
+                    low = __ldcg(s.word + j);
+                    int first, deg;
+                    column_run(d, j, first, deg);
+                    edges = (unsigned)deg;
+                    dist[j] = sssp_value(low);
                 }
             }
+        } else {
+            const int gwarp = tid >> 5, nwarps = nthreads >> 5;
+            for (int w0 = gwarp; w0 < s.n_words; w0 += 8 * nwarps) {
+                uint32_t b[8];
+                int v[8], deg[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int w = w0 + q * nwarps;
-                if (w >= s.n_words) break;
-                if ((b[q] >> lane) & 1u) dist[(int64_t)w * 32 + lane] = sssp_value(v[q]);
-                if (lane == 0) F[w] = 0u;
-                found += __popc(b[q]);
-                low = min(low, v[q]);
-                edges += (unsigned)deg[q];
+                for (int q = 0; q < 8; ++q) { const int w = w0 + q * nwarps; b[q] = w < s.n_words ? __ldcg(next.bits + w) : 0u; }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    v[q] = 0x7F800000; deg[q] = 0;
+                    if ((b[q] >> lane) & 1u) {
+                        const int j = (w0 + q * nwarps) * 32 + lane;
+                        v[q] = __ldcg(s.word + j);
+                        if (d.col_degree) deg[q] = (int)d.col_degree[j];      // (a byte each: with the column pointers the pass took a third longer)
+                        else { int first; column_run(d, j, first, deg[q]); deg[q] = (int)degree_code((uint32_t)deg[q]); }
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int w = w0 + q * nwarps;
+                    if (w >= s.n_words) break;
+                    if ((b[q] >> lane) & 1u) dist[(int64_t)w * 32 + lane] = sssp_value(v[q]);
+                    if (lane == 0) F[w] = 0u;
+                    found += __popc(b[q]);
+                    low = min(low, v[q]);
+                    edges += degree_of_code((uint32_t)deg[q]);
+                }
             }
         }
         low = __reduce_min_sync(FULL, low);
@@ -494,7 +703,9 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int
             edges = sh.edges[lane];
 #pragma unroll
             for (int o = 16; o; o >>= 1) edges += __shfl_xor_sync(FULL, edges, o);
-            if (lane == 0 && found) { atomicAdd(s.ctr + (t + 1) % 3, found); atomicMin(s.low + (t + 1) % 3, low); atomicAdd(s.edges + (t + 1) % 3, edges); }
+            if (listed) {
+                if (lane == 0 && blockIdx.x == 0) { s.ctr[(t + 1) % 3] = n_marked; s.low[(t + 1) % 3] = low; s.edges[(t + 1) % 3] = edges; }
+            } else if (lane == 0 && found) { atomicAdd(s.ctr + (t + 1) % 3, found); atomicMin(s.low + (t + 1) % 3, low); atomicAdd(s.edges + (t + 1) % 3, edges); }
         }
         grid.sync();
     }

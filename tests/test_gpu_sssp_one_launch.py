@@ -76,3 +76,62 @@ def test_rows_that_begin_with_extreme_weights(low):
         assert np.array_equal(dist.cpu().numpy(), want)
     assert np.isfinite(want[1501:1601]).sum() > 90
     h.close()
+
+
+@pytest.mark.parametrize("fan", [1, 1023, 1024, 1025, 6000])
+@pytest.mark.parametrize("dtype", [B.F32, B.PATTERN])
+def test_listed_and_unlisted_frontiers(fan, dtype):
+    """Frontiers at the length up to which a step's marked vertices are kept as a list, in turn with longer and shorter ones: the source
+    reaches `fan` vertices, they reach a third of that and one vertex with a long column, then single vertices; a part that is not reached keeps the
+    pushed steps a small share of the elements.  (Dyadic weights: every path sum is exact.)"""
+    n = 40011
+    rng = np.random.default_rng(fan)
+    a = 16 + np.arange(fan)
+    b = 8000 + np.arange(max(1, fan // 3))
+    u = [np.full(fan, 3), a, np.full(1, a[0]), np.full(700, 20000), [20001, 20002, 20003], rng.integers(22000, n, 300000)]
+    v = [a, b[rng.integers(0, b.size, fan)], [20000], 20001 + np.arange(700), [21000, 21001, 21002], rng.integers(22000, n, 300000)]
+    keys = wl.sorted_unique(np.concatenate(v).astype(np.int64) * n + np.concatenate(u))
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    val = np.ones(keys.size, np.float32) if dtype == B.PATTERN else (1 + rng.integers(0, 63, keys.size)).astype(np.float32) / 8.0
+    csr = wl.CSR(n, n, ptr, idx, val)
+    h, A = Handle(csr, dtype), ref_matrix(csr)
+    dist = torch.empty(n, dtype=torch.float32, device="cuda")
+    for src in (3, 20000, int(a[-1])):
+        steps = []
+        for path in (B.PATH_AUTO, B.PATH_PUSH, B.PATH_AUTO):
+            h.set_opts(force_path=path)
+            steps.append(B.db_sssp(h.h, src, dist))
+            torch.cuda.synchronize()
+            assert np.array_equal(dist.cpu().numpy().astype(np.float64), oracle.ref_sssp(A, src))
+        assert steps[0] == steps[1] == steps[2]
+    h.close()
+
+
+@pytest.mark.parametrize("length", [1, 3, 4, 31, 32, 33, 63, 64, 65, 543, 545, 1100, 2600])
+def test_rows_of_a_pulled_step(length):
+    """Rows at the lengths where a lane hands a row over and where what is left of it is one chunk or several, dense blocks among their elements; the
+    vertices they lie behind are reached in one step, so that the next one is pulled, and once more with better distances a step later."""
+    n = 6007
+    rng = np.random.default_rng(length)
+    src, late = 0, 1
+    mid = np.arange(32, 32 + 2700)                         # reached from the source; half of them again, for less, by way of `late`
+    rows = [mid, [late], mid[::2], np.repeat(np.arange(3000, 3200), length), np.repeat(np.arange(3200, 3232), 32)]
+    cols = [np.zeros(mid.size), [src], np.full(mid[::2].size, late), np.concatenate([rng.choice(mid, length, replace=False) for _ in range(200)]),
+            np.tile(np.arange(32, 64), 32)]
+    key = np.concatenate(rows).astype(np.int64) * n + np.concatenate(cols).astype(np.int64)
+    keys = wl.sorted_unique(key)
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    val = (8 + rng.integers(0, 500, keys.size)).astype(np.float32) / 8.0
+    r = np.repeat(np.arange(n), np.diff(ptr))
+    val[(r == late) | (idx == late)] = 1.0 / 8.0
+    csr = wl.CSR(n, n, ptr, idx, val)
+    h, A = Handle(csr, B.F32), ref_matrix(csr)
+    dist = torch.empty(n, dtype=torch.float32, device="cuda")
+    steps = []
+    for path in (B.PATH_AUTO, B.PATH_PUSH):
+        h.set_opts(force_path=path)
+        steps.append(B.db_sssp(h.h, src, dist))
+        torch.cuda.synchronize()
+        assert np.array_equal(dist.cpu().numpy().astype(np.float64), oracle.ref_sssp(A, src))
+    assert steps[0] == steps[1]
+    h.close()
