@@ -64,7 +64,7 @@ __device__ __forceinline__ void append_words(int word, int32_t *list, int32_t *c
 struct NextLevel {
     uint32_t *N;                 // frontier masks
     int32_t *words, *n_words;    // list of the words that became nonzero
-    int32_t *n_blocks, *n_tasks, *n_hubs;
+    int32_t *n_blocks, *n_tasks, *n_hubs, *n_edges;
     int4 *hubs;
     uint2 *tasks;
     bool emit;                   // the worklist is written by this level itself
@@ -77,7 +77,8 @@ struct NextLevel {
 constexpr int BFS_EMIT_STEPS = 16;
 // Up to this many warp steps the bookkeeping is the claiming lanes': a second atomic per vertex found, but neither a pass nor a barrier
 // behind the level.  Larger levels leave it to a pass over the words that became nonzero, one update for up to 32 vertices: levels of 2^22
-// vertices that reach most of them through a few thousand hubs took 78 - 150 us with an atomic each, 59 - 116 with the pass.  (Limit 512:
+// vertices that reach most of them through a few thousand hubs took 78 - 150 us with an atomic each, 59 - 116 with the pass, and 37 - 71 since the pass writes
+// the levels too and nobody waits for an atomic's reply.  (Limit 512:
 // levels of a few thousand steps 2 - 5 us longer; 4096 to 65536: no difference on graphs of 17,000 to 2^22 vertices.)
 constexpr int BFS_MARK_STEPS = 16384;
 
@@ -98,9 +99,13 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
     const int n_tasks = n_recs + table.total;                    // task records, then the steps of the hub runs
     auto item = [&](int i) { return worklist_item(tasks, n_recs, table, i); };
     const uint2 none = make_uint2(0u, 0u);
-    int found = 0, blocks = 0;
+    int found = 0, blocks = 0, edges = 0;
     // claims the rows `hit` of row block `brow` (called by a full warp; hit = 0: nothing in this lane)
     auto publish = [&](int brow, uint32_t hit) {
+        if (!MARK) {                                   // (nobody waits for a reply: levels, list and counts are the pass behind the level)
+            if (hit) atomicOr(&nx.N[brow >> 1], hit << ((brow & 1) * 16));
+            return;
+        }
         uint32_t old = 0, fresh = 0;
         const int sh = (brow & 1) * 16;
         if (hit) {
@@ -115,6 +120,7 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
                 atomicOr(&d.ws.visited32[brow >> 1], fresh << sh);
                 found += __popc(fresh);
                 blocks += newly;
+                if (d.col_degree) for (uint32_t f = fresh; f; f &= f - 1) edges += (int)degree_of_code(d.col_degree[brow * 16 + __ffs(f) - 1]);
             }
         }
         append_words(fresh && !old ? brow >> 1 : -1, nx.words, nx.n_words, lane);
@@ -211,7 +217,8 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
     }
     found = __reduce_add_sync(FULL, found);
     blocks = __reduce_add_sync(FULL, blocks);
-    if (MARK && lane == 0 && found) { atomicAdd(&d.ws.ctr->bfs_reached, found); atomicAdd(nx.n_blocks, blocks); }
+    edges = __reduce_add_sync(FULL, edges);
+    if (MARK && lane == 0 && found) { atomicAdd(&d.ws.ctr->bfs_reached, found); atomicAdd(nx.n_blocks, blocks); atomicAdd(nx.n_edges, edges); }
 }
 
 // Boolean pull: one warp per row-block segment (a segment has at most MAX_SEG_ENTRIES = 4 x 32
@@ -325,6 +332,8 @@ __device__ void bfs_pull(const Device &d, const Scope &sc, const uint32_t *F, ui
 }
 
 // Boolean pull over the row-run index (square matrices, unless the index was switched off).
+// What bounds it is DRAM: a sector per row that is not settled by its first element (R-MAT scale 22, a frontier of 160 K vector blocks: 38 us without the
+// look at the first elements, 26 with it; in scattered order, where the runs used to begin anywhere, 40 -> 22), and the whole runs of rows with no frontier neighbour.
 // Entries with a payload are evaluated first, from the per-row-block position list, and a row
 // block is left as soon as each of its wanted rows has a parent; then every row that is still
 // wanted walks its own INLINE run and stops at its first frontier neighbour -- the early exit of
@@ -351,7 +360,8 @@ template <int DT>
 __device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *N, uint32_t *Z, int32_t *nz_out, int32_t *words_out,
                                 int32_t *nwords_out, int32_t *levels, int depth, bool wide, uint32_t *s_need) {
     const int lane = threadIdx.x & 31;
-    const int gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    // (neighbouring words on different SMs: on an R-MAT graph that was not relabelled they are heavy together)
+    const int gwarp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const int n_words = (d.mb + 1) / 2;
     constexpr uint32_t NONE = 0xFFFFFFFFu;          // no entry: local column 31 never matches a 16-bit mask
@@ -412,6 +422,34 @@ __device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *N, u
                 }
                 if ((fk >> lane) & 1u) levels[(size_t)(w0 + k) * 32 + lane] = depth;
                 if (lane == k) found |= fk;
+            }
+        }
+        // The first column of every wanted row's run, the one with the highest degree, from an array of their own: lane = row, eight words at a time.
+        // Under a frontier that holds the hubs most rows end here, with neither their run's place nor its first sector fetched.
+        {
+            constexpr int U = 8;
+            const uint32_t wanted = need & ~found;
+            uint32_t todo = __ballot_sync(FULL, wanted != 0u);
+            while (todo) {
+                int k[U];
+                uint32_t v[U], xm[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    k[u] = __ffs(todo) - 1;                   // (-1: no more words)
+                    todo &= todo - 1;
+                    const uint32_t word = __shfl_sync(FULL, wanted, k[u] & 31);
+                    v[u] = k[u] >= 0 && ((word >> lane) & 1u) ? __ldcs(d.row_first + (size_t)(w0 + k[u]) * 32 + lane) : NONE;
+                    if (v[u] != NONE && !DBS_CHK_INDEX(d, v[u] & IDX_MASK, d.nb)) v[u] = NONE;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) xm[u] = v[u] != NONE ? mask_of(F, v[u] & IDX_MASK) : 0u;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool got = (xm[u] >> (v[u] >> 27)) & 1u;
+                    const uint32_t fk = __ballot_sync(FULL, got);
+                    if (got) levels[(size_t)(w0 + k[u]) * 32 + lane] = depth;
+                    if (lane == k[u]) found |= fk;
+                }
             }
         }
         // rows: bit k of `mine` = row (lane + k) mod 32 of word w0 + k is still wanted.  (The rotation matters where
@@ -554,11 +592,13 @@ __device__ void bfs_worklist(const Device &d, const Scope &sc, const uint32_t *F
 // worklist is short: a frontier of a few hub vertices fills few vector blocks but owns a good
 // part of all stored elements, and a pull, which stops every row at its first frontier
 // neighbour, reads less than the push of all those elements would (edge_frac = the share of
-// the view's entries above which the push is given up; 0 = block ratio only).  `steps`: warp steps of the worklist.
-__device__ __forceinline__ int bfs_level_path(const Device &d, int n_nzblk, int steps, float th3, float edge_frac, int force_path) {
+// the view's entries above which the push is given up; 0 = block ratio only).  `steps`: warp steps of the worklist;
+// `edges`: elements it would hold at least, where they were counted (such a frontier's worklist is not built at all: a few thousand hubs make hundreds of
+// thousands of records, 10 us on 2^22 vertices).
+__device__ __forceinline__ int bfs_level_path(const Device &d, int n_nzblk, int steps, int edges, float th3, float edge_frac, int force_path) {
     int path = bfs_path(n_nzblk, d.nb, th3, force_path);
     if (path == DBSPMSPV_PATH_PUSH && force_path == DBSPMSPV_PATH_AUTO && edge_frac > 0.f && d.rowrun_ptr != nullptr &&
-        (float)steps * (float)PUSH_CHUNK > edge_frac * (float)d.n_entries) path = DBSPMSPV_PATH_PULL;
+        ((float)edges > edge_frac * (float)d.n_entries || (float)steps * (float)PUSH_CHUNK > edge_frac * (float)d.n_entries)) path = DBSPMSPV_PATH_PULL;
     return path;
 }
 
@@ -586,13 +626,14 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
     const int n_hubs = min(ctr->bfs_hubs[cur], HUB_CAP);
     int steps = n_tasks;                                // of the worklist: the task records plus the steps of the listed hub runs
     for (int k = 0; k < n_hubs; ++k) steps += (d.ws.hubs[cur * HUB_CAP + k].z + PUSH_CHUNK - 1) / PUSH_CHUNK;
-    const int path = bfs_level_path(d, n_nzblk, steps, th3, edge_frac, force_path);
+    const int path = bfs_level_path(d, n_nzblk, steps, ctr->bfs_edges[cur], th3, edge_frac, force_path);
     // counters that come into use at the next level are reset now: nobody reads or writes them
     // during this one (the previous level was their last reader, behind a barrier)
     if (sc.tid == 0) {
         ctr->bfs_cnt[spare][0] = 0;
         ctr->bfs_cnt[spare][1] = 0;
         ctr->bfs_hubs[spare] = 0;
+        ctr->bfs_edges[spare] = 0;
         ctr->bfs_nwords[q_next] = 0;
         if (depth <= DBSPMSPV_MAX_BFS_LEVELS_RECORDED) {
             ctr->bfs_level_path[depth - 1] = path;
@@ -613,25 +654,36 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
         uint2 *const tasks = lv & 1 ? d.ws.tasks2 : d.ws.tasks, *const tasks_next = lv & 1 ? d.ws.tasks : d.ws.tasks2;
         const bool mark = steps <= BFS_MARK_STEPS;
         const bool emit = mark && n_hubs == 0 && n_tasks <= BFS_EMIT_STEPS && bfs_path(min(PUSH_CHUNK * n_tasks, d.nb), d.nb, th3, force_path) == DBSPMSPV_PATH_PUSH;
-        const NextLevel nx{N, words_out, &ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][0], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], hubs_next, tasks_next, emit};
+        const NextLevel nx{N, words_out, &ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][0], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], &ctr->bfs_edges[nxt], hubs_next, tasks_next, emit};
         if (mark) bfs_push<DT, true>(d, sc, F, tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
         else bfs_push<DT, false>(d, sc, F, tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
         grid.sync();
         if (emit) return;                              // (the next level's worklist is there)
         if (!mark) {
-            // visited is updated, the nonempty blocks and the vertices found are counted: over the words that became nonzero
-            const int n_listed = ctr->bfs_nwords[q_out];
-            int found = 0, nz = 0;
-            for (int i = sc.tid; i < n_listed; i += sc.nthreads) {
-                const int k = words_out[i];
-                const uint32_t nm = N[k];
-                d.ws.visited32[k] |= nm;
-                found += __popc(nm);
-                nz += ((nm & 0xFFFFu) != 0) + ((nm >> 16) != 0);
+            // levels, visited, the list of nonzero words and the counts: a warp takes 32 words, then writes the levels of one nonzero word after the other, lane = row
+            int found = 0, nz = 0, edges = 0;
+            for (int k0 = sc.tid & ~31; k0 < n_words; k0 += sc.nthreads) {
+                const int k = k0 + lane;
+                const uint32_t nm = k < n_words ? __ldcg(N + k) : 0u;
+                if (nm) {
+                    d.ws.visited32[k] |= nm;
+                    found += __popc(nm);
+                    nz += ((nm & 0xFFFFu) != 0) + ((nm >> 16) != 0);
+                }
+                append_words(nm ? k : -1, words_out, &ctr->bfs_nwords[q_out], lane);
+                for (uint32_t todo = __ballot_sync(FULL, nm != 0u); todo; todo &= todo - 1) {
+                    const int q = __ffs(todo) - 1;
+                    if ((__shfl_sync(FULL, nm, q) >> lane) & 1u) {
+                        const size_t row = (size_t)(k0 + q) * 32 + lane;
+                        levels[row] = depth;
+                        if (d.col_degree) edges += (int)degree_of_code(d.col_degree[row]);
+                    }
+                }
             }
             found = __reduce_add_sync(FULL, found);
             nz = __reduce_add_sync(FULL, nz);
-            if (lane == 0 && found) { atomicAdd(&ctr->bfs_reached, found); atomicAdd(&ctr->bfs_cnt[nxt][0], nz); }
+            edges = __reduce_add_sync(FULL, edges);
+            if (lane == 0 && found) { atomicAdd(&ctr->bfs_reached, found); atomicAdd(&ctr->bfs_cnt[nxt][0], nz); atomicAdd(&ctr->bfs_edges[nxt], edges); }
             grid.sync();
         }
     } else {
@@ -662,7 +714,7 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
     // the push worklist is rebuilt if the block ratio of the next level asks for a push (the
     // selector's input is known now; the level may still turn to a pull when the list is long)
     const int next_n = ctr->bfs_cnt[nxt][0];
-    if (next_n && bfs_path(next_n, d.nb, th3, force_path) == DBSPMSPV_PATH_PUSH) {
+    if (next_n && bfs_level_path(d, next_n, 0, ctr->bfs_edges[nxt], th3, edge_frac, force_path) == DBSPMSPV_PATH_PUSH) {
         bfs_worklist(d, sc, N, words_out, ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], hubs_next, lv & 1 ? d.ws.tasks : d.ws.tasks2);
         grid.sync();
     }
@@ -706,7 +758,7 @@ __global__ void __launch_bounds__(BFS_CTA) k_bfs(Device d, int32_t src, int32_t 
     }
     if (blockIdx.x == 0 && threadIdx.x < 32) {
         if (lane == 0) {
-            for (int k = 0; k < 3; ++k) { ctr->bfs_cnt[k][0] = 0; ctr->bfs_cnt[k][1] = 0; ctr->bfs_hubs[k] = 0; }
+            for (int k = 0; k < 3; ++k) { ctr->bfs_cnt[k][0] = 0; ctr->bfs_cnt[k][1] = 0; ctr->bfs_hubs[k] = 0; ctr->bfs_edges[k] = 0; }
             for (int k = 0; k < 4; ++k) ctr->bfs_nwords[k] = k == 3;         // (the source's mask word is list 3 = "produced by level -1")
             ctr->bfs_reached = 1;
             d.ws.bfs_words[(size_t)3 * d.ws.bfs_words_stride] = src_word;

@@ -534,17 +534,23 @@ __global__ void k_col_degree(int32_t nb, const int32_t *colptr, uint8_t *code) {
     const int32_t *cp = colptr + 17 * (j >> 4) + (j & 15);
     code[j] = (uint8_t)degree_code((uint32_t)(cp[1] - cp[0]));
 }
-// ---- row-run index of the INLINE elements (DB-BFS pull levels)
+// ---- row-run index of the INLINE elements (DB-BFS pull levels): by row, the columns of the highest degree first
 __global__ void k_rowrun_keys(int32_t n_entries, int64_t m, const int32_t *entry_row, const uint32_t *csr_idx,
-                              const uint8_t *csr_aux, uint64_t *keys, uint32_t *vals) {
+                              const uint8_t *csr_aux, const uint8_t *col_degree, uint64_t *keys, uint32_t *vals) {
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (p >= n_entries) return;
     const uint32_t idx = csr_idx[p], rc = csr_aux[p];
     const bool inl = (idx >> TYPE_SHIFT) == DBSPMSPV_BLK_INLINE;
     const uint64_t row = inl ? (uint64_t)entry_row[p] * 16 + (rc >> 4) : (uint64_t)m;   // others sort behind every row
-    const uint64_t col = inl ? (uint64_t)(idx & IDX_MASK) * 16 + (rc & 15u) : 0u;
-    keys[p] = (row << 31) | col;
+    keys[p] = (row << ROWRUN_KEY_SHIFT) | (inl ? 255u - col_degree[(int64_t)(idx & IDX_MASK) * 16 + (rc & 15u)] : 0u);
     vals[p] = (idx & IDX_MASK) | ((rc & 15u) << 27);
+}
+
+// The first element of every row's run.
+__global__ void k_row_first(int64_t m, const int32_t *ptr, const uint32_t *rowrun, uint32_t *first) {
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= (m + 31) / 32 * 32) return;
+    first[i] = i < m && ptr[i] < ptr[i + 1] ? rowrun[ptr[i]] : 0xFFFFFFFFu;
 }
 
 // The stored elements by row and weight (see Device::weightrun): key, and the element's number as value.
@@ -1023,7 +1029,7 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
     }
 
     // row-run index for the pull levels of DB-BFS
-    d.rowrun_ptr = nullptr; d.rowrun_idx = nullptr; d.col_degree = nullptr;
+    d.rowrun_ptr = nullptr; d.rowrun_idx = nullptr; d.col_degree = nullptr; d.row_first = nullptr;
     if (m == n && !h->copts.no_bfs_index) {
         uint8_t *cd;
         DBS_KEEP(cd, (int64_t)d.nb * 16 + 16);
@@ -1033,13 +1039,13 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         uint32_t *rv, *rv_alt;
         DBS_GET(rk, n_entries); DBS_GET(rk_alt, n_entries); DBS_GET(rv, n_entries); DBS_GET(rv_alt, n_entries);
         if (n_entries) {
-            k_rowrun_keys<<<grid_for(n_entries), TPB, 0, st>>>(n_entries, m, h->block_row, d.csr.idx, d.csr.aux, rk, rv);
-            DBS_TRY(sort_pairs(tp, rk, rk_alt, rv, rv_alt, (int64_t)n_entries, 31 + bits_for((uint64_t)m), st));
+            k_rowrun_keys<<<grid_for(n_entries), TPB, 0, st>>>(n_entries, m, h->block_row, d.csr.idx, d.csr.aux, d.col_degree, rk, rv);
+            DBS_TRY(sort_pairs(tp, rk, rk_alt, rv, rv_alt, (int64_t)n_entries, ROWRUN_KEY_SHIFT + bits_for((uint64_t)m), st));
         }
         int32_t *rp;
         DBS_KEEP(rp, m + 1);
         d.rowrun_ptr = rp;
-        k_rowrun_ptr<<<grid_for(m + 1), TPB, 0, st>>>(m, rk, 31, n_entries, rp);
+        k_rowrun_ptr<<<grid_for(m + 1), TPB, 0, st>>>(m, rk, ROWRUN_KEY_SHIFT, n_entries, rp);
         int32_t n_inline = 0;      // the entries with a payload sort behind every row
         DBS_CUDA(cudaMemcpyAsync(&n_inline, rp + m, 4, cudaMemcpyDeviceToHost, st));
         DBS_CUDA(cudaStreamSynchronize(st));
@@ -1047,9 +1053,13 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         DBS_KEEP(ri, (int64_t)n_inline + 4);      // (slack: the pull reads whole aligned groups of four)
         d.rowrun_idx = ri;
         if (n_inline) DBS_CUDA(cudaMemcpyAsync(ri, rv, (size_t)n_inline * 4, cudaMemcpyDeviceToDevice, st));
+        uint32_t *rf;
+        DBS_KEEP(rf, (m + 31) / 32 * 32);
+        d.row_first = rf;
+        if (m) k_row_first<<<grid_for((m + 31) / 32 * 32), TPB, 0, st>>>(m, rp, ri, rf);
         DBS_CUDA(cudaStreamSynchronize(st));
         tp.release(rk); tp.release(rk_alt); tp.release(rv); tp.release(rv_alt);
-        h->bfs_index_bytes += ((int64_t)m + 1) * 4 + (int64_t)n_inline * 4 + (int64_t)d.nb * 16;
+        h->bfs_index_bytes += ((int64_t)m + 1) * 4 + (int64_t)n_inline * 4 + (int64_t)d.nb * 16 + (int64_t)m * 4;
     }
 
     // Streaming decode of payload-dominated handles: the chunk table

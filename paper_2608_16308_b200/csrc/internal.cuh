@@ -93,6 +93,7 @@ constexpr uint32_t HUB_CLEAR = 0x80000000u; // an untouched private accumulator 
 constexpr uint32_t ACC_CLEAR = 0x80000000u;
 constexpr float ACC_FLAG_MIN = 7.8886090522101181e-31f;     // 2^-100
 constexpr int SSSP_WEIGHT_BITS = 16;
+constexpr int ROWRUN_KEY_SHIFT = 8;
 constexpr uint32_t PAD_IDX = 7u << TYPE_SHIFT;   // class code of the slack behind the last view entry: no kernel acts on it
 // The streaming pull of hypersparse handles takes the block-CSR view in chunks of LEAN_CHUNK
 // entries, one chunk (eight entries per lane) per warp pass.
@@ -205,6 +206,7 @@ struct Counters {    // device-resident scalars of one call
                             // set that is reset meanwhile)
     int32_t bfs_nwords[4];  // BFS: lengths of the four rotating lists of nonzero mask words (Workspace::bfs_words)
     int32_t bfs_cnt[3][2];  // BFS: {nonempty frontier blocks, tasks}
+    int32_t bfs_edges[3];   // BFS: elements of the frontier's columns, at least (counted by push levels)
     int32_t bfs_level_path[DBSPMSPV_MAX_BFS_LEVELS_RECORDED];
     int32_t bfs_level_nzblk[DBSPMSPV_MAX_BFS_LEVELS_RECORDED];
     // BFS: device time stamps (ns): [0] kernel start, [1 + L] start of level L, then the end of the last level
@@ -249,11 +251,12 @@ struct Device {           // everything the kernels need, passed by value
     int32_t n_chunks;
     int32_t payload_chunk;  // entries with a payload per push task (see allocate_workspace)
     // Row-run index for the pull levels of DB-BFS (square matrices, unless switched off): the
-    // INLINE elements once more, row by row -- rowrun_idx[k] = column block | local column << 27
+    // INLINE elements once more, row by row, the columns of the highest degree first -- rowrun_idx[k] = column block | local column << 27
     // for k in [rowrun_ptr[i], rowrun_ptr[i + 1]) -- so that a row can stop at its first frontier
     // neighbour.  Null when not built.
     const int32_t *rowrun_ptr;
     const uint32_t *rowrun_idx;
+    const uint32_t *row_first;     // every row's first element once more (0xFFFFFFFF: none): the column with the highest degree
     const uint8_t *col_degree;     // degree_code of every column's INLINE elements (null when the index is not built)
     // All elements of fp32 handles once more, every row's by weight (column, weight bits), for the large steps of
     // db_sssp: a row stops at the first weight that cannot improve it.  Row i is [weight_ptr[i], weight_ptr[i + 1]), ordered by the upper

@@ -192,3 +192,28 @@ def test_push_levels_past_the_step_limit():
             assert np.array_equal(bfs(h, s), want)
             assert h.get_stats().bfs_reached == int((want >= 0).sum())
     h.close()
+
+
+@pytest.mark.parametrize("n", [65535, 65537, 70001, 70016])
+def test_large_levels_of_ragged_graphs(n):
+    """Push levels past the step limit (levels, visited and counts come from a pass over the masks behind them) and pull levels in which most rows end at their
+    first element, on graphs whose last mask word is not full; the levels start at an address that is not a multiple of 16 bytes."""
+    rng = np.random.default_rng(n)
+    hub = rng.integers(0, 64, 4 * n)
+    u, v = np.r_[hub, rng.integers(0, n, 12 * n)], rng.integers(0, n, 16 * n)
+    keep = u != v
+    keys = wl.sorted_unique(np.r_[u[keep] * n + v[keep], v[keep] * n + u[keep]].astype(np.int64))
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    g = wl.CSR(n, n, ptr, idx, None)
+    h, A = Handle(g, B.PATTERN), ref_matrix(g)
+    levels = torch.empty(n + 1, dtype=torch.int32, device="cuda")[1:]
+    for src in (n - 1, 5):
+        want = oracle.ref_bfs(A, src)
+        for path in PATHS:
+            h.set_opts(force_path=path)
+            levels.fill_(7)
+            B.db_bfs(h.h, src, levels)
+            torch.cuda.synchronize()
+            assert np.array_equal(levels.cpu().numpy(), want)
+            assert h.get_stats().bfs_reached == int((want >= 0).sum())
+    h.close()
