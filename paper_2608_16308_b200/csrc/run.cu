@@ -2085,6 +2085,17 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     return DBSPMSPV_OK;
 }
 
+// Columns up to which the one-kernel form of a call is the faster one (see small_call.cuh).  Without long columns or payload blocks the chain is two kernels: uniform
+// rows, 16 K / 64 K / 256 K / 1 M of them, 6.2 / 6.3 / 6.5 / 9.9 us whatever x holds, against 6.6 / 7.3 / 6.9 / 7.6 with 48 columns, 7.0 / 7.9 / 7.3 / 8.2 with 96 and
+// 8.4 / 8.6 / 9.0 / 10.0 with 250.  With long columns it is three: R-MAT in scattered order, 256 K / 1 M rows, 9.2 / 13.7 us, against 8.5 / 9.8 with 96 columns,
+// 9.4 / 12 with 160, 9.9 / 11.3 with 250.  (Handles with more payload blocks stay at the old limit: both ways vary by half with the columns that x lists.)
+static int small_call_limit(const dbspmspv_handle_s *h) {
+    const Device &d = h->d;
+    if (d.long_cap == 0) return d.m <= (1 << 17) ? 48 : d.m <= (1 << 19) ? 64 : 224;
+    if ((int64_t)d.n_payload * 2048 > d.n_entries) return SMALL_MAX_NNZ_X;
+    return d.m <= (1 << 19) ? 96 : 160;
+}
+
 template <int DT>
 static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_val, int32_t nnz_x,
                      int semiring, int32_t *y_idx, float *y_val, int64_t y_capacity, int32_t *y_nnz,
@@ -2095,7 +2106,7 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
     {
         const size_t ywords = (size_t)(d.mb + 1) / 2, cbwords = (size_t)(d.nb + 31) / 32;
         const size_t smem = ((ywords + SMALL_CLUSTER - 1) / SMALL_CLUSTER + (cbwords + SMALL_CLUSTER - 1) / SMALL_CLUSTER) * sizeof(uint32_t);
-        if (nnz_x > 0 && nnz_x <= SMALL_MAX_NNZ_X && d.n_entries > 0 && !h->heavy_stage && !h->ropts.validate && !h->ropts.timing &&
+        if (nnz_x > 0 && nnz_x <= small_call_limit(h) && d.n_entries > 0 && !h->heavy_stage && !h->ropts.validate && !h->ropts.timing &&
             !h->ropts.no_small_call && h->ropts.force_path != DBSPMSPV_PATH_PULL && !pull_possible(h, nnz_x, h->ropts.th3) &&
             smem <= SMALL_MAX_SMEM && (int64_t)ywords * 32 * (int64_t)sizeof(int32_t) <= d.ws.task_capacity * (int64_t)sizeof(*d.ws.tasks)) {
             const int mode = semiring == DBSPMSPV_OR_AND ? 1 : semiring == DBSPMSPV_MIN_PLUS ? 2 : 0;

@@ -42,7 +42,8 @@ constexpr int SMALL_CLUSTER = 8;               // thread blocks of the cluster (
 // One warp per listed column.  Calls back to back, one kernel against the chain of push and finishing kernel (median of five x): R-MAT scale 20,
 // 16 / 64 / 128 / 256 columns 8.7 / 10.0 / 14.4 / 17.5 us against 14.6 whatever x holds; scale 17, 64 / 128 / 256 8.1 / 13.0 / 14.1 against 9.9;
 // 16 K uniform rows 7.3 / 8.1 / 8.5 against 7.1, a million 8.6 / 9.6 / 10.2 against 10.5; 27-point operator on 90^3 cells 16.3 / 17.0 / 18.7 against 13.2.
-// The chain has become the faster one from about 64 - 128 columns on (from fewer where the matrix is small or holds payload blocks).
+// The chain has become the faster one from about 64 - 128 columns on (from fewer where the matrix is small or holds payload blocks); small_call_limit
+// says where a handle's calls change over.
 constexpr int SMALL_MAX_NNZ_X = 256;
 constexpr int SMALL_HUB_RUN = 512;             // a run from this length on is walked by the whole cluster
 constexpr int SMALL_HUB_CAP = 128;
