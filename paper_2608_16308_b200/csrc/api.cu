@@ -202,7 +202,7 @@ int dbspmspv_destroy(dbspmspv_handle_t h) {
     cudaFree(const_cast<int32_t *>(d.seg_rb));
     cudaFree(const_cast<uint32_t *>(d.row_present32));
     cudaFree(const_cast<int32_t *>(d.rowrun_ptr)); cudaFree(const_cast<uint32_t *>(d.rowrun_idx)); cudaFree(const_cast<uint2 *>(d.weightrun));
-    cudaFree(const_cast<uint8_t *>(d.col_degree)); cudaFree(const_cast<uint32_t *>(d.row_first)); cudaFree(const_cast<int32_t *>(d.weight_ptr)); cudaFree(const_cast<float *>(d.row_lightest));
+    cudaFree(const_cast<int32_t *>(d.weight_ptr));        // (row_lightest, row_first and col_degree lie behind the row pointers)
     cudaFree(const_cast<int32_t *>(d.csr_inl)); cudaFree(const_cast<int32_t *>(d.payload_pos));
     cudaFree(const_cast<int32_t *>(d.lean_rows)); cudaFree(const_cast<int32_t *>(d.lean_chunk_ord));
     cudaFree(const_cast<int4 *>(d.stage_chunks));

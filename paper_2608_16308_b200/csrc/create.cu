@@ -930,6 +930,9 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
             else DBS_ENCODE(DBSPMSPV_PATTERN);
 #undef DBS_ENCODE
         }
+        DBS_CUDA(cudaStreamSynchronize(st));
+        tp.release(blk_start); tp.release(block_of); tp.release(poff); tp.release(psize);
+        tp.release(brow); tp.release(bcol); tp.release(ecount); tp.release(eoff); tp.release(type);
         // every row's elements by weight, for the pulled steps of db_sssp
         d.weightrun = nullptr; d.weight_ptr = nullptr; d.row_lightest = nullptr;
         h->bfs_index_bytes = 0;
@@ -938,10 +941,11 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
             uint32_t *wv, *wv_alt;
             int32_t *wp;
             uint2 *wr;
-            float *lightest;
             const float *weights = static_cast<const float *>(uval);
             DBS_GET(wk, nnzu); DBS_GET(wk_alt, nnzu); DBS_GET(wv, nnzu); DBS_GET(wv_alt, nnzu);
-            DBS_KEEP(wp, m + 1); DBS_KEEP(wr, nnzu + 4); DBS_KEEP(lightest, m);
+            const int64_t wp_pad = (m + 1 + 31) / 32 * 32;          // (one allocation: row pointers, lightest weights)
+            DBS_KEEP(wp, wp_pad + m); DBS_KEEP(wr, nnzu + 4);
+            float *lightest = reinterpret_cast<float *>(wp + wp_pad);
             d.weight_ptr = wp; d.weightrun = wr; d.row_lightest = lightest;
             k_weightrun_keys<<<grid_for(nnzu), TPB, 0, st>>>(nnzu, ukey, weights, wk, wv);
             DBS_TRY(sort_pairs(tp, wk, wk_alt, wv, wv_alt, nnzu, SSSP_WEIGHT_BITS + bits_for((uint64_t)m), st));
@@ -952,9 +956,7 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
             tp.release(wk); tp.release(wk_alt); tp.release(wv); tp.release(wv_alt);
             h->bfs_index_bytes += nnzu * 8 + ((int64_t)m * 2 + 1) * 4;
         }
-        DBS_CUDA(cudaStreamSynchronize(st));
-        tp.release(ukey); tp.release(uval); tp.release(blk_start); tp.release(block_of); tp.release(poff); tp.release(psize);
-        tp.release(brow); tp.release(bcol); tp.release(ecount); tp.release(eoff); tp.release(type);
+        tp.release(ukey); tp.release(uval);
         DBS_GET(k1, n_entries); DBS_GET(k1_alt, n_entries); DBS_GET(ids, n_entries); DBS_GET(ids_alt, n_entries);
         if (n_entries) {
             k_csr_keys<<<grid_for(n_entries), TPB, 0, st>>>(n_entries, t_row, t_idx, t_aux, k1, ids);
@@ -1031,9 +1033,13 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
     // row-run index for the pull levels of DB-BFS
     d.rowrun_ptr = nullptr; d.rowrun_idx = nullptr; d.col_degree = nullptr; d.row_first = nullptr;
     if (m == n && !h->copts.no_bfs_index) {
-        uint8_t *cd;
-        DBS_KEEP(cd, (int64_t)d.nb * 16 + 16);
-        d.col_degree = cd;
+        // one allocation: row pointers, first elements, degrees
+        const int64_t rp_pad = (m + 1 + 31) / 32 * 32, rf_pad = (m + 31) / 32 * 32;
+        int32_t *rp;
+        DBS_KEEP(rp, rp_pad + rf_pad + ((int64_t)d.nb * 16 + 16 + 3) / 4);
+        uint32_t *rf = reinterpret_cast<uint32_t *>(rp + rp_pad);
+        uint8_t *cd = reinterpret_cast<uint8_t *>(rf + rf_pad);
+        d.rowrun_ptr = rp; d.row_first = rf; d.col_degree = cd;
         if (d.nb) k_col_degree<<<grid_for((int64_t)d.nb * 16), TPB, 0, st>>>(d.nb, d.csc.colptr, cd);
         uint64_t *rk, *rk_alt;
         uint32_t *rv, *rv_alt;
@@ -1042,9 +1048,6 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
             k_rowrun_keys<<<grid_for(n_entries), TPB, 0, st>>>(n_entries, m, h->block_row, d.csr.idx, d.csr.aux, d.col_degree, rk, rv);
             DBS_TRY(sort_pairs(tp, rk, rk_alt, rv, rv_alt, (int64_t)n_entries, ROWRUN_KEY_SHIFT + bits_for((uint64_t)m), st));
         }
-        int32_t *rp;
-        DBS_KEEP(rp, m + 1);
-        d.rowrun_ptr = rp;
         k_rowrun_ptr<<<grid_for(m + 1), TPB, 0, st>>>(m, rk, ROWRUN_KEY_SHIFT, n_entries, rp);
         int32_t n_inline = 0;      // the entries with a payload sort behind every row
         DBS_CUDA(cudaMemcpyAsync(&n_inline, rp + m, 4, cudaMemcpyDeviceToHost, st));
@@ -1053,9 +1056,6 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         DBS_KEEP(ri, (int64_t)n_inline + 4);      // (slack: the pull reads whole aligned groups of four)
         d.rowrun_idx = ri;
         if (n_inline) DBS_CUDA(cudaMemcpyAsync(ri, rv, (size_t)n_inline * 4, cudaMemcpyDeviceToDevice, st));
-        uint32_t *rf;
-        DBS_KEEP(rf, (m + 31) / 32 * 32);
-        d.row_first = rf;
         if (m) k_row_first<<<grid_for((m + 31) / 32 * 32), TPB, 0, st>>>(m, rp, ri, rf);
         DBS_CUDA(cudaStreamSynchronize(st));
         tp.release(rk); tp.release(rk_alt); tp.release(rv); tp.release(rv_alt);
