@@ -32,6 +32,7 @@
 #include "internal.cuh"
 #include "microkernels.cuh"
 #include "minplus.cuh"
+#include "push_direct.cuh"
 
 namespace dbs {
 
@@ -226,16 +227,24 @@ struct LeanScratch {        // per warp
     float stmp[32];
 };
 
-template <int DT, typename Out>
+template <int DT, typename Out, bool LONG>
 __global__ void __launch_bounds__(LEAN_CTA, 1)
-k_pull_lean(Device d, Out out, float th3, int force_path, int popc_threshold, int filter_words) {
+k_pull_lean(Device d, Out out, float th3, int force_path, int popc_threshold, int filter_words, int boolean_push) {
     extern __shared__ __align__(128) uint8_t s_lean[];
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *filter = reinterpret_cast<uint32_t *>(s_lean);
     LeanScratch *ls = reinterpret_cast<LeanScratch *>(s_lean + (size_t)filter_words * 4) + warp;
     pdl_wait();
-    if (select_path(d, th3, force_path) != DBSPMSPV_PATH_PULL) return;
+    if (select_path(d, th3, force_path) != DBSPMSPV_PATH_PULL) {
+        if constexpr (LONG) {                          // the push's listed chunks (see k_push_long)
+            const int gw = warp * gridDim.x + blockIdx.x, nw = gridDim.x * LEAN_WARPS;
+            constexpr int MODE = Out::MINPLUS ? 2 : DT == DBSPMSPV_PATTERN ? 1 : 0;
+            if (MODE == 0 && boolean_push) push_long_chunks<DT, 1, false>(d, gw, nw);
+            else push_long_chunks<DT, MODE, false>(d, gw, nw);
+        }
+        return;
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) d.ws.ctr->path = DBSPMSPV_PATH_PULL;
     const int gwarp = warp * gridDim.x + blockIdx.x;      // (neighbouring chunks on different SMs: the last, partial round of chunks is spread over all of them)
     const int nwarps = gridDim.x * LEAN_WARPS;

@@ -40,7 +40,8 @@ constexpr int PD_WARPS = PD_CTA / 32;
 constexpr int PD_ILP = 4;            // warp steps in flight
 static_assert(PD_CHUNK % 32 == 0, "whole entries per lane");
 constexpr int pd_per_sm(bool masks) { return masks ? 5 : 6; }   // resident thread blocks per SM (registers)
-constexpr int PD_MASK_WORDS = 32;    // mask words of a thread block's round (MASKS): eight threads per word, four columns each
+// Mask words of a thread block's round (MASKS): eight threads per word, four columns each.  (Eight columns, four thread blocks per SM: R-MAT scale 20, x = 10 %, 39.7 -> 42.8 us a call.)
+constexpr int PD_MASK_WORDS = 32;
 
 // MODE 0: (+, *), 1: Boolean, 2: (min, +)
 template <int DT, int MODE>
@@ -372,13 +373,15 @@ k_push_direct(Device d, const int32_t *__restrict__ x_idx, const void *__restric
 
 // The listed chunks, a warp at a time; the next chunk's record is fetched a round ahead.
 // (Nothing is listed when the path decided on the device is the pull.)
+// Where the path is decided on the device and the matrix is small, the streaming pull, launched in any case, takes them when the decision was the push: a launch less
+// (R-MAT 20 K rows, x = 30 %: 14.5 -> 12.6 us a call; 40 K vertices, masked, 10 %: 15.7 -> 15.0; 256 K rows, 10 %: 22.1 -> 21.1; with 16 to 31 M entries, where
+// the warps of its one thread block per SM are too few, up to 1 % longer, and payload runs of four columns 8 %).
+constexpr int LONG_IN_PULL_ENTRIES = 8 << 20;
 template <int DT, int MODE, bool GROUPS>
-__global__ void __launch_bounds__(PD_CTA, 6) k_push_long(Device d) {
+__device__ __forceinline__ void push_long_chunks(const Device &d, int gwarp, int nwarps) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN && MODE != 1;
     constexpr int U = PD_CHUNK / 32;
     const int lane = threadIdx.x & 31;
-    const int gwarp = (int)(blockIdx.x * PD_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * PD_CTA) >> 5;
-    pdl_wait();
     const int n = min(d.ws.ctr->n_long, d.long_cap);
     int4 next = gwarp < n ? d.ws.long_runs[gwarp] : make_int4(0, 0, 0, 0);
     for (int i = gwarp; i < n; i += nwarps) {
@@ -411,6 +414,12 @@ __global__ void __launch_bounds__(PD_CTA, 6) k_push_long(Device d) {
         for (int u = 0; u < U; ++u)
             if (idx[u] < (1u << TYPE_SHIFT)) push_product<DT, MODE>(d, idx[u], (int)(aux[u] >> 4), Val<DT>::inline_value(w[u]), xs);
     }
+}
+
+template <int DT, int MODE, bool GROUPS>
+__global__ void __launch_bounds__(PD_CTA, 6) k_push_long(Device d) {
+    pdl_wait();
+    push_long_chunks<DT, MODE, GROUPS>(d, (int)(blockIdx.x * PD_CTA + threadIdx.x) >> 5, (int)(gridDim.x * PD_CTA) >> 5);
 }
 
 }  // namespace dbs

@@ -1979,9 +1979,9 @@ static int launch_compute(dbspmspv_handle_s *h, CallList &calls, Out out, float 
 }
 
 // The streaming pull of hypersparse handles (lean_pull.cuh), launched behind k_compute.
-template <int DT, typename Out>
-static int launch_lean(dbspmspv_handle_s *h, CallList &calls, Out out, float th3) {
-    bool &configured = Out::MINPLUS ? h->lean_configured_min : Out::MASKS ? h->lean_configured : h->lean_configured_dense;
+template <int DT, typename Out, bool LONG = false>
+static int launch_lean(dbspmspv_handle_s *h, CallList &calls, Out out, float th3, int boolean_push = 0) {
+    bool &configured = (Out::MINPLUS ? h->lean_configured_min : Out::MASKS ? h->lean_configured : h->lean_configured_dense)[LONG];
     // filter size: the power of two that holds one bit per column, capped
     const int n_words = (h->d.nb + 1) / 2;
     int filter_words = 32;
@@ -1991,11 +1991,11 @@ static int launch_lean(dbspmspv_handle_s *h, CallList &calls, Out out, float th3
         // (the attribute belongs to the kernel, not to the handle: the largest size, or a handle with few columns would lower it
         // below what one with many, configured before, asks for)
         constexpr int most = LEAN_FILTER_MAX_WORDS * 4 + LEAN_WARPS * (int)sizeof(LeanScratch);
-        auto kernel = k_pull_lean<DT, Out>;
+        auto kernel = k_pull_lean<DT, Out, LONG>;
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess) return DBSPMSPV_ERR_CUDA;
         configured = true;
     }
-    calls.add(k_pull_lean<DT, Out>, h->sm_count, LEAN_CTA, smem, true, h->d, out, th3, h->ropts.force_path, h->ropts.popc_threshold, filter_words);
+    calls.add(k_pull_lean<DT, Out, LONG>, h->sm_count, LEAN_CTA, smem, true, h->d, out, th3, h->ropts.force_path, h->ropts.popc_threshold, filter_words, boolean_push);
     return DBSPMSPV_OK;
 }
 
@@ -2126,6 +2126,7 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
         const bool may_push = !may_pull || fp != DBSPMSPV_PATH_PULL;
         const int mode = boolean ? 1 : minplus ? 2 : 0;
         const bool groups = h->payload_rich && nnz_x >= PD_GROUPS_MIN_NNZ_X;
+        const bool long_in_pull = any && may_pull && may_push && d.long_cap && !groups && d.n_entries <= LONG_IN_PULL_ENTRIES;
         // private accumulators for the hub row blocks, when x is long enough for their atomics to queue up
         const int hub_min = h->ropts.hub_min_nnz_x ? h->ropts.hub_min_nnz_x : HUB_MIN_NNZ_X;
         h->d.hub_on = may_push && d.n_hub_blocks > 0 && hub_min > 0 && nnz_x >= hub_min ? (nnz_x < HUB_ALL_NNZ_X ? 4 : HUB_COPIES) : 0;
@@ -2151,7 +2152,7 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
                     if (g > most) g = most;
                     calls.add(list_kernel, g, PD_CTA, 0, false, d, x_idx, xv, nnz_x, (int)h->ropts.validate, h->ropts.th3, fp, cols, (nnz_x + cols * g - 1) / (cols * g));
                 }
-                if (d.long_cap) calls.add(long_kernel, 6 * h->sm_count, PD_CTA, 0, true, d);
+                if (d.long_cap && !long_in_pull) calls.add(long_kernel, 6 * h->sm_count, PD_CTA, 0, true, d);
             };
             constexpr int VT = DT == DBSPMSPV_PATTERN ? DBSPMSPV_F32 : DT;       // (pattern handles have no (+, *))
             if (mode == 1 && groups) push(k_push_direct<DT, 1, false, true>, k_push_direct<DT, 1, true, true>, k_push_long<DT, 1, true>);
@@ -2162,8 +2163,10 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
             else if (DT != DBSPMSPV_PATTERN) push(k_push_direct<VT, 0, false, false>, k_push_direct<VT, 0, true, false>, k_push_long<VT, 0, false>);
         }
         if (any && may_pull) {
-            const int s = minplus ? launch_lean<DT, OutSparseMin>(h, calls, OutSparseMin{d.ws.y_acc, d.ws.y_mask32}, h->ropts.th3)
-                                  : launch_lean<DT, OutSparse>(h, calls, OutSparse{d.ws.y_acc, d.ws.y_mask32}, h->ropts.th3);
+            const OutSparse out{d.ws.y_acc, d.ws.y_mask32};
+            const OutSparseMin out_min{d.ws.y_acc, d.ws.y_mask32};
+            const int s = minplus ? (long_in_pull ? launch_lean<DT, OutSparseMin, true>(h, calls, out_min, h->ropts.th3) : launch_lean<DT, OutSparseMin>(h, calls, out_min, h->ropts.th3))
+                                  : (long_in_pull ? launch_lean<DT, OutSparse, true>(h, calls, out, h->ropts.th3, mode == 1) : launch_lean<DT, OutSparse>(h, calls, out, h->ropts.th3));
             if (s != DBSPMSPV_OK) return s;
         }
         if (!may_pull && (mode == 1 || !groups)) clear = CLEAR_MASKS;      // (x was staged for the payload entries only)
