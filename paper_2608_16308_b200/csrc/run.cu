@@ -1761,6 +1761,130 @@ __global__ void __launch_bounds__(CMP_TPB, FOLD ? 5 : 8) k_finish(Device d, int3
     finish_clear_x(d, x_idx, nnz_x, clear, bi, stride, j0);
 }
 
+// The same over two tiles per thread block, for accumulators of more tiles than fit on the GPU at once with results in a good part of the rows: the second tile waits in
+// shared memory, so that a thread block needs no more registers, the two are counted and lined up as one, and most of the second wave with its ticket, loads, count and wait
+// is spared.  (27-point operator, x in runs: 150^3 cells, 2 %, 37.3 -> 32.2 us a call; 160^3, 5 %, 48.8 -> 47.9.  With results in nearly all rows the second tile's way through
+// shared memory costs more than the wave: 144^3, 30 %, 149 -> 154, 150^3, 10 %, 124 -> 130.)
+__global__ void __launch_bounds__(CMP_TPB, 8) k_finish_pair(Device d, int32_t *__restrict__ y_idx, float *__restrict__ y_val,
+                                                           int64_t y_capacity, int32_t *__restrict__ y_nnz, int boolean,
+                                                           const int32_t *__restrict__ x_idx, int32_t nnz_x, int clear,
+                                                           const uint32_t *__restrict__ row_mask, int complement) {
+    __shared__ __align__(16) uint4 s_second[2][CMP_TPB];
+    __shared__ int s_cnt[CMP_TPB / 32], s_ticket, s_parity, s_base;
+    __shared__ int32_t s_oidx[CMP_TPB * 8];
+    __shared__ float s_oval[CMP_TPB * 8];
+    Counters *ctr = d.ws.ctr;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (nnz_x == 0) pdl_wait();
+    if (tid == 0) { const int w = atomicAdd(&ctr->finish_ticket, 1); s_ticket = w & (FINISH_PARITY - 1); s_parity = w & FINISH_PARITY ? 1 : 0; }
+    __syncthreads();
+    const int unit = s_ticket, parity = s_parity, n_units = (d.ws.n_tiles + 1) / 2;
+    const int stride = gridDim.x * CMP_TPB, at = unit * CMP_TPB + tid;
+    const int j0 = (!(clear & CLEAR_SWEEP) && at < nnz_x) ? x_idx[at] : -1;
+    pdl_wait();
+    if (unit < n_units) {
+        const int n_bytes = (d.mb + 1) / 2 * 4;
+        uint8_t *mask8 = reinterpret_cast<uint8_t *>(d.ws.y_mask32);
+        const int bi = unit * 2 * CMP_TPB + tid, bj = bi + CMP_TPB;         // bytes of the hit mask: rows 8 bi .. 8 bi + 7 and 8 bj .. 8 bj + 7
+        const uint4 untouched = make_uint4(ACC_CLEAR, ACC_CLEAR, ACC_CLEAR, ACC_CLEAR);
+        uint4 *acc_i = reinterpret_cast<uint4 *>(d.ws.y_acc + (size_t)bi * 8), *acc_j = reinterpret_cast<uint4 *>(d.ws.y_acc + (size_t)bj * 8);
+        uint32_t v[8], bits_i = 0u, bits_j = 0u;
+        uint32_t flags_j = 0u;
+        if (bj < n_bytes) {                            // (every thread reads back what it copied itself)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(&s_second[h][tid])), "l"(acc_j + h) : "memory");
+            flags_j = mask8[bj];
+        }
+        if (bi < n_bytes) {
+            const uint4 a = __ldcg(acc_i), b = __ldcg(acc_i + 1);
+            const uint32_t flags = mask8[bi];
+            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+            uint32_t hits = flags;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) hits |= (v[r] != ACC_CLEAR ? 1u : 0u) << r;
+            if (hits) { acc_i[0] = untouched; acc_i[1] = untouched; }
+            if (flags) mask8[bi] = 0;
+            bits_i = row_mask ? hits & (reinterpret_cast<const uint8_t *>(row_mask)[bi] ^ (complement ? 0xFFu : 0u)) : hits;
+        }
+        auto second = [&](uint32_t (&w)[8]) {
+            const uint4 a = s_second[0][tid], b = s_second[1][tid];
+            w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+        };
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if (bj < n_bytes) {
+            uint32_t w[8], hits = flags_j;
+            second(w);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) hits |= (w[r] != ACC_CLEAR ? 1u : 0u) << r;
+            if (hits) { acc_j[0] = untouched; acc_j[1] = untouched; }
+            if (flags_j) mask8[bj] = 0;
+            bits_j = row_mask ? hits & (reinterpret_cast<const uint8_t *>(row_mask)[bj] ^ (complement ? 0xFFu : 0u)) : hits;
+        }
+        const int c = __popc(bits_i) | __popc(bits_j) << 16;               // (2048 at most: both counts in one scan)
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) s_cnt[warp] = incl;
+        __syncthreads();
+        int before = incl - c, total = 0;
+#pragma unroll
+        for (int k = 0; k < CMP_TPB / 32; ++k) {
+            if (k < warp) before += s_cnt[k];
+            total += s_cnt[k];
+        }
+        const int total_i = total & 0xFFFF, total_j = total >> 16;
+        // (every call rewrites every tile's word, read or not: the next call may take one tile per thread block)
+        if (tid == 1 && unit + n_units < d.ws.n_tiles) d.ws.tile_status[unit + n_units] = parity;
+        if (tid == 0) {
+            asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(d.ws.tile_status + unit), "r"((total_i + total_j) * 2 + parity) : "memory");
+            atomicAdd(d.ws.tile_group + parity * d.ws.n_tile_groups + unit / FINISH_GROUP, (1ull << 32) + (unsigned)(total_i + total_j));
+        }
+        if (unit == 0)
+            for (int k = tid; k < d.ws.n_tile_groups; k += CMP_TPB) d.ws.tile_group[(parity ^ 1) * d.ws.n_tile_groups + k] = 0ull;
+        auto gather = [&](uint32_t bits, int first_row, const uint32_t (&w)[8], int pos) {
+#pragma unroll
+            for (int bit = 0; bit < 8; ++bit) {
+                if ((bits >> bit) & 1u) {
+                    s_oidx[pos] = first_row + bit;
+                    s_oval[pos] = boolean == 1 ? 1.0f : boolean == 2 ? minplus_of_word(w[bit]) : __uint_as_float(w[bit]) + 0.0f;
+                    ++pos;
+                }
+            }
+        };
+        auto write = [&](int64_t base, int n) {
+            for (int k = tid; k < n; k += CMP_TPB) {
+                const int64_t pos = base + k;
+                if (pos < y_capacity) {
+                    y_idx[pos] = s_oidx[k];
+                    if (y_val) y_val[pos] = s_oval[k];
+                }
+            }
+        };
+        if (bits_i) gather(bits_i, bi * 8, v, before & 0xFFFF);
+        if (warp == 0) {
+            const int sum = entries_before(d, unit, parity, lane);
+            if (lane == 0) { s_base = sum; if (sum < 0) ctr->status = DBSPMSPV_ERR_TIMEOUT; }
+        }
+        __syncthreads();
+        const int base = max(s_base, 0);
+        write(base, total_i);
+        __syncthreads();
+        if (bits_j) {
+            uint32_t w[8];
+            second(w);
+            gather(bits_j, bj * 8, w, before >> 16);
+        }
+        __syncthreads();
+        write((int64_t)base + total_i, total_j);
+        if (unit == n_units - 1 && tid == 0) finish_counters(d, base + total_i + total_j, y_capacity, y_nnz);
+    }
+    if (unit == (int)gridDim.x - 1 && tid == 0) ctr->finish_ticket = parity ? 0 : FINISH_PARITY;
+    finish_clear_x(d, x_idx, nnz_x, clear, at, stride, j0);
+}
+
 // The same over FINISH_WIDE tiles at most per thread block, for accumulators of more tiles than fit on the GPU at once (in waves, each tile
 // with its ticket, loads, count and wait: 16 us on four million rows even for an empty result; 8 here).  First all tiles are
 // counted, their loads side by side; then the rows that hold results are fetched again, from L2, and written.  (Four million
@@ -2198,6 +2322,8 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
     if (per_block > 1)
         calls.add(d.hub_on ? k_finish_wide<true> : k_finish_wide<false>, (nt + per_block - 1) / per_block + extra, CMP_TPB, 0, calls.n > 0, d, per_block, y_idx, y_val, y_capacity, y_nnz,
                   minplus ? 2 : (int)boolean, x_idx, nnz_x, clear, d.hub_on ? (minplus ? 2 : 1) : 0, row_mask, complement);
+    else if (nt > 8 * h->sm_count && !d.hub_on && (int64_t)nnz_x * 16 <= d.n)      // (see k_finish_pair)
+        calls.add(k_finish_pair, (nt + 1) / 2 + extra, CMP_TPB, 0, calls.n > 0, d, y_idx, y_val, y_capacity, y_nnz, minplus ? 2 : (int)boolean, x_idx, nnz_x, clear, row_mask, complement);
     else
         calls.add(d.hub_on ? k_finish<true> : k_finish<false>, nt + extra, CMP_TPB, 0, calls.n > 0, d, y_idx, y_val, y_capacity, y_nnz, minplus ? 2 : (int)boolean, x_idx, nnz_x, clear,
                   d.hub_on ? (minplus ? 2 : 1) : 0, row_mask, complement);

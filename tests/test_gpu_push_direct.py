@@ -223,3 +223,56 @@ def test_wide_finish_behind_a_push_of_whole_blocks(tiles):
                 else:
                     check_against_oracle(got, w, boolean=semiring == B.OR_AND)
     h.close()
+
+
+@pytest.mark.parametrize("m", [2048 * 1185 - 5, 2048 * 1186, 2048 * 1187 + 16])       # (148 SMs: more than one wave; a last pair of one tile, of two)
+@pytest.mark.parametrize("blocks", [False, True])
+def test_paired_finish(m, blocks):
+    """The finishing kernel of two tiles per thread block behind a longer x, in turn with that of a short x on the same handle (another number of tiles per
+    thread block); rows at both ends of tiles, full ones and empty ones, masked and not, a capacity in the middle of a tile."""
+    n = 4001
+    rng = np.random.default_rng(m)
+    rows = np.unique(np.r_[0, 2047, 2048, 4095, 4096, m - 1, np.arange(6144, 10240), rng.integers(0, m, 40000)])
+    if blocks:
+        rbs = np.unique(rows // 16)[::4]
+        rbs = rbs[rbs < m // 16]
+        r = (16 * rbs[:, None] + np.arange(16)).reshape(-1, 16, 1)
+        c = (16 * rng.integers(0, n // 16, rbs.size)[:, None] + np.arange(16)).reshape(-1, 1, 16)
+        keys = wl.sorted_unique((r * np.int64(n) + c).ravel()[rng.random(rbs.size * 256) < 0.8])
+    else:
+        keys = wl.sorted_unique(np.r_[rows, rows].astype(np.int64) * n + rng.integers(0, n, 2 * rows.size))
+    ptr, idx = wl.csr_from_sorted_keys(m, n, keys)
+    csr = wl.CSR(m, n, ptr, idx, rng.choice(np.float32([1.5, -0.75, 0.0, -0.0, 2.0 ** -60]), keys.size).astype(np.float32))
+    h, A = Handle(csr, B.F32), ref_matrix(csr)
+    assert h.stats.n_hub_row_blocks == 0
+    drop = rng.random(m) < 0.5
+    mask = torch.from_numpy(np.packbits(np.r_[drop, np.zeros(-m % 32, bool)], bitorder="little").view(np.int32).copy()).to("cuda")
+    h.set_opts(no_small_call=1)
+    for k in (1500, 20, 200, 3900):
+        at = rng.choice(n, k, replace=False).astype(np.int32)
+        x = wl.SparseVec(n, at, rng.choice(np.float32([1.0, -2.0, 2.0 ** -60]), k).astype(np.float32))
+        xi, xv = torch.from_numpy(at).to("cuda"), torch.from_numpy(x.val).to("cuda")
+        for semiring in (B.PLUS_TIMES, B.OR_AND, B.MIN_PLUS):
+            if semiring == B.MIN_PLUS:
+                wi, wv = oracle.ref_minplus(A, x.idx, x.val)
+                want = (wi, wv, np.abs(wv))
+            else:
+                want = oracle.ref_pull(A, x.idx, x.val)
+            got, w = h.run(x, semiring=semiring), want
+            for masked in (False, True):
+                if masked:
+                    B.dbspmspv_run_masked(h.h, xi, xv, k, semiring, mask, 1, h.y_idx, h.y_val, m, h.y_nnz)
+                    kk = int(h.y_nnz.item())
+                    got = (h.y_idx[:kk].cpu().numpy(), h.y_val[:kk].cpu().numpy(), kk)
+                    w = tuple(v[~drop[want[0]]] for v in want)
+                if semiring == B.MIN_PLUS:
+                    assert np.array_equal(got[0], w[0]) and np.array_equal(got[1], w[1].astype(np.float32))
+                else:
+                    check_against_oracle(got, w, boolean=semiring == B.OR_AND)
+    cap = want[0].size // 3
+    h.y_idx.fill_(-1)
+    yi, _, kk = h.run(x, semiring=B.OR_AND, capacity=cap)
+    assert kk == want[0].size and (h.y_idx[cap:].cpu().numpy() == -1).all()
+    h.get_stats(raise_on_device_status=False)
+    check_against_oracle(h.run(x, semiring=B.OR_AND), oracle.ref_pull(A, x.idx, x.val), boolean=True)
+    h.close()
