@@ -27,8 +27,6 @@
 
 namespace dbs {
 
-constexpr int DC_SLOW_FLAG = 1 << 30;
-
 // x entry j of vector `b` as the products see it
 __device__ __forceinline__ float dc_x(const Device &d, const void *x, int64_t ldx, int b, int64_t j) {
     if (d.decode_x_f32) return __bfloat162float(__float2bfloat16_rn(static_cast<const float *>(x)[b * ldx + j]));
@@ -113,46 +111,51 @@ constexpr int DC_CTA = DC_WARPS * 32;
 constexpr int DC_ILP = 8;            // 16-byte loads in flight per lane: 4 KB per warp
 constexpr int DC_LANES = DC_ROWS / 8;    // lanes that share a column (eight rows each)
 constexpr int DC_SLOTS = 32 / DC_LANES;  // columns of a warp's load
-constexpr int DC_XILP = 4;           // groups of eight x entries a thread fetches at once
+constexpr int DC_XILP = 2;           // groups of eight x entries a lane fetches at once
 static_assert(DC_ROWS == 64, "two halving exchanges over the column slots");
 
-// One vector.  Lane (q, p) = (lane / 8, lane % 8): rows 8 p .. 8 p + 7 of the strip, every fourth column of the list.
+// Vector blocks of x that rank `rank` of C takes; its warps take them in turn, four neighbours at a time.  Entries of a warp's list, at most.
+__host__ __device__ inline int dc_blocks(int nb, int c, int rank) { return (nb - rank + c - 1) / c; }
+__host__ __device__ inline int dc_warp_entries(int nb, int c) { return (dc_blocks(nb, c, 0) + 4 * DC_WARPS - 1) / (4 * DC_WARPS) * 64; }
+
+// One vector.  A warp blocks a share of x for itself -- pieces of 64 entries spread over x, so that longer active runs meet all warps -- and goes on to the columns it
+// found: nobody waits for a list of the whole thread block.  (With one, three barriers and an atomic per warp stood between x and the first weight, and clusters
+// met twice more.  4096 x 11008, 10 / 50 % active: 6.4 / 12.4 -> 5.1 / 11.4 us; 2000 x 2000 4.8 -> 3.8; 12288 x 4096, 30 %: 8.1 -> 7.9.)
+// Lane (q, p) = (lane / 8, lane % 8): rows 8 p .. 8 p + 7 of the strip, every fourth column of the list.
 template <int C>
 __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(DC_CTA, 2)
 k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float th3, int force_path) {
     namespace cg = cooperative_groups;
     extern __shared__ __align__(16) uint8_t s_dyn[];
-    float2 *s_list = reinterpret_cast<float2 *>(s_dyn);              // (column bits, value)
     __shared__ __align__(8) float s_part[DC_WARPS][DC_ROWS];
     __shared__ float s_sum[C][DC_ROWS];
-    __shared__ int s_n, s_nz, s_seen[C];                             // entries; nonzero vector blocks; those of every rank, plus DC_SLOW_FLAG if it met a non-finite entry
+    __shared__ int s_nz[DC_WARPS], s_seen[C];                         // nonzero vector blocks of every warp; of every rank
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = C > 1 ? (int)cg::this_cluster().block_rank() : 0, strip = blockIdx.x / C;
-    if (tid == 0) { s_n = 0; s_nz = 0; }
+    // (a cluster: every block has started before its shared memory is written; met again behind the weights)
+    if (C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     pdl_wait();
-    if (C > 1) cg::this_cluster().sync(); else __syncthreads();       // (a cluster: every block has started before its shared memory is written)
+    const int blocks = dc_blocks(d.nb, C, rank);
+    float2 *list = reinterpret_cast<float2 *>(s_dyn) + warp * dc_warp_entries(d.nb, C);              // (column bits, value)
     bool odd = false;                                                 // some entry is not finite
-    // ---- the list of the entries that take part: eight consecutive ones per thread and round, this rank's vector blocks only
+    int n = 0, nz = 0;
     {
         const bool aligned = (reinterpret_cast<uintptr_t>(x) & 15u) == 0;
         const DcTest test(d);
-        const int units = (d.nb - rank + C - 1) / C * 2;             // halves of this rank's vector blocks
-        int nz = 0;
-        for (int u0 = warp * 32; u0 < units; u0 += DC_CTA * DC_XILP) {
+        for (int b0 = 4 * warp; b0 < blocks; b0 += 16 * DC_WARPS * DC_XILP) {    // two lanes per vector block, eight entries each
             uint4 v[DC_XILP];
             int j0[DC_XILP];
 #pragma unroll
             for (int q = 0; q < DC_XILP; ++q) {
-                const int u = u0 + q * DC_CTA + lane;
-                j0[q] = ((u >> 1) * C + rank) * 16 + (u & 1) * 8;
+                const int b = b0 + (q * 4 + (lane >> 3)) * 4 * DC_WARPS + ((lane >> 1) & 3);
+                j0[q] = (b * C + rank) * 16 + (lane & 1) * 8;
                 v[q] = make_uint4(0u, 0u, 0u, 0u);
-                if (u < units) v[q] = dc_load8(d, x, 0, 0, j0[q], aligned);
+                if (b < blocks) v[q] = dc_load8(d, x, 0, 0, j0[q], aligned);
             }
-            uint32_t bits = 0;                                        // eight per group
+            uint32_t bits = 0;                                        // eight per load
 #pragma unroll
             for (int q = 0; q < DC_XILP; ++q) {
-                if (u0 + q * DC_CTA >= units) break;                  // warp-uniform
-                const uint32_t w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};       // (entries past n are 0: they never take part)
+                const uint32_t w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};          // (entries past n are 0: they never take part)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const uint32_t m = test(w[k]);
@@ -164,65 +167,46 @@ k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float
             int incl = cnt;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
-            int base = 0;
-            if (lane == 31 && incl) base = atomicAdd(&s_n, incl);
-            int at = __shfl_sync(FULL, base, 31) + incl - cnt;
+            int at = n + incl - cnt;
+            n += __shfl_sync(FULL, incl, 31);
             const uint32_t both = bits | __shfl_xor_sync(FULL, bits, 1);
 #pragma unroll
             for (int q = 0; q < DC_XILP; ++q) {
-                if (u0 + q * DC_CTA >= units) break;
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
-                    if ((bits >> (8 * q + k)) & 1u) {
-                        s_list[at++] = make_float2(__int_as_float(j0[q] + k), dc_entry(v[q], k));
-                    }
+                    if ((bits >> (8 * q + k)) & 1u) list[at++] = make_float2(__int_as_float(j0[q] + k), dc_entry(v[q], k));
                 nz += __popc(__ballot_sync(FULL, (both >> (8 * q)) & 0xFFu) & 0x55555555u);
             }
         }
-        if (lane == 0 && nz) atomicAdd(&s_nz, nz);
-        odd = __syncthreads_or(odd);
-        if (C > 1) {
-            // (every rank has to know whether any met a non-finite entry)
-            cg::cluster_group cluster = cg::this_cluster();
-            if (tid < C) cluster.map_shared_rank(s_seen, tid)[rank] = s_nz | (odd ? DC_SLOW_FLAG : 0);
-            cluster.sync();
-#pragma unroll
-            for (int r = 0; r < C; ++r) odd |= (s_seen[r] & DC_SLOW_FLAG) != 0;
-        } else if (tid == 0) {
-            s_seen[0] = s_nz;
-        }
-        if (strip == 0 && rank == 0 && tid == 0) {
-            int total = 0;
-#pragma unroll
-            for (int r = 0; r < C; ++r) total += s_seen[r] & (DC_SLOW_FLAG - 1);
-            dc_record(d, total, th3, force_path);
-        }
-        if (odd) {
-            float a[1][DC_PER_LANE];
-            dc_slow<1>(d, x, 0, 1, strip, warp * C + rank, DC_WARPS * C, lane, a);
-#pragma unroll
-            for (int h = 0; h < DC_PER_LANE; ++h) s_part[warp][lane + 32 * h] = a[0][h];
-        } else {
-#pragma unroll
-            for (int h = 0; h < DC_PER_LANE; ++h) s_part[warp][lane + 32 * h] = 0.f;
-        }
+        __syncwarp();
     }
-    __syncthreads();
-    const int n = odd ? 0 : s_n;
-    if (n > 0) {                                                      // block-uniform
+    if (__any_sync(FULL, odd)) {                                      // this warp's columns, every element tested
+        float a[DC_PER_LANE] = {};
+        const uint16_t *w = reinterpret_cast<const uint16_t *>(d.cols) + (size_t)strip * d.n * DC_ROWS + lane;
+        for (int k = 0; k < n; ++k) {
+            const float2 e = list[k];
+#pragma unroll
+            for (int h = 0; h < DC_PER_LANE; ++h) {
+                const uint32_t u = w[(size_t)__float_as_int(e.x) * DC_ROWS + 32 * h];
+                if (u != DC_ABSENT) a[h] += __uint_as_float(u << 16) * e.y;
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < DC_PER_LANE; ++h) s_part[warp][lane + 32 * h] = a[h];
+    } else {
         const uint4 *w = d.cols + (size_t)strip * d.n * (DC_ROWS / 8) + (lane & (DC_LANES - 1));
         float acc[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) acc[r] = 0.f;
-        for (int k0 = warp * DC_SLOTS + lane / DC_LANES; k0 - lane / DC_LANES < n; k0 += DC_WARPS * DC_SLOTS * DC_ILP) {
+        for (int k0 = 0; k0 < n; k0 += DC_SLOTS * DC_ILP) {
             uint4 v[DC_ILP];
             float xv[DC_ILP];
 #pragma unroll
             for (int u = 0; u < DC_ILP; ++u) {
-                const int k = k0 + u * DC_WARPS * DC_SLOTS;
+                const int k = k0 + u * DC_SLOTS + lane / DC_LANES;
                 v[u] = make_uint4(0u, 0u, 0u, 0u);
                 xv[u] = 0.f;
-                if (k < n) { const float2 e = s_list[k]; xv[u] = e.y; v[u] = __ldcs(w + (size_t)__float_as_int(e.x) * (DC_ROWS / 8)); }
+                if (k < n) { const float2 e = list[k]; xv[u] = e.y; v[u] = __ldcs(w + (size_t)__float_as_int(e.x) * (DC_ROWS / 8)); }
             }
 #pragma unroll
             for (int u = 0; u < DC_ILP; ++u) {
@@ -243,24 +227,38 @@ k_decode_cols(Device d, const void *__restrict__ x, float *__restrict__ y, float
         for (int i = 0; i < 2; ++i) a2[i] = (h8 ? a4[i + 2] : a4[i]) + __shfl_xor_sync(FULL, h8 ? a4[i] : a4[i + 2], 8);
         *reinterpret_cast<float2 *>(&s_part[warp][(lane & 7) * 8 + (h16 ? 4 : 0) + (h8 ? 2 : 0)]) = make_float2(a2[0], a2[1]);
     }
+    if (lane == 0) s_nz[warp] = nz;
     __syncthreads();
     float sum = 0.f;
     if (tid < DC_ROWS) {
 #pragma unroll
         for (int k = 0; k < DC_WARPS; ++k) sum += s_part[k][tid];
     }
+    int seen = 0;
+    if (tid == 0) {
+#pragma unroll
+        for (int k = 0; k < DC_WARPS; ++k) seen += s_nz[k];
+    }
     if (C > 1) {
         cg::cluster_group cluster = cg::this_cluster();
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         if (tid < DC_ROWS) cluster.map_shared_rank(&s_sum[0][0], 0)[rank * DC_ROWS + tid] = sum;
+        if (tid == 0) cluster.map_shared_rank(s_seen, 0)[rank] = seen;
         cluster.sync();
         if (rank == 0 && tid < DC_ROWS) {
             sum = 0.f;
 #pragma unroll
             for (int r = 0; r < C; ++r) sum += s_sum[r][tid];
         }
+        if (rank == 0 && tid == 0) {
+            seen = 0;
+#pragma unroll
+            for (int r = 0; r < C; ++r) seen += s_seen[r];
+        }
     }
     const int64_t row = (int64_t)strip * DC_ROWS + tid;
     if (rank == 0 && tid < DC_ROWS && row < d.m) y[row] = sum;
+    if (strip == 0 && rank == 0 && tid == 0) dc_record(d, seen, th3, force_path);
 }
 
 constexpr int DCB_WARPS = 16;

@@ -2353,7 +2353,7 @@ static int decode_columns_c(dbspmspv_handle_s *h, CallList &calls, const void *x
         DBS_CUDA(cudaFuncSetAttribute(k_decode_cols<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSED_MAX_SMEM));
         h->cols_configured = true;
     }
-    calls.add(k_decode_cols<C>, strips * C, DC_CTA, (size_t)((d.nb + C - 1) / C) * 16 * sizeof(float2), false, d, x, y, h->ropts.th3_decode, h->ropts.force_path);
+    calls.add(k_decode_cols<C>, strips * C, DC_CTA, (size_t)DC_WARPS * dc_warp_entries(d.nb, C) * sizeof(float2), false, d, x, y, h->ropts.th3_decode, h->ropts.force_path);
     return DBSPMSPV_OK;
 }
 static int decode_columns(dbspmspv_handle_s *h, const void *x, int64_t ldx, float *y, int64_t ldy, int nvec, cudaStream_t st) {
