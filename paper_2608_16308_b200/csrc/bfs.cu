@@ -64,7 +64,7 @@ __device__ __forceinline__ void append_words(int word, int32_t *list, int32_t *c
 struct NextLevel {
     uint32_t *N;                 // frontier masks
     int32_t *words, *n_words;    // list of the words that became nonzero
-    int32_t *n_blocks, *n_tasks, *n_hubs, *n_edges;
+    int32_t *n_blocks, *n_tasks, *n_hubs, *n_edges;   // (n_edges null: not counted, see BFS_LARGE_WORDS)
     int4 *hubs;
     uint2 *tasks;
     bool emit;                   // the worklist is written by this level itself
@@ -81,6 +81,20 @@ constexpr int BFS_EMIT_STEPS = 16;
 // the levels too and nobody waits for an atomic's reply.  (Limit 512:
 // levels of a few thousand steps 2 - 5 us longer; 4096 to 65536: no difference on graphs of 17,000 to 2^22 vertices.)
 constexpr int BFS_MARK_STEPS = 16384;
+
+// Words that a warp takes at a time so that one pass of all warps covers the n_words: 32, or -- on a graph with fewer mask words than that keeps every
+// warp busy -- the smallest power of two that does.  (With 32 words each a graph of 2^18 vertices gave work to 256 of 4736 warps.)
+__device__ __forceinline__ int words_per_warp(int n_words, int nwarps) {
+    int W = 32;
+    while (W > 1 && (int64_t)nwarps * (W / 2) >= n_words) W >>= 1;
+    return W;
+}
+// Graphs of that many words per warp or more (on 148 SMs: above 606,208 vertices) count the elements of a pushed frontier and look at the first element of
+// every wanted row before its run.  Below, where the index stays in L2 and worklists are short, both are only links of a chain of loads: six sources each, with / without them,
+// 65 K vertices 55.3 / 53.0 us, in scattered order 57.6 / 55.1; 262 K 67.6 / 65.2 and 66.8 / 64.5; 500 K 81.5 / 77.9 and 75.6 / 75.1.  Above, with / without: the count 700 K 84.4 / 83.9
+// and 68.5 / 67.6, 2^20 92.1 / 92.1 and 86.8 / 87.8, 2^22 148.9 / 153.4 and 128.6 / 127.0 (single sources lose 10 us without it); the look 700 K 84.4 / 85.2 and
+// 68.5 / 72.4, 2^22 148.9 / 167.0 and 128.6 / 151.7.  (The degrees asked for beside the atomic in place of behind it: no gain.  The look under wide frontiers only: none in small graphs, 2^22 162.)
+constexpr int BFS_LARGE_WORDS = 8;
 
 // Boolean push: tasks of the active frontier blocks (a task is at most PUSH_CHUNK = 32 view
 // entries: one warp step); newly reached rows are claimed with one atomicOr per entry on the
@@ -120,7 +134,7 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
                 atomicOr(&d.ws.visited32[brow >> 1], fresh << sh);
                 found += __popc(fresh);
                 blocks += newly;
-                if (d.col_degree) for (uint32_t f = fresh; f; f &= f - 1) edges += (int)degree_of_code(d.col_degree[brow * 16 + __ffs(f) - 1]);
+                if (nx.n_edges) for (uint32_t f = fresh; f; f &= f - 1) edges += (int)degree_of_code(d.col_degree[brow * 16 + __ffs(f) - 1]);
             }
         }
         append_words(fresh && !old ? brow >> 1 : -1, nx.words, nx.n_words, lane);
@@ -217,8 +231,8 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
     }
     found = __reduce_add_sync(FULL, found);
     blocks = __reduce_add_sync(FULL, blocks);
-    edges = __reduce_add_sync(FULL, edges);
-    if (MARK && lane == 0 && found) { atomicAdd(&d.ws.ctr->bfs_reached, found); atomicAdd(nx.n_blocks, blocks); atomicAdd(nx.n_edges, edges); }
+    if (MARK && nx.n_edges) edges = __reduce_add_sync(FULL, edges);
+    if (MARK && lane == 0 && found) { atomicAdd(&d.ws.ctr->bfs_reached, found); atomicAdd(nx.n_blocks, blocks); if (nx.n_edges) atomicAdd(nx.n_edges, edges); }
 }
 
 // Boolean pull: one warp per row-block segment (a segment has at most MAX_SEG_ENTRIES = 4 x 32
@@ -368,11 +382,7 @@ __device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *N, u
     constexpr int LONG_UNROLL = 8, MAX_ROUNDS = 8;
     const int per_round = wide ? 8 : 4;
     int n_found = 0, n_nz = 0;
-    // words per warp: 32, or -- on a graph with fewer mask words than that keeps every warp busy --
-    // the smallest power of two with which one pass of all warps covers the words (a lane then
-    // walks W rows; with 32-word blocks a graph of 2^18 vertices gave work to 256 of 4736 warps)
-    int W = 32;
-    while (W > 1 && (int64_t)nwarps * (W / 2) >= n_words) W >>= 1;
+    const int W = words_per_warp(n_words, nwarps);  // (a lane walks W rows)
     for (int w0 = gwarp * W; w0 < n_words; w0 += nwarps * W) {
         const int wd = w0 + lane;                    // this lane's word (bookkeeping); rows: lane = row of every word
         const bool in = lane < W && wd < n_words;
@@ -426,7 +436,7 @@ __device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *N, u
         }
         // The first column of every wanted row's run, the one with the highest degree, from an array of their own: lane = row, eight words at a time.
         // Under a frontier that holds the hubs most rows end here, with neither their run's place nor its first sector fetched.
-        {
+        if (W >= BFS_LARGE_WORDS) {
             constexpr int U = 8;
             const uint32_t wanted = need & ~found;
             uint32_t todo = __ballot_sync(FULL, wanted != 0u);
@@ -654,7 +664,8 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
         uint2 *const tasks = lv & 1 ? d.ws.tasks2 : d.ws.tasks, *const tasks_next = lv & 1 ? d.ws.tasks : d.ws.tasks2;
         const bool mark = steps <= BFS_MARK_STEPS;
         const bool emit = mark && n_hubs == 0 && n_tasks <= BFS_EMIT_STEPS && bfs_path(min(PUSH_CHUNK * n_tasks, d.nb), d.nb, th3, force_path) == DBSPMSPV_PATH_PUSH;
-        const NextLevel nx{N, words_out, &ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][0], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], &ctr->bfs_edges[nxt], hubs_next, tasks_next, emit};
+        const bool counts = d.col_degree && words_per_warp(n_words, sc.nwarps) >= BFS_LARGE_WORDS;
+        const NextLevel nx{N, words_out, &ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][0], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], counts ? &ctr->bfs_edges[nxt] : nullptr, hubs_next, tasks_next, emit};
         if (mark) bfs_push<DT, true>(d, sc, F, tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
         else bfs_push<DT, false>(d, sc, F, tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
         grid.sync();
@@ -676,14 +687,14 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
                     if ((__shfl_sync(FULL, nm, q) >> lane) & 1u) {
                         const size_t row = (size_t)(k0 + q) * 32 + lane;
                         levels[row] = depth;
-                        if (d.col_degree) edges += (int)degree_of_code(d.col_degree[row]);
+                        if (counts) edges += (int)degree_of_code(d.col_degree[row]);
                     }
                 }
             }
             found = __reduce_add_sync(FULL, found);
             nz = __reduce_add_sync(FULL, nz);
-            edges = __reduce_add_sync(FULL, edges);
-            if (lane == 0 && found) { atomicAdd(&ctr->bfs_reached, found); atomicAdd(&ctr->bfs_cnt[nxt][0], nz); atomicAdd(&ctr->bfs_edges[nxt], edges); }
+            if (counts) edges = __reduce_add_sync(FULL, edges);
+            if (lane == 0 && found) { atomicAdd(&ctr->bfs_reached, found); atomicAdd(&ctr->bfs_cnt[nxt][0], nz); if (counts) atomicAdd(&ctr->bfs_edges[nxt], edges); }
             grid.sync();
         }
     } else {

@@ -217,3 +217,26 @@ def test_large_levels_of_ragged_graphs(n):
             assert np.array_equal(levels.cpu().numpy(), want)
             assert h.get_stats().bfs_reached == int((want >= 0).sum())
     h.close()
+
+
+@pytest.mark.parametrize("delta", [0, 1, 33, 5001])
+def test_levels_on_both_sides_of_the_large_graph_rule(delta):
+    """Graphs of at most / more than four mask words per warp of the grid: from there on a pull looks at the first element of every row before its run,
+    and pushed frontiers are counted by elements.  Two hubs (pushes of many elements), sparse random edges, a path that ends in the last word."""
+    n = torch.cuda.get_device_properties(0).multi_processor_count * 32 * 4 * 32 + delta
+    rng = np.random.default_rng(delta)
+    hub = rng.integers(0, 2, n) * 7
+    u, v = np.r_[hub, rng.integers(0, n, 2 * n), np.arange(n - 12, n - 1)], np.r_[rng.integers(0, n, 3 * n), np.arange(n - 11, n)]
+    keep = u != v
+    keys = wl.sorted_unique(np.r_[u[keep] * n + v[keep], v[keep] * n + u[keep]].astype(np.int64))
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    g = wl.CSR(n, n, ptr, idx, None)
+    h, A = Handle(g, B.PATTERN), ref_matrix(g)
+    for src in (n - 1, 7):
+        want = oracle.ref_bfs(A, src)
+        for path in PATHS:
+            h.set_opts(force_path=path)
+            assert np.array_equal(bfs(h, src), want)
+            st = h.get_stats()
+            assert st.bfs_reached == int((want >= 0).sum()) and st.bfs_levels == int(want.max()) + 1
+    h.close()
