@@ -2209,13 +2209,16 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     return DBSPMSPV_OK;
 }
 
-// Columns up to which the one-kernel form of a call is the faster one (see small_call.cuh).  Without long columns or payload blocks the chain is two kernels: uniform
-// rows, 16 K / 64 K / 256 K / 1 M of them, 6.2 / 6.3 / 6.5 / 9.9 us whatever x holds, against 6.6 / 7.3 / 6.9 / 7.6 with 48 columns, 7.0 / 7.9 / 7.3 / 8.2 with 96 and
-// 8.4 / 8.6 / 9.0 / 10.0 with 250.  With long columns it is three: R-MAT in scattered order, 256 K / 1 M rows, 9.2 / 13.7 us, against 8.5 / 9.8 with 96 columns,
-// 9.4 / 12 with 160, 9.9 / 11.3 with 250.  (Handles with more payload blocks stay at the old limit: both ways vary by half with the columns that x lists.)
+// Columns up to which the one-kernel form of a call is the faster one (see small_call.cuh).  The chain's first kernels are bound by their launches: two of them without long
+// columns (6.0 us a call on one host, 6.5 on another), three with (8.2 and 9.0); from 2^18 rows on the finishing kernel's tiles add to that.  The one-kernel form
+// goes by the columns, 48 / 64 / 96 / 144 / 224 of them, against the chain on the slower host, uniform rows: 128 K rows 6.7 / 6.8 / 7.3 / 8.1 / 8.4 against 6.5;
+// 256 K 6.8 / 6.9 / 7.4 / 8.2 / 8.6 against 7.7 / 7.2 / 6.5 / 6.5 / 6.5; 512 K 7.0 / 7.1 / 7.6 / 8.4 / 8.9 against 8.4 / 8.0 / 7.8 / 7.7 / 7.3; 700 K 7.2 / 7.3 / 7.7 / 8.6 / 9.0 against
+// 9.8 / 9.7 / 9.4 / 9.0 / 8.6; a million 7.5 / 7.6 / 8.1 / 9.1 / 9.5 against 9.9 / 9.9 / 9.9 / 9.9 / 9.6.  (64 columns up to 2^19 rows and 224 above: 7.6 -> 8.2 us with 65 columns of 512 K rows,
+// 9.1 instead of 7.1 with 224 of 600 K.)  With long columns the form's time jumps when x lists one: means of six R-MAT matrices in scattered order, 16 K rows, 48 / 96 / 144 columns
+// 7.7 / 8.5 / 9.0, 256 K rows, 96 columns 8.5; 1 M rows, 96 / 160 / 250 9.8 / 12 / 11.3 against a chain of 13.7.  (Handles with more payload blocks stay at the old limit: both ways vary by half with the columns that x lists.)
 static int small_call_limit(const dbspmspv_handle_s *h) {
     const Device &d = h->d;
-    if (d.long_cap == 0) return d.m <= (1 << 17) ? 48 : d.m <= (1 << 19) ? 64 : 224;
+    if (d.long_cap == 0) return d.m <= (1 << 17) ? 48 : d.m <= 5 << 16 ? 64 : d.m <= 5 << 17 ? 96 : d.m <= 7 << 17 ? 144 : 224;
     if ((int64_t)d.n_payload * 2048 > d.n_entries) return SMALL_MAX_NNZ_X;
     return d.m <= (1 << 19) ? 96 : 160;
 }

@@ -508,3 +508,33 @@ def test_one_kernel_form_of_a_short_call():
         check_against_oracle((h.y_idx[:kk].cpu().numpy(), h.y_val[:kk].cpu().numpy(), kk), tuple(a[keep] for a in want))
         check_against_oracle(h.run(x), want)                  # the dropped rows left nothing behind
     h.close()
+
+
+@pytest.mark.parametrize("m,hub,limit", [(1 << 17, False, 48), ((1 << 17) + 1, False, 64), (5 << 16, False, 64), ((5 << 16) + 1, False, 96), (5 << 17, False, 96),
+                                         ((5 << 17) + 1, False, 144), (7 << 17, False, 144), ((7 << 17) + 1, False, 224), (70000, True, 96), (1 << 19, True, 96), ((1 << 19) + 1, True, 160)])
+def test_length_of_x_at_which_short_calls_change_over(m, hub, limit):
+    """x of exactly the limit of the one-kernel form and of one entry more, on both sides of every line in the number of rows, without and with a long column:
+    one launch and several, the oracle's result either way, all semirings."""
+    rng = np.random.default_rng(limit)
+    r, c = np.repeat(np.arange(m), 2), rng.integers(0, m, 2 * m)
+    if hub:
+        r, c = np.r_[r, rng.integers(0, m, 6000)], np.r_[c, np.full(6000, 77)]
+    keys = wl.sorted_unique(r.astype(np.int64) * m + c)
+    ptr, idx = wl.csr_from_sorted_keys(m, m, keys)
+    csr = wl.CSR(m, m, ptr, idx, rng.standard_normal(keys.size).astype(np.float32))
+    h, A = Handle(csr, B.F32), ref_matrix(csr)
+    for k in (limit, limit + 1):
+        at = rng.choice(m, k, replace=False).astype(np.int32)
+        if 77 not in at:
+            at[k // 2] = 77
+        x = wl.SparseVec(m, at, rng.standard_normal(k).astype(np.float32))
+        want = oracle.ref_pull(A, x.idx, x.val)
+        before = h.get_stats().kernel_launches
+        check_against_oracle(h.run(x), want)
+        launches = h.get_stats().kernel_launches - before
+        assert launches == 1 if k == limit else launches >= 2 + hub
+        check_against_oracle(h.run(x, semiring=B.OR_AND), want, boolean=True)
+        wi, wv = oracle.ref_minplus(A, x.idx, x.val)
+        yi, yv, _ = h.run(x, semiring=B.MIN_PLUS)
+        assert np.array_equal(yi, wi) and np.array_equal(yv, wv.astype(np.float32))
+    h.close()
