@@ -1761,10 +1761,13 @@ __global__ void __launch_bounds__(CMP_TPB, FOLD ? 5 : 8) k_finish(Device d, int3
     finish_clear_x(d, x_idx, nnz_x, clear, bi, stride, j0);
 }
 
-// The same over two tiles per thread block, for accumulators of more tiles than fit on the GPU at once with results in a good part of the rows: the second tile waits in
-// shared memory, so that a thread block needs no more registers, the two are counted and lined up as one, and most of the second wave with its ticket, loads, count and wait
-// is spared.  (27-point operator, x in runs: 150^3 cells, 2 %, 37.3 -> 32.2 us a call; 160^3, 5 %, 48.8 -> 47.9.  With results in nearly all rows the second tile's way through
-// shared memory costs more than the wave: 144^3, 30 %, 149 -> 154, 150^3, 10 %, 124 -> 130.)
+// The same over two tiles per thread block, for accumulators of more tiles than fit on the GPU at once behind a push of blocks: the second tile waits in shared memory, so
+// that a thread block needs no more registers, the two are counted and lined up as one, and most of the second wave with its ticket, loads, count and wait is spared.
+// What it gains is the tiles that hold nothing, so it is kept to handles whose elements sit in blocks, which x in runs reaches in stretches; one tile / two, us a call at x = 2 / 3 / 4.5 %:
+// 27-point operators, x in runs, 140^3 cells 36.2 / 42.0 / 50.7 and 33.9 / 40.0 / 48.9, 150^3 35.1 / 42.7 / 53.8 and 31.5 / 39.7 / 50.7, 160^3 33.4 / 38.1 / 46.5 and 30.1 / 35.7 / 45.0; bands of 48
+// elements, 4 M rows, 43.1 / 50.1 / 62.2 and 38.5 / 45.2 / 57.0; scattered x within 1 % of each other.  With results in every tile half as many thread blocks are the slower form
+// (uniform rows of 8, 2.5 M of them 15.3 / 17.0 / 20.1 and 17.5 / 19.6 / 22.9, 3.2 M 18.5 / 21.2 / 26.2 and 19.6 / 22.4 / 27.1), also just past the first wave (136^3 scattered 49.4 / 66.8 / 90.9 and
+// 50.6 / 69.0 / 92.7), and in nearly all rows the second tile's way through shared memory costs more than the wave (144^3, 30 %, 149 and 154).
 __global__ void __launch_bounds__(CMP_TPB, 8) k_finish_pair(Device d, int32_t *__restrict__ y_idx, float *__restrict__ y_val,
                                                            int64_t y_capacity, int32_t *__restrict__ y_nnz, int boolean,
                                                            const int32_t *__restrict__ x_idx, int32_t nnz_x, int clear,
@@ -2325,7 +2328,7 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
     if (per_block > 1)
         calls.add(d.hub_on ? k_finish_wide<true> : k_finish_wide<false>, (nt + per_block - 1) / per_block + extra, CMP_TPB, 0, calls.n > 0, d, per_block, y_idx, y_val, y_capacity, y_nnz,
                   minplus ? 2 : (int)boolean, x_idx, nnz_x, clear, d.hub_on ? (minplus ? 2 : 1) : 0, row_mask, complement);
-    else if (nt > 8 * h->sm_count && !d.hub_on && (int64_t)nnz_x * 16 <= d.n)      // (see k_finish_pair)
+    else if ((h->heavy_stage || h->payload_rich) && nt > 9 * h->sm_count && !d.hub_on && (int64_t)nnz_x * 16 <= d.n)      // (see k_finish_pair)
         calls.add(k_finish_pair, (nt + 1) / 2 + extra, CMP_TPB, 0, calls.n > 0, d, y_idx, y_val, y_capacity, y_nnz, minplus ? 2 : (int)boolean, x_idx, nnz_x, clear, row_mask, complement);
     else
         calls.add(d.hub_on ? k_finish<true> : k_finish<false>, nt + extra, CMP_TPB, 0, calls.n > 0, d, y_idx, y_val, y_capacity, y_nnz, minplus ? 2 : (int)boolean, x_idx, nnz_x, clear,

@@ -105,3 +105,44 @@ def test_batches_in_a_row_over_columns():
 
 def test_batches_in_a_row_over_blocks():
     check_batches_in_a_row(1008, 1040, 4)           # (too few rows for the column copy: tensor-core kernel and its two fallbacks)
+
+
+# one thread block per strip: up to 8192 columns are a warp's first round over x, the widest layer fills the lists' shared memory exactly; two per strip: up to 16384
+@pytest.mark.parametrize("shape", [(4768, 8191), (4768, 8192), (4768, 8193), (4800, 10000), (4768, 25600), (4000, 16385), (4000, 25600)])
+def test_one_vector_of_more_than_one_round(shape):
+    """Single vectors whose warps take more than one round over x: every entry active, a third of them scattered, in runs, only columns of the later rounds, and a
+    non-finite entry in the first, in a later round and in both."""
+    m, n = shape
+    gen = torch.Generator(device=DEV).manual_seed(n)
+    keep = torch.rand((m, n), generator=gen, device=DEV) < 0.3
+    val = torch.randn((m, n), generator=gen, device=DEV).to(torch.bfloat16).float()
+    val[val == 0] = 0.5
+    ptr = torch.zeros(m + 1, dtype=torch.int64, device=DEV)
+    torch.cumsum(keep.sum(dim=1), 0, out=ptr[1:])
+    w = wl.CSR(m, n, ptr.cpu().numpy(), keep.nonzero()[:, 1].to(torch.int32).cpu().numpy(), val[keep].cpu().numpy())
+    del val
+    h, A = Handle(w, B.BF16), ref_matrix(w, bf16=True)
+    rng = np.random.default_rng(m + n)
+    full = np.where(rng.random(n) < 0.5, -1.0, 1.0) * (0.1 + rng.random(n))
+    cut = 16384 if m < 4737 else 8192
+    late = np.arange(n) >= min(cut, n - 16)
+    runs = (np.arange(n) // 192) % 3 == 1
+    xs = [full, full * (rng.random(n) < 0.3), full * runs, full * late, full * (rng.random(n) < 0.1)]
+    for at in ([5], [n - 3], [7, n - 1]):
+        xs.append(full * (rng.random(n) < 0.3))
+        xs[-1][at] = np.array([np.inf, np.nan][:len(at)])
+    for x in xs:
+        x = wl.bf16_bits_to_f32(wl.f32_to_bf16_bits(x.astype(np.float32)))
+        y = torch.full((m + 3,), 55.0, device=DEV)
+        before = h.get_stats().kernel_launches
+        B.dbspmspv_decode(h.h, bits(x), y)
+        torch.cuda.synchronize()
+        st = h.get_stats()
+        assert st.kernel_launches - before == 1
+        active = np.zeros((n + 15) // 16 * 16, bool)
+        active[:n] = x != 0
+        assert st.last_n_nzblk == int(active.reshape(-1, 16).any(axis=1).sum())
+        yh = y.cpu().numpy()
+        check(yh[:m], *oracle.ref_decode(A, x)[:2])
+        assert (yh[m:] == 55.0).all()
+    h.close()

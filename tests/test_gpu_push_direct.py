@@ -225,7 +225,8 @@ def test_wide_finish_behind_a_push_of_whole_blocks(tiles):
     h.close()
 
 
-@pytest.mark.parametrize("m", [2048 * 1185 - 5, 2048 * 1186, 2048 * 1187 + 16])       # (148 SMs: more than one wave; a last pair of one tile, of two)
+# (148 SMs: more than one wave, one tile per thread block; from 1333 tiles on the handle of blocks takes pairs: a last pair of one tile, of two)
+@pytest.mark.parametrize("m", [2048 * 1185 - 5, 2048 * 1186, 2048 * 1187 + 16, 2048 * 1333 - 5, 2048 * 1334, 2048 * 1335 + 16])
 @pytest.mark.parametrize("blocks", [False, True])
 def test_paired_finish(m, blocks):
     """The finishing kernel of two tiles per thread block behind a longer x, in turn with that of a short x on the same handle (another number of tiles per
