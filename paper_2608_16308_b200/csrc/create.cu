@@ -778,6 +778,40 @@ int bits_for(uint64_t v) { int b = 0; while (v) { ++b; v >>= 1; } return b ? b :
             if (cudaMalloc(&p__, b__) != cudaSuccess) return DBSPMSPV_ERR_ALLOC; } \
         (ptr) = static_cast<decltype(ptr)>(p__); } while (0)
 
+// Every row's elements by weight (Device::weightrun).  What is alive at once decides how large a matrix can be built: the sort holds 24 bytes per stored element beside the
+// builder's keys and values (12), so it runs when the encoder's arrays are gone and the block-CSC view is not there yet.  (Peak of a create in bytes per stored element with the
+// sort beside the encoder's arrays and both views / so: 27-point operator on 150^3 cells 69.1 / 42.5, and 42.0 before the runs held payload elements; R-MAT 84.6 / 71.7, uniform rows of
+// eight 89.7 / 76.0, whose peak is the encoder.)  Where it does not fit all the same, the handle goes without: its searches push.
+int weight_index(dbspmspv_handle_s *h, TempPool &tp, int64_t nnz, const uint64_t *ukey, const float *weights, cudaStream_t st) {
+    Device &d = h->d;
+    const int64_t m = d.m, ptr_pad = (m + 1 + 31) / 32 * 32;
+    uint64_t *keys = nullptr, *keys_alt = nullptr;
+    uint32_t *from = nullptr, *from_alt = nullptr;
+    int32_t *ptr = nullptr;                         // (one allocation: row pointers, lightest weights)
+    uint2 *run = nullptr;
+    auto make = [&]() -> int {
+        DBS_GET(keys, nnz); DBS_GET(keys_alt, nnz); DBS_GET(from, nnz); DBS_GET(from_alt, nnz);
+        DBS_KEEP(ptr, ptr_pad + m); DBS_KEEP(run, nnz + 4);
+        k_weightrun_keys<<<grid_for(nnz), TPB, 0, st>>>(nnz, ukey, weights, keys, from);
+        DBS_TRY(sort_pairs(tp, keys, keys_alt, from, from_alt, nnz, SSSP_WEIGHT_BITS + bits_for((uint64_t)m), st));
+        k_rowrun_ptr<<<grid_for(m + 1), TPB, 0, st>>>(m, keys, SSSP_WEIGHT_BITS, (int32_t)nnz, ptr);
+        k_weightrun<<<grid_for(nnz + 4), TPB, 0, st>>>(nnz, from, ukey, weights, run);
+        k_row_lightest<<<grid_for(m), TPB, 0, st>>>(m, ptr, run, reinterpret_cast<float *>(ptr + ptr_pad));
+        DBS_CUDA(cudaStreamSynchronize(st));
+        return DBSPMSPV_OK;
+    };
+    const int status = make();
+    if (status == DBSPMSPV_ERR_ALLOC) DBS_CUDA(cudaStreamSynchronize(st));
+    for (void *p : {(void *)keys, (void *)keys_alt, (void *)from, (void *)from_alt}) if (p) tp.release(p);
+    if (status != DBSPMSPV_OK) {
+        cudaFree(ptr); cudaFree(run);
+        return status == DBSPMSPV_ERR_ALLOC ? DBSPMSPV_OK : status;
+    }
+    d.weight_ptr = ptr; d.weightrun = run; d.row_lightest = reinterpret_cast<const float *>(ptr + ptr_pad);
+    h->bfs_index_bytes += nnz * 8 + (m * 2 + 1) * 4;
+    return DBSPMSPV_OK;
+}
+
 int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t *row_ptr,
           const int32_t *rows, const int32_t *cols, const void *val, cudaStream_t st) {
     TempPool tp;
@@ -904,10 +938,7 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
     // kernel acts on
     k_fill_words<<<1, VIEW_PAD, 0, st>>>(d.csr.idx + n_entries, VIEW_PAD, PAD_IDX);
     DBS_CUDA(cudaMemsetAsync(d.csr.w + n_entries, 0, VIEW_PAD * 4, st)); DBS_CUDA(cudaMemsetAsync(d.csr.aux + n_entries, 0, VIEW_PAD, st));
-    DBS_KEEP(d.csc.colptr, (int64_t)d.nb * 17); d.csr.colptr = nullptr;
-    DBS_KEEP(d.csc.ptr, d.nb + 1); DBS_KEEP(d.csc.idx, n_entries + VIEW_PAD); DBS_KEEP(d.csc.w, n_entries + VIEW_PAD); DBS_KEEP(d.csc.aux, n_entries + VIEW_PAD);
-    DBS_CUDA(cudaMemsetAsync(d.csc.idx + n_entries, 0, VIEW_PAD * 4, st)); DBS_CUDA(cudaMemsetAsync(d.csc.w + n_entries, 0, VIEW_PAD * 4, st)); DBS_CUDA(cudaMemsetAsync(d.csc.aux + n_entries, 0, VIEW_PAD, st));
-    DBS_KEEP(h->csc2csr, n_entries);
+    d.csr.colptr = nullptr;
     DBS_KEEP(h->block_row, n_entries);
     { int32_t *t; DBS_KEEP(t, (int64_t)d.mb + 1); d.csr_inl = t; }
     d.entry_row = h->block_row;
@@ -933,30 +964,6 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         DBS_CUDA(cudaStreamSynchronize(st));
         tp.release(blk_start); tp.release(block_of); tp.release(poff); tp.release(psize);
         tp.release(brow); tp.release(bcol); tp.release(ecount); tp.release(eoff); tp.release(type);
-        // every row's elements by weight, for the pulled steps of db_sssp
-        d.weightrun = nullptr; d.weight_ptr = nullptr; d.row_lightest = nullptr;
-        h->bfs_index_bytes = 0;
-        if (m == n && !h->copts.no_bfs_index && dt == DBSPMSPV_F32 && !h->heavy_stage && nnzu > 0 && nnzu <= 0x7FFFFFF0) {
-            uint64_t *wk, *wk_alt;
-            uint32_t *wv, *wv_alt;
-            int32_t *wp;
-            uint2 *wr;
-            const float *weights = static_cast<const float *>(uval);
-            DBS_GET(wk, nnzu); DBS_GET(wk_alt, nnzu); DBS_GET(wv, nnzu); DBS_GET(wv_alt, nnzu);
-            const int64_t wp_pad = (m + 1 + 31) / 32 * 32;          // (one allocation: row pointers, lightest weights)
-            DBS_KEEP(wp, wp_pad + m); DBS_KEEP(wr, nnzu + 4);
-            float *lightest = reinterpret_cast<float *>(wp + wp_pad);
-            d.weight_ptr = wp; d.weightrun = wr; d.row_lightest = lightest;
-            k_weightrun_keys<<<grid_for(nnzu), TPB, 0, st>>>(nnzu, ukey, weights, wk, wv);
-            DBS_TRY(sort_pairs(tp, wk, wk_alt, wv, wv_alt, nnzu, SSSP_WEIGHT_BITS + bits_for((uint64_t)m), st));
-            k_rowrun_ptr<<<grid_for(m + 1), TPB, 0, st>>>(m, wk, SSSP_WEIGHT_BITS, (int32_t)nnzu, wp);
-            k_weightrun<<<grid_for(nnzu + 4), TPB, 0, st>>>(nnzu, wv, ukey, weights, wr);
-            k_row_lightest<<<grid_for(m), TPB, 0, st>>>(m, wp, wr, lightest);
-            DBS_CUDA(cudaStreamSynchronize(st));
-            tp.release(wk); tp.release(wk_alt); tp.release(wv); tp.release(wv_alt);
-            h->bfs_index_bytes += nnzu * 8 + ((int64_t)m * 2 + 1) * 4;
-        }
-        tp.release(ukey); tp.release(uval);
         DBS_GET(k1, n_entries); DBS_GET(k1_alt, n_entries); DBS_GET(ids, n_entries); DBS_GET(ids_alt, n_entries);
         if (n_entries) {
             k_csr_keys<<<grid_for(n_entries), TPB, 0, st>>>(n_entries, t_row, t_idx, t_aux, k1, ids);
@@ -969,6 +976,11 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         tp.release(t_idx); tp.release(t_w); tp.release(t_aux); tp.release(t_row);
         tp.release(k1); tp.release(k1_alt); tp.release(ids); tp.release(ids_alt);
     }
+    // every row's elements by weight, for the pulled steps of db_sssp (here: see weight_index)
+    h->bfs_index_bytes = 0;
+    if (m == n && !h->copts.no_bfs_index && dt == DBSPMSPV_F32 && !h->heavy_stage && nnzu > 0 && nnzu <= 0x7FFFFFF0)
+        DBS_TRY(weight_index(h, tp, nnzu, ukey, static_cast<const float *>(uval), st));
+    tp.release(ukey); tp.release(uval);
 
     // Hub row blocks: the (at most HUB_BLOCKS_MAX) row blocks with the most view entries, if
     // they hold HUB_BLOCK_MIN_ENTRIES or more.  Chosen on the host from the row block pointers.
@@ -1003,6 +1015,10 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
 
     // block-CSC view: sort the primary entries by column block, and inside it payload entries
     // first (by row block), then the INLINE elements column by column
+    DBS_KEEP(d.csc.colptr, (int64_t)d.nb * 17);
+    DBS_KEEP(d.csc.ptr, d.nb + 1); DBS_KEEP(d.csc.idx, n_entries + VIEW_PAD); DBS_KEEP(d.csc.w, n_entries + VIEW_PAD); DBS_KEEP(d.csc.aux, n_entries + VIEW_PAD);
+    DBS_CUDA(cudaMemsetAsync(d.csc.idx + n_entries, 0, VIEW_PAD * 4, st)); DBS_CUDA(cudaMemsetAsync(d.csc.w + n_entries, 0, VIEW_PAD * 4, st)); DBS_CUDA(cudaMemsetAsync(d.csc.aux + n_entries, 0, VIEW_PAD, st));
+    DBS_KEEP(h->csc2csr, n_entries);
     {
         uint64_t *k2, *k2_alt;
         int32_t *ids, *ids_alt, *bcol_sorted;
