@@ -591,8 +591,11 @@ __device__ void sssp_pull_long(const Device &d, const SsspState &s, const float 
 
 constexpr int SSSP_SMEM = (int)(sizeof(SsspShared) > sizeof(SsspPullShared) ? sizeof(SsspShared) : sizeof(SsspPullShared));
 static_assert(sizeof(SsspListShared) <= sizeof(SsspShared), "the phases share one allocation");
+// The arguments stay in the constant bank: the lists and bitmaps are taken by the step's number, for which every thread kept a copy of its own in local memory, that
+// spilled more besides (216 -> 88 bytes of stack; R-MAT 300 K / 500 K / 2^20 vertices 242 / 252 / 359 -> 222 / 227 / 331 us a search, in scattered order 202 / 237 / 333 -> 186 / 217 / 306; 27-point
+// operator on 90^3 cells, an inner source, 3029 -> 2947).  The phases as functions of their own, which share no registers: 233 / 239 / 343 us.
 template <int DT>
-__global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(Device d, SsspState s, int32_t src, float *dist, int start, int max_steps, unsigned long long pull_edges) {
+__global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ Device d, const __grid_constant__ SsspState s, int32_t src, float *dist, int start, int max_steps, unsigned long long pull_edges) {
     namespace cg = cooperative_groups;
     extern __shared__ __align__(16) uint8_t s_dyn[];
     SsspShared &sh = *reinterpret_cast<SsspShared *>(s_dyn);
