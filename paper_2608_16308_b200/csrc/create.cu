@@ -801,7 +801,7 @@ int weight_index(dbspmspv_handle_s *h, TempPool &tp, int64_t nnz, const uint64_t
         return DBSPMSPV_OK;
     };
     const int status = make();
-    if (status == DBSPMSPV_ERR_ALLOC) DBS_CUDA(cudaStreamSynchronize(st));
+    if (status == DBSPMSPV_ERR_ALLOC) { cudaGetLastError(); DBS_CUDA(cudaStreamSynchronize(st)); }
     for (void *p : {(void *)keys, (void *)keys_alt, (void *)from, (void *)from_alt}) if (p) tp.release(p);
     if (status != DBSPMSPV_OK) {
         cudaFree(ptr); cudaFree(run);
