@@ -98,11 +98,11 @@ constexpr int BFS_LARGE_WORDS = 8;
 
 // Boolean push: tasks of the active frontier blocks (a task is at most PUSH_CHUNK = 32 view
 // entries: one warp step); newly reached rows are claimed with one atomicOr per entry on the
-// next-frontier masks (the winner writes the level).  Like the pull, the loop is software-
+// next-frontier masks.  Like the pull, the loop is software-
 // pipelined: while task k is evaluated, the visited masks of k+1, the view entries of k+2 and
 // the task record of k+3 (in this warp's stride) are in flight.
-// The winner also lists the word it turned nonzero and, with MARK, does the level's bookkeeping for the vertex: it is marked visited
-// and, if asked for (NextLevel::emit), the tasks of its column go to the next level's worklist.
+// With MARK the winner does the level's bookkeeping for the vertex: it writes its level, marks it visited, lists the word it turned nonzero
+// and, if asked for (NextLevel::emit), the tasks of its column go to the next level's worklist.  Without it nobody looks at a reply: all that is the pass behind the level.
 template <int DT, bool MARK>
 __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, const uint2 *tasks, int n_recs, const int4 *hubs, int n_hubs,
                          int32_t *levels, int depth, const NextLevel &nx) {
@@ -130,15 +130,13 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
         const bool newly = fresh && ((old >> sh) & 0xFFFFu) == 0;
         if (fresh) {
             write_levels(levels, brow, fresh, depth);
-            if (MARK) {
-                atomicOr(&d.ws.visited32[brow >> 1], fresh << sh);
-                found += __popc(fresh);
-                blocks += newly;
-                if (nx.n_edges) for (uint32_t f = fresh; f; f &= f - 1) edges += (int)degree_of_code(d.col_degree[brow * 16 + __ffs(f) - 1]);
-            }
+            atomicOr(&d.ws.visited32[brow >> 1], fresh << sh);
+            found += __popc(fresh);
+            blocks += newly;
+            if (nx.n_edges) for (uint32_t f = fresh; f; f &= f - 1) edges += (int)degree_of_code(d.col_degree[brow * 16 + __ffs(f) - 1]);
         }
         append_words(fresh && !old ? brow >> 1 : -1, nx.words, nx.n_words, lane);
-        if (!MARK || !nx.emit) return;
+        if (!nx.emit) return;
         // the vertices found, 32 at a time (blocks with a payload reach several rows at once): vertex k belongs to the last lane whose prefix is <= k
         int incl = __popc(fresh);
 #pragma unroll

@@ -20,7 +20,8 @@
 //   * Several vectors (k_decode_cols_batch) share one pass over the union of their columns on the tensor cores: D[vector][row] += X[vector][k] W[k][row],
 //     16 columns per mma.sync m16n8k16, the W fragments straight from global memory -- a lane loads eight rows of the four columns its fragment
 //     holds and pairs the columns with byte permutes, no shared memory and no expansion in between.
-//   * A non-finite x entry may only meet stored elements: such calls (checked while x is blocked) take a plain loop that tests every element.
+//   * A non-finite x entry may only meet stored elements: what met one while x was blocked -- the warp, of a single vector; the whole call, of several -- takes a plain
+//     loop that tests every element.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -299,7 +300,9 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
     __shared__ int s_cnt[DCB_WARPS], s_nz[DCB_WARPS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // While x is staged nothing else asks for weights: the beginning of this block's piece, as it lies when most columns are reached, goes to L2 meanwhile.
-    // (Large layers and three vectors or more: 11008 x 4096 and eight vectors 25.1 -> 24.5 us; 3000 x 3000 no gain, 1500 x 1500 0.3 longer.)
+    // (Large layers and three vectors or more.  Five layers in turn, so that none waits in L2, without / with it: 12288 x 4096, three vectors with 2 / 5 / 15 / 30 % active entries 12.0 / 14.4 /
+    // 19.2 / 24.4 and 11.5 / 13.8 / 18.4 / 23.3 us, eight 18.0 / 21.8 / 29.1 / 27.7 and 17.6 / 21.2 / 28.2 / 27.0; 9000 x 2000, three 9.0 / 9.7 / 12.1 / 14.7 and 9.1 / 9.7 / 11.8 / 14.1.  It pays with few
+    // active entries too.  3000 x 3000 no gain, 1500 x 1500 0.3 longer.)
     {
         const int64_t total = (d.m + DC_ROWS - 1) / DC_ROWS * d.n * DC_ROWS * 2, from = (int64_t)((double)total * blockIdx.x / gridDim.x) / 128 * 128 + (int64_t)tid * DCB_PREFETCH;
         if (total >= DCB_PREFETCH_MIN && nvec > 2 && tid < 8 && from + DCB_PREFETCH <= total)

@@ -10,7 +10,8 @@
 //   long     the listed long runs and payload runs, a warp per chunk (only if there are any);
 //   settle   the marked vertices copy their word into the caller's distances -- the values the next
 //            step starts from, which no one lowers meanwhile -- and are counted;
-// with a grid barrier after each.  A step that reaches few edges also lists what it marks; a frontier that is listed and short is expanded
+// with a grid barrier after each.  A step that reaches few edges (of INLINE runs, which is what is counted: steps of a 27-point operator list a little longer, and gain by it
+// like the others) also lists what it marks; a frontier that is listed and short is expanded
 // from its list in one phase, long runs and payload entries included, and settled by one thread block (sssp_expand_list).  A step finds the same improvements, distance for distance, as the product did: `word`
 // holds the minimum over everything seen so far, a vertex is marked iff its word went below the distance it had before the step.
 //
@@ -32,12 +33,12 @@ constexpr int SSSP_WARPS = SSSP_CTA / 32;
 constexpr int SSSP_WORDS = SSSP_CTA / 8;          // frontier words of a thread block's round: eight threads per word, four columns each
 constexpr int SSSP_COLS = SSSP_CTA * 4;
 constexpr int SSSP_ILP = 4;                       // warp steps in flight
-// A step whose frontier reaches more than this share of the stored elements is pulled.  Shares of 2 / 5 / 10 / 20 %: symmetrised R-MAT scale 20,
-// three sources, 559 - 661 / 561 - 670 / 571 - 664 / 575 - 665 us a search, with its vertices in scattered order 354 - 415 / 355 - 415 / 316 - 372 / 353 - 372;
-// scale 17 within 7 % of each other.
+// A step whose frontier reaches more than this share of the stored elements is pulled.  Shares of 5 / 10 / 15 %, symmetrised R-MAT, means of four sources, in brackets with the
+// vertices in scattered order: 40 K vertices 168 / 168 / 168 us a search (157 / 157 / 159), 131 K 187 / 184 / 187 (169 / 168 / 168), 300 K 223 / 209 / 209 (185 / 191 / 190),
+// 500 K 228 / 233 / 233 (217 / 229 / 228), 2^20 331 / 344 / 351 (305 / 299 / 308).
 constexpr float SSSP_PULL_SHARE = 0.05f;
-// Rounds of four elements that a lane walks of a row.  2 / 4 / 6 / 8: R-MAT scale 20, two sources, 514 / 466 / 451 / 459 and 418 / 384 / 372 / 381 us a search, with
-// its vertices in scattered order 487 / 436 / - / 423.
+// Rounds of four elements that a lane walks of a row.  4 / 6 / 8, the same matrices: 131 K vertices 184 / 185 / 187 us a search (164 / 166 / 169), 300 K 221 / 221 / 223 (186 / 184 / 185),
+// 500 K 234 / 230 / 228 (222 / 217 / 217), 2^20 340 / 332 / 331 (317 / 308 / 305).
 constexpr int SSSP_ROUNDS = 8;
 constexpr int SSSP_CHUNK = 512;                   // elements of a listed chunk of a longer row
 // A step whose frontier reaches at most so many edges lists the vertices it marks; a list of at most SSSP_LIST vertices serves the next step.
@@ -375,14 +376,14 @@ __device__ __forceinline__ int sssp_bound(float xmin, float w) {
 // cannot improve it: smallest distance of the frontier + weight >= the row's best.  In the late large steps of an R-MAT search that leaves a
 // seventh of the elements, and a row reached for the first time soon has a best of its own.  Columns outside the
 // frontier improve nothing (their edges were relaxed when they entered it), so they need no test.
-// Rows that their lightest element (Device::row_lightest) cannot improve are sorted out 64 at a time; the others go to a queue of the warp, from which
+// Rows that their lightest element (Device::row_lightest) cannot improve are sorted out 32 at a time; the others go to a queue of the warp, from which
 // a lane takes the next one as soon as it has finished a row, four elements (one 32-byte sector) a round.  What is left of a row that has not
 // stopped after SSSP_ROUNDS rounds is listed in chunks, which all warps share out behind a grid barrier (walked by the warp that met them, the
 // hub rows of an R-MAT graph, neighbours all, took one warp 300 us); of a row of several chunks only those whose first weight can still improve it.
 // Handles of unit weights walk the row-run index.
-// What bounds it: the L1 tag stage, a distance gathered per element (12 M in the first pulled step of R-MAT scale 20, about one a clock and SM), and the rows that come
-// last.  That step took 156 us when a lane walked seven rows of its own and the blocks with a payload followed, a warp at a time, 80 now; the whole search 669, 561 and
-// 532 us from three sources, 443, 364 and 346 now; in scattered order 355 - 466, 303 - 407 now.  A frontier bitmap in shared memory in front of the gathers: 80 -> 103 (L1 is what it
+// What bounds it: a distance gathered per element, one a clock and SM at most (12 M in the first pulled step of R-MAT scale 20: 41 of its 80 us), then the rows that come last, while
+// most warps stand at the barrier (the L1 is 14 % busy over a whole search).  That step took 156 us when a lane walked seven rows of its own and the blocks with a payload followed, a warp
+// at a time; the whole search 670, 560 and 530 us from three sources, 400, 328 and 312 now; in scattered order 354 - 466, 270 - 367 now.  A frontier bitmap in shared memory in front of the gathers: 80 -> 103 (L1 is what it
 // takes away); less shared memory by half the columns a round in sssp_expand: within 2 %.
 struct SsspPullShared {
     int4 queue[SSSP_WARPS][64];       // {row, first, end, best so far} of the rows that wait for a lane
