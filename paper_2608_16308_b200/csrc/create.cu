@@ -778,10 +778,10 @@ int bits_for(uint64_t v) { int b = 0; while (v) { ++b; v >>= 1; } return b ? b :
             if (cudaMalloc(&p__, b__) != cudaSuccess) return DBSPMSPV_ERR_ALLOC; } \
         (ptr) = static_cast<decltype(ptr)>(p__); } while (0)
 
-// Every row's elements by weight (Device::weightrun).  What is alive at once decides how large a matrix can be built: the sort holds 24 bytes per stored element beside the
-// builder's keys and values (12), so it runs when the encoder's arrays are gone and the block-CSC view is not there yet.  (Peak of a create in bytes per stored element with the
-// sort beside the encoder's arrays and both views / so: 27-point operator on 150^3 cells 69.1 / 42.5, and 42.0 before the runs held payload elements; R-MAT 84.6 / 71.7, uniform rows of
-// eight 89.7 / 76.0, whose peak is the encoder.)  Where it does not fit all the same, the handle goes without: its searches push.
+// Every row's elements by weight (Device::weightrun).  Its sort holds 24 bytes per stored element beside the builder's keys and values, the encoder's arrays and both views, which on
+// handles with payload blocks is the peak of a create (27-point operator on 150^3 cells 69 bytes per element, 42 without; R-MAT and uniform rows have theirs, 85 and 90, in the
+// encoder).  Where that does not fit the handle goes without: its searches push.  (Sorted between the two views, the block-CSC view allocated behind it: 43, 72 and 76 bytes, but creates
+// 3 % longer, 9 % on 16 K rows.)
 int weight_index(dbspmspv_handle_s *h, TempPool &tp, int64_t nnz, const uint64_t *ukey, const float *weights, cudaStream_t st) {
     Device &d = h->d;
     const int64_t m = d.m, ptr_pad = (m + 1 + 31) / 32 * 32;
@@ -938,7 +938,10 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
     // kernel acts on
     k_fill_words<<<1, VIEW_PAD, 0, st>>>(d.csr.idx + n_entries, VIEW_PAD, PAD_IDX);
     DBS_CUDA(cudaMemsetAsync(d.csr.w + n_entries, 0, VIEW_PAD * 4, st)); DBS_CUDA(cudaMemsetAsync(d.csr.aux + n_entries, 0, VIEW_PAD, st));
-    d.csr.colptr = nullptr;
+    DBS_KEEP(d.csc.colptr, (int64_t)d.nb * 17); d.csr.colptr = nullptr;
+    DBS_KEEP(d.csc.ptr, d.nb + 1); DBS_KEEP(d.csc.idx, n_entries + VIEW_PAD); DBS_KEEP(d.csc.w, n_entries + VIEW_PAD); DBS_KEEP(d.csc.aux, n_entries + VIEW_PAD);
+    DBS_CUDA(cudaMemsetAsync(d.csc.idx + n_entries, 0, VIEW_PAD * 4, st)); DBS_CUDA(cudaMemsetAsync(d.csc.w + n_entries, 0, VIEW_PAD * 4, st)); DBS_CUDA(cudaMemsetAsync(d.csc.aux + n_entries, 0, VIEW_PAD, st));
+    DBS_KEEP(h->csc2csr, n_entries);
     DBS_KEEP(h->block_row, n_entries);
     { int32_t *t; DBS_KEEP(t, (int64_t)d.mb + 1); d.csr_inl = t; }
     d.entry_row = h->block_row;
@@ -964,6 +967,11 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         DBS_CUDA(cudaStreamSynchronize(st));
         tp.release(blk_start); tp.release(block_of); tp.release(poff); tp.release(psize);
         tp.release(brow); tp.release(bcol); tp.release(ecount); tp.release(eoff); tp.release(type);
+        // every row's elements by weight, for the pulled steps of db_sssp
+        h->bfs_index_bytes = 0;
+        if (m == n && !h->copts.no_bfs_index && dt == DBSPMSPV_F32 && !h->heavy_stage && nnzu > 0 && nnzu <= 0x7FFFFFF0)
+            DBS_TRY(weight_index(h, tp, nnzu, ukey, static_cast<const float *>(uval), st));
+        tp.release(ukey); tp.release(uval);
         DBS_GET(k1, n_entries); DBS_GET(k1_alt, n_entries); DBS_GET(ids, n_entries); DBS_GET(ids_alt, n_entries);
         if (n_entries) {
             k_csr_keys<<<grid_for(n_entries), TPB, 0, st>>>(n_entries, t_row, t_idx, t_aux, k1, ids);
@@ -976,11 +984,6 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
         tp.release(t_idx); tp.release(t_w); tp.release(t_aux); tp.release(t_row);
         tp.release(k1); tp.release(k1_alt); tp.release(ids); tp.release(ids_alt);
     }
-    // every row's elements by weight, for the pulled steps of db_sssp (here: see weight_index)
-    h->bfs_index_bytes = 0;
-    if (m == n && !h->copts.no_bfs_index && dt == DBSPMSPV_F32 && !h->heavy_stage && nnzu > 0 && nnzu <= 0x7FFFFFF0)
-        DBS_TRY(weight_index(h, tp, nnzu, ukey, static_cast<const float *>(uval), st));
-    tp.release(ukey); tp.release(uval);
 
     // Hub row blocks: the (at most HUB_BLOCKS_MAX) row blocks with the most view entries, if
     // they hold HUB_BLOCK_MIN_ENTRIES or more.  Chosen on the host from the row block pointers.
@@ -1015,10 +1018,6 @@ int build(dbspmspv_handle_s *h, int64_t m, int64_t n, int64_t nnz, const int64_t
 
     // block-CSC view: sort the primary entries by column block, and inside it payload entries
     // first (by row block), then the INLINE elements column by column
-    DBS_KEEP(d.csc.colptr, (int64_t)d.nb * 17);
-    DBS_KEEP(d.csc.ptr, d.nb + 1); DBS_KEEP(d.csc.idx, n_entries + VIEW_PAD); DBS_KEEP(d.csc.w, n_entries + VIEW_PAD); DBS_KEEP(d.csc.aux, n_entries + VIEW_PAD);
-    DBS_CUDA(cudaMemsetAsync(d.csc.idx + n_entries, 0, VIEW_PAD * 4, st)); DBS_CUDA(cudaMemsetAsync(d.csc.w + n_entries, 0, VIEW_PAD * 4, st)); DBS_CUDA(cudaMemsetAsync(d.csc.aux + n_entries, 0, VIEW_PAD, st));
-    DBS_KEEP(h->csc2csr, n_entries);
     {
         uint64_t *k2, *k2_alt;
         int32_t *ids, *ids_alt, *bcol_sorted;

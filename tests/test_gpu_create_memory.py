@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 def test_index_by_weight_is_left_out_where_it_does_not_fit():
-    """27-point operator on 102^3 cells (28 M elements, a good part of them in blocks).  With 100 bytes per stored element left every index is built; with 50 the
+    """27-point operator on 102^3 cells (28 M elements, a good part of them in blocks).  With 100 bytes per stored element left every index is built; with 56 the
     runs by weight, whose sort is the peak of the build, do not fit, and the handle comes without them.  Weights of one: the distances are the
     Chebyshev distances on the grid, either way."""
     d = 102
@@ -26,7 +26,7 @@ def test_index_by_weight_is_left_out_where_it_does_not_fit():
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     cudart, index = ctypes.CDLL("libcudart.so.12"), []
-    for left in (100, 50):
+    for left in (100, 56):
         held = ctypes.c_void_p()
         assert cudart.cudaMalloc(ctypes.byref(held), ctypes.c_size_t(torch.cuda.mem_get_info()[0] - left * g.nnz)) == 0
         try:
