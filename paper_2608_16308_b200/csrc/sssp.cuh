@@ -382,7 +382,7 @@ __device__ __forceinline__ int sssp_bound(float xmin, float w) {
 // hub rows of an R-MAT graph, neighbours all, took one warp 300 us); of a row of several chunks only those whose first weight can still improve it.
 // Handles of unit weights walk the row-run index.
 // What bounds it: a distance gathered per element, one a clock and SM at most (12 M in the first pulled step of R-MAT scale 20: 41 of its 80 us), then the rows that come last, while
-// most warps stand at the barrier (the L1 is 14 % busy over a whole search).  That step took 156 us when a lane walked seven rows of its own and the blocks with a payload followed, a warp
+// most warps stand at the barrier (the L1 is 11 % busy over a whole search).  That step took 156 us when a lane walked seven rows of its own and the blocks with a payload followed, a warp
 // at a time; the whole search 670, 560 and 530 us from three sources, 400, 328 and 312 now; in scattered order 354 - 466, 270 - 367 now.  A frontier bitmap in shared memory in front of the gathers: 80 -> 103 (L1 is what it
 // takes away); less shared memory by half the columns a round in sssp_expand: within 2 %.
 struct SsspPullShared {
