@@ -8,9 +8,12 @@
 //            distance goes straight into the target's word with an atomic minimum, and the thread whose atomic lowered
 //            it marks the target in the next frontier;
 //   long     the listed long runs and payload runs, a warp per chunk (only if there are any);
-//   settle   the marked vertices copy their word into the caller's distances -- the values the next
+//   settle   the marked vertices copy their word into the array of distances -- the values the next
 //            step starts from, which no one lowers meanwhile -- and are counted;
-// with a grid barrier after each.  A step that reaches few edges (of INLINE runs, which is what is counted: steps of a 27-point operator list a little longer, and gain by it
+// with a grid barrier after each.  A large step is pulled (sssp_pull), row by row; on handles with weights it writes the words of all rows into the other of the two arrays, which then
+// holds the distances, and counts what it lowers itself: no settling behind it.  (Six pulled steps of a search paid 7 - 10 us each for it, most of it two barriers' worth of latency: R-MAT,
+// symmetrised, 16 K vertices 151 -> 131 us a search, 131 K 195 -> 173, in scattered order 168 -> 149, 300 K 180 -> 167 and 142 -> 133, 2^20 364 -> 351 and 306 -> 290.)  A pushed step behind a
+// pulled one begins with a pass that makes the arrays agree.  The caller's distances are written at the end.  A step that reaches few edges (of INLINE runs, which is what is counted: steps of a 27-point operator list a little longer, and gain by it
 // like the others) also lists what it marks; a frontier that is listed and short is expanded
 // from its list in one phase, long runs and payload entries included, and settled by one thread block (sssp_expand_list).  A step finds the same improvements, distance for distance, as the product did: `word`
 // holds the minimum over everything seen so far, a vertex is marked iff its word went below the distance it had before the step.
@@ -33,12 +36,15 @@ constexpr int SSSP_WARPS = SSSP_CTA / 32;
 constexpr int SSSP_WORDS = SSSP_CTA / 8;          // frontier words of a thread block's round: eight threads per word, four columns each
 constexpr int SSSP_COLS = SSSP_CTA * 4;
 constexpr int SSSP_ILP = 4;                       // warp steps in flight
-// A step whose frontier reaches more than this share of the stored elements is pulled.  Shares of 5 / 10 / 15 %, symmetrised R-MAT, means of four sources, in brackets with the
-// vertices in scattered order: 40 K vertices 168 / 168 / 168 us a search (157 / 157 / 159), 131 K 187 / 184 / 187 (169 / 168 / 168), 300 K 223 / 209 / 209 (185 / 191 / 190),
-// 500 K 228 / 233 / 233 (217 / 229 / 228), 2^20 331 / 344 / 351 (305 / 299 / 308).
-constexpr float SSSP_PULL_SHARE = 0.05f;
-// Rounds of four elements that a lane walks of a row.  4 / 6 / 8, the same matrices: 131 K vertices 184 / 185 / 187 us a search (164 / 166 / 169), 300 K 221 / 221 / 223 (186 / 184 / 185),
-// 500 K 234 / 230 / 228 (222 / 217 / 217), 2^20 340 / 332 / 331 (317 / 308 / 305).
+// A step whose frontier reaches more than this share of the stored elements is pulled.  Shares of 5 / 10 / 15 / 20 %, symmetrised R-MAT, means of twelve sources, in brackets with the
+// vertices in scattered order: 131 K vertices 172 / 169 / 167 / 168 us a search (128 / 127 / 127 / 128), 300 K 142 / 142 / 143 / 142 (146 / 144 / 143 / 142), 500 K 232 / 229 / 229 / 229,
+// 2^20 315 / 307 / 309 / 308 (291 / 286 / 286 / 286).
+constexpr float SSSP_PULL_SHARE = 0.1f;
+// Once a step has been pulled the rows have bests that prune, and a pulled step that finds little costs a pass over the rows: the share for the steps behind it.  5 / 0.5 / 0.2 / 0.05 %, six
+// sources: 131 K vertices 180 / 174 / 173 / 172 (156 / 149 / 149 / 149), 300 K 175 / 168 / 167 / 167 (136 / 133 / 133 / 134), 500 K 253 / 242 / 240 / 239, 2^20 371 / 362 / 362 / 356 (307 / 296 / 294 / 301).
+constexpr float SSSP_LATE_SHARE = 0.002f;
+// Rounds of four elements that a lane walks of a row.  6 / 8 / 12, the same six: 131 K vertices 177 / 173 / 180 (153 / 149 / 158), 300 K 172 / 167 / 175 (137 / 133 / 136), 500 K 246 / 240 / 240,
+// 2^20 373 / 362 / 363 (300 / 294 / 299).
 constexpr int SSSP_ROUNDS = 8;
 constexpr int SSSP_CHUNK = 512;                   // elements of a listed chunk of a longer row
 // A step whose frontier reaches at most so many edges lists the vertices it marks; a list of at most SSSP_LIST vertices serves the next step.
@@ -48,9 +54,9 @@ constexpr unsigned SSSP_LIST_EDGES = 1u << 17;
 constexpr int SSSP_MAX_STEPS = 1024;              // steps of one launch, at most: a cycle of negative weight ends on the host
 
 struct SsspState {
-    int *word;                // n: ordered words of the smallest distance seen
+    int *word[2];             // distances (ordered words): a step reads them from one array, which nobody writes meanwhile, and lowers them in the other
     uint32_t *bits[2];        // frontiers of alternating steps, one bit per vertex
-    int32_t *ctr;             // [0..2] vertices of the frontier, [3..5] listed chunks (sets rotate by step), [6] steps made, [18..20] vertices listed by the step
+    int32_t *ctr;             // [0..2] vertices of the frontier, [3..5] listed chunks (sets rotate by step), [6] steps made, [7] array of the distances, [18..20] vertices listed by the step
     int *low;                 // smallest word of the frontier, rotating with the counters
     unsigned long long *edges;   // out-edges of the frontier in INLINE runs (to an eighth), likewise
     int4 *chunks;             // {row, first, end, -} of the listed chunks of long rows
@@ -64,46 +70,68 @@ __device__ __forceinline__ int sssp_word(float v) { return ordered_word(__float_
 __device__ __forceinline__ float sssp_value(int w) { return __int_as_float(ordered_word(w)); }
 
 struct SsspShared {
-    unsigned long long edges[SSSP_WARPS];
     int pre[SSSP_COLS + 1];                       // elements before a column of the round
     int2 run[SSSP_COLS];                          // position of its first entry minus that; its distance
     uint16_t own[SSSP_COLS * PD_LONG / 32];       // column that owns the first element of a step of 32
     int cnt[SSSP_WARPS], sum[SSSP_WARPS], rec[SSSP_WARPS], base;
 };
 
-// What a pushed step marks: bits, and (list not null) the list of the vertices whose bit it set.
+// What a pushed step lowers (words that agreed with the distances when it began) and marks: bits, and (list not null) the list of the vertices whose bit it set.
 struct SsspNext {
+    const int *was;
+    int *word;
     uint32_t *bits;
     int32_t *list, *n_list;
-    const float *dist;
 };
+
+// What a step adds to the next one's counters (its vertices own fewer than 2^32 edges together), summed up per thread block.  Called by all of its threads.
+struct SsspSums {
+    unsigned edges[SSSP_WARPS];
+    int found[SSSP_WARPS], low[SSSP_WARPS];
+};
+__device__ __forceinline__ bool sssp_sum(SsspSums &sums, int &found, int &low, unsigned &edges) {       // true: this thread holds the thread block's sums
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    found = __reduce_add_sync(FULL, found);
+    low = __reduce_min_sync(FULL, low);
+    edges = __reduce_add_sync(FULL, edges);
+    if (lane == 0) { sums.found[warp] = found; sums.low[warp] = low; sums.edges[warp] = edges; }
+    __syncthreads();
+    if (warp != 0) return false;
+    found = __reduce_add_sync(FULL, sums.found[lane]);
+    low = __reduce_min_sync(FULL, sums.low[lane]);
+    edges = __reduce_add_sync(FULL, sums.edges[lane]);
+    return lane == 0;
+}
+__device__ __forceinline__ void sssp_count(const SsspState &s, SsspSums &sums, int set, int found, int low, unsigned edges) {
+    if (sssp_sum(sums, found, low, edges) && found) { atomicAdd(s.ctr + set, found); atomicMin(s.low + set, low); atomicAdd(s.edges + set, (unsigned long long)edges); }
+}
 
 // The candidates of up to U targets per lane (target < 0: none); called by a whole warp.
 template <int U>
-__device__ __forceinline__ void sssp_relax(const SsspState &s, const SsspNext &next, const int (&target)[U], const float (&cand)[U]) {
+__device__ __forceinline__ void sssp_relax(const SsspNext &next, const int (&target)[U], const float (&cand)[U]) {
     int seen[U];
     if (!next.list) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) seen[u] = target[u] >= 0 ? __ldca(s.word + target[u]) : 0;
+        for (int u = 0; u < U; ++u) seen[u] = target[u] >= 0 ? __ldca(next.word + target[u]) : 0;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (target[u] < 0) continue;
             const int c = sssp_word(cand[u]);
-            if (c >= seen[u] || c >= __ldcg(s.word + target[u])) continue;
-            if (c < atomicMin(s.word + target[u], c)) atomicOr(next.bits + (target[u] >> 5), 1u << (target[u] & 31));
+            if (c >= seen[u] || c >= __ldcg(next.word + target[u])) continue;
+            if (c < atomicMin(next.word + target[u], c)) atomicOr(next.bits + (target[u] >> 5), 1u << (target[u] & 31));
         }
         return;
     }
     // few edges: what counts is the chain.  The atomics go out with no look at the words in front, and the one that found the distance
     // of the step's beginning was the vertex's first.
     uint32_t fresh = 0u;
-    float was[U];
+    int was[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
-        if (target[u] >= 0) { was[u] = __ldcg(next.dist + target[u]); seen[u] = atomicMin(s.word + target[u], sssp_word(cand[u])); }
+        if (target[u] >= 0) { was[u] = __ldcg(next.was + target[u]); seen[u] = atomicMin(next.word + target[u], sssp_word(cand[u])); }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        if (target[u] < 0 || sssp_word(cand[u]) >= seen[u] || seen[u] != sssp_word(was[u])) continue;
+        if (target[u] < 0 || sssp_word(cand[u]) >= seen[u] || seen[u] != was[u]) continue;
         atomicOr(next.bits + (target[u] >> 5), 1u << (target[u] & 31));
         fresh |= 1u << u;
     }
@@ -121,7 +149,7 @@ __device__ __forceinline__ void sssp_relax(const SsspState &s, const SsspNext &n
 }
 
 template <int DT>
-__device__ void sssp_expand(const Device &d, const SsspState &s, const float *dist, const uint32_t *F, const SsspNext &next, int32_t *n_long, SsspShared &sh) {
+__device__ void sssp_expand(const Device &d, const SsspState &s, const uint32_t *F, const SsspNext &next, int32_t *n_long, SsspShared &sh) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rounds = (s.n_words + SSSP_WORDS * (int)gridDim.x - 1) / (SSSP_WORDS * (int)gridDim.x);
@@ -144,7 +172,7 @@ __device__ void sssp_expand(const Device &d, const SsspState &s, const float *di
             for (int k = 0; k < 5; ++k) c[k] = cp[k];
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if ((listed >> k) & 1u) { first[k] = c[k]; deg[k] = c[k + 1] - c[k]; xv[k] = __ldcg(dist + j0 + k); if (!DBS_CHK_RANGE(d, first[k], deg[k])) deg[k] = 0; }
+                if ((listed >> k) & 1u) { first[k] = c[k]; deg[k] = c[k + 1] - c[k]; xv[k] = sssp_value(__ldcg(next.was + j0 + k)); if (!DBS_CHK_RANGE(d, first[k], deg[k])) deg[k] = 0; }
             if (d.n_payload) payload_run(d, j0 >> 4, pfirst, pdeg);
             // long runs and runs of payload entries: chunks for the second half of the step
 #pragma unroll
@@ -230,14 +258,14 @@ __device__ void sssp_expand(const Device &d, const SsspState &s, const float *di
                 cand[u] = x[u] + Val<DT>::inline_value(w[u]);
             }
             if (s0 + SSSP_CTA * SSSP_ILP < tot_e) fetch(s0 + SSSP_CTA * SSSP_ILP);
-            sssp_relax<SSSP_ILP>(s, next, target, cand);
+            sssp_relax<SSSP_ILP>(next, target, cand);
         }
         __syncthreads();                               // (the next round overwrites the layout)
     }
 }
 
 template <int DT>
-__device__ void sssp_long(const Device &d, const SsspState &s, const SsspNext &next, int n) {
+__device__ void sssp_long(const Device &d, const SsspNext &next, int n) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int U = PD_CHUNK / 32;
     const int lane = threadIdx.x & 31;
@@ -275,7 +303,7 @@ __device__ void sssp_long(const Device &d, const SsspState &s, const SsspNext &n
         run = ahead;
         ahead = record(i + 2 * nwarps);
         fetch(run);
-        sssp_relax<U>(s, next, target, cand);
+        sssp_relax<U>(next, target, cand);
     }
 }
 
@@ -288,7 +316,7 @@ struct SsspListShared {
     int sum[SSSP_WARPS];
 };
 template <int DT>
-__device__ void sssp_expand_list(const Device &d, const SsspState &s, const float *dist, const int32_t *list, int cnt, const SsspNext &next, SsspListShared &sh) {
+__device__ void sssp_expand_list(const Device &d, const int32_t *list, int cnt, const SsspNext &next, SsspListShared &sh) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int U = PD_CHUNK / 32;
     static_assert(PD_PAYLOAD / 2 == U, "one element per lane and step either way");
@@ -296,7 +324,7 @@ __device__ void sssp_expand_list(const Device &d, const SsspState &s, const floa
     int j = 0, first = 0, deg = 0, pfirst = 0, pdeg = 0;
     if (tid < cnt) {
         j = __ldcg(list + tid);
-        sh.x[tid] = __ldcg(dist + j);
+        sh.x[tid] = sssp_value(__ldcg(next.was + j));
         column_run(d, j, first, deg);
         if (d.n_payload) payload_run(d, j >> 4, pfirst, pdeg);
         if (!DBS_CHK_RANGE(d, first, deg)) deg = 0;
@@ -343,14 +371,10 @@ __device__ void sssp_expand_list(const Device &d, const SsspState &s, const floa
 #pragma unroll
             for (int u = 0; u < U; ++u) { target[u] = in[u] ? (int)(rb[u] * 16u) + (lane & 15) : -1; cand[u] += x; }
         }
-        sssp_relax<U>(s, next, target, cand);
+        sssp_relax<U>(next, target, cand);
     }
 }
 
-// A row's new best.
-__device__ __forceinline__ void sssp_lower(const SsspState &s, uint32_t *next, int row, int best) {
-    if (best < atomicMin(s.word + row, best)) atomicOr(next + (row >> 5), 1u << (row & 31));
-}
 // Elements k0 .. k0 + 3 (k0 a multiple of four) of the runs: columns and weights, one 32-byte sector in one load.
 template <bool VAL>
 __device__ __forceinline__ void sssp_four(const Device &d, int k0, uint32_t (&col)[4], float (&w)[4]) {
@@ -388,6 +412,7 @@ __device__ __forceinline__ int sssp_bound(float xmin, float w) {
 struct SsspPullShared {
     int4 queue[SSSP_WARPS][64];       // {row, first, end, best so far} of the rows that wait for a lane
     int4 longs[SSSP_WARPS][32];                   // {row, first, end, best} of what is left of long rows
+    int queue_degree[SSSP_WARPS][64];             // their columns' elements, at least
     int cursor;                                   // groups of rows taken by the thread block's warps
 };
 
@@ -418,14 +443,20 @@ __device__ __forceinline__ void sssp_list_long(const Device &d, const SsspState 
     for (int c = 0; c < chunks; ++c) s.chunks[at++] = make_int4(r.x, r.y + c * SSSP_CHUNK, min(r.z, r.y + (c + 1) * SSSP_CHUNK), 0);
 }
 
+// Handles with weights write the words of the other array, all of them, and mark and count what they lower: the step needs no pass behind it.  What is counted of a row (its column's degree) comes with
+// the row's own words, 32 rows at a time: fetched where a row ends, a whole warp waits for it in most rounds (2^20 vertices 358 -> 400 us a search), and so it does for a look at the old frontier's
+// marks that would spare the words that do not change (358 -> 405).  The distances of the 4 to 32 K columns of the highest degree in shared memory, where 34 to 69 % of the elements lie: nothing
+// gained with 4 K of them (before what it costs to bring them there), slower with more -- what they take from the L1 are the lines that the other gathers wait in.
 template <int DT>
-__device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist, const uint32_t *F, uint32_t *next, int low, int32_t *n_long, SsspPullShared &sh) {
+__device__ void sssp_pull(const Device &d, const SsspState &s, int c, uint32_t *F, uint32_t *next, int t, int low, int32_t *n_long, SsspPullShared &sh, SsspSums &sums) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int NONE = 0x7F800000;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gwarp = (int)(blockIdx.x * SSSP_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const float xmin = sssp_value(low);
+    const int *const dist = s.word[c];
+    int *const word = s.word[c ^ 1];
     const int32_t *ptr = VAL ? d.weight_ptr : d.rowrun_ptr;
     auto bound = [&](float w) { return sssp_bound<VAL>(xmin, w); };
     // The thread block's groups of rows, spread over the matrix, are taken by its warps in turn.  (On an R-MAT graph that was not relabelled neighbouring rows are
@@ -435,7 +466,9 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
     if (threadIdx.x == 0) sh.cursor = 0;
     __syncthreads();
     int4 *queue = sh.queue[warp], *longs = sh.longs[warp];
+    int *queue_degree = sh.queue_degree[warp];
     int row_g = 0, p_g = 0, e_g = 0, have_g = 0;       // a row of the next group
+    uint32_t code_g = 0u;
     float w_g = 1.0f;
     bool more = true;
     auto fetch = [&]() {
@@ -444,18 +477,26 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
         i = __shfl_sync(FULL, i, 0);
         more = i < per_block;
         if (!more) return;
-        const int64_t r = ((int64_t)i * gridDim.x + (blockIdx.x + i) % gridDim.x) * 32 + lane;
-        row_g = (int)r; p_g = 0; e_g = 0; have_g = 0;
-        if (r < d.n) { p_g = ptr[r]; e_g = ptr[r + 1]; have_g = __ldcg(s.word + r); if (VAL) w_g = d.row_lightest[r]; }
+        const int64_t g = (int64_t)i * gridDim.x + (blockIdx.x + i) % gridDim.x, r = g * 32 + lane;
+        row_g = (int)(r < d.n ? r : d.n); p_g = 0; e_g = 0; have_g = 0;
+        if (r < d.n) { p_g = ptr[r]; e_g = ptr[r + 1]; have_g = __ldcg(dist + r); if (VAL) { w_g = d.row_lightest[r]; code_g = d.col_degree[r]; } }
+        if (VAL && lane == 0 && g < s.n_words) F[g] = 0u;           // (nobody looks at the frontier's marks; the bitmap is the one of the step after the next)
     };
     fetch();
     int head = 0, cnt = 0, n_listed = 0;
     int row = -1, p = 0, e = 0, have = 0, best = NONE, q_long = 0;      // the row being walked: elements [p, e), from q_long on it is long
+    int found = 0, lowest = NONE, degree = 0;
+    unsigned edges = 0;
     for (;;) {
         while (more && cnt < 32) {                     // (no more than that: what a warp has claimed no other one can take)
             const bool pass = p_g < e_g && sssp_word(xmin + w_g) < have_g;
             const uint32_t m = __ballot_sync(FULL, pass);
-            if (pass) queue[(head + cnt + __popc(m & lt)) & 63] = make_int4(row_g, p_g, e_g, have_g);
+            if (pass) {
+                const int at = (head + cnt + __popc(m & lt)) & 63;
+                queue[at] = make_int4(row_g, p_g, e_g, have_g);
+                if (VAL) queue_degree[at] = (int)degree_of_code(code_g);
+            }
+            if (VAL && row_g < d.n) __stcg(word + row_g, have_g);       // (what the row's walk finds comes on top, from this warp too)
             cnt += __popc(m);
             fetch();
         }
@@ -467,6 +508,7 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
             if (row < 0 && k < cnt) {
                 const int4 q = queue[(head + k) & 63];
                 row = q.x; p = q.y; e = q.z; have = best = q.w; q_long = (p & ~3) + SSSP_ROUNDS * 4;
+                if (VAL) degree = queue_degree[(head + k) & 63];
             }
             const int took = min(__popc(idle), cnt);
             head += took; cnt -= took;
@@ -475,27 +517,30 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
         if (row >= 0) {
             // (a row that was never reached needs several rounds: two groups at a time until something is found)
             uint32_t col[8];
-            float w[8], x[8];
+            float w[8];
+            int x[8];
             const int q0 = p & ~3;
             const bool two = best == NONE && q0 + 4 < e;
             sssp_four<VAL>(d, q0, reinterpret_cast<uint32_t (&)[4]>(col[0]), reinterpret_cast<float (&)[4]>(w[0]));
             if (two) sssp_four<VAL>(d, q0 + 4, reinterpret_cast<uint32_t (&)[4]>(col[4]), reinterpret_cast<float (&)[4]>(w[4]));
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                x[j] = __int_as_float(NONE);
-                if ((j < 4 || two) && q0 + j >= p && q0 + j < e && sssp_word(xmin + w[j]) < best && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
+                x[j] = NONE;
+                const bool go = (j < 4 || two) && q0 + j >= p && q0 + j < e && sssp_word(xmin + w[j]) < best;
+                if (go && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
             }
             float last = w[3];
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-                if (j < 4 || two) { best = min(best, sssp_word(x[j] + w[j])); last = w[j]; }
+                if (j < 4 || two) { best = min(best, sssp_word(sssp_value(x[j]) + w[j])); last = w[j]; }
             p = q0 + (two ? 8 : 4);
             const bool over = p >= e || bound(last) >= best;
             left = !over && p >= q_long;
             if ((over || left) && best < have) {
-                // (below the best that the step found in place: the row is marked whoever else lowers it, and nobody waits for the replies)
-                atomicMin(s.word + row, best);
+                // (a row has one owner; the chunks of a long one follow behind a barrier.  Without values the payload entries lower it too.)
+                if (VAL) __stcg(word + row, best); else atomicMin(word + row, best);
                 atomicOr(next + (row >> 5), 1u << (row & 31));
+                if (VAL) { ++found; lowest = min(lowest, best); edges += (unsigned)degree; }
             }
             if (over) row = -1;
         }
@@ -508,7 +553,7 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
     }
     __syncwarp();
     if (n_listed) sssp_list_long<VAL>(d, s, longs, n_listed, xmin, n_long, lane);
-    if (VAL) return;
+    if (VAL) { sssp_count(s, sums, (t + 1) % 3, found, lowest, edges); return; }
     // entries with a payload (unit weights): one block per warp at a time, columns of the frontier only (the blocks sit where a power-law graph is dense, among
     // the vertices that settle first: late large steps skip most of them); the next entry is fetched meanwhile
     struct Entry { uint32_t idx, w, aux; int rb; };
@@ -531,9 +576,9 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
         if (type == DBSPMSPV_BLK_INLINE || !DBS_CHK_INDEX(d, e.rb, d.mb)) continue;      // (only a replaced entry is INLINE here; warp-uniform)
         const uint32_t xm = mask_of(F, cb);
         if (!xm) continue;                                                               // warp-uniform
-        block_rows_min_warp<DT>(type, e.w, e.aux, xm, dist + (size_t)cb * 16, d.payload, lane, [&](int r, uint32_t key) {
+        block_rows_min_warp<DT>(type, e.w, e.aux, xm, reinterpret_cast<const float *>(dist) + (size_t)cb * 16, d.payload, lane, [&](int r, uint32_t key) {
             const int c = sssp_word(minplus_value(key)), row = e.rb * 16 + r;
-            if (c < __ldcg(s.word + row)) sssp_lower(s, next, row, c);
+            if (c < __ldcg(word + row) && c < atomicMin(word + row, c)) atomicOr(next + (row >> 5), 1u << (row & 31));
         });
     }
 }
@@ -541,53 +586,65 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, const float *dist
 // The listed chunks of long rows, a warp per chunk, four elements per lane and step.  The next chunk's record, best and first elements are
 // fetched while this one's distances arrive.
 template <int DT>
-__device__ void sssp_pull_long(const Device &d, const SsspState &s, const float *dist, uint32_t *next, int low, int n) {
+__device__ void sssp_pull_long(const Device &d, const SsspState &s, int c, uint32_t *next, int t, int low, int n, SsspSums &sums) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
+    constexpr int NONE = 0x7F800000;
     const int lane = threadIdx.x & 31;
     const int gwarp = (int)(blockIdx.x * SSSP_CTA + threadIdx.x) >> 5, nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
     const float xmin = sssp_value(low);
+    const int *const dist = s.word[c];
+    int *const word = s.word[c ^ 1];
     auto record = [&](int i) { return i < n ? __ldcg(s.chunks + i) : make_int4(0, 0, 0, 0); };
-    int4 c = record(gwarp), ahead = record(gwarp + nwarps);
+    int4 now_c = record(gwarp), ahead = record(gwarp + nwarps);
     uint32_t col[4] = {0u, 0u, 0u, 0u};
     float w[4] = {0.f, 0.f, 0.f, 0.f};
     int had = 0;
+    int found = 0, lowest = NONE;
+    unsigned edges = 0;
     auto first = [&](const int4 &r) {
         const int k0 = (r.y & ~3) + 4 * lane;
-        if (k0 < r.z) { had = __ldcg(s.word + r.x); sssp_four<VAL>(d, k0, col, w); }
+        if (k0 < r.z) { had = __ldcg(word + r.x); sssp_four<VAL>(d, k0, col, w); }
     };
-    first(c);
+    first(now_c);
     for (int i = gwarp; i < n; i += nwarps) {
         had = __shfl_sync(FULL, had, 0);               // (lane 0 of a chunk always has elements)
-        const int start = had, row = c.x, p = c.y, e = c.z;
+        const int start = had, row = now_c.x, p = now_c.y, e = now_c.z;
         int now = had;
         for (int q = (p & ~3) + 4 * lane;; q += 128) {
-            float x[4], wq[4];
+            float wq[4];
+            int x[4];
             const bool in = q < e, more = q - 4 * lane + 128 < e;             // (warp-uniform: the chunk goes on)
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                x[j] = __int_as_float(0x7F800000);
+                x[j] = NONE;
                 wq[j] = w[j];
-                if (in && q + j >= p && q + j < e && sssp_word(xmin + w[j]) < now && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
+                const bool go = in && q + j >= p && q + j < e && sssp_word(xmin + w[j]) < now;
+                if (go && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
             }
             if (more) { if (q + 128 < e) sssp_four<VAL>(d, q + 128, col, w); }
-            else { c = ahead; ahead = record(i + 2 * nwarps); first(c); }
+            else { now_c = ahead; ahead = record(i + 2 * nwarps); first(now_c); }
             int mine = now;
             if (in)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mine = min(mine, sssp_word(x[j] + wq[j]));
+                for (int j = 0; j < 4; ++j) mine = min(mine, sssp_word(sssp_value(x[j]) + wq[j]));
             now = __reduce_min_sync(FULL, mine);
             if (!more) break;
             const bool over = sssp_bound<VAL>(xmin, wq[3]) >= now;
             if (__shfl_sync(FULL, (int)over, 31)) {    // (the last lane's weight is the largest of the step)
-                c = ahead; ahead = record(i + 2 * nwarps); first(c);
+                now_c = ahead; ahead = record(i + 2 * nwarps); first(now_c);
                 break;
             }
         }
         if (lane == 0 && now < start) {
-            atomicMin(s.word + row, now);
-            atomicOr(next + (row >> 5), 1u << (row & 31));
+            atomicMin(word + row, now);
+            const uint32_t bit = 1u << (row & 31);
+            if (VAL) {                                 // (a row of several chunks is counted by the one that marks it)
+                lowest = min(lowest, now);
+                if (!(atomicOr(next + (row >> 5), bit) & bit)) { ++found; edges += degree_of_code(d.col_degree[row]); }
+            } else atomicOr(next + (row >> 5), bit);
         }
     }
+    if (VAL) sssp_count(s, sums, (t + 1) % 3, found, lowest, edges);
 }
 
 constexpr int SSSP_SMEM = (int)(sizeof(SsspShared) > sizeof(SsspPullShared) ? sizeof(SsspShared) : sizeof(SsspPullShared));
@@ -596,55 +653,81 @@ static_assert(sizeof(SsspListShared) <= sizeof(SsspShared), "the phases share on
 // spilled more besides (216 -> 88 bytes of stack; R-MAT 300 K / 500 K / 2^20 vertices 242 / 252 / 359 -> 222 / 227 / 331 us a search, in scattered order 202 / 237 / 333 -> 186 / 217 / 306; 27-point
 // operator on 90^3 cells, an inner source, 3029 -> 2947).  The phases as functions of their own, which share no registers: 233 / 239 / 343 us.
 template <int DT>
-__global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ Device d, const __grid_constant__ SsspState s, int32_t src, float *dist, int start, int max_steps, unsigned long long pull_edges) {
+__global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ Device d, const __grid_constant__ SsspState s, int32_t src, float *dist_out, int start, int max_steps, unsigned long long pull_edges, unsigned long long late_edges) {
     namespace cg = cooperative_groups;
     extern __shared__ __align__(16) uint8_t s_dyn[];
+    __shared__ SsspSums sums;
+    constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     SsspShared &sh = *reinterpret_cast<SsspShared *>(s_dyn);
     cg::grid_group grid = cg::this_grid();
     const int tid = blockIdx.x * SSSP_CTA + threadIdx.x, nthreads = gridDim.x * SSSP_CTA, lane = threadIdx.x & 31;
     if (start) {                                       // (a later launch of the same search continues where the one before stopped)
-        const int64_t n = d.n;
-        for (int64_t v = tid; v < n; v += nthreads) { s.word[v] = v == src ? 0 : 0x7F800000; dist[v] = v == src ? 0.0f : __int_as_float(0x7F800000); }
+        const int64_t n = (int64_t)s.n_words * 32;
+        for (int64_t v = tid; v < n; v += nthreads) s.word[0][v] = s.word[1][v] = v == src ? 0 : 0x7F800000;
         for (int k = tid; k < s.n_words; k += nthreads) { s.bits[0][k] = k == src >> 5 ? 1u << (src & 31) : 0u; s.bits[1][k] = 0u; }
         if (tid < 6) s.ctr[tid] = tid == 0 ? 1 : 0;
         if (tid == 6) {
             int first, deg;
             column_run(d, src, first, deg);
-            s.ctr[6] = 0;
+            s.ctr[6] = 0; s.ctr[7] = 0;
             for (int k = 0; k < 3; ++k) { s.low[k] = k == 0 ? 0 : 0x7F800000; s.edges[k] = k == 0 ? (unsigned long long)deg : 0ull; s.ctr[18 + k] = 0; }
             s.list[1][0] = src;
         }
         grid.sync();
     }
-    int t = s.ctr[6];
+    int t = s.ctr[6], c = s.ctr[7];
+    bool late = false;                                 // a step has been pulled
     bool listed = start != 0;                          // the frontier is in list[(t + 1) & 1]
+    bool agree = true;                                 // both arrays hold the distances (else array c does)
     for (int made = 0; made < max_steps; ++made, ++t) {
         const int cnt = __ldcg(s.ctr + t % 3);         // grid-uniform, as all that is decided from it
-        if (cnt == 0) break;
-        uint32_t *F = s.bits[t & 1];
         const unsigned long long edges_now = __ldcg(s.edges + t % 3);
+        const int low_now = __ldcg(s.low + t % 3);
+        if (cnt == 0) break;
+        uint32_t *F = s.bits[t & 1], *N = s.bits[(t + 1) & 1];
         int32_t *n_long = s.ctr + 3 + t % 3, *n_list = s.ctr + 18 + t % 3;
-        const bool pulled = edges_now > pull_edges, lists = !pulled && edges_now <= SSSP_LIST_EDGES;
-        const SsspNext next{s.bits[(t + 1) & 1], lists ? s.list[t & 1] : nullptr, n_list, dist};
+        const bool pulled = edges_now > (late ? late_edges : pull_edges), lists = !pulled && edges_now <= SSSP_LIST_EDGES;
         if (tid == 0) { s.ctr[3 + (t + 1) % 3] = 0; s.ctr[18 + (t + 1) % 3] = 0; }      // (their last reader was step t - 2)
-        if (pulled) {
-            const int low = __ldcg(s.low + t % 3);
-            sssp_pull<DT>(d, s, dist, F, next.bits, low, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn));
+        late = late || pulled;
+        if (VAL && pulled) {
+            if (tid == 0) { s.ctr[(t + 2) % 3] = 0; s.low[(t + 2) % 3] = 0x7F800000; s.edges[(t + 2) % 3] = 0ull; }
+            sssp_pull<DT>(d, s, c, F, N, t, low_now, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), sums);
             grid.sync();
             const int n = __ldcg(n_long);
             if (n > 0) {                               // grid-uniform
-                sssp_pull_long<DT>(d, s, dist, next.bits, low, n);
+                sssp_pull_long<DT>(d, s, c, N, t, low_now, n, sums);
+                grid.sync();
+            }
+            c ^= 1;
+            agree = false;
+            listed = false;
+            continue;
+        }
+        if (!agree) {                                  // behind a pulled step: what it lowered, in the other array too
+            for (int w = tid >> 5; w < s.n_words; w += nthreads >> 5)
+                if ((__ldcg(F + w) >> lane) & 1u) s.word[c ^ 1][w * 32 + lane] = __ldcg(s.word[c] + w * 32 + lane);
+            grid.sync();
+            agree = true;
+        }
+        int *const dist = s.word[c], *const word = s.word[c ^ 1];
+        const SsspNext next{dist, word, N, lists ? s.list[t & 1] : nullptr, n_list};
+        if (pulled) {
+            sssp_pull<DT>(d, s, c, F, N, t, low_now, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), sums);
+            grid.sync();
+            const int n = __ldcg(n_long);
+            if (n > 0) {                               // grid-uniform
+                sssp_pull_long<DT>(d, s, c, N, t, low_now, n, sums);
                 grid.sync();
             }
         } else if (listed) {
-            sssp_expand_list<DT>(d, s, dist, s.list[(t + 1) & 1], cnt, next, *reinterpret_cast<SsspListShared *>(s_dyn));
+            sssp_expand_list<DT>(d, s.list[(t + 1) & 1], cnt, next, *reinterpret_cast<SsspListShared *>(s_dyn));
             grid.sync();
         } else {
-            sssp_expand<DT>(d, s, dist, F, next, n_long, sh);
+            sssp_expand<DT>(d, s, F, next, n_long, sh);
             grid.sync();
             const int n = __ldcg(n_long);
             if (n > 0) {                               // grid-uniform
-                sssp_long<DT>(d, s, next, n);
+                sssp_long<DT>(d, next, n);
                 grid.sync();
             }
         }
@@ -653,18 +736,18 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
         const int n_marked = lists ? __ldcg(n_list) : 0;
         listed = lists && n_marked <= SSSP_LIST;
         int found = 0, low = 0x7F800000;
-        unsigned long long edges = 0;
+        unsigned edges = 0;
         if (listed) {                                  // one thread block settles, the others clear the old frontier if it is not listed
             if (!was_listed) for (int k = tid; k < s.n_words; k += nthreads) F[k] = 0u;
             if (blockIdx.x == 0) {
                 if (was_listed && (int)threadIdx.x < cnt) F[__ldcg(s.list[(t + 1) & 1] + threadIdx.x) >> 5] = 0u;
                 if ((int)threadIdx.x < n_marked) {
                     const int j = __ldcg(s.list[t & 1] + threadIdx.x);
-                    low = __ldcg(s.word + j);
+                    low = __ldcg(word + j);
                     int first, deg;
                     column_run(d, j, first, deg);
                     edges = (unsigned)deg;
-                    dist[j] = sssp_value(low);
+                    dist[j] = low;
                 }
             }
         } else {
@@ -673,13 +756,13 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
                 uint32_t b[8];
                 int v[8], deg[8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) { const int w = w0 + q * nwarps; b[q] = w < s.n_words ? __ldcg(next.bits + w) : 0u; }
+                for (int q = 0; q < 8; ++q) { const int w = w0 + q * nwarps; b[q] = w < s.n_words ? __ldcg(N + w) : 0u; }
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     v[q] = 0x7F800000; deg[q] = 0;
                     if ((b[q] >> lane) & 1u) {
                         const int j = (w0 + q * nwarps) * 32 + lane;
-                        v[q] = __ldcg(s.word + j);
+                        v[q] = __ldcg(word + j);
                         if (d.col_degree) deg[q] = (int)d.col_degree[j];      // (a byte each: with the column pointers the pass took a third longer)
                         else { int first; column_run(d, j, first, deg[q]); deg[q] = (int)degree_code((uint32_t)deg[q]); }
                     }
@@ -688,33 +771,28 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
                 for (int q = 0; q < 8; ++q) {
                     const int w = w0 + q * nwarps;
                     if (w >= s.n_words) break;
-                    if ((b[q] >> lane) & 1u) dist[(int64_t)w * 32 + lane] = sssp_value(v[q]);
+                    if ((b[q] >> lane) & 1u) dist[w * 32 + lane] = v[q];
                     if (lane == 0) F[w] = 0u;
                     found += __popc(b[q]);
                     low = min(low, v[q]);
                     edges += degree_of_code((uint32_t)deg[q]);
                 }
             }
+            if (lane != 0) found = 0;                  // (a word's marks are counted once)
         }
-        low = __reduce_min_sync(FULL, low);
-#pragma unroll
-        for (int o = 16; o; o >>= 1) edges += __shfl_xor_sync(FULL, edges, o);
-        if (lane == 0) { sh.cnt[threadIdx.x >> 5] = found; sh.sum[threadIdx.x >> 5] = low; sh.edges[threadIdx.x >> 5] = edges; }
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            found = __reduce_add_sync(FULL, sh.cnt[lane]);
-            low = __reduce_min_sync(FULL, sh.sum[lane]);
-            edges = sh.edges[lane];
-#pragma unroll
-            for (int o = 16; o; o >>= 1) edges += __shfl_xor_sync(FULL, edges, o);
-            if (listed) {
-                if (lane == 0 && blockIdx.x == 0) { s.ctr[(t + 1) % 3] = n_marked; s.low[(t + 1) % 3] = low; s.edges[(t + 1) % 3] = edges; }
-            } else if (lane == 0 && found) { atomicAdd(s.ctr + (t + 1) % 3, found); atomicMin(s.low + (t + 1) % 3, low); atomicAdd(s.edges + (t + 1) % 3, edges); }
-        }
+        if (listed) {
+            if (sssp_sum(sums, found, low, edges) && blockIdx.x == 0) { s.ctr[(t + 1) % 3] = n_marked; s.low[(t + 1) % 3] = low; s.edges[(t + 1) % 3] = edges; }
+        } else sssp_count(s, sums, (t + 1) % 3, found, low, edges);
         grid.sync();
     }
-    // (everyone read ctr[6] before the first barrier, or leaves without a step)
-    if (tid == 0) { s.ctr[6] = t; s.report[0] = t; s.report[1] = __ldcg(s.ctr + t % 3); }
+    // the distances themselves; a search that goes on starts from arrays that agree
+    for (int64_t v = tid; v < d.n; v += nthreads) {
+        const int w = __ldcg(s.word[c] + v);
+        dist_out[v] = sssp_value(w);
+        if (!agree) s.word[c ^ 1][v] = w;
+    }
+    // (everyone read ctr[6] and ctr[7] before the first barrier, or leaves without a step)
+    if (tid == 0) { s.ctr[6] = t; s.ctr[7] = c; s.report[0] = t; s.report[1] = __ldcg(s.ctr + t % 3); }
 }
 
 }  // namespace dbs

@@ -135,3 +135,32 @@ def test_rows_of_a_pulled_step(length):
         assert np.array_equal(dist.cpu().numpy().astype(np.float64), oracle.ref_sssp(A, src))
     assert steps[0] == steps[1]
     h.close()
+
+
+@pytest.mark.parametrize("length", [40, 333, 1200])
+@pytest.mark.parametrize("base", [4096.0, -4096.0])
+def test_many_pulled_steps_in_a_row(length, base):
+    """A path whose vertices also have an edge each from the source, of weights that rise twice as fast as the path's: every step improves all that is left of it, so the
+    steps are pulled one after the other -- 1200 of them in more than one launch -- until the frontier is a few vertices, the path's end and a tail behind it.
+    (Distances of both signs; whole numbers: every sum is exact.)"""
+    n = length + 107
+    k = np.arange(length)
+    rows = np.r_[1 + k, 2 + k[:-1], length + 1 + np.arange(6)]
+    cols = np.r_[np.zeros(length, np.int64), 1 + k[:-1], length + np.arange(6)]
+    val = np.r_[base + 2.0 * k, np.ones(length - 1), np.full(6, 3.0)].astype(np.float32)
+    order = np.argsort(rows.astype(np.int64) * n + cols)
+    ptr, idx = wl.csr_from_sorted_keys(n, n, (rows.astype(np.int64) * n + cols)[order])
+    want = np.full(n, np.inf, np.float32)
+    want[0] = 0.0
+    want[1:length + 1] = base + k
+    want[length + 1:length + 7] = base + length - 1 + 3.0 * (1 + np.arange(6))
+    h = Handle(wl.CSR(n, n, ptr, idx, val[order]), B.F32)
+    dist = torch.empty(n, dtype=torch.float32, device="cuda")
+    steps = []
+    for path in (B.PATH_AUTO, B.PATH_PUSH, B.PATH_AUTO):
+        h.set_opts(force_path=path)
+        steps.append(B.db_sssp(h.h, 0, dist))
+        torch.cuda.synchronize()
+        assert np.array_equal(dist.cpu().numpy(), want)
+    assert steps[0] == steps[1] == steps[2] and steps[0] > length
+    h.close()
