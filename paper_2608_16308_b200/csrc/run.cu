@@ -2612,15 +2612,14 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     // chunks of long rows: a row has more than 4 (SSSP_ROUNDS - 1) elements before any of it is listed
     const size_t chunk_bytes = ((size_t)h->nnz / (4 * (SSSP_ROUNDS - 1)) + (size_t)h->nnz / SSSP_CHUNK + 64) * sizeof(int4);
     if (!h->sssp_state) {
-        if (cudaMalloc(&h->sssp_state, 2 * (word_bytes + bit_bytes) + 256 + 2 * SSSP_LIST * sizeof(int32_t) + chunk_bytes) != cudaSuccess) { h->sssp_state = nullptr; return DBSPMSPV_ERR_ALLOC; }
+        if (cudaMalloc(&h->sssp_state, 2 * word_bytes + 3 * bit_bytes + 256 + 2 * SSSP_LIST * sizeof(int32_t) + chunk_bytes) != cudaSuccess) { h->sssp_state = nullptr; return DBSPMSPV_ERR_ALLOC; }
         DBS_CUDA(cudaFuncSetAttribute(k_sssp<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SSSP_SMEM));
     }
     uint8_t *p = static_cast<uint8_t *>(h->sssp_state);
     for (int k = 0; k < 2; ++k) { s.word[k] = reinterpret_cast<int *>(p); p += word_bytes; }
-    for (int k = 0; k < 2; ++k) { s.bits[k] = reinterpret_cast<uint32_t *>(p); p += bit_bytes; }
-    s.ctr = reinterpret_cast<int32_t *>(p); p += 256;
-    s.low = s.ctr + 8;
-    s.edges = reinterpret_cast<unsigned long long *>(s.ctr + 12);
+    for (int k = 0; k < 3; ++k) { s.bits[k] = reinterpret_cast<uint32_t *>(p); p += bit_bytes; }
+    s.set = reinterpret_cast<SsspSet *>(p);
+    s.ctr = reinterpret_cast<int32_t *>(p + 3 * sizeof(SsspSet)); p += 256;
     for (int k = 0; k < 2; ++k) { s.list[k] = reinterpret_cast<int32_t *>(p); p += SSSP_LIST * sizeof(int32_t); }
     s.chunks = reinterpret_cast<int4 *>(p);
     s.report = h->sssp_host;
@@ -2629,8 +2628,7 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     for (int64_t made = 0;; start = 0) {
         int max_steps = (int)(d.n + 1 - made < SSSP_MAX_STEPS ? d.n + 1 - made : SSSP_MAX_STEPS);
         const bool can_pull = DT == DBSPMSPV_PATTERN ? d.rowrun_ptr != nullptr : d.weightrun != nullptr && d.col_degree != nullptr;
-        unsigned long long pull_edges = can_pull ? (unsigned long long)(SSSP_PULL_SHARE * (float)d.n_entries) : ~0ull;
-        unsigned long long late_edges = can_pull ? (unsigned long long)(SSSP_LATE_SHARE * (float)d.n_entries) : ~0ull;
+        unsigned pull_edges = can_pull ? (unsigned)(SSSP_PULL_SHARE * (float)d.n_entries) : ~0u, late_edges = can_pull ? (unsigned)(SSSP_LATE_SHARE * (float)d.n_entries) : ~0u;
         void *args[] = {&dev, &s, &src, &dist, &start, &max_steps, &pull_edges, &late_edges};
         DBS_CUDA(cudaLaunchCooperativeKernel((void *)k_sssp<DT>, dim3(h->sm_count), dim3(SSSP_CTA), args, SSSP_SMEM, st));
         ++h->kernel_launches;

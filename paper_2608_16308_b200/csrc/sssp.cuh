@@ -3,24 +3,25 @@
 // The search is the synchronous iteration of (min, +) products: step t relaxes the out-edges of the
 // vertices whose distance improved in step t - 1, with the distances they had at the end of that step.  As a host loop over
 // dbspmspv_run it paid, per step, a blocking of x, an accumulator that was filled and compacted, a relaxation pass and a
-// round trip to the host (R-MAT scale 20: 9 steps, 1.17 ms, of which 0.2 ms an idle GPU).  Here a step is
+// round trip to the host (R-MAT scale 20: 9 steps, 1.17 ms, of which 0.2 ms an idle GPU).  Here a step reads the distances from one of two arrays of words, which nobody writes meanwhile, and lowers the
+// words of the other one, which then holds the distances:
 //   expand   the columns of the frontier (a bitmap) laid end to end per thread block as in the direct push (push_direct.cuh); a candidate
-//            distance goes straight into the target's word with an atomic minimum, and the thread whose atomic lowered
-//            it marks the target in the next frontier;
+//            distance goes straight into the target's word with an atomic minimum, and the thread whose atomic is the first to bring
+//            it below the distance marks the target in the next frontier and counts it;
 //   long     the listed long runs and payload runs, a warp per chunk (only if there are any);
-//   settle   the marked vertices copy their word into the array of distances -- the values the next
-//            step starts from, which no one lowers meanwhile -- and are counted;
-// with a grid barrier after each.  A large step is pulled (sssp_pull), row by row; on handles with weights it writes the words of all rows into the other of the two arrays, which then
-// holds the distances, and counts what it lowers itself: no settling behind it.  (Six pulled steps of a search paid 7 - 10 us each for it, most of it two barriers' worth of latency: R-MAT,
-// symmetrised, 16 K vertices 151 -> 131 us a search, 131 K 195 -> 173, in scattered order 168 -> 149, 300 K 180 -> 167 and 142 -> 133, 2^20 364 -> 351 and 306 -> 290.)  A pushed step behind a
-// pulled one begins with a pass that makes the arrays agree.  The caller's distances are written at the end.  A step that reaches few edges (of INLINE runs, which is what is counted: steps of a 27-point operator list a little longer, and gain by it
+// with a grid barrier after each.  The other array has the distances of two steps ago: they differ from the present ones in the vertices of the frontier, which whoever expands them brings down
+// as well, in whatever order.  (With one array a pass behind every step copied and counted what was marked, one more barrier and 5 - 10 us a step.)
+// A large step is pulled (sssp_pull), row by row.  A step that reaches few edges (of INLINE runs, which is what is counted: steps of a 27-point operator list a little longer, and gain by it
 // like the others) also lists what it marks; a frontier that is listed and short is expanded
-// from its list in one phase, long runs and payload entries included, and settled by one thread block (sssp_expand_list).  A step finds the same improvements, distance for distance, as the product did: `word`
-// holds the minimum over everything seen so far, a vertex is marked iff its word went below the distance it had before the step.
+// from its list in one phase, long runs and payload entries included (sssp_expand_list).  A step finds the same improvements, distance for distance, as the product did: a vertex is marked iff its word
+// went below the distance it had before the step.  The caller's distances are written at the end.
 //
-// What bounds a large step is the gather of one target word per edge.  It goes through L1 first (a stale word is never too small,
-// so a candidate that does not beat it is done); only a candidate that does looks at L2, and only one that beats that too pays an atomic:
-// the words of hub rows, which thousands of edges reach, settle after a few atomics.
+// What a small step costs is its trips to L2, one after the other, 0.6 us each with what surrounds it: the counters that decide the next step lie in one 16-byte word (SsspSet), fetched once behind the barrier.
+// (As five words fetched one by one, with a pass that settled the marked vertices: 16 K vertices 119 -> 102 us a search, 131 K 165 -> 139 (124 -> 104), 300 K 141 -> 126 (140 -> 121), 2^20 305 -> 290 (288 -> 260);
+// with the marked vertices settled behind the pulled steps too: 152, 195 (168), 180 (142 with other sources), 364 (306).)
+//
+// What bounds a large step is the gather of one target distance per edge.  It goes through L1 (a candidate that does not beat the distance is done); only one that does looks at the word
+// in L2, and only one that beats that too pays an atomic: the words of hub rows, which thousands of edges reach, settle after a few atomics.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -53,12 +54,17 @@ constexpr int SSSP_LIST = SSSP_CTA;
 constexpr unsigned SSSP_LIST_EDGES = 1u << 17;
 constexpr int SSSP_MAX_STEPS = 1024;              // steps of one launch, at most: a cycle of negative weight ends on the host
 
+// What a step leaves to the next one, in one 16-byte word: a barrier is followed by one trip to L2.
+struct alignas(16) SsspSet {
+    unsigned edges, found;    // out-edges of the frontier in INLINE runs (to an eighth); its vertices
+    int low;                  // its smallest word
+    int n_long;               // chunks of long runs or rows that the step itself listed
+};
 struct SsspState {
     int *word[2];             // distances (ordered words): a step reads them from one array, which nobody writes meanwhile, and lowers them in the other
-    uint32_t *bits[2];        // frontiers of alternating steps, one bit per vertex
-    int32_t *ctr;             // [0..2] vertices of the frontier, [3..5] listed chunks (sets rotate by step), [6] steps made, [7] array of the distances, [18..20] vertices listed by the step
-    int *low;                 // smallest word of the frontier, rotating with the counters
-    unsigned long long *edges;   // out-edges of the frontier in INLINE runs (to an eighth), likewise
+    uint32_t *bits[3];        // frontiers, one bit per vertex: the step's, the one it marks, the one before (being cleared), in turn
+    SsspSet *set;             // three of them, in turn
+    int32_t *ctr;             // [0] steps made, [1] array of the distances, [2..4] places taken in the step's list
     int4 *chunks;             // {row, first, end, -} of the listed chunks of long rows
     int32_t *list[2];         // the vertices marked by alternating steps, SSSP_LIST at most
     int32_t *report;          // page-locked host words: steps made, vertices of the frontier that was left
@@ -76,7 +82,36 @@ struct SsspShared {
     int cnt[SSSP_WARPS], sum[SSSP_WARPS], rec[SSSP_WARPS], base;
 };
 
-// What a pushed step lowers (words that agreed with the distances when it began) and marks: bits, and (list not null) the list of the vertices whose bit it set.
+// What a step finds: vertices that it lowers, the smallest of their words, their out-edges (fewer than 2^32 together).  Every thread keeps its own.
+struct SsspTally {
+    int found = 0, low = 0x7F800000;
+    unsigned edges = 0;
+};
+// Into the next step's counters, summed up per thread block.  Called by all of its threads.
+struct SsspSums { int found[SSSP_WARPS], low[SSSP_WARPS]; unsigned edges[SSSP_WARPS]; };
+__device__ __forceinline__ void sssp_count(const SsspState &s, SsspSums &sums, int set, const SsspTally &tally) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int found = __reduce_add_sync(FULL, tally.found), low = __reduce_min_sync(FULL, tally.low);
+    unsigned edges = __reduce_add_sync(FULL, tally.edges);
+    if (lane == 0) { sums.found[warp] = found; sums.low[warp] = low; sums.edges[warp] = edges; }
+    __syncthreads();
+    if (warp != 0) return;
+    found = __reduce_add_sync(FULL, sums.found[lane]);
+    low = __reduce_min_sync(FULL, sums.low[lane]);
+    edges = __reduce_add_sync(FULL, sums.edges[lane]);
+    if (lane == 0 && found) {
+        atomicAdd(reinterpret_cast<unsigned long long *>(&s.set[set].edges), (unsigned long long)(unsigned)found << 32 | edges);
+        atomicMin(&s.set[set].low, low);
+    }
+}
+__device__ __forceinline__ unsigned sssp_degree(const Device &d, int j) {
+    if (d.col_degree) return degree_of_code(d.col_degree[j]);
+    int first, deg;
+    column_run(d, j, first, deg);
+    return degree_of_code(degree_code((uint32_t)deg));
+}
+
+// A pushed step reads the distances, `was`, lowers the words of the other array and marks what it lowers: bits, and (list not null) a list.
 struct SsspNext {
     const int *was;
     int *word;
@@ -84,54 +119,37 @@ struct SsspNext {
     int32_t *list, *n_list;
 };
 
-// What a step adds to the next one's counters (its vertices own fewer than 2^32 edges together), summed up per thread block.  Called by all of its threads.
-struct SsspSums {
-    unsigned edges[SSSP_WARPS];
-    int found[SSSP_WARPS], low[SSSP_WARPS];
-};
-__device__ __forceinline__ bool sssp_sum(SsspSums &sums, int &found, int &low, unsigned &edges) {       // true: this thread holds the thread block's sums
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    found = __reduce_add_sync(FULL, found);
-    low = __reduce_min_sync(FULL, low);
-    edges = __reduce_add_sync(FULL, edges);
-    if (lane == 0) { sums.found[warp] = found; sums.low[warp] = low; sums.edges[warp] = edges; }
-    __syncthreads();
-    if (warp != 0) return false;
-    found = __reduce_add_sync(FULL, sums.found[lane]);
-    low = __reduce_min_sync(FULL, sums.low[lane]);
-    edges = __reduce_add_sync(FULL, sums.edges[lane]);
-    return lane == 0;
-}
-__device__ __forceinline__ void sssp_count(const SsspState &s, SsspSums &sums, int set, int found, int low, unsigned edges) {
-    if (sssp_sum(sums, found, low, edges) && found) { atomicAdd(s.ctr + set, found); atomicMin(s.low + set, low); atomicAdd(s.edges + set, (unsigned long long)edges); }
-}
-
-// The candidates of up to U targets per lane (target < 0: none); called by a whole warp.
+// The candidates of up to U targets per lane (target < 0: none); called by a whole warp.  The one that brings a word below the distance is the vertex's first.  (A vertex of the frontier itself
+// may still have its word of two steps ago when it is met, a larger one: it is brought down to the distance by whoever expands it, before or after.)
 template <int U>
-__device__ __forceinline__ void sssp_relax(const SsspNext &next, const int (&target)[U], const float (&cand)[U]) {
-    int seen[U];
+__device__ __forceinline__ void sssp_relax(const Device &d, const SsspNext &next, const int (&target)[U], const float (&cand)[U], SsspTally &tally) {
+    int was[U], seen[U];
     if (!next.list) {
+        // (the distances come through L1: nobody writes them in this step)
 #pragma unroll
-        for (int u = 0; u < U; ++u) seen[u] = target[u] >= 0 ? __ldca(next.word + target[u]) : 0;
+        for (int u = 0; u < U; ++u) was[u] = target[u] >= 0 ? __ldca(next.was + target[u]) : (int)0x80000000;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (target[u] < 0) continue;
             const int c = sssp_word(cand[u]);
-            if (c >= seen[u] || c >= __ldcg(next.word + target[u])) continue;
-            if (c < atomicMin(next.word + target[u], c)) atomicOr(next.bits + (target[u] >> 5), 1u << (target[u] & 31));
+            if (c >= was[u] || c >= __ldcg(next.word + target[u])) continue;
+            if (atomicMin(next.word + target[u], c) < was[u]) { tally.low = min(tally.low, c); continue; }
+            atomicOr(next.bits + (target[u] >> 5), 1u << (target[u] & 31));
+            tally.low = min(tally.low, c);
+            ++tally.found;
+            tally.edges += sssp_degree(d, target[u]);
         }
         return;
     }
-    // few edges: what counts is the chain.  The atomics go out with no look at the words in front, and the one that found the distance
-    // of the step's beginning was the vertex's first.
+    // few edges: what counts is the chain.  The atomics go out with no look at the words in front.
     uint32_t fresh = 0u;
-    int was[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
         if (target[u] >= 0) { was[u] = __ldcg(next.was + target[u]); seen[u] = atomicMin(next.word + target[u], sssp_word(cand[u])); }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        if (target[u] < 0 || sssp_word(cand[u]) >= seen[u] || seen[u] != was[u]) continue;
+        if (target[u] < 0 || sssp_word(cand[u]) >= was[u]) continue;
+        tally.low = min(tally.low, sssp_word(cand[u]));
+        if (seen[u] < was[u]) continue;
         atomicOr(next.bits + (target[u] >> 5), 1u << (target[u] & 31));
         fresh |= 1u << u;
     }
@@ -142,14 +160,19 @@ __device__ __forceinline__ void sssp_relax(const SsspNext &next, const int (&tar
     for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
     int base = 0;
     if (lane == 31) base = atomicAdd(next.n_list, incl);
+    unsigned edges = 0;                                // (their degrees arrive beside the place in the list)
+#pragma unroll
+    for (int u = 0; u < U; ++u) if ((fresh >> u) & 1u) edges += sssp_degree(d, target[u]);
     int at = __shfl_sync(FULL, base, 31) + incl - mine;
 #pragma unroll
     for (int u = 0; u < U; ++u)
         if ((fresh >> u) & 1u) { if (at < SSSP_LIST) next.list[at] = target[u]; ++at; }
+    tally.found += mine;
+    tally.edges += edges;
 }
 
 template <int DT>
-__device__ void sssp_expand(const Device &d, const SsspState &s, const uint32_t *F, const SsspNext &next, int32_t *n_long, SsspShared &sh) {
+__device__ void sssp_expand(const Device &d, const SsspState &s, const uint32_t *F, const SsspNext &next, int32_t *n_long, SsspShared &sh, SsspTally &tally) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rounds = (s.n_words + SSSP_WORDS * (int)gridDim.x - 1) / (SSSP_WORDS * (int)gridDim.x);
@@ -172,7 +195,13 @@ __device__ void sssp_expand(const Device &d, const SsspState &s, const uint32_t 
             for (int k = 0; k < 5; ++k) c[k] = cp[k];
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if ((listed >> k) & 1u) { first[k] = c[k]; deg[k] = c[k + 1] - c[k]; xv[k] = sssp_value(__ldcg(next.was + j0 + k)); if (!DBS_CHK_RANGE(d, first[k], deg[k])) deg[k] = 0; }
+                if ((listed >> k) & 1u) {
+                    first[k] = c[k]; deg[k] = c[k + 1] - c[k];
+                    const int w = __ldcg(next.was + j0 + k);
+                    xv[k] = sssp_value(w);
+                    atomicMin(next.word + j0 + k, w);
+                    if (!DBS_CHK_RANGE(d, first[k], deg[k])) deg[k] = 0;
+                }
             if (d.n_payload) payload_run(d, j0 >> 4, pfirst, pdeg);
             // long runs and runs of payload entries: chunks for the second half of the step
 #pragma unroll
@@ -258,14 +287,14 @@ __device__ void sssp_expand(const Device &d, const SsspState &s, const uint32_t 
                 cand[u] = x[u] + Val<DT>::inline_value(w[u]);
             }
             if (s0 + SSSP_CTA * SSSP_ILP < tot_e) fetch(s0 + SSSP_CTA * SSSP_ILP);
-            sssp_relax<SSSP_ILP>(next, target, cand);
+            sssp_relax<SSSP_ILP>(d, next, target, cand, tally);
         }
         __syncthreads();                               // (the next round overwrites the layout)
     }
 }
 
 template <int DT>
-__device__ void sssp_long(const Device &d, const SsspNext &next, int n) {
+__device__ void sssp_long(const Device &d, const SsspNext &next, int n, SsspTally &tally) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int U = PD_CHUNK / 32;
     const int lane = threadIdx.x & 31;
@@ -303,7 +332,7 @@ __device__ void sssp_long(const Device &d, const SsspNext &next, int n) {
         run = ahead;
         ahead = record(i + 2 * nwarps);
         fetch(run);
-        sssp_relax<U>(next, target, cand);
+        sssp_relax<U>(d, next, target, cand, tally);
     }
 }
 
@@ -316,7 +345,7 @@ struct SsspListShared {
     int sum[SSSP_WARPS];
 };
 template <int DT>
-__device__ void sssp_expand_list(const Device &d, const int32_t *list, int cnt, const SsspNext &next, SsspListShared &sh) {
+__device__ void sssp_expand_list(const Device &d, const int32_t *list, int cnt, const SsspNext &next, SsspListShared &sh, SsspTally &tally) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int U = PD_CHUNK / 32;
     static_assert(PD_PAYLOAD / 2 == U, "one element per lane and step either way");
@@ -324,7 +353,9 @@ __device__ void sssp_expand_list(const Device &d, const int32_t *list, int cnt, 
     int j = 0, first = 0, deg = 0, pfirst = 0, pdeg = 0;
     if (tid < cnt) {
         j = __ldcg(list + tid);
-        sh.x[tid] = sssp_value(__ldcg(next.was + j));
+        const int w = __ldcg(next.was + j);
+        sh.x[tid] = sssp_value(w);
+        if (blockIdx.x == 0) atomicMin(next.word + j, w);
         column_run(d, j, first, deg);
         if (d.n_payload) payload_run(d, j >> 4, pfirst, pdeg);
         if (!DBS_CHK_RANGE(d, first, deg)) deg = 0;
@@ -371,7 +402,7 @@ __device__ void sssp_expand_list(const Device &d, const int32_t *list, int cnt, 
 #pragma unroll
             for (int u = 0; u < U; ++u) { target[u] = in[u] ? (int)(rb[u] * 16u) + (lane & 15) : -1; cand[u] += x; }
         }
-        sssp_relax<U>(next, target, cand);
+        sssp_relax<U>(d, next, target, cand, tally);
     }
 }
 
@@ -416,6 +447,14 @@ struct SsspPullShared {
     int cursor;                                   // groups of rows taken by the thread block's warps
 };
 
+// A row lowered to `best`, below its distance `had`, by one of several threads that may.
+__device__ __forceinline__ void sssp_lower(const Device &d, int *word, uint32_t *next, int row, int best, int had, SsspTally &tally) {
+    tally.low = min(tally.low, best);
+    if (atomicMin(word + row, best) < had) return;     // (not the first)
+    atomicOr(next + (row >> 5), 1u << (row & 31));
+    ++tally.found;
+    tally.edges += sssp_degree(d, row);
+}
 // Chunks of the n <= 32 long rows that a warp has met.
 template <bool VAL>
 __device__ __forceinline__ void sssp_list_long(const Device &d, const SsspState &s, const int4 *longs, int n, float xmin, int32_t *n_long, int lane) {
@@ -443,12 +482,12 @@ __device__ __forceinline__ void sssp_list_long(const Device &d, const SsspState 
     for (int c = 0; c < chunks; ++c) s.chunks[at++] = make_int4(r.x, r.y + c * SSSP_CHUNK, min(r.z, r.y + (c + 1) * SSSP_CHUNK), 0);
 }
 
-// Handles with weights write the words of the other array, all of them, and mark and count what they lower: the step needs no pass behind it.  What is counted of a row (its column's degree) comes with
+// The words of the other array are written, all of them; with weights a row has one writer until the chunks, without (payload entries lower it too) they are lowered by atomics.  What is counted of a row (its column's degree) comes with
 // the row's own words, 32 rows at a time: fetched where a row ends, a whole warp waits for it in most rounds (2^20 vertices 358 -> 400 us a search), and so it does for a look at the old frontier's
 // marks that would spare the words that do not change (358 -> 405).  The distances of the 4 to 32 K columns of the highest degree in shared memory, where 34 to 69 % of the elements lie: nothing
 // gained with 4 K of them (before what it costs to bring them there), slower with more -- what they take from the L1 are the lines that the other gathers wait in.
 template <int DT>
-__device__ void sssp_pull(const Device &d, const SsspState &s, int c, uint32_t *F, uint32_t *next, int t, int low, int32_t *n_long, SsspPullShared &sh, SsspSums &sums) {
+__device__ void sssp_pull(const Device &d, const SsspState &s, int c, const uint32_t *F, uint32_t *next, int low, int32_t *n_long, SsspPullShared &sh, SsspTally &tally) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int NONE = 0x7F800000;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -480,13 +519,11 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, int c, uint32_t *
         const int64_t g = (int64_t)i * gridDim.x + (blockIdx.x + i) % gridDim.x, r = g * 32 + lane;
         row_g = (int)(r < d.n ? r : d.n); p_g = 0; e_g = 0; have_g = 0;
         if (r < d.n) { p_g = ptr[r]; e_g = ptr[r + 1]; have_g = __ldcg(dist + r); if (VAL) { w_g = d.row_lightest[r]; code_g = d.col_degree[r]; } }
-        if (VAL && lane == 0 && g < s.n_words) F[g] = 0u;           // (nobody looks at the frontier's marks; the bitmap is the one of the step after the next)
     };
     fetch();
     int head = 0, cnt = 0, n_listed = 0;
     int row = -1, p = 0, e = 0, have = 0, best = NONE, q_long = 0;      // the row being walked: elements [p, e), from q_long on it is long
-    int found = 0, lowest = NONE, degree = 0;
-    unsigned edges = 0;
+    int degree = 0;
     for (;;) {
         while (more && cnt < 32) {                     // (no more than that: what a warp has claimed no other one can take)
             const bool pass = p_g < e_g && sssp_word(xmin + w_g) < have_g;
@@ -496,7 +533,9 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, int c, uint32_t *
                 queue[at] = make_int4(row_g, p_g, e_g, have_g);
                 if (VAL) queue_degree[at] = (int)degree_of_code(code_g);
             }
-            if (VAL && row_g < d.n) __stcg(word + row_g, have_g);       // (what the row's walk finds comes on top, from this warp too)
+            if (row_g < d.n) {                         // (what the row's walk finds comes on top, from this warp too)
+                if (VAL) __stcg(word + row_g, have_g); else atomicMin(word + row_g, have_g);
+            }
             cnt += __popc(m);
             fetch();
         }
@@ -537,10 +576,11 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, int c, uint32_t *
             const bool over = p >= e || bound(last) >= best;
             left = !over && p >= q_long;
             if ((over || left) && best < have) {
-                // (a row has one owner; the chunks of a long one follow behind a barrier.  Without values the payload entries lower it too.)
-                if (VAL) __stcg(word + row, best); else atomicMin(word + row, best);
-                atomicOr(next + (row >> 5), 1u << (row & 31));
-                if (VAL) { ++found; lowest = min(lowest, best); edges += (unsigned)degree; }
+                if (VAL) {
+                    __stcg(word + row, best);
+                    atomicOr(next + (row >> 5), 1u << (row & 31));
+                    ++tally.found; tally.low = min(tally.low, best); tally.edges += (unsigned)degree;
+                } else sssp_lower(d, word, next, row, best, have, tally);
             }
             if (over) row = -1;
         }
@@ -553,7 +593,7 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, int c, uint32_t *
     }
     __syncwarp();
     if (n_listed) sssp_list_long<VAL>(d, s, longs, n_listed, xmin, n_long, lane);
-    if (VAL) { sssp_count(s, sums, (t + 1) % 3, found, lowest, edges); return; }
+    if (VAL) return;
     // entries with a payload (unit weights): one block per warp at a time, columns of the frontier only (the blocks sit where a power-law graph is dense, among
     // the vertices that settle first: late large steps skip most of them); the next entry is fetched meanwhile
     struct Entry { uint32_t idx, w, aux; int rb; };
@@ -577,8 +617,8 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, int c, uint32_t *
         const uint32_t xm = mask_of(F, cb);
         if (!xm) continue;                                                               // warp-uniform
         block_rows_min_warp<DT>(type, e.w, e.aux, xm, reinterpret_cast<const float *>(dist) + (size_t)cb * 16, d.payload, lane, [&](int r, uint32_t key) {
-            const int c = sssp_word(minplus_value(key)), row = e.rb * 16 + r;
-            if (c < __ldcg(word + row) && c < atomicMin(word + row, c)) atomicOr(next + (row >> 5), 1u << (row & 31));
+            const int v = sssp_word(minplus_value(key)), row = e.rb * 16 + r, had = __ldcg(dist + row);
+            if (v < had) sssp_lower(d, word, next, row, v, had, tally);
         });
     }
 }
@@ -586,7 +626,7 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, int c, uint32_t *
 // The listed chunks of long rows, a warp per chunk, four elements per lane and step.  The next chunk's record, best and first elements are
 // fetched while this one's distances arrive.
 template <int DT>
-__device__ void sssp_pull_long(const Device &d, const SsspState &s, int c, uint32_t *next, int t, int low, int n, SsspSums &sums) {
+__device__ void sssp_pull_long(const Device &d, const SsspState &s, int c, uint32_t *next, int low, int n, SsspTally &tally) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int NONE = 0x7F800000;
     const int lane = threadIdx.x & 31;
@@ -599,8 +639,6 @@ __device__ void sssp_pull_long(const Device &d, const SsspState &s, int c, uint3
     uint32_t col[4] = {0u, 0u, 0u, 0u};
     float w[4] = {0.f, 0.f, 0.f, 0.f};
     int had = 0;
-    int found = 0, lowest = NONE;
-    unsigned edges = 0;
     auto first = [&](const int4 &r) {
         const int k0 = (r.y & ~3) + 4 * lane;
         if (k0 < r.z) { had = __ldcg(word + r.x); sssp_four<VAL>(d, k0, col, w); }
@@ -636,15 +674,13 @@ __device__ void sssp_pull_long(const Device &d, const SsspState &s, int c, uint3
             }
         }
         if (lane == 0 && now < start) {
-            atomicMin(word + row, now);
+            // (a row of several chunks is counted by the one that marks it)
             const uint32_t bit = 1u << (row & 31);
-            if (VAL) {                                 // (a row of several chunks is counted by the one that marks it)
-                lowest = min(lowest, now);
-                if (!(atomicOr(next + (row >> 5), bit) & bit)) { ++found; edges += degree_of_code(d.col_degree[row]); }
-            } else atomicOr(next + (row >> 5), bit);
+            atomicMin(word + row, now);
+            tally.low = min(tally.low, now);
+            if (!(atomicOr(next + (row >> 5), bit) & bit)) { ++tally.found; tally.edges += sssp_degree(d, row); }
         }
     }
-    if (VAL) sssp_count(s, sums, (t + 1) % 3, found, lowest, edges);
 }
 
 constexpr int SSSP_SMEM = (int)(sizeof(SsspShared) > sizeof(SsspPullShared) ? sizeof(SsspShared) : sizeof(SsspPullShared));
@@ -653,146 +689,66 @@ static_assert(sizeof(SsspListShared) <= sizeof(SsspShared), "the phases share on
 // spilled more besides (216 -> 88 bytes of stack; R-MAT 300 K / 500 K / 2^20 vertices 242 / 252 / 359 -> 222 / 227 / 331 us a search, in scattered order 202 / 237 / 333 -> 186 / 217 / 306; 27-point
 // operator on 90^3 cells, an inner source, 3029 -> 2947).  The phases as functions of their own, which share no registers: 233 / 239 / 343 us.
 template <int DT>
-__global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ Device d, const __grid_constant__ SsspState s, int32_t src, float *dist_out, int start, int max_steps, unsigned long long pull_edges, unsigned long long late_edges) {
+__global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ Device d, const __grid_constant__ SsspState s, int32_t src, float *dist_out, int start, int max_steps, unsigned pull_edges, unsigned late_edges) {
     namespace cg = cooperative_groups;
     extern __shared__ __align__(16) uint8_t s_dyn[];
     __shared__ SsspSums sums;
-    constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     SsspShared &sh = *reinterpret_cast<SsspShared *>(s_dyn);
     cg::grid_group grid = cg::this_grid();
-    const int tid = blockIdx.x * SSSP_CTA + threadIdx.x, nthreads = gridDim.x * SSSP_CTA, lane = threadIdx.x & 31;
+    const int tid = blockIdx.x * SSSP_CTA + threadIdx.x, nthreads = gridDim.x * SSSP_CTA;
     if (start) {                                       // (a later launch of the same search continues where the one before stopped)
         const int64_t n = (int64_t)s.n_words * 32;
         for (int64_t v = tid; v < n; v += nthreads) s.word[0][v] = s.word[1][v] = v == src ? 0 : 0x7F800000;
-        for (int k = tid; k < s.n_words; k += nthreads) { s.bits[0][k] = k == src >> 5 ? 1u << (src & 31) : 0u; s.bits[1][k] = 0u; }
-        if (tid < 6) s.ctr[tid] = tid == 0 ? 1 : 0;
-        if (tid == 6) {
+        for (int k = tid; k < s.n_words; k += nthreads) { s.bits[0][k] = k == src >> 5 ? 1u << (src & 31) : 0u; s.bits[1][k] = 0u; }       // (the third is cleared by the first step)
+        if (tid == 0) {
             int first, deg;
             column_run(d, src, first, deg);
-            s.ctr[6] = 0; s.ctr[7] = 0;
-            for (int k = 0; k < 3; ++k) { s.low[k] = k == 0 ? 0 : 0x7F800000; s.edges[k] = k == 0 ? (unsigned long long)deg : 0ull; s.ctr[18 + k] = 0; }
+            for (int k = 0; k < 5; ++k) s.ctr[k] = 0;
+            for (int k = 0; k < 3; ++k) s.set[k] = SsspSet{k == 0 ? (unsigned)deg : 0u, k == 0 ? 1u : 0u, k == 0 ? 0 : 0x7F800000, 0};
             s.list[1][0] = src;
         }
         grid.sync();
     }
-    int t = s.ctr[6], c = s.ctr[7];
+    auto read = [&](int k) {
+        const int4 v = __ldcg(reinterpret_cast<const int4 *>(s.set + k));
+        return SsspSet{(unsigned)v.x, (unsigned)v.y, v.z, v.w};
+    };
+    int t = __ldcg(s.ctr), c = __ldcg(s.ctr + 1);      // array c holds the distances; so does the other one, but for the frontier, of which it has larger ones
     bool late = false;                                 // a step has been pulled
-    bool listed = start != 0;                          // the frontier is in list[(t + 1) & 1]
-    bool agree = true;                                 // both arrays hold the distances (else array c does)
-    for (int made = 0; made < max_steps; ++made, ++t) {
-        const int cnt = __ldcg(s.ctr + t % 3);         // grid-uniform, as all that is decided from it
-        const unsigned long long edges_now = __ldcg(s.edges + t % 3);
-        const int low_now = __ldcg(s.low + t % 3);
-        if (cnt == 0) break;
-        uint32_t *F = s.bits[t & 1], *N = s.bits[(t + 1) & 1];
-        int32_t *n_long = s.ctr + 3 + t % 3, *n_list = s.ctr + 18 + t % 3;
-        const bool pulled = edges_now > (late ? late_edges : pull_edges), lists = !pulled && edges_now <= SSSP_LIST_EDGES;
-        if (tid == 0) { s.ctr[3 + (t + 1) % 3] = 0; s.ctr[18 + (t + 1) % 3] = 0; }      // (their last reader was step t - 2)
+    bool lists = start != 0;                           // the step before listed what it marked, in list[(t + 1) & 1]
+    SsspSet now = read(t % 3);                         // grid-uniform, as all that is decided from it
+    for (int made = 0; made < max_steps && now.found; ++made, ++t, c ^= 1) {
+        const uint32_t *F = s.bits[t % 3];
+        uint32_t *N = s.bits[(t + 1) % 3], *Z = s.bits[(t + 2) % 3];
+        const int nxt = (t + 1) % 3;
+        int32_t *n_long = &s.set[nxt].n_long, *n_list = s.ctr + 2 + t % 3;
+        const bool listed = lists && now.found <= SSSP_LIST, pulled = now.edges > (late ? late_edges : pull_edges);
         late = late || pulled;
-        if (VAL && pulled) {
-            if (tid == 0) { s.ctr[(t + 2) % 3] = 0; s.low[(t + 2) % 3] = 0x7F800000; s.edges[(t + 2) % 3] = 0ull; }
-            sssp_pull<DT>(d, s, c, F, N, t, low_now, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), sums);
-            grid.sync();
-            const int n = __ldcg(n_long);
-            if (n > 0) {                               // grid-uniform
-                sssp_pull_long<DT>(d, s, c, N, t, low_now, n, sums);
-                grid.sync();
-            }
-            c ^= 1;
-            agree = false;
-            listed = false;
-            continue;
-        }
-        if (!agree) {                                  // behind a pulled step: what it lowered, in the other array too
-            for (int w = tid >> 5; w < s.n_words; w += nthreads >> 5)
-                if ((__ldcg(F + w) >> lane) & 1u) s.word[c ^ 1][w * 32 + lane] = __ldcg(s.word[c] + w * 32 + lane);
-            grid.sync();
-            agree = true;
-        }
-        int *const dist = s.word[c], *const word = s.word[c ^ 1];
-        const SsspNext next{dist, word, N, lists ? s.list[t & 1] : nullptr, n_list};
-        if (pulled) {
-            sssp_pull<DT>(d, s, c, F, N, t, low_now, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), sums);
-            grid.sync();
-            const int n = __ldcg(n_long);
-            if (n > 0) {                               // grid-uniform
-                sssp_pull_long<DT>(d, s, c, N, t, low_now, n, sums);
-                grid.sync();
-            }
-        } else if (listed) {
-            sssp_expand_list<DT>(d, s.list[(t + 1) & 1], cnt, next, *reinterpret_cast<SsspListShared *>(s_dyn));
-            grid.sync();
-        } else {
-            sssp_expand<DT>(d, s, F, next, n_long, sh);
-            grid.sync();
-            const int n = __ldcg(n_long);
-            if (n > 0) {                               // grid-uniform
-                sssp_long<DT>(d, next, n);
-                grid.sync();
-            }
-        }
-        if (tid == 0) { s.ctr[(t + 2) % 3] = 0; s.low[(t + 2) % 3] = 0x7F800000; s.edges[(t + 2) % 3] = 0ull; }
-        const bool was_listed = listed;
-        const int n_marked = lists ? __ldcg(n_list) : 0;
-        listed = lists && n_marked <= SSSP_LIST;
-        int found = 0, low = 0x7F800000;
-        unsigned edges = 0;
-        if (listed) {                                  // one thread block settles, the others clear the old frontier if it is not listed
-            if (!was_listed) for (int k = tid; k < s.n_words; k += nthreads) F[k] = 0u;
-            if (blockIdx.x == 0) {
-                if (was_listed && (int)threadIdx.x < cnt) F[__ldcg(s.list[(t + 1) & 1] + threadIdx.x) >> 5] = 0u;
-                if ((int)threadIdx.x < n_marked) {
-                    const int j = __ldcg(s.list[t & 1] + threadIdx.x);
-                    low = __ldcg(word + j);
-                    int first, deg;
-                    column_run(d, j, first, deg);
-                    edges = (unsigned)deg;
-                    dist[j] = low;
-                }
-            }
-        } else {
-            const int gwarp = tid >> 5, nwarps = nthreads >> 5;
-            for (int w0 = gwarp; w0 < s.n_words; w0 += 8 * nwarps) {
-                uint32_t b[8];
-                int v[8], deg[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) { const int w = w0 + q * nwarps; b[q] = w < s.n_words ? __ldcg(N + w) : 0u; }
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    v[q] = 0x7F800000; deg[q] = 0;
-                    if ((b[q] >> lane) & 1u) {
-                        const int j = (w0 + q * nwarps) * 32 + lane;
-                        v[q] = __ldcg(word + j);
-                        if (d.col_degree) deg[q] = (int)d.col_degree[j];      // (a byte each: with the column pointers the pass took a third longer)
-                        else { int first; column_run(d, j, first, deg[q]); deg[q] = (int)degree_code((uint32_t)deg[q]); }
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int w = w0 + q * nwarps;
-                    if (w >= s.n_words) break;
-                    if ((b[q] >> lane) & 1u) dist[w * 32 + lane] = v[q];
-                    if (lane == 0) F[w] = 0u;
-                    found += __popc(b[q]);
-                    low = min(low, v[q]);
-                    edges += degree_of_code((uint32_t)deg[q]);
-                }
-            }
-            if (lane != 0) found = 0;                  // (a word's marks are counted once)
-        }
-        if (listed) {
-            if (sssp_sum(sums, found, low, edges) && blockIdx.x == 0) { s.ctr[(t + 1) % 3] = n_marked; s.low[(t + 1) % 3] = low; s.edges[(t + 1) % 3] = edges; }
-        } else sssp_count(s, sums, (t + 1) % 3, found, low, edges);
+        lists = !pulled && now.edges <= SSSP_LIST_EDGES;
+        if (tid == 0) { s.ctr[2 + nxt] = 0; s.set[(t + 2) % 3] = SsspSet{0u, 0u, 0x7F800000, 0}; }      // (their last readers were the steps t - 2 and t - 1)
+        const SsspNext next{s.word[c], s.word[c ^ 1], N, lists ? s.list[t & 1] : nullptr, n_list};
+        SsspTally tally;
+        if (pulled) sssp_pull<DT>(d, s, c, F, N, now.low, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), tally);
+        else if (listed) sssp_expand_list<DT>(d, s.list[(t + 1) & 1], (int)now.found, next, *reinterpret_cast<SsspListShared *>(s_dyn), tally);
+        else sssp_expand<DT>(d, s, F, next, n_long, sh, tally);
+        for (int k = tid; k < s.n_words; k += nthreads) Z[k] = 0u;
+        sssp_count(s, sums, nxt, tally);
         grid.sync();
+        const int low = now.low;
+        now = read(nxt);
+        if (now.n_long > 0) {                          // chunks of long runs or rows
+            SsspTally more;
+            if (pulled) sssp_pull_long<DT>(d, s, c, N, low, now.n_long, more);
+            else sssp_long<DT>(d, next, now.n_long, more);
+            sssp_count(s, sums, nxt, more);
+            grid.sync();
+            now = read(nxt);
+        }
     }
-    // the distances themselves; a search that goes on starts from arrays that agree
-    for (int64_t v = tid; v < d.n; v += nthreads) {
-        const int w = __ldcg(s.word[c] + v);
-        dist_out[v] = sssp_value(w);
-        if (!agree) s.word[c ^ 1][v] = w;
-    }
-    // (everyone read ctr[6] and ctr[7] before the first barrier, or leaves without a step)
-    if (tid == 0) { s.ctr[6] = t; s.ctr[7] = c; s.report[0] = t; s.report[1] = __ldcg(s.ctr + t % 3); }
+    // the distances themselves
+    for (int64_t v = tid; v < d.n; v += nthreads) dist_out[v] = sssp_value(__ldcg(s.word[c] + v));
+    // (everyone read the counters before the first barrier, or leaves without a step)
+    if (tid == 0) { s.ctr[0] = t; s.ctr[1] = c; s.report[0] = t; s.report[1] = (int)now.found; }
 }
 
 }  // namespace dbs
