@@ -482,6 +482,70 @@ __device__ __forceinline__ void sssp_list_long(const Device &d, const SsspState 
     for (int c = 0; c < chunks; ++c) s.chunks[at++] = make_int4(r.x, r.y + c * SSSP_CHUNK, min(r.z, r.y + (c + 1) * SSSP_CHUNK), 0);
 }
 
+// A pulled step of a graph with no more rows than the GPU has lanes (handles with weights): 1 << share lanes share a row, four elements each a round, so that a row is a round or two instead of up to
+// eight one after the other; what is left of it after SSSP_SHARED_ROUNDS of them is listed.  What bounds the step there is that chain (a round takes 2 us whatever it holds) with most warps idle.
+// A lane per row / so: 16 K vertices 102 / 78 us a search, in scattered order 113 / 88, 40 K 113 / 95, 65 K 104 / 86 in scattered order, 131 K 140 / 129 (104 / 96); two lanes per row also on 300 K
+// 125 / 121 (120 / 124), on 500 K 205 / 232: not above the number of lanes.  Four lanes on 65 K 96 in place of 87, on 40 K the same: as many as there are for every row.  Eight rounds: 83, 93, 100, 102, 137 (102).
+constexpr int SSSP_SHARED_ROUNDS = 4;
+static_assert(8 * SSSP_SHARED_ROUNDS - 3 > 4 * (SSSP_ROUNDS - 1), "the list of chunks has room for rows of that length (run.cu)");
+__device__ __forceinline__ int sssp_row_share(int64_t n, int nthreads) {
+    int share = n <= nthreads ? 1 : 0;
+    while (share && share < 3 && n << (share + 1) <= nthreads) ++share;
+    return share;
+}
+__device__ void sssp_pull_shared(const Device &d, const SsspState &s, int c, uint32_t *next, int share, int low, int32_t *n_long, SsspPullShared &sh, SsspTally &tally) {
+    constexpr int NONE = 0x7F800000;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane & ((1 << share) - 1), rows = 32 >> share;
+    const int nwarps = (int)(gridDim.x * SSSP_CTA) >> 5;
+    const float xmin = sssp_value(low);
+    const int *const dist = s.word[c];
+    int *const word = s.word[c ^ 1];
+    // (neighbouring rows on different SMs: they are heavy together on an R-MAT graph that was not relabelled)
+    for (int64_t r0 = (int64_t)(warp * (int)gridDim.x + (int)blockIdx.x) * rows; r0 < d.n; r0 += (int64_t)nwarps * rows) {
+        const int64_t r = r0 + (lane >> share);
+        int p = 0, e = 0, have = 0, degree = 0;
+        float lightest = 0.f;
+        if (r < d.n) { p = d.weight_ptr[r]; e = d.weight_ptr[r + 1]; have = __ldcg(dist + r); lightest = d.row_lightest[r]; degree = (int)d.col_degree[r]; }
+        int best = have;
+        bool walks = p < e && sssp_word(xmin + lightest) < have;
+        for (int round = 0; round < SSSP_SHARED_ROUNDS && __any_sync(FULL, walks); ++round) {
+            const int q = (p & ~3) + 4 * sub;
+            uint32_t col[4];
+            float w[4] = {0.f, 0.f, 0.f, 0.f};
+            int x[4] = {NONE, NONE, NONE, NONE};
+            if (walks && q < e) {
+                sssp_four<true>(d, q, col, w);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (q + j >= p && q + j < e && sssp_word(xmin + w[j]) < best && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
+            }
+            int mine = best;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) mine = min(mine, sssp_word(sssp_value(x[j]) + w[j]));
+            for (int o = 1; o < 1 << share; o <<= 1) mine = min(mine, __shfl_xor_sync(FULL, mine, o));
+            const float last = __shfl_sync(FULL, w[3], lane | ((1 << share) - 1));      // (the largest weight of the round)
+            best = mine;
+            p = (p & ~3) + (4 << share);
+            walks = walks && p < e && sssp_bound<true>(xmin, last) < best;
+        }
+        if (sub == 0 && r < d.n) {
+            __stcg(word + r, best);
+            if (best < have) {
+                atomicOr(next + (r >> 5), 1u << (r & 31));
+                ++tally.found; tally.low = min(tally.low, best); tally.edges += degree_of_code((uint32_t)degree);
+            }
+        }
+        const uint32_t left = __ballot_sync(FULL, walks && sub == 0);
+        if (left) {
+            int4 *longs = sh.longs[warp];
+            if (walks && sub == 0) longs[__popc(left & ((1u << lane) - 1u))] = make_int4((int)r, p, e, best);
+            __syncwarp();
+            sssp_list_long<true>(d, s, longs, __popc(left), xmin, n_long, lane);
+            __syncwarp();
+        }
+    }
+}
+
 // The words of the other array are written, all of them; with weights a row has one writer until the chunks, without (payload entries lower it too) they are lowered by atomics.  What is counted of a row (its column's degree) comes with
 // the row's own words, 32 rows at a time: fetched where a row ends, a whole warp waits for it in most rounds (2^20 vertices 358 -> 400 us a search), and so it does for a look at the old frontier's
 // marks that would spare the words that do not change (358 -> 405).  The distances of the 4 to 32 K columns of the highest degree in shared memory, where 34 to 69 % of the elements lie: nothing
@@ -728,7 +792,9 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
         if (tid == 0) { s.ctr[2 + nxt] = 0; s.set[(t + 2) % 3] = SsspSet{0u, 0u, 0x7F800000, 0}; }      // (their last readers were the steps t - 2 and t - 1)
         const SsspNext next{s.word[c], s.word[c ^ 1], N, lists ? s.list[t & 1] : nullptr, n_list};
         SsspTally tally;
-        if (pulled) sssp_pull<DT>(d, s, c, F, N, now.low, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), tally);
+        const int share = DT != DBSPMSPV_PATTERN ? sssp_row_share(d.n, nthreads) : 0;
+        if (pulled && share) sssp_pull_shared(d, s, c, N, share, now.low, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), tally);
+        else if (pulled) sssp_pull<DT>(d, s, c, F, N, now.low, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), tally);
         else if (listed) sssp_expand_list<DT>(d, s.list[(t + 1) & 1], (int)now.found, next, *reinterpret_cast<SsspListShared *>(s_dyn), tally);
         else sssp_expand<DT>(d, s, F, next, n_long, sh, tally);
         for (int k = tid; k < s.n_words; k += nthreads) Z[k] = 0u;

@@ -111,7 +111,18 @@ def test_listed_and_unlisted_frontiers(fan, dtype):
 def test_rows_of_a_pulled_step(length):
     """Rows at the lengths where a lane hands a row over and where what is left of it is one chunk or several, dense blocks among their elements; the
     vertices they lie behind are reached in one step, so that the next one is pulled, and once more with better distances a step later."""
-    n = 6007
+    rows_of_a_pulled_step(6007, length)
+
+
+@pytest.mark.parametrize("length", [3, 16, 17, 29, 33, 65, 129, 545])
+@pytest.mark.parametrize("lanes", [8, 4, 2, 1, 0])
+def test_lanes_that_share_a_row_of_a_pulled_step(length, lanes):
+    """The same rows in graphs of as many vertices as leave two, four or eight lanes of the GPU for each, with the last rows at the end of the range, and of one more than it has lanes."""
+    threads = 1024 * torch.cuda.get_device_properties(0).multi_processor_count
+    rows_of_a_pulled_step(threads // lanes if lanes else threads + 1, length)
+
+
+def rows_of_a_pulled_step(n, length):
     rng = np.random.default_rng(length)
     src, late = 0, 1
     mid = np.arange(32, 32 + 2700)                         # reached from the source; half of them again, for less, by way of `late`
