@@ -8,6 +8,7 @@
 
 #include "internal.cuh"
 #include "microkernels.cuh"
+#include "push_direct.cuh"
 #include "worklist.cuh"
 
 namespace cg = cooperative_groups;
@@ -50,31 +51,32 @@ struct Scope {
     int gwarp, nwarps;      // warp index / count in the scope
 };
 
-// Appends word indices (one per lane with `word` >= 0) to a list: one atomic per warp.
-__device__ __forceinline__ void append_words(int word, int32_t *list, int32_t *count, int lane) {
-    const uint32_t m = __ballot_sync(FULL, word >= 0);
-    if (!m) return;
-    int base = 0;
-    if (lane == __ffs(m) - 1) base = atomicAdd(count, __popc(m));
-    base = __shfl_sync(FULL, base, __ffs(m) - 1);
-    if (word >= 0) list[base + __popc(m & ((1u << lane) - 1u))] = word;
-}
-
-// Where a push level puts what it finds: the next level's frontier and worklist.
+// Where a level puts what it finds: the next level's frontier.
 struct NextLevel {
-    uint32_t *N;                 // frontier masks
-    int32_t *words, *n_words;    // list of the words that became nonzero
-    int32_t *n_blocks, *n_tasks, *n_hubs, *n_edges;   // (n_edges null: not counted, see BFS_LARGE_WORDS)
-    int4 *hubs;
-    uint2 *tasks;
-    bool emit;                   // the worklist is written by this level itself
+    uint32_t *N;                 // masks
+    int32_t *words, *verts;      // lists of the words that became nonzero and of the first BFS_LIST vertices
+    Counters::BfsSet *set;
+    bool counts;                 // the elements of the frontier's columns are counted (see BFS_LARGE_WORDS)
 };
-// A push level of at most this many warp steps, behind which the next one is a push whatever it finds, writes the next level's worklist
-// itself, one phase and one grid barrier (with a pass of its own behind a barrier of its own a level that moves next to nothing took 8.5 us,
-// now 6).  A larger one reaches thousands of vertices: the warps would queue for space in the list (with 256 steps the level took 13 us, and
-// 100 K vertices 72 us in place of 65); and a list that a pull follows is written for nothing (17,000 vertices: a level that
-// reaches a fifth of the blocks from two of them 12.4 us with the list, 6.1 without).
-constexpr int BFS_EMIT_STEPS = 16;
+// Appends what the lanes of a warp found: `mine` vertices each, which put(k, place) writes for k < mine, and (new_word) a mask word that became nonzero.  One atomic for both lists.
+template <typename Put>
+__device__ __forceinline__ void append_found(const NextLevel &nx, int word, bool new_word, int mine, int lane, Put put) {
+    const uint32_t m = __ballot_sync(FULL, new_word);
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
+    unsigned long long base = 0;
+    if (lane == 31) base = atomicAdd(reinterpret_cast<unsigned long long *>(&nx.set->n_verts), (unsigned long long)__popc(m) << 32 | (unsigned)incl);
+    base = __shfl_sync(FULL, base, 31);
+    if (new_word) nx.words[(int)(base >> 32) + __popc(m & ((1u << lane) - 1u))] = word;
+    const int at = (int)(uint32_t)base + incl - mine;
+    for (int k = 0; k < mine && at + k < BFS_LIST; ++k) put(k, at + k);
+}
+// ... the set bits of a word each
+__device__ __forceinline__ void append_words(const NextLevel &nx, int word, uint32_t mask, bool new_word, int lane) {
+    uint32_t left = mask;
+    append_found(nx, word, new_word, __popc(mask), lane, [&](int, int place) { nx.verts[place] = word * 32 + __ffs(left) - 1; left &= left - 1; });
+}
 // Up to this many warp steps the bookkeeping is the claiming lanes': a second atomic per vertex found, but neither a pass nor a barrier
 // behind the level.  Larger levels leave it to a pass over the words that became nonzero, one update for up to 32 vertices: levels of 2^22
 // vertices that reach most of them through a few thousand hubs took 78 - 150 us with an atomic each, 59 - 116 with the pass, and 37 - 71 since the pass writes
@@ -101,8 +103,8 @@ constexpr int BFS_LARGE_WORDS = 8;
 // next-frontier masks.  Like the pull, the loop is software-
 // pipelined: while task k is evaluated, the visited masks of k+1, the view entries of k+2 and
 // the task record of k+3 (in this warp's stride) are in flight.
-// With MARK the winner does the level's bookkeeping for the vertex: it writes its level, marks it visited, lists the word it turned nonzero
-// and, if asked for (NextLevel::emit), the tasks of its column go to the next level's worklist.  Without it nobody looks at a reply: all that is the pass behind the level.
+// With MARK the winner does the level's bookkeeping for the vertex: it writes its level, marks it visited, lists it and the word it turned nonzero.
+// Without it nobody looks at a reply: all that is the pass behind the level.
 template <int DT, bool MARK>
 __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, const uint2 *tasks, int n_recs, const int4 *hubs, int n_hubs,
                          int32_t *levels, int depth, const NextLevel &nx) {
@@ -113,7 +115,7 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
     const int n_tasks = n_recs + table.total;                    // task records, then the steps of the hub runs
     auto item = [&](int i) { return worklist_item(tasks, n_recs, table, i); };
     const uint2 none = make_uint2(0u, 0u);
-    int found = 0, blocks = 0, edges = 0;
+    int blocks = 0, edges = 0;
     // claims the rows `hit` of row block `brow` (called by a full warp; hit = 0: nothing in this lane)
     auto publish = [&](int brow, uint32_t hit) {
         if (!MARK) {                                   // (nobody waits for a reply: levels, list and counts are the pass behind the level)
@@ -131,34 +133,10 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
         if (fresh) {
             write_levels(levels, brow, fresh, depth);
             atomicOr(&d.ws.visited32[brow >> 1], fresh << sh);
-            found += __popc(fresh);
             blocks += newly;
-            if (nx.n_edges) for (uint32_t f = fresh; f; f &= f - 1) edges += (int)degree_of_code(d.col_degree[brow * 16 + __ffs(f) - 1]);
+            if (nx.counts) for (uint32_t f = fresh; f; f &= f - 1) edges += (int)degree_of_code(d.col_degree[brow * 16 + __ffs(f) - 1]);
         }
-        append_words(fresh && !old ? brow >> 1 : -1, nx.words, nx.n_words, lane);
-        if (!nx.emit) return;
-        // the vertices found, 32 at a time (blocks with a payload reach several rows at once): vertex k belongs to the last lane whose prefix is <= k
-        int incl = __popc(fresh);
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
-        const int excl = incl - __popc(fresh), total = __shfl_sync(FULL, incl, 31);
-        for (int k0 = 0; k0 < total; k0 += 32) {
-            const int k = k0 + lane;
-            int o = 0;
-#pragma unroll
-            for (int st = 16; st; st >>= 1) { const int t = __shfl_sync(FULL, excl, o + st); if (t <= k) o += st; }
-            uint32_t m = __shfl_sync(FULL, fresh, o);
-            const int vb = __shfl_sync(FULL, brow, o), skip = k - __shfl_sync(FULL, excl, o);
-            int first = 0, deg = 0;
-            if (k < total) {
-                for (int t = 0; t < skip; ++t) m &= m - 1;
-                column_run(d, vb * 16 + __ffs(m) - 1, first, deg);
-            }
-            emit_tasks(d, false, vb, first, deg, lane, nx.n_tasks, nx.n_blocks, PUSH_CHUNK, nx.n_hubs, nx.hubs, nx.tasks);
-        }
-        int pfirst = 0, pdeg = 0;
-        if (newly) payload_run(d, brow, pfirst, pdeg);
-        if (__any_sync(FULL, pdeg > 0)) emit_tasks(d, false, brow, pfirst, pdeg, lane, nx.n_tasks, nx.n_blocks, d.payload_chunk, nullptr, nullptr, nx.tasks);
+        append_words(nx, brow >> 1, fresh << sh, fresh && !old, lane);
     };
     struct Entries { uint32_t idx, aux, xm; int n, start; };   // n: entries of the task (0 = no task)
     auto entries_of = [&](int t, const uint2 &task) {
@@ -227,10 +205,119 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
         // rotate the pipeline
         e0 = e1; e1 = e2; need0 = need1; t2 = t3;
     }
-    found = __reduce_add_sync(FULL, found);
+    if (!MARK) return;
     blocks = __reduce_add_sync(FULL, blocks);
-    if (MARK && nx.n_edges) edges = __reduce_add_sync(FULL, edges);
-    if (MARK && lane == 0 && found) { atomicAdd(&d.ws.ctr->bfs_reached, found); atomicAdd(nx.n_blocks, blocks); if (nx.n_edges) atomicAdd(nx.n_edges, edges); }
+    if (nx.counts) edges = __reduce_add_sync(FULL, edges);
+    if (lane == 0 && blocks) { atomicAdd(&nx.set->n_blocks, blocks); if (nx.counts) atomicAdd(&nx.set->edges, edges); }
+}
+
+// A short listed frontier, pushed without a worklist: every thread block lays the vertices' runs of INLINE elements and of the payload entries of their column blocks end to end in chunks, the
+// warps of the grid share them out, and the claiming lanes do the bookkeeping.  Such a level moves next to nothing; it is the chain list -> column pointers -> entries -> visited -> claim -> list, one
+// barrier behind it (a worklist is one more phase and barrier in front).  Every frontier of at most BFS_LIST vertices has its list, whichever way its level went.  Searches, symmetrised R-MAT, eight
+// sources each, with worklists / so, in brackets in scattered order: 16 K vertices 45.6 / 40.2 us (42.2 / 39.4), 65 K 54.7 / 48.2 (50.3 / 43.0), 262 K 53.4 / 42.8 (57.7 / 46.6), 2^20 75.3 / 61.6
+// (75.7 / 67.2), 2^22 138.8 / 130.2 (112.6 / 110.2); part of it are the counters of a level, one 16-byte load behind its last barrier in place of four to seven loads one after the other.
+struct BfsListShared {
+    int pre[BFS_LIST + 1];                            // chunks before a vertex
+    int vertex[BFS_LIST], first[BFS_LIST], deg[BFS_LIST], pfirst[BFS_LIST], pdeg[BFS_LIST];
+    int sum[BFS_CTA / 32], elems[BFS_CTA / 32];
+};
+static_assert(BFS_LIST == BFS_CTA, "a thread per listed vertex");
+// Lays the chunks out; returns their number, and the elements behind them (the same in every thread).
+__device__ int bfs_list_layout(const Device &d, const int32_t *verts, int cnt, BfsListShared &sh, int &n_elems) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int j = 0, first = 0, deg = 0, pfirst = 0, pdeg = 0;
+    if (tid < cnt) {
+        j = __ldcg(verts + tid);
+        if (!DBS_CHK_INDEX(d, j, d.n)) j = 0;
+        column_run(d, j, first, deg);
+        payload_run(d, j >> 4, pfirst, pdeg);
+    }
+    sh.vertex[tid] = j; sh.first[tid] = first; sh.deg[tid] = deg; sh.pfirst[tid] = pfirst; sh.pdeg[tid] = pdeg;
+    const int mine = (deg + PD_CHUNK - 1) / PD_CHUNK + (pdeg + PD_PAYLOAD - 1) / PD_PAYLOAD;
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += t; }
+    const int elems = __reduce_add_sync(FULL, deg + pdeg);
+    if (lane == 31) { sh.sum[warp] = incl; sh.elems[warp] = elems; }
+    __syncthreads();
+    const int v = sh.sum[lane], total = __reduce_add_sync(FULL, v);
+    n_elems = __reduce_add_sync(FULL, sh.elems[lane]);
+    sh.pre[tid] = incl - mine + __reduce_add_sync(FULL, lane < warp ? v : 0);
+    if (tid == 0) sh.pre[BFS_LIST] = total;
+    __syncthreads();
+    return total;
+}
+template <int DT>
+__device__ void bfs_push_list(const Device &d, int total, const BfsListShared &sh, int32_t *levels, int depth, const NextLevel &nx) {
+    constexpr int U = PD_CHUNK / 32;
+    static_assert(PD_PAYLOAD / 2 == U, "one element per lane and step either way");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int blocks = 0, edges = 0;
+    // (neighbouring chunks on different SMs)
+    for (int c = warp * (int)gridDim.x + (int)blockIdx.x; c < total; c += (int)gridDim.x * (BFS_CTA / 32)) {
+        int o = 0;                                     // the last vertex with at most c chunks before it
+#pragma unroll
+        for (int st = BFS_LIST / 2; st; st >>= 1) if (sh.pre[o + st] <= c) o += st;
+        const int k = c - sh.pre[o], n_inline = (sh.deg[o] + PD_CHUNK - 1) / PD_CHUNK;
+        int target[U];
+        if (k < n_inline) {                            // warp-uniform
+            const int at = k * PD_CHUNK + lane;
+            uint32_t idx[U], w[U], aux[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                idx[u] = PAD_IDX; w[u] = 0u; aux[u] = 0u;
+                if (at + u * 32 < sh.deg[o]) push_entry<false>(d, sh.first[o] + at + u * 32, idx[u], w[u], aux[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) target[u] = idx[u] < (1u << TYPE_SHIFT) ? (int)((idx[u] & IDX_MASK) * 16u + (aux[u] >> 4)) : -1;
+        } else {
+            const int at = (k - n_inline) * PD_PAYLOAD;
+            bool in[U];
+            float value[U];
+            uint32_t rb[U];
+            payload_elements<DBSPMSPV_PATTERN, U>(d, sh.pfirst[o] + at, min(PD_PAYLOAD, sh.pdeg[o] - at), sh.vertex[o] & 15, lane, in, value, rb);
+#pragma unroll
+            for (int u = 0; u < U; ++u) target[u] = in[u] ? (int)(rb[u] * 16u) + (lane & 15) : -1;
+        }
+        uint32_t seen[U], old[U], fresh = 0u, opened = 0u;
+#pragma unroll
+        for (int u = 0; u < U; ++u) seen[u] = target[u] >= 0 ? __ldcg(d.ws.visited32 + (target[u] >> 5)) : 0xFFFFFFFFu;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            old[u] = 0xFFFFFFFFu;
+            if (!((seen[u] >> (target[u] & 31)) & 1u)) old[u] = atomicOr(nx.N + (target[u] >> 5), 1u << (target[u] & 31));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (!((old[u] >> (target[u] & 31)) & 1u)) {
+                fresh |= 1u << u;
+                levels[target[u]] = depth;
+                atomicOr(d.ws.visited32 + (target[u] >> 5), 1u << (target[u] & 31));
+                blocks += ((old[u] >> (target[u] & 16)) & 0xFFFFu) == 0u;
+                if (!old[u]) opened |= 1u << u;
+            }
+        if (!__any_sync(FULL, fresh != 0u)) continue;
+        // both lists with one scan and one atomic (vertices in the low half of each)
+        const int mine = __popc(fresh) | __popc(opened) << 16;
+        int incl = mine;
+#pragma unroll
+        for (int st = 1; st < 32; st <<= 1) { const int t = __shfl_up_sync(FULL, incl, st); if (lane >= st) incl += t; }
+        unsigned long long base = 0;
+        if (lane == 31) base = atomicAdd(reinterpret_cast<unsigned long long *>(&nx.set->n_verts), (unsigned long long)(unsigned)(incl >> 16) << 32 | (unsigned)(incl & 0xFFFF));
+        if (nx.counts)
+#pragma unroll
+            for (int u = 0; u < U; ++u) if ((fresh >> u) & 1u) edges += (int)degree_of_code(d.col_degree[target[u]]);
+        base = __shfl_sync(FULL, base, 31);
+        int v = (int)(uint32_t)base + ((incl - mine) & 0xFFFF), w = (int)(base >> 32) + ((incl - mine) >> 16);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if ((fresh >> u) & 1u) { if (v < BFS_LIST) nx.verts[v] = target[u]; ++v; }
+            if ((opened >> u) & 1u) nx.words[w++] = target[u] >> 5;
+        }
+    }
+    blocks = __reduce_add_sync(FULL, blocks);
+    if (nx.counts) edges = __reduce_add_sync(FULL, edges);
+    if (lane == 0 && blocks) { atomicAdd(&nx.set->n_blocks, blocks); if (nx.counts) atomicAdd(&nx.set->edges, edges); }
 }
 
 // Boolean pull: one warp per row-block segment (a segment has at most MAX_SEG_ENTRIES = 4 x 32
@@ -369,8 +456,8 @@ __device__ void bfs_pull(const Device &d, const Scope &sc, const uint32_t *F, ui
 constexpr float BFS_WIDE_PULL = DBS_BFS_WIDE_PULL;
 
 template <int DT>
-__device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *N, uint32_t *Z, int32_t *nz_out, int32_t *words_out,
-                                int32_t *nwords_out, int32_t *levels, int depth, bool wide, uint32_t *s_need) {
+__device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *Z, const NextLevel &nx, int32_t *levels, int depth, bool wide, uint32_t *s_need) {
+    uint32_t *const N = nx.N;
     const int lane = threadIdx.x & 31;
     // (neighbouring words on different SMs: on an R-MAT graph that was not relabelled they are heavy together)
     const int gwarp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
@@ -379,7 +466,7 @@ __device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *N, u
     constexpr uint32_t NONE = 0xFFFFFFFFu;          // no entry: local column 31 never matches a 16-bit mask
     constexpr int LONG_UNROLL = 8, MAX_ROUNDS = 8;
     const int per_round = wide ? 8 : 4;
-    int n_found = 0, n_nz = 0;
+    int n_nz = 0;
     const int W = words_per_warp(n_words, nwarps);  // (a lane walks W rows)
     for (int w0 = gwarp * W; w0 < n_words; w0 += nwarps * W) {
         const int wd = w0 + lane;                    // this lane's word (bookkeeping); rows: lane = row of every word
@@ -550,19 +637,11 @@ __device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *N, u
         found &= need;
         if (in) N[wd] = found;
         if (found) d.ws.visited32[wd] |= found;
-        n_found += __popc(found);
         n_nz += ((found & 0xFFFFu) != 0) + ((found >> 16) != 0);
-        const uint32_t listed = __ballot_sync(FULL, found != 0u);
-        if (listed) {
-            int base = 0;
-            if (lane == 0) base = atomicAdd(nwords_out, __popc(listed));
-            base = __shfl_sync(FULL, base, 0);
-            if (found) words_out[base + __popc(listed & ((1u << lane) - 1u))] = wd;
-        }
+        if (__any_sync(FULL, found != 0u)) append_words(nx, wd, found, found != 0u, lane);
     }
-    n_found = __reduce_add_sync(FULL, n_found);
     n_nz = __reduce_add_sync(FULL, n_nz);
-    if (lane == 0 && n_found) { atomicAdd(&d.ws.ctr->bfs_reached, n_found); atomicAdd(nz_out, n_nz); }
+    if (lane == 0 && n_nz) atomicAdd(&nx.set->n_blocks, n_nz);
 }
 
 // Per-level selector (Section 3.3.1): push iff N_nzblk / N_blk < th3.  Monotone in n_nzblk.
@@ -612,12 +691,13 @@ __device__ __forceinline__ int bfs_level_path(const Device &d, int n_nzblk, int 
 
 // One level of the search: the expansion of the frontier of level lv.  Three mask buffers rotate:
 // F holds the frontier, N receives the next one, Z (the frontier before) is cleared meanwhile and
-// becomes N of the next level.  Four lists of nonzero mask words rotate with them -- the list of
-// the frontier produced by level L is list L % 4 -- and three sets of per-level counters, so
-// that nothing is moved or reset behind an extra barrier.
+// becomes N of the next level.  Four lists of nonzero mask words and of vertices rotate with them -- the lists of
+// the frontier produced by level L are number L % 4 -- and three sets of per-level counters, so
+// that nothing is moved or reset behind an extra barrier.  `now`: the counters of the frontier (in: this level's, out: the next one's, fetched once behind the last barrier);
+// z_words: mask words of Z.
 template <int DT>
-__device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc, int lv, int32_t *levels, float th3,
-                          float edge_frac, int force_path, uint32_t *s_need) {
+__device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc, int lv, Counters::BfsSet &now, int z_words, int32_t *levels, float th3,
+                          float edge_frac, int force_path, uint32_t *s_need, BfsListShared &sh) {
     Counters *ctr = d.ws.ctr;
     const int lane = threadIdx.x & 31;
     const int n_words = (d.mb + 1) / 2;
@@ -625,120 +705,108 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
     const int cur = lv % 3, nxt = (lv + 1) % 3, spare = (lv + 2) % 3;
     const uint32_t *F = buf[cur];
     uint32_t *N = buf[nxt], *Z = buf[spare];
-    const int q_out = lv & 3, q_z = (lv + 2) & 3, q_next = (lv + 1) & 3;    // lists: produced now / of Z / produced next
-    int32_t *words_out = d.ws.bfs_words + (size_t)q_out * d.ws.bfs_words_stride;
+    const int q_in = (lv + 3) & 3, q_out = lv & 3, q_z = (lv + 2) & 3;      // lists: of the frontier / produced now / of Z
     const int32_t *words_z = d.ws.bfs_words + (size_t)q_z * d.ws.bfs_words_stride;
     const int depth = lv + 1;
-    const int n_nzblk = ctr->bfs_cnt[cur][0];
-    const int n_tasks = ctr->bfs_cnt[cur][1];
-    const int n_hubs = min(ctr->bfs_hubs[cur], HUB_CAP);
-    int steps = n_tasks;                                // of the worklist: the task records plus the steps of the listed hub runs
-    for (int k = 0; k < n_hubs; ++k) steps += (d.ws.hubs[cur * HUB_CAP + k].z + PUSH_CHUNK - 1) / PUSH_CHUNK;
-    const int path = bfs_level_path(d, n_nzblk, steps, ctr->bfs_edges[cur], th3, edge_frac, force_path);
+    const bool counts = d.col_degree && words_per_warp(n_words, sc.nwarps) >= BFS_LARGE_WORDS;
+    const NextLevel nx{N, d.ws.bfs_words + (size_t)q_out * d.ws.bfs_words_stride, d.ws.bfs_verts + q_out * BFS_LIST, &ctr->bfs_set[nxt], counts};
     // counters that come into use at the next level are reset now: nobody reads or writes them
     // during this one (the previous level was their last reader, behind a barrier)
     if (sc.tid == 0) {
-        ctr->bfs_cnt[spare][0] = 0;
-        ctr->bfs_cnt[spare][1] = 0;
-        ctr->bfs_hubs[spare] = 0;
-        ctr->bfs_edges[spare] = 0;
-        ctr->bfs_nwords[q_next] = 0;
+        ctr->bfs_set[spare] = Counters::BfsSet{0, 0, 0, 0};
+        ctr->bfs_work[nxt][0] = 0;
+        ctr->bfs_work[nxt][1] = 0;
         if (depth <= DBSPMSPV_MAX_BFS_LEVELS_RECORDED) {
-            ctr->bfs_level_path[depth - 1] = path;
-            ctr->bfs_level_nzblk[depth - 1] = n_nzblk;
+            ctr->bfs_level_nzblk[depth - 1] = now.n_blocks;
             ctr->bfs_stamp[depth] = global_timer_ns();
         }
     }
-    int4 *hubs_next = d.ws.hubs + nxt * HUB_CAP;
+    auto took = [&](int path) { if (sc.tid == 0 && depth <= DBSPMSPV_MAX_BFS_LEVELS_RECORDED) ctr->bfs_level_path[depth - 1] = path; };
+    auto next = [&]() {
+        grid.sync();
+        const int4 v = __ldcg(reinterpret_cast<const int4 *>(&ctr->bfs_set[nxt]));
+        now = Counters::BfsSet{v.x, v.y, v.z, v.w};
+    };
+    int path = bfs_level_path(d, now.n_blocks, 0, now.edges, th3, edge_frac, force_path);
+    if (path == DBSPMSPV_PATH_PUSH && now.n_verts <= BFS_LIST) {
+        int elems;
+        const int total = bfs_list_layout(d, d.ws.bfs_verts + q_in * BFS_LIST, now.n_verts, sh, elems);
+        path = bfs_level_path(d, now.n_blocks, 0, elems, th3, edge_frac, force_path);
+        if (path == DBSPMSPV_PATH_PUSH && elems <= BFS_MARK_STEPS * PUSH_CHUNK) {
+            took(path);
+            for (int i = sc.tid; i < z_words; i += sc.nthreads) Z[words_z[i]] = 0u;
+            bfs_push_list<DT>(d, total, sh, levels, depth, nx);
+            next();
+            return;
+        }
+    }
+    int n_tasks = 0, n_hubs = 0, steps = 0;
+    int4 *const hubs = d.ws.hubs + cur * HUB_CAP;
+    if (path == DBSPMSPV_PATH_PUSH) {
+        // (the level may still turn to a pull when the worklist is long)
+        bfs_worklist(d, sc, F, d.ws.bfs_words + (size_t)q_in * d.ws.bfs_words_stride, now.n_words, &ctr->bfs_work[cur][0], &ctr->bfs_work[cur][1], hubs, d.ws.tasks);
+        grid.sync();
+        n_tasks = __ldcg(&ctr->bfs_work[cur][0]);
+        n_hubs = min(__ldcg(&ctr->bfs_work[cur][1]), HUB_CAP);
+        steps = n_tasks;                                // the task records plus the steps of the listed hub runs
+        for (int k = 0; k < n_hubs; ++k) steps += (hubs[k].z + PUSH_CHUNK - 1) / PUSH_CHUNK;
+        path = bfs_level_path(d, now.n_blocks, steps, now.edges, th3, edge_frac, force_path);
+    }
+    took(path);
     if (path != DBSPMSPV_PATH_PUSH && d.rowrun_ptr != nullptr) {
         // a pull over the row-run index does its own bookkeeping (it owns the mask words it writes)
-        bfs_pull_rows<DT>(d, F, N, Z, &ctr->bfs_cnt[nxt][0], words_out, &ctr->bfs_nwords[q_out], levels, depth,
-                          (float)n_nzblk < BFS_WIDE_PULL * (float)d.nb, s_need + (threadIdx.x >> 5) * 32);
-        grid.sync();
-    } else if (path == DBSPMSPV_PATH_PUSH) {
+        bfs_pull_rows<DT>(d, F, Z, nx, levels, depth, (float)now.n_blocks < BFS_WIDE_PULL * (float)d.nb, s_need + (threadIdx.x >> 5) * 32);
+        next();
+        return;
+    }
+    const bool mark = path == DBSPMSPV_PATH_PUSH && steps <= BFS_MARK_STEPS;
+    if (path == DBSPMSPV_PATH_PUSH) {
         // Z (the frontier before this one) is cleared through its list
-        const int nz_words = ctr->bfs_nwords[q_z];
-        for (int i = sc.tid; i < nz_words; i += sc.nthreads) Z[words_z[i]] = 0u;
-        uint2 *const tasks = lv & 1 ? d.ws.tasks2 : d.ws.tasks, *const tasks_next = lv & 1 ? d.ws.tasks : d.ws.tasks2;
-        const bool mark = steps <= BFS_MARK_STEPS;
-        const bool emit = mark && n_hubs == 0 && n_tasks <= BFS_EMIT_STEPS && bfs_path(min(PUSH_CHUNK * n_tasks, d.nb), d.nb, th3, force_path) == DBSPMSPV_PATH_PUSH;
-        const bool counts = d.col_degree && words_per_warp(n_words, sc.nwarps) >= BFS_LARGE_WORDS;
-        const NextLevel nx{N, words_out, &ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][0], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], counts ? &ctr->bfs_edges[nxt] : nullptr, hubs_next, tasks_next, emit};
-        if (mark) bfs_push<DT, true>(d, sc, F, tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
-        else bfs_push<DT, false>(d, sc, F, tasks, n_tasks, d.ws.hubs + cur * HUB_CAP, n_hubs, levels, depth, nx);
-        grid.sync();
-        if (emit) return;                              // (the next level's worklist is there)
-        if (!mark) {
-            // levels, visited, the list of nonzero words and the counts: a warp takes its words, then writes the levels of one nonzero word after the other, lane = row
-            // (32 words each kept 684 of 4736 warps busy on 700 K vertices: a search with such a level 107 us, 104 with the words spread)
-            int found = 0, nz = 0, edges = 0;
-            const int W = words_per_warp(n_words, sc.nwarps);
-            for (int k0 = sc.gwarp * W; k0 < n_words; k0 += sc.nwarps * W) {
-                const int k = k0 + lane;
-                const uint32_t nm = lane < W && k < n_words ? __ldcg(N + k) : 0u;
-                if (nm) {
-                    d.ws.visited32[k] |= nm;
-                    found += __popc(nm);
-                    nz += ((nm & 0xFFFFu) != 0) + ((nm >> 16) != 0);
-                }
-                append_words(nm ? k : -1, words_out, &ctr->bfs_nwords[q_out], lane);
-                for (uint32_t todo = __ballot_sync(FULL, nm != 0u); todo; todo &= todo - 1) {
-                    const int q = __ffs(todo) - 1;
-                    if ((__shfl_sync(FULL, nm, q) >> lane) & 1u) {
-                        const size_t row = (size_t)(k0 + q) * 32 + lane;
-                        levels[row] = depth;
-                        if (counts) edges += (int)degree_of_code(d.col_degree[row]);
-                    }
+        for (int i = sc.tid; i < z_words; i += sc.nthreads) Z[words_z[i]] = 0u;
+        if (mark) bfs_push<DT, true>(d, sc, F, d.ws.tasks, n_tasks, hubs, n_hubs, levels, depth, nx);
+        else bfs_push<DT, false>(d, sc, F, d.ws.tasks, n_tasks, hubs, n_hubs, levels, depth, nx);
+    } else bfs_pull<DT>(d, sc, F, N, levels, depth);    // over the row-block segments (no row-run index)
+    if (mark) { next(); return; }
+    grid.sync();
+    // Levels, visited, the lists and the counts: a warp takes its words, then writes the levels of one nonzero word after the other, lane = row
+    // (32 words each kept 684 of 4736 warps busy on 700 K vertices: a search with such a level 107 us, 104 with the words spread).  (A pull over segments has written its levels, and left Z.)
+    const bool pulled = path != DBSPMSPV_PATH_PUSH;
+    int nz = 0, edges = 0;
+    const int W = words_per_warp(n_words, sc.nwarps);
+    for (int k0 = sc.gwarp * W; k0 < n_words; k0 += sc.nwarps * W) {
+        const int k = k0 + lane;
+        const bool in = lane < W && k < n_words;
+        const uint32_t nm = in ? __ldcg(N + k) : 0u;
+        if (nm) {
+            d.ws.visited32[k] |= nm;
+            nz += ((nm & 0xFFFFu) != 0) + ((nm >> 16) != 0);
+        }
+        if (pulled && in) Z[k] = 0u;
+        if (__any_sync(FULL, nm != 0u)) append_words(nx, k, nm, nm != 0u, lane);
+        if (!pulled)
+            for (uint32_t todo = __ballot_sync(FULL, nm != 0u); todo; todo &= todo - 1) {
+                const int q = __ffs(todo) - 1;
+                if ((__shfl_sync(FULL, nm, q) >> lane) & 1u) {
+                    const size_t row = (size_t)(k0 + q) * 32 + lane;
+                    levels[row] = depth;
+                    if (counts) edges += (int)degree_of_code(d.col_degree[row]);
                 }
             }
-            found = __reduce_add_sync(FULL, found);
-            nz = __reduce_add_sync(FULL, nz);
-            if (counts) edges = __reduce_add_sync(FULL, edges);
-            if (lane == 0 && found) { atomicAdd(&ctr->bfs_reached, found); atomicAdd(&ctr->bfs_cnt[nxt][0], nz); if (counts) atomicAdd(&ctr->bfs_edges[nxt], edges); }
-            grid.sync();
-        }
-    } else {
-        // pull over the row-block segments (no row-run index): the masks produced are scanned as a
-        // whole: visited is updated, the nonempty blocks counted, the nonzero words listed
-        bfs_pull<DT>(d, sc, F, N, levels, depth);
-        grid.sync();
-        int found = 0, nz = 0;
-        for (int k0 = sc.tid & ~31; k0 < n_words; k0 += sc.nthreads) {
-            const int k = k0 + lane;
-            uint32_t nm = 0;
-            if (k < n_words) {
-                nm = N[k];
-                if (nm) {
-                    d.ws.visited32[k] |= nm;
-                    found += __popc(nm);
-                    nz += ((nm & 0xFFFFu) != 0) + ((nm >> 16) != 0);
-                }
-                if (Z[k]) Z[k] = 0u;
-            }
-            append_words(nm ? k : -1, words_out, &ctr->bfs_nwords[q_out], lane);
-        }
-        found = __reduce_add_sync(FULL, found);
-        nz = __reduce_add_sync(FULL, nz);
-        if (lane == 0 && found) { atomicAdd(&ctr->bfs_reached, found); atomicAdd(&ctr->bfs_cnt[nxt][0], nz); }
-        grid.sync();
     }
-    // the push worklist is rebuilt if the block ratio of the next level asks for a push (the
-    // selector's input is known now; the level may still turn to a pull when the list is long)
-    const int next_n = ctr->bfs_cnt[nxt][0];
-    if (next_n && bfs_level_path(d, next_n, 0, ctr->bfs_edges[nxt], th3, edge_frac, force_path) == DBSPMSPV_PATH_PUSH) {
-        bfs_worklist(d, sc, N, words_out, ctr->bfs_nwords[q_out], &ctr->bfs_cnt[nxt][1], &ctr->bfs_hubs[nxt], hubs_next, lv & 1 ? d.ws.tasks : d.ws.tasks2);
-        grid.sync();
-    }
+    nz = __reduce_add_sync(FULL, nz);
+    if (counts) edges = __reduce_add_sync(FULL, edges);
+    if (lane == 0 && nz) { atomicAdd(&nx.set->n_blocks, nz); if (counts) atomicAdd(&nx.set->edges, edges); }
+    next();
 }
 
 template <int DT>
 __global__ void __launch_bounds__(BFS_CTA) k_bfs(Device d, int32_t src, int32_t *levels, float th3, float edge_frac,
                                                  int force_path, int max_levels) {
     __shared__ uint32_t s_need[BFS_CTA];                      // per warp: the wanted rows of its 32 words (transposed pull)
+    __shared__ BfsListShared s_list;
     cg::grid_group grid = cg::this_grid();
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int nthreads = gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31;
     const int n_words = (d.mb + 1) / 2;
     Counters *ctr = d.ws.ctr;
     const Scope sc{tid, nthreads, tid >> 5, nthreads >> 5};
@@ -767,25 +835,20 @@ __global__ void __launch_bounds__(BFS_CTA) k_bfs(Device d, int32_t src, int32_t 
         d.ws.visited32[k] = ~d.row_present32[k] | (mine ? src_bit : 0u);
         d.ws.x_mask32[k] = mine ? src_bit : 0u; d.ws.y_mask32[k] = 0u; d.ws.z_mask32[k] = 0u;
     }
-    if (blockIdx.x == 0 && threadIdx.x < 32) {
-        if (lane == 0) {
-            for (int k = 0; k < 3; ++k) { ctr->bfs_cnt[k][0] = 0; ctr->bfs_cnt[k][1] = 0; ctr->bfs_hubs[k] = 0; ctr->bfs_edges[k] = 0; }
-            for (int k = 0; k < 4; ++k) ctr->bfs_nwords[k] = k == 3;         // (the source's mask word is list 3 = "produced by level -1")
-            ctr->bfs_reached = 1;
-            d.ws.bfs_words[(size_t)3 * d.ws.bfs_words_stride] = src_word;
-        }
-        __syncwarp();
-        __threadfence();
-        const int jb = src >> 4;
-        int first = 0, deg = 0;
-        if (lane == 0) column_run(d, src, first, deg);
-        else if (lane == 1) payload_run(d, jb, first, deg);
-        emit_tasks(d, lane == 0, jb, first, deg, lane, &ctr->bfs_cnt[0][1], &ctr->bfs_cnt[0][0], PUSH_CHUNK, &ctr->bfs_hubs[0], d.ws.hubs);
+    if (tid == 0) {
+        for (int k = 0; k < 3; ++k) { ctr->bfs_set[k] = Counters::BfsSet{k == 0, k == 0, k == 0, 0}; ctr->bfs_work[k][0] = 0; ctr->bfs_work[k][1] = 0; }
+        d.ws.bfs_words[(size_t)3 * d.ws.bfs_words_stride] = src_word;        // (the source's lists are number 3 = "produced by level -1")
+        d.ws.bfs_verts[3 * BFS_LIST] = src;
     }
     grid.sync();
-    int lv = 0;
-    while (lv < max_levels && ctr->bfs_cnt[lv % 3][0] != 0) {
-        bfs_level<DT>(d, grid, sc, lv, levels, th3, edge_frac, force_path, s_need);    // ends with a grid barrier
+    int lv = 0, z_words = 0;
+    int64_t reached = 1;
+    Counters::BfsSet now{1, 1, 1, 0};
+    while (lv < max_levels && now.n_blocks != 0) {
+        const int f_words = now.n_words;
+        bfs_level<DT>(d, grid, sc, lv, now, z_words, levels, th3, edge_frac, force_path, s_need, s_list);    // ends with a grid barrier
+        z_words = f_words;
+        reached += now.n_verts;
         ++lv;
     }
     // leave the shared workspace as dbspmspv_run expects it: all masks clear.  The frontier before
@@ -795,13 +858,13 @@ __global__ void __launch_bounds__(BFS_CTA) k_bfs(Device d, int32_t src, int32_t 
         uint32_t *const buf[3] = {d.ws.x_mask32, d.ws.y_mask32, d.ws.z_mask32};
         uint32_t *Z = buf[(lv + 2) % 3], *F = buf[lv % 3];
         const int32_t *wz = d.ws.bfs_words + (size_t)((lv + 2) & 3) * d.ws.bfs_words_stride;
-        const int nz_words = ctr->bfs_nwords[(lv + 2) & 3];
-        for (int i = tid; i < nz_words; i += nthreads) Z[wz[i]] = 0u;
-        if (ctr->bfs_cnt[lv % 3][0] != 0)
+        for (int i = tid; i < z_words; i += nthreads) Z[wz[i]] = 0u;
+        if (now.n_blocks != 0)
             for (int k = tid; k < n_words; k += nthreads) F[k] = 0u;
     }
     if (tid == 0) {
         ctr->bfs_levels = lv;
+        ctr->bfs_reached = (int32_t)reached;
         if (lv < DBSPMSPV_MAX_BFS_LEVELS_RECORDED + 1) ctr->bfs_stamp[lv + 1] = global_timer_ns();
     }
 }

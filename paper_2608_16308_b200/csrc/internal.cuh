@@ -122,6 +122,7 @@ constexpr int PD_GROUPS_MIN_NNZ_X = 8192;
 // into tasks: it is listed once and every warp of the traversal strides over its 32-entry steps.
 constexpr int HUB_MIN_ENTRIES = 8192;
 constexpr int HUB_CAP = 32;
+constexpr int BFS_LIST = 1024;      // vertices of a frontier that is kept as a list too (db_bfs)
 // Stage of the single-kernel decode: payload bytes per chunk, at most (a chunk also has at
 // most 32 view entries: one per lane)
 #ifndef DBS_STAGE_BYTES
@@ -201,12 +202,13 @@ struct Counters {    // device-resident scalars of one call
     int32_t finish_ticket;  // k_finish: thread blocks started in this call, plus FINISH_PARITY in every other call
     int32_t n_long;         // direct push: chunks listed in this call
     int32_t n_hubs;         // hub runs of this call's push worklist (may exceed HUB_CAP: the rest became tasks)
-    int32_t bfs_hubs[3];    // BFS: the same per level (the per-level counters rotate three ways: the
-                            // level's own, the ones it accumulates for the next level, and a spare
-                            // set that is reset meanwhile)
-    int32_t bfs_nwords[4];  // BFS: lengths of the four rotating lists of nonzero mask words (Workspace::bfs_words)
-    int32_t bfs_cnt[3][2];  // BFS: {nonempty frontier blocks, tasks}
-    int32_t bfs_edges[3];   // BFS: elements of the frontier's columns, at least (counted by push levels)
+    // BFS: what a level leaves to the next one, in one 16-byte word.  Three rotate: the level's own, the one it accumulates for the next level, and a spare that is reset meanwhile.
+    struct alignas(16) BfsSet {
+        int32_t n_verts, n_words;   // vertices found; mask words that they lie in (lengths of Workspace::bfs_verts, bfs_words)
+        int32_t n_blocks;           // nonempty vector blocks
+        int32_t edges;              // elements of their columns, at least (counted by push levels)
+    } bfs_set[3];
+    int32_t bfs_work[3][2];     // BFS: the level's worklist, {tasks, hub runs}, likewise
     int32_t bfs_level_path[DBSPMSPV_MAX_BFS_LEVELS_RECORDED];
     int32_t bfs_level_nzblk[DBSPMSPV_MAX_BFS_LEVELS_RECORDED];
     // BFS: device time stamps (ns): [0] kernel start, [1 + L] start of level L, then the end of the last level
@@ -216,7 +218,6 @@ struct Counters {    // device-resident scalars of one call
 struct Workspace {
     float *x_dense;       // n (padded to a multiple of 32): dense copy of x (Section 3.2.2)
     uint32_t *x_mask32;   // vector-block masks, two 16-bit masks per word
-    uint2 *tasks2;        // BFS: a second worklist (a push level writes the next level's while it reads its own)
     uint2 *tasks;         // push worklist: (column block | (entries - 1) << 27, first CSC-view position)
     int4 *hubs;           // 3 x HUB_CAP hub runs (column block, first position, entries, -): see worklist.cuh
     float *y_acc;         // m (padded): dense accumulator, all ACC_CLEAR between calls
@@ -231,6 +232,7 @@ struct Workspace {
     int32_t *bfs_words;   // BFS: four lists of bfs_words_stride ints: the nonzero mask words of the frontiers produced by
                           // the levels L, L-1, L-2 (rotating, list L % 4 is written while level L runs)
     int32_t bfs_words_stride;
+    int32_t *bfs_verts;   // BFS: the first BFS_LIST vertices of those frontiers, likewise
     Counters *ctr;
     int64_t task_capacity;
     int32_t n_tiles;
@@ -416,6 +418,14 @@ __device__ __forceinline__ void chk_entry(const Device &d, bool csr_view, uint32
 // 16-bit load instead of a word load plus shift and mask (the GPU is little-endian).
 __device__ __forceinline__ uint32_t mask_of(const uint32_t *mask32, int blk) {
     return reinterpret_cast<const uint16_t *>(mask32)[blk];
+}
+
+// Global selector (Section 3.3.1): s_b = N_nzblk / N_blk; push iff s_b < th3.  Evaluated on
+// the device by every thread block from the counter the blocking kernel produced.
+__device__ __forceinline__ int select_path(const Device &d, float th3, int force_path) {
+    if (force_path == DBSPMSPV_PATH_PUSH || force_path == DBSPMSPV_PATH_PULL) return force_path;
+    const float sb = (float)d.ws.ctr->n_nzblk / (float)d.nb;
+    return sb < th3 ? DBSPMSPV_PATH_PUSH : DBSPMSPV_PATH_PULL;
 }
 
 // A count in eight bits, monotone: exact below 8, then three bits behind the leading one (the eighth below, at most, is cut off).

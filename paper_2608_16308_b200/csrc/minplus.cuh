@@ -159,7 +159,6 @@ __device__ __forceinline__ void block_rows_min_warp(int type, uint32_t w, uint32
 
 constexpr int MINPLUS_CTA = 256;
 
-__device__ __forceinline__ int select_path(const Device &d, float th3, int force_path);
 
 template <int DT>
 __global__ void __launch_bounds__(MINPLUS_CTA, 4) k_minplus_push(Device d, float th3, int force_path) {

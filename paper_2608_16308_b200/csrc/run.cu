@@ -12,7 +12,6 @@
 #include "mma_block.cuh"
 
 namespace dbs {
-__device__ __forceinline__ int select_path(const Device &d, float th3, int force_path);
 
 // ------------------------------------------------------------------------------------------
 // Output of a traversal.  The sparse path accumulates into the handle's dense accumulator (see
@@ -101,7 +100,6 @@ __global__ void k_xblock_sparse(Device d, const int32_t *__restrict__ x_idx, con
                      EMIT ? &d.ws.ctr->n_hubs : nullptr, d.ws.hubs);
 }
 
-__device__ __forceinline__ int select_path(const Device &d, float th3, int force_path);
 
 // Dense input (Sections 4.1, 4.3): every warp reads 32 elements, one ballot gives the two
 // 16-bit masks of its two vector blocks.  Also clears the dense output.
@@ -712,15 +710,6 @@ __device__ void pull_body(const Device &d, Out out, int popc_threshold, float *s
     // given back (bounded, like every wait here)
     if (next_in_flight) mbar_wait_bounded(&pw->bar[cur ^ 1], (parity >> (cur ^ 1)) & 1u);
 }
-
-// Global selector (Section 3.3.1): s_b = N_nzblk / N_blk; push iff s_b < th3.  Evaluated on
-// the device by every thread block from the counter the blocking kernel produced.
-__device__ __forceinline__ int select_path(const Device &d, float th3, int force_path) {
-    if (force_path == DBSPMSPV_PATH_PUSH || force_path == DBSPMSPV_PATH_PULL) return force_path;
-    const float sb = (float)d.ws.ctr->n_nzblk / (float)d.nb;
-    return sb < th3 ? DBSPMSPV_PATH_PUSH : DBSPMSPV_PATH_PULL;
-}
-
 #ifndef DBS_MIN_CTAS
 #define DBS_MIN_CTAS 1
 #endif
@@ -2169,7 +2158,7 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     const size_t zwords = xwords > ywords ? xwords : ywords;
     const size_t o_xd = carve(xwords * 32 * sizeof(float)), o_yacc = carve(ywords * 32 * sizeof(float)),
                  o_long = carve((size_t)d.long_cap * sizeof(*ws.long_runs)), o_tasks = carve((size_t)ws.task_capacity * sizeof(*ws.tasks)),
-                 o_tasks2 = carve((d.m == d.n ? (size_t)ws.task_capacity : 1) * sizeof(*ws.tasks)),
+                 o_verts = carve((d.m == d.n ? 4 * BFS_LIST : 1) * sizeof(*ws.bfs_verts)),
                  o_xm = carve(xwords * 4), o_ym = carve(ywords * 4), o_zm = carve(zwords * 4),
                  o_words = carve(4 * zwords * sizeof(*ws.bfs_words)), o_vis = carve((d.m == d.n ? ywords : 1) * 4),
                  o_hubs = carve((size_t)3 * HUB_CAP * sizeof(*ws.hubs)), o_tile = carve((size_t)ws.n_tiles * sizeof(*ws.tile_status)),
@@ -2183,7 +2172,7 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     ws.x_dense = reinterpret_cast<decltype(ws.x_dense)>(base + o_xd);
     ws.y_acc = reinterpret_cast<decltype(ws.y_acc)>(base + o_yacc);
     ws.long_runs = reinterpret_cast<decltype(ws.long_runs)>(base + o_long);
-    ws.tasks2 = reinterpret_cast<decltype(ws.tasks2)>(base + o_tasks2);
+    ws.bfs_verts = reinterpret_cast<decltype(ws.bfs_verts)>(base + o_verts);
     ws.tasks = reinterpret_cast<decltype(ws.tasks)>(base + o_tasks);
     ws.x_mask32 = reinterpret_cast<decltype(ws.x_mask32)>(base + o_xm);
     ws.y_mask32 = reinterpret_cast<decltype(ws.y_mask32)>(base + o_ym);

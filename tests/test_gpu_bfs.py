@@ -240,3 +240,47 @@ def test_levels_on_both_sides_of_the_large_graph_rule(delta):
             st = h.get_stats()
             assert st.bfs_reached == int((want >= 0).sum()) and st.bfs_levels == int(want.max()) + 1
     h.close()
+
+
+@pytest.mark.parametrize("fan", [1, 1023, 1024, 1025, 6000])
+def test_listed_and_unlisted_frontiers(fan):
+    """Frontiers at the length up to which they are kept as a list of vertices (1024), in turn with longer and shorter ones: the source reaches `fan` vertices, they reach a third of that
+    and one vertex whose column is long, then single vertices; dense blocks (with a payload) among the first ones; a part that is not reached keeps the levels a small share of the graph."""
+    n = 40011
+    rng = np.random.default_rng(fan)
+    a = 16 + np.arange(fan)
+    b = 8000 + np.arange(max(1, fan // 3))
+    u = [np.full(fan, 3), a, np.full(1, a[0]), np.full(700, 20000), [20001, 20002, 20003], np.repeat(np.arange(16, 48), 24), rng.integers(22000, n, 100000)]
+    v = [a, b[rng.integers(0, b.size, fan)], [20000], 20001 + np.arange(700), [21000, 21001, 21002], np.tile(np.arange(30000, 30024), 32), rng.integers(22000, n, 100000)]
+    keys = wl.sorted_unique(np.concatenate(v).astype(np.int64) * n + np.concatenate(u))
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    g = wl.CSR(n, n, ptr, idx, None)
+    h, A = Handle(g, B.PATTERN), ref_matrix(g)
+    for src in (3, 20000, int(a[-1])):
+        want = oracle.ref_bfs(A, src)
+        for path in PATHS:
+            h.set_opts(force_path=path)
+            assert np.array_equal(bfs(h, src), want)
+            st = h.get_stats()
+            assert st.bfs_reached == int((want >= 0).sum()) and st.bfs_levels == int(want.max()) + 1
+    h.close()
+
+
+@pytest.mark.parametrize("n", [170001, 178001])
+def test_short_frontier_of_many_elements(n):
+    """Three vertices that reach all others: 510,000 and 534,000 elements, on both sides of what a listed frontier is pushed from its list with (524,288)."""
+    hubs = np.array([5, 70000, n - 1])
+    u = np.r_[np.full(3, 9), np.repeat(hubs, n)]
+    v = np.r_[hubs, np.tile(np.arange(n), 3)]
+    keep = u != v
+    keys = wl.sorted_unique(v[keep].astype(np.int64) * n + u[keep])
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    g = wl.CSR(n, n, ptr, idx, None)
+    h, A = Handle(g, B.PATTERN), ref_matrix(g)
+    for src in (9, 70000):
+        want = oracle.ref_bfs(A, src)
+        for path in PATHS:
+            h.set_opts(force_path=path)
+            assert np.array_equal(bfs(h, src), want)
+            assert h.get_stats().bfs_reached == n
+    h.close()
