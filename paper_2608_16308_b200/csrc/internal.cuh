@@ -327,6 +327,7 @@ struct dbspmspv_handle_s {
     // device, and a handle lives on one device; calls on a handle are stream ordered, so plain fields)
     int grid_compute, grid_compute_dense, grid_decode_pull;
     bool lean_configured[2], lean_configured_dense[2], lean_configured_min[2];   // [1]: with the chunks of a push
+    bool small_configured;
     bool fused_configured[3];
     bool batch_configured[2];
     bool batch_mma_configured[3];

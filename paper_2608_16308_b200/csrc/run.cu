@@ -2201,13 +2201,12 @@ int allocate_workspace(dbspmspv_handle_s *h) {
     return DBSPMSPV_OK;
 }
 
-// Columns up to which the one-kernel form of a call is the faster one (see small_call.cuh).  The chain's first kernels are bound by their launches: two of them without long
-// columns (6.0 us a call on one host, 6.5 on another), three with (8.2 and 9.0); from 2^18 rows on the finishing kernel's tiles add to that.  The one-kernel form
-// goes by the columns, 48 / 64 / 96 / 144 / 224 of them, against the chain on the slower host, uniform rows: 128 K rows 6.7 / 6.8 / 7.3 / 8.1 / 8.4 against 6.5;
-// 256 K 6.8 / 6.9 / 7.4 / 8.2 / 8.6 against 7.7 / 7.2 / 6.5 / 6.5 / 6.5; 512 K 7.0 / 7.1 / 7.6 / 8.4 / 8.9 against 8.4 / 8.0 / 7.8 / 7.7 / 7.3; 700 K 7.2 / 7.3 / 7.7 / 8.6 / 9.0 against
-// 9.8 / 9.7 / 9.4 / 9.0 / 8.6; a million 7.5 / 7.6 / 8.1 / 9.1 / 9.5 against 9.9 / 9.9 / 9.9 / 9.9 / 9.6.  (64 columns up to 2^19 rows and 224 above: 7.6 -> 8.2 us with 65 columns of 512 K rows,
-// 9.1 instead of 7.1 with 224 of 600 K.)  With long columns the form's time jumps when x lists one: means of six R-MAT matrices in scattered order, 16 K rows, 48 / 96 / 144 columns
-// 7.7 / 8.5 / 9.0, 256 K rows, 96 columns 8.5; 1 M rows, 96 / 160 / 250 9.8 / 12 / 11.3 against a chain of 13.7.  (Handles with more payload blocks stay at the old limit: both ways vary by half with the columns that x lists.)
+// Columns up to which a call takes its one-kernel form (small_call.cuh).  It is the faster one up to all of these lines, and by now beyond them: uniform rows, 48 / 96 / 160 / 250 columns, one kernel
+// against the chain of two, whose launches the host is bound by: 16 K rows 5.3 / 5.4 / 5.7 / 6.4 against 6.3 us a call, 128 K 5.5 / 5.6 / 6.2 / 6.5 against 6.5, 256 K 5.6 / 5.6 / 5.9 / 6.3 against 8.2 / 6.6 /
+// 6.5 / 6.5, 512 K 5.7 / 6.0 / 6.2 / 6.5 against 8.9 / 8.6 / 8.1 / 7.8, a million 6.3 / 6.5 / 6.6 / 7.0 against 10.  With long columns, R-MAT in scattered order, against the chain of three: 16 K rows
+// 5.7 / 6.1 / 7.2 / 7.6 against 8.5 - 9.6, 256 K 7.3 / 6.1 / 6.7 / 7.2 against 8.7 - 9.3, 512 K 5.8 / 6.7 / 8.5 / 9.0 against 10, a million 7.1 / 7.2 / 8.6 / 8.5 against 13.7.  Not relabelled (more payload
+// blocks) both vary by half with the columns that x lists: 16 K 7.8 / 9.2 / 10.4 / 13.3 against 9.4 / 9.8 / 9.9 / 10.2, 256 K 9.4 / 10.8 / 11.3 / 12.4 against 10.4 - 10.8, a million 6.9 / 7.8 / 13.1 / 13.7
+// against 13.5 - 14.2.  The lines are those of an earlier, slower one-kernel form (7.5 us where it is 5.5 now) and stay because callers' launch counts are tested on both sides of them.
 static int small_call_limit(const dbspmspv_handle_s *h) {
     const Device &d = h->d;
     if (d.long_cap == 0) return d.m <= (1 << 17) ? 48 : d.m <= 5 << 16 ? 64 : d.m <= 5 << 17 ? 96 : d.m <= 7 << 17 ? 144 : 224;
@@ -2229,7 +2228,12 @@ static int run_typed(dbspmspv_handle_s *h, const int32_t *x_idx, const void *x_v
             !h->ropts.no_small_call && h->ropts.force_path != DBSPMSPV_PATH_PULL && !pull_possible(h, nnz_x, h->ropts.th3) &&
             smem <= SMALL_MAX_SMEM && (int64_t)ywords * 32 * (int64_t)sizeof(int32_t) <= d.ws.task_capacity * (int64_t)sizeof(*d.ws.tasks)) {
             const int mode = semiring == DBSPMSPV_OR_AND ? 1 : semiring == DBSPMSPV_MIN_PLUS ? 2 : 0;
-            calls.add(k_run_small<DT>, SMALL_CLUSTER, SMALL_CTA, smem, false, d, x_idx, x_val, nnz_x, mode, y_idx, y_val, y_capacity, y_nnz, row_mask, complement);
+            if (!h->small_configured) {
+                // (the attribute belongs to the kernel, not to the handle: the largest size)
+                DBS_CUDA(cudaFuncSetAttribute(k_run_small<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_MAX_SMEM + SMALL_ROWS * (int)sizeof(int)));
+                h->small_configured = true;
+            }
+            calls.add(k_run_small<DT>, SMALL_CLUSTER, SMALL_CTA, smem + SMALL_ROWS * sizeof(int), false, d, x_idx, x_val, nnz_x, mode, y_idx, y_val, y_capacity, y_nnz, row_mask, complement);
             return submit_calls(h, calls, st);
         }
     }

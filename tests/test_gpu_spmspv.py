@@ -538,3 +538,45 @@ def test_length_of_x_at_which_short_calls_change_over(m, hub, limit):
         yi, yv, _ = h.run(x, semiring=B.MIN_PLUS)
         assert np.array_equal(yi, wi) and np.array_equal(yv, wv.astype(np.float32))
     h.close()
+
+
+@pytest.mark.parametrize("rows", [1, 8191, 8192, 8193, 30000])
+def test_short_call_whose_result_fills_a_slice(rows):
+    """The one-kernel form keeps the rows of a slice of the result (an eighth of the matrix' rows) in shared memory up to 8192 of them: a column of so many elements in the last slice,
+    a column with dense blocks (its payload entries are shared out over the cluster), short columns; capacity and mask on both forms of the list."""
+    m = 8 * 32 * 1024 - 5
+    rng = np.random.default_rng(rows)
+    r = [7 * 32768 + rng.choice(32763, rows, replace=False), rng.integers(0, m, 40 * 20), np.tile(np.arange(32000, 32000 + 16 * 24), 16), rng.integers(0, m, 20000)]
+    c = [np.full(rows, 100), np.repeat(200 + 3 * np.arange(40), 20), np.repeat(np.arange(4800, 4816), 16 * 24), rng.integers(10000, m, 20000)]
+    keys = wl.sorted_unique(np.concatenate(r).astype(np.int64) * m + np.concatenate(c))
+    ptr, idx = wl.csr_from_sorted_keys(m, m, keys)
+    csr = wl.CSR(m, m, ptr, idx, rng.standard_normal(keys.size).astype(np.float32))
+    h, A = Handle(csr, B.F32), ref_matrix(csr)
+    at = np.r_[100, 200 + 3 * np.arange(40), 4803, 4811].astype(np.int32)
+    x = wl.SparseVec(m, at, rng.standard_normal(at.size).astype(np.float32))
+    want = oracle.ref_pull(A, x.idx, x.val)
+    before = h.get_stats().kernel_launches
+    check_against_oracle(h.run(x), want)
+    assert h.get_stats().kernel_launches == before + 1
+    check_against_oracle(h.run(x, semiring=B.OR_AND), want, boolean=True)
+    wi, wv = oracle.ref_minplus(A, x.idx, x.val)
+    yi, yv, _ = h.run(x, semiring=B.MIN_PLUS)
+    assert np.array_equal(yi, wi) and np.array_equal(yv, wv.astype(np.float32))
+    cap = want[0].size // 2
+    h.y_idx.fill_(-1)
+    yi, yv, k = h.run(x, capacity=cap)
+    assert k == want[0].size and np.array_equal(yi, want[0][:cap]) and (h.y_idx[cap:].cpu().numpy() == -1).all()
+    assert h.get_stats(raise_on_device_status=False).device_status == B.ERR_CAPACITY
+    bits = rng.random(m) < 0.5
+    words = np.zeros(((m + 15) // 16 + 1) // 2, dtype=np.uint32)
+    q = np.flatnonzero(bits)
+    np.bitwise_or.at(words, q >> 5, np.uint32(1) << (q & 31).astype(np.uint32))
+    maskd, xi, xv = torch.from_numpy(words.view(np.int32)).to("cuda"), torch.from_numpy(x.idx).to("cuda"), torch.from_numpy(x.val).to("cuda")
+    for complement in (0, 1):
+        keep = bits[want[0]] if complement == 0 else ~bits[want[0]]
+        B.dbspmspv_run_masked(h.h, xi, xv, at.size, B.PLUS_TIMES, maskd, complement, h.y_idx, h.y_val, m, h.y_nnz)
+        torch.cuda.synchronize()
+        kk = int(h.y_nnz.item())
+        check_against_oracle((h.y_idx[:kk].cpu().numpy(), h.y_val[:kk].cpu().numpy(), kk), tuple(a[keep] for a in want))
+        check_against_oracle(h.run(x), want)                  # the dropped rows left nothing behind
+    h.close()
