@@ -383,17 +383,29 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
         for (int p = tid; p < n_steps * 8; p += DCB_CTA) {
             const int s = p >> 3;
             if (!whole && (first <= last ? s < first || s > last : s < first && s > last)) continue;      // (a step this block does not visit)
+            // (the places behind the list hold column 0: fetched, and dropped)
             const uint32_t c2 = reinterpret_cast<const uint32_t *>(s_col)[p];
-            float v[NV][2];
+            uint32_t v[NV];
+            if (d.decode_x_f32) {
+                const float *xf = static_cast<const float *>(x);
+                float f[NV][2];
 #pragma unroll
-            for (int b = 0; b < NV; ++b) {
-                v[b][0] = v[b][1] = 0.f;
-                if (b < nvec && 2 * p < n) v[b][0] = dc_x(d, x, ldx, b, c2 & 0xFFFFu);
-                if (b < nvec && 2 * p + 1 < n) v[b][1] = dc_x(d, x, ldx, b, c2 >> 16);
+                for (int b = 0; b < NV; ++b) { const float *row = xf + (b < nvec ? b : 0) * ldx; f[b][0] = row[c2 & 0xFFFFu]; f[b][1] = row[c2 >> 16]; }
+#pragma unroll
+                for (int b = 0; b < NV; ++b)
+                    v[b] = (__float_as_uint(__bfloat162float(__float2bfloat16_rn(f[b][0]))) >> 16) | (__float_as_uint(__bfloat162float(__float2bfloat16_rn(f[b][1]))) & 0xFFFF0000u);
+            } else {
+                const uint16_t *xh = static_cast<const uint16_t *>(x);
+                uint16_t f[NV][2];
+#pragma unroll
+                for (int b = 0; b < NV; ++b) { const uint16_t *row = xh + (b < nvec ? b : 0) * ldx; f[b][0] = row[c2 & 0xFFFFu]; f[b][1] = row[c2 >> 16]; }
+#pragma unroll
+                for (int b = 0; b < NV; ++b) v[b] = (uint32_t)f[b][0] | (uint32_t)f[b][1] << 16;
             }
+            const uint32_t there = 2 * p + 1 < n ? 0xFFFFFFFFu : 2 * p < n ? 0xFFFFu : 0u;
 #pragma unroll
             for (int b = 0; b < NV; ++b) {
-                const uint32_t w = (__float_as_uint(v[b][0]) >> 16) | (__float_as_uint(v[b][1]) & 0xFFFF0000u);
+                const uint32_t w = b < nvec ? v[b] & there : 0u;
                 s_x[place(p, b)] = w & dc_pair_mask(test(w));
             }
         }
