@@ -310,10 +310,18 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
     }
     // (x may be read before the wait: the kernel in front zeroes y, and let this one start when everything before it had ended)
     // ---- x into shared memory: the entries that take part, by pairs of columns, and the union of the vectors' columns.
-    // A warp owns consecutive groups of eight columns; word (pair, vector) is rotated inside its row of 32 words so that neither the
-    // writes (32 pairs, one vector) nor the fragment reads (four pairs, NV vectors) meet in a bank.
+    // A warp owns consecutive groups of eight columns; the 16-byte pieces (pair, four vectors) are permuted inside their row of 32 words so that neither the
+    // writes (a piece each) nor the fragment reads (four pairs, NV vectors) meet in a bank.
     constexpr int PAIRS = 32 / NV;                                     // pairs per row
-    auto place = [&](int p, int b) { return p / PAIRS * 32 + (((p % PAIRS) * NV + b) ^ (p / PAIRS & 31)); };
+    auto place = [&](int p, int b) { return p / PAIRS * 32 + (((p % PAIRS) * NV + b) ^ ((p / PAIRS & 7) << 2)); };
+    auto store = [&](int p, const uint32_t (&w)[NV]) {
+#pragma unroll
+        for (int b = 0; b < NV; b += 4) *reinterpret_cast<uint4 *>(s_x + place(p, b)) = make_uint4(w[b], w[b + 1], w[b + 2], w[b + 3]);
+    };
+    // Without a cut every entry that is not zero takes part, and a zero may as well (the absent weights are zeros, too): nothing is masked.  (What bounded this phase is its instructions, five times as many
+    // with the general test and a word at a time: five layers in turn, eight vectors, 11008 x 4096, 30 % active 25.3 -> 23.5 us a call, 3000 x 3000, 5 / 50 % 14.3 / 15.4 -> 12.3 / 13.4, 1024 x 12288, 5 %
+    // 20.6 -> 15.0, 4096 x 11008, 30 % 32.1 -> 26.9; two vectors 20.3 -> 19.2, 8.8 / 11.9 -> 8.0 / 11.1, 12.6 -> 9.9, 24.0 -> 21.2)
+    const bool plain = d.decode_tau == 0.f && !d.decode_relu;
     bool odd = false;
     uint64_t bits = 0;
     const int groups = d.nb * 2, rounds = (groups + DCB_CTA - 1) / DCB_CTA, u0 = warp * rounds * 32 + lane;
@@ -331,16 +339,30 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
             }
             uint32_t any[4] = {0u, 0u, 0u, 0u}, strange = 0u;
 #pragma unroll
-            for (int b = 0; b < NV; ++b) {
-                const uint32_t w[4] = {h[b].x, h[b].y, h[b].z, h[b].w};
+            for (int k = 0; k < 4; ++k) {
+                uint32_t w[NV];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t m = test(w[k]);
-                    any[k] |= m;
-                    strange |= m & dc_odd(w[k]);
-                    if (u < groups) s_x[place(u * 4 + k, b)] = w[k] & dc_pair_mask(m);
+                for (int b = 0; b < NV; ++b) w[b] = k == 0 ? h[b].x : k == 1 ? h[b].y : k == 2 ? h[b].z : h[b].w;
+                if (plain) {
+#pragma unroll
+                    for (int b = 0; b < NV; ++b) {
+                        const uint32_t a = w[b] & 0x7FFF7FFFu;
+                        any[k] |= a + 0x7FFF7FFFu;                     // (bits 15 and 31)
+                        strange |= a + 0x00800080u;
+                    }
+                    any[k] &= 0x80008000u;
+                } else {
+#pragma unroll
+                    for (int b = 0; b < NV; ++b) {
+                        const uint32_t m = test(w[b]);
+                        any[k] |= m;
+                        strange |= m & dc_odd(w[b]);
+                        w[b] &= dc_pair_mask(m);
+                    }
                 }
+                if (u < groups) store(u * 4 + k, w);
             }
+            strange &= 0x80008000u;
             odd |= strange != 0u;
             uint32_t in = 0;
 #pragma unroll
@@ -405,9 +427,10 @@ k_decode_cols_batch(Device d, const void *__restrict__ x, int64_t ldx, float *__
             const uint32_t there = 2 * p + 1 < n ? 0xFFFFFFFFu : 2 * p < n ? 0xFFFFu : 0u;
 #pragma unroll
             for (int b = 0; b < NV; ++b) {
-                const uint32_t w = b < nvec ? v[b] & there : 0u;
-                s_x[place(p, b)] = w & dc_pair_mask(test(w));
+                v[b] = b < nvec ? v[b] & there : 0u;
+                if (!plain) v[b] &= dc_pair_mask(test(v[b]));
             }
+            store(p, v);
         }
         __syncthreads();
     }
