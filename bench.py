@@ -124,13 +124,13 @@ class ByteModel:
         whole --, cleared entry by entry or, for a long x, swept).  y: the accumulator's read-modify-write per result row, its
         4 bytes per row and the flag bit read by the finishing kernel, the rows that were hit put back, the sorted output.  (The
         private accumulators of hub rows, at most 256 KB, are not counted.)  one_kernel: the single-kernel form of a short call --
-        x is read once as a list, the row bitmap lives in shared memory, y is the accumulator read-modify-write, the row list
-        written and read back, the gather-and-clear and the output."""
+        x is read once as a list, the row bitmap and the row list live in shared memory, y is the accumulator read-modify-write,
+        the gather-and-clear and the output."""
         f = fmt if fmt is not None else self.format_bytes(x_idx, path)
         m, n, nx, active = self.csr.m, self.csr.n, x_idx.size, f["active_vector_blocks"]
         fmt_total = f["view_bytes"] + f["payload_bytes"] + f["pointer_bytes"]
         if one_kernel:
-            xbytes, ybytes = 8.0 * nx, 32.0 * y_nnz
+            xbytes, ybytes = 8.0 * nx, 24.0 * y_nnz
             return {"format": fmt_total, "x": xbytes, "y": ybytes, "accumulator_scan": 0.0, "total": fmt_total + xbytes + ybytes,
                     "traversal_kernel": fmt_total + xbytes + ybytes}
         if self.from_list(nx, path):
