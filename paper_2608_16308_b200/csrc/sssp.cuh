@@ -99,10 +99,10 @@ __device__ __forceinline__ void sssp_count(const SsspState &s, SsspSums &sums, i
     found = __reduce_add_sync(FULL, sums.found[lane]);
     low = __reduce_min_sync(FULL, sums.low[lane]);
     edges = __reduce_add_sync(FULL, sums.edges[lane]);
-    if (lane == 0 && found) {
-        atomicAdd(reinterpret_cast<unsigned long long *>(&s.set[set].edges), (unsigned long long)(unsigned)found << 32 | edges);
-        atomicMin(&s.set[set].low, low);
-    }
+    if (lane != 0) return;
+    // (a thread block may have lowered vertices further that all had been counted elsewhere: the smallest word can be one of theirs)
+    if (found) atomicAdd(reinterpret_cast<unsigned long long *>(&s.set[set].edges), (unsigned long long)(unsigned)found << 32 | edges);
+    if (low < 0x7F800000) atomicMin(&s.set[set].low, low);
 }
 __device__ __forceinline__ unsigned sssp_degree(const Device &d, int j) {
     if (d.col_degree) return degree_of_code(d.col_degree[j]);

@@ -175,3 +175,56 @@ def test_many_pulled_steps_in_a_row(length, base):
         assert np.array_equal(dist.cpu().numpy(), want)
     assert steps[0] == steps[1] == steps[2] and steps[0] > length
     h.close()
+
+
+def check_steps(csr, src, repeats=1):
+    """Distances and steps of the one launch against the oracle and the host loop's."""
+    h, A = Handle(csr, B.F32), ref_matrix(csr)
+    want = oracle.ref_sssp(A, src)
+    dist = torch.empty(csr.n, dtype=torch.float32, device="cuda")
+    steps = []
+    for path in [B.PATH_PUSH] + [B.PATH_AUTO] * repeats:
+        h.set_opts(force_path=path)
+        steps.append(B.db_sssp(h.h, src, dist))
+        torch.cuda.synchronize()
+        assert np.array_equal(dist.cpu().numpy().astype(np.float64), want)
+    assert len(set(steps)) == 1
+    h.close()
+
+
+def graph(n, edges):
+    """CSR of {(from, to): weight}, an edge each."""
+    u, v, w = (np.concatenate([np.broadcast_to(e[i], np.broadcast_shapes(*(np.shape(q) for q in e))).ravel() for e in edges]) for i in range(3))
+    keys, at = np.unique(v.astype(np.int64) * n + u.astype(np.int64), return_index=True)
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    return wl.CSR(n, n, ptr, idx, w[at].astype(np.float32))
+
+
+@pytest.mark.parametrize("n,mids", [(18001, 200), (18001, 700), (40011, 700), (170001, 200), (170001, 5000)])
+def test_smallest_distance_found_in_a_listed_chunk(n, mids):
+    """A pulled step that brings a row down twice: its first elements make it 150, and 61 comes from the end of the row, which is listed in chunks.  The second time the row
+    has been counted already, and 61 is all the same what the next pulled step's rows are cut by: row `r`, at 140, is improved by 61 + 30 and by nothing else."""
+    src, hub, r = 0, 33, 55
+    mid = 80 + 17 * np.arange(mids)
+    far = mid[-1] + 17 * (1 + np.arange(40))
+    light = np.where(np.arange(mids) == mids - 1, 1.0, 100.0)
+    last = np.where(np.arange(mids) == mids - 1, 60.0, 50.0)
+    check_steps(graph(n, [(src, mid, light), (mid, hub, last), (mid[:1], r, 40.0), (hub, r, 30.0), (hub, far, 5.0)]), src)
+
+
+@pytest.mark.parametrize("mids,early", [(600, 0), (2000, 0), (2000, 80)])
+def test_smallest_distance_of_a_pushed_step(mids, early):
+    """A pushed step whose frontier, spread over all thread blocks, reaches one vertex from everywhere: the first to lower it counts it, the others bring it further down, and the next step, a pulled one,
+    has rows that only the least of these distances improves.  From a listed frontier, from a bitmap, and with so many edges that nothing is listed (`early`: neighbours that were
+    reached for nothing, so that nothing else is found)."""
+    rng = np.random.default_rng(mids + early)
+    reach = 2000000 if early else 100000
+    src, hub, rows = 0, 33, 64 + 17 * np.arange(90)
+    mid = 2000 + 17 * rng.permutation(mids)
+    sinks = reach // 2 - 17 * (1 + np.arange(max(early, 1)))
+    out = np.arange(reach // 2, reach, 4)
+    edges = [(src, mid, 1.0), (mid, hub, 2.0 + np.arange(mids)), (src, rows, 5.0 + np.arange(90)), (hub, rows, 1.0), (hub, out, 7.0), (src, sinks, 0.0)]
+    if early:
+        edges.append((mid[:, None], sinks[None, :], 1.0))
+    noise = reach + rng.integers(0, reach, (2, reach))                                  # (not reached)
+    check_steps(graph(2 * reach, edges + [(noise[0], noise[1], 1.0)]), src, repeats=6)
