@@ -5,6 +5,7 @@
 // cooperative launch: levels are separated by grid-wide barriers (co-residency is guaranteed
 // by the cooperative launch), so there is no host round trip per level.
 #include <cooperative_groups.h>
+#include <cstddef>
 
 #include "internal.cuh"
 #include "microkernels.cuh"
@@ -76,6 +77,13 @@ __device__ __forceinline__ void append_found(const NextLevel &nx, int word, bool
 __device__ __forceinline__ void append_words(const NextLevel &nx, int word, uint32_t mask, bool new_word, int lane) {
     uint32_t left = mask;
     append_found(nx, word, new_word, __popc(mask), lane, [&](int, int place) { nx.verts[place] = word * 32 + __ffs(left) - 1; left &= left - 1; });
+}
+// What the lanes of a warp counted: vector blocks that became nonempty, and elements -- of vertices in other warps' blocks too -- in one atomic.
+__device__ __forceinline__ void add_counts(const NextLevel &nx, int blocks, int edges, int lane) {
+    static_assert(offsetof(Counters::BfsSet, edges) == offsetof(Counters::BfsSet, n_blocks) + 4 && offsetof(Counters::BfsSet, n_blocks) % 8 == 0, "one 8-byte word");
+    blocks = __reduce_add_sync(FULL, blocks);
+    if (nx.counts) edges = __reduce_add_sync(FULL, edges);
+    if (lane == 0 && (blocks | edges)) atomicAdd(reinterpret_cast<unsigned long long *>(&nx.set->n_blocks), (unsigned long long)(unsigned)edges << 32 | (unsigned)blocks);
 }
 // Up to this many warp steps the bookkeeping is the claiming lanes': a second atomic per vertex found, but neither a pass nor a barrier
 // behind the level.  Larger levels leave it to a pass over the words that became nonzero, one update for up to 32 vertices: levels of 2^22
@@ -205,10 +213,7 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
         // rotate the pipeline
         e0 = e1; e1 = e2; need0 = need1; t2 = t3;
     }
-    if (!MARK) return;
-    blocks = __reduce_add_sync(FULL, blocks);
-    if (nx.counts) edges = __reduce_add_sync(FULL, edges);
-    if (lane == 0 && blocks) { atomicAdd(&nx.set->n_blocks, blocks); if (nx.counts) atomicAdd(&nx.set->edges, edges); }
+    if (MARK) add_counts(nx, blocks, edges, lane);
 }
 
 // A short listed frontier, pushed without a worklist: every thread block lays the vertices' runs of INLINE elements and of the payload entries of their column blocks end to end in chunks, the
@@ -315,9 +320,7 @@ __device__ void bfs_push_list(const Device &d, int total, const BfsListShared &s
             if ((opened >> u) & 1u) nx.words[w++] = target[u] >> 5;
         }
     }
-    blocks = __reduce_add_sync(FULL, blocks);
-    if (nx.counts) edges = __reduce_add_sync(FULL, edges);
-    if (lane == 0 && blocks) { atomicAdd(&nx.set->n_blocks, blocks); if (nx.counts) atomicAdd(&nx.set->edges, edges); }
+    add_counts(nx, blocks, edges, lane);
 }
 
 // Boolean pull: one warp per row-block segment (a segment has at most MAX_SEG_ENTRIES = 4 x 32
@@ -793,9 +796,7 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
                 }
             }
     }
-    nz = __reduce_add_sync(FULL, nz);
-    if (counts) edges = __reduce_add_sync(FULL, edges);
-    if (lane == 0 && nz) { atomicAdd(&nx.set->n_blocks, nz); if (counts) atomicAdd(&nx.set->edges, edges); }
+    add_counts(nx, nz, edges, lane);
     next();
 }
 
