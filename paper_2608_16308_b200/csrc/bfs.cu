@@ -221,23 +221,23 @@ __device__ void bfs_push(const Device &d, const Scope &sc, const uint32_t *F, co
 // barrier behind it (a worklist is one more phase and barrier in front).  Every frontier of at most BFS_LIST vertices has its list, whichever way its level went.  Searches, symmetrised R-MAT, eight
 // sources each, with worklists / so, in brackets in scattered order: 16 K vertices 45.6 / 40.2 us (42.2 / 39.4), 65 K 54.7 / 48.2 (50.3 / 43.0), 262 K 53.4 / 42.8 (57.7 / 46.6), 2^20 75.3 / 61.6
 // (75.7 / 67.2), 2^22 138.8 / 130.2 (112.6 / 110.2); part of it are the counters of a level, one 16-byte load behind its last barrier in place of four to seven loads one after the other.
+// (Only the scan is kept: a chunk's warp fetches its vertex and the places of its runs once more, from L1.  With those in shared memory too, 25 KB in place of 4, the pull levels of large graphs, whose
+// gathers of frontier masks live in the L1 that this takes away, were longer: searches on 2 M uniform rows of eight 233 us, 225 so.)
 struct BfsListShared {
     int pre[BFS_LIST + 1];                            // chunks before a vertex
-    int vertex[BFS_LIST], first[BFS_LIST], deg[BFS_LIST], pfirst[BFS_LIST], pdeg[BFS_LIST];
     int sum[BFS_CTA / 32], elems[BFS_CTA / 32];
 };
 static_assert(BFS_LIST == BFS_CTA, "a thread per listed vertex");
 // Lays the chunks out; returns their number, and the elements behind them (the same in every thread).
 __device__ int bfs_list_layout(const Device &d, const int32_t *verts, int cnt, BfsListShared &sh, int &n_elems) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int j = 0, first = 0, deg = 0, pfirst = 0, pdeg = 0;
+    int first, deg = 0, pdeg = 0;
     if (tid < cnt) {
-        j = __ldcg(verts + tid);
+        int j = verts[tid];
         if (!DBS_CHK_INDEX(d, j, d.n)) j = 0;
         column_run(d, j, first, deg);
-        payload_run(d, j >> 4, pfirst, pdeg);
+        payload_run(d, j >> 4, first, pdeg);
     }
-    sh.vertex[tid] = j; sh.first[tid] = first; sh.deg[tid] = deg; sh.pfirst[tid] = pfirst; sh.pdeg[tid] = pdeg;
     const int mine = (deg + PD_CHUNK - 1) / PD_CHUNK + (pdeg + PD_PAYLOAD - 1) / PD_PAYLOAD;
     int incl = mine;
 #pragma unroll
@@ -253,7 +253,7 @@ __device__ int bfs_list_layout(const Device &d, const int32_t *verts, int cnt, B
     return total;
 }
 template <int DT>
-__device__ void bfs_push_list(const Device &d, int total, const BfsListShared &sh, int32_t *levels, int depth, const NextLevel &nx) {
+__device__ void bfs_push_list(const Device &d, const int32_t *verts, int total, const BfsListShared &sh, int32_t *levels, int depth, const NextLevel &nx) {
     constexpr int U = PD_CHUNK / 32;
     static_assert(PD_PAYLOAD / 2 == U, "one element per lane and step either way");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -263,7 +263,11 @@ __device__ void bfs_push_list(const Device &d, int total, const BfsListShared &s
         int o = 0;                                     // the last vertex with at most c chunks before it
 #pragma unroll
         for (int st = BFS_LIST / 2; st; st >>= 1) if (sh.pre[o + st] <= c) o += st;
-        const int k = c - sh.pre[o], n_inline = (sh.deg[o] + PD_CHUNK - 1) / PD_CHUNK;
+        int j = verts[o], first, deg, pfirst, pdeg;
+        if (!DBS_CHK_INDEX(d, j, d.n)) j = 0;
+        column_run(d, j, first, deg);
+        payload_run(d, j >> 4, pfirst, pdeg);
+        const int k = c - sh.pre[o], n_inline = (deg + PD_CHUNK - 1) / PD_CHUNK;
         int target[U];
         if (k < n_inline) {                            // warp-uniform
             const int at = k * PD_CHUNK + lane;
@@ -271,7 +275,7 @@ __device__ void bfs_push_list(const Device &d, int total, const BfsListShared &s
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 idx[u] = PAD_IDX; w[u] = 0u; aux[u] = 0u;
-                if (at + u * 32 < sh.deg[o]) push_entry<false>(d, sh.first[o] + at + u * 32, idx[u], w[u], aux[u]);
+                if (at + u * 32 < deg) push_entry<false>(d, first + at + u * 32, idx[u], w[u], aux[u]);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) target[u] = idx[u] < (1u << TYPE_SHIFT) ? (int)((idx[u] & IDX_MASK) * 16u + (aux[u] >> 4)) : -1;
@@ -280,7 +284,7 @@ __device__ void bfs_push_list(const Device &d, int total, const BfsListShared &s
             bool in[U];
             float value[U];
             uint32_t rb[U];
-            payload_elements<DBSPMSPV_PATTERN, U>(d, sh.pfirst[o] + at, min(PD_PAYLOAD, sh.pdeg[o] - at), sh.vertex[o] & 15, lane, in, value, rb);
+            payload_elements<DBSPMSPV_PATTERN, U>(d, pfirst + at, min(PD_PAYLOAD, pdeg - at), j & 15, lane, in, value, rb);
 #pragma unroll
             for (int u = 0; u < U; ++u) target[u] = in[u] ? (int)(rb[u] * 16u) + (lane & 15) : -1;
         }
@@ -692,6 +696,12 @@ __device__ __forceinline__ int bfs_level_path(const Device &d, int n_nzblk, int 
     return path;
 }
 
+// (a level uses one or the other; behind a layout that is given up nobody looks at it any more)
+union BfsShared {
+    uint32_t need[BFS_CTA];                           // per warp: the wanted rows of its 32 words (transposed pull)
+    BfsListShared list;
+};
+
 // One level of the search: the expansion of the frontier of level lv.  Three mask buffers rotate:
 // F holds the frontier, N receives the next one, Z (the frontier before) is cleared meanwhile and
 // becomes N of the next level.  Four lists of nonzero mask words and of vertices rotate with them -- the lists of
@@ -700,7 +710,7 @@ __device__ __forceinline__ int bfs_level_path(const Device &d, int n_nzblk, int 
 // z_words: mask words of Z.
 template <int DT>
 __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc, int lv, Counters::BfsSet &now, int z_words, int32_t *levels, float th3,
-                          float edge_frac, int force_path, uint32_t *s_need, BfsListShared &sh) {
+                          float edge_frac, int force_path, BfsShared &sh) {
     Counters *ctr = d.ws.ctr;
     const int lane = threadIdx.x & 31;
     const int n_words = (d.mb + 1) / 2;
@@ -733,12 +743,13 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
     int path = bfs_level_path(d, now.n_blocks, 0, now.edges, th3, edge_frac, force_path);
     if (path == DBSPMSPV_PATH_PUSH && now.n_verts <= BFS_LIST) {
         int elems;
-        const int total = bfs_list_layout(d, d.ws.bfs_verts + q_in * BFS_LIST, now.n_verts, sh, elems);
+        const int32_t *const verts = d.ws.bfs_verts + q_in * BFS_LIST;
+        const int total = bfs_list_layout(d, verts, now.n_verts, sh.list, elems);
         path = bfs_level_path(d, now.n_blocks, 0, elems, th3, edge_frac, force_path);
         if (path == DBSPMSPV_PATH_PUSH && elems <= BFS_MARK_STEPS * PUSH_CHUNK) {
             took(path);
             for (int i = sc.tid; i < z_words; i += sc.nthreads) Z[words_z[i]] = 0u;
-            bfs_push_list<DT>(d, total, sh, levels, depth, nx);
+            bfs_push_list<DT>(d, verts, total, sh.list, levels, depth, nx);
             next();
             return;
         }
@@ -758,7 +769,7 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
     took(path);
     if (path != DBSPMSPV_PATH_PUSH && d.rowrun_ptr != nullptr) {
         // a pull over the row-run index does its own bookkeeping (it owns the mask words it writes)
-        bfs_pull_rows<DT>(d, F, Z, nx, levels, depth, (float)now.n_blocks < BFS_WIDE_PULL * (float)d.nb, s_need + (threadIdx.x >> 5) * 32);
+        bfs_pull_rows<DT>(d, F, Z, nx, levels, depth, (float)now.n_blocks < BFS_WIDE_PULL * (float)d.nb, sh.need + (threadIdx.x >> 5) * 32);
         next();
         return;
     }
@@ -803,8 +814,7 @@ __device__ void bfs_level(const Device &d, cg::grid_group &grid, const Scope &sc
 template <int DT>
 __global__ void __launch_bounds__(BFS_CTA) k_bfs(Device d, int32_t src, int32_t *levels, float th3, float edge_frac,
                                                  int force_path, int max_levels) {
-    __shared__ uint32_t s_need[BFS_CTA];                      // per warp: the wanted rows of its 32 words (transposed pull)
-    __shared__ BfsListShared s_list;
+    __shared__ BfsShared sh;
     cg::grid_group grid = cg::this_grid();
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int nthreads = gridDim.x * blockDim.x;
@@ -847,7 +857,7 @@ __global__ void __launch_bounds__(BFS_CTA) k_bfs(Device d, int32_t src, int32_t 
     Counters::BfsSet now{1, 1, 1, 0};
     while (lv < max_levels && now.n_blocks != 0) {
         const int f_words = now.n_words;
-        bfs_level<DT>(d, grid, sc, lv, now, z_words, levels, th3, edge_frac, force_path, s_need, s_list);    // ends with a grid barrier
+        bfs_level<DT>(d, grid, sc, lv, now, z_words, levels, th3, edge_frac, force_path, sh);    // ends with a grid barrier
         z_words = f_words;
         reached += now.n_verts;
         ++lv;
