@@ -494,17 +494,19 @@ __device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *Z, c
             while (todo) {
                 const int k = __ffs(todo) - 1;
                 todo &= todo - 1;
+                // (Up to 16 entries a row block: a half-warp for each of the two, one chain of loads per word; more: the whole warp for one after the other.  Searches on 27-point operators, 100^3 / 150^3 cells,
+                // the row blocks one after the other 1535 / 7130 us, so 1420 / 6530; half-warps whatever the length: 1 % less there, R-MAT of 700 K vertices, whose hub row blocks have hundreds, 81 -> 87.)
                 const uint32_t need_k = __shfl_sync(FULL, need, k);
+                const int beg0 = __shfl_sync(FULL, pb0, k), end0 = __shfl_sync(FULL, pe0, k), beg1 = __shfl_sync(FULL, pb1, k), end1 = __shfl_sync(FULL, pe1, k);
                 uint32_t fk = 0u;
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                    const uint32_t need16 = (need_k >> (16 * hf)) & 0xFFFFu;
-                    const int pbeg = __shfl_sync(FULL, hf ? pb1 : pb0, k), pend = __shfl_sync(FULL, hf ? pe1 : pe0, k);
-                    if (!need16 || pend <= pbeg) continue;        // warp-uniform
-                    uint32_t hit = 0;
-                    for (int base = pbeg; base < pend; base += 32) {
-                        const int pos = base + lane;
-                        if (pos < pend) {
+                const int step = max(end0 - beg0, end1 - beg1) <= 16 ? 16 : 32;
+#pragma unroll 1
+                for (int part = step & 16 ? lane & 16 : 0; ; part += 16) {
+                    const uint32_t need_part = need_k & (0xFFFFu << part);
+                    const int pend = part ? end1 : end0;
+                    for (int pos = (part ? beg1 : beg0) + (lane & (step - 1)); __any_sync(FULL, pos < pend && (need_part & ~fk)); pos += step) {      // (until every wanted row has a parent)
+                        uint32_t hit = 0;
+                        if (pos < pend && (need_part & ~fk)) {
                             uint32_t idx = d.csr.idx[pos], aux = d.csr.aux[pos];
 #ifdef DBS_BOUNDS_CHECK
                             { uint32_t w_ = d.csr.w[pos]; DBS_CHK_ENTRY(d, true, idx, w_, aux); }
@@ -513,14 +515,13 @@ __device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *Z, c
                             if (xm) {
                                 const int type = idx >> TYPE_SHIFT;
                                 const uint32_t w = d.csr.w[pos];
-                                hit |= type == DBSPMSPV_BLK_COO ? lane_block_bool<DT>(type, w, aux, xm, d.payload)
-                                                                : lane_heavy_bool(type, d.payload + (size_t)w * 4, xm);
+                                hit = type == DBSPMSPV_BLK_COO ? lane_block_bool<DT>(type, w, aux, xm, d.payload)
+                                                               : lane_heavy_bool(type, d.payload + (size_t)w * 4, xm);
                             }
                         }
-                        hit = __reduce_or_sync(FULL, hit);
-                        if ((hit & need16) == need16) break;      // every wanted row of the block has a parent
+                        fk |= __reduce_or_sync(FULL, hit << part) & need_k;
                     }
-                    fk |= (hit & need16) << (16 * hf);
+                    if (step == 16 || part) break;
                 }
                 if ((fk >> lane) & 1u) levels[(size_t)(w0 + k) * 32 + lane] = depth;
                 if (lane == k) found |= fk;
@@ -587,11 +588,28 @@ __device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *Z, c
                 rounds = 0;
                 fetch_next();
             }
-            if (active) {
-                // a round = the aligned group(s) of four entries from position p on: 16-byte loads
+            // (one form with the second group's loads left out: 150^3 cells 7400 us, 8 M uniform rows of four 866; a form each 6530 and 823)
+            if (active && !wide) {
+                // a round = the aligned group of four entries from position p on: one 16-byte load
+                const int q0 = p & ~3;
+                const uint4 v4 = __ldcs(reinterpret_cast<const uint4 *>(d.rowrun_idx + q0));       // (the array has slack behind its end)
+                uint32_t v[4] = {v4.x, v4.y, v4.z, v4.w}, xm[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) if (q0 + j < p || q0 + j >= e || (v[j] != NONE && !DBS_CHK_INDEX(d, v[j] & IDX_MASK, d.nb))) v[j] = NONE;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) xm[j] = v[j] != NONE ? mask_of(F, v[j] & IDX_MASK) : 0u;
+                bool got = false;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) got |= ((xm[j] >> (v[j] >> 27)) & 1u) != 0;
+                p = q0 + 4;
+                if (got) { res |= 1u << k; levels[(size_t)(w0 + k) * 32 + ((lane + k) & 31)] = depth; active = false; }
+                else if (p >= e) active = false;
+                else if (++rounds == MAX_ROUNDS) { longm |= 1u << k; active = false; }     // a long row: finished by the whole warp below
+            } else if (active) {
+                // under a small frontier, two groups a round
                 const int q0 = p & ~3;
                 uint4 v4 = __ldcs(reinterpret_cast<const uint4 *>(d.rowrun_idx + q0)), w4 = make_uint4(NONE, NONE, NONE, NONE);   // (the array has slack behind its end)
-                if (wide && q0 + 4 < e) w4 = __ldcs(reinterpret_cast<const uint4 *>(d.rowrun_idx + q0 + 4));
+                if (q0 + 4 < e) w4 = __ldcs(reinterpret_cast<const uint4 *>(d.rowrun_idx + q0 + 4));
                 uint32_t v[8] = {v4.x, v4.y, v4.z, v4.w, w4.x, w4.y, w4.z, w4.w}, xm[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) if (q0 + j < p || q0 + j >= e || (v[j] != NONE && !DBS_CHK_INDEX(d, v[j] & IDX_MASK, d.nb))) v[j] = NONE;
@@ -600,7 +618,7 @@ __device__ void bfs_pull_rows(const Device &d, const uint32_t *F, uint32_t *Z, c
                 bool got = false;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) got |= ((xm[j] >> (v[j] >> 27)) & 1u) != 0;
-                p = q0 + per_round;
+                p = q0 + 8;
                 if (got) { res |= 1u << k; levels[(size_t)(w0 + k) * 32 + ((lane + k) & 31)] = depth; active = false; }
                 else if (p >= e) active = false;
                 else if (++rounds == MAX_ROUNDS) { longm |= 1u << k; active = false; }     // a long row: finished by the whole warp below

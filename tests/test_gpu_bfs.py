@@ -284,3 +284,33 @@ def test_short_frontier_of_many_elements(n):
             assert np.array_equal(bfs(h, src), want)
             assert h.get_stats().bfs_reached == n
     h.close()
+
+
+def test_pulled_row_blocks_by_their_entries_with_a_payload():
+    """A pulled level takes the two row blocks of a mask word side by side while both have at most 16 entries with a payload: every pair of counts around that and around a warp's 32.  (These rows have
+    no other parents; a dense block has 40 elements, and one row without any.)"""
+    counts = [0, 1, 15, 16, 17, 32, 33, 65]
+    pairs = [(a, b) for a in counts for b in counts]
+    n = 60000 + 5
+    rng = np.random.default_rng(5)
+    rows, cols = [], []
+    for w, pair in enumerate(pairs):
+        for half, count in enumerate(pair):
+            for cb in np.sort(rng.choice(np.arange(400, 2400), count, replace=False)):          # dense blocks, one row of each left out
+                r, c = np.divmod(np.setdiff1d(np.arange(256), 16 * (cb % 16) + np.arange(16))[rng.choice(240, 40, replace=False)], 16)
+                rows.append(16 * (2 * w + half) + r)
+                cols.append(16 * cb + c)
+    rows += [rng.integers(2048, n, 300000), 40000 + np.arange(300)]
+    cols += [40000 + rng.integers(0, n - 40000, 300000), np.full(300, 7)]
+    keys = wl.sorted_unique(np.concatenate(rows).astype(np.int64) * n + np.concatenate(cols))
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    g = wl.CSR(n, n, ptr, idx, None)
+    h, A = Handle(g, B.PATTERN), ref_matrix(g)
+    st = h.get_stats()
+    assert st.bfs_index_bytes > 0 and sum(st.class_blocks[2:]) == sum(a + b for a, b in pairs)
+    for src in (7, 16 * 400 + 3, 40007, n - 1):
+        want = oracle.ref_bfs(A, src)
+        for path in PATHS:
+            h.set_opts(force_path=path)
+            assert np.array_equal(bfs(h, src), want)
+    h.close()
