@@ -64,7 +64,7 @@ struct SsspState {
     int *word[2];             // distances (ordered words): a step reads them from one array, which nobody writes meanwhile, and lowers them in the other
     uint32_t *bits[3];        // frontiers, one bit per vertex: the step's, the one it marks, the one before (being cleared), in turn
     SsspSet *set;             // three of them, in turn
-    int32_t *ctr;             // [0] steps made, [1] array of the distances, [2..4] places taken in the step's list
+    int32_t *ctr;             // [0] steps made, [1] array of the distances, [2..4] places taken in the step's list, [5] a step has been pulled
     int4 *chunks;             // {row, first, end, -} of the listed chunks of long rows
     int32_t *list[2];         // the vertices marked by alternating steps, SSSP_LIST at most
     int32_t *report;          // page-locked host words: steps made, vertices of the frontier that was left
@@ -773,7 +773,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
         if (tid == 0) {
             int first, deg;
             column_run(d, src, first, deg);
-            for (int k = 0; k < 5; ++k) s.ctr[k] = 0;
+            for (int k = 0; k < 6; ++k) s.ctr[k] = 0;
             for (int k = 0; k < 3; ++k) s.set[k] = SsspSet{k == 0 ? (unsigned)deg : 0u, k == 0 ? 1u : 0u, k == 0 ? 0 : 0x7F800000, 0};
             s.list[1][0] = src;
         }
@@ -784,7 +784,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
         return SsspSet{(unsigned)v.x, (unsigned)v.y, v.z, v.w};
     };
     int t = __ldcg(s.ctr), c = __ldcg(s.ctr + 1);      // array c holds the distances; so does the other one, but for the frontier, of which it has larger ones
-    bool late = false;                                 // a step has been pulled
+    bool late = __ldcg(s.ctr + 5) != 0;                // a step has been pulled, in this launch or one before
     bool lists = start != 0;                           // the step before listed what it marked, in list[(t + 1) & 1]
     SsspSet now = read(t % 3);                         // grid-uniform, as all that is decided from it
     for (int made = 0; made < max_steps && now.found; ++made, ++t, c ^= 1) {
@@ -820,7 +820,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
     // the distances themselves
     for (int64_t v = tid; v < d.n; v += nthreads) dist_out[v] = sssp_value(__ldcg(s.word[c] + v));
     // (everyone read the counters before the first barrier, or leaves without a step)
-    if (tid == 0) { s.ctr[0] = t; s.ctr[1] = c; s.report[0] = t; s.report[1] = (int)now.found; }
+    if (tid == 0) { s.ctr[0] = t; s.ctr[1] = c; s.ctr[5] = late; s.report[0] = t; s.report[1] = (int)now.found; }
 }
 
 }  // namespace dbs
