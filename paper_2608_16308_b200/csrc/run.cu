@@ -2616,12 +2616,17 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     for (int k = 0; k < 2; ++k) { s.list[k] = reinterpret_cast<int32_t *>(p); p += SSSP_LIST * sizeof(int32_t); }
     s.chunks = reinterpret_cast<int4 *>(p);
     s.report = h->sssp_host;
+    // edges from which a step is pulled, the first one and those behind it (sssp.cuh)
+    const bool weights = DT != DBSPMSPV_PATTERN;
+    const float rows = (float)d.n, pull = weights && h->payload_rich ? SSSP_PULL_SHARE_PAYLOAD : SSSP_PULL_SHARE;
+    float late = SSSP_LATE_SHARE * (float)d.n_entries;
+    if (weights) late = fmaxf(late, rows * fminf(SSSP_LATE_ROWS * (rows / (1 << 20)) * (rows / (1 << 20)), 1.0f));
     Device dev = d;
     int start = 1;
     for (int64_t made = 0;; start = 0) {
         int max_steps = (int)(d.n + 1 - made < SSSP_MAX_STEPS ? d.n + 1 - made : SSSP_MAX_STEPS);
         const bool can_pull = DT == DBSPMSPV_PATTERN ? d.rowrun_ptr != nullptr : d.weightrun != nullptr && d.col_degree != nullptr;
-        unsigned pull_edges = can_pull ? (unsigned)(SSSP_PULL_SHARE * (float)d.n_entries) : ~0u, late_edges = can_pull ? (unsigned)(SSSP_LATE_SHARE * (float)d.n_entries) : ~0u;
+        unsigned pull_edges = can_pull ? (unsigned)(pull * (float)d.n_entries) : ~0u, late_edges = can_pull ? (unsigned)fminf(late, pull * (float)d.n_entries) : ~0u;
         void *args[] = {&dev, &s, &src, &dist, &start, &max_steps, &pull_edges, &late_edges};
         DBS_CUDA(cudaLaunchCooperativeKernel((void *)k_sssp<DT>, dim3(h->sm_count), dim3(SSSP_CTA), args, SSSP_SMEM, st));
         ++h->kernel_launches;

@@ -228,3 +228,21 @@ def test_smallest_distance_of_a_pushed_step(mids, early):
         edges.append((mid[:, None], sinks[None, :], 1.0))
     noise = reach + rng.integers(0, reach, (2, reach))                                  # (not reached)
     check_steps(graph(2 * reach, edges + [(noise[0], noise[1], 1.0)]), src, repeats=6)
+
+
+def test_pulled_steps_of_a_handle_with_many_payload_blocks():
+    """A 27-point operator on 21^3 cells, a good part of its elements in blocks with a payload: its steps are pulled from a smaller share of the elements on; noise beside it, not reached, leaves its larger steps
+    on both sides of that share."""
+    d, far = 21, 21 ** 3
+    g, rng = wl.stencil27(d, seed=3), np.random.default_rng(3)
+    n = 2 * far
+    cells = g.rows(), g.col_idx
+    edges = [(cells[1], cells[0], (1 + rng.integers(0, 63, g.nnz)) / 8.0)]
+    noise = far + rng.integers(0, far, (2, 250000))
+    csr = graph(n, edges + [(noise[0], noise[1], 1.0)])
+    h = Handle(csr, B.F32)
+    st = h.get_stats()
+    assert csr.nnz < 8 * sum(st.class_nnz[1:]) and 2 * sum(st.class_nnz[2:]) < csr.nnz
+    h.close()
+    for src in (0, d // 2 * (1 + d + d * d)):
+        check_steps(csr, src, repeats=2)
