@@ -60,6 +60,7 @@ constexpr int SSSP_CHUNK = 512;                   // elements of a listed chunk 
 // (The bitmap of 2^20 vertices is two rounds of every thread block, whatever it holds: a step of a few vertices took 14 us, 26 with a long run.)
 constexpr int SSSP_LIST = SSSP_CTA;
 constexpr unsigned SSSP_LIST_EDGES = 1u << 17;
+constexpr int SSSP_STARTS = 1, SSSP_GOES_ON = 0, SSSP_GOES_ON_LATE = 2;      // a launch: the first of its search, or one behind it (a step has been pulled before)
 constexpr int SSSP_MAX_STEPS = 1024;              // steps of one launch, at most: a cycle of negative weight ends on the host
 
 // What a step leaves to the next one, in one 16-byte word: a barrier is followed by one trip to L2.
@@ -72,10 +73,10 @@ struct SsspState {
     int *word[2];             // distances (ordered words): a step reads them from one array, which nobody writes meanwhile, and lowers them in the other
     uint32_t *bits[3];        // frontiers, one bit per vertex: the step's, the one it marks, the one before (being cleared), in turn
     SsspSet *set;             // three of them, in turn
-    int32_t *ctr;             // [0] steps made, [1] array of the distances, [2..4] places taken in the step's list, [5] a step has been pulled
+    int32_t *ctr;             // [0] steps made, [1] array of the distances, [2..4] places taken in the step's list
     int4 *chunks;             // {row, first, end, -} of the listed chunks of long rows
     int32_t *list[2];         // the vertices marked by alternating steps, SSSP_LIST at most
-    int32_t *report;          // page-locked host words: steps made, vertices of the frontier that was left
+    int32_t *report;          // page-locked host words: steps made, vertices of the frontier that was left, whether a step has been pulled
     int32_t n_words;
 };
 
@@ -774,14 +775,14 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
     SsspShared &sh = *reinterpret_cast<SsspShared *>(s_dyn);
     cg::grid_group grid = cg::this_grid();
     const int tid = blockIdx.x * SSSP_CTA + threadIdx.x, nthreads = gridDim.x * SSSP_CTA;
-    if (start) {                                       // (a later launch of the same search continues where the one before stopped)
+    if (start == SSSP_STARTS) {                                       // (a later launch of the same search continues where the one before stopped)
         const int64_t n = (int64_t)s.n_words * 32;
         for (int64_t v = tid; v < n; v += nthreads) s.word[0][v] = s.word[1][v] = v == src ? 0 : 0x7F800000;
         for (int k = tid; k < s.n_words; k += nthreads) { s.bits[0][k] = k == src >> 5 ? 1u << (src & 31) : 0u; s.bits[1][k] = 0u; }       // (the third is cleared by the first step)
         if (tid == 0) {
             int first, deg;
             column_run(d, src, first, deg);
-            for (int k = 0; k < 6; ++k) s.ctr[k] = 0;
+            for (int k = 0; k < 5; ++k) s.ctr[k] = 0;
             for (int k = 0; k < 3; ++k) s.set[k] = SsspSet{k == 0 ? (unsigned)deg : 0u, k == 0 ? 1u : 0u, k == 0 ? 0 : 0x7F800000, 0};
             s.list[1][0] = src;
         }
@@ -792,8 +793,8 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
         return SsspSet{(unsigned)v.x, (unsigned)v.y, v.z, v.w};
     };
     int t = __ldcg(s.ctr), c = __ldcg(s.ctr + 1);      // array c holds the distances; so does the other one, but for the frontier, of which it has larger ones
-    bool late = __ldcg(s.ctr + 5) != 0;                // a step has been pulled, in this launch or one before
-    bool lists = start != 0;                           // the step before listed what it marked, in list[(t + 1) & 1]
+    bool late = start == SSSP_GOES_ON_LATE;            // a step has been pulled, in this launch or one before
+    bool lists = start == SSSP_STARTS;                 // the step before listed what it marked, in list[(t + 1) & 1]
     SsspSet now = read(t % 3);                         // grid-uniform, as all that is decided from it
     for (int made = 0; made < max_steps && now.found; ++made, ++t, c ^= 1) {
         const uint32_t *F = s.bits[t % 3];
@@ -828,7 +829,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
     // the distances themselves
     for (int64_t v = tid; v < d.n; v += nthreads) dist_out[v] = sssp_value(__ldcg(s.word[c] + v));
     // (everyone read the counters before the first barrier, or leaves without a step)
-    if (tid == 0) { s.ctr[0] = t; s.ctr[1] = c; s.ctr[5] = late; s.report[0] = t; s.report[1] = (int)now.found; }
+    if (tid == 0) { s.ctr[0] = t; s.ctr[1] = c; s.report[0] = t; s.report[1] = (int)now.found; s.report[2] = late; }
 }
 
 }  // namespace dbs
