@@ -16,10 +16,7 @@ namespace cg = cooperative_groups;
 
 namespace dbs {
 
-#ifndef DBS_BFS_CTA
-#define DBS_BFS_CTA 1024   // one thread block per SM: a grid barrier over 148 blocks costs far less than over a thousand
-#endif
-constexpr int BFS_CTA = DBS_BFS_CTA;
+constexpr int BFS_CTA = BFS_LIST;   // one thread block per SM (a grid barrier over 148 blocks costs far less than over a thousand), a thread per listed vertex
 
 // Rows of one hypersparse block reached from the active columns (one lane per block).
 template <int DT>
@@ -227,7 +224,6 @@ struct BfsListShared {
     int pre[BFS_LIST + 1];                            // chunks before a vertex
     int sum[BFS_CTA / 32], elems[BFS_CTA / 32];
 };
-static_assert(BFS_LIST == BFS_CTA, "a thread per listed vertex");
 // Lays the chunks out; returns their number, and the elements behind them (the same in every thread).
 __device__ int bfs_list_layout(const Device &d, const int32_t *verts, int cnt, BfsListShared &sh, int &n_elems) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
