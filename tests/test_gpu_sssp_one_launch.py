@@ -246,3 +246,42 @@ def test_pulled_steps_of_a_handle_with_many_payload_blocks():
     h.close()
     for src in (0, d // 2 * (1 + d + d * d)):
         check_steps(csr, src, repeats=2)
+
+
+@pytest.mark.parametrize("layers,width", [(60, 64), (200, 64), (200, 80)])
+def test_many_pulled_steps_of_unit_weights(layers, width):
+    """Layers of vertices one behind the other, linked by INLINE elements and by one dense block each, behind a source whose column holds a seventh of the elements: its step is pulled, and so are
+    those of the layers, a row's word lowered by its INLINE elements and by the dense block's warp.  (Unit weights: a handle without values.)"""
+    rng = np.random.default_rng(layers + width)
+    src, first = 0, 48
+    u, v = [], []
+    for k in range(layers - 1):
+        at, per = first + k * width, width // 16
+        dense = int(rng.integers(per * per))
+        for b in range(per * per):
+            r, c = np.divmod(rng.choice(256, 40 if b == dense else 7, replace=False), 16)
+            u.append(at + 16 * (b % per) + c)
+            v.append(at + width + 16 * (b // per) + r)
+    u, v = np.concatenate(u), np.concatenate(v)
+    hub = u.size // 6
+    far = first + layers * width
+    n = far + hub + 5
+    u = np.r_[u, np.zeros(width + hub, np.int64)]
+    v = np.r_[v, first + np.arange(width), far + np.arange(hub)]
+    keys = wl.sorted_unique(v.astype(np.int64) * n + u)
+    ptr, idx = wl.csr_from_sorted_keys(n, n, keys)
+    csr = wl.CSR(n, n, ptr, idx, np.ones(keys.size, np.float32))
+    h, A = Handle(csr, B.PATTERN), ref_matrix(csr)
+    st = h.get_stats()
+    assert sum(st.class_blocks[2:]) == layers - 1 and 2 * sum(st.class_nnz[2:]) < csr.nnz < 10 * (width + hub)
+    want = oracle.ref_sssp(A, src)
+    assert np.isfinite(want[far - width:far]).any()
+    dist = torch.empty(n, dtype=torch.float32, device="cuda")
+    steps = []
+    for path in (B.PATH_AUTO, B.PATH_PUSH, B.PATH_AUTO):
+        h.set_opts(force_path=path)
+        steps.append(B.db_sssp(h.h, src, dist))
+        torch.cuda.synchronize()
+        assert np.array_equal(dist.cpu().numpy().astype(np.float64), want)
+    assert steps[0] == steps[1] == steps[2] and steps[0] >= layers
+    h.close()
