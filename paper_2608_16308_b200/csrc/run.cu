@@ -2623,7 +2623,7 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     if (weights) late = fmaxf(late, rows * fminf(SSSP_LATE_ROWS * (rows / (1 << 20)) * (rows / (1 << 20)), 1.0f));
     Device dev = d;
     int start = SSSP_STARTS;
-    for (int64_t made = 0;; start = h->sssp_host[2] ? SSSP_GOES_ON_LATE : SSSP_GOES_ON) {
+    for (int64_t made = 0;; start = h->sssp_host[2]) {
         int max_steps = (int)(d.n + 1 - made < SSSP_MAX_STEPS ? d.n + 1 - made : SSSP_MAX_STEPS);
         const bool can_pull = DT == DBSPMSPV_PATTERN ? d.rowrun_ptr != nullptr : d.weightrun != nullptr && d.col_degree != nullptr;
         unsigned pull_edges = can_pull ? (unsigned)(pull * (float)d.n_entries) : ~0u, late_edges = can_pull ? (unsigned)fminf(late, pull * (float)d.n_entries) : ~0u;

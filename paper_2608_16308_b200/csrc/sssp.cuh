@@ -60,7 +60,7 @@ constexpr int SSSP_CHUNK = 512;                   // elements of a listed chunk 
 // (The bitmap of 2^20 vertices is two rounds of every thread block, whatever it holds: a step of a few vertices took 14 us, 26 with a long run.)
 constexpr int SSSP_LIST = SSSP_CTA;
 constexpr unsigned SSSP_LIST_EDGES = 1u << 17;
-constexpr int SSSP_STARTS = 1, SSSP_GOES_ON = 0, SSSP_GOES_ON_LATE = 2;      // a launch: the first of its search, or one behind it (a step has been pulled before)
+constexpr int SSSP_STARTS = 1, SSSP_LATE = 2, SSSP_BELOW_ZERO = 4;      // a launch: the first of its search, or one behind it (a step has been pulled before; a distance has been below zero)
 constexpr int SSSP_MAX_STEPS = 1024;              // steps of one launch, at most: a cycle of negative weight ends on the host
 
 // What a step leaves to the next one, in one 16-byte word: a barrier is followed by one trip to L2.
@@ -76,7 +76,7 @@ struct SsspState {
     int32_t *ctr;             // [0] steps made, [1] array of the distances, [2..4] places taken in the step's list
     int4 *chunks;             // {row, first, end, -} of the listed chunks of long rows
     int32_t *list[2];         // the vertices marked by alternating steps, SSSP_LIST at most
-    int32_t *report;          // page-locked host words: steps made, vertices of the frontier that was left, whether a step has been pulled
+    int32_t *report;          // page-locked host words: steps made, vertices of the frontier that was left, SSSP_LATE, SSSP_BELOW_ZERO of what came before
     int32_t n_words;
 };
 
@@ -437,9 +437,9 @@ __device__ __forceinline__ void sssp_four(const Device &d, int k0, uint32_t (&co
 // No element behind one of weight w can do better than this (the order goes by the upper bits).  The lower bits of an infinite or NaN weight
 // must not be cut off: below -infinity in the order of words there are only NaNs, and the bound of a NaN would end the row.
 template <bool VAL>
-__device__ __forceinline__ int sssp_bound(float xmin, float w) {
+__device__ __forceinline__ float sssp_bound(float xmin, float w) {
     constexpr int least = (int)0x807FFFFFu;        // sssp_word(-infinity)
-    return sssp_word(xmin + (VAL ? sssp_value(max(sssp_word(w) & ~((1 << (32 - SSSP_WEIGHT_BITS)) - 1), least)) : w));
+    return xmin + (VAL ? sssp_value(max(sssp_word(w) & ~((1 << (32 - SSSP_WEIGHT_BITS)) - 1), least)) : w);
 }
 
 // A large step pulled.  Every row walks its own elements, which lie by weight (Device::weightrun), and stops at the first that
@@ -451,6 +451,9 @@ __device__ __forceinline__ int sssp_bound(float xmin, float w) {
 // stopped after SSSP_ROUNDS rounds is listed in chunks, which all warps share out behind a grid barrier (walked by the warp that met them, the
 // hub rows of an R-MAT graph, neighbours all, took one warp 300 us); of a row of several chunks only those whose first weight can still improve it.
 // Handles of unit weights walk the row-run index.
+// The sums of a walk are compared as floats (a distance is never -0, and fminf leaves NaNs out like the order of words does), and a gathered word is taken for its bits until a distance has been below zero:
+// where most rows are walked to their end, instructions bound the step.  Every sum turned into a word and every distance back / sums as floats / so: 27-point operator, weights in [0.05, 1.05), four sources,
+// 90^3 cells 6180 / 5180 / 5000 us a search, 120^3 15040 / 12580 / 12180, 150^3 35290 / 29620 / 28960; R-MAT 131 K vertices 117 / 110 / 110, 300 K 157 / 147 / 147, 2^20 183 / 171 / 168.
 // What bounds it: a distance gathered per element, one a clock and SM at most (12 M in the first pulled step of R-MAT scale 20: 41 of its 80 us), then the rows that come last, while
 // most warps stand at the barrier (the L1 is 11 % busy over a whole search).  That step took 156 us when a lane walked seven rows of its own and the blocks with a payload followed, a warp
 // at a time; the whole search 670, 560 and 530 us from three sources, 400, 328 and 312 now; in scattered order 354 - 466, 270 - 367 now.  A frontier bitmap in shared memory in front of the gathers: 80 -> 103 (L1 is what it
@@ -477,7 +480,8 @@ __device__ __forceinline__ void sssp_list_long(const Device &d, const SsspState 
     int chunks = (r.z - r.y + SSSP_CHUNK - 1) / SSSP_CHUNK;
     if (VAL)
         for (uint32_t todo = __ballot_sync(FULL, chunks > 1); todo; todo &= todo - 1) {      // the warp looks at 32 chunks of a row at a time
-            const int src = __ffs(todo) - 1, first = __shfl_sync(FULL, r.y, src), all = __shfl_sync(FULL, chunks, src), best = __shfl_sync(FULL, r.w, src);
+            const int src = __ffs(todo) - 1, first = __shfl_sync(FULL, r.y, src), all = __shfl_sync(FULL, chunks, src);
+            const float best = sssp_value(__shfl_sync(FULL, r.w, src));
             int kept = 0;
             while (kept < all) {
                 const int c = kept + lane;
@@ -521,8 +525,8 @@ __device__ void sssp_pull_shared(const Device &d, const SsspState &s, int c, uin
         int p = 0, e = 0, have = 0, degree = 0;
         float lightest = 0.f;
         if (r < d.n) { p = d.weight_ptr[r]; e = d.weight_ptr[r + 1]; have = __ldcg(dist + r); lightest = d.row_lightest[r]; degree = (int)d.col_degree[r]; }
-        int best = have;
-        bool walks = p < e && sssp_word(xmin + lightest) < have;
+        float best = sssp_value(have);
+        bool walks = p < e && xmin + lightest < best;
         for (int round = 0; round < SSSP_SHARED_ROUNDS && __any_sync(FULL, walks); ++round) {
             const int q = (p & ~3) + 4 * sub;
             uint32_t col[4];
@@ -532,28 +536,29 @@ __device__ void sssp_pull_shared(const Device &d, const SsspState &s, int c, uin
                 sssp_four<true>(d, q, col, w);
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    if (q + j >= p && q + j < e && sssp_word(xmin + w[j]) < best && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
+                    if (q + j >= p && q + j < e && xmin + w[j] < best && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
             }
-            int mine = best;
+            float mine = best;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) mine = min(mine, sssp_word(sssp_value(x[j]) + w[j]));
-            for (int o = 1; o < 1 << share; o <<= 1) mine = min(mine, __shfl_xor_sync(FULL, mine, o));
+            for (int j = 0; j < 4; ++j) mine = fminf(mine, sssp_value(x[j]) + w[j]);
+            for (int o = 1; o < 1 << share; o <<= 1) mine = fminf(mine, __shfl_xor_sync(FULL, mine, o));
             const float last = __shfl_sync(FULL, w[3], lane | ((1 << share) - 1));      // (the largest weight of the round)
             best = mine;
             p = (p & ~3) + (4 << share);
             walks = walks && p < e && sssp_bound<true>(xmin, last) < best;
         }
         if (sub == 0 && r < d.n) {
-            __stcg(word + r, best);
-            if (best < have) {
+            const int now = sssp_word(best);
+            __stcg(word + r, now);
+            if (now < have) {
                 atomicOr(next + (r >> 5), 1u << (r & 31));
-                ++tally.found; tally.low = min(tally.low, best); tally.edges += degree_of_code((uint32_t)degree);
+                ++tally.found; tally.low = min(tally.low, now); tally.edges += degree_of_code((uint32_t)degree);
             }
         }
         const uint32_t left = __ballot_sync(FULL, walks && sub == 0);
         if (left) {
             int4 *longs = sh.longs[warp];
-            if (walks && sub == 0) longs[__popc(left & ((1u << lane) - 1u))] = make_int4((int)r, p, e, best);
+            if (walks && sub == 0) longs[__popc(left & ((1u << lane) - 1u))] = make_int4((int)r, p, e, sssp_word(best));
             __syncwarp();
             sssp_list_long<true>(d, s, longs, __popc(left), xmin, n_long, lane);
             __syncwarp();
@@ -566,7 +571,7 @@ __device__ void sssp_pull_shared(const Device &d, const SsspState &s, int c, uin
 // marks that would spare the words that do not change (358 -> 405).  The distances of the 4 to 32 K columns of the highest degree in shared memory, where 34 to 69 % of the elements lie: nothing
 // gained with 4 K of them (before what it costs to bring them there), slower with more -- what they take from the L1 are the lines that the other gathers wait in.
 template <int DT>
-__device__ void sssp_pull(const Device &d, const SsspState &s, int c, const uint32_t *F, uint32_t *next, int low, int32_t *n_long, SsspPullShared &sh, SsspTally &tally) {
+__device__ void sssp_pull(const Device &d, const SsspState &s, int c, const uint32_t *F, uint32_t *next, int low, bool below_zero, int32_t *n_long, SsspPullShared &sh, SsspTally &tally) {
     constexpr bool VAL = DT != DBSPMSPV_PATTERN;
     constexpr int NONE = 0x7F800000;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -601,7 +606,8 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, int c, const uint
     };
     fetch();
     int head = 0, cnt = 0, n_listed = 0;
-    int row = -1, p = 0, e = 0, have = 0, best = NONE, q_long = 0;      // the row being walked: elements [p, e), from q_long on it is long
+    int row = -1, p = 0, e = 0, q_long = 0;            // the row being walked: elements [p, e), from q_long on it is long
+    float have = 0.f, best = __int_as_float(NONE);     // its distance before the step, and now
     int degree = 0;
     for (;;) {
         while (more && cnt < 32) {                     // (no more than that: what a warp has claimed no other one can take)
@@ -625,7 +631,7 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, int c, const uint
             const int k = __popc(idle & lt);
             if (row < 0 && k < cnt) {
                 const int4 q = queue[(head + k) & 63];
-                row = q.x; p = q.y; e = q.z; have = best = q.w; q_long = (p & ~3) + SSSP_ROUNDS * 4;
+                row = q.x; p = q.y; e = q.z; have = best = sssp_value(q.w); q_long = (p & ~3) + SSSP_ROUNDS * 4;
                 if (VAL) degree = queue_degree[(head + k) & 63];
             }
             const int took = min(__popc(idle), cnt);
@@ -638,35 +644,39 @@ __device__ void sssp_pull(const Device &d, const SsspState &s, int c, const uint
             float w[8];
             int x[8];
             const int q0 = p & ~3;
-            const bool two = best == NONE && q0 + 4 < e;
+            const bool two = best == __int_as_float(NONE) && q0 + 4 < e;
             sssp_four<VAL>(d, q0, reinterpret_cast<uint32_t (&)[4]>(col[0]), reinterpret_cast<float (&)[4]>(w[0]));
             if (two) sssp_four<VAL>(d, q0 + 4, reinterpret_cast<uint32_t (&)[4]>(col[4]), reinterpret_cast<float (&)[4]>(w[4]));
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 x[j] = NONE;
-                const bool go = (j < 4 || two) && q0 + j >= p && q0 + j < e && sssp_word(xmin + w[j]) < best;
+                const bool go = (j < 4 || two) && q0 + j >= p && q0 + j < e && xmin + w[j] < best;
                 if (go && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
             }
             float last = w[3];
+            if (VAL && below_zero)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) x[j] = __float_as_int(sssp_value(x[j]));
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-                if (j < 4 || two) { best = min(best, sssp_word(sssp_value(x[j]) + w[j])); last = w[j]; }
+                if (j < 4 || two) { best = fminf(best, __int_as_float(x[j]) + w[j]); last = w[j]; }
             p = q0 + (two ? 8 : 4);
-            const bool over = p >= e || bound(last) >= best;
+            const bool over = p >= e || !(bound(last) < best);
             left = !over && p >= q_long;
             if ((over || left) && best < have) {
+                const int now = sssp_word(best);
                 if (VAL) {
-                    __stcg(word + row, best);
+                    __stcg(word + row, now);
                     atomicOr(next + (row >> 5), 1u << (row & 31));
-                    ++tally.found; tally.low = min(tally.low, best); tally.edges += (unsigned)degree;
-                } else sssp_lower(d, word, next, row, best, have, tally);
+                    ++tally.found; tally.low = min(tally.low, now); tally.edges += (unsigned)degree;
+                } else sssp_lower(d, word, next, row, now, sssp_word(have), tally);
             }
             if (over) row = -1;
         }
         const uint32_t lm = __ballot_sync(FULL, left);
         if (lm) {
             if (n_listed + __popc(lm) > 32) { __syncwarp(); sssp_list_long<VAL>(d, s, longs, n_listed, xmin, n_long, lane); n_listed = 0; __syncwarp(); }
-            if (left) { longs[n_listed + __popc(lm & lt)] = make_int4(row, p, e, best); row = -1; }
+            if (left) { longs[n_listed + __popc(lm & lt)] = make_int4(row, p, e, sssp_word(best)); row = -1; }
             n_listed += __popc(lm);
         }
     }
@@ -728,6 +738,7 @@ __device__ void sssp_pull_long(const Device &d, const SsspState &s, int c, uint3
         const int start = had, row = now_c.x, p = now_c.y, e = now_c.z;
         int now = had;
         for (int q = (p & ~3) + 4 * lane;; q += 128) {
+            const float best = sssp_value(now);
             float wq[4];
             int x[4];
             const bool in = q < e, more = q - 4 * lane + 128 < e;             // (warp-uniform: the chunk goes on)
@@ -735,18 +746,18 @@ __device__ void sssp_pull_long(const Device &d, const SsspState &s, int c, uint3
             for (int j = 0; j < 4; ++j) {
                 x[j] = NONE;
                 wq[j] = w[j];
-                const bool go = in && q + j >= p && q + j < e && sssp_word(xmin + w[j]) < now;
+                const bool go = in && q + j >= p && q + j < e && xmin + w[j] < best;
                 if (go && DBS_CHK_INDEX(d, col[j], d.n)) x[j] = __ldca(dist + col[j]);
             }
             if (more) { if (q + 128 < e) sssp_four<VAL>(d, q + 128, col, w); }
             else { now_c = ahead; ahead = record(i + 2 * nwarps); first(now_c); }
-            int mine = now;
+            float mine = best;
             if (in)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mine = min(mine, sssp_word(sssp_value(x[j]) + wq[j]));
-            now = __reduce_min_sync(FULL, mine);
+                for (int j = 0; j < 4; ++j) mine = fminf(mine, sssp_value(x[j]) + wq[j]);
+            now = __reduce_min_sync(FULL, sssp_word(mine));
             if (!more) break;
-            const bool over = sssp_bound<VAL>(xmin, wq[3]) >= now;
+            const bool over = !(sssp_bound<VAL>(xmin, wq[3]) < sssp_value(now));
             if (__shfl_sync(FULL, (int)over, 31)) {    // (the last lane's weight is the largest of the step)
                 now_c = ahead; ahead = record(i + 2 * nwarps); first(now_c);
                 break;
@@ -765,8 +776,9 @@ __device__ void sssp_pull_long(const Device &d, const SsspState &s, int c, uint3
 constexpr int SSSP_SMEM = (int)(sizeof(SsspShared) > sizeof(SsspPullShared) ? sizeof(SsspShared) : sizeof(SsspPullShared));
 static_assert(sizeof(SsspListShared) <= sizeof(SsspShared), "the phases share one allocation");
 // The arguments stay in the constant bank: the lists and bitmaps are taken by the step's number, for which every thread kept a copy of its own in local memory, that
-// spilled more besides (216 -> 88 bytes of stack; R-MAT 300 K / 500 K / 2^20 vertices 242 / 252 / 359 -> 222 / 227 / 331 us a search, in scattered order 202 / 237 / 333 -> 186 / 217 / 306; 27-point
-// operator on 90^3 cells, an inner source, 3029 -> 2947).  The phases as functions of their own, which share no registers: 233 / 239 / 343 us.
+// spilled more besides (then 216 -> 88 bytes of stack, 144 by now; R-MAT 300 K / 500 K / 2^20 vertices 242 / 252 / 359 -> 222 / 227 / 331 us a search, in scattered order 202 / 237 / 333 -> 186 / 217 / 306; 27-point
+// operator on 90^3 cells, an inner source, 3029 -> 2947).  The phases as functions of their own, which share no registers: 233 / 239 / 343 us.  No phase holds the spills alone (each of them left out takes at most 40 of 120
+// bytes away): a kernel without the rows shared among lanes needs 120 all the same, and with what a row's walk keeps moved to shared memory large searches were up to 4 % longer.
 template <int DT>
 __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ Device d, const __grid_constant__ SsspState s, int32_t src, float *dist_out, int start, int max_steps, unsigned pull_edges, unsigned late_edges) {
     namespace cg = cooperative_groups;
@@ -775,7 +787,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
     SsspShared &sh = *reinterpret_cast<SsspShared *>(s_dyn);
     cg::grid_group grid = cg::this_grid();
     const int tid = blockIdx.x * SSSP_CTA + threadIdx.x, nthreads = gridDim.x * SSSP_CTA;
-    if (start == SSSP_STARTS) {                                       // (a later launch of the same search continues where the one before stopped)
+    if (start & SSSP_STARTS) {                         // (a later launch of the same search continues where the one before stopped)
         const int64_t n = (int64_t)s.n_words * 32;
         for (int64_t v = tid; v < n; v += nthreads) s.word[0][v] = s.word[1][v] = v == src ? 0 : 0x7F800000;
         for (int k = tid; k < s.n_words; k += nthreads) { s.bits[0][k] = k == src >> 5 ? 1u << (src & 31) : 0u; s.bits[1][k] = 0u; }       // (the third is cleared by the first step)
@@ -793,8 +805,9 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
         return SsspSet{(unsigned)v.x, (unsigned)v.y, v.z, v.w};
     };
     int t = __ldcg(s.ctr), c = __ldcg(s.ctr + 1);      // array c holds the distances; so does the other one, but for the frontier, of which it has larger ones
-    bool late = start == SSSP_GOES_ON_LATE;            // a step has been pulled, in this launch or one before
-    bool lists = start == SSSP_STARTS;                 // the step before listed what it marked, in list[(t + 1) & 1]
+    bool late = (start & SSSP_LATE) != 0;              // a step has been pulled, in this launch or one before
+    bool below_zero = (start & SSSP_BELOW_ZERO) != 0;  // a distance has been below zero, likewise: its word is not its bits
+    bool lists = (start & SSSP_STARTS) != 0;           // the step before listed what it marked, in list[(t + 1) & 1]
     SsspSet now = read(t % 3);                         // grid-uniform, as all that is decided from it
     for (int made = 0; made < max_steps && now.found; ++made, ++t, c ^= 1) {
         const uint32_t *F = s.bits[t % 3];
@@ -803,13 +816,14 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
         int32_t *n_long = &s.set[nxt].n_long, *n_list = s.ctr + 2 + t % 3;
         const bool listed = lists && now.found <= SSSP_LIST, pulled = now.edges > (late ? late_edges : pull_edges);
         late = late || pulled;
+        below_zero = below_zero || now.low < 0;
         lists = !pulled && now.edges <= SSSP_LIST_EDGES;
         if (tid == 0) { s.ctr[2 + nxt] = 0; s.set[(t + 2) % 3] = SsspSet{0u, 0u, 0x7F800000, 0}; }      // (their last readers were the steps t - 2 and t - 1)
         const SsspNext next{s.word[c], s.word[c ^ 1], N, lists ? s.list[t & 1] : nullptr, n_list};
         SsspTally tally;
         const int share = DT != DBSPMSPV_PATTERN ? sssp_row_share(d.n, nthreads) : 0;
         if (pulled && share) sssp_pull_shared(d, s, c, N, share, now.low, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), tally);
-        else if (pulled) sssp_pull<DT>(d, s, c, F, N, now.low, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), tally);
+        else if (pulled) sssp_pull<DT>(d, s, c, F, N, now.low, below_zero, n_long, *reinterpret_cast<SsspPullShared *>(s_dyn), tally);
         else if (listed) sssp_expand_list<DT>(d, s.list[(t + 1) & 1], (int)now.found, next, *reinterpret_cast<SsspListShared *>(s_dyn), tally);
         else sssp_expand<DT>(d, s, F, next, n_long, sh, tally);
         for (int k = tid; k < s.n_words; k += nthreads) Z[k] = 0u;
@@ -829,7 +843,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
     // the distances themselves
     for (int64_t v = tid; v < d.n; v += nthreads) dist_out[v] = sssp_value(__ldcg(s.word[c] + v));
     // (everyone read the counters before the first barrier, or leaves without a step)
-    if (tid == 0) { s.ctr[0] = t; s.ctr[1] = c; s.report[0] = t; s.report[1] = (int)now.found; s.report[2] = late; }
+    if (tid == 0) { s.ctr[0] = t; s.ctr[1] = c; s.report[0] = t; s.report[1] = (int)now.found; s.report[2] = (late ? SSSP_LATE : 0) | (below_zero ? SSSP_BELOW_ZERO : 0); }
 }
 
 }  // namespace dbs

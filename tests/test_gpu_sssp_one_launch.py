@@ -285,3 +285,31 @@ def test_many_pulled_steps_of_unit_weights(layers, width):
         assert np.array_equal(dist.cpu().numpy().astype(np.float64), want)
     assert steps[0] == steps[1] == steps[2] and steps[0] >= layers
     h.close()
+
+
+@pytest.mark.parametrize("length", [333, 2000])
+@pytest.mark.parametrize("base,step", [(4096.0, 1.0), (-4096.0, 1.0), (300.0, -1.0)])
+def test_pulled_steps_of_more_rows_than_lanes(length, base, step):
+    """The path of test_many_pulled_steps_in_a_row in a graph with more vertices than the GPU has lanes, where a lane walks a row: distances above zero, below, and such that pass through zero while
+    the search goes on (a distance's word is its bits above zero only), in the second launch too."""
+    n = length + 107 + 170000
+    k = np.arange(length)
+    rows = np.r_[1 + k, 2 + k[:-1], length + 1 + np.arange(6)]
+    cols = np.r_[np.zeros(length, np.int64), 1 + k[:-1], length + np.arange(6)]
+    val = np.r_[base + (step + 1.0) * k, np.full(length - 1, step), np.full(6, 3.0)].astype(np.float32)
+    order = np.argsort(rows.astype(np.int64) * n + cols)
+    ptr, idx = wl.csr_from_sorted_keys(n, n, (rows.astype(np.int64) * n + cols)[order])
+    want = np.full(n, np.inf, np.float32)
+    want[0] = 0.0
+    want[1:length + 1] = base + step * k
+    want[length + 1:length + 7] = base + step * (length - 1) + 3.0 * (1 + np.arange(6))
+    h = Handle(wl.CSR(n, n, ptr, idx, val[order]), B.F32)
+    dist = torch.empty(n, dtype=torch.float32, device="cuda")
+    steps = []
+    for path in (B.PATH_AUTO, B.PATH_PUSH, B.PATH_AUTO):
+        h.set_opts(force_path=path)
+        steps.append(B.db_sssp(h.h, 0, dist))
+        torch.cuda.synchronize()
+        assert np.array_equal(dist.cpu().numpy(), want)
+    assert steps[0] == steps[1] == steps[2] and steps[0] > length
+    h.close()
