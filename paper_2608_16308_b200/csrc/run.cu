@@ -2618,9 +2618,10 @@ static int sssp_one_launch(dbspmspv_handle_s *h, int32_t src, float *dist, int32
     s.report = h->sssp_host;
     // edges from which a step is pulled, the first one and those behind it (sssp.cuh)
     const bool weights = DT != DBSPMSPV_PATTERN;
-    const float rows = (float)d.n, pull = weights && h->payload_rich ? SSSP_PULL_SHARE_PAYLOAD : SSSP_PULL_SHARE;
+    const bool rich = weights && h->payload_rich;
+    const float rows = (float)d.n, pull = rich && d.n <= (int64_t)h->sm_count * SSSP_CTA ? SSSP_PULL_SHARE_PAYLOAD : SSSP_PULL_SHARE;
     float late = SSSP_LATE_SHARE * (float)d.n_entries;
-    if (weights) late = fmaxf(late, rows * fminf(SSSP_LATE_ROWS * (rows / (1 << 20)) * (rows / (1 << 20)), 1.0f));
+    if (weights) late = fmaxf(late, rows * fminf(SSSP_LATE_ROWS * (rows / (1 << 20)) * (rows / (1 << 20)), rich ? SSSP_LATE_ROWS : 1.0f));
     Device dev = d;
     int start = SSSP_STARTS;
     for (int64_t made = 0;; start = h->sssp_host[2]) {

@@ -41,8 +41,9 @@ constexpr int SSSP_ILP = 4;                       // warp steps in flight
 // vertices in scattered order: 131 K vertices 172 / 169 / 167 / 168 us a search (128 / 127 / 127 / 128), 300 K 142 / 142 / 143 / 142 (146 / 144 / 143 / 142), 500 K 232 / 229 / 229 / 229,
 // 2^20 315 / 307 / 309 / 308 (291 / 286 / 286 / 286).
 constexpr float SSSP_PULL_SHARE = 0.1f;
-// ... on handles of weights with many payload blocks (payload_rich), whose entries a push takes one by one: 5 % instead of 10 %, 27-point operators, three sources, 150^3 cells 12850 / 8750 / 8670 -> 12450 / 8090 / 8670 us,
-// 120^3 5990 / 3990 / 4070 -> 6070 / 4030 / 4070.
+// ... on handles of weights with many payload blocks (payload_rich), whose entries a push takes one by one, while their rows are shared among lanes, which makes a pulled step cheap: 27-point operators, weights
+// of one size / in [0.05, 1.05), which improve a vertex more often, four sources, 5 -> 10 %: 40^3 cells 408 -> 568 / 493 -> 540 us a search, 90^3 2493 -> 2517 / 5000 -> 4863, 120^3 4971 -> 5006 / 12181 -> 11725,
+// 150^3 10084 -> 10356 / 28964 -> 27580 (before the rules on shares 11517 / 27904).
 constexpr float SSSP_PULL_SHARE_PAYLOAD = 0.05f;
 // Once a step has been pulled the rows have bests that prune, and a pulled step that finds little costs a pass over the rows: the share for the steps behind it.  5 / 0.5 / 0.2 / 0.05 %, six
 // sources: 131 K vertices 180 / 174 / 173 / 172 (156 / 149 / 149 / 149), 300 K 175 / 168 / 167 / 167 (136 / 133 / 133 / 134), 500 K 253 / 242 / 240 / 239, 2^20 371 / 362 / 362 / 356 (307 / 296 / 294 / 301).
@@ -50,7 +51,7 @@ constexpr float SSSP_LATE_SHARE = 0.002f;
 // With weights that pass is what the step costs on large graphs: it has to be worth an edge for so many rows too -- an eighth of them at 2^20, rising with the square to all of them, the more of the rows' words no longer
 // stay in L2 (and with fewer elements a row than R-MAT's 32 the share of the elements says little about it).  A share of 0.2 % alone / an eighth / a quarter / a half / all of the rows, uniform rows of 4 or 8:
 // 2 M x 4 1135 / 1004 / 931 / 896 / 896 us a search, x 8 1483 / 1399 / 1347 / 1290 / 1239, 8 M x 4 4123 / 3620 / 3480 / 3393 / 3393, x 8 5514 / 5157 / 4969 / 4781 / 4602; R-MAT 2^20 286 / 287 / 288 / 291 / 294 (251 / 252 / 253 / 254 /
-// 260).  (Unit weights: the share alone is the better rule, 8 M uniform rows x 8 764 / 776 / 775 / 791 / 793, R-MAT of 4 M vertices x 8 234 / 242 / 249 / 258 / 259.)
+// 260); on handles with many payload blocks no more than that eighth, 150^3 cells, weights in [0.05, 1.05), an eighth / a half 27580 / 27754.  (Unit weights: the share alone is the better rule, 8 M uniform rows x 8 764 / 776 / 775 / 791 / 793, R-MAT of 4 M vertices x 8 234 / 242 / 249 / 258 / 259.)
 constexpr float SSSP_LATE_ROWS = 0.125f;
 // Rounds of four elements that a lane walks of a row.  6 / 8 / 12, the same six: 131 K vertices 177 / 173 / 180 (153 / 149 / 158), 300 K 172 / 167 / 175 (137 / 133 / 136), 500 K 246 / 240 / 240,
 // 2^20 373 / 362 / 363 (300 / 294 / 299).

@@ -313,3 +313,16 @@ def test_pulled_steps_of_more_rows_than_lanes(length, base, step):
         assert np.array_equal(dist.cpu().numpy(), want)
     assert steps[0] == steps[1] == steps[2] and steps[0] > length
     h.close()
+
+
+def test_pulled_steps_of_a_large_handle_with_many_payload_blocks():
+    """A 27-point operator on 55^3 cells, more rows than the GPU has lanes: its steps are pulled from the larger share of the elements on, those behind them from an eighth of the rows' number of edges at most."""
+    d = 55
+    g, rng = wl.stencil27(d, seed=3), np.random.default_rng(3)
+    cells = g.rows(), g.col_idx
+    csr = graph(g.n, [(cells[1], cells[0], (1 + rng.integers(0, 63, g.nnz)) / 8.0)])
+    h = Handle(csr, B.F32)
+    st = h.get_stats()
+    assert csr.nnz < 8 * sum(st.class_nnz[1:]) and 2 * sum(st.class_nnz[2:]) < csr.nnz
+    h.close()
+    check_steps(csr, d // 2 * (1 + d + d * d))
