@@ -788,7 +788,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
     SsspShared &sh = *reinterpret_cast<SsspShared *>(s_dyn);
     cg::grid_group grid = cg::this_grid();
     const int tid = blockIdx.x * SSSP_CTA + threadIdx.x, nthreads = gridDim.x * SSSP_CTA;
-    if (start & SSSP_STARTS) {                         // (a later launch of the same search continues where the one before stopped)
+    if (start == SSSP_STARTS) {                        // (a later launch of the same search continues where the one before stopped)
         const int64_t n = (int64_t)s.n_words * 32;
         for (int64_t v = tid; v < n; v += nthreads) s.word[0][v] = s.word[1][v] = v == src ? 0 : 0x7F800000;
         for (int k = tid; k < s.n_words; k += nthreads) { s.bits[0][k] = k == src >> 5 ? 1u << (src & 31) : 0u; s.bits[1][k] = 0u; }       // (the third is cleared by the first step)
@@ -807,8 +807,9 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
     };
     int t = __ldcg(s.ctr), c = __ldcg(s.ctr + 1);      // array c holds the distances; so does the other one, but for the frontier, of which it has larger ones
     bool late = (start & SSSP_LATE) != 0;              // a step has been pulled, in this launch or one before
-    bool below_zero = (start & SSSP_BELOW_ZERO) != 0;  // a distance has been below zero, likewise: its word is not its bits
-    bool lists = (start & SSSP_STARTS) != 0;           // the step before listed what it marked, in list[(t + 1) & 1]
+    constexpr bool VAL = DT != DBSPMSPV_PATTERN;
+    bool below_zero = VAL && (start & SSSP_BELOW_ZERO);      // a distance has been below zero, likewise: its word is not its bits
+    bool lists = start == SSSP_STARTS;                 // the step before listed what it marked, in list[(t + 1) & 1]
     SsspSet now = read(t % 3);                         // grid-uniform, as all that is decided from it
     for (int made = 0; made < max_steps && now.found; ++made, ++t, c ^= 1) {
         const uint32_t *F = s.bits[t % 3];
@@ -817,7 +818,7 @@ __global__ void __launch_bounds__(SSSP_CTA, 1) k_sssp(const __grid_constant__ De
         int32_t *n_long = &s.set[nxt].n_long, *n_list = s.ctr + 2 + t % 3;
         const bool listed = lists && now.found <= SSSP_LIST, pulled = now.edges > (late ? late_edges : pull_edges);
         late = late || pulled;
-        below_zero = below_zero || now.low < 0;
+        if (VAL) below_zero = below_zero || now.low < 0;
         lists = !pulled && now.edges <= SSSP_LIST_EDGES;
         if (tid == 0) { s.ctr[2 + nxt] = 0; s.set[(t + 2) % 3] = SsspSet{0u, 0u, 0x7F800000, 0}; }      // (their last readers were the steps t - 2 and t - 1)
         const SsspNext next{s.word[c], s.word[c ^ 1], N, lists ? s.list[t & 1] : nullptr, n_list};
